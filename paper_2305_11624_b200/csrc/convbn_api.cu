@@ -446,8 +446,7 @@ int run_conv_dgrad(const convbn_desc *d, const Problem &pb, const void *dz, cons
         LAUNCH("stem_dgrad", launch_stem_dgrad(pb, dz, w, scale, dx, st));
         *which = "stem-mma";
     } else if (grouped_path(d, pb) && grouped8_eligible(pb)) {
-        LAUNCH("grouped_flip", launch_grouped8_flip_weights(pb, w, scale, wbd_scratch, st));
-        LAUNCH("grouped_dgrad", launch_grouped8_dgrad(pb, dz, wbd_scratch, dx, st));
+        LAUNCH("grouped_dgrad", launch_grouped8_dgrad(pb, dz, w, scale, dx, st));
         *which = "grouped-mma";
     } else if (grouped_path(d, pb) && pb.stride_h == 1 && pb.stride_w == 1) {
         s = UmmaConvShape{pb.n, pb.h_out, pb.w_out, pb.c_out, pb.h_in, pb.w_in, pb.c_in, pb.kh, pb.kw,
@@ -733,6 +732,12 @@ int convbn_tune_fwd(const convbn_desc *desc, const void *x, const void *w, const
         const BnFold fold{gamma, beta, run_mean, run_var, b, pb.eps, vec3};
         LAUNCH("dw_fwd", launch_dw_tma(pb, x, w, nullptr, z, st, &fold));
         t_last_kernel[CONVBN_PHASE_TUNE_FWD] = "depthwise";
+        return CONVBN_OK;
+    }
+    if (grouped_path(desc, pb) && grouped8_eligible(pb)) {
+        const BnFold fold{gamma, beta, run_mean, run_var, b, pb.eps, vec3};
+        LAUNCH("grouped_fwd", launch_grouped8_fwd(pb, x, w, nullptr, z, st, &fold));
+        t_last_kernel[CONVBN_PHASE_TUNE_FWD] = "grouped-mma";
         return CONVBN_OK;
     }
     LAUNCH("reparam", launch_reparam(pb, desc->dtype, desc->layout, w, b, gamma, beta, run_mean, run_var, vec3, wf,

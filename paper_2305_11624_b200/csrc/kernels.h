@@ -203,11 +203,11 @@ cudaError_t launch_dw_wgrad(const Problem &pb, const void *dz, const void *x, fl
 bool grouped_bd_eligible(const Problem &pb);
 // 8 channels per group, unit stride and dilation, at most 10 taps: warp-level MMAs fed by a TMA patch ring
 bool grouped8_eligible(const Problem &pb);
+// (fold != NULL replaces `bias`; backward data rotates, transposes and scales omega by s_vec (NULL = 1) on the fly)
 cudaError_t launch_grouped8_fwd(const Problem &pb, const void *x, const void *w, const float *bias, void *z,
-                                cudaStream_t st);
-cudaError_t launch_grouped8_flip_weights(const Problem &pb, const void *w, const float *s_vec, void *wt,
-                                         cudaStream_t st);
-cudaError_t launch_grouped8_dgrad(const Problem &pb, const void *dz, const void *wt, void *dx, cudaStream_t st);
+                                cudaStream_t st, const BnFold *fold = nullptr);
+cudaError_t launch_grouped8_dgrad(const Problem &pb, const void *dz, const void *w, const float *s_vec, void *dx,
+                                  cudaStream_t st);
 // backward weight: part [slots][C][taps 8] and bsum [slots][C] floats, slots = grouped8_wgrad_slots(pb)
 int grouped8_wgrad_slots(const Problem &pb);
 cudaError_t launch_grouped8_wgrad(const Problem &pb, const void *dz, const void *x, float *part, float *bsum,

@@ -38,8 +38,15 @@ __device__ __forceinline__ void ldmatrix_x4(uint32_t &r0, uint32_t &r1, uint32_t
                  : "memory");
 }
 
+// The reverse: register i of lane (g, t) holds elements [row g][columns 2t, 2t + 1] of matrix i; lanes 8i..8i+7 give
+// the addresses of its 16-byte rows.
+__device__ __forceinline__ void stmatrix_x4(uint32_t smem_addr, uint32_t r0, uint32_t r1, uint32_t r2, uint32_t r3) {
+    asm volatile("stmatrix.sync.aligned.m8n8.x4.shared.b16 [%0], {%1, %2, %3, %4};"
+                 ::"r"(smem_addr), "r"(r0), "r"(r1), "r"(r2), "r"(r3)
+                 : "memory");
+}
 
-// The same with every matrix transposed on the way: register i of lane (g, t) receives elements
+// ldmatrix with every matrix transposed on the way: register i of lane (g, t) receives elements
 // [row 2t][column g] and [row 2t + 1][column g] of matrix i.
 __device__ __forceinline__ void ldmatrix_x4_trans(uint32_t &r0, uint32_t &r1, uint32_t &r2, uint32_t &r3,
                                                   uint32_t smem_addr) {

@@ -124,6 +124,15 @@ __device__ __forceinline__ void named_bar_sync(uint32_t id, uint32_t count) {
 __device__ __forceinline__ void named_bar_arrive(uint32_t id, uint32_t count) {
     asm volatile("barrier.cta.arrive %0, %1;" ::"r"(id), "r"(count) : "memory");
 }
+// Barrier over `count` threads that also tells every one of them whether `ok` held for all.
+__device__ __forceinline__ bool named_bar_all(uint32_t id, uint32_t count, bool ok) {
+    uint32_t all;
+    asm volatile("{\n\t.reg .pred p, q;\n\tsetp.ne.u32 p, %3, 0;\n\tbarrier.cta.red.and.pred q, %1, %2, p;\n\tselp.u32 %0, 1, 0, q;\n\t}"
+                 : "=r"(all)
+                 : "r"(id), "r"(count), "r"(ok ? 1u : 0u)
+                 : "memory");
+    return all != 0;
+}
 
 // ---- TMA loads (global -> this CTA's shared memory, completion on an mbarrier) ----------------
 __device__ __forceinline__ void tma_load_2d(void *smem_dst, const CUtensorMap *map, uint64_t *bar, int x, int y) {

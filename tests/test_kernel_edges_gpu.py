@@ -1,0 +1,25 @@
+"""Sizes at which the tiling, the remainders or the dispatch of a kernel change, against the fp64 oracle."""
+import pytest
+
+import parity
+from paper_2305_11624_b200 import inputs as I
+
+pytestmark = pytest.mark.gpu
+
+L = I.LayerSpec
+SPECS = [
+    # 8 channels per group: more chunks of channels than the grid has slots left over (the grid is rounded to chunks),
+    # the widest row one box takes, a last band of one row
+    L("g8_chunks", 13, 704, 9, 10, 704, 3, 3, pad=1, groups=88, bias=True),
+    L("g8_wide", 1, 64, 5, 254, 64, 3, 3, pad=1, groups=8, dtype="f16"),
+    L("g8_last_row", 9, 128, 17, 29, 128, 3, 3, pad=1, groups=16),
+]
+
+
+@pytest.mark.parametrize("spec", SPECS, ids=lambda s: s.name)
+def test_tune_block(spec):
+    t = parity.make_inputs(spec, 77)
+    ref = parity.oracle_tune(spec, t)
+    for deferred in (False, True):
+        got = parity.run_tune_gpu(spec, t, deferred=deferred)
+        parity.compare(got, ref, parity.TOL[spec.dtype], parity.TUNE_OUTPUTS, spec.name, dtype=spec.dtype)
