@@ -126,6 +126,10 @@ struct Plan {
     bool stem = false;
     bool stem_win_wgrad = false;   // stem weight gradient straight from X (window operand), fused epilogue
     size_t wbd = 0;        // block-diagonal expanded weights [C_out][taps][64], storage dtype
+    // Eval backward of a dense tensor-core layer: s commutes with both contractions, so dX and domega come from dZ through
+    // the Tune kernels and no s dZ tensor exists (eval_inner: offset of their workspace)
+    bool eval_direct = false;
+    size_t eval_inner = 0;
     bool umma_wgrad = false, dw_wgrad = false, dw_tma_wgrad = false, grouped_wgrad = false, grouped8_wgrad = false;
     UmmaWgradPlan uw;
 };
@@ -134,8 +138,12 @@ bool fused_bwd_path(const convbn_desc *d, const Problem &pb) {
     return d->dtype == CONVBN_BF16 && d->layout == CONVBN_NHWC && fused_bwd1x1_eligible(pb);
 }
 
+bool strided_dgrad_ok(const convbn_desc *d, const Problem &pb);
+bool umma_dgrad_shape(const convbn_desc *d, const Problem &pb, UmmaConvShape *s);
+
 Plan make_plan(const convbn_desc *d, const Problem &pb, int phase) {
     Plan pl;
+    UmmaConvShape us;
     if (phase == CONVBN_PHASE_TUNE_BWD) {
         if (!fused_bwd_path(d, pb)) {       // the two passes run side by side: each has its own region
             const Plan a = make_plan(d, pb, CONVBN_PHASE_TUNE_BWD_DATA), b2 = make_plan(d, pb, CONVBN_PHASE_TUNE_BWD_WEIGHT);
@@ -246,6 +254,14 @@ Plan make_plan(const convbn_desc *d, const Problem &pb, int phase) {
             pl.xpk = take(xpk_bytes); pl.wst = take(wst_bytes);
             break;
         case CONVBN_PHASE_EVAL_BWD:
+            pl.eval_direct = pl.umma_wgrad && (strided_dgrad_ok(d, pb) || umma_dgrad_shape(d, pb, &us));
+            if (pl.eval_direct) {
+                pl.vec3 = take(3 * (size_t)pb.c_out * sizeof(float));
+                pl.part_g = take((size_t)pl.bn_splits * pb.c_out * sizeof(float));
+                pl.bsum = take((size_t)pl.bn_splits * pb.c_out * sizeof(float));
+                pl.eval_inner = take(make_plan(d, pb, CONVBN_PHASE_TUNE_BWD).total);
+                break;
+            }
             pl.dy = take((size_t)pb.p * pb.c_out * elem_size(d->dtype));
             pl.w_scaled = take(wbytes);
             pl.wbd = take(wbd_bytes);
@@ -570,11 +586,12 @@ int run_conv_dgrad(const convbn_desc *d, const Problem &pb, const void *dz, cons
 // Parameter gradients from dZ and X, shared by all modes.
 //   vec3 != NULL (Tune): dw = s domega', dbeta, db = s dbeta, dgamma          (Table 2, Tune row)
 //   vec3 == NULL        : dw = domega', db = sum dZ if db != NULL               (Deploy / Eval rows)
+//   scale_only          : dw = s domega' alone, s the first C_out floats of vec3 (dense tensor-core path)
 int run_param_grads(const convbn_desc *d, const Problem &pb, const Plan &pl, const void *dz, const void *x,
                     const void *w, const float *vec3, const float *b, const float *mean, float *dw, float *db,
-                    float *dgamma, float *dbeta, void *ws, cudaStream_t st, const char **which) {
+                    float *dgamma, float *dbeta, void *ws, cudaStream_t st, const char **which, bool scale_only = false) {
     float *partials = (float *)at(ws, pl.partials), *bsum = (float *)at(ws, pl.bsum);
-    const bool need_bsum = vec3 || db;
+    const bool need_bsum = (vec3 || db) && !scale_only;
     const bool tc = pl.grouped_wgrad || pl.umma_wgrad || pl.stem;   // tensor-core paths sum dZ inside the GEMM
     if (need_bsum && !tc && !pl.dw_tma_wgrad)
         LAUNCH("channel_sum", launch_channel_sum_partial(pb, d->dtype, d->layout, dz, bsum, pl.bsplits, st));
@@ -955,9 +972,16 @@ int convbn_eval_fwd(const convbn_desc *desc, const void *x, const void *w, const
     CK(check_ws(pl, workspace, workspace_bytes));
     cudaStream_t st = (cudaStream_t)stream;
     float *vec3 = (float *)at(workspace, pl.vec3);
+    UmmaConvShape us;
+    if (!pl.stem && !grouped_path(desc, pb) && umma_fwd_shape(desc, pb, &us) && !umma_strip_eligible(us)) {
+        // the GEMM's epilogue stores Y and its normalisation Z
+        const BnFold fold{gamma, beta, run_mean, run_var, b, pb.eps, nullptr};
+        LAUNCH("umma_fwd", launch_umma_conv(us, x, w, nullptr, y_saved, st, &fold, z));
+        t_last_kernel[CONVBN_PHASE_EVAL_FWD] = "umma";
+        return CONVBN_OK;
+    }
     // BN acts on Y, which already holds the conv bias: shift = beta - mean s
-    LAUNCH("reparam", launch_reparam(pb, desc->dtype, desc->layout, w, nullptr, gamma, beta, run_mean, run_var, vec3,
-                      nullptr, nullptr, st));
+    LAUNCH("bn_vec3", launch_bn_vec3(pb.c_out, pb.eps, nullptr, gamma, beta, run_mean, run_var, vec3, st));
     CK(run_conv_fwd(desc, pb, x, w, b, y_saved, pl, workspace, st, &t_last_kernel[CONVBN_PHASE_EVAL_FWD]));
     LAUNCH("bn_eval_fwd", launch_bn_eval_fwd(pb, desc->dtype, desc->layout, y_saved, vec3, z, st));
     return CONVBN_OK;
@@ -985,6 +1009,40 @@ int convbn_eval_bwd(const convbn_desc *desc, const void *dz, const void *x, cons
     cudaStream_t st = (cudaStream_t)stream;
     void *dy = at(workspace, pl.dy);
     float *pg = (float *)at(workspace, pl.part_g), *pbm = (float *)at(workspace, pl.bsum);
+    if (pl.eval_direct) {
+        // dX = omega_rot (*) (s dZ) = (s omega)_rot (*) dZ and domega = (s dZ) (.) X = s (dZ (.) X) (Table 2, Eval row):
+        // the sums over dZ and Y run beside the two contractions, which read dZ itself
+        float *vec3 = (float *)at(workspace, pl.vec3);
+        void *inner = at(workspace, pl.eval_inner);
+        const Plan pt = make_plan(desc, pb, CONVBN_PHASE_TUNE_BWD);
+        const bool fused = fused_bwd_path(desc, pb);
+        LAUNCH("bn_vec3", launch_bn_vec3(pb.c_out, pb.eps, nullptr, gamma, nullptr, run_mean, run_var, vec3, st));
+        return side_by_side(
+            st,
+            [&](cudaStream_t st) -> int {
+                LAUNCH("bn_eval_bwd", launch_bn_eval_bwd(pb, desc->dtype, desc->layout, dz, y_saved, gamma, run_mean, run_var,
+                                                         nullptr, pg, pbm, pl.bn_splits, st));
+                LAUNCH("bn_eval_finish", launch_bn_eval_finish(pb, pg, pbm, pl.bn_splits, gamma, run_var, db, dgamma, dbeta, st));
+                if (fused) return CONVBN_OK;
+                const char *unused = nullptr;
+                return run_param_grads(desc, pb, make_plan(desc, pb, CONVBN_PHASE_TUNE_BWD_WEIGHT), dz, x, w, vec3, nullptr,
+                                       run_mean, dw, nullptr, nullptr, nullptr, at(inner, pt.w_scaled), st, &unused, true);
+            },
+            [&]() -> int {
+                if (fused) {
+                    LAUNCH("umma_bwd", launch_fused_bwd1x1(pb, dz, x, w, vec3, dx, (float *)at(inner, pt.partials),
+                                                           (float *)at(inner, pt.bsum), (unsigned int *)at(inner, pt.counters), st));
+                    LAUNCH("wgrad_epilogue_fused",
+                           launch_wgrad_epilogue_fused(pb, pt.uw, (const float *)at(inner, pt.partials),
+                                                       (const float *)at(inner, pt.bsum), w, vec3, nullptr, run_mean, dw,
+                                                       (float *)at(inner, pt.dotpart), (unsigned int *)at(inner, pt.counters),
+                                                       nullptr, nullptr, nullptr, false, st));
+                    t_last_kernel[CONVBN_PHASE_EVAL_BWD] = "umma-fused-bwd";
+                    return CONVBN_OK;
+                }
+                return run_conv_dgrad(desc, pb, dz, w, vec3, inner, nullptr, dx, st, &t_last_kernel[CONVBN_PHASE_EVAL_BWD]);
+            });
+    }
     LAUNCH("bn_eval_bwd", launch_bn_eval_bwd(pb, desc->dtype, desc->layout, dz, y_saved, gamma, run_mean, run_var, dy, pg,
                           pbm, pl.bn_splits, st));
     LAUNCH("bn_eval_finish", launch_bn_eval_finish(pb, pg, pbm, pl.bn_splits, gamma, run_var, db, dgamma, dbeta, st));
@@ -1172,7 +1230,7 @@ int convbn_tconv_tune_fwd(const convbn_desc *desc, const void *x, const void *w,
     const int taps = desc->kh * desc->kw, cig = desc->c_in / desc->groups, cog = desc->c_out / desc->groups;
     float *vec3 = (float *)saved;
     void *wf = at(workspace, v.off_w), *inner = at(workspace, v.off_inner);
-    LAUNCH("tconv_vec3", launch_tconv_vec3(desc->c_out, (float)desc->eps, b, gamma, beta, run_mean, run_var, vec3, st));
+    LAUNCH("tconv_vec3", launch_bn_vec3(desc->c_out, (float)desc->eps, b, gamma, beta, run_mean, run_var, vec3, st));
     LAUNCH("tconv_rescale", launch_tconv_rescale(desc->dtype, nhwc, (long long)v.wcount, taps, cig, cog, w, vec3, wf, st));
     // Z = omega' scattered over X: the backward-data pass of the convolution with the same weights
     const char *which = nullptr;

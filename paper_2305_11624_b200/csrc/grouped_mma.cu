@@ -4,8 +4,8 @@
 // One group is a GEMM with N = 8 and K = 8 per tap (about 36 FLOP per byte moved): far too narrow for a
 // 128-row tcgen05 tile, whose block-diagonal emulation spends 8x the MMA work and was bound by it, but an
 // exact fit for the warp-level m16n8k16 MMA: 16 pixels x (2 taps x 8 input channels) x 8 output channels.
-// The kernel is organised around the memory stream.  Work item = (image, band of R output rows, 64-channel
-// chunk); a producer warp brings the item's input patch ((R + kh - 1) rows x (W + kw - 1) columns x 64
+// The kernel is organised around the memory stream.  Work item = (image, band of R output rows (of a column strip),
+// 64-channel chunk); a producer warp brings the item's input patch ((R + kh - 1) rows x (W + kw - 1) columns x 64
 // channels, zero fill outside the image) into a ring of shared-memory stages with one TMA box (128-byte
 // swizzle).  Compute warp w owns group w of the chunk: its A fragments are ldmatrix loads of [pixel][8
 // channels] rows at the tap's shifted start address (virtual pixels, row pitch W + kw - 1: the outputs of
@@ -40,6 +40,7 @@ struct GroupedCtl {
 struct GroupedGeom {
     int n, ho, wo, c, kh, kw, lower_h, lower_w;
     int R, Wt, rows_in, tiles_h;
+    int cols, tiles_w;         // output columns of a band (convolution only: wide images are cut into column strips)
     int stages;
     uint32_t patch_bytes;      // bytes one TMA box writes
     uint32_t stage_stride;     // allocation per stage (multiple of 1024, includes the read-ahead tail)
@@ -73,7 +74,7 @@ __global__ void __launch_bounds__(kGThreads, 3) grouped8_conv_kernel(const __gri
     pdl_wait();
     pdl_launch_dependents();
     if (threadIdx.x == 0) { CONVBN_TRACE_POINT(0); }
-    const uint32_t items = (uint32_t)g.n * g.tiles_h * chunks;   // chunk fastest: the chunks of a patch run together
+    const uint32_t items = (uint32_t)g.n * g.tiles_h * g.tiles_w * chunks;   // chunk fastest: a patch's chunks run together
     if (warp == 8) {
         if (lane == 0) {
             uint32_t s = 0, ph = 0;
@@ -81,10 +82,12 @@ __global__ void __launch_bounds__(kGThreads, 3) grouped8_conv_kernel(const __gri
             for (uint32_t it = blockIdx.x; it < items; it += gridDim.x) {
                 const int cc = (int)(it % (uint32_t)chunks);
                 const uint32_t t1 = it / (uint32_t)chunks;
-                const int h0 = (int)(t1 % (uint32_t)g.tiles_h) * g.R, img = (int)(t1 / (uint32_t)g.tiles_h);
+                const uint32_t t2 = t1 / (uint32_t)g.tiles_w;
+                const int w0 = (int)(t1 - t2 * (uint32_t)g.tiles_w) * g.cols;
+                const int h0 = (int)(t2 % (uint32_t)g.tiles_h) * g.R, img = (int)(t2 / (uint32_t)g.tiles_h);
                 if (!mbar_wait_bounded(&ctl->empty[s], ph ^ 1u, abort_flag)) { ok = false; break; }
                 mbar_arrive_expect_tx(&ctl->full[s], g.patch_bytes);
-                tma_load_4d(ring + (size_t)s * g.stage_stride, &tm_act, &ctl->full[s], cc * 64, g.lower_w,
+                tma_load_4d(ring + (size_t)s * g.stage_stride, &tm_act, &ctl->full[s], cc * 64, w0 + g.lower_w,
                             h0 + g.lower_h, img);
                 if (++s == (uint32_t)g.stages) { s = 0; ph ^= 1u; }
             }
@@ -151,8 +154,9 @@ __global__ void __launch_bounds__(kGThreads, 3) grouped8_conv_kernel(const __gri
     uint32_t s = 0, ph = 0;
     bool ok = true;
     for (uint32_t it = blockIdx.x; it < items && ok; it += gridDim.x) {
-        const uint32_t t1 = it / (uint32_t)chunks;
-        const int h0 = (int)(t1 % (uint32_t)g.tiles_h) * g.R, img = (int)(t1 / (uint32_t)g.tiles_h);
+        const uint32_t t1 = it / (uint32_t)chunks, t2 = t1 / (uint32_t)g.tiles_w;
+        const int w0 = (int)(t1 - t2 * (uint32_t)g.tiles_w) * g.cols;
+        const int h0 = (int)(t2 % (uint32_t)g.tiles_h) * g.R, img = (int)(t2 / (uint32_t)g.tiles_h);
         ok = mbar_wait_bounded(&ctl->full[s], ph, abort_flag);
         // the image buffer is free once the box of the item before has been read out of it; the warps leave together
         if (threadIdx.x == 0) tma_store_wait_read<0>();
@@ -190,15 +194,15 @@ __global__ void __launch_bounds__(kGThreads, 3) grouped8_conv_kernel(const __gri
 #pragma unroll
             for (int u = 0; u < kGTiles; u += 2) {
                 const int v = v0 + 16 * u + lane, ti = v / g.Wt, tj = v - ti * g.Wt;
-                const int row = (ti < g.R && tj < g.wo) ? ti * g.wo + tj : g.R * g.wo;
+                const int row = (ti < g.R && tj < g.cols) ? ti * g.cols + tj : g.R * g.cols;
                 stmatrix_x4(image_s + (uint32_t)row * 128u + (uint32_t)((warp ^ (row & 7)) << 4), o[2 * u], o[2 * u + 1],
                             o[2 * u + 2], o[2 * u + 3]);
             }
         }
         fence_proxy_async_smem();
         named_bar_sync(1, 256);
-        if (threadIdx.x == 0) {                    // rows below the image are clipped by the map
-            tma_store_4d(&tm_out, image, cc * 64, 0, h0, img);
+        if (threadIdx.x == 0) {                    // rows and columns outside the image are clipped by the map
+            tma_store_4d(&tm_out, image, cc * 64, w0, h0, img);
             tma_store_commit();
         }
         __syncwarp();
@@ -412,8 +416,7 @@ GroupedPlan plan_grouped8(int n, int h_in, int w_in, int c, int ho, int wo, int 
                           bool with_dz = false) {
     GroupedPlan pl;
     (void)h_in; (void)w_in;
-    const int wt = wo + kw - 1;
-    if (wt > 256 || wt < 8 || kh * kw > 2 * kGMaxKSteps || c % 64) return pl;
+    if (kh * kw > 2 * kGMaxKSteps || c % 64) return pl;
     const int sms = device_sm_count();
     // The compute warps of one block (8, two per scheduler) cannot hide the ldmatrix -> MMA latency on their own, so
     // the bands are kept small enough for two or three blocks per SM, two stages each (a third stage costs blocks:
@@ -421,6 +424,13 @@ GroupedPlan plan_grouped8(int n, int h_in, int w_in, int c, int ho, int wo, int 
     // and its fixed cost, derated for how many blocks share the SM.  C = 256, 28 x 28, N = 64, forward: R = 2 20.9 us,
     // 3 23.6, 4 19.2, 5 23.8, 7 23.6, 10 27.4.
     double best = -1.0;
+    // Column strips of at most 64 keep several rows in a band of a wide image (a band is one TMA box of at most 256
+    // columns, and two stages of it have to fit).  The weight gradient takes none: its dZ band relies on zeros to the
+    // right of the image.  Narrow images are not cut: at 28 x 28, N = 64 two strips of 14 cost 64.7 us per forward +
+    // backward, none 61.6.
+    const int tiles_w = with_dz ? 1 : (wo + 63) / 64;
+    const int cols = (wo + tiles_w - 1) / tiles_w, wt = cols + kw - 1;
+    if (wt > 256 || wt < 8) return pl;
     for (int r = 1; r <= ho && r + kh - 1 <= 256; ++r) {
         const int rows_in = r + kh - 1;
         // stage = the box, plus what the last group of tiles reads past it
@@ -429,9 +439,9 @@ GroupedPlan plan_grouped8(int n, int h_in, int w_in, int c, int ho, int wo, int 
         size_t stride = (need * 128 + 1023) / 1024 * 1024;
         const size_t dz_off = stride;                          // the dZ band sits behind the X patch
         if (with_dz) stride += ((size_t)((r * wt + 15) / 16 * 16) * 128 + 1023) / 1024 * 1024;
-        const size_t out_bytes = with_dz ? 0 : ((size_t)(r * wo + 1) * 128 + 1023) / 1024 * 1024;
+        const size_t out_bytes = with_dz ? 0 : ((size_t)(r * cols + 1) * 128 + 1023) / 1024 * 1024;
         const int tiles_h = (ho + r - 1) / r;
-        const long long items = (long long)n * tiles_h * (c / 64);
+        const long long items = (long long)n * tiles_h * tiles_w * (c / 64);
         for (int stages = 2; stages <= 4; ++stages) {
             const size_t smem = 1024 + (size_t)stages * stride + out_bytes + sizeof(GroupedCtl);
             if (smem > 220 * 1024) break;
@@ -444,7 +454,8 @@ GroupedPlan plan_grouped8(int n, int h_in, int w_in, int c, int ho, int wo, int 
             if (best < 0 || cost < best) {
                 best = cost;
                 pl.ok = true;
-                pl.g.R = r; pl.g.Wt = wt; pl.g.rows_in = rows_in; pl.g.tiles_h = tiles_h; pl.g.stages = stages;
+                pl.g.R = r; pl.g.Wt = wt; pl.g.rows_in = rows_in; pl.g.tiles_h = tiles_h;
+                pl.g.cols = cols; pl.g.tiles_w = tiles_w; pl.g.stages = stages;
                 pl.g.patch_bytes = (uint32_t)((size_t)rows_in * wt * 128);
                 pl.g.stage_stride = (uint32_t)stride;
                 pl.g.out_bytes = (uint32_t)out_bytes;
@@ -490,7 +501,7 @@ static cudaError_t launch_grouped8(int n, int ha, int wa, int c, int ho, int wo,
                                              (unsigned long long)n};
         const unsigned long long ostr[4] = {0, (unsigned long long)c * 2, (unsigned long long)wo * c * 2,
                                             (unsigned long long)ho * wo * c * 2};
-        const unsigned int obox[4] = {64, (unsigned)wo, (unsigned)pl.g.R, 1};
+        const unsigned int obox[4] = {64, (unsigned)pl.g.cols, (unsigned)pl.g.R, 1};
         if (!make_tmap_tiled_bf16(&tout, out, 4, odims, ostr, obox)) return cudaErrorInvalidValue;
     }
     int *err = nullptr;

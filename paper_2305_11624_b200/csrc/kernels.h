@@ -65,9 +65,10 @@ struct BnFold {
     float eps;
     float *vec3;
 };
-// fold != NULL replaces `bias` (dense output mode only).
+// fold != NULL replaces `bias` (dense output mode only).  With out2 (Eval mode) out = wmat (*) act + fold->b and
+// out2 = gamma (out - mean) / sqrt(var + eps) + beta from the rounded out; nothing is written to fold->vec3.
 cudaError_t launch_umma_conv(const UmmaConvShape &s, const void *act, const void *wmat, const float *bias,
-                             void *out, cudaStream_t st, const BnFold *fold = nullptr);
+                             void *out, cudaStream_t st, const BnFold *fold = nullptr, void *out2 = nullptr);
 // Stride-1 multi-tap convolutions with the input patch staged once per tile (see umma_strip.cu): same
 // contract as launch_umma_conv (dense output mode, groups = 1).  Eligibility depends on the image size.
 bool umma_strip_eligible(const UmmaConvShape &s);
@@ -247,7 +248,7 @@ cudaError_t launch_wgrad_epilogue(const Problem &pb, int dtype, const float *par
 cudaError_t launch_bn_eval_fwd(const Problem &pb, int dtype, int layout, const void *y,
                                const float *vec3_eval /* [s | beta - mean s | r] */, void *z,
                                cudaStream_t st);
-// dy = s dz; part_g[split][c] = sum dz (y - mean) r; part_b[split][c] = sum dz
+// dy = s dz (dy == NULL: not wanted); part_g[split][c] = sum dz (y - mean) r; part_b[split][c] = sum dz
 cudaError_t launch_bn_eval_bwd(const Problem &pb, int dtype, int layout, const void *dz,
                                const void *y, const float *gamma, const float *mean,
                                const float *var, void *dy, float *part_g, float *part_b,
@@ -274,7 +275,7 @@ cudaError_t launch_selftest_wait_timeout(unsigned long long limit_ns, cudaStream
 // ---- TransposedConv-BN: pointwise pieces around the convolution kernels (tconv_kernels.cu) ---------------
 // Weights [C_in][taps][C_out/G] (nhwc) or [C_in][C_out/G][taps]; the scale belongs to the output channel
 // co = (ci / cig) cog + j.
-cudaError_t launch_tconv_vec3(int c_out, float eps, const float *b, const float *gamma, const float *beta,
+cudaError_t launch_bn_vec3(int c_out, float eps, const float *b, const float *gamma, const float *beta,
                               const float *mean, const float *var, float *vec3, cudaStream_t st);
 cudaError_t launch_tconv_rescale(int dtype, bool nhwc, long long count, int taps, int cig, int cog, const void *w,
                                  const float *s, void *w_out, cudaStream_t st);

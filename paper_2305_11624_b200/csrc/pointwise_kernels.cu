@@ -437,8 +437,9 @@ __global__ void __launch_bounds__(256) bn_eval_fwd_nhwc8_kernel(int c_out, long 
     }
 }
 
-// dy = s dz and per-block partial sums of dz (y - mean) r and dz, one partial row per block
-// (Table 2, Eval row); layout and block shape as above, lanes combined per channel in thread order.
+// dy = s dz (if dy != NULL) and per-block partial sums of dz (y - mean) r and dz, one partial row per block
+// (Table 2, Eval row); layout and block shape as above, lanes combined per channel in thread order.  Bound by the
+// reads: four vectors of each tensor are requested before the first is used.
 template <bool H>
 __global__ void __launch_bounds__(256) bn_eval_bwd_nhwc8_kernel(int c_out, long long p, int pix_per_block, float eps,
                                                                 const uint4 *__restrict__ dz,
@@ -449,6 +450,8 @@ __global__ void __launch_bounds__(256) bn_eval_bwd_nhwc8_kernel(int c_out, long 
                                                                 uint4 *__restrict__ dy, float *__restrict__ part_g,
                                                                 float *__restrict__ part_b) {
     __shared__ float red[256][9];
+    pdl_wait();
+    pdl_launch_dependents();
     const int v = c_out / 8, cv = threadIdx.x % v;
     float s8[8], r8[8], m8[8], ag[8], ab[8];
 #pragma unroll
@@ -462,22 +465,33 @@ __global__ void __launch_bounds__(256) bn_eval_bwd_nhwc8_kernel(int c_out, long 
     const long long vec0 = (long long)blockIdx.x * pix_per_block * v;
     long long vec1 = vec0 + (long long)pix_per_block * v;
     if (vec1 > p * v) vec1 = p * v;
-    for (long long i = vec0 + threadIdx.x; i < vec1; i += blockDim.x) {
-        const uint4 qd = dz[i], qy = y[i];
-        const uint32_t ud[4] = {qd.x, qd.y, qd.z, qd.w}, uy[4] = {qy.x, qy.y, qy.z, qy.w};
-        uint32_t o[4];
+    constexpr int U = 4;
+    for (long long i0 = vec0 + threadIdx.x; i0 < vec1; i0 += U * blockDim.x) {
+        uint4 qd[U], qy[U];
 #pragma unroll
-        for (int e = 0; e < 4; ++e) {
-            float d0, d1, y0, y1;
-            unpack2_t<H>(ud[e], d0, d1);
-            unpack2_t<H>(uy[e], y0, y1);
-            ag[2 * e] = fmaf(d0, (y0 - m8[2 * e]) * r8[2 * e], ag[2 * e]);
-            ag[2 * e + 1] = fmaf(d1, (y1 - m8[2 * e + 1]) * r8[2 * e + 1], ag[2 * e + 1]);
-            ab[2 * e] += d0;
-            ab[2 * e + 1] += d1;
-            o[e] = pack2_t<H>(s8[2 * e] * d0, s8[2 * e + 1] * d1);
+        for (int u = 0; u < U; ++u) {
+            const long long i = i0 + u * (int)blockDim.x;
+            qd[u] = i < vec1 ? dz[i] : make_uint4(0u, 0u, 0u, 0u);
+            qy[u] = i < vec1 ? y[i] : make_uint4(0u, 0u, 0u, 0u);
         }
-        dy[i] = make_uint4(o[0], o[1], o[2], o[3]);
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            const uint32_t ud[4] = {qd[u].x, qd[u].y, qd[u].z, qd[u].w}, uy[4] = {qy[u].x, qy[u].y, qy[u].z, qy[u].w};
+            uint32_t o[4];
+#pragma unroll
+            for (int e = 0; e < 4; ++e) {
+                float d0, d1, y0, y1;
+                unpack2_t<H>(ud[e], d0, d1);
+                unpack2_t<H>(uy[e], y0, y1);
+                ag[2 * e] = fmaf(d0, (y0 - m8[2 * e]) * r8[2 * e], ag[2 * e]);
+                ag[2 * e + 1] = fmaf(d1, (y1 - m8[2 * e + 1]) * r8[2 * e + 1], ag[2 * e + 1]);
+                ab[2 * e] += d0;
+                ab[2 * e + 1] += d1;
+                o[e] = pack2_t<H>(s8[2 * e] * d0, s8[2 * e + 1] * d1);
+            }
+            const long long i = i0 + u * (int)blockDim.x;
+            if (dy && i < vec1) dy[i] = make_uint4(o[0], o[1], o[2], o[3]);
+        }
     }
     for (int pass = 0; pass < 2; ++pass) {
 #pragma unroll
@@ -556,12 +570,10 @@ cudaError_t launch_bn_eval_bwd(const Problem &pb, int dtype, int layout, const v
         const int v = pb.c_out / 8, block = (256 / v) * v;
         const long long per = (pb.p + splits - 1) / splits;
         if (call_f16())
-            bn_eval_bwd_nhwc8_kernel<true><<<splits, block, 0, st>>>(pb.c_out, pb.p, (int)per, pb.eps, (const uint4 *)dz,
-                                                                     (const uint4 *)y, gamma, mean, var, (uint4 *)dy, part_g, part_b);
-        else
-            bn_eval_bwd_nhwc8_kernel<false><<<splits, block, 0, st>>>(pb.c_out, pb.p, (int)per, pb.eps, (const uint4 *)dz,
-                                                                      (const uint4 *)y, gamma, mean, var, (uint4 *)dy, part_g, part_b);
-        return cudaGetLastError();
+            return launch_pdl(bn_eval_bwd_nhwc8_kernel<true>, dim3(splits), dim3(block), 0, st, pb.c_out, pb.p, (int)per, pb.eps,
+                              (const uint4 *)dz, (const uint4 *)y, gamma, mean, var, (uint4 *)dy, part_g, part_b);
+        return launch_pdl(bn_eval_bwd_nhwc8_kernel<false>, dim3(splits), dim3(block), 0, st, pb.c_out, pb.p, (int)per, pb.eps,
+                          (const uint4 *)dz, (const uint4 *)y, gamma, mean, var, (uint4 *)dy, part_g, part_b);
     }
     const int threads = pb.c_out >= 256 ? 256 : ((pb.c_out + 31) / 32) * 32;
     dim3 grid((pb.c_out + threads - 1) / threads, splits);
@@ -582,29 +594,47 @@ cudaError_t launch_bn_eval_bwd(const Problem &pb, int dtype, int layout, const v
     return cudaGetLastError();
 }
 
-__global__ void bn_eval_finish_kernel(int c_out, float eps, const float *__restrict__ part_g,
-                                      const float *__restrict__ part_b, int splits,
-                                      const float *__restrict__ gamma, const float *__restrict__ var,
-                                      float *__restrict__ db, float *__restrict__ dgamma,
-                                      float *__restrict__ dbeta) {
-    const int c = blockIdx.x * blockDim.x + threadIdx.x;
-    if (c >= c_out) return;
+// 32 channels per block; warp g adds slices g, g + 32, ..., four of each array in flight, and the 32 groups are added in
+// order (one thread per channel walking up to 592 slices took 38 us).
+__global__ void __launch_bounds__(1024) bn_eval_finish_kernel(int c_out, float eps, const float *__restrict__ part_g,
+                                                              const float *__restrict__ part_b, int splits,
+                                                              const float *__restrict__ gamma, const float *__restrict__ var,
+                                                              float *__restrict__ db, float *__restrict__ dgamma,
+                                                              float *__restrict__ dbeta) {
+    __shared__ float red[2][32][33];
+    pdl_wait();
+    pdl_launch_dependents();
+    const int lane = threadIdx.x & 31, grp = threadIdx.x >> 5, c = blockIdx.x * 32 + lane;
     float g = 0.f, bsum = 0.f;
-    for (int sp = 0; sp < splits; ++sp) {
-        g += part_g[(long long)sp * c_out + c];
-        bsum += part_b[(long long)sp * c_out + c];
+    if (c < c_out)
+        for (int sp = grp; sp < splits; sp += 128) {
+            float vg[4], vb[4];
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+                const bool in = sp + 32 * u < splits;
+                vg[u] = in ? __ldcg(part_g + (long long)(sp + 32 * u) * c_out + c) : 0.f;
+                vb[u] = in ? __ldcg(part_b + (long long)(sp + 32 * u) * c_out + c) : 0.f;
+            }
+            g += (vg[0] + vg[1]) + (vg[2] + vg[3]);
+            bsum += (vb[0] + vb[1]) + (vb[2] + vb[3]);
+        }
+    red[0][grp][lane] = g;
+    red[1][grp][lane] = bsum;
+    __syncthreads();
+    if (grp == 0 && c < c_out) {
+        g = bsum = 0.f;
+        for (int i = 0; i < 32; ++i) { g += red[0][i][lane]; bsum += red[1][i][lane]; }
+        dgamma[c] = g;
+        dbeta[c] = bsum;
+        if (db) db[c] = gamma[c] / sqrtf(var[c] + eps) * bsum;
     }
-    dgamma[c] = g;
-    dbeta[c] = bsum;
-    if (db) db[c] = gamma[c] / sqrtf(var[c] + eps) * bsum;
 }
 
 cudaError_t launch_bn_eval_finish(const Problem &pb, const float *part_g, const float *part_b,
                                   int splits, const float *gamma, const float *var, float *db,
                                   float *dgamma, float *dbeta, cudaStream_t st) {
-    bn_eval_finish_kernel<<<(pb.c_out + 127) / 128, 128, 0, st>>>(pb.c_out, pb.eps, part_g, part_b, splits,
-                                                                 gamma, var, db, dgamma, dbeta);
-    return cudaGetLastError();
+    return launch_pdl(bn_eval_finish_kernel, dim3((pb.c_out + 31) / 32), dim3(1024), 0, st, pb.c_out, pb.eps, part_g, part_b,
+                      splits, gamma, var, db, dgamma, dbeta);
 }
 
 }  // namespace convbn

@@ -20,15 +20,17 @@ __device__ __forceinline__ int tconv_channel(long long idx, int taps, int cig, i
     return (ci / cig) * cog + j;
 }
 
-// vec3 = [s | b' | r]  (Sec. 3.3 definitions)
-__global__ void tconv_vec3_kernel(int c_out, float eps, const float *__restrict__ b, const float *__restrict__ gamma,
+// vec3 = [s | b' | r]  (Sec. 3.3 definitions; beta may be NULL where b' is not used)
+__global__ void bn_vec3_kernel(int c_out, float eps, const float *__restrict__ b, const float *__restrict__ gamma,
                                   const float *__restrict__ beta, const float *__restrict__ mean,
                                   const float *__restrict__ var, float *__restrict__ vec3) {
+    pdl_wait();
+    pdl_launch_dependents();
     const int c = blockIdx.x * blockDim.x + threadIdx.x;
     if (c >= c_out) return;
     const float r = 1.0f / sqrtf(var[c] + eps), s = gamma[c] * r;
     vec3[c] = s;
-    vec3[c_out + c] = ((b ? b[c] : 0.0f) - mean[c]) * s + beta[c];
+    vec3[c_out + c] = ((b ? b[c] : 0.0f) - mean[c]) * s + (beta ? beta[c] : 0.0f);
     vec3[2 * c_out + c] = r;
 }
 
@@ -101,10 +103,9 @@ int grid_for(long long count) {
 
 }  // namespace
 
-cudaError_t launch_tconv_vec3(int c_out, float eps, const float *b, const float *gamma, const float *beta,
+cudaError_t launch_bn_vec3(int c_out, float eps, const float *b, const float *gamma, const float *beta,
                               const float *mean, const float *var, float *vec3, cudaStream_t st) {
-    tconv_vec3_kernel<<<(c_out + 127) / 128, 128, 0, st>>>(c_out, eps, b, gamma, beta, mean, var, vec3);
-    return cudaGetLastError();
+    return launch_pdl(bn_vec3_kernel, dim3((c_out + 127) / 128), dim3(128), 0, st, c_out, eps, b, gamma, beta, mean, var, vec3);
 }
 
 cudaError_t launch_tconv_rescale(int dtype, bool nhwc, long long count, int taps, int cig, int cog, const void *w,

@@ -49,6 +49,9 @@ struct ConvGemm {
     int resident;            // 1: the CTA's whole weight slab [BN][K] stays in shared memory (loaded once)
     int f16;                 // 16-bit storage type: 0 bf16, 1 IEEE half
     BnFold fold;             // fold.gamma != NULL: scale and shift formed in the kernel from the BN parameters
+    // 1 (Eval mode, dense stores): Y = acc + fold.b goes to tm_out and Z = s Y + (beta - mean s), from the rounded Y,
+    // to tm_out2.  A pass of its own re-read Y: conv + pass took 37 us for the 64 -> 256 layer at 56 x 56, N = 32.
+    int dual;
 };
 
 struct ConvSmemCtl {
@@ -69,6 +72,7 @@ template <int BN>
 __global__ void __launch_bounds__(kConvThreads) umma_conv_kernel(const __grid_constant__ CUtensorMap tm_act,
                                                                 const __grid_constant__ CUtensorMap tm_w,
                                                                 const __grid_constant__ CUtensorMap tm_out,
+                                                                const __grid_constant__ CUtensorMap tm_out2,
                                                                 const ConvGemm g, const float *__restrict__ bias,
                                                                 int *err) {
     extern __shared__ uint8_t smem_raw[];
@@ -83,6 +87,7 @@ __global__ void __launch_bounds__(kConvThreads) umma_conv_kernel(const __grid_co
     ConvSmemCtl *ctl = (ConvSmemCtl *)(staging + kStagingBytes);
     float *bias_s = (float *)(((uintptr_t)(ctl + 1) + 15) & ~(uintptr_t)15);   // cn floats
     float *scale_s = bias_s + g.cn;                                            // cn floats (fold mode)
+    float *shift_s = scale_s + g.cn;                                           // cn floats (dual mode)
     const bool fold = g.fold.gamma != nullptr;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int stages = g.stages;
@@ -123,7 +128,14 @@ __global__ void __launch_bounds__(kConvThreads) umma_conv_kernel(const __grid_co
     if (threadIdx.x == 0) { prefetch_tensormap(&tm_act); prefetch_tensormap(&tm_w); prefetch_tensormap(&tm_out); }
     pdl_wait();
     if (threadIdx.x == 0) CONVBN_TRACE_POINT(1);
-    if (fold) {
+    if (g.dual) {
+        for (int c = threadIdx.x; c < g.cn; c += kConvThreads) {
+            const float sc = g.fold.gamma[c] * (1.0f / sqrtf(g.fold.var[c] + g.fold.eps));
+            bias_s[c] = g.fold.b ? g.fold.b[c] : 0.f;
+            scale_s[c] = sc;
+            shift_s[c] = g.fold.beta[c] - g.fold.mean[c] * sc;
+        }
+    } else if (fold) {
         // On-the-fly reparameterisation (Sec. 3.3 / 3.4): s = gamma / sqrt(var + eps), b' = (b - mu) s + beta.
         // s multiplies the fp32 accumulator (the associative law of Sec. 3.2.2), so omega is used unrounded.
         for (int c = threadIdx.x; c < g.cn; c += kConvThreads) {
@@ -326,7 +338,7 @@ __global__ void __launch_bounds__(kConvThreads) umma_conv_kernel(const __grid_co
                             float f[8];
     #pragma unroll
                             for (int e = 0; e < 8; ++e) f[e] = __uint_as_float(v[j + e]);
-                            if (fold) {
+                            if (fold && !g.dual) {
                                 const float4 s0 = *(const float4 *)(scale_s + n0 + c0 + j);
                                 const float4 s1 = *(const float4 *)(scale_s + n0 + c0 + j + 4);
                                 f[0] *= s0.x; f[1] *= s0.y; f[2] *= s0.z; f[3] *= s0.w;
@@ -360,6 +372,38 @@ __global__ void __launch_bounds__(kConvThreads) umma_conv_kernel(const __grid_co
                             tma_store_2d(&tm_out, buf, n0 + c0, (int)(m0 + quarter * 32));
                         }
                         tma_store_commit();
+                    }
+                    if (g.dual) {
+                        uint4 zq[8];
+                        auto normalise = [&](auto half_tag) {
+                            constexpr bool H = decltype(half_tag)::value;
+#pragma unroll
+                            for (int j = 0; j < 8; ++j) {
+                                const uint4 q = *(const uint4 *)(row + (((j ^ (lane & 7)) & 7) << 4));
+                                const uint32_t u[4] = {q.x, q.y, q.z, q.w};
+                                uint32_t o[4];
+#pragma unroll
+                                for (int e = 0; e < 4; ++e) {
+                                    const float2 sc = *(const float2 *)(scale_s + n0 + c0 + j * 8 + 2 * e);
+                                    const float2 sh = *(const float2 *)(shift_s + n0 + c0 + j * 8 + 2 * e);
+                                    float lo, hi2;
+                                    unpack2_t<H>(u[e], lo, hi2);
+                                    o[e] = pack2_t<H>(fmaf(sc.x, lo, sh.x), fmaf(sc.y, hi2, sh.y));
+                                }
+                                zq[j] = make_uint4(o[0], o[1], o[2], o[3]);
+                            }
+                        };
+                        if (g.f16) normalise(std::true_type{}); else normalise(std::false_type{});
+                        if (lane == 0) tma_store_wait_read<0>();
+                        __syncwarp();
+#pragma unroll
+                        for (int j = 0; j < 8; ++j) *(uint4 *)(row + (((j ^ (lane & 7)) & 7) << 4)) = zq[j];
+                        fence_proxy_async_smem();
+                        __syncwarp();
+                        if (lane == 0) {
+                            tma_store_2d(&tm_out2, buf, n0 + c0, (int)(m0 + quarter * 32));
+                            tma_store_commit();
+                        }
                     }
                 }
             }
@@ -489,10 +533,10 @@ bool umma_conv_eligible(const UmmaConvShape &s) {
 static int sm_count() { return device_sm_count(); }
 
 template <int BN>
-static cudaError_t launch_bn(const CUtensorMap &ta, const CUtensorMap &tw, const CUtensorMap &tout, ConvGemm g,
-                             const float *bias, int *err, cudaStream_t st) {
+static cudaError_t launch_bn(const CUtensorMap &ta, const CUtensorMap &tw, const CUtensorMap &tout,
+                             const CUtensorMap &tout2, ConvGemm g, const float *bias, int *err, cudaStream_t st) {
     const size_t a_bytes = (size_t)kBM * kBK * 2, b_bytes = (size_t)BN * kBK * 2;
-    size_t fixed = 1024 + kStagingBytes + sizeof(ConvSmemCtl) + 2 * (size_t)g.cn * sizeof(float) + 16;
+    size_t fixed = 1024 + kStagingBytes + sizeof(ConvSmemCtl) + (g.dual ? 3 : 2) * (size_t)g.cn * sizeof(float) + 16;
     const int num_kb = g.taps_h * g.taps_w * (g.blockdiag ? 1 : g.ca / kBK);
     const long long m_tiles = (g.p + kBM - 1) / kBM, n_tiles = (g.cn + BN - 1) / BN;
     long long grid_l = m_tiles * n_tiles < sm_count() ? m_tiles * n_tiles : sm_count();
@@ -516,7 +560,7 @@ static cudaError_t launch_bn(const CUtensorMap &ta, const CUtensorMap &tw, const
     static PerDevice carve;
     prefer_max_shared_once(umma_conv_kernel<BN>, &carve);
     const unsigned grid = (unsigned)grid_l;
-    return launch_pdl(umma_conv_kernel<BN>, dim3(grid), dim3(kConvThreads), smem, st, ta, tw, tout, g, bias, err);
+    return launch_pdl(umma_conv_kernel<BN>, dim3(grid), dim3(kConvThreads), smem, st, ta, tw, tout, tout2, g, bias, err);
 }
 
 // Tile width: fewest rounds of tiles over the SMs, weighted by the time of one tile (N = 64 tiles are
@@ -537,8 +581,9 @@ static int pick_bn(long long tiles_m, int cn) {
 }
 
 cudaError_t launch_umma_conv(const UmmaConvShape &s, const void *act, const void *wmat, const float *bias,
-                             void *out, cudaStream_t st, const BnFold *fold) {
+                             void *out, cudaStream_t st, const BnFold *fold, void *out2) {
     ConvGemm g;
+    g.dual = out2 ? 1 : 0;
     g.ho = s.ho; g.wo = s.wo; g.cn = s.cn; g.ca = s.ca; g.taps_h = s.taps_h; g.taps_w = s.taps_w;
     g.lower_h = s.lower_h; g.lower_w = s.lower_w; g.stride_h = s.stride_h; g.stride_w = s.stride_w;
     g.dil_h = s.dil_h; g.dil_w = s.dil_w; g.p = (long long)s.n * s.ho * s.wo; g.stages = 1;
@@ -564,9 +609,11 @@ cudaError_t launch_umma_conv(const UmmaConvShape &s, const void *act, const void
     int *err = nullptr;
     cudaError_t e = error_word_address(&err);
     if (e != cudaSuccess) return e;
-    if (bn == 64) return launch_bn<64>(ta, tw, tout, g, bias, err, st);
-    if (bn == 128) return launch_bn<128>(ta, tw, tout, g, bias, err, st);
-    return launch_bn<256>(ta, tw, tout, g, bias, err, st);
+    CUtensorMap tout2 = tout;
+    if (out2 && !make_tmap_matrix_bf16(&tout2, out2, g.p, s.cn, 32, 64)) return cudaErrorInvalidValue;
+    if (bn == 64) return launch_bn<64>(ta, tw, tout, tout2, g, bias, err, st);
+    if (bn == 128) return launch_bn<128>(ta, tw, tout, tout2, g, bias, err, st);
+    return launch_bn<256>(ta, tw, tout, tout2, g, bias, err, st);
 }
 
 // Forward pass of a small-C_in layer on the packed input (see stem_kernels.cu): tiles of 8 x 16 output
@@ -575,6 +622,7 @@ cudaError_t launch_stem_fwd(const Problem &pb, const void *x_packed, const void 
                             cudaStream_t st, const BnFold *fold) {
     const int krows = stem_krows(pb);
     ConvGemm g;
+    g.dual = 0;
     g.ho = pb.h_out; g.wo = pb.w_out; g.cn = pb.c_out; g.ca = 64; g.taps_h = krows; g.taps_w = 1;
     g.lower_h = g.lower_w = 0; g.stride_h = g.stride_w = g.dil_h = g.dil_w = 1;
     g.stem = 1; g.stem_tw = 16; g.stem_th = 8;
@@ -605,7 +653,7 @@ cudaError_t launch_stem_fwd(const Problem &pb, const void *x_packed, const void 
     int *err = nullptr;
     cudaError_t e = error_word_address(&err);
     if (e != cudaSuccess) return e;
-    return launch_bn<64>(ta, tw, tout, g, bias, err, st);
+    return launch_bn<64>(ta, tw, tout, tout, g, bias, err, st);
 }
 
 }  // namespace convbn
