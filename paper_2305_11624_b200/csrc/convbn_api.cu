@@ -1139,7 +1139,7 @@ struct TconvView {
     Problem pb;                // and its problem
     int h_out, w_out;          // output extent of the transposed layer
     size_t wcount;             // weight elements
-    size_t off_w, off_zero, off_dwp, off_bsum, off_inner, total;
+    size_t off_w, off_count, off_dwp, off_bsum, off_fwd, off_bwd, total;   // off_fwd / off_bwd: the inner plans' regions
     int bsplits;
     Problem sum_pb;            // a 1x1 problem whose output is the transposed layer's output (for the channel sums)
     Plan fwd, bwd;             // plans of the inner convolution: plain forward, plain backward
@@ -1171,12 +1171,26 @@ int tconv_view(const convbn_desc *d, TconvView *v) {
     size_t off = 0;
     auto take = [&](size_t bytes) { const size_t at0 = off; off += (bytes + 255) / 256 * 256; return at0; };
     v->off_w = take(v->wcount * elem_size(d->dtype));
-    v->off_zero = take((size_t)d->c_in * sizeof(float));
+    v->off_count = take((size_t)(d->c_out / 32 + 1) * sizeof(unsigned int));
     v->off_dwp = take(v->wcount * sizeof(float));
     v->off_bsum = take((size_t)v->bsplits * d->c_out * sizeof(float));
-    v->off_inner = off;
-    v->total = off + (v->fwd.total > v->bwd.total ? v->fwd.total : v->bwd.total);
+    v->off_fwd = take(v->fwd.total);
+    v->off_bwd = take(v->bwd.total);
+    v->total = off;
     return CONVBN_OK;
+}
+
+// The forward pass as one GEMM [input pixels][C_in] x [C_in][taps C_out]: kernel = stride, no padding, no dilation.
+bool tconv_gemm_shape(const convbn_desc *d, const TconvView &v, UmmaConvShape *s) {
+    if (d->dtype != CONVBN_BF16 || d->layout != CONVBN_NHWC || d->groups != 1 || d->kh != d->stride_h || d->kw != d->stride_w ||
+        d->pad_h || d->pad_w || d->dil_h != 1 || d->dil_w != 1 || d->c_out % 64 || d->kh * d->kw * (long long)d->c_out > 4096)
+        return false;
+    *s = UmmaConvShape{d->n, d->h_in, d->w_in, d->c_in, d->h_in, d->w_in, d->kh * d->kw * d->c_out, 1, 1, 0, 0, 1, 1, 1, 1, 0};
+    const long long row = (long long)v.w_out * d->c_out;
+    if (row * d->kh > (1LL << 30)) return false;
+    s->out_sn = row * v.h_out; s->out_sh = (int)(row * d->kh); s->out_sw = d->kw * d->c_out;
+    s->tap_c = d->c_out; s->tap_kw = d->kw; s->tap_sh = (int)row; s->tap_sw = d->c_out;
+    return umma_conv_eligible(*s);
 }
 
 // An IEEE-half transposed layer runs as its bf16 twin: `twin` receives the descriptor to use from here on and
@@ -1229,8 +1243,15 @@ int convbn_tconv_tune_fwd(const convbn_desc *desc, const void *x, const void *w,
     const bool nhwc = desc->layout == CONVBN_NHWC;
     const int taps = desc->kh * desc->kw, cig = desc->c_in / desc->groups, cog = desc->c_out / desc->groups;
     float *vec3 = (float *)saved;
-    void *wf = at(workspace, v.off_w), *inner = at(workspace, v.off_inner);
-    LAUNCH("tconv_vec3", launch_bn_vec3(desc->c_out, (float)desc->eps, b, gamma, beta, run_mean, run_var, vec3, st));
+    void *wf = at(workspace, v.off_w), *inner = at(workspace, v.off_bwd);
+    UmmaConvShape us;
+    if (tconv_gemm_shape(desc, v, &us)) {
+        // kernel = stride: no two taps meet, Z is one GEMM on omega as it is, s and b' in its epilogue
+        const BnFold fold{gamma, beta, run_mean, run_var, b, (float)desc->eps, vec3};
+        LAUNCH("tconv_gemm", launch_umma_conv(us, x, w, nullptr, z, st, &fold));
+        return CONVBN_OK;
+    }
+    LAUNCH("bn_vec3", launch_bn_vec3(desc->c_out, (float)desc->eps, b, gamma, beta, run_mean, run_var, vec3, st));
     LAUNCH("tconv_rescale", launch_tconv_rescale(desc->dtype, nhwc, (long long)v.wcount, taps, cig, cog, w, vec3, wf, st));
     // Z = omega' scattered over X: the backward-data pass of the convolution with the same weights
     const char *which = nullptr;
@@ -1266,22 +1287,38 @@ int convbn_tconv_tune_bwd(const convbn_desc *desc, const void *dz, const void *x
     const bool nhwc = desc->layout == CONVBN_NHWC;
     const int taps = desc->kh * desc->kw, cig = desc->c_in / desc->groups, cog = desc->c_out / desc->groups;
     const float *vec3 = (const float *)saved;
-    void *wf = at(workspace, v.off_w), *inner = at(workspace, v.off_inner);
-    float *zero = (float *)at(workspace, v.off_zero), *dwp = (float *)at(workspace, v.off_dwp);
-    float *bsum = (float *)at(workspace, v.off_bsum);
-    // omega' is re-formed from omega and the saved scale (Sec. 3.4: Tune mode keeps X and a few vectors)
-    LAUNCH("tconv_rescale", launch_tconv_rescale(desc->dtype, nhwc, (long long)v.wcount, taps, cig, cog, w, vec3, wf, st));
-    CU(cudaMemsetAsync(zero, 0, (size_t)desc->c_in * sizeof(float), st));
-    // dX gathers dZ through omega': the forward pass of that convolution, without a bias
-    const char *which = nullptr;
-    CK(run_conv_fwd(&v.conv, v.pb, dz, wf, zero, dx, v.fwd, inner, st, &which));
-    // domega' contracts X with windows of dZ: that convolution's weight gradient with the two tensors exchanged
-    CK(run_param_grads(&v.conv, v.pb, v.bwd, x, dz, wf, nullptr, nullptr, nullptr, dwp, nullptr, nullptr, nullptr, inner,
-                       st, &which));
-    LAUNCH("channel_sum", launch_channel_sum_partial(v.sum_pb, desc->dtype, desc->layout, dz, bsum, v.bsplits, st));
-    LAUNCH("tconv_epilogue", launch_tconv_param_epilogue(desc->dtype, nhwc, desc->c_out, taps, cig, cog, dwp, w, vec3, b,
-                                                         run_mean, bsum, v.bsplits, dw, db, dgamma, dbeta, st));
-    return CONVBN_OK;
+    void *wf = at(workspace, v.off_w), *inner = at(workspace, v.off_fwd), *inner_b = at(workspace, v.off_bwd);
+    float *dwp = (float *)at(workspace, v.off_dwp), *bsum = (float *)at(workspace, v.off_bsum);
+    unsigned int *counters = (unsigned int *)at(workspace, v.off_count);
+    // dX gathers dZ through omega' (re-formed from omega and the saved scale, Sec. 3.4): the forward pass of that
+    // convolution, without a bias.  domega' contracts X with windows of dZ: that convolution's weight gradient with the
+    // two tensors exchanged.  The two passes share nothing they write and run side by side.
+    return side_by_side(
+        st,
+        [&](cudaStream_t st) -> int {
+            const char *which = nullptr;
+            LAUNCH("channel_sum", launch_channel_sum_partial(v.sum_pb, desc->dtype, desc->layout, dz, bsum, v.bsplits, st));
+            if (v.bwd.umma_wgrad) {
+                float *partials = (float *)at(inner_b, v.bwd.partials);
+                // (the GEMM's own sums, of X here, are not needed)
+                LAUNCH("umma_wgrad", launch_umma_wgrad(v.pb, v.bwd.uw, x, dz, partials, (float *)at(inner_b, v.bwd.bsum), counters,
+                                                       st, desc->c_out / 32));
+                LAUNCH("tconv_epilogue", launch_tconv_wgrad_epilogue(desc->c_in, desc->c_out, taps, partials, v.bwd.uw.splits, w,
+                                                                     vec3, b, run_mean, bsum, v.bsplits, dwp, counters, dw, db,
+                                                                     dgamma, dbeta, st));
+                return CONVBN_OK;
+            }
+            CK(run_param_grads(&v.conv, v.pb, v.bwd, x, dz, w, nullptr, nullptr, nullptr, dwp, nullptr, nullptr, nullptr, inner_b,
+                               st, &which));
+            LAUNCH("tconv_epilogue", launch_tconv_param_epilogue(desc->dtype, nhwc, desc->c_out, taps, cig, cog, dwp, w, vec3, b,
+                                                                 run_mean, bsum, v.bsplits, dw, db, dgamma, dbeta, st));
+            return CONVBN_OK;
+        },
+        [&]() -> int {
+            const char *which = nullptr;
+            LAUNCH("tconv_rescale", launch_tconv_rescale(desc->dtype, nhwc, (long long)v.wcount, taps, cig, cog, w, vec3, wf, st));
+            return run_conv_fwd(&v.conv, v.pb, dz, wf, nullptr, dx, v.fwd, inner, st, &which);
+        });
 }
 
 int convbn_check(void *stream) {

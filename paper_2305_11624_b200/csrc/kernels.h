@@ -42,10 +42,13 @@ struct UmmaConvShape {
     // 1: grouped convolution run as a block-diagonal GEMM: output channels [64 b, 64 b + 64) read only
     // activation channels [64 b, 64 b + 64) and wmat is [cn][taps * 64] (zeros outside a channel's group).
     int blockdiag = 0;
-    // Strided output, used when out_sw != 0 (no bias in this mode): output pixel (n, i, j) is written at
+    // Strided output, used when out_sw != 0: output pixel (n, i, j) is written at
     // out + n out_sn + i out_sh + j out_sw (elements) instead of densely.
     long long out_sn = 0;
     int out_sh = 0, out_sw = 0;
+    // Transposed convolution with kernel = stride: see ConvGemm in umma_conv.cu.  Needs the strided output, 1 x 1 "taps"
+    // here, tap_c a multiple of 64 and cn = kh kw tap_c; wmat is the layer's weight tensor [ca][kh kw tap_c].
+    int tap_c = 0, tap_kw = 0, tap_sh = 0, tap_sw = 0;
     // Sub-pixel output (stride-2 backward data of a layer with at most 4 input channels, strip kernel only,
     // cn = 16): output "pixel" (n, i, j) holds the 2 x 2 input positions (2 i + a, 2 j + b); GEMM column
     // 8 a + b sub_cin + ci is written to out[n][2 i + a][2 j + b][ci] of a [n][sub_hin][sub_win][sub_cin]
@@ -115,9 +118,9 @@ bool umma_wgrad_eligible(const Problem &pb);
 UmmaWgradPlan umma_wgrad_plan(const Problem &pb);
 // partials: [splits][kdim][C_out] fp32 (k-major: the transpose of the weight layout)
 // bsum    : [splits][C_out] fp32 per-slice sums of dZ over pixels (from a ones row in the GEMM)
-// counters: C_out / 32 words zeroed for the fused epilogue (may be NULL)
+// counters: C_out / 32 words (or `ncounters`) zeroed for the fused epilogue (may be NULL)
 cudaError_t launch_umma_wgrad(const Problem &pb, const UmmaWgradPlan &pl, const void *dz, const void *x,
-                              float *partials, float *bsum, unsigned int *counters, cudaStream_t st);
+                              float *partials, float *bsum, unsigned int *counters, cudaStream_t st, int ncounters = -1);
 // Everything after the GEMM in one kernel: dw[co][k] = scale[co] * sum_splits partials (scale = first
 // C_out floats of vec3, 1 if NULL); with need_sums also dbeta, db, dgamma (vec3 given) or db = sum dZ.
 // dotpart: [kt][C_out] scratch; counters: C_out / 32 zeroed words.
@@ -281,6 +284,13 @@ cudaError_t launch_tconv_rescale(int dtype, bool nhwc, long long count, int taps
                                  const float *s, void *w_out, cudaStream_t st);
 cudaError_t launch_tconv_bias(int dtype, bool nhwc, long long count, int c, long long hw, const float *bias, void *z,
                               cudaStream_t st);
+// The same from the weight-gradient GEMM's partial tiles [splits][taps C_out][C_in] (groups = 1, NHWC, channels multiples
+// of 64): adds them, transposes, scales and finishes the per-channel gradients in one kernel.  dotpart: [C_in / 32][taps
+// C_out] scratch, counters: C_out / 32 zeroed words, bsum: [bsplits][C_out].
+cudaError_t launch_tconv_wgrad_epilogue(int c_in, int c_out, int taps, const float *part, int splits, const void *w,
+                                        const float *vec3, const float *b, const float *mean, const float *bsum,
+                                        int bsplits, float *dotpart, unsigned int *counters, float *dw, float *db,
+                                        float *dgamma, float *dbeta, cudaStream_t st);
 // dwp: fp32 domega' in the weight layout; bsum: [bsplits][C_out] partial sums of dZ
 cudaError_t launch_tconv_param_epilogue(int dtype, bool nhwc, int c_out, int taps, int cig, int cog, const float *dwp,
                                         const void *w, const float *vec3, const float *b, const float *mean,

@@ -440,7 +440,7 @@ __global__ void __launch_bounds__(256) bn_eval_fwd_nhwc8_kernel(int c_out, long 
 // dy = s dz (if dy != NULL) and per-block partial sums of dz (y - mean) r and dz, one partial row per block
 // (Table 2, Eval row); layout and block shape as above, lanes combined per channel in thread order.  Bound by the
 // reads: four vectors of each tensor are requested before the first is used.
-template <bool H>
+template <bool H, bool DY>
 __global__ void __launch_bounds__(256) bn_eval_bwd_nhwc8_kernel(int c_out, long long p, int pix_per_block, float eps,
                                                                 const uint4 *__restrict__ dz,
                                                                 const uint4 *__restrict__ y,
@@ -453,12 +453,11 @@ __global__ void __launch_bounds__(256) bn_eval_bwd_nhwc8_kernel(int c_out, long 
     pdl_wait();
     pdl_launch_dependents();
     const int v = c_out / 8, cv = threadIdx.x % v;
-    float s8[8], r8[8], m8[8], ag[8], ab[8];
+    float s8[8], m8[8], ag[8], ab[8];
 #pragma unroll
     for (int e = 0; e < 8; ++e) {
         const int c = cv * 8 + e;
-        r8[e] = 1.0f / sqrtf(var[c] + eps);
-        s8[e] = gamma[c] * r8[e];
+        if constexpr (DY) s8[e] = gamma[c] * (1.0f / sqrtf(var[c] + eps));
         m8[e] = mean[c];
         ag[e] = ab[e] = 0.f;
     }
@@ -483,14 +482,14 @@ __global__ void __launch_bounds__(256) bn_eval_bwd_nhwc8_kernel(int c_out, long 
                 float d0, d1, y0, y1;
                 unpack2_t<H>(ud[e], d0, d1);
                 unpack2_t<H>(uy[e], y0, y1);
-                ag[2 * e] = fmaf(d0, (y0 - m8[2 * e]) * r8[2 * e], ag[2 * e]);
-                ag[2 * e + 1] = fmaf(d1, (y1 - m8[2 * e + 1]) * r8[2 * e + 1], ag[2 * e + 1]);
+                ag[2 * e] = fmaf(d0, y0 - m8[2 * e], ag[2 * e]);
+                ag[2 * e + 1] = fmaf(d1, y1 - m8[2 * e + 1], ag[2 * e + 1]);
                 ab[2 * e] += d0;
                 ab[2 * e + 1] += d1;
-                o[e] = pack2_t<H>(s8[2 * e] * d0, s8[2 * e + 1] * d1);
+                if constexpr (DY) o[e] = pack2_t<H>(s8[2 * e] * d0, s8[2 * e + 1] * d1);
             }
             const long long i = i0 + u * (int)blockDim.x;
-            if (dy && i < vec1) dy[i] = make_uint4(o[0], o[1], o[2], o[3]);
+            if (DY && i < vec1) dy[i] = make_uint4(o[0], o[1], o[2], o[3]);
         }
     }
     for (int pass = 0; pass < 2; ++pass) {
@@ -501,6 +500,7 @@ __global__ void __launch_bounds__(256) bn_eval_bwd_nhwc8_kernel(int c_out, long 
             const int g = c / 8, e = c % 8;
             float sum = 0.f;
             for (int th = g; th < (int)blockDim.x; th += v) sum += red[th][e];
+            if (!pass) sum *= 1.0f / sqrtf(var[c] + eps);          // r
             (pass ? part_b : part_g)[(long long)blockIdx.x * c_out + c] = sum;
         }
         __syncthreads();
@@ -569,10 +569,9 @@ cudaError_t launch_bn_eval_bwd(const Problem &pb, int dtype, int layout, const v
     if (channel_sum_fast(pb, dtype, layout)) {
         const int v = pb.c_out / 8, block = (256 / v) * v;
         const long long per = (pb.p + splits - 1) / splits;
-        if (call_f16())
-            return launch_pdl(bn_eval_bwd_nhwc8_kernel<true>, dim3(splits), dim3(block), 0, st, pb.c_out, pb.p, (int)per, pb.eps,
-                              (const uint4 *)dz, (const uint4 *)y, gamma, mean, var, (uint4 *)dy, part_g, part_b);
-        return launch_pdl(bn_eval_bwd_nhwc8_kernel<false>, dim3(splits), dim3(block), 0, st, pb.c_out, pb.p, (int)per, pb.eps,
+        auto kern = call_f16() ? (dy ? bn_eval_bwd_nhwc8_kernel<true, true> : bn_eval_bwd_nhwc8_kernel<true, false>)
+                               : (dy ? bn_eval_bwd_nhwc8_kernel<false, true> : bn_eval_bwd_nhwc8_kernel<false, false>);
+        return launch_pdl(kern, dim3(splits), dim3(block), 0, st, pb.c_out, pb.p, (int)per, pb.eps,
                           (const uint4 *)dz, (const uint4 *)y, gamma, mean, var, (uint4 *)dy, part_g, part_b);
     }
     const int threads = pb.c_out >= 256 ? 256 : ((pb.c_out + 31) / 32) * 32;

@@ -94,6 +94,83 @@ __global__ void __launch_bounds__(256) tconv_param_epilogue_kernel(int c_out, in
     }
 }
 
+// Block (bx, by): input channels [32 bx, +32) x weight rows k = (tap, co) [32 by, +32), one output channel group since
+// 32 divides C_out.  Thread (tx = ci, ty = k) adds its element over the slices, eight loads in flight, in slice order;
+// the tile is transposed through shared memory, scaled by s[co] and stored along k.  The last block of a group of 32
+// output channels (a counter) adds the dot products and the sums of dZ in fixed order.  Bound by the read of the
+// partials (L2): 256 -> 128 channels, 2 x 2, 29 slices: 15 MB; with the transposition, the scale and the per-channel
+// sums in kernels of their own the same work took 87 us.
+__global__ void __launch_bounds__(1024) tconv_wgrad_epilogue_kernel(int c_in, int c_out, int kdim, const float *__restrict__ part,
+                                                                    int splits, const __nv_bfloat16 *__restrict__ w,
+                                                                    const float *__restrict__ vec3, const float *__restrict__ b,
+                                                                    const float *__restrict__ mean, const float *__restrict__ bsum,
+                                                                    int bsplits, float *__restrict__ dotpart,
+                                                                    unsigned int *__restrict__ counters, float *__restrict__ dw,
+                                                                    float *__restrict__ db, float *__restrict__ dgamma,
+                                                                    float *__restrict__ dbeta, int f16) {
+    __shared__ float tile[32][33], prod[32][33];
+    __shared__ int is_last;
+    pdl_wait();
+    pdl_launch_dependents();
+    const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
+    const int ci0 = blockIdx.x * 32, k0 = blockIdx.y * 32, co0 = k0 % c_out;
+    const float wv = load_h16(w + (size_t)(ci0 + ty) * kdim + k0 + tx, f16);
+    {
+        const float *src = part + (size_t)(k0 + ty) * c_in + ci0 + tx;
+        const size_t slice = (size_t)kdim * c_in;
+        float acc = 0.f;
+        for (int sp = 0; sp < splits; sp += 8) {
+            float v[8];
+#pragma unroll
+            for (int u = 0; u < 8; ++u) v[u] = sp + u < splits ? __ldcg(src + (size_t)(sp + u) * slice) : 0.f;
+#pragma unroll
+            for (int u = 0; u < 8; ++u) acc += v[u];
+        }
+        tile[ty][tx] = acc;
+    }
+    __syncthreads();
+    const float v = tile[tx][ty];                       // (ci = ty, k = tx) from here on
+    dw[(size_t)(ci0 + ty) * kdim + k0 + tx] = vec3[co0 + tx] * v;
+    prod[ty][tx] = v * wv;
+    __syncthreads();
+    {
+        float d = prod[tx][ty];                         // warp ty adds the 32 input channels of row k0 + ty
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) d += __shfl_xor_sync(0xffffffffu, d, o);
+        if (tx == 0) dotpart[(size_t)blockIdx.x * kdim + k0 + ty] = d;
+    }
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        __threadfence();
+        const unsigned int per_group = gridDim.x * (unsigned)(kdim / c_out);
+        is_last = atomicAdd(&counters[co0 / 32], 1u) == per_group - 1;
+    }
+    __syncthreads();
+    if (!is_last) return;
+    __threadfence();
+    // thread (tx = channel, ty = row group): rows of dotpart are (input-channel block, tap), then the slices of sum dZ
+    float d = 0.f, sum = 0.f;
+    const int taps = kdim / c_out, rows = (int)gridDim.x * taps;
+    for (int r = ty; r < rows; r += 32) d += __ldcg(dotpart + (size_t)(r / taps) * kdim + (r % taps) * c_out + co0 + tx);
+    for (int sp = ty; sp < bsplits; sp += 128) {
+        float q[4];
+#pragma unroll
+        for (int u = 0; u < 4; ++u) q[u] = sp + 32 * u < bsplits ? __ldcg(bsum + (size_t)(sp + 32 * u) * c_out + co0 + tx) : 0.f;
+        sum += (q[0] + q[1]) + (q[2] + q[3]);
+    }
+    tile[ty][tx] = d;
+    prod[ty][tx] = sum;
+    __syncthreads();
+    if (ty == 0) {
+        const int co = co0 + tx;
+        d = sum = 0.f;
+        for (int i = 0; i < 32; ++i) { d += tile[i][tx]; sum += prod[i][tx]; }
+        dbeta[co] = sum;
+        if (db) db[co] = vec3[co] * sum;
+        dgamma[co] = vec3[2 * c_out + co] * (d + sum * ((b ? b[co] : 0.0f) - mean[co]));
+    }
+}
+
 int grid_for(long long count) {
     long long blocks = (count + 255) / 256;
     const long long cap = (long long)device_sm_count() * 16;
@@ -106,6 +183,17 @@ int grid_for(long long count) {
 cudaError_t launch_bn_vec3(int c_out, float eps, const float *b, const float *gamma, const float *beta,
                               const float *mean, const float *var, float *vec3, cudaStream_t st) {
     return launch_pdl(bn_vec3_kernel, dim3((c_out + 127) / 128), dim3(128), 0, st, c_out, eps, b, gamma, beta, mean, var, vec3);
+}
+
+cudaError_t launch_tconv_wgrad_epilogue(int c_in, int c_out, int taps, const float *part, int splits, const void *w,
+                                        const float *vec3, const float *b, const float *mean, const float *bsum,
+                                        int bsplits, float *dotpart, unsigned int *counters, float *dw, float *db,
+                                        float *dgamma, float *dbeta, cudaStream_t st) {
+    static PerDevice carve;
+    prefer_max_shared_once(tconv_wgrad_epilogue_kernel, &carve);
+    return launch_pdl(tconv_wgrad_epilogue_kernel, dim3(c_in / 32, taps * c_out / 32), dim3(1024), 0, st, c_in, c_out,
+                      taps * c_out, part, splits, (const __nv_bfloat16 *)w, vec3, b, mean, bsum, bsplits, dotpart, counters,
+                      dw, db, dgamma, dbeta, call_f16());
 }
 
 cudaError_t launch_tconv_rescale(int dtype, bool nhwc, long long count, int taps, int cig, int cog, const void *w,

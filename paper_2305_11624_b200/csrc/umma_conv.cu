@@ -49,9 +49,10 @@ struct ConvGemm {
     int resident;            // 1: the CTA's whole weight slab [BN][K] stays in shared memory (loaded once)
     int f16;                 // 16-bit storage type: 0 bf16, 1 IEEE half
     BnFold fold;             // fold.gamma != NULL: scale and shift formed in the kernel from the BN parameters
-    // 1 (Eval mode, dense stores): Y = acc + fold.b goes to tm_out and Z = s Y + (beta - mean s), from the rounded Y,
-    // to tm_out2.  A pass of its own re-read Y: conv + pass took 37 us for the 64 -> 256 layer at 56 x 56, N = 32.
-    int dual;
+    // Transposed convolution whose kernel is its stride (tap_c != 0): GEMM column tap tap_c + c of pixel (i, j) is channel
+    // c of output pixel (i kh + r, j kw + q), tap = r kw + q, in out_strided; out_sh / out_sw are the steps of i and j,
+    // tap_sh / tap_sw those of r and q.  The weight tensor is then read as it is, [ca][cn], as an MN-major operand.
+    int tap_c, tap_kw, tap_sh, tap_sw;
 };
 
 struct ConvSmemCtl {
@@ -68,14 +69,23 @@ struct ConvSmemCtl {
 // [128 (t / n_tiles), +128) and output channels [BN (t % n_tiles), +BN).  The accumulator is
 // double-buffered in tensor memory (2 x BN columns), so the MMAs of a tile overlap the epilogue of
 // the tile before, and the TMA ring runs ahead across tile boundaries.
-template <int BN>
-__global__ void __launch_bounds__(kConvThreads) umma_conv_kernel(const __grid_constant__ CUtensorMap tm_act,
+//
+// MODE kDual (Eval mode, dense stores): Y = acc + fold.b goes to tm_out and Z = s Y + (beta - mean s), from the rounded
+// Y, to tm_out2.  A pass of its own re-read Y: conv + pass took 37 us for the 64 -> 256 layer at 56 x 56, N = 32.  (An
+// instantiation of its own: as a run-time branch it cost the plain kernel 40 registers, and with 168 of them no block
+// of the kernels beside it fits next to a CTA: 3x3 512 -> 512 at 7 x 7, N = 64, forward + backward 85 -> 93 us.  The
+// bound of 512 threads holds the plain kernel to 128 registers for the same reason.)
+// MODE kTap: the transposed convolution of ConvGemm::tap_c.
+enum ConvMode { kPlain, kDual, kTap };
+template <int BN, ConvMode MODE>
+__global__ void __launch_bounds__(MODE == kDual ? kConvThreads : 512) umma_conv_kernel(const __grid_constant__ CUtensorMap tm_act,
                                                                 const __grid_constant__ CUtensorMap tm_w,
                                                                 const __grid_constant__ CUtensorMap tm_out,
                                                                 const __grid_constant__ CUtensorMap tm_out2,
                                                                 const ConvGemm g, const float *__restrict__ bias,
                                                                 int *err) {
     extern __shared__ uint8_t smem_raw[];
+    constexpr bool DUAL = MODE == kDual, TAP = MODE == kTap;
     constexpr uint32_t kABytes = kBM * kBK * 2, kBBytes = BN * kBK * 2;
     const int cchunks = g.blockdiag ? 1 : g.ca / kBK;
     const int num_kb = g.taps_h * g.taps_w * cchunks;
@@ -87,7 +97,7 @@ __global__ void __launch_bounds__(kConvThreads) umma_conv_kernel(const __grid_co
     ConvSmemCtl *ctl = (ConvSmemCtl *)(staging + kStagingBytes);
     float *bias_s = (float *)(((uintptr_t)(ctl + 1) + 15) & ~(uintptr_t)15);   // cn floats
     float *scale_s = bias_s + g.cn;                                            // cn floats (fold mode)
-    float *shift_s = scale_s + g.cn;                                           // cn floats (dual mode)
+    float *shift_s = scale_s + g.cn;                                           // cn floats (DUAL)
     const bool fold = g.fold.gamma != nullptr;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int stages = g.stages;
@@ -128,7 +138,8 @@ __global__ void __launch_bounds__(kConvThreads) umma_conv_kernel(const __grid_co
     if (threadIdx.x == 0) { prefetch_tensormap(&tm_act); prefetch_tensormap(&tm_w); prefetch_tensormap(&tm_out); }
     pdl_wait();
     if (threadIdx.x == 0) CONVBN_TRACE_POINT(1);
-    if (g.dual) {
+    const int pc = TAP ? g.tap_c : g.cn;               // channels the per-channel parameters belong to
+    if constexpr (DUAL) {
         for (int c = threadIdx.x; c < g.cn; c += kConvThreads) {
             const float sc = g.fold.gamma[c] * (1.0f / sqrtf(g.fold.var[c] + g.fold.eps));
             bias_s[c] = g.fold.b ? g.fold.b[c] : 0.f;
@@ -138,14 +149,14 @@ __global__ void __launch_bounds__(kConvThreads) umma_conv_kernel(const __grid_co
     } else if (fold) {
         // On-the-fly reparameterisation (Sec. 3.3 / 3.4): s = gamma / sqrt(var + eps), b' = (b - mu) s + beta.
         // s multiplies the fp32 accumulator (the associative law of Sec. 3.2.2), so omega is used unrounded.
-        for (int c = threadIdx.x; c < g.cn; c += kConvThreads) {
+        for (int c = threadIdx.x; c < pc; c += kConvThreads) {
             const float r = 1.0f / sqrtf(g.fold.var[c] + g.fold.eps);
             const float sc = g.fold.gamma[c] * r;
             const float bf = ((g.fold.b ? g.fold.b[c] : 0.f) - g.fold.mean[c]) * sc + g.fold.beta[c];
             scale_s[c] = sc;
             bias_s[c] = bf;
             if (blockIdx.x == 0 && g.fold.vec3) {
-                g.fold.vec3[c] = sc; g.fold.vec3[g.cn + c] = bf; g.fold.vec3[2 * g.cn + c] = r;
+                g.fold.vec3[c] = sc; g.fold.vec3[pc + c] = bf; g.fold.vec3[2 * pc + c] = r;
             }
         }
     } else if (bias) {
@@ -169,7 +180,13 @@ __global__ void __launch_bounds__(kConvThreads) umma_conv_kernel(const __grid_co
         if (g.resident && lane == 1) {
             const int n0 = (int)(blockIdx.x % n_tiles) * BN;
             mbar_arrive_expect_tx(&ctl->bfull, (uint32_t)num_kb * kBBytes);
-            for (int kb = 0; kb < num_kb; ++kb) tma_load_2d(slab + (size_t)kb * kBBytes, &tm_w, &ctl->bfull, kb * kBK, n0);
+            for (int kb = 0; kb < num_kb; ++kb) {
+                uint8_t *dst = slab + (size_t)kb * kBBytes;
+                if constexpr (TAP)
+                    for (int c = 0; c < BN; c += 64) tma_load_2d(dst + c * 128, &tm_w, &ctl->bfull, n0 + c, kb * kBK);
+                else
+                    tma_load_2d(dst, &tm_w, &ctl->bfull, kb * kBK, n0);
+            }
         }
         uint32_t mt, nt;
         for (uint32_t i = 0; ok && tile_of(i, mt, nt); ++i) {
@@ -206,7 +223,10 @@ __global__ void __launch_bounds__(kConvThreads) umma_conv_kernel(const __grid_co
                     tma_load_im2col_4d(a_dst, &tm_act, &ctl->full[s], (g.blockdiag ? n0 : 0) + cc * kBK, base_w, base_h, img0,
                                        (uint16_t)(q * g.dil_w), (uint16_t)(r * g.dil_h));
                 } else if (lane == 1 && !g.resident) {
-                    tma_load_2d(b_dst, &tm_w, &ctl->full[s], kb * kBK, n0);
+                    if constexpr (TAP)
+                        for (int c = 0; c < BN; c += 64) tma_load_2d(b_dst + c * 128, &tm_w, &ctl->full[s], n0 + c, kb * kBK);
+                    else
+                        tma_load_2d(b_dst, &tm_w, &ctl->full[s], kb * kBK, n0);
                 }
                 if (++cc == cchunks) { cc = 0; if (++q == g.taps_w) { q = 0; ++r; } }
                 if (++s == stages) { s = 0; ph ^= 1u; }
@@ -223,9 +243,11 @@ __global__ void __launch_bounds__(kConvThreads) umma_conv_kernel(const __grid_co
     } else if (warp == 1) {
         // ---------------- MMA issuer ----------------
         if (elect_one()) {
-            const uint32_t idesc = idesc_h16_f32(kBM, BN, 0, 0, g.f16);
-            const uint32_t hi = smem_desc_hi_sw128(1024);
-            const uint32_t tiles_lo = smem_desc_lo(smem_u32(tiles), 16), slab_lo = smem_desc_lo(smem_u32(slab), 16);
+            // MN-major weights: 64-column blocks of [64 k][128 bytes], 8192 bytes apart; 16 k = 2048 bytes
+            const uint32_t idesc = idesc_h16_f32(kBM, BN, 0, TAP ? 1 : 0, g.f16);
+            const uint32_t hi = smem_desc_hi_sw128(1024), b_lead = TAP ? 8192u : 16u;
+            const uint32_t tiles_lo = smem_desc_lo(smem_u32(tiles), 16), slab_lo = smem_desc_lo(smem_u32(slab), b_lead);
+            const uint32_t ring_b_lo = smem_desc_lo(smem_u32(tiles) + kABytes, b_lead);
             int s = 0;
             uint32_t ph = 0;
             bool ok = true;
@@ -249,12 +271,13 @@ __global__ void __launch_bounds__(kConvThreads) umma_conv_kernel(const __grid_co
                     tc_fence_after_sync();
                     // descriptors as halves: only the start-address field (16-byte units) moves
                     const uint32_t a_lo = tiles_lo + (uint32_t)s * (kStageBytes >> 4);
-                    const uint32_t b_lo = g.resident ? slab_lo + (uint32_t)kb * (kBBytes >> 4) : a_lo + (kABytes >> 4);
+                    const uint32_t b_lo = g.resident ? slab_lo + (uint32_t)kb * (kBBytes >> 4)
+                                                     : ring_b_lo + (uint32_t)s * (kStageBytes >> 4);
                     if (kb == 0) umma_bf16_ss_halves<false>(d_tmem, a_lo, hi, b_lo, hi, idesc);
                     else umma_bf16_ss_halves<true>(d_tmem, a_lo, hi, b_lo, hi, idesc);
 #pragma unroll
                     for (int k = 1; k < kBK / kUmmaK; ++k)
-                        umma_bf16_ss_halves<true>(d_tmem, a_lo + (uint32_t)k * 2u, hi, b_lo + (uint32_t)k * 2u, hi, idesc);
+                        umma_bf16_ss_halves<true>(d_tmem, a_lo + (uint32_t)k * 2u, hi, b_lo + (uint32_t)k * (TAP ? 128u : 2u), hi, idesc);
                     umma_commit(&ctl->empty[s]);
                     if (++s == stages) { s = 0; ph ^= 1u; }
                 }
@@ -293,9 +316,16 @@ __global__ void __launch_bounds__(kConvThreads) umma_conv_kernel(const __grid_co
                 if ((long long)m < g.p) {
                     const uint32_t tq = m / (uint32_t)g.wo, img = tq / (uint32_t)g.ho;
                     srow = g.out_strided + (size_t)img * g.out_sn + (size_t)(tq - img * (uint32_t)g.ho) * g.out_sh +
-                           (size_t)(m - tq * (uint32_t)g.wo) * g.out_sw + n0;
+                           (size_t)(m - tq * (uint32_t)g.wo) * g.out_sw;
+                    if constexpr (TAP) {                    // (a tile lies inside one tap: BN divides tap_c)
+                        const int tap = n0 / g.tap_c, tr = tap / g.tap_kw;
+                        srow += (size_t)tr * g.tap_sh + (size_t)(tap - tr * g.tap_kw) * g.tap_sw + (n0 - tap * g.tap_c);
+                    } else {
+                        srow += n0;
+                    }
                 }
             }
+            const int p0 = TAP ? n0 % g.tap_c : n0;         // first per-channel parameter of this tile
 #pragma unroll 1
             for (int c0 = 0; c0 < BN; c0 += 64) {
                 uint32_t v[64];
@@ -310,21 +340,7 @@ __global__ void __launch_bounds__(kConvThreads) umma_conv_kernel(const __grid_co
                     __syncwarp();
                     if (lane == 0) mbar_arrive(&ctl->tmem_empty[acc]);
                 }
-                if (c0 < ncols && g.out_strided) {
-                    if (srow) {
-#pragma unroll
-                        for (int j = 0; j < 64; j += 8) {
-                            if (c0 + j < ncols) {
-                                uint4 pk;
-                                pk.x = pack2_h16(__uint_as_float(v[j]), __uint_as_float(v[j + 1]), g.f16);
-                                pk.y = pack2_h16(__uint_as_float(v[j + 2]), __uint_as_float(v[j + 3]), g.f16);
-                                pk.z = pack2_h16(__uint_as_float(v[j + 4]), __uint_as_float(v[j + 5]), g.f16);
-                                pk.w = pack2_h16(__uint_as_float(v[j + 6]), __uint_as_float(v[j + 7]), g.f16);
-                                *(uint4 *)(srow + c0 + j) = pk;
-                            }
-                        }
-                    }
-                } else if (c0 < ncols) {
+                if (c0 < ncols) {
                     uint8_t *buf = stage_buf;
                     // the previous store read this buffer: wait until it no longer does (shared memory
                     // is better spent on ring slots than on a second staging buffer)
@@ -338,15 +354,15 @@ __global__ void __launch_bounds__(kConvThreads) umma_conv_kernel(const __grid_co
                             float f[8];
     #pragma unroll
                             for (int e = 0; e < 8; ++e) f[e] = __uint_as_float(v[j + e]);
-                            if (fold && !g.dual) {
-                                const float4 s0 = *(const float4 *)(scale_s + n0 + c0 + j);
-                                const float4 s1 = *(const float4 *)(scale_s + n0 + c0 + j + 4);
+                            if (fold && !DUAL) {
+                                const float4 s0 = *(const float4 *)(scale_s + p0 + c0 + j);
+                                const float4 s1 = *(const float4 *)(scale_s + p0 + c0 + j + 4);
                                 f[0] *= s0.x; f[1] *= s0.y; f[2] *= s0.z; f[3] *= s0.w;
                                 f[4] *= s1.x; f[5] *= s1.y; f[6] *= s1.z; f[7] *= s1.w;
                             }
                             if (bias || fold) {
-                                const float4 b0 = *(const float4 *)(bias_s + n0 + c0 + j);
-                                const float4 b1 = *(const float4 *)(bias_s + n0 + c0 + j + 4);
+                                const float4 b0 = *(const float4 *)(bias_s + p0 + c0 + j);
+                                const float4 b1 = *(const float4 *)(bias_s + p0 + c0 + j + 4);
                                 f[0] += b0.x; f[1] += b0.y; f[2] += b0.z; f[3] += b0.w;
                                 f[4] += b1.x; f[5] += b1.y; f[6] += b1.z; f[7] += b1.w;
                             }
@@ -359,6 +375,19 @@ __global__ void __launch_bounds__(kConvThreads) umma_conv_kernel(const __grid_co
                         }
                     };
                     if (g.f16) pack_rows(std::true_type{}); else pack_rows(std::false_type{});
+                    if (TAP || g.out_strided) {
+                        // eight lanes write the 128 bytes of a pixel, four pixels per instruction
+                        __syncwarp();
+#pragma unroll 2
+                        for (int it = 0; it < 8; ++it) {
+                            const int rr = it * 4 + (lane >> 3), ch = lane & 7;
+                            __nv_bfloat16 *dst = (__nv_bfloat16 *)__shfl_sync(0xffffffffu, (unsigned long long)srow, rr);
+                            const uint4 q = *(const uint4 *)(buf + rr * 128 + (((ch ^ (rr & 7)) & 7) << 4));
+                            if (dst && c0 + ch * 8 < ncols) *(uint4 *)(dst + c0 + ch * 8) = q;
+                        }
+                        __syncwarp();
+                        continue;
+                    }
                     fence_proxy_async_smem();
                     __syncwarp();
                     if (lane == 0) {
@@ -373,7 +402,7 @@ __global__ void __launch_bounds__(kConvThreads) umma_conv_kernel(const __grid_co
                         }
                         tma_store_commit();
                     }
-                    if (g.dual) {
+                    if constexpr (DUAL) {
                         uint4 zq[8];
                         auto normalise = [&](auto half_tag) {
                             constexpr bool H = decltype(half_tag)::value;
@@ -532,11 +561,11 @@ bool umma_conv_eligible(const UmmaConvShape &s) {
 
 static int sm_count() { return device_sm_count(); }
 
-template <int BN>
+template <int BN, ConvMode MODE = kPlain>
 static cudaError_t launch_bn(const CUtensorMap &ta, const CUtensorMap &tw, const CUtensorMap &tout,
                              const CUtensorMap &tout2, ConvGemm g, const float *bias, int *err, cudaStream_t st) {
     const size_t a_bytes = (size_t)kBM * kBK * 2, b_bytes = (size_t)BN * kBK * 2;
-    size_t fixed = 1024 + kStagingBytes + sizeof(ConvSmemCtl) + (g.dual ? 3 : 2) * (size_t)g.cn * sizeof(float) + 16;
+    size_t fixed = 1024 + kStagingBytes + sizeof(ConvSmemCtl) + (MODE == kDual ? 3 : 2) * (size_t)g.cn * sizeof(float) + 16;
     const int num_kb = g.taps_h * g.taps_w * (g.blockdiag ? 1 : g.ca / kBK);
     const long long m_tiles = (g.p + kBM - 1) / kBM, n_tiles = (g.cn + BN - 1) / BN;
     long long grid_l = m_tiles * n_tiles < sm_count() ? m_tiles * n_tiles : sm_count();
@@ -556,11 +585,19 @@ static cudaError_t launch_bn(const CUtensorMap &ta, const CUtensorMap &tw, const
     g.stages = stages;
     const size_t smem = stages * stage + fixed;
     static PerDevice attr_done;
-    if (cudaError_t e = max_dynamic_smem_once(umma_conv_kernel<BN>, 224 * 1024, &attr_done); e != cudaSuccess) return e;
+    if (cudaError_t e = max_dynamic_smem_once(umma_conv_kernel<BN, MODE>, 224 * 1024, &attr_done); e != cudaSuccess) return e;
     static PerDevice carve;
-    prefer_max_shared_once(umma_conv_kernel<BN>, &carve);
+    prefer_max_shared_once(umma_conv_kernel<BN, MODE>, &carve);
     const unsigned grid = (unsigned)grid_l;
-    return launch_pdl(umma_conv_kernel<BN>, dim3(grid), dim3(kConvThreads), smem, st, ta, tw, tout, tout2, g, bias, err);
+    return launch_pdl(umma_conv_kernel<BN, MODE>, dim3(grid), dim3(kConvThreads), smem, st, ta, tw, tout, tout2, g, bias, err);
+}
+
+template <ConvMode MODE>
+static cudaError_t launch_mode(int bn, const CUtensorMap &ta, const CUtensorMap &tw, const CUtensorMap &tout,
+                               const CUtensorMap &tout2, const ConvGemm &g, const float *bias, int *err, cudaStream_t st) {
+    if (bn == 64) return launch_bn<64, MODE>(ta, tw, tout, tout2, g, bias, err, st);
+    if (bn == 128) return launch_bn<128, MODE>(ta, tw, tout, tout2, g, bias, err, st);
+    return launch_bn<256, MODE>(ta, tw, tout, tout2, g, bias, err, st);
 }
 
 // Tile width: fewest rounds of tiles over the SMs, weighted by the time of one tile (N = 64 tiles are
@@ -583,7 +620,6 @@ static int pick_bn(long long tiles_m, int cn) {
 cudaError_t launch_umma_conv(const UmmaConvShape &s, const void *act, const void *wmat, const float *bias,
                              void *out, cudaStream_t st, const BnFold *fold, void *out2) {
     ConvGemm g;
-    g.dual = out2 ? 1 : 0;
     g.ho = s.ho; g.wo = s.wo; g.cn = s.cn; g.ca = s.ca; g.taps_h = s.taps_h; g.taps_w = s.taps_w;
     g.lower_h = s.lower_h; g.lower_w = s.lower_w; g.stride_h = s.stride_h; g.stride_w = s.stride_w;
     g.dil_h = s.dil_h; g.dil_w = s.dil_w; g.p = (long long)s.n * s.ho * s.wo; g.stages = 1;
@@ -593,27 +629,30 @@ cudaError_t launch_umma_conv(const UmmaConvShape &s, const void *act, const void
     g.fold = fold ? *fold : BnFold{nullptr, nullptr, nullptr, nullptr, nullptr, 0.f, nullptr};
     g.out_strided = s.out_sw ? (__nv_bfloat16 *)out : nullptr;
     g.out_sn = s.out_sn; g.out_sh = s.out_sh; g.out_sw = s.out_sw;
+    g.tap_c = s.tap_c; g.tap_kw = s.tap_kw; g.tap_sh = s.tap_sh; g.tap_sw = s.tap_sw;
     // The bounding box of base pixels has ho x wo positions: upper = lower + (out-1) stride - (in-1).
     const int upper_h = s.lower_h + (s.ho - 1) * s.stride_h - (s.ha - 1);
     const int upper_w = s.lower_w + (s.wo - 1) * s.stride_w - (s.wa - 1);
     const long long tiles_m = (g.p + kBM - 1) / kBM;
-    const int bn = s.blockdiag ? 64 : pick_bn(tiles_m, s.cn);
+    int bn = s.blockdiag ? 64 : pick_bn(tiles_m, s.cn);
+    while (s.tap_c && s.tap_c % bn) bn /= 2;            // a tile lies inside one tap
     CUtensorMap ta, tw, tout;
     // (in strided mode the output map is encoded but never used: every row is stored by its thread)
     if (!make_tmap_matrix_bf16(&tout, out, s.out_sw ? 32 : g.p, s.cn, 32, 64)) return cudaErrorInvalidValue;
     if (!make_tmap_im2col_bf16(&ta, act, s.n, s.ha, s.wa, s.ca, s.lower_h, s.lower_w, upper_h, upper_w, s.stride_h,
                                s.stride_w, kBM, kBK))
         return cudaErrorInvalidValue;
-    if (!make_tmap_matrix_bf16(&tw, wmat, s.cn, (long long)s.taps_h * s.taps_w * (s.blockdiag ? 64 : s.ca), bn, kBK))
+    if (s.tap_c ? !make_tmap_matrix_bf16(&tw, wmat, s.ca, s.cn, kBK, 64)
+                : !make_tmap_matrix_bf16(&tw, wmat, s.cn, (long long)s.taps_h * s.taps_w * (s.blockdiag ? 64 : s.ca), bn, kBK))
         return cudaErrorInvalidValue;
     int *err = nullptr;
     cudaError_t e = error_word_address(&err);
     if (e != cudaSuccess) return e;
     CUtensorMap tout2 = tout;
     if (out2 && !make_tmap_matrix_bf16(&tout2, out2, g.p, s.cn, 32, 64)) return cudaErrorInvalidValue;
-    if (bn == 64) return launch_bn<64>(ta, tw, tout, tout2, g, bias, err, st);
-    if (bn == 128) return launch_bn<128>(ta, tw, tout, tout2, g, bias, err, st);
-    return launch_bn<256>(ta, tw, tout, tout2, g, bias, err, st);
+    if (out2) return launch_mode<kDual>(bn, ta, tw, tout, tout2, g, bias, err, st);
+    if (g.tap_c) return launch_mode<kTap>(bn, ta, tw, tout, tout2, g, bias, err, st);
+    return launch_mode<kPlain>(bn, ta, tw, tout, tout2, g, bias, err, st);
 }
 
 // Forward pass of a small-C_in layer on the packed input (see stem_kernels.cu): tiles of 8 x 16 output
@@ -622,7 +661,7 @@ cudaError_t launch_stem_fwd(const Problem &pb, const void *x_packed, const void 
                             cudaStream_t st, const BnFold *fold) {
     const int krows = stem_krows(pb);
     ConvGemm g;
-    g.dual = 0;
+    g.tap_c = 0;
     g.ho = pb.h_out; g.wo = pb.w_out; g.cn = pb.c_out; g.ca = 64; g.taps_h = krows; g.taps_w = 1;
     g.lower_h = g.lower_w = 0; g.stride_h = g.stride_w = g.dil_h = g.dil_w = 1;
     g.stem = 1; g.stem_tw = 16; g.stem_th = 8;

@@ -286,7 +286,7 @@ void wgrad_epilogue_shape(const Problem &pb, UmmaWgradPlan *pl) {
 template <int BN>
 static cudaError_t launch_w(const CUtensorMap &tx, const CUtensorMap &tdz, WgradGemm g, const UmmaWgradPlan &pl,
                             const Problem &pb, float *partials, float *bsum, unsigned int *counters, int *err,
-                            cudaStream_t st) {
+                            cudaStream_t st, int ncounters = -1) {
     constexpr size_t stage = 2 * kChunkBytes + (BN / 64) * kChunkBytes;
     int stages = BN == 128 ? 3 : 4;                    // 128-wide: 3 x 32 KB, so that two CTAs share an SM
     const long long max_kb = (pl.per_split + kWP - 1) / kWP;
@@ -302,11 +302,11 @@ static cudaError_t launch_w(const CUtensorMap &tx, const CUtensorMap &tdz, Wgrad
     dim3 grid((unsigned)((g.kdim / 64 + (g.no_ones ? 1 : 2)) / 2), (unsigned)((pb.c_out + BN - 1) / BN),
               (unsigned)pl.splits);
     return launch_pdl(umma_wgrad_kernel<BN>, grid, dim3(kWThreads), smem, st, tx, tdz, g, partials, bsum, counters,
-                      pb.c_out / 32, err);
+                      ncounters >= 0 ? ncounters : pb.c_out / 32, err);
 }
 
 cudaError_t launch_umma_wgrad(const Problem &pb, const UmmaWgradPlan &pl, const void *dz, const void *x,
-                              float *partials, float *bsum, unsigned int *counters, cudaStream_t st) {
+                              float *partials, float *bsum, unsigned int *counters, cudaStream_t st, int ncounters) {
     WgradGemm g;
     g.ho = pb.h_out; g.wo = pb.w_out; g.c_in = pb.c_in; g.c_out = pb.c_out; g.taps_w = pb.kw;
     g.lower_h = -pb.pad_h; g.lower_w = -pb.pad_w; g.stride_h = pb.stride_h; g.stride_w = pb.stride_w;
@@ -325,9 +325,9 @@ cudaError_t launch_umma_wgrad(const Problem &pb, const UmmaWgradPlan &pl, const 
     cudaError_t e = error_word_address(&err);
     if (e != cudaSuccess) return e;
     const int bn = g.blockdiag ? 64 : wgrad_bn(pb);
-    if (bn == 64) return launch_w<64>(tx, tdz, g, pl, pb, partials, bsum, counters, err, st);
-    if (bn == 128) return launch_w<128>(tx, tdz, g, pl, pb, partials, bsum, counters, err, st);
-    return launch_w<256>(tx, tdz, g, pl, pb, partials, bsum, counters, err, st);
+    if (bn == 64) return launch_w<64>(tx, tdz, g, pl, pb, partials, bsum, counters, err, st, ncounters);
+    if (bn == 128) return launch_w<128>(tx, tdz, g, pl, pb, partials, bsum, counters, err, st, ncounters);
+    return launch_w<256>(tx, tdz, g, pl, pb, partials, bsum, counters, err, st, ncounters);
 }
 
 // ---- epilogue over k-major partials ------------------------------------------------------------

@@ -23,3 +23,16 @@ def test_tune_block(spec):
     for deferred in (False, True):
         got = parity.run_tune_gpu(spec, t, deferred=deferred)
         parity.compare(got, ref, parity.TOL[spec.dtype], parity.TUNE_OUTPUTS, spec.name, dtype=spec.dtype)
+
+
+TCONV = [  # (dtype, n, c_in, h, w, c_out, k, stride, pad, dil, groups, bias): kernel = stride, the GEMM on omega as it is
+    ("bf16", 3, 64, 5, 7, 192, 2, 2, 0, 1, 1, True),        # tiles of 64 columns, fewer pixels than a tile
+    ("f16", 1, 192, 13, 11, 64, 3, 3, 0, 1, 1, False),      # nine taps, a last tile of 15 pixels
+    ("bf16", 2, 256, 21, 24, 256, 2, 2, 0, 1, 1, True),     # a tap of 256 columns
+]
+
+
+@pytest.mark.parametrize("case", TCONV, ids=lambda c: "%s_c%d_o%d_k%d" % (c[0], c[2], c[5], c[6]))
+def test_tconv_block(case):
+    import test_tconv
+    test_tconv.test_library_matches_the_oracle(case)
