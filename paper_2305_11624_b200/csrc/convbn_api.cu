@@ -134,6 +134,10 @@ struct Plan {
     UmmaWgradPlan uw;
 };
 
+bool f32_path(const convbn_desc *d, const Problem &pb) {
+    return d->dtype == CONVBN_F32 && d->layout == CONVBN_NCHW && f32_conv_eligible(pb);
+}
+
 bool fused_bwd_path(const convbn_desc *d, const Problem &pb) {
     return d->dtype == CONVBN_BF16 && d->layout == CONVBN_NHWC && fused_bwd1x1_eligible(pb);
 }
@@ -432,6 +436,9 @@ int run_conv_fwd(const convbn_desc *d, const Problem &pb, const void *x, const v
     } else if (dw_path(d, pb)) {
         LAUNCH("dw_fwd", launch_dw_fwd(pb, x, w, bias, z, st));
         *which = "depthwise";
+    } else if (f32_path(d, pb)) {
+        LAUNCH("direct_fwd", launch_f32_fwd(pb, (const float *)x, (const float *)w, bias, (float *)z, st));
+        *which = "direct";
     } else {
         LAUNCH("direct_fwd", launch_direct_fwd(pb, d->dtype, d->layout, x, w, bias, z, st));
         *which = "direct";
@@ -571,6 +578,10 @@ int run_conv_dgrad(const convbn_desc *d, const Problem &pb, const void *dz, cons
             LAUNCH("dw_dgrad", launch_dw_dgrad(pb, dz, wd, dx, st));
         }
         *which = "depthwise";
+    } else if (f32_path(d, pb)) {
+        LAUNCH("direct_dgrad", launch_f32_bwd(pb, (const float *)dz, nullptr, (const float *)w, scale, (float *)dx, nullptr,
+                                              nullptr, nullptr, nullptr, nullptr, nullptr, nullptr, st));
+        *which = "direct";
     } else {
         const void *wd = w;
         if (scale) {
@@ -590,6 +601,12 @@ int run_conv_dgrad(const convbn_desc *d, const Problem &pb, const void *dz, cons
 int run_param_grads(const convbn_desc *d, const Problem &pb, const Plan &pl, const void *dz, const void *x,
                     const void *w, const float *vec3, const float *b, const float *mean, float *dw, float *db,
                     float *dgamma, float *dbeta, void *ws, cudaStream_t st, const char **which, bool scale_only = false) {
+    if (f32_path(d, pb)) {
+        LAUNCH("direct_wgrad", launch_f32_bwd(pb, (const float *)dz, (const float *)x, (const float *)w, nullptr, nullptr, vec3, b,
+                                              mean, dw, db, dgamma, dbeta, st));
+        *which = "direct";
+        return CONVBN_OK;
+    }
     float *partials = (float *)at(ws, pl.partials), *bsum = (float *)at(ws, pl.bsum);
     const bool need_bsum = (vec3 || db) && !scale_only;
     const bool tc = pl.grouped_wgrad || pl.umma_wgrad || pl.stem;   // tensor-core paths sum dZ inside the GEMM
@@ -751,6 +768,12 @@ int convbn_tune_fwd(const convbn_desc *desc, const void *x, const void *w, const
         t_last_kernel[CONVBN_PHASE_TUNE_FWD] = "depthwise";
         return CONVBN_OK;
     }
+    if (f32_path(desc, pb)) {
+        const BnFold fold{gamma, beta, run_mean, run_var, b, pb.eps, vec3};
+        LAUNCH("direct_fwd", launch_f32_fwd(pb, (const float *)x, (const float *)w, nullptr, (float *)z, st, &fold));
+        t_last_kernel[CONVBN_PHASE_TUNE_FWD] = "direct";
+        return CONVBN_OK;
+    }
     if (grouped_path(desc, pb) && grouped8_eligible(pb)) {
         const BnFold fold{gamma, beta, run_mean, run_var, b, pb.eps, vec3};
         LAUNCH("grouped_fwd", launch_grouped8_fwd(pb, x, w, nullptr, z, st, &fold));
@@ -877,6 +900,13 @@ static int tune_bwd_impl(const convbn_desc *desc, const void *dz, const void *x,
         return CONVBN_EALIGN;
     const Plan pl = make_plan(desc, pb, CONVBN_PHASE_TUNE_BWD);
     CK(check_ws(pl, workspace, workspace_bytes));
+    if (f32_path(desc, pb)) {            // both passes in one launch
+        cudaStream_t st = (cudaStream_t)stream;
+        LAUNCH("direct_bwd", launch_f32_bwd(pb, (const float *)dz, (const float *)x, (const float *)w, (const float *)saved,
+                                            (float *)dx, (const float *)saved, b, run_mean, dw, db, dgamma, dbeta, st));
+        t_last_kernel[CONVBN_PHASE_TUNE_BWD] = "two-calls";
+        return CONVBN_OK;
+    }
     if (!fused_bwd_path(desc, pb)) {
         void *ws_w = workspace ? at(workspace, pl.w_scaled) : nullptr;
         const size_t bytes_d = pl.w_scaled, bytes_w = pl.total - pl.w_scaled;

@@ -1,0 +1,384 @@
+// fp32 NCHW convolutions with unit stride and dilation, groups = 1 and a 1x1 or 3x3 kernel, up to 128 channels: the
+// small fp32 blocks of unit tests, gradient checks and small networks.  (Other fp32 shapes: direct_kernels.cu.)
+//
+// At these sizes a pass is bound by its launches and by the length of each thread's chain of loads (a 3x3 block of
+// 16 -> 32 channels at 16 x 16, N = 2 is 14 MFLOP; one thread per output took 12 to 33 us a kernel in seven launches), so
+// each direction is ONE launch:
+//   forward   Z = s (omega (*) X) + b', s and b' formed in the kernel;
+//   backward  blocks of two kinds: domega', sum dZ and all parameter gradients in clusters of eight blocks that add up
+//             through distributed shared memory, and dX = (s omega)_rot (*) dZ.
+#include <cooperative_groups.h>
+
+#include "kernels.h"
+
+namespace cg = cooperative_groups;
+
+namespace convbn {
+namespace {
+
+constexpr int kFThreads = 256;
+constexpr int kFPix = 64;           // output pixels of a convolution block (of one image plane)
+constexpr int kFChunk = 16;         // input channels whose weights are staged at a time
+constexpr int kFCluster = 8;        // blocks of a weight-gradient cluster
+constexpr int kFCo = 4;             // output channels of a cluster
+constexpr int kFRun = 8;            // consecutive pixels a thread slides its window over
+
+// out[n][oc][p] = scale[oc] sum_{ic, tap} act[n][ic][p + tap - pad] wt(oc, ic, tap) + shift[oc]
+struct F32Conv {
+    const float *act, *w;
+    float *out;
+    int n, ic, h, wd, oc, ho, wo, pad;     // pad: of this pass
+    const float *k_scale;                  // DGRAD: s of the layer's output channel, here the input channel (NULL = 1)
+    const float *bias;                     // without fold (NULL = 0)
+    int tiles;                             // pixel tiles of a plane
+};
+
+// Block (oc tile, pixel tile, image).  256 threads = 64 pixels x 4 groups.  S == 1: the groups are R output channels each,
+// the input channels go by in chunks of 16.  S == 4: the groups split the input channels and are added up at the end, R
+// output channels per block, which keeps the chain of a thread short when there are too few blocks to hide it.
+// Weights are staged as [ic][tap][oc]; a thread's value of the activation meets R of them in one or two broadcasts.
+template <int K, int R, int S, bool DGRAD>
+__device__ __forceinline__ void conv_tile(const F32Conv &c, int oc0, int tile, int img, const float *scale_s, const float *shift_s,
+                                          float *smem) {
+    constexpr int KK = K * K, OCT = S == 1 ? 4 * R : R;
+    const int lane = threadIdx.x % kFPix, grp = threadIdx.x / kFPix;
+    const int p = tile * kFPix + lane, hw = c.ho * c.wo;
+    const bool valid = p < hw;
+    const int y = valid ? p / c.wo : 0, x = valid ? p - y * c.wo : 0;
+    bool ok[KK];
+#pragma unroll
+    for (int r = 0; r < K; ++r)
+#pragma unroll
+        for (int q = 0; q < K; ++q) {
+            const int yy = y - c.pad + r, xx = x - c.pad + q;
+            ok[r * K + q] = valid && yy >= 0 && yy < c.h && xx >= 0 && xx < c.wd;
+        }
+    const float *a0 = c.act + (size_t)img * c.ic * c.h * c.wd + (ptrdiff_t)(y - c.pad) * c.wd + (x - c.pad);
+    float acc[R];
+#pragma unroll
+    for (int j = 0; j < R; ++j) acc[j] = 0.f;
+    const int chunk = S == 1 ? kFChunk : c.ic;
+    for (int ic0 = 0; ic0 < c.ic; ic0 += chunk) {
+        const int nic = c.ic - ic0 < chunk ? c.ic - ic0 : chunk;
+        if (ic0) __syncthreads();
+        // consecutive threads read consecutive weights: the source rows are [ic][tap] (forward) or [oc][tap] (DGRAD)
+        if constexpr (DGRAD) {
+            for (int i = threadIdx.x; i < nic * OCT * KK; i += kFThreads) {
+                const int t = i % KK, o = (i / KK) % OCT, ci = i / (KK * OCT);
+                float v = 0.f;
+                if (oc0 + o < c.oc) {
+                    v = c.w[((size_t)(ic0 + ci) * c.oc + oc0 + o) * KK + t];
+                    if (c.k_scale) v *= c.k_scale[ic0 + ci];
+                }
+                smem[(ci * KK + KK - 1 - t) * OCT + o] = v;
+            }
+        } else {
+            for (int i = threadIdx.x; i < nic * OCT * KK; i += kFThreads) {
+                const int t = i % KK, ci = (i / KK) % nic, o = i / (KK * nic);
+                smem[(ci * KK + t) * OCT + o] = oc0 + o < c.oc ? c.w[((size_t)(oc0 + o) * c.ic + ic0 + ci) * KK + t] : 0.f;
+            }
+        }
+        __syncthreads();
+        const int per = S == 1 ? nic : (nic + 3) / 4, lo = S == 1 ? 0 : grp * per, hi = S == 1 ? nic : min(nic, lo + per);
+#pragma unroll 2
+        for (int ci = lo; ci < hi; ++ci) {
+            const float *a = a0 + (size_t)(ic0 + ci) * c.h * c.wd;
+            float v[KK];
+#pragma unroll
+            for (int t = 0; t < KK; ++t) v[t] = ok[t] ? __ldg(a + (t / K) * c.wd + t % K) : 0.f;
+            const float *ws = smem + ci * KK * OCT + (S == 1 ? grp * R : 0);
+#pragma unroll
+            for (int t = 0; t < KK; ++t)
+#pragma unroll
+                for (int j = 0; j < R; j += 4) {
+                    const float4 q = *(const float4 *)(ws + t * OCT + j);
+                    acc[j] = fmaf(v[t], q.x, acc[j]); acc[j + 1] = fmaf(v[t], q.y, acc[j + 1]);
+                    acc[j + 2] = fmaf(v[t], q.z, acc[j + 2]); acc[j + 3] = fmaf(v[t], q.w, acc[j + 3]);
+                }
+        }
+    }
+    if constexpr (S == 4) {
+        __syncthreads();
+#pragma unroll
+        for (int j = 0; j < R; ++j) smem[(grp * R + j) * kFPix + lane] = acc[j];
+        __syncthreads();
+        static_assert(R == 4, "one output channel per group at the end");
+        acc[0] = (smem[(0 * R + grp) * kFPix + lane] + smem[(1 * R + grp) * kFPix + lane]) +
+                 (smem[(2 * R + grp) * kFPix + lane] + smem[(3 * R + grp) * kFPix + lane]);
+    }
+    constexpr int NO = S == 1 ? R : 1;
+#pragma unroll
+    for (int j = 0; j < NO; ++j) {
+        const int o = S == 1 ? grp * R + j : grp;
+        if (valid && oc0 + o < c.oc)
+            c.out[((size_t)img * c.oc + oc0 + o) * hw + p] = DGRAD ? acc[j] : fmaf(acc[j], scale_s[o], shift_s[o]);
+    }
+}
+
+constexpr int conv_smem_floats(int kk, int r, int s, int ic) {
+    const int w = s == 1 ? kFChunk * kk * 4 * r : ic * kk * r;
+    return s == 4 && w < kFThreads * r ? kFThreads * r : w;
+}
+
+template <int K, int R, int S>
+__global__ void __launch_bounds__(kFThreads) f32_fwd_kernel(const F32Conv c, const BnFold fold) {
+    extern __shared__ __align__(16) float f32_smem[];
+    constexpr int OCT = S == 1 ? 4 * R : R;
+    __shared__ float scale_s[OCT], shift_s[OCT];
+    pdl_wait();
+    pdl_launch_dependents();
+    const int oc0 = blockIdx.y * OCT;
+    if (threadIdx.x < OCT) {
+        const int o = oc0 + threadIdx.x;
+        float sc = 1.f, sh = 0.f;
+        if (o < c.oc) {
+            if (fold.gamma) {
+                const float r = 1.0f / sqrtf(fold.var[o] + fold.eps);
+                sc = fold.gamma[o] * r;
+                sh = ((fold.b ? fold.b[o] : 0.f) - fold.mean[o]) * sc + fold.beta[o];
+                if (blockIdx.x == 0 && blockIdx.z == 0 && fold.vec3) {
+                    fold.vec3[o] = sc; fold.vec3[c.oc + o] = sh; fold.vec3[2 * c.oc + o] = r;
+                }
+            } else if (c.bias) {
+                sh = c.bias[o];
+            }
+        }
+        scale_s[threadIdx.x] = sc;
+        shift_s[threadIdx.x] = sh;
+    }
+    conv_tile<K, R, S, false>(c, oc0, blockIdx.x, blockIdx.z, scale_s, shift_s, f32_smem);
+}
+
+struct F32Wgrad {
+    const float *x, *dz, *w;
+    const float *vec3, *b, *mean;          // vec3 NULL: dw = domega', db = sum dZ
+    float *dw, *db, *dgamma, *dbeta;
+    int n, c_in, h, wd, c_out, ho, wo, pad;
+    int cip;                               // power of two >= c_in, 4 .. 128: threads along the input channels
+    int rows, bands;                       // output rows of a band, bands of an image
+    int xp, zp;                            // pitches of a staged row of X / dZ
+    int x_ci;                              // floats between the channels of the staged X (odd)
+};
+
+// Cluster = kFCo output channels, block rank r takes the row bands r, r + 8, ... of all images.  A band of X (all channels,
+// its halo rows, zeros outside) and of dZ is staged; thread (ci, channel pair, pixel group) slides a K x K window of X
+// along runs of eight pixels: K new values and two of dZ per 2 K K multiply-adds.  The pixel groups are added in the block,
+// the blocks through distributed shared memory, in rank order; rank j < 4 then finishes output channel j:
+//   domega = s domega', dbeta = sum dZ, db = s dbeta, dgamma = r (sum domega' omega + dbeta (b - mu_hat))   (Table 2)
+template <int K>
+__device__ __forceinline__ void wgrad_cluster(const F32Wgrad &g, int co0, float *smem) {
+    constexpr int KK = K * K;
+    cg::cluster_group cluster = cg::this_cluster();
+    const int rank = (int)cluster.block_rank();
+    const int ci = threadIdx.x % g.cip, rest = threadIdx.x / g.cip;
+    const int pair = rest & 1, pg = rest >> 1, npg = kFThreads / (2 * g.cip);
+    float *xs = smem, *zs = smem + (size_t)g.c_in * g.x_ci + 1;
+    float acc[2][KK], sum[2] = {0.f, 0.f};
+#pragma unroll
+    for (int t = 0; t < KK; ++t) acc[0][t] = acc[1][t] = 0.f;
+    const int xrows = g.rows + K - 1, runs = g.zp / kFRun, items = g.n * g.bands;
+    for (int it = rank; it < items; it += kFCluster) {
+        const int img = it / g.bands, y0 = (it - img * g.bands) * g.rows;
+        __syncthreads();
+        for (int i = threadIdx.x; i < g.c_in * xrows * g.xp; i += kFThreads) {
+            const int x = i % g.xp, t = i / g.xp, r = t % xrows, c = t / xrows;
+            const int yy = y0 - g.pad + r, xx = x - g.pad;
+            xs[(size_t)c * g.x_ci + r * g.xp + x] = (yy >= 0 && yy < g.h && xx >= 0 && xx < g.wd)
+                                                        ? __ldg(g.x + (((size_t)img * g.c_in + c) * g.h + yy) * g.wd + xx) : 0.f;
+        }
+        for (int i = threadIdx.x; i < kFCo * g.rows * g.zp; i += kFThreads) {
+            const int x = i % g.zp, t = i / g.zp, r = t % g.rows, o = t / g.rows;
+            zs[i] = (co0 + o < g.c_out && y0 + r < g.ho && x < g.wo)
+                        ? __ldg(g.dz + (((size_t)img * g.c_out + co0 + o) * g.ho + y0 + r) * g.wo + x) : 0.f;
+        }
+        __syncthreads();
+        if (ci < g.c_in)
+            for (int j = pg; j < g.rows * runs; j += npg) {
+                const int r = j / runs, x = (j - r * runs) * kFRun;
+                const float *xr = xs + (size_t)ci * g.x_ci + r * g.xp + x;
+                const float *z0 = zs + ((2 * pair) * g.rows + r) * g.zp + x, *z1 = z0 + g.rows * g.zp;
+                float win[K][K];
+#pragma unroll
+                for (int a = 0; a < K; ++a)
+#pragma unroll
+                    for (int q = 0; q < K - 1; ++q) win[a][q] = xr[a * g.xp + q];
+#pragma unroll
+                for (int i = 0; i < kFRun; ++i) {
+                    const float d0 = z0[i], d1 = z1[i];
+#pragma unroll
+                    for (int a = 0; a < K; ++a) win[a][(i + K - 1) % K] = xr[a * g.xp + i + K - 1];
+#pragma unroll
+                    for (int a = 0; a < K; ++a)
+#pragma unroll
+                        for (int q = 0; q < K; ++q) {
+                            const float v = win[a][(i + q) % K];
+                            acc[0][a * K + q] = fmaf(d0, v, acc[0][a * K + q]);
+                            acc[1][a * K + q] = fmaf(d1, v, acc[1][a * K + q]);
+                        }
+                    sum[0] += d0;
+                    sum[1] += d1;
+                }
+            }
+    }
+    // pixel groups -> block: [thread][K K + 1], then part[co][c_in K K + 1] (the last entry is sum dZ)
+    __syncthreads();
+    const int kd = g.c_in * KK, row = kd + 1;
+    float *part = smem, *red = smem + kFCo * row;
+    for (int h = 0; h < 2; ++h) {
+        float *mine = red + ((size_t)((pg * g.cip + ci) * 2 + pair)) * (KK + 1);
+#pragma unroll
+        for (int t = 0; t < KK; ++t) mine[t] = acc[h][t];
+        mine[KK] = sum[h];
+        __syncthreads();
+        for (int i = threadIdx.x; i < 2 * row; i += kFThreads) {
+            const int pr = i / row, e = i - pr * row;
+            const int c = e < kd ? e / KK : 0, t = e < kd ? e % KK : KK;
+            float v = 0.f;
+            for (int q = 0; q < npg; ++q) v += red[((size_t)((q * g.cip + c) * 2 + pr)) * (KK + 1) + t];
+            part[(2 * pr + h) * row + e] = v;
+        }
+        __syncthreads();
+    }
+    cluster.sync();
+    const int co = co0 + rank;
+    if (rank < kFCo && co < g.c_out) {
+        const float s = g.vec3 ? g.vec3[co] : 1.f;
+        float dot = 0.f, dsum = 0.f;
+        for (int e = threadIdx.x; e < row; e += kFThreads) {
+            float v[kFCluster];
+#pragma unroll
+            for (int b = 0; b < kFCluster; ++b) v[b] = cluster.map_shared_rank(part, b)[rank * row + e];
+            float tot = 0.f;
+#pragma unroll
+            for (int b = 0; b < kFCluster; ++b) tot += v[b];
+            if (e < kd) {
+                const size_t o = (size_t)co * kd + e;
+                g.dw[o] = s * tot;
+                if (g.vec3) dot = fmaf(tot, g.w[o], dot);
+            } else {
+                dsum = tot;
+            }
+        }
+        __shared__ float fin[2][kFThreads / 32];
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) { dot += __shfl_xor_sync(0xffffffffu, dot, o); dsum += __shfl_xor_sync(0xffffffffu, dsum, o); }
+        if (threadIdx.x % 32 == 0) { fin[0][threadIdx.x / 32] = dot; fin[1][threadIdx.x / 32] = dsum; }
+        __syncthreads();
+        if (threadIdx.x == 0) {
+            dot = dsum = 0.f;
+            for (int i = 0; i < kFThreads / 32; ++i) { dot += fin[0][i]; dsum += fin[1][i]; }
+            if (g.vec3) {
+                g.dbeta[co] = dsum;
+                if (g.db) g.db[co] = s * dsum;
+                g.dgamma[co] = g.vec3[2 * g.c_out + co] * (dot + dsum * ((g.b ? g.b[co] : 0.f) - g.mean[co]));
+            } else if (g.db) {
+                g.db[co] = dsum;
+            }
+        }
+    }
+    cluster.sync();          // a block's shared memory stays until its neighbours have read it
+}
+
+// blocks [0, nw): weight-gradient clusters; [nw, nw + nd): dX tiles (rounded up to whole clusters)
+template <int K, int R, int S>
+__global__ void __cluster_dims__(kFCluster, 1, 1) __launch_bounds__(kFThreads) f32_bwd_kernel(const F32Wgrad g, int nw, const F32Conv c,
+                                                                                          int oc_tiles) {
+    extern __shared__ __align__(16) float f32_smem[];
+    pdl_wait();
+    pdl_launch_dependents();
+    const int b = (int)blockIdx.x;
+    if (b < nw) {
+        wgrad_cluster<K>(g, (b / kFCluster) * kFCo, f32_smem);
+        return;
+    }
+    constexpr int OCT = S == 1 ? 4 * R : R;
+    const int i = b - nw, t = i / oc_tiles, img = t / c.tiles;
+    if (img < c.n) conv_tile<K, R, S, true>(c, (i - t * oc_tiles) * OCT, t - img * c.tiles, img, nullptr, nullptr, f32_smem);
+}
+
+// S = 4 while the 32-channel blocks of S = 1 would not give every SM two (16 -> 32 channels at 16 x 16, N = 2: 8 of them)
+bool split_channels(int n, int oc, int hw) {
+    return (long long)n * ((oc + 31) / 32) * ((hw + kFPix - 1) / kFPix) < 2LL * device_sm_count();
+}
+
+bool wgrad_geometry(const Problem &pb, F32Wgrad *g, size_t *bytes) {
+    g->n = pb.n; g->c_in = pb.c_in; g->h = pb.h_in; g->wd = pb.w_in; g->c_out = pb.c_out; g->ho = pb.h_out; g->wo = pb.w_out;
+    g->pad = pb.pad_h;
+    g->cip = 4;
+    while (g->cip < pb.c_in) g->cip *= 2;
+    g->zp = (pb.w_out + kFRun - 1) / kFRun * kFRun;
+    g->xp = g->zp + pb.kw - 1;
+    const size_t kk = (size_t)pb.kh * pb.kw, red = kFCo * (pb.c_in * kk + 1) + kFThreads * (kk + 1);
+    // the largest band of at most eight rows that leaves every block of a cluster one, within 96 KB (two blocks per SM)
+    for (int rows = pb.h_out < 8 ? pb.h_out : 8; rows >= 1; --rows) {
+        const int bands = (pb.h_out + rows - 1) / rows, x_ci = ((rows + pb.kh - 1) * g->xp) | 1;
+        size_t stage = (size_t)pb.c_in * x_ci + 1 + (size_t)kFCo * rows * g->zp;
+        if (stage < red) stage = red;
+        if (stage * sizeof(float) > 96 * 1024 && rows > 1) continue;
+        if ((long long)pb.n * bands < kFCluster && rows > 1) continue;
+        g->rows = rows; g->bands = bands; g->x_ci = x_ci;
+        *bytes = stage * sizeof(float);
+        return *bytes <= 200 * 1024;
+    }
+    return false;
+}
+
+template <class F>
+cudaError_t by_shape(int k, bool split, F f) {
+    using I1 = std::integral_constant<int, 1>;
+    using I3 = std::integral_constant<int, 3>;
+    using I4 = std::integral_constant<int, 4>;
+    using I8 = std::integral_constant<int, 8>;
+    if (k == 1) return split ? f(I1(), I4(), I4()) : f(I1(), I8(), I1());
+    return split ? f(I3(), I4(), I4()) : f(I3(), I8(), I1());
+}
+
+}  // namespace
+
+bool f32_conv_eligible(const Problem &pb) {
+    if (pb.groups != 1 || pb.kh != pb.kw || (pb.kh != 1 && pb.kh != 3) || pb.stride_h != 1 || pb.stride_w != 1 ||
+        pb.dil_h != 1 || pb.dil_w != 1 || pb.pad_h != pb.pad_w || pb.pad_h >= pb.kh || pb.c_in > 128 || pb.c_out > 128)
+        return false;
+    if (pb.n > 65535 || pb.pin * pb.c_in >= (1LL << 30) || pb.p * pb.c_out >= (1LL << 30)) return false;
+    F32Wgrad g;
+    size_t bytes;
+    return wgrad_geometry(pb, &g, &bytes);
+}
+
+cudaError_t launch_f32_fwd(const Problem &pb, const float *x, const float *w, const float *bias, float *z, cudaStream_t st,
+                           const BnFold *fold) {
+    F32Conv c{x, w, z, pb.n, pb.c_in, pb.h_in, pb.w_in, pb.c_out, pb.h_out, pb.w_out, pb.pad_h, nullptr, bias, 0};
+    c.tiles = (pb.h_out * pb.w_out + kFPix - 1) / kFPix;
+    const BnFold fd = fold ? *fold : BnFold{nullptr, nullptr, nullptr, nullptr, nullptr, 0.f, nullptr};
+    return by_shape(pb.kh, split_channels(pb.n, pb.c_out, pb.h_out * pb.w_out), [&](auto k, auto r, auto s) {
+        constexpr int K = decltype(k)::value, R = decltype(r)::value, S = decltype(s)::value, OCT = S == 1 ? 4 * R : R;
+        const size_t smem = conv_smem_floats(K * K, R, S, pb.c_in) * sizeof(float);
+        return launch_pdl(f32_fwd_kernel<K, R, S>, dim3(c.tiles, (c.oc + OCT - 1) / OCT, c.n), dim3(kFThreads), smem, st, c, fd);
+    });
+}
+
+cudaError_t launch_f32_bwd(const Problem &pb, const float *dz, const float *x, const float *w, const float *scale, float *dx,
+                           const float *vec3, const float *b, const float *mean, float *dw, float *db, float *dgamma,
+                           float *dbeta, cudaStream_t st) {
+    F32Wgrad g{};
+    size_t wbytes = 0;
+    if (!wgrad_geometry(pb, &g, &wbytes)) return cudaErrorInvalidValue;
+    g.x = x; g.dz = dz; g.w = w; g.vec3 = vec3; g.b = b; g.mean = mean; g.dw = dw; g.db = db; g.dgamma = dgamma; g.dbeta = dbeta;
+    // dX is a convolution of dZ with the rotated weights: padding k - 1 - pad
+    F32Conv c{dz, w, dx, pb.n, pb.c_out, pb.h_out, pb.w_out, pb.c_in, pb.h_in, pb.w_in, pb.kh - 1 - pb.pad_h, scale, nullptr, 0};
+    c.tiles = (pb.h_in * pb.w_in + kFPix - 1) / kFPix;
+    const int nw = dw ? (pb.c_out + kFCo - 1) / kFCo * kFCluster : 0;
+    return by_shape(pb.kh, split_channels(pb.n, pb.c_in, pb.h_in * pb.w_in), [&](auto k, auto r, auto s) {
+        constexpr int K = decltype(k)::value, R = decltype(r)::value, S = decltype(s)::value, OCT = S == 1 ? 4 * R : R;
+        const int oc_tiles = (c.oc + OCT - 1) / OCT;
+        const long long nd = dx ? ((long long)oc_tiles * c.tiles * c.n + kFCluster - 1) / kFCluster * kFCluster : 0;
+        size_t smem = nw ? wbytes : 0;
+        const size_t cbytes = conv_smem_floats(K * K, R, S, c.ic) * sizeof(float);
+        if (nd && cbytes > smem) smem = cbytes;
+        static PerDevice attr;
+        if (cudaError_t e = max_dynamic_smem_once(f32_bwd_kernel<K, R, S>, 200 * 1024, &attr); e != cudaSuccess) return e;
+        return launch_pdl(f32_bwd_kernel<K, R, S>, dim3((unsigned)(nw + nd)), dim3(kFThreads), smem, st, g, nw, c, oc_tiles);
+    });
+}
+
+}  // namespace convbn

@@ -31,6 +31,25 @@ int direct_wgrad_splits(const Problem &pb);
 cudaError_t launch_direct_wgrad(const Problem &pb, int dtype, int layout, const void *dz,
                                 const void *x, float *partials, int splits, cudaStream_t st);
 
+// BatchNorm parameters for in-kernel reparameterisation: the kernel forms s and b' per output channel,
+// computes out = s * (wmat (*) act) + b' and (CTA 0) writes [s | b' | r] to vec3 (3 cn floats, may be NULL).
+struct BnFold {
+    const float *gamma, *beta, *mean, *var, *b;   // b may be NULL
+    float eps;
+    float *vec3;
+};
+
+// ---- fp32 NCHW, unit stride and dilation, 1x1 or 3x3, at most 128 channels: one launch per direction (f32_kernels.cu) ----
+bool f32_conv_eligible(const Problem &pb);
+// out = w (*) x + bias, or with fold the Tune-mode block
+cudaError_t launch_f32_fwd(const Problem &pb, const float *x, const float *w, const float *bias, float *z, cudaStream_t st,
+                           const BnFold *fold = nullptr);
+// dx != NULL: dX = (scale omega)_rot (*) dZ (scale NULL = 1).  dw != NULL: the parameter gradients (vec3 NULL: dw =
+// domega', db = sum dZ if wanted).
+cudaError_t launch_f32_bwd(const Problem &pb, const float *dz, const float *x, const float *w, const float *scale, float *dx,
+                           const float *vec3, const float *b, const float *mean, float *dw, float *db, float *dgamma,
+                           float *dbeta, cudaStream_t st);
+
 // ---- tensor-core implicit-GEMM convolution (bf16 NHWC, groups = 1) -----------------------------
 // out[n,ho,wo,:cn] = bias + sum over taps (r,q) and channels c of
 //     act[n, lower_h + ho stride_h + r dil_h, lower_w + wo stride_w + q dil_w, c] * wmat[:, (r taps_w + q) ca + c]
@@ -61,13 +80,6 @@ struct UmmaConvShape {
     unsigned sub_mask[4] = {0, 0, 0, 0};
 };
 bool umma_conv_eligible(const UmmaConvShape &s);
-// BatchNorm parameters for in-kernel reparameterisation: the kernel forms s and b' per output channel,
-// computes out = s * (wmat (*) act) + b' and (CTA 0) writes [s | b' | r] to vec3 (3 cn floats, may be NULL).
-struct BnFold {
-    const float *gamma, *beta, *mean, *var, *b;   // b may be NULL
-    float eps;
-    float *vec3;
-};
 // fold != NULL replaces `bias` (dense output mode only).  With out2 (Eval mode) out = wmat (*) act + fold->b and
 // out2 = gamma (out - mean) / sqrt(var + eps) + beta from the rounded out; nothing is written to fold->vec3.
 cudaError_t launch_umma_conv(const UmmaConvShape &s, const void *act, const void *wmat, const float *bias,

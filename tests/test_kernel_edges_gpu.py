@@ -13,6 +13,14 @@ SPECS = [
     L("g8_chunks", 13, 704, 9, 10, 704, 3, 3, pad=1, groups=88, bias=True),
     L("g8_wide", 1, 64, 5, 254, 64, 3, 3, pad=1, groups=8, dtype="f16"),
     L("g8_last_row", 9, 128, 17, 29, 128, 3, 3, pad=1, groups=16),
+    # fp32 NCHW: one channel and one pixel row, 128 channels (nothing left for pixel groups), a plane of 64 pixels and one
+    # more, more bands than blocks of a cluster, output channels that end inside a block and inside a cluster
+    L("f32_tiny", 1, 1, 1, 5, 3, 3, 3, pad=1, dtype="f32", layout="nchw", bias=True),
+    L("f32_c128", 2, 128, 5, 13, 128, 3, 3, pad=1, dtype="f32", layout="nchw"),
+    L("f32_65", 3, 5, 13, 5, 9, 1, 1, dtype="f32", layout="nchw", bias=True),
+    L("f32_many", 16, 33, 40, 37, 35, 3, 3, pad=1, dtype="f32", layout="nchw"),
+    L("f32_nopad", 1, 20, 9, 30, 34, 3, 3, pad=0, dtype="f32", layout="nchw", bias=True),
+    L("f32_pad2", 1, 7, 6, 9, 6, 3, 3, pad=2, dtype="f32", layout="nchw"),
 ]
 
 
