@@ -53,6 +53,23 @@ class Desc(ctypes.Structure):
 _lib = None
 
 
+def _signatures():
+    """argtypes of the entry points that take pointers: ctypes then converts plain integers itself, without an object per
+    argument (d: descriptor, p: pointer or stream, z: size, i: int, q: long long, f: double)."""
+    kinds = {"d": ctypes.POINTER(Desc), "p": ctypes.c_void_p, "z": ctypes.c_size_t, "i": ctypes.c_int,
+             "q": ctypes.c_longlong, "f": ctypes.c_double}
+    table = {
+        "convbn_tune_fwd": "dppppppppppzp", "convbn_tune_bwd_data": "dpppppzp", "convbn_tune_bwd_weight": "dppppppppppp" "zp",
+        "convbn_tune_bwd": "dppppppppppppzp", "convbn_tune_bwd_begin": "dppppppppppppzp", "convbn_tune_bwd_join": "p",
+        "convbn_tconv_tune_fwd": "dppppppppppzp", "convbn_tconv_tune_bwd": "dppppppppppppzp",
+        "convbn_tune_bwd_weight_noalloc": "dppppppppppp", "convbn_eval_fwd": "dppppppppppzp",
+        "convbn_eval_bwd": "dpppppppppppppzp", "convbn_deploy_prepare": "dppppppppp", "convbn_deploy_fwd": "dpppppzp",
+        "convbn_deploy_bwd": "dpppppppzp", "convbn_relu": "ippqp", "convbn_add_relu": "ipppqp", "convbn_relu_bwd": "ipppqp",
+        "convbn_add": "ipppqp", "convbn_workspace_bytes": "di", "convbn_saved_bytes": "di", "convbn_check": "p",
+    }
+    return {name: [kinds[k] for k in sig] for name, sig in table.items()}
+
+
 def lib():
     """Load the compiled library (raises OSError with the build hint if it is absent)."""
     global _lib
@@ -68,29 +85,35 @@ def lib():
         L.convbn_last_kernel.restype = ctypes.c_char_p
         for name in EXPORTS:
             getattr(L, name)
+        for name, types in _signatures().items():
+            getattr(L, name).argtypes = types
         _lib = L
     return _lib
 
 
-def _ptr(t) -> ctypes.c_void_p:
-    if t is None:
-        return ctypes.c_void_p(None)
-    if isinstance(t, int):
-        return ctypes.c_void_p(t)
-    return ctypes.c_void_p(t.data_ptr())
+def _ptr(t):
+    """Address for a c_void_p parameter: a tensor's, an integer as it is, None for NULL."""
+    if t is None or type(t) is int:
+        return t
+    return t.data_ptr()
 
 
-def _stream(stream) -> ctypes.c_void_p:
+def _vp(t) -> ctypes.c_void_p:
+    """The same as an object, for entry points without declared argument types."""
+    return ctypes.c_void_p(_ptr(t))
+
+
+def _stream(stream):
     if stream is None:
         import torch
-        return ctypes.c_void_p(torch.cuda.current_stream().cuda_stream)
+        return torch._C._cuda_getCurrentRawStream(torch._C._cuda_getDevice())
     if isinstance(stream, int):
-        return ctypes.c_void_p(stream)
-    return ctypes.c_void_p(stream.cuda_stream)
+        return stream
+    return stream.cuda_stream
 
 
 def _nbytes(t) -> int:
-    return 0 if t is None else t.numel() * t.element_size()
+    return 0 if t is None else t.nbytes
 
 
 def _raise(status: int, where: str):
@@ -122,46 +145,46 @@ def convbn_linear_desc(rows: int, in_features: int, out_features: int, dtype: in
 
 
 def convbn_saved_bytes(desc: Desc, mode: int) -> int:
-    return int(lib().convbn_saved_bytes(ctypes.byref(desc), ctypes.c_int(mode)))
+    return int(lib().convbn_saved_bytes(desc, mode))
 
 
 def convbn_workspace_bytes(desc: Desc, phase: int) -> int:
-    return int(lib().convbn_workspace_bytes(ctypes.byref(desc), ctypes.c_int(phase)))
+    return int(lib().convbn_workspace_bytes(desc, phase))
 
 
 def convbn_tune_fwd(desc, x, w, b, gamma, beta, run_mean, run_var, z, saved, workspace=None,
                     workspace_bytes: Optional[int] = None, stream=None):
     wb = _nbytes(workspace) if workspace_bytes is None else workspace_bytes
-    _raise(lib().convbn_tune_fwd(ctypes.byref(desc), _ptr(x), _ptr(w), _ptr(b), _ptr(gamma),
+    _raise(lib().convbn_tune_fwd(desc, _ptr(x), _ptr(w), _ptr(b), _ptr(gamma),
                                  _ptr(beta), _ptr(run_mean), _ptr(run_var), _ptr(z), _ptr(saved),
-                                 _ptr(workspace), ctypes.c_size_t(wb), _stream(stream)),
+                                 _ptr(workspace), wb, _stream(stream)),
            "convbn_tune_fwd")
 
 
 def convbn_tune_bwd_data(desc, dz, w, saved, dx, workspace=None,
                          workspace_bytes: Optional[int] = None, stream=None):
     wb = _nbytes(workspace) if workspace_bytes is None else workspace_bytes
-    _raise(lib().convbn_tune_bwd_data(ctypes.byref(desc), _ptr(dz), _ptr(w), _ptr(saved), _ptr(dx),
-                                      _ptr(workspace), ctypes.c_size_t(wb), _stream(stream)),
+    _raise(lib().convbn_tune_bwd_data(desc, _ptr(dz), _ptr(w), _ptr(saved), _ptr(dx),
+                                      _ptr(workspace), wb, _stream(stream)),
            "convbn_tune_bwd_data")
 
 
 def convbn_tune_bwd_weight(desc, dz, x, w, b, run_mean, saved, dw, db, dgamma, dbeta,
                            workspace=None, workspace_bytes: Optional[int] = None, stream=None):
     wb = _nbytes(workspace) if workspace_bytes is None else workspace_bytes
-    _raise(lib().convbn_tune_bwd_weight(ctypes.byref(desc), _ptr(dz), _ptr(x), _ptr(w), _ptr(b),
+    _raise(lib().convbn_tune_bwd_weight(desc, _ptr(dz), _ptr(x), _ptr(w), _ptr(b),
                                         _ptr(run_mean), _ptr(saved), _ptr(dw), _ptr(db),
                                         _ptr(dgamma), _ptr(dbeta), _ptr(workspace),
-                                        ctypes.c_size_t(wb), _stream(stream)),
+                                        wb, _stream(stream)),
            "convbn_tune_bwd_weight")
 
 
 def convbn_tune_bwd(desc, dz, x, w, b, run_mean, saved, dx, dw, db, dgamma, dbeta, workspace=None,
                     workspace_bytes: Optional[int] = None, stream=None):
     wb = _nbytes(workspace) if workspace_bytes is None else workspace_bytes
-    _raise(lib().convbn_tune_bwd(ctypes.byref(desc), _ptr(dz), _ptr(x), _ptr(w), _ptr(b), _ptr(run_mean),
+    _raise(lib().convbn_tune_bwd(desc, _ptr(dz), _ptr(x), _ptr(w), _ptr(b), _ptr(run_mean),
                                  _ptr(saved), _ptr(dx), _ptr(dw), _ptr(db), _ptr(dgamma), _ptr(dbeta),
-                                 _ptr(workspace), ctypes.c_size_t(wb), _stream(stream)),
+                                 _ptr(workspace), wb, _stream(stream)),
            "convbn_tune_bwd")
 
 
@@ -169,9 +192,9 @@ def convbn_tune_bwd_begin(desc, dz, x, w, b, run_mean, saved, dx, dw, db, dgamma
                           workspace_bytes: Optional[int] = None, stream=None):
     """convbn_tune_bwd that returns with the parameter-gradient pass still running on the library's side lane."""
     wb = _nbytes(workspace) if workspace_bytes is None else workspace_bytes
-    _raise(lib().convbn_tune_bwd_begin(ctypes.byref(desc), _ptr(dz), _ptr(x), _ptr(w), _ptr(b), _ptr(run_mean),
+    _raise(lib().convbn_tune_bwd_begin(desc, _ptr(dz), _ptr(x), _ptr(w), _ptr(b), _ptr(run_mean),
                                        _ptr(saved), _ptr(dx), _ptr(dw), _ptr(db), _ptr(dgamma), _ptr(dbeta),
-                                       _ptr(workspace), ctypes.c_size_t(wb), _stream(stream)), "convbn_tune_bwd_begin")
+                                       _ptr(workspace), wb, _stream(stream)), "convbn_tune_bwd_begin")
 
 
 def convbn_tune_bwd_join(stream=None) -> None:
@@ -194,17 +217,17 @@ def convbn_tconv_workspace_bytes(desc) -> int:
 def convbn_tconv_tune_fwd(desc, x, w, b, gamma, beta, run_mean, run_var, z, saved, workspace=None,
                           workspace_bytes: Optional[int] = None, stream=None):
     wb = _nbytes(workspace) if workspace_bytes is None else workspace_bytes
-    _raise(lib().convbn_tconv_tune_fwd(ctypes.byref(desc), _ptr(x), _ptr(w), _ptr(b), _ptr(gamma), _ptr(beta),
+    _raise(lib().convbn_tconv_tune_fwd(desc, _ptr(x), _ptr(w), _ptr(b), _ptr(gamma), _ptr(beta),
                                        _ptr(run_mean), _ptr(run_var), _ptr(z), _ptr(saved), _ptr(workspace),
-                                       ctypes.c_size_t(wb), _stream(stream)), "convbn_tconv_tune_fwd")
+                                       wb, _stream(stream)), "convbn_tconv_tune_fwd")
 
 
 def convbn_tconv_tune_bwd(desc, dz, x, w, b, run_mean, saved, dx, dw, db, dgamma, dbeta, workspace=None,
                           workspace_bytes: Optional[int] = None, stream=None):
     wb = _nbytes(workspace) if workspace_bytes is None else workspace_bytes
-    _raise(lib().convbn_tconv_tune_bwd(ctypes.byref(desc), _ptr(dz), _ptr(x), _ptr(w), _ptr(b), _ptr(run_mean),
+    _raise(lib().convbn_tconv_tune_bwd(desc, _ptr(dz), _ptr(x), _ptr(w), _ptr(b), _ptr(run_mean),
                                        _ptr(saved), _ptr(dx), _ptr(dw), _ptr(db), _ptr(dgamma), _ptr(dbeta),
-                                       _ptr(workspace), ctypes.c_size_t(wb), _stream(stream)), "convbn_tconv_tune_bwd")
+                                       _ptr(workspace), wb, _stream(stream)), "convbn_tconv_tune_bwd")
 
 
 def convbn_tune_bwd_weight_noalloc(desc, dz, x, w, b, run_mean, saved, dw, db, dgamma, dbeta,
@@ -213,7 +236,7 @@ def convbn_tune_bwd_weight_noalloc(desc, dz, x, w, b, run_mean, saved, dw, db, d
     no workspace argument, the library's built-in 16 MiB scratch array is used instead.  Raises
     ConvBNError(ECAPACITY) when the layer needs more scratch than that.  Calls sharing a device
     must not overlap on it."""
-    _raise(lib().convbn_tune_bwd_weight_noalloc(ctypes.byref(desc), _ptr(dz), _ptr(x), _ptr(w),
+    _raise(lib().convbn_tune_bwd_weight_noalloc(desc, _ptr(dz), _ptr(x), _ptr(w),
                                                 _ptr(b), _ptr(run_mean), _ptr(saved), _ptr(dw),
                                                 _ptr(db), _ptr(dgamma), _ptr(dbeta), _stream(stream)),
            "convbn_tune_bwd_weight_noalloc")
@@ -222,24 +245,24 @@ def convbn_tune_bwd_weight_noalloc(desc, dz, x, w, b, run_mean, saved, dw, db, d
 def convbn_eval_fwd(desc, x, w, b, gamma, beta, run_mean, run_var, z, y_saved, workspace=None,
                     workspace_bytes: Optional[int] = None, stream=None):
     wb = _nbytes(workspace) if workspace_bytes is None else workspace_bytes
-    _raise(lib().convbn_eval_fwd(ctypes.byref(desc), _ptr(x), _ptr(w), _ptr(b), _ptr(gamma),
+    _raise(lib().convbn_eval_fwd(desc, _ptr(x), _ptr(w), _ptr(b), _ptr(gamma),
                                  _ptr(beta), _ptr(run_mean), _ptr(run_var), _ptr(z), _ptr(y_saved),
-                                 _ptr(workspace), ctypes.c_size_t(wb), _stream(stream)),
+                                 _ptr(workspace), wb, _stream(stream)),
            "convbn_eval_fwd")
 
 
 def convbn_eval_bwd(desc, dz, x, y_saved, w, gamma, run_mean, run_var, dx, dw, db, dgamma, dbeta,
                     workspace=None, workspace_bytes: Optional[int] = None, stream=None):
     wb = _nbytes(workspace) if workspace_bytes is None else workspace_bytes
-    _raise(lib().convbn_eval_bwd(ctypes.byref(desc), _ptr(dz), _ptr(x), _ptr(y_saved), _ptr(w),
+    _raise(lib().convbn_eval_bwd(desc, _ptr(dz), _ptr(x), _ptr(y_saved), _ptr(w),
                                  _ptr(gamma), _ptr(run_mean), _ptr(run_var), _ptr(dx), _ptr(dw),
                                  _ptr(db), _ptr(dgamma), _ptr(dbeta), _ptr(workspace),
-                                 ctypes.c_size_t(wb), _stream(stream)),
+                                 wb, _stream(stream)),
            "convbn_eval_bwd")
 
 
 def convbn_deploy_prepare(desc, w, b, gamma, beta, run_mean, run_var, w_fused, b_fused, stream=None):
-    _raise(lib().convbn_deploy_prepare(ctypes.byref(desc), _ptr(w), _ptr(b), _ptr(gamma), _ptr(beta),
+    _raise(lib().convbn_deploy_prepare(desc, _ptr(w), _ptr(b), _ptr(gamma), _ptr(beta),
                                        _ptr(run_mean), _ptr(run_var), _ptr(w_fused), _ptr(b_fused),
                                        _stream(stream)),
            "convbn_deploy_prepare")
@@ -248,17 +271,17 @@ def convbn_deploy_prepare(desc, w, b, gamma, beta, run_mean, run_var, w_fused, b
 def convbn_deploy_fwd(desc, x, w_fused, b_fused, z, workspace=None,
                       workspace_bytes: Optional[int] = None, stream=None):
     wb = _nbytes(workspace) if workspace_bytes is None else workspace_bytes
-    _raise(lib().convbn_deploy_fwd(ctypes.byref(desc), _ptr(x), _ptr(w_fused), _ptr(b_fused), _ptr(z),
-                                   _ptr(workspace), ctypes.c_size_t(wb), _stream(stream)),
+    _raise(lib().convbn_deploy_fwd(desc, _ptr(x), _ptr(w_fused), _ptr(b_fused), _ptr(z),
+                                   _ptr(workspace), wb, _stream(stream)),
            "convbn_deploy_fwd")
 
 
 def convbn_deploy_bwd(desc, dz, x, w_fused, dx, dw_fused, db_fused, workspace=None,
                       workspace_bytes: Optional[int] = None, stream=None):
     wb = _nbytes(workspace) if workspace_bytes is None else workspace_bytes
-    _raise(lib().convbn_deploy_bwd(ctypes.byref(desc), _ptr(dz), _ptr(x), _ptr(w_fused), _ptr(dx),
+    _raise(lib().convbn_deploy_bwd(desc, _ptr(dz), _ptr(x), _ptr(w_fused), _ptr(dx),
                                    _ptr(dw_fused), _ptr(db_fused), _ptr(workspace),
-                                   ctypes.c_size_t(wb), _stream(stream)),
+                                   wb, _stream(stream)),
            "convbn_deploy_bwd")
 
 
@@ -268,22 +291,22 @@ def _dtype_of(t) -> int:
 
 
 def convbn_relu(a, out, stream=None):
-    _raise(lib().convbn_relu(ctypes.c_int(_dtype_of(a)), _ptr(a), _ptr(out), ctypes.c_longlong(a.numel()), _stream(stream)),
+    _raise(lib().convbn_relu(_dtype_of(a), _ptr(a), _ptr(out), a.numel(), _stream(stream)),
            "convbn_relu")
 
 
 def convbn_add_relu(a, b, out, stream=None):
-    _raise(lib().convbn_add_relu(ctypes.c_int(_dtype_of(a)), _ptr(a), _ptr(b), _ptr(out), ctypes.c_longlong(a.numel()),
+    _raise(lib().convbn_add_relu(_dtype_of(a), _ptr(a), _ptr(b), _ptr(out), a.numel(),
                                  _stream(stream)), "convbn_add_relu")
 
 
 def convbn_relu_bwd(a, y, out, stream=None):
-    _raise(lib().convbn_relu_bwd(ctypes.c_int(_dtype_of(a)), _ptr(a), _ptr(y), _ptr(out), ctypes.c_longlong(a.numel()),
+    _raise(lib().convbn_relu_bwd(_dtype_of(a), _ptr(a), _ptr(y), _ptr(out), a.numel(),
                                  _stream(stream)), "convbn_relu_bwd")
 
 
 def convbn_add(a, b, out, stream=None):
-    _raise(lib().convbn_add(ctypes.c_int(_dtype_of(a)), _ptr(a), _ptr(b), _ptr(out), ctypes.c_longlong(a.numel()),
+    _raise(lib().convbn_add(_dtype_of(a), _ptr(a), _ptr(b), _ptr(out), a.numel(),
                             _stream(stream)), "convbn_add")
 
 
@@ -293,7 +316,7 @@ def convbn_check(stream=None) -> None:
 
 def convbn_selftest_wait_timeout(stream=None) -> None:
     """Queue the failure-path self-test: the next convbn_check() raises ConvBNError(ETIMEOUT)."""
-    _raise(lib().convbn_selftest_wait_timeout(_stream(stream)), "convbn_selftest_wait_timeout")
+    _raise(lib().convbn_selftest_wait_timeout(ctypes.c_void_p(_stream(stream))), "convbn_selftest_wait_timeout")
 
 
 def convbn_host_step_arena_bytes(desc: Desc) -> int:
@@ -304,11 +327,11 @@ def convbn_tune_step_host(desc, x, dz, w, b, gamma, beta, run_mean, run_var, z, 
                           dbeta, device_arena, arena_bytes: Optional[int] = None, stream=None):
     """All tensors but ``device_arena`` are HOST tensors (page-locked for asynchronous copies)."""
     ab = _nbytes(device_arena) if arena_bytes is None else arena_bytes
-    _raise(lib().convbn_tune_step_host(ctypes.byref(desc), _ptr(x), _ptr(dz), _ptr(w), _ptr(b),
-                                       _ptr(gamma), _ptr(beta), _ptr(run_mean), _ptr(run_var),
-                                       _ptr(z), _ptr(dx), _ptr(dw), _ptr(db), _ptr(dgamma),
-                                       _ptr(dbeta), _ptr(device_arena), ctypes.c_size_t(ab),
-                                       _stream(stream)),
+    _raise(lib().convbn_tune_step_host(ctypes.byref(desc), _vp(x), _vp(dz), _vp(w), _vp(b),
+                                       _vp(gamma), _vp(beta), _vp(run_mean), _vp(run_var),
+                                       _vp(z), _vp(dx), _vp(dw), _vp(db), _vp(dgamma),
+                                       _vp(dbeta), _vp(device_arena), ctypes.c_size_t(ab),
+                                       ctypes.c_void_p(_stream(stream))),
            "convbn_tune_step_host")
 
 
@@ -316,17 +339,17 @@ def convbn_tune_step_host_begin(desc, x, dz, w, b, gamma, beta, run_mean, run_va
                           dbeta, device_arena, arena_bytes: Optional[int] = None, stream=None):
     """All tensors but ``device_arena`` are HOST tensors (page-locked for asynchronous copies)."""
     ab = _nbytes(device_arena) if arena_bytes is None else arena_bytes
-    _raise(lib().convbn_tune_step_host_begin(ctypes.byref(desc), _ptr(x), _ptr(dz), _ptr(w), _ptr(b),
-                                       _ptr(gamma), _ptr(beta), _ptr(run_mean), _ptr(run_var),
-                                       _ptr(z), _ptr(dx), _ptr(dw), _ptr(db), _ptr(dgamma),
-                                       _ptr(dbeta), _ptr(device_arena), ctypes.c_size_t(ab),
-                                       _stream(stream)),
+    _raise(lib().convbn_tune_step_host_begin(ctypes.byref(desc), _vp(x), _vp(dz), _vp(w), _vp(b),
+                                       _vp(gamma), _vp(beta), _vp(run_mean), _vp(run_var),
+                                       _vp(z), _vp(dx), _vp(dw), _vp(db), _vp(dgamma),
+                                       _vp(dbeta), _vp(device_arena), ctypes.c_size_t(ab),
+                                       ctypes.c_void_p(_stream(stream))),
            "convbn_tune_step_host_begin")
 
 
 def convbn_tune_step_host_join(stream=None) -> None:
     """Make `stream` wait for the downloads of every convbn_tune_step_host_begin call of this thread on this device."""
-    _raise(lib().convbn_tune_step_host_join(_stream(stream)), "convbn_tune_step_host_join")
+    _raise(lib().convbn_tune_step_host_join(ctypes.c_void_p(_stream(stream))), "convbn_tune_step_host_join")
 
 
 def convbn_profile_begin() -> None:
