@@ -129,6 +129,16 @@ int convbn_tune_fwd(const convbn_desc *desc, const void *x, const void *w, const
                     const float *run_var, void *z, void *saved, void *workspace,
                     size_t workspace_bytes, void *stream);
 
+/* convbn_tune_fwd followed by what a residual network does with Z, in the convolution's own epilogue where its kernel is
+ * a tensor-core one (a pass of its own elsewhere):
+ *     z = max(Z + add, 0)      add [like z, 16-byte aligned] or NULL, no max with relu = 0
+ * Values and roundings are those of convbn_tune_fwd followed by convbn_relu / convbn_add_relu / convbn_add.  `add` may
+ * not overlap z.  Other arguments, workspace and errors as for convbn_tune_fwd. */
+int convbn_tune_fwd_glue(const convbn_desc *desc, const void *x, const void *w, const float *b,
+                         const float *gamma, const float *beta, const float *run_mean,
+                         const float *run_var, void *z, void *saved, const void *add, int relu,
+                         void *workspace, size_t workspace_bytes, void *stream);
+
 /* Backward, data:  dX = omega'_rot (*) dZ  (the transposed convolution of dZ with omega').
  * in : dz, w (the same omega given to the forward), saved (from convbn_tune_fwd)
  * out: dx, same shape as x.  Every element of dx is written. */
@@ -267,6 +277,16 @@ int convbn_tune_bwd_begin(const convbn_desc *desc, const void *dz, const void *x
                           const float *run_mean, const void *saved, void *dx, float *dw, float *db, float *dgamma,
                           float *dbeta, void *workspace, size_t workspace_bytes, void *stream);
 int convbn_tune_bwd_join(void *stream);
+
+/* convbn_tune_bwd (begin = 0) or convbn_tune_bwd_begin (begin = 1) followed by what a residual network does with dX, in the
+ * same way as convbn_tune_fwd_glue:
+ *     dx = dX + add            add [like dx, 16-byte aligned] or NULL: the gradient that arrives over the skip connection
+ *     dx = 0 where x <= 0      with relu_mask != 0: x is the output of the ReLU in front of the block
+ * Values and roundings are those of convbn_add and convbn_relu_bwd.  `add` may not overlap dx. */
+int convbn_tune_bwd_glue(const convbn_desc *desc, const void *dz, const void *x, const void *w, const float *b,
+                         const float *run_mean, const void *saved, void *dx, float *dw, float *db, float *dgamma,
+                         float *dbeta, const void *add, int relu_mask, int begin, void *workspace,
+                         size_t workspace_bytes, void *stream);
 
 /* ---- TransposedConv-BN in Tune mode (Sec. 3.2.2: the rewrite holds for any linear layer in front of a frozen BatchNorm;
  *      Sec. 3.3 definitions; Table 2, Tune row, with the transposed convolution in place of the convolution) ------------

@@ -57,6 +57,11 @@ class _Layer:
         self.blk = Block(spec, device=device, modes=(mode,), allocate="params")
         self.blk.randomize_params(seed)
         self.mode = mode
+        if mode == "tune":          # sizes of what the passes allocate (functions of the descriptor and the device)
+            with torch.cuda.device(self.blk.device):
+                self.saved_bytes = max(16, C.convbn_saved_bytes(self.blk.desc, C.MODE_TUNE))
+                self.fwd_bytes = max(256, C.convbn_workspace_bytes(self.blk.desc, C.PHASE_TUNE_FWD))
+                self.bwd_bytes = max(256, C.convbn_workspace_bytes(self.blk.desc, C.PHASE_TUNE_BWD))
         if mode == "deploy":
             b = self.blk
             b.w_fused = torch.empty_like(b.w)
@@ -67,43 +72,58 @@ class _Layer:
         self.out_elems = n * c_out * self.blk.h_out * self.blk.w_out
         self.in_elems = n * c_in * hw[0] * hw[1]
 
-    def forward(self, x):
+    def forward(self, x, add=None, relu=False):
+        """The block's output, or max(output + add, 0): in Tune mode the addend and the ReLU are part of the block's own
+        kernel, otherwise they are passes of their own."""
         b = self.blk
         b.x = x
-        b.z = torch.empty(self.out_elems, dtype=b.tdtype, device=b.device)
+        z = torch.empty(self.out_elems, dtype=b.tdtype, device=b.device)
         if self.mode == "tune":
-            b.saved = torch.empty(max(16, C.convbn_saved_bytes(b.desc, C.MODE_TUNE)), dtype=torch.uint8, device=b.device)
-            b.with_scratch(C.PHASE_TUNE_FWD, b.tune_fwd)
-        elif self.mode == "eval":
+            b.saved = torch.empty(self.saved_bytes, dtype=torch.uint8, device=b.device)
+            ws = torch.empty(self.fwd_bytes, dtype=torch.uint8, device=b.device)
+            C.convbn_tune_fwd_glue(b.desc, x, b.w, b.b, b.gamma, b.beta, b.mu_hat, b.var_hat, z, b.saved, add, relu, ws,
+                                   self.fwd_bytes)
+            return z
+        b.z = z
+        if self.mode == "eval":
             b.y_saved = torch.empty(C.convbn_saved_bytes(b.desc, C.MODE_EVAL), dtype=torch.uint8, device=b.device)
             b.with_scratch(C.PHASE_EVAL_FWD, b.eval_fwd)
         else:
             b.with_scratch(C.PHASE_DEPLOY_FWD, b.deploy_fwd)
-        z, b.z = b.z, None
+        b.z = None
+        if add is not None:
+            (C.convbn_add_relu if relu else C.convbn_add)(z, add, z)
+        elif relu:
+            C.convbn_relu(z, z)
         return z
 
-    def backward(self, dz, held=None):
-        """Gradient with respect to the block's input; drops what the block kept for it.  With `held` (a list, Tune
-        mode) the parameter-gradient pass stays on the library's side stream: what it still reads (dZ, X, the saved
-        vectors, the scratch) is parked in `held` until the caller has joined."""
+    def backward(self, dz, held=None, add=None, relu_mask=False):
+        """Gradient with respect to the block's input, plus `add`, and with `relu_mask` zero where the input (the output
+        of a ReLU) is not positive; drops what the block kept for it.  With `held` (a list, Tune mode) the
+        parameter-gradient pass stays on the library's side stream: what it still reads (dZ, X, the saved vectors, the
+        scratch) is parked in `held` until the caller has joined."""
         b = self.blk
-        b.dz = dz
-        b.dx = torch.empty(self.in_elems, dtype=b.tdtype, device=b.device)
-        if self.mode == "tune" and held is not None:
-            b.workspace = torch.empty(max(256, C.convbn_workspace_bytes(b.desc, C.PHASE_TUNE_BWD)), dtype=torch.uint8,
-                                      device=b.device)
-            b.tune_bwd_begin()
-            held.append((b.workspace, b.saved, b.x, b.dz))
-            b.workspace = b.saved = None
-        elif self.mode == "tune":
-            b.with_scratch(C.PHASE_TUNE_BWD, b.tune_bwd)
+        dx = torch.empty(self.in_elems, dtype=b.tdtype, device=b.device)
+        x, b.x = b.x, None
+        if self.mode == "tune":
+            ws = torch.empty(self.bwd_bytes, dtype=torch.uint8, device=b.device)
+            C.convbn_tune_bwd_glue(b.desc, dz, x, b.w, b.b, b.mu_hat, b.saved, dx, b.dw, b.db, b.dgamma, b.dbeta, add,
+                                   relu_mask, held is not None, ws, self.bwd_bytes)
+            if held is not None:
+                held.append((ws, b.saved, x, dz))
             b.saved = None
-        elif self.mode == "eval":
+            return dx
+        b.dz, b.dx, b.x = dz, dx, x
+        if self.mode == "eval":
             b.with_scratch(C.PHASE_EVAL_BWD, b.eval_bwd)
             b.y_saved = None
         else:
             b.with_scratch(C.PHASE_DEPLOY_BWD, b.deploy_bwd)
-        dx, b.dx, b.dz, b.x = b.dx, None, None, None
+        b.dx = b.dz = b.x = None
+        if add is not None:
+            C.convbn_add(dx, add, dx)
+        if relu_mask:
+            C.convbn_relu_bwd(dx, x, dx)
         return dx
 
 
@@ -156,48 +176,42 @@ class BackboneReplay:
         every ReLU output (whose signs are the decisions a comparison has to share)."""
         relu_outs = []
         if self.stem:
-            s = self.stem.forward(ins["image"])
-            C.convbn_relu(s, s)
+            s = self.stem.forward(ins["image"], relu=True)
         x = ins["x"]
         for c1, c2, c3, ds in self.blocks:
-            a = c1.forward(x); C.convbn_relu(a, a)
-            b = c2.forward(a); C.convbn_relu(b, b)
-            c = c3.forward(b)
-            idt = ds.forward(x) if ds is not None else x
-            C.convbn_add_relu(c, idt, c)                       # out = relu(c + idt), in place in c's buffer
+            a = c1.forward(x, relu=True)
+            b = c2.forward(a, relu=True)
+            c = c3.forward(b, add=ds.forward(x) if ds is not None else x, relu=True)    # out = relu(c3(b) + identity)
             relu_outs.append((x, a, b, c))
             if keep is not None:
                 keep.setdefault("relu_outputs", []).append((a.clone(), b.clone(), c.clone()))
             x = c
-            del idt
         if keep is not None:
             keep["out"] = x.clone()
-        g = ins["g"].clone()
+        g = torch.empty_like(ins["g"])
+        C.convbn_relu_bwd(ins["g"], x, g)                      # through the last block's ReLU
+        del x, a, b, c
         # Tune mode: the parameter gradients of a bottleneck's blocks run beside its input-gradient chain and are
         # joined once per bottleneck, after which what they were reading can be released
         held = [] if self.mode == "tune" and self.async_param_grads else None
-        for (c1, c2, c3, ds), (xin, a, b, out) in zip(reversed(self.blocks), reversed(relu_outs)):
-            C.convbn_relu_bwd(g, out, g)                       # through the block's final ReLU; g feeds both branches
-            gb = c3.backward(g, held); C.convbn_relu_bwd(gb, b, gb)
-            ga = c2.backward(gb, held); C.convbn_relu_bwd(ga, a, ga)
-            gx = c1.backward(ga, held)
-            if ds is not None:
-                gs = ds.backward(g, held)
-                C.convbn_add(gx, gs, gx)
-                del gs
-            else:
-                C.convbn_add(gx, g, gx)
+        for i in range(len(self.blocks) - 1, -1, -1):
+            c1, c2, c3, ds = self.blocks[i]
+            relu_outs.pop()
+            gb = c3.backward(g, held, relu_mask=True)
+            ga = c2.backward(gb, held, relu_mask=True)
+            del gb
+            gs = ds.backward(g, held) if ds is not None else g
+            # the two branches meet; the input of every block but the first is the ReLU output of the block below
+            g = c1.backward(ga, held, add=gs, relu_mask=i > 0)
+            del ga, gs
             if held is not None:
                 C.convbn_tune_bwd_join()
                 held.clear()
-            g = gx
-            del gb, ga
-        relu_outs.clear()
         if keep is not None:
             keep["dx"] = g.clone()
         if self.stem:
-            gs = ins["g_stem"].clone()
-            C.convbn_relu_bwd(gs, s, gs)
+            gs = torch.empty_like(ins["g_stem"])
+            C.convbn_relu_bwd(ins["g_stem"], s, gs)
             gi = self.stem.backward(gs)
             if keep is not None:
                 keep["d_image"] = gi.clone()

@@ -26,7 +26,7 @@ EXPORTS = (
     "convbn_status_string", "convbn_last_kernel", "convbn_host_step_arena_bytes",
     "convbn_tune_step_host", "convbn_tune_step_host_begin", "convbn_tune_step_host_join", "convbn_profile_begin", "convbn_profile_end",
     "convbn_tune_bwd_weight_noalloc", "convbn_selftest_wait_timeout", "convbn_tune_bwd", "convbn_linear_desc", "convbn_relu", "convbn_add_relu", "convbn_relu_bwd", "convbn_add",
-    "convbn_tune_bwd_begin", "convbn_tune_bwd_join",
+    "convbn_tune_bwd_begin", "convbn_tune_bwd_join", "convbn_tune_fwd_glue", "convbn_tune_bwd_glue",
     "convbn_tconv_out_shape", "convbn_tconv_workspace_bytes", "convbn_tconv_tune_fwd", "convbn_tconv_tune_bwd",
 )
 
@@ -61,6 +61,7 @@ def _signatures():
     table = {
         "convbn_tune_fwd": "dppppppppppzp", "convbn_tune_bwd_data": "dpppppzp", "convbn_tune_bwd_weight": "dppppppppppp" "zp",
         "convbn_tune_bwd": "dppppppppppppzp", "convbn_tune_bwd_begin": "dppppppppppppzp", "convbn_tune_bwd_join": "p",
+        "convbn_tune_fwd_glue": "dppppppppppipzp", "convbn_tune_bwd_glue": "dppppppppppppiipzp",
         "convbn_tconv_tune_fwd": "dppppppppppzp", "convbn_tconv_tune_bwd": "dppppppppppppzp",
         "convbn_tune_bwd_weight_noalloc": "dppppppppppp", "convbn_eval_fwd": "dppppppppppzp",
         "convbn_eval_bwd": "dpppppppppppppzp", "convbn_deploy_prepare": "dppppppppp", "convbn_deploy_fwd": "dpppppzp",
@@ -200,6 +201,24 @@ def convbn_tune_bwd_begin(desc, dz, x, w, b, run_mean, saved, dx, dw, db, dgamma
 def convbn_tune_bwd_join(stream=None) -> None:
     """Make `stream` wait for every parameter-gradient pass begun by this thread on the current device."""
     _raise(lib().convbn_tune_bwd_join(_stream(stream)), "convbn_tune_bwd_join")
+
+
+def convbn_tune_fwd_glue(desc, x, w, b, gamma, beta, run_mean, run_var, z, saved, add, relu, workspace=None,
+                         workspace_bytes: Optional[int] = None, stream=None):
+    """convbn_tune_fwd with the addend and the ReLU of a residual network in its epilogue."""
+    wb = _nbytes(workspace) if workspace_bytes is None else workspace_bytes
+    _raise(lib().convbn_tune_fwd_glue(desc, _ptr(x), _ptr(w), _ptr(b), _ptr(gamma), _ptr(beta), _ptr(run_mean),
+                                      _ptr(run_var), _ptr(z), _ptr(saved), _ptr(add), 1 if relu else 0, _ptr(workspace), wb,
+                                      _stream(stream)), "convbn_tune_fwd_glue")
+
+
+def convbn_tune_bwd_glue(desc, dz, x, w, b, run_mean, saved, dx, dw, db, dgamma, dbeta, add, relu_mask, begin,
+                         workspace=None, workspace_bytes: Optional[int] = None, stream=None):
+    """convbn_tune_bwd (or, with `begin`, convbn_tune_bwd_begin) with dx += add and the mask x > 0 in its epilogue."""
+    wb = _nbytes(workspace) if workspace_bytes is None else workspace_bytes
+    _raise(lib().convbn_tune_bwd_glue(desc, _ptr(dz), _ptr(x), _ptr(w), _ptr(b), _ptr(run_mean), _ptr(saved), _ptr(dx),
+                                      _ptr(dw), _ptr(db), _ptr(dgamma), _ptr(dbeta), _ptr(add), 1 if relu_mask else 0,
+                                      1 if begin else 0, _ptr(workspace), wb, _stream(stream)), "convbn_tune_bwd_glue")
 
 
 def convbn_tconv_out_shape(desc):

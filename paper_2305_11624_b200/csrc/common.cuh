@@ -81,6 +81,25 @@ __device__ __forceinline__ void unpack2_t(uint32_t bits, float &lo, float &hi) {
     if constexpr (F16) { const float2 f = __half22float2(*reinterpret_cast<const __half2 *>(&bits)); lo = f.x; hi = f.y; }
     else { lo = __uint_as_float(bits << 16); hi = __uint_as_float(bits & 0xFFFF0000u); }
 }
+// max(v, 0) of two finite 16-bit values: a set sign bit clears its half
+__device__ __forceinline__ uint32_t relu2_h16(uint32_t v) { return v & ~(((v >> 15) & 0x00010001u) * 0xFFFFu); }
+// What a residual network does next with a block's result, on eight 16-bit values: v + a (rounded again, as an add of two
+// stored tensors is), max(v, 0), v where m > 0 and 0 elsewhere.
+template <bool F16>
+__device__ __forceinline__ uint4 post_chunk(uint4 v, bool add, const uint4 &a, bool relu, bool mask, const uint4 &m) {
+    uint32_t vw[4] = {v.x, v.y, v.z, v.w};
+    const uint32_t aw[4] = {a.x, a.y, a.z, a.w}, mw[4] = {m.x, m.y, m.z, m.w};
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+        float lo, hi, l2, h2;
+        unpack2_t<F16>(vw[i], lo, hi);
+        if (add) { unpack2_t<F16>(aw[i], l2, h2); lo += l2; hi += h2; }
+        if (relu) { lo = fmaxf(lo, 0.f); hi = fmaxf(hi, 0.f); }
+        if (mask) { unpack2_t<F16>(mw[i], l2, h2); lo = l2 > 0.f ? lo : 0.f; hi = h2 > 0.f ? hi : 0.f; }
+        vw[i] = pack2_t<F16>(lo, hi);
+    }
+    return make_uint4(vw[0], vw[1], vw[2], vw[3]);
+}
 __device__ __forceinline__ uint16_t pack1_h16(float a, int f16) {
     if (f16) { const __half h = __float2half_rn(a); return *reinterpret_cast<const uint16_t *>(&h); }
     const __nv_bfloat16 h = __float2bfloat16_rn(a);

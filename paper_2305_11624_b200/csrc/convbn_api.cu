@@ -450,7 +450,10 @@ int run_conv_fwd(const convbn_desc *d, const Problem &pb, const void *x, const v
 // w_scratch receives omega' in the layout the chosen kernel wants.
 int run_conv_dgrad(const convbn_desc *d, const Problem &pb, const void *dz, const void *w, const float *scale,
                    void *w_scratch, void *wbd_scratch, void *dx, cudaStream_t st, const char **which,
-                   const float *out_bias = nullptr, bool *bias_done = nullptr) {
+                   const float *out_bias = nullptr, bool *bias_done = nullptr, const PostOp *post = nullptr,
+                   bool *post_done = nullptr) {
+    // post (optional): applied to dX by the tensor-core paths; *post_done says whether it was
+    if (post_done) *post_done = false;
     // out_bias (C_in floats, optional): added to dX by the paths whose epilogue can do it; *bias_done says whether it was
     // (the transposed-convolution forward pass is this pass plus a bias)
     if (bias_done) *bias_done = false;
@@ -486,7 +489,8 @@ int run_conv_dgrad(const convbn_desc *d, const Problem &pb, const void *dz, cons
         // stride 2: the four parity classes of the input position as column blocks of ONE stride-1
         // convolution over dZ (one launch, the dZ patch staged once, absent taps skipped)
         LAUNCH("subpixel_weights", launch_subpixel_weights(pb, w, scale, w_scratch, st));
-        LAUNCH("strip_dgrad", launch_umma_strip_conv(s, dz, w_scratch, nullptr, dx, st));
+        LAUNCH("strip_dgrad", launch_umma_strip_conv(s, dz, w_scratch, nullptr, dx, st, nullptr, post));
+        if (post_done) *post_done = true;
         *which = "umma-subpixel";
     } else if (strided_dgrad_ok(d, pb)) {
         // Strided backward data, one stride-1 GEMM per residue class (a, b) of the input position:
@@ -520,6 +524,9 @@ int run_conv_dgrad(const convbn_desc *d, const Problem &pb, const void *dz, cons
                 }
             LAUNCH("reparam_dgrad", launch_reparam_dgrad_classes(pb, w, scale, w_scratch, where, st));
         }
+        // (positions that no class writes keep the zero of the memset: a mask leaves it, an addend would not)
+        const bool here = post && post->any() && !(any_empty && (post->add || post->relu));
+        if (post_done) *post_done = here;
         size_t woff = 0;
         for (int a = 0; a < pb.stride_h && a < pb.h_in; ++a)
             for (int b2 = 0; b2 < pb.stride_w && b2 < pb.w_in; ++b2) {
@@ -539,20 +546,26 @@ int run_conv_dgrad(const convbn_desc *d, const Problem &pb, const void *dz, cons
                 if (!merged)
                     LAUNCH("reparam_dgrad", launch_reparam_dgrad_class(pb, w, scale, wc, ch.count, cw.count, ch.r_max,
                                                                        cw.r_max, pb.stride_h, pb.stride_w, st));
-                LAUNCH("umma_dgrad", launch_umma_conv(cs, dz, wc, nullptr,
-                                                      (char *)dx + ((size_t)a * pb.w_in + b2) * pb.c_in *
-                                                                       elem_size(d->dtype), st));
+                const size_t coff = ((size_t)a * pb.w_in + b2) * pb.c_in * elem_size(d->dtype);
+                PostOp cp;
+                if (here) {
+                    cp = *post;
+                    if (cp.add) cp.add = (const char *)cp.add + coff;
+                    if (cp.mask) cp.mask = (const char *)cp.mask + coff;
+                }
+                LAUNCH("umma_dgrad", launch_umma_conv(cs, dz, wc, nullptr, (char *)dx + coff, st, nullptr, nullptr, &cp));
             }
         *which = "umma-strided";
     } else if (umma_dgrad_shape(d, pb, &s)) {
         LAUNCH("reparam_dgrad", launch_reparam_dgrad(pb, w, scale, w_scratch, st));
         if (umma_strip_eligible(s)) {
-            LAUNCH("strip_dgrad", launch_umma_strip_conv(s, dz, w_scratch, out_bias, dx, st));
+            LAUNCH("strip_dgrad", launch_umma_strip_conv(s, dz, w_scratch, out_bias, dx, st, nullptr, post));
             *which = "umma-strip";
         } else {
-            LAUNCH("umma_dgrad", launch_umma_conv(s, dz, w_scratch, out_bias, dx, st));
+            LAUNCH("umma_dgrad", launch_umma_conv(s, dz, w_scratch, out_bias, dx, st, nullptr, nullptr, post));
             *which = "umma";
         }
+        if (post_done) *post_done = true;
         if (bias_done && out_bias) *bias_done = true;
     } else if (dw_path(d, pb)) {
         if (pb.stride_h == 1 && pb.stride_w == 1) {
@@ -591,6 +604,15 @@ int run_conv_dgrad(const convbn_desc *d, const Problem &pb, const void *dz, cons
         LAUNCH("direct_dgrad", launch_direct_dgrad(pb, d->dtype, d->layout, dz, wd, dx, st));
         *which = "direct";
     }
+    return CONVBN_OK;
+}
+
+// The fused glue of `post` as passes of its own over t, for the paths whose epilogue does not do it.
+int run_post(const convbn_desc *d, const PostOp &post, void *t, long long count, cudaStream_t st) {
+    const int dtype = d->dtype == CONVBN_BF16 && call_f16() ? CONVBN_F16 : d->dtype;
+    if (post.add) LAUNCH("glue", launch_glue(post.relu ? 1 : 3, dtype, t, post.add, t, count, st));
+    else if (post.relu) LAUNCH("glue", launch_glue(0, dtype, t, nullptr, t, count, st));
+    if (post.mask) LAUNCH("glue", launch_glue(2, dtype, t, post.mask, t, count, st));
     return CONVBN_OK;
 }
 
@@ -712,10 +734,9 @@ size_t convbn_workspace_bytes(const convbn_desc *desc, int phase) {
     return make_plan(desc, pb, phase).total;
 }
 
-int convbn_tune_fwd(const convbn_desc *desc, const void *x, const void *w, const float *b,
-                    const float *gamma, const float *beta, const float *run_mean,
-                    const float *run_var, void *z, void *saved, void *workspace,
-                    size_t workspace_bytes, void *stream) {
+static int tune_fwd_impl(const convbn_desc *desc, const void *x, const void *w, const float *b, const float *gamma,
+                         const float *beta, const float *run_mean, const float *run_var, void *z, void *saved,
+                         const PostOp &post, void *workspace, size_t workspace_bytes, void *stream) {
     HalfCall half(desc);              // CONVBN_F16: checked here, then run as the 16-bit path with the half flag set
     if (half.status != CONVBN_OK) return half.status;
     desc = half.use;
@@ -726,19 +747,20 @@ int convbn_tune_fwd(const convbn_desc *desc, const void *x, const void *w, const
     if (!x || !w || !gamma || !beta || !run_mean || !run_var || !z || !saved) return CONVBN_EINVAL;
     if (!aligned(x, 16) || !aligned(w, 16) || !aligned(z, 16) || !aligned(saved, 16) ||
         !aligned(b, 4) || !aligned(gamma, 4) || !aligned(beta, 4) || !aligned(run_mean, 4) ||
-        !aligned(run_var, 4))
+        !aligned(run_var, 4) || !aligned(post.add, 16))
         return CONVBN_EALIGN;
     const Plan pl = make_plan(desc, pb, CONVBN_PHASE_TUNE_FWD);
     CK(check_ws(pl, workspace, workspace_bytes));
     cudaStream_t st = (cudaStream_t)stream;
     float *vec3 = (float *)saved;
     void *wf = at(workspace, pl.w_scaled);
+    const long long count = pb.p * pb.c_out;
     UmmaConvShape us;
     if (pl.stem && stem_window_eligible(pb)) {
         const BnFold fold{gamma, beta, run_mean, run_var, b, pb.eps, vec3};
-        LAUNCH("stem_fwd", launch_stem_window_fwd(pb, x, w, nullptr, z, st, &fold));
+        LAUNCH("stem_fwd", launch_stem_window_fwd(pb, x, w, nullptr, z, st, &fold, post.relu && !post.add));
         t_last_kernel[CONVBN_PHASE_TUNE_FWD] = "umma-stem";
-        return CONVBN_OK;
+        return post.add ? run_post(desc, post, z, count, st) : CONVBN_OK;
     }
     if (pl.stem) {
         const BnFold fold{gamma, beta, run_mean, run_var, b, pb.eps, vec3};
@@ -746,17 +768,17 @@ int convbn_tune_fwd(const convbn_desc *desc, const void *x, const void *w, const
         LAUNCH("stem_expand", launch_stem_expand_weights(pb, w, nullptr, at(workspace, pl.wst), st));
         LAUNCH("stem_fwd", launch_stem_fwd(pb, at(workspace, pl.xpk), at(workspace, pl.wst), nullptr, z, st, &fold));
         t_last_kernel[CONVBN_PHASE_TUNE_FWD] = "umma-stem";
-        return CONVBN_OK;
+        return run_post(desc, post, z, count, st);
     }
     if (!grouped_path(desc, pb) && umma_fwd_shape(desc, pb, &us)) {
         // dense tensor-core path: s, b' and the saved vectors are formed inside the GEMM kernel and s is
         // applied to the fp32 accumulator, so one launch does the whole forward pass
         const BnFold fold{gamma, beta, run_mean, run_var, b, pb.eps, vec3};
         if (umma_strip_eligible(us)) {
-            LAUNCH("strip_fwd", launch_umma_strip_conv(us, x, w, nullptr, z, st, &fold));
+            LAUNCH("strip_fwd", launch_umma_strip_conv(us, x, w, nullptr, z, st, &fold, &post));
             t_last_kernel[CONVBN_PHASE_TUNE_FWD] = "umma-strip";
         } else {
-            LAUNCH("umma_fwd", launch_umma_conv(us, x, w, nullptr, z, st, &fold));
+            LAUNCH("umma_fwd", launch_umma_conv(us, x, w, nullptr, z, st, &fold, nullptr, &post));
             t_last_kernel[CONVBN_PHASE_TUNE_FWD] = "umma";
         }
         return CONVBN_OK;
@@ -766,28 +788,43 @@ int convbn_tune_fwd(const convbn_desc *desc, const void *x, const void *w, const
         const BnFold fold{gamma, beta, run_mean, run_var, b, pb.eps, vec3};
         LAUNCH("dw_fwd", launch_dw_tma(pb, x, w, nullptr, z, st, &fold));
         t_last_kernel[CONVBN_PHASE_TUNE_FWD] = "depthwise";
-        return CONVBN_OK;
+        return run_post(desc, post, z, count, st);
     }
     if (f32_path(desc, pb)) {
         const BnFold fold{gamma, beta, run_mean, run_var, b, pb.eps, vec3};
         LAUNCH("direct_fwd", launch_f32_fwd(pb, (const float *)x, (const float *)w, nullptr, (float *)z, st, &fold));
         t_last_kernel[CONVBN_PHASE_TUNE_FWD] = "direct";
-        return CONVBN_OK;
+        return run_post(desc, post, z, count, st);
     }
     if (grouped_path(desc, pb) && grouped8_eligible(pb)) {
         const BnFold fold{gamma, beta, run_mean, run_var, b, pb.eps, vec3};
         LAUNCH("grouped_fwd", launch_grouped8_fwd(pb, x, w, nullptr, z, st, &fold));
         t_last_kernel[CONVBN_PHASE_TUNE_FWD] = "grouped-mma";
-        return CONVBN_OK;
+        return run_post(desc, post, z, count, st);
     }
     LAUNCH("reparam", launch_reparam(pb, desc->dtype, desc->layout, w, b, gamma, beta, run_mean, run_var, vec3, wf,
                       nullptr, st));
     CK(run_conv_fwd(desc, pb, x, wf, vec3 + pb.c_out, z, pl, workspace, st, &t_last_kernel[CONVBN_PHASE_TUNE_FWD]));
-    return CONVBN_OK;
+    return run_post(desc, post, z, count, st);
 }
 
-int convbn_tune_bwd_data(const convbn_desc *desc, const void *dz, const void *w, const void *saved,
-                         void *dx, void *workspace, size_t workspace_bytes, void *stream) {
+int convbn_tune_fwd(const convbn_desc *desc, const void *x, const void *w, const float *b, const float *gamma,
+                    const float *beta, const float *run_mean, const float *run_var, void *z, void *saved, void *workspace,
+                    size_t workspace_bytes, void *stream) {
+    return tune_fwd_impl(desc, x, w, b, gamma, beta, run_mean, run_var, z, saved, PostOp(), workspace, workspace_bytes, stream);
+}
+
+int convbn_tune_fwd_glue(const convbn_desc *desc, const void *x, const void *w, const float *b, const float *gamma,
+                         const float *beta, const float *run_mean, const float *run_var, void *z, void *saved,
+                         const void *add, int relu, void *workspace, size_t workspace_bytes, void *stream) {
+    PostOp post;
+    post.add = add;
+    post.relu = relu ? 1 : 0;
+    return tune_fwd_impl(desc, x, w, b, gamma, beta, run_mean, run_var, z, saved, post, workspace, workspace_bytes, stream);
+}
+
+static int tune_bwd_data_impl(const convbn_desc *desc, const void *dz, const void *w, const void *saved, void *dx,
+                              const PostOp &post, void *workspace, size_t workspace_bytes, void *stream) {
     HalfCall half(desc);              // CONVBN_F16: checked here, then run as the 16-bit path with the half flag set
     if (half.status != CONVBN_OK) return half.status;
     desc = half.use;
@@ -802,9 +839,15 @@ int convbn_tune_bwd_data(const convbn_desc *desc, const void *dz, const void *w,
     CK(check_ws(pl, workspace, workspace_bytes));
     cudaStream_t st = (cudaStream_t)stream;
     void *wf = at(workspace, pl.w_scaled);
+    bool post_done = false;
     CK(run_conv_dgrad(desc, pb, dz, w, (const float *)saved, wf, at(workspace, pl.wbd), dx, st,
-                      &t_last_kernel[CONVBN_PHASE_TUNE_BWD_DATA]));
-    return CONVBN_OK;
+                      &t_last_kernel[CONVBN_PHASE_TUNE_BWD_DATA], nullptr, nullptr, &post, &post_done));
+    return post_done ? CONVBN_OK : run_post(desc, post, dx, pb.pin * pb.c_in, st);
+}
+
+int convbn_tune_bwd_data(const convbn_desc *desc, const void *dz, const void *w, const void *saved, void *dx, void *workspace,
+                         size_t workspace_bytes, void *stream) {
+    return tune_bwd_data_impl(desc, dz, w, saved, dx, PostOp(), workspace, workspace_bytes, stream);
 }
 
 int convbn_tune_bwd_weight(const convbn_desc *desc, const void *dz, const void *x, const void *w,
@@ -884,7 +927,8 @@ int side_by_side(cudaStream_t st, Side &&side, Main &&main_pass) {
 extern "C" {
 static int tune_bwd_impl(const convbn_desc *desc, const void *dz, const void *x, const void *w, const float *b,
                          const float *run_mean, const void *saved, void *dx, float *dw, float *db, float *dgamma,
-                         float *dbeta, void *workspace, size_t workspace_bytes, void *stream, bool defer_join) {
+                         float *dbeta, void *workspace, size_t workspace_bytes, void *stream, bool defer_join,
+                         const PostOp &post = PostOp()) {
     HalfCall half(desc);              // CONVBN_F16: checked here, then run as the 16-bit path with the half flag set
     if (half.status != CONVBN_OK) return half.status;
     desc = half.use;
@@ -896,7 +940,7 @@ static int tune_bwd_impl(const convbn_desc *desc, const void *dz, const void *x,
     if ((b == nullptr) != (db == nullptr)) return CONVBN_EINVAL;
     if (!aligned(dz, 16) || !aligned(x, 16) || !aligned(w, 16) || !aligned(saved, 16) || !aligned(dx, 16) ||
         !aligned(dw, 16) || !aligned(b, 4) || !aligned(run_mean, 4) || !aligned(db, 4) || !aligned(dgamma, 4) ||
-        !aligned(dbeta, 4))
+        !aligned(dbeta, 4) || !aligned(post.add, 16))
         return CONVBN_EALIGN;
     const Plan pl = make_plan(desc, pb, CONVBN_PHASE_TUNE_BWD);
     CK(check_ws(pl, workspace, workspace_bytes));
@@ -905,14 +949,14 @@ static int tune_bwd_impl(const convbn_desc *desc, const void *dz, const void *x,
         LAUNCH("direct_bwd", launch_f32_bwd(pb, (const float *)dz, (const float *)x, (const float *)w, (const float *)saved,
                                             (float *)dx, (const float *)saved, b, run_mean, dw, db, dgamma, dbeta, st));
         t_last_kernel[CONVBN_PHASE_TUNE_BWD] = "two-calls";
-        return CONVBN_OK;
+        return run_post(desc, post, dx, pb.pin * pb.c_in, st);
     }
     if (!fused_bwd_path(desc, pb)) {
         void *ws_w = workspace ? at(workspace, pl.w_scaled) : nullptr;
         const size_t bytes_d = pl.w_scaled, bytes_w = pl.total - pl.w_scaled;
         t_last_kernel[CONVBN_PHASE_TUNE_BWD] = "two-calls";
         if (g_prof.on) {                 // per-kernel timing wants one stream, deferred or not
-            CK(convbn_tune_bwd_data(desc, dz, w, saved, dx, workspace, bytes_d, stream));
+            CK(tune_bwd_data_impl(desc, dz, w, saved, dx, post, workspace, bytes_d, stream));
             return convbn_tune_bwd_weight(desc, dz, x, w, b, run_mean, saved, dw, db, dgamma, dbeta, ws_w, bytes_w, stream);
         }
         SideLane *lane = nullptr;
@@ -924,7 +968,7 @@ static int tune_bwd_impl(const convbn_desc *desc, const void *dz, const void *x,
                                               lane->stream);
         // whatever happened on the lane, the caller's stream joins it again (a capture must not be left forked)
         const bool joined = cudaEventRecord(lane->join, lane->stream) == cudaSuccess;
-        const int sd = convbn_tune_bwd_data(desc, dz, w, saved, dx, workspace, bytes_d, stream);
+        const int sd = tune_bwd_data_impl(desc, dz, w, saved, dx, post, workspace, bytes_d, stream);
         if (!joined) return CONVBN_ECUDA;
         if (defer_join) lane->pending = true;
         else if (cudaStreamWaitEvent(st, lane->join, 0) != cudaSuccess) return CONVBN_ECUDA;
@@ -935,7 +979,7 @@ static int tune_bwd_impl(const convbn_desc *desc, const void *dz, const void *x,
     float *dotpart = (float *)at(workspace, pl.dotpart);
     unsigned int *counters = (unsigned int *)at(workspace, pl.counters);
     const float *vec3 = (const float *)saved;
-    LAUNCH("umma_bwd", launch_fused_bwd1x1(pb, dz, x, w, vec3, dx, partials, bsum, counters, st));
+    LAUNCH("umma_bwd", launch_fused_bwd1x1(pb, dz, x, w, vec3, dx, partials, bsum, counters, st, &post));
     t_last_kernel[CONVBN_PHASE_TUNE_BWD] = "umma-fused-bwd";
     if (defer_join && !g_prof.on) {
         // dX is complete on the caller's stream; the parameter gradients are finished on the side lane
@@ -967,6 +1011,17 @@ int convbn_tune_bwd_begin(const convbn_desc *desc, const void *dz, const void *x
                           float *dbeta, void *workspace, size_t workspace_bytes, void *stream) {
     return tune_bwd_impl(desc, dz, x, w, b, run_mean, saved, dx, dw, db, dgamma, dbeta, workspace, workspace_bytes, stream,
                          true);
+}
+
+int convbn_tune_bwd_glue(const convbn_desc *desc, const void *dz, const void *x, const void *w, const float *b,
+                         const float *run_mean, const void *saved, void *dx, float *dw, float *db, float *dgamma,
+                         float *dbeta, const void *add, int relu_mask, int begin, void *workspace, size_t workspace_bytes,
+                         void *stream) {
+    PostOp post;
+    post.add = add;
+    post.mask = relu_mask ? x : nullptr;
+    return tune_bwd_impl(desc, dz, x, w, b, run_mean, saved, dx, dw, db, dgamma, dbeta, workspace, workspace_bytes, stream,
+                         begin != 0, post);
 }
 
 int convbn_tune_bwd_join(void *stream) {

@@ -31,6 +31,13 @@ int direct_wgrad_splits(const Problem &pb);
 cudaError_t launch_direct_wgrad(const Problem &pb, int dtype, int layout, const void *dz,
                                 const void *x, float *partials, int splits, cudaStream_t st);
 
+// Glue fused into a convolution's epilogue (16-bit storage, all tensors of the output's shape and layout): see post_chunk
+// in common.cuh.  NULL / 0: not wanted.
+struct PostOp {
+    const void *add = nullptr, *mask = nullptr;
+    int relu = 0;
+    bool any() const { return add || mask || relu; }
+};
 // BatchNorm parameters for in-kernel reparameterisation: the kernel forms s and b' per output channel,
 // computes out = s * (wmat (*) act) + b' and (CTA 0) writes [s | b' | r] to vec3 (3 cn floats, may be NULL).
 struct BnFold {
@@ -83,12 +90,14 @@ bool umma_conv_eligible(const UmmaConvShape &s);
 // fold != NULL replaces `bias` (dense output mode only).  With out2 (Eval mode) out = wmat (*) act + fold->b and
 // out2 = gamma (out - mean) / sqrt(var + eps) + beta from the rounded out; nothing is written to fold->vec3.
 cudaError_t launch_umma_conv(const UmmaConvShape &s, const void *act, const void *wmat, const float *bias,
-                             void *out, cudaStream_t st, const BnFold *fold = nullptr, void *out2 = nullptr);
+                             void *out, cudaStream_t st, const BnFold *fold = nullptr, void *out2 = nullptr,
+                             const PostOp *post = nullptr);
 // Stride-1 multi-tap convolutions with the input patch staged once per tile (see umma_strip.cu): same
 // contract as launch_umma_conv (dense output mode, groups = 1).  Eligibility depends on the image size.
 bool umma_strip_eligible(const UmmaConvShape &s);
 cudaError_t launch_umma_strip_conv(const UmmaConvShape &s, const void *act, const void *wmat, const float *bias,
-                                   void *out, cudaStream_t st, const BnFold *fold = nullptr);
+                                   void *out, cudaStream_t st, const BnFold *fold = nullptr,
+                                   const PostOp *post = nullptr);
 // Backward data of a stride-2 layer with C_in <= 4 as ONE stride-1 convolution over dZ (Sec. 3.2.1: the
 // transposed convolution, regrouped by the parity of the input position): the four parity classes of an
 // input position become 4 C_in output columns of a GEMM whose taps are the dZ offsets any class needs;
@@ -172,7 +181,7 @@ cudaError_t launch_wgrad_epilogue_stem(const Problem &pb, const UmmaWgradPlan &p
 // staged once in shared memory, the im2col windows formed by the MMA operand addressing.  No packed copy.
 bool stem_window_eligible(const Problem &pb);
 cudaError_t launch_stem_window_fwd(const Problem &pb, const void *x, const void *w, const float *bias, void *z,
-                                   cudaStream_t st, const BnFold *fold = nullptr);
+                                   cudaStream_t st, const BnFold *fold = nullptr, int relu = 0);
 // Weight gradient of the same layers (C_in <= 3, C_out = 64) straight from X and dZ: one fp32 partial
 // [kdim][C_out] and one row of sums of dZ per CTA (stem_window_wgrad_ctas of them), in the layout the fused
 // epilogue of the dense weight-gradient path reads; `counters` are zeroed for it.
@@ -279,7 +288,8 @@ cudaError_t launch_bn_eval_finish(const Problem &pb, const float *part_g, const 
 bool fused_bwd1x1_eligible(const Problem &pb);
 int fused_bwd1x1_ctas(const Problem &pb);
 cudaError_t launch_fused_bwd1x1(const Problem &pb, const void *dz, const void *x, const void *w, const float *vec3,
-                                void *dx, float *partials, float *bsum, unsigned int *counters, cudaStream_t st);
+                                void *dx, float *partials, float *bsum, unsigned int *counters, cudaStream_t st,
+                                const PostOp *post = nullptr);
 
 // ---- elementwise glue between blocks (glue_kernels.cu): mode 0 relu(a), 1 relu(a + b), 2 a masked by b > 0, 3 a + b
 cudaError_t launch_glue(int mode, int dtype, const void *a, const void *b, void *out, long long count, cudaStream_t st);

@@ -39,6 +39,7 @@ struct WinGemm {
     long long total_rows;  // n * h_out
     int f16;               // 16-bit storage type: 0 bf16, 1 IEEE half
     BnFold fold;
+    int relu;              // 1: max(Z, 0) is stored
 };
 
 struct WinCtl {
@@ -345,6 +346,7 @@ __global__ void __launch_bounds__(kWinThreads) stem_window_fwd_kernel(const __gr
                                 pk.y = pack2_h16(fmaf(__uint_as_float(v[j + 2]), s0.z, b0.z), fmaf(__uint_as_float(v[j + 3]), s0.w, b0.w), g.f16);
                                 pk.z = pack2_h16(fmaf(__uint_as_float(v[j + 4]), s1.x, b1.x), fmaf(__uint_as_float(v[j + 5]), s1.y, b1.y), g.f16);
                                 pk.w = pack2_h16(fmaf(__uint_as_float(v[j + 6]), s1.z, b1.z), fmaf(__uint_as_float(v[j + 7]), s1.w, b1.w), g.f16);
+                                if (g.relu) { pk.x = relu2_h16(pk.x); pk.y = relu2_h16(pk.y); pk.z = relu2_h16(pk.z); pk.w = relu2_h16(pk.w); }
                                 *(uint4 *)(row + (((4 * half + (j >> 3)) ^ (lane & 7)) << 4)) = pk;
                             }
                         }
@@ -778,7 +780,7 @@ cudaError_t launch_stem_window_wgrad(const Problem &pb, const void *dz, const vo
 }
 
 cudaError_t launch_stem_window_fwd(const Problem &pb, const void *x, const void *w, const float *bias, void *z,
-                                   cudaStream_t st, const BnFold *fold) {
+                                   cudaStream_t st, const BnFold *fold, int relu) {
     const WinPlan pl = plan_window(pb);
     if (!pl.ok) return cudaErrorInvalidValue;
     WinGemm g;
@@ -788,6 +790,7 @@ cudaError_t launch_stem_window_fwd(const Problem &pb, const void *x, const void 
     g.colblocks = (pb.w_out + 127) / 128; g.nstrips = pl.nstrips; g.strip_bytes = pl.strip_bytes;
     g.kblocks = pl.kblocks; g.total_rows = (long long)pb.n * pb.h_out;
     g.f16 = call_f16();
+    g.relu = relu;
     g.fold = fold ? *fold : BnFold{nullptr, nullptr, nullptr, nullptr, nullptr, 0.f, nullptr};
     CUtensorMap tout;
     const unsigned long long dims[3] = {(unsigned long long)pb.c_out, (unsigned long long)pb.w_out,

@@ -27,6 +27,9 @@ struct FusedBwd {
     int m_tiles;            // ceil(p / 128)
     const float *vec3;      // saved [s | b' | r]
     int f16;                // 16-bit storage type: 0 bf16, 1 IEEE half
+    __nv_bfloat16 *dx;      // POST: plain stores of dX with post_add and post_mask (tensors of its shape; may be NULL)
+    const __nv_bfloat16 *post_add, *post_mask;
+    int post_relu;
 };
 
 struct FbCtl {
@@ -53,7 +56,7 @@ struct FbShape {
     static_assert((CI == 64) != (CO == 64) && kWide % 128 == 0 && kWide <= 256, "supported channel counts");
 };
 
-template <int CI, int CO>
+template <int CI, int CO, bool POST>
 __global__ void __launch_bounds__(kFbThreads) fused_bwd1x1_kernel(const __grid_constant__ CUtensorMap tm_dz,
                                                                  const __grid_constant__ CUtensorMap tm_x,
                                                                  const __grid_constant__ CUtensorMap tm_dx,
@@ -244,6 +247,31 @@ __global__ void __launch_bounds__(kFbThreads) fused_bwd1x1_kernel(const __grid_c
                     }
                 };
                 if (g.f16) pack_rows(std::true_type{}); else pack_rows(std::false_type{});
+                if constexpr (POST) {
+                    // eight lanes write the 128 bytes of a pixel; the other tensors' values of all eight are requested first
+                    __syncwarp();
+                    const int ch = lane & 7;
+                    uint4 av[8], mv[8];
+                    const long long row0 = (long long)t * 128 + quarter * 32 + (lane >> 3);
+                    const size_t off0 = (size_t)row0 * CI + c0 + ch * 8;
+#pragma unroll
+                    for (int it = 0; it < 8; ++it) {
+                        const bool on = row0 + it * 4 < g.p;
+                        av[it] = mv[it] = make_uint4(0u, 0u, 0u, 0u);
+                        if (on && g.post_add) av[it] = *(const uint4 *)(g.post_add + off0 + (size_t)it * 4 * CI);
+                        if (on && g.post_mask) mv[it] = *(const uint4 *)(g.post_mask + off0 + (size_t)it * 4 * CI);
+                    }
+#pragma unroll
+                    for (int it = 0; it < 8; ++it) {
+                        const int rr = it * 4 + (lane >> 3);
+                        const uint4 q = *(const uint4 *)(buf_s + rr * 128 + (((ch ^ (rr & 7)) & 7) << 4));
+                        const uint4 o = g.f16 ? post_chunk<true>(q, g.post_add, av[it], g.post_relu, g.post_mask, mv[it])
+                                              : post_chunk<false>(q, g.post_add, av[it], g.post_relu, g.post_mask, mv[it]);
+                        if (row0 + it * 4 < g.p) *(uint4 *)(g.dx + off0 + (size_t)it * 4 * CI) = o;
+                    }
+                    __syncwarp();
+                    continue;
+                }
                 fence_proxy_async_smem();
                 __syncwarp();
                 if (lane == 0) {
@@ -313,16 +341,23 @@ __global__ void __launch_bounds__(kFbThreads) fused_bwd1x1_kernel(const __grid_c
 
 // ---- host side --------------------------------------------------------------------------------------
 namespace {
-template <int CI, int CO>
-cudaError_t launch_fb(const CUtensorMap &tdz, const CUtensorMap &tx, const CUtensorMap &tdx, const FusedBwd &g, unsigned grid,
+template <int CI, int CO, bool POST>
+cudaError_t launch_fb_as(const CUtensorMap &tdz, const CUtensorMap &tx, const CUtensorMap &tdx, const FusedBwd &g, unsigned grid,
                       const void *w, float *partials, float *bsum, unsigned int *counters, int *err, cudaStream_t st) {
     using S = FbShape<CI, CO>;
     const size_t smem = 1024 + (size_t)kFbStages * S::kStageBytes + (size_t)CI * CO * 2 + 1024 + 8 * 4096 + sizeof(FbCtl) + 64;
     static PerDevice attr, carve;
-    if (cudaError_t e = max_dynamic_smem_once(fused_bwd1x1_kernel<CI, CO>, 227 * 1024, &attr); e != cudaSuccess) return e;
-    prefer_max_shared_once(fused_bwd1x1_kernel<CI, CO>, &carve);
-    return launch_pdl(fused_bwd1x1_kernel<CI, CO>, dim3(grid), dim3(kFbThreads), smem, st, tdz, tx, tdx, g,
+    if (cudaError_t e = max_dynamic_smem_once(fused_bwd1x1_kernel<CI, CO, POST>, 227 * 1024, &attr); e != cudaSuccess) return e;
+    prefer_max_shared_once(fused_bwd1x1_kernel<CI, CO, POST>, &carve);
+    return launch_pdl(fused_bwd1x1_kernel<CI, CO, POST>, dim3(grid), dim3(kFbThreads), smem, st, tdz, tx, tdx, g,
                       (const __nv_bfloat16 *)w, partials, bsum, counters, CO / 32, err);
+}
+template <int CI, int CO>
+cudaError_t launch_fb(const CUtensorMap &tdz, const CUtensorMap &tx, const CUtensorMap &tdx, const FusedBwd &g, unsigned grid,
+                      const void *w, float *partials, float *bsum, unsigned int *counters, int *err, cudaStream_t st) {
+    if (g.post_add || g.post_mask || g.post_relu)
+        return launch_fb_as<CI, CO, true>(tdz, tx, tdx, g, grid, w, partials, bsum, counters, err, st);
+    return launch_fb_as<CI, CO, false>(tdz, tx, tdx, g, grid, w, partials, bsum, counters, err, st);
 }
 }  // namespace
 
@@ -338,10 +373,14 @@ int fused_bwd1x1_ctas(const Problem &pb) {
 }
 
 cudaError_t launch_fused_bwd1x1(const Problem &pb, const void *dz, const void *x, const void *w, const float *vec3, void *dx,
-                                float *partials, float *bsum, unsigned int *counters, cudaStream_t st) {
+                                float *partials, float *bsum, unsigned int *counters, cudaStream_t st, const PostOp *post) {
     if (!fused_bwd1x1_eligible(pb)) return cudaErrorInvalidValue;
     FusedBwd g;
     g.p = pb.p; g.m_tiles = (int)((pb.p + 127) / 128); g.vec3 = vec3; g.f16 = call_f16();
+    g.dx = (__nv_bfloat16 *)dx;
+    g.post_add = post ? (const __nv_bfloat16 *)post->add : nullptr;
+    g.post_mask = post ? (const __nv_bfloat16 *)post->mask : nullptr;
+    g.post_relu = post ? post->relu : 0;
     CUtensorMap tdz, tx, tdx;
     if (!make_tmap_matrix_bf16(&tdz, dz, pb.p, pb.c_out, 128, 64)) return cudaErrorInvalidValue;
     if (!make_tmap_matrix_bf16(&tx, x, pb.p, pb.c_in, 128, 64)) return cudaErrorInvalidValue;

@@ -53,6 +53,8 @@ struct ConvGemm {
     // c of output pixel (i kh + r, j kw + q), tap = r kw + q, in out_strided; out_sh / out_sw are the steps of i and j,
     // tap_sh / tap_sw those of r and q.  The weight tensor is then read as it is, [ca][cn], as an MN-major operand.
     int tap_c, tap_kw, tap_sh, tap_sw;
+    const __nv_bfloat16 *post_add, *post_mask;      // at the output's offsets
+    int post_relu;
 };
 
 struct ConvSmemCtl {
@@ -76,7 +78,8 @@ struct ConvSmemCtl {
 // of the kernels beside it fits next to a CTA: 3x3 512 -> 512 at 7 x 7, N = 64, forward + backward 85 -> 93 us.  The
 // bound of 512 threads holds the plain kernel to 128 registers for the same reason.)
 // MODE kTap: the transposed convolution of ConvGemm::tap_c.
-enum ConvMode { kPlain, kDual, kTap };
+// MODE kPost: post_add, post_relu, post_mask follow (strided stores, dense ones included).
+enum ConvMode { kPlain, kDual, kTap, kPost };
 template <int BN, ConvMode MODE>
 __global__ void __launch_bounds__(MODE == kDual ? kConvThreads : 512) umma_conv_kernel(const __grid_constant__ CUtensorMap tm_act,
                                                                 const __grid_constant__ CUtensorMap tm_w,
@@ -85,7 +88,7 @@ __global__ void __launch_bounds__(MODE == kDual ? kConvThreads : 512) umma_conv_
                                                                 const ConvGemm g, const float *__restrict__ bias,
                                                                 int *err) {
     extern __shared__ uint8_t smem_raw[];
-    constexpr bool DUAL = MODE == kDual, TAP = MODE == kTap;
+    constexpr bool DUAL = MODE == kDual, TAP = MODE == kTap, POST = MODE == kPost;
     constexpr uint32_t kABytes = kBM * kBK * 2, kBBytes = BN * kBK * 2;
     const int cchunks = g.blockdiag ? 1 : g.ca / kBK;
     const int num_kb = g.taps_h * g.taps_w * cchunks;
@@ -375,6 +378,36 @@ __global__ void __launch_bounds__(MODE == kDual ? kConvThreads : 512) umma_conv_
                         }
                     };
                     if (g.f16) pack_rows(std::true_type{}); else pack_rows(std::false_type{});
+                    if constexpr (POST) {
+                        // as below, with the other tensors' values of four pixels requested before the first is used
+                        __syncwarp();
+                        const int ch = lane & 7;
+#pragma unroll 1
+                        for (int i0 = 0; i0 < 8; i0 += 4) {
+                            uint4 av[4], mv[4];
+                            ptrdiff_t at8[4];
+#pragma unroll
+                            for (int k = 0; k < 4; ++k) {
+                                const __nv_bfloat16 *dst = (const __nv_bfloat16 *)__shfl_sync(
+                                    0xffffffffu, (unsigned long long)srow, (i0 + k) * 4 + (lane >> 3));
+                                const bool on = dst && c0 + ch * 8 < ncols;
+                                at8[k] = on ? dst - g.out_strided + c0 + ch * 8 : -1;
+                                av[k] = mv[k] = make_uint4(0u, 0u, 0u, 0u);
+                                if (on && g.post_add) av[k] = *(const uint4 *)(g.post_add + at8[k]);
+                                if (on && g.post_mask) mv[k] = *(const uint4 *)(g.post_mask + at8[k]);
+                            }
+#pragma unroll
+                            for (int k = 0; k < 4; ++k) {
+                                const int rr = (i0 + k) * 4 + (lane >> 3);
+                                const uint4 q = *(const uint4 *)(buf + rr * 128 + (((ch ^ (rr & 7)) & 7) << 4));
+                                const uint4 o = g.f16 ? post_chunk<true>(q, g.post_add, av[k], g.post_relu, g.post_mask, mv[k])
+                                                      : post_chunk<false>(q, g.post_add, av[k], g.post_relu, g.post_mask, mv[k]);
+                                if (at8[k] >= 0) *(uint4 *)(g.out_strided + at8[k]) = o;
+                            }
+                        }
+                        __syncwarp();
+                        continue;
+                    }
                     if (TAP || g.out_strided) {
                         // eight lanes write the 128 bytes of a pixel, four pixels per instruction
                         __syncwarp();
@@ -618,7 +651,7 @@ static int pick_bn(long long tiles_m, int cn) {
 }
 
 cudaError_t launch_umma_conv(const UmmaConvShape &s, const void *act, const void *wmat, const float *bias,
-                             void *out, cudaStream_t st, const BnFold *fold, void *out2) {
+                             void *out, cudaStream_t st, const BnFold *fold, void *out2, const PostOp *post) {
     ConvGemm g;
     g.ho = s.ho; g.wo = s.wo; g.cn = s.cn; g.ca = s.ca; g.taps_h = s.taps_h; g.taps_w = s.taps_w;
     g.lower_h = s.lower_h; g.lower_w = s.lower_w; g.stride_h = s.stride_h; g.stride_w = s.stride_w;
@@ -629,6 +662,14 @@ cudaError_t launch_umma_conv(const UmmaConvShape &s, const void *act, const void
     g.fold = fold ? *fold : BnFold{nullptr, nullptr, nullptr, nullptr, nullptr, 0.f, nullptr};
     g.out_strided = s.out_sw ? (__nv_bfloat16 *)out : nullptr;
     g.out_sn = s.out_sn; g.out_sh = s.out_sh; g.out_sw = s.out_sw;
+    const bool with_post = post && post->any();
+    if (with_post && !s.out_sw) {
+        g.out_strided = (__nv_bfloat16 *)out;
+        g.out_sn = (long long)s.ho * s.wo * s.cn; g.out_sh = s.wo * s.cn; g.out_sw = s.cn;
+    }
+    g.post_add = with_post ? (const __nv_bfloat16 *)post->add : nullptr;
+    g.post_mask = with_post ? (const __nv_bfloat16 *)post->mask : nullptr;
+    g.post_relu = with_post ? post->relu : 0;
     g.tap_c = s.tap_c; g.tap_kw = s.tap_kw; g.tap_sh = s.tap_sh; g.tap_sw = s.tap_sw;
     // The bounding box of base pixels has ho x wo positions: upper = lower + (out-1) stride - (in-1).
     const int upper_h = s.lower_h + (s.ho - 1) * s.stride_h - (s.ha - 1);
@@ -650,6 +691,7 @@ cudaError_t launch_umma_conv(const UmmaConvShape &s, const void *act, const void
     if (e != cudaSuccess) return e;
     CUtensorMap tout2 = tout;
     if (out2 && !make_tmap_matrix_bf16(&tout2, out2, g.p, s.cn, 32, 64)) return cudaErrorInvalidValue;
+    if (with_post) return launch_mode<kPost>(bn, ta, tw, tout, tout2, g, bias, err, st);
     if (out2) return launch_mode<kDual>(bn, ta, tw, tout, tout2, g, bias, err, st);
     if (g.tap_c) return launch_mode<kTap>(bn, ta, tw, tout, tout2, g, bias, err, st);
     return launch_mode<kPlain>(bn, ta, tw, tout, tout2, g, bias, err, st);
@@ -661,7 +703,7 @@ cudaError_t launch_stem_fwd(const Problem &pb, const void *x_packed, const void 
                             cudaStream_t st, const BnFold *fold) {
     const int krows = stem_krows(pb);
     ConvGemm g;
-    g.tap_c = 0;
+    g.tap_c = 0; g.post_add = g.post_mask = nullptr; g.post_relu = 0;
     g.ho = pb.h_out; g.wo = pb.w_out; g.cn = pb.c_out; g.ca = 64; g.taps_h = krows; g.taps_w = 1;
     g.lower_h = g.lower_w = 0; g.stride_h = g.stride_w = g.dil_h = g.dil_w = 1;
     g.stem = 1; g.stem_tw = 16; g.stem_th = 8;

@@ -56,6 +56,8 @@ struct StripGemm {
     uint32_t sub_mask[4];             // taps with weights, per class
     __nv_bfloat16 *out;
     BnFold fold;
+    const __nv_bfloat16 *post_add, *post_mask;      // POST: at the output's offsets
+    int post_relu;
 };
 
 struct StripCtl {
@@ -79,7 +81,8 @@ __device__ __forceinline__ void quad_swap(uint4 &lo, uint4 &hi, int mask, bool u
     if (upper) lo = recv; else hi = recv;
 }
 
-template <int BN>
+// POST: post_add, post_relu, post_mask follow in the epilogue.
+template <int BN, bool POST>
 __global__ void __launch_bounds__(kSThreads) umma_strip_conv_kernel(const __grid_constant__ CUtensorMap tm_act,
                                                                    const __grid_constant__ CUtensorMap tm_w,
                                                                    const StripGemm g, const float *__restrict__ bias,
@@ -410,9 +413,23 @@ __global__ void __launch_bounds__(kSThreads) umma_strip_conv_kernel(const __grid
                     quad_swap(pk[2], pk[3], 1, (lane & 1) != 0);
                     quad_swap(pk[0], pk[2], 2, (lane & 2) != 0);
                     quad_swap(pk[1], pk[3], 2, (lane & 2) != 0);
+                    uint4 av[4], mv[4];
+                    if constexpr (POST) {
 #pragma unroll
-                    for (int k = 0; k < 4; ++k)
+                        for (int k = 0; k < 4; ++k) {
+                            const ptrdiff_t off = rowp[k] - g.out + c0 + qc * 8;
+                            av[k] = mv[k] = make_uint4(0u, 0u, 0u, 0u);
+                            if (rowok[k] && g.post_add) av[k] = *(const uint4 *)(g.post_add + off);
+                            if (rowok[k] && g.post_mask) mv[k] = *(const uint4 *)(g.post_mask + off);
+                        }
+                    }
+#pragma unroll
+                    for (int k = 0; k < 4; ++k) {
+                        if constexpr (POST)
+                            pk[k] = g.f16 ? post_chunk<true>(pk[k], g.post_add, av[k], g.post_relu, g.post_mask, mv[k])
+                                          : post_chunk<false>(pk[k], g.post_add, av[k], g.post_relu, g.post_mask, mv[k]);
                         if (rowok[k]) *(uint4 *)(rowp[k] + c0 + qc * 8) = pk[k];
+                    }
                 }
                 }
             }
@@ -558,16 +575,16 @@ bool make_tmap_nhwc_box(CUtensorMap *tm, const void *base, int n, int h, int w, 
 }
 
 
-template <int BN>
+template <int BN, bool POST = false>
 cudaError_t launch_strip(const CUtensorMap &ta, const CUtensorMap &tw, const StripGemm &g, size_t smem,
                          const float *bias, int *err, cudaStream_t st) {
     static PerDevice attr;
-    if (cudaError_t e = max_dynamic_smem_once(umma_strip_conv_kernel<BN>, 226 * 1024, &attr); e != cudaSuccess) return e;
+    if (cudaError_t e = max_dynamic_smem_once(umma_strip_conv_kernel<BN, POST>, 226 * 1024, &attr); e != cudaSuccess) return e;
     static PerDevice carve;
-    prefer_max_shared_once(umma_strip_conv_kernel<BN>, &carve);
+    prefer_max_shared_once(umma_strip_conv_kernel<BN, POST>, &carve);
     const long long total = (long long)g.n * g.tiles_h * g.tiles_w * (g.cn / BN);
     const unsigned grid = (unsigned)(total < strip_sm_count() ? total : strip_sm_count());
-    return launch_pdl(umma_strip_conv_kernel<BN>, dim3(grid), dim3(kSThreads), smem, st, ta, tw, g, bias, err);
+    return launch_pdl(umma_strip_conv_kernel<BN, POST>, dim3(grid), dim3(kSThreads), smem, st, ta, tw, g, bias, err);
 }
 
 }  // namespace
@@ -577,7 +594,7 @@ bool umma_strip_eligible(const UmmaConvShape &s) {
 }
 
 cudaError_t launch_umma_strip_conv(const UmmaConvShape &s, const void *act, const void *wmat, const float *bias,
-                                   void *out, cudaStream_t st, const BnFold *fold) {
+                                   void *out, cudaStream_t st, const BnFold *fold, const PostOp *post) {
     const StripPlan pl = plan_strip(s);
     if (!pl.ok) return cudaErrorInvalidValue;
     StripGemm g;
@@ -606,6 +623,15 @@ cudaError_t launch_umma_strip_conv(const UmmaConvShape &s, const void *act, cons
     int *err = nullptr;
     cudaError_t e = error_word_address(&err);
     if (e != cudaSuccess) return e;
+    const bool with_post = post && post->any();
+    g.post_add = with_post ? (const __nv_bfloat16 *)post->add : nullptr;
+    g.post_mask = with_post ? (const __nv_bfloat16 *)post->mask : nullptr;
+    g.post_relu = with_post ? post->relu : 0;
+    if (with_post) {
+        if (pl.bn == 16) return cudaErrorInvalidValue;
+        if (pl.bn == 64) return launch_strip<64, true>(ta, tw, g, pl.smem, bias, err, st);
+        return launch_strip<128, true>(ta, tw, g, pl.smem, bias, err, st);
+    }
     if (pl.bn == 16) return launch_strip<16>(ta, tw, g, pl.smem, bias, err, st);
     if (pl.bn == 64) return launch_strip<64>(ta, tw, g, pl.smem, bias, err, st);
     return launch_strip<128>(ta, tw, g, pl.smem, bias, err, st);

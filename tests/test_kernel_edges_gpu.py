@@ -44,3 +44,53 @@ TCONV = [  # (dtype, n, c_in, h, w, c_out, k, stride, pad, dil, groups, bias): k
 def test_tconv_block(case):
     import test_tconv
     test_tconv.test_library_matches_the_oracle(case)
+
+
+GLUE = [  # every kernel whose epilogue does the glue, and one that leaves it to passes of its own
+    L("glue_1x1", 3, 128, 9, 13, 320, 1, 1, dtype="f16"),                     # GEMM, a last tile of 64 columns
+    L("glue_strided", 2, 64, 11, 9, 128, 3, 3, stride=2, pad=1),              # a GEMM per parity class
+    L("glue_empty", 2, 64, 10, 9, 64, 1, 1, stride=2),                        # positions without a class
+    L("glue_strip", 2, 64, 21, 30, 192, 3, 3, pad=1),
+    L("glue_subpixel", 1, 128, 33, 34, 128, 3, 3, stride=2, pad=1, dtype="f16"),
+    L("glue_fused", 3, 256, 17, 15, 64, 1, 1), L("glue_fused_wide", 3, 64, 17, 15, 128, 1, 1, dtype="f16"),
+    L("glue_stem", 2, 3, 37, 40, 64, 7, 7, stride=2, pad=3),
+    L("glue_dw", 2, 32, 9, 21, 32, 3, 3, pad=1, groups=32),
+    L("glue_f32", 2, 6, 9, 7, 10, 3, 3, pad=1, dtype="f32", layout="nchw"),
+]
+
+
+@pytest.mark.parametrize("spec", GLUE, ids=lambda s: s.name)
+def test_glue_in_the_epilogue_equals_the_passes(spec):
+    """convbn_tune_fwd_glue / _bwd_glue against the plain calls followed by the elementwise ones: the same bits."""
+    import torch
+    from paper_2305_11624_b200 import convbn as C
+    from paper_2305_11624_b200.harness import Block
+    blk = Block(spec)
+    blk.randomize(3)
+    blk.x.relu_()                                       # the mask's tensor is a ReLU output
+    add_z, add_x = torch.randn_like(blk.z.normal_()), torch.randn_like(blk.x)
+    blk.tune_fwd(); blk.tune_bwd()
+    z, dx = blk.z.clone(), blk.dx.clone()
+    grads = [t.clone() for t in (blk.dw, blk.dgamma, blk.dbeta)]
+    C.convbn_check()
+    for add, relu in ((None, True), (add_z, True), (add_z, False)):
+        want = torch.empty_like(z)
+        (C.convbn_add_relu if relu else C.convbn_add)(z, add, want) if add is not None else C.convbn_relu(z, want)
+        blk.z.fill_(float("nan"))
+        C.convbn_tune_fwd_glue(blk.desc, blk.x, blk.w, blk.b, blk.gamma, blk.beta, blk.mu_hat, blk.var_hat, blk.z, blk.saved,
+                               add, relu, blk.workspace)
+        assert torch.equal(blk.z, want), (add is not None, relu)
+    for add, mask, begin in ((None, True, False), (add_x, True, True), (add_x, False, False)):
+        want = dx.clone()
+        if add is not None:
+            C.convbn_add(want, add, want)
+        if mask:
+            C.convbn_relu_bwd(want, blk.x, want)
+        for t in (blk.dx, blk.dw, blk.dgamma, blk.dbeta):
+            t.fill_(float("nan"))
+        C.convbn_tune_bwd_glue(blk.desc, blk.dz, blk.x, blk.w, blk.b, blk.mu_hat, blk.saved, blk.dx, blk.dw, blk.db,
+                               blk.dgamma, blk.dbeta, add, mask, begin, blk.workspace)
+        C.convbn_tune_bwd_join()
+        assert torch.equal(blk.dx, want), (add is not None, mask)
+        assert all(torch.equal(a, b) for a, b in zip((blk.dw, blk.dgamma, blk.dbeta), grads))
+    C.convbn_check()
