@@ -84,21 +84,24 @@ __device__ __forceinline__ void unpack2_t(uint32_t bits, float &lo, float &hi) {
 // max(v, 0) of two finite 16-bit values: a set sign bit clears its half
 __device__ __forceinline__ uint32_t relu2_h16(uint32_t v) { return v & ~(((v >> 15) & 0x00010001u) * 0xFFFFu); }
 // What a residual network does next with a block's result, on eight 16-bit values: v + a (rounded again, as an add of two
-// stored tensors is), max(v, 0), v where m > 0 and 0 elsewhere.
+// stored tensors is), max(v, 0), v where m > 0 and 0 elsewhere.  Two values per instruction: the 16-bit sum is the rounded
+// exact one, which an fp32 sum rounded to 16 bits is too (24 >= 2 * 11 + 2 significant bits).
+template <bool F16>
+__device__ __forceinline__ uint32_t post_pair(uint32_t v, bool add, uint32_t a, bool relu, bool mask, uint32_t m) {
+    using P = typename std::conditional<F16, __half2, __nv_bfloat162>::type;
+    P x = *reinterpret_cast<const P *>(&v);
+    const uint32_t z32 = 0u;
+    const P z = *reinterpret_cast<const P *>(&z32);
+    if (add) x = __hadd2_rn(x, *reinterpret_cast<const P *>(&a));
+    if (relu) x = __hmax2(x, z);
+    uint32_t r = *reinterpret_cast<const uint32_t *>(&x);
+    if (mask) r &= __hgt2_mask(*reinterpret_cast<const P *>(&m), z);
+    return r;
+}
 template <bool F16>
 __device__ __forceinline__ uint4 post_chunk(uint4 v, bool add, const uint4 &a, bool relu, bool mask, const uint4 &m) {
-    uint32_t vw[4] = {v.x, v.y, v.z, v.w};
-    const uint32_t aw[4] = {a.x, a.y, a.z, a.w}, mw[4] = {m.x, m.y, m.z, m.w};
-#pragma unroll
-    for (int i = 0; i < 4; ++i) {
-        float lo, hi, l2, h2;
-        unpack2_t<F16>(vw[i], lo, hi);
-        if (add) { unpack2_t<F16>(aw[i], l2, h2); lo += l2; hi += h2; }
-        if (relu) { lo = fmaxf(lo, 0.f); hi = fmaxf(hi, 0.f); }
-        if (mask) { unpack2_t<F16>(mw[i], l2, h2); lo = l2 > 0.f ? lo : 0.f; hi = h2 > 0.f ? hi : 0.f; }
-        vw[i] = pack2_t<F16>(lo, hi);
-    }
-    return make_uint4(vw[0], vw[1], vw[2], vw[3]);
+    return make_uint4(post_pair<F16>(v.x, add, a.x, relu, mask, m.x), post_pair<F16>(v.y, add, a.y, relu, mask, m.y),
+                      post_pair<F16>(v.z, add, a.z, relu, mask, m.z), post_pair<F16>(v.w, add, a.w, relu, mask, m.w));
 }
 __device__ __forceinline__ uint16_t pack1_h16(float a, int f16) {
     if (f16) { const __half h = __float2half_rn(a); return *reinterpret_cast<const uint16_t *>(&h); }

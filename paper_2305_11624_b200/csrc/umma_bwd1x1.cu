@@ -214,6 +214,19 @@ __global__ void __launch_bounds__(kFbThreads) fused_bwd1x1_kernel(const __grid_c
         for (int t = tile_lo; t < tile_hi && ok; ++t, ++i) {
             const uint32_t buf = S::kDxBufs == 2 ? (i & 1u) : 0u, use = S::kDxBufs == 2 ? (i >> 1) : i;
             if (S::kDxBufs == 2 && (int)buf != egroup) continue;        // the two groups take alternate tiles
+            uint4 av[8], mv[8];                  // POST: eight lanes hold the 128 bytes of a pixel, four pixels an instruction
+            const long long row0 = (long long)t * 128 + quarter * 32 + (lane >> 3);
+            auto fetch_post = [&](int c0) {
+                const size_t off = (size_t)row0 * CI + c0 + (lane & 7) * 8;
+#pragma unroll
+                for (int it = 0; it < 8; ++it) {
+                    const bool on = row0 + it * 4 < g.p;
+                    av[it] = mv[it] = make_uint4(0u, 0u, 0u, 0u);
+                    if (on && g.post_add) av[it] = *(const uint4 *)(g.post_add + off + (size_t)it * 4 * CI);
+                    if (on && g.post_mask) mv[it] = *(const uint4 *)(g.post_mask + off + (size_t)it * 4 * CI);
+                }
+            };
+            if constexpr (POST) fetch_post(S::kDxBufs == 2 ? 0 : egroup * (CI / 2));
             ok = __all_sync(0xffffffffu, mbar_wait_bounded(&ctl->dx_full[buf], use & 1u, abort_flag));
             if (!ok) break;
             tc_fence_after_sync();
@@ -248,19 +261,9 @@ __global__ void __launch_bounds__(kFbThreads) fused_bwd1x1_kernel(const __grid_c
                 };
                 if (g.f16) pack_rows(std::true_type{}); else pack_rows(std::false_type{});
                 if constexpr (POST) {
-                    // eight lanes write the 128 bytes of a pixel; the other tensors' values of all eight are requested first
                     __syncwarp();
                     const int ch = lane & 7;
-                    uint4 av[8], mv[8];
-                    const long long row0 = (long long)t * 128 + quarter * 32 + (lane >> 3);
                     const size_t off0 = (size_t)row0 * CI + c0 + ch * 8;
-#pragma unroll
-                    for (int it = 0; it < 8; ++it) {
-                        const bool on = row0 + it * 4 < g.p;
-                        av[it] = mv[it] = make_uint4(0u, 0u, 0u, 0u);
-                        if (on && g.post_add) av[it] = *(const uint4 *)(g.post_add + off0 + (size_t)it * 4 * CI);
-                        if (on && g.post_mask) mv[it] = *(const uint4 *)(g.post_mask + off0 + (size_t)it * 4 * CI);
-                    }
 #pragma unroll
                     for (int it = 0; it < 8; ++it) {
                         const int rr = it * 4 + (lane >> 3);
@@ -269,6 +272,7 @@ __global__ void __launch_bounds__(kFbThreads) fused_bwd1x1_kernel(const __grid_c
                                               : post_chunk<false>(q, g.post_add, av[it], g.post_relu, g.post_mask, mv[it]);
                         if (row0 + it * 4 < g.p) *(uint4 *)(g.dx + off0 + (size_t)it * 4 * CI) = o;
                     }
+                    if (c0 + 64 < c_hi) fetch_post(c0 + 64);
                     __syncwarp();
                     continue;
                 }

@@ -63,6 +63,7 @@ struct ConvSmemCtl {
     uint64_t tmem_full[2];     // MMA issuer -> epilogue, one per accumulator buffer
     uint64_t tmem_empty[2];    // epilogue -> MMA issuer (4 arrivals: one per epilogue warp)
     uint64_t bfull;            // resident weight slab has landed
+    uint64_t post_full[8];     // kPost: an epilogue warp's boxes of the other tensors have landed
     uint32_t tmem_base;
     int abort_flag;
 };
@@ -78,17 +79,21 @@ struct ConvSmemCtl {
 // of the kernels beside it fits next to a CTA: 3x3 512 -> 512 at 7 x 7, N = 64, forward + backward 85 -> 93 us.  The
 // bound of 512 threads holds the plain kernel to 128 registers for the same reason.)
 // MODE kTap: the transposed convolution of ConvGemm::tap_c.
-// MODE kPost: post_add, post_relu, post_mask follow (strided stores, dense ones included).
-enum ConvMode { kPlain, kDual, kTap, kPost };
+// MODE kPost: post_add, post_relu, post_mask follow.  A warp's [32 rows][64 columns] of the other tensors are brought into
+// buffers of their own by TMA, the next one while this one is used (read from global memory beside the stores, the
+// 64 -> 256 layer at 56 x 56, N = 32 took 90 us with an addend).  MODE kPostStrided: the same for strided outputs, whose
+// rows are no box: read from global memory.
+enum ConvMode { kPlain, kDual, kTap, kPost, kPostStrided };
 template <int BN, ConvMode MODE>
-__global__ void __launch_bounds__(MODE == kDual ? kConvThreads : 512) umma_conv_kernel(const __grid_constant__ CUtensorMap tm_act,
+__global__ void __launch_bounds__(MODE == kPlain || MODE == kTap ? 512 : kConvThreads) umma_conv_kernel(const __grid_constant__ CUtensorMap tm_act,
                                                                 const __grid_constant__ CUtensorMap tm_w,
                                                                 const __grid_constant__ CUtensorMap tm_out,
                                                                 const __grid_constant__ CUtensorMap tm_out2,
+                                                                const __grid_constant__ CUtensorMap tm_mask,
                                                                 const ConvGemm g, const float *__restrict__ bias,
                                                                 int *err) {
     extern __shared__ uint8_t smem_raw[];
-    constexpr bool DUAL = MODE == kDual, TAP = MODE == kTap, POST = MODE == kPost;
+    constexpr bool DUAL = MODE == kDual, TAP = MODE == kTap, POST = MODE == kPost, POST_STRIDED = MODE == kPostStrided;
     constexpr uint32_t kABytes = kBM * kBK * 2, kBBytes = BN * kBK * 2;
     const int cchunks = g.blockdiag ? 1 : g.ca / kBK;
     const int num_kb = g.taps_h * g.taps_w * cchunks;
@@ -97,7 +102,8 @@ __global__ void __launch_bounds__(MODE == kDual ? kConvThreads : 512) umma_conv_
     uint8_t *tiles = (uint8_t *)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
     uint8_t *slab = tiles + (size_t)g.stages * kStageBytes;            // resident weights: num_kb x [BN][64]
     uint8_t *staging = slab + (g.resident ? (size_t)num_kb * kBBytes : 0);   // 8 warps x 2 x [32 rows][128 B]
-    ConvSmemCtl *ctl = (ConvSmemCtl *)(staging + kStagingBytes);
+    const int extra = POST ? (g.post_add != nullptr) + (g.post_mask != nullptr) : 0;     // staging areas of the other tensors
+    ConvSmemCtl *ctl = (ConvSmemCtl *)(staging + (size_t)(1 + extra) * kStagingBytes);
     float *bias_s = (float *)(((uintptr_t)(ctl + 1) + 15) & ~(uintptr_t)15);   // cn floats
     float *scale_s = bias_s + g.cn;                                            // cn floats (fold mode)
     float *shift_s = scale_s + g.cn;                                           // cn floats (DUAL)
@@ -128,6 +134,8 @@ __global__ void __launch_bounds__(MODE == kDual ? kConvThreads : 512) umma_conv_
         for (int s = 0; s < stages; ++s) { mbar_init(&ctl->full[s], 1); mbar_init(&ctl->empty[s], 1); }
         for (int a = 0; a < 2; ++a) { mbar_init(&ctl->tmem_full[a], 1); mbar_init(&ctl->tmem_empty[a], 4); }
         mbar_init(&ctl->bfull, 1);
+        if constexpr (POST)
+            for (int a = 0; a < 8; ++a) mbar_init(&ctl->post_full[a], 1);
         ctl->abort_flag = 0;
         fence_barrier_init();
     }
@@ -298,6 +306,21 @@ __global__ void __launch_bounds__(MODE == kDual ? kConvThreads : 512) umma_conv_
         const uint32_t egroup = (uint32_t)(warp - 2) >> 2; // 0: warps 2-5, 1: warps 6-9
         uint8_t *stage_buf = staging + (size_t)(warp - 2) * kStagingWarpBytes;
         uint32_t mt, nt;
+        // kPost: tm_out2 is the addend's map.  One box of each tensor in flight per warp.
+        uint8_t *add_buf = stage_buf + kStagingBytes, *mask_buf = add_buf + (g.post_add ? kStagingBytes : 0);
+        uint32_t post_ph = 0;
+        bool post_pending = false;
+        auto fetch_post = [&](uint32_t ti, int c0) {          // chunk c0 of tile ti of this CTA, if there is one
+            uint32_t m, n;
+            post_pending = extra > 0 && tile_of(ti, m, n);
+            if (!post_pending || lane != 0) return;
+            uint64_t *bar = &ctl->post_full[warp - 2];
+            mbar_arrive_expect_tx(bar, (uint32_t)extra * kStagingWarpBytes);
+            const int x = (int)n * BN + c0, y = (int)(m * kBM) + quarter * 32;
+            if (g.post_add) tma_load_2d(add_buf, &tm_out2, bar, x, y);
+            if (g.post_mask) tma_load_2d(mask_buf, &tm_mask, bar, x, y);
+        };
+        if constexpr (POST) fetch_post(egroup, 0);
         for (uint32_t i = egroup; tile_of(i, mt, nt); i += 2) {
             const uint32_t acc = egroup;
             CONVBN_TRACE_T0();
@@ -350,8 +373,18 @@ __global__ void __launch_bounds__(MODE == kDual ? kConvThreads : 512) umma_conv_
                     if (lane == 0) tma_store_wait_read<0>();
                     __syncwarp();
                     uint8_t *row = buf + lane * 128;
-                    auto pack_rows = [&](auto half_tag) {
-                        constexpr bool H = decltype(half_tag)::value;
+                    if constexpr (POST) {
+                        if (post_pending) {
+                            const bool here = mbar_wait_bounded(&ctl->post_full[warp - 2], post_ph, abort_flag);
+                            post_ph ^= 1u;
+                            if (!here && lane == 0) { atomicOr(err, ERRW_TIMEOUT); ctl->abort_flag = 1; }
+                            __syncwarp();
+                        }
+                    }
+                    // (what follows the rounding is fixed outside the loop over the columns: one uniform branch per chunk)
+                    auto pack_rows = [&](auto half_tag, auto add_tag, auto relu_tag, auto mask_tag) {
+                        constexpr bool H = decltype(half_tag)::value, ADD = decltype(add_tag)::value;
+                        constexpr bool RELU = decltype(relu_tag)::value, MASK = decltype(mask_tag)::value;
     #pragma unroll
                         for (int j = 0; j < 64; j += 8) {
                             float f[8];
@@ -374,11 +407,31 @@ __global__ void __launch_bounds__(MODE == kDual ? kConvThreads : 512) umma_conv_
                             pk.y = pack2_t<H>(f[2], f[3]);
                             pk.z = pack2_t<H>(f[4], f[5]);
                             pk.w = pack2_t<H>(f[6], f[7]);
-                            *(uint4 *)(row + ((((j >> 3) ^ (lane & 7)) & 7) << 4)) = pk;
+                            const int at16 = (((j >> 3) ^ (lane & 7)) & 7) << 4;
+                            if constexpr (POST) {
+                                uint4 a4 = make_uint4(0u, 0u, 0u, 0u), m4 = a4;
+                                if constexpr (ADD) a4 = *(const uint4 *)(add_buf + lane * 128 + at16);
+                                if constexpr (MASK) m4 = *(const uint4 *)(mask_buf + lane * 128 + at16);
+                                pk = post_chunk<H>(pk, ADD, a4, RELU, MASK, m4);
+                            }
+                            *(uint4 *)(row + at16) = pk;
                         }
                     };
-                    if (g.f16) pack_rows(std::true_type{}); else pack_rows(std::false_type{});
+                    auto pack = [&](auto add_tag, auto relu_tag, auto mask_tag) {
+                        if (g.f16) pack_rows(std::true_type{}, add_tag, relu_tag, mask_tag);
+                        else pack_rows(std::false_type{}, add_tag, relu_tag, mask_tag);
+                    };
+                    constexpr std::true_type yes{};
+                    constexpr std::false_type no{};
+                    if constexpr (!POST) pack(no, no, no);
+                    else if (g.post_mask) { if (g.post_add) pack(yes, no, yes); else pack(no, no, yes); }
+                    else if (g.post_add) { if (g.post_relu) pack(yes, yes, no); else pack(yes, no, no); }
+                    else pack(no, yes, no);
                     if constexpr (POST) {
+                        __syncwarp();                          // every lane has read its rows of the boxes
+                        if (c0 + 64 < ncols) fetch_post(i, c0 + 64); else fetch_post(i + 2, 0);
+                    }
+                    if constexpr (POST_STRIDED) {
                         // as below, with the other tensors' values of four pixels requested before the first is used
                         __syncwarp();
                         const int ch = lane & 7;
@@ -471,6 +524,8 @@ __global__ void __launch_bounds__(MODE == kDual ? kConvThreads : 512) umma_conv_
             }
         }
         if (warp == 2 && lane == 0) CONVBN_TRACE_POINT(9);
+        if constexpr (POST)                                 // (after a give-up: let the boxes in flight land)
+            if (post_pending) mbar_wait_bounded(&ctl->post_full[warp - 2], post_ph, nullptr, 200000000ull);
         if (lane == 0) tma_store_wait_all<0>();             // global writes done before the CTA exits
         if (warp == 2 && lane == 0) CONVBN_TRACE_POINT(10);
     }
@@ -596,9 +651,11 @@ static int sm_count() { return device_sm_count(); }
 
 template <int BN, ConvMode MODE = kPlain>
 static cudaError_t launch_bn(const CUtensorMap &ta, const CUtensorMap &tw, const CUtensorMap &tout,
-                             const CUtensorMap &tout2, ConvGemm g, const float *bias, int *err, cudaStream_t st) {
+                             const CUtensorMap &tout2, const CUtensorMap &tmask, ConvGemm g, const float *bias, int *err,
+                             cudaStream_t st) {
     const size_t a_bytes = (size_t)kBM * kBK * 2, b_bytes = (size_t)BN * kBK * 2;
-    size_t fixed = 1024 + kStagingBytes + sizeof(ConvSmemCtl) + (MODE == kDual ? 3 : 2) * (size_t)g.cn * sizeof(float) + 16;
+    const int extra = MODE == kPost ? (g.post_add != nullptr) + (g.post_mask != nullptr) : 0;
+    size_t fixed = 1024 + (size_t)(1 + extra) * kStagingBytes + sizeof(ConvSmemCtl) + (MODE == kDual ? 3 : 2) * (size_t)g.cn * sizeof(float) + 16;
     const int num_kb = g.taps_h * g.taps_w * (g.blockdiag ? 1 : g.ca / kBK);
     const long long m_tiles = (g.p + kBM - 1) / kBM, n_tiles = (g.cn + BN - 1) / BN;
     long long grid_l = m_tiles * n_tiles < sm_count() ? m_tiles * n_tiles : sm_count();
@@ -622,15 +679,16 @@ static cudaError_t launch_bn(const CUtensorMap &ta, const CUtensorMap &tw, const
     static PerDevice carve;
     prefer_max_shared_once(umma_conv_kernel<BN, MODE>, &carve);
     const unsigned grid = (unsigned)grid_l;
-    return launch_pdl(umma_conv_kernel<BN, MODE>, dim3(grid), dim3(kConvThreads), smem, st, ta, tw, tout, tout2, g, bias, err);
+    return launch_pdl(umma_conv_kernel<BN, MODE>, dim3(grid), dim3(kConvThreads), smem, st, ta, tw, tout, tout2, tmask, g, bias, err);
 }
 
 template <ConvMode MODE>
 static cudaError_t launch_mode(int bn, const CUtensorMap &ta, const CUtensorMap &tw, const CUtensorMap &tout,
-                               const CUtensorMap &tout2, const ConvGemm &g, const float *bias, int *err, cudaStream_t st) {
-    if (bn == 64) return launch_bn<64, MODE>(ta, tw, tout, tout2, g, bias, err, st);
-    if (bn == 128) return launch_bn<128, MODE>(ta, tw, tout, tout2, g, bias, err, st);
-    return launch_bn<256, MODE>(ta, tw, tout, tout2, g, bias, err, st);
+                               const CUtensorMap &tout2, const CUtensorMap &tmask, const ConvGemm &g, const float *bias,
+                               int *err, cudaStream_t st) {
+    if (bn == 64) return launch_bn<64, MODE>(ta, tw, tout, tout2, tmask, g, bias, err, st);
+    if (bn == 128) return launch_bn<128, MODE>(ta, tw, tout, tout2, tmask, g, bias, err, st);
+    return launch_bn<256, MODE>(ta, tw, tout, tout2, tmask, g, bias, err, st);
 }
 
 // Tile width: fewest rounds of tiles over the SMs, weighted by the time of one tile (N = 64 tiles are
@@ -663,10 +721,6 @@ cudaError_t launch_umma_conv(const UmmaConvShape &s, const void *act, const void
     g.out_strided = s.out_sw ? (__nv_bfloat16 *)out : nullptr;
     g.out_sn = s.out_sn; g.out_sh = s.out_sh; g.out_sw = s.out_sw;
     const bool with_post = post && post->any();
-    if (with_post && !s.out_sw) {
-        g.out_strided = (__nv_bfloat16 *)out;
-        g.out_sn = (long long)s.ho * s.wo * s.cn; g.out_sh = s.wo * s.cn; g.out_sw = s.cn;
-    }
     g.post_add = with_post ? (const __nv_bfloat16 *)post->add : nullptr;
     g.post_mask = with_post ? (const __nv_bfloat16 *)post->mask : nullptr;
     g.post_relu = with_post ? post->relu : 0;
@@ -677,6 +731,7 @@ cudaError_t launch_umma_conv(const UmmaConvShape &s, const void *act, const void
     const long long tiles_m = (g.p + kBM - 1) / kBM;
     int bn = s.blockdiag ? 64 : pick_bn(tiles_m, s.cn);
     while (s.tap_c && s.tap_c % bn) bn /= 2;            // a tile lies inside one tap
+    if (!s.out_sw && (g.post_add || g.post_mask) && bn > 128) bn = 128;       // room for the other tensors' staging areas
     CUtensorMap ta, tw, tout;
     // (in strided mode the output map is encoded but never used: every row is stored by its thread)
     if (!make_tmap_matrix_bf16(&tout, out, s.out_sw ? 32 : g.p, s.cn, 32, 64)) return cudaErrorInvalidValue;
@@ -691,10 +746,16 @@ cudaError_t launch_umma_conv(const UmmaConvShape &s, const void *act, const void
     if (e != cudaSuccess) return e;
     CUtensorMap tout2 = tout;
     if (out2 && !make_tmap_matrix_bf16(&tout2, out2, g.p, s.cn, 32, 64)) return cudaErrorInvalidValue;
-    if (with_post) return launch_mode<kPost>(bn, ta, tw, tout, tout2, g, bias, err, st);
-    if (out2) return launch_mode<kDual>(bn, ta, tw, tout, tout2, g, bias, err, st);
-    if (g.tap_c) return launch_mode<kTap>(bn, ta, tw, tout, tout2, g, bias, err, st);
-    return launch_mode<kPlain>(bn, ta, tw, tout, tout2, g, bias, err, st);
+    CUtensorMap tmask = tout;
+    if (with_post && !s.out_sw) {
+        if (g.post_add && !make_tmap_matrix_bf16(&tout2, post->add, g.p, s.cn, 32, 64)) return cudaErrorInvalidValue;
+        if (g.post_mask && !make_tmap_matrix_bf16(&tmask, post->mask, g.p, s.cn, 32, 64)) return cudaErrorInvalidValue;
+        return launch_mode<kPost>(bn, ta, tw, tout, tout2, tmask, g, bias, err, st);
+    }
+    if (with_post) return launch_mode<kPostStrided>(bn, ta, tw, tout, tout2, tmask, g, bias, err, st);
+    if (out2) return launch_mode<kDual>(bn, ta, tw, tout, tout2, tmask, g, bias, err, st);
+    if (g.tap_c) return launch_mode<kTap>(bn, ta, tw, tout, tout2, tmask, g, bias, err, st);
+    return launch_mode<kPlain>(bn, ta, tw, tout, tout2, tmask, g, bias, err, st);
 }
 
 // Forward pass of a small-C_in layer on the packed input (see stem_kernels.cu): tiles of 8 x 16 output
@@ -734,7 +795,7 @@ cudaError_t launch_stem_fwd(const Problem &pb, const void *x_packed, const void 
     int *err = nullptr;
     cudaError_t e = error_word_address(&err);
     if (e != cudaSuccess) return e;
-    return launch_bn<64>(ta, tw, tout, tout, g, bias, err, st);
+    return launch_bn<64>(ta, tw, tout, tout, tout, g, bias, err, st);
 }
 
 }  // namespace convbn
