@@ -145,8 +145,7 @@ bool fused_bwd_path(const convbn_desc *d, const Problem &pb) {
 bool strided_dgrad_ok(const convbn_desc *d, const Problem &pb);
 bool umma_dgrad_shape(const convbn_desc *d, const Problem &pb, UmmaConvShape *s);
 
-// partial_wgrad: the weight-gradient GEMM leaves partial tiles for an epilogue of the caller's
-Plan make_plan(const convbn_desc *d, const Problem &pb, int phase, bool partial_wgrad = false) {
+Plan make_plan(const convbn_desc *d, const Problem &pb, int phase) {
     Plan pl;
     UmmaConvShape us;
     if (phase == CONVBN_PHASE_TUNE_BWD) {
@@ -221,9 +220,9 @@ Plan make_plan(const convbn_desc *d, const Problem &pb, int phase, bool partial_
         }
     }
     if (pl.umma_wgrad) {
-        pl.uw = umma_wgrad_plan(pb, partial_wgrad);
-        pl.bsplits = pl.uw.scratch_splits;
-        part_bytes = wrows * pl.uw.scratch_splits * sizeof(float);
+        pl.uw = umma_wgrad_plan(pb);
+        pl.bsplits = pl.uw.splits;
+        part_bytes = wrows * pl.uw.splits * sizeof(float);
         dot_bytes = (size_t)pl.uw.kt * pb.c_out * sizeof(float);
     }
     switch (phase) {
@@ -663,13 +662,6 @@ int run_param_grads(const convbn_desc *d, const Problem &pb, const Plan &pl, con
     } else if (pl.umma_wgrad) {
         float *dotpart = (float *)at(ws, pl.dotpart);
         unsigned int *counters = (unsigned int *)at(ws, pl.counters);
-        if (pl.uw.final) {
-            const WgradFinal fin{w, vec3, dw, vec3 && need_bsum ? dotpart : nullptr};
-            LAUNCH("umma_wgrad", launch_umma_wgrad(pb, pl.uw, dz, x, partials, bsum, nullptr, st, -1, &fin));
-            if (need_bsum) LAUNCH("wgrad_finish", launch_wgrad_finish(pb, pl.uw, dotpart, bsum, vec3, b, mean, db, dgamma, dbeta, st));
-            *which = "umma";
-            return CONVBN_OK;
-        }
         LAUNCH("umma_wgrad", launch_umma_wgrad(pb, pl.uw, dz, x, partials, bsum, counters, st));
         LAUNCH("wgrad_epilogue_fused", launch_wgrad_epilogue_fused(pb, pl.uw, partials, bsum, w, vec3, b, mean, dw,
                                                                    dotpart, counters, db, dgamma, dbeta, need_bsum,
@@ -1259,7 +1251,7 @@ int tconv_view(const convbn_desc *d, TconvView *v) {
     CK(make_problem(&one, &v->sum_pb));
     v->bsplits = channel_sum_splits(v->sum_pb);
     v->fwd = make_plan(&v->conv, v->pb, CONVBN_PHASE_DEPLOY_FWD);
-    v->bwd = make_plan(&v->conv, v->pb, CONVBN_PHASE_DEPLOY_BWD, true);
+    v->bwd = make_plan(&v->conv, v->pb, CONVBN_PHASE_DEPLOY_BWD);
     v->wcount = (size_t)d->c_in * (d->c_out / d->groups) * d->kh * d->kw;
     size_t off = 0;
     auto take = [&](size_t bytes) { const size_t at0 = off; off += (bytes + 255) / 256 * 256; return at0; };

@@ -130,34 +130,18 @@ cudaError_t launch_reparam_dgrad_class(const Problem &pb, const void *w, const f
 
 // ---- tensor-core weight gradient (bf16 NHWC, groups = 1, channels multiples of 64) ---------------
 struct UmmaWgradPlan {
-    int splits = 1;           // partial tiles (clusters of pixel slices)
-    int cluster = 1;          // pixel slices that a cluster adds up: splits x cluster slices in all
-    int bn = 64;              // columns of a tile
-    int final = 0;            // 1: splits = 1 and the GEMM stores domega itself
-    int scratch_splits = 1;   // partial tiles the scratch is sized for (never fewer than splits)
+    int splits = 1;           // pixel slices = partial tiles
     long long per_split = 0;  // pixels per slice
     int kt = 1;               // k ranges of the epilogue (rows of dotpart)
     int kr = 8;               // k rows per epilogue block (8 or 2)
 };
 bool umma_wgrad_eligible(const Problem &pb);
-// partial_only: the caller wants partial tiles (an epilogue of its own)
-UmmaWgradPlan umma_wgrad_plan(const Problem &pb, bool partial_only = false);
-// Where a plan with `final` leaves domega (vec3 NULL: unscaled) and, if dotpart is given, [kt][C_out] dot products with w
-// for launch_wgrad_finish, which forms dbeta, db and dgamma from them and from bsum (vec3 NULL: db alone).
-struct WgradFinal {
-    const void *w;
-    const float *vec3;
-    float *dw, *dotpart;
-};
-cudaError_t launch_wgrad_finish(const Problem &pb, const UmmaWgradPlan &pl, const float *dotpart, const float *dsum,
-                                const float *vec3, const float *b, const float *mean, float *db, float *dgamma, float *dbeta,
-                                cudaStream_t st);
+UmmaWgradPlan umma_wgrad_plan(const Problem &pb);
 // partials: [splits][kdim][C_out] fp32 (k-major: the transpose of the weight layout)
 // bsum    : [splits][C_out] fp32 per-slice sums of dZ over pixels (from a ones row in the GEMM)
 // counters: C_out / 32 words (or `ncounters`) zeroed for the fused epilogue (may be NULL)
 cudaError_t launch_umma_wgrad(const Problem &pb, const UmmaWgradPlan &pl, const void *dz, const void *x,
-                              float *partials, float *bsum, unsigned int *counters, cudaStream_t st, int ncounters = -1,
-                              const WgradFinal *fin = nullptr);
+                              float *partials, float *bsum, unsigned int *counters, cudaStream_t st, int ncounters = -1);
 // Everything after the GEMM in one kernel: dw[co][k] = scale[co] * sum_splits partials (scale = first
 // C_out floats of vec3, 1 if NULL); with need_sums also dbeta, db, dgamma (vec3 given) or db = sum dZ.
 // dotpart: [kt][C_out] scratch; counters: C_out / 32 zeroed words.

@@ -134,21 +134,6 @@ __device__ __forceinline__ bool named_bar_all(uint32_t id, uint32_t count, bool 
     return all != 0;
 }
 
-// ---- thread-block clusters -----------------------------------------------------------------------------
-// Every thread of every block of the cluster arrives, then waits; shared-memory writes made before are visible after.
-__device__ __forceinline__ void cluster_sync_all() {
-    asm volatile("barrier.cluster.arrive.release;\n\tbarrier.cluster.wait.acquire;" ::: "memory");
-}
-// Address of the same shared-memory location in block `rank` of the cluster, and a store to it.
-__device__ __forceinline__ uint32_t cluster_map(uint32_t smem_addr, uint32_t rank) {
-    uint32_t a;
-    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(a) : "r"(smem_addr), "r"(rank));
-    return a;
-}
-__device__ __forceinline__ void cluster_store(uint32_t addr, uint32_t v) {
-    asm volatile("st.shared::cluster.u32 [%0], %1;" ::"r"(addr), "r"(v) : "memory");
-}
-
 // ---- TMA loads (global -> this CTA's shared memory, completion on an mbarrier) ----------------
 __device__ __forceinline__ void tma_load_2d(void *smem_dst, const CUtensorMap *map, uint64_t *bar, int x, int y) {
     asm volatile(

@@ -5,17 +5,9 @@
 // reduction index p as their slow axis in NHWC memory, so both are fed to tcgen05.mma as MN-major
 // tiles: the A tile is two [64 pixels][64 channels] im2col loads of X (two consecutive 64-wide slices
 // of k), the B tile is BN/64 plain [64 pixels][64 channels] boxes of dZ.  The pixel range is cut into
-// slices (grid.z); every CTA accumulates its slice in tensor memory in fp32.  The slices are added up, in fixed order and
-// from the fp32 sums (never from rounded values), in one of three ways (umma_wgrad_plan chooses):
-//   * the slices of a tile are one cluster of 1, 2, 4 or 8 CTAs, which exchange column blocks of their accumulators
-//     through distributed shared memory, add them and store domega, transposed and scaled, themselves; a small kernel
-//     finishes the per-channel gradients (wgrad_finish_kernel);
-//   * several clusters per tile: each writes one fp32 partial tile part[group][k][co] and a second kernel adds those
-//     (wgrad_epilogue_fused_kernel);
-//   * single CTAs write partial tiles (block-diagonal and packed-stem modes).
-// Partial tiles of every CTA were 9 to 19 MB per layer, written and read again by an epilogue of 10 to 16 us.
-#include <string.h>
-
+// `splits` slices (grid.z); every CTA accumulates its slice in tensor memory in fp32 and writes one
+// fp32 partial tile part[split][k][co].  A second kernel adds the slices in fixed order and forms
+// domega, dgamma, ... from the fp32 sums (never from rounded values).
 #include "kernels.h"
 #include "sm100_ptx.cuh"
 
@@ -43,12 +35,6 @@ struct WgradGemm {
     int stem, stem_tiles_w, stem_tiles_h;
     int no_ones;            // 1: no slice of ones (the packed stem input carries a constant-1 slot instead)
     int f16;                // 16-bit storage type: 0 bf16, 1 IEEE half
-    // RED instantiations
-    int cluster;            // CTAs of a cluster (slices blockIdx.z / cluster * cluster ... of one tile)
-    int final;              // 1: one cluster per tile, domega and the dot products are stored here
-    const __nv_bfloat16 *w; // [C_out][kdim]
-    const float *vec3;      // NULL: domega = domega', no dot products
-    float *dw, *dotpart;    // dotpart: [4 k-tiles][C_out], or NULL
 };
 
 struct WgradSmemCtl {
@@ -59,18 +45,7 @@ struct WgradSmemCtl {
     int abort_flag;
 };
 
-// One step of adding 32 values over 32 lanes: lanes whose bit is set keep the upper half of the values.
-template <int N>
-__device__ __forceinline__ void halve_over_lanes(float (&v)[32], int lane) {
-#pragma unroll
-    for (int i = 0; i < N / 2; ++i) {
-        const bool up = lane & (N / 2);
-        const float send = up ? v[i] : v[i + N / 2], keep = up ? v[i + N / 2] : v[i];
-        v[i] = keep + __shfl_xor_sync(0xffffffffu, send, N / 2);
-    }
-}
-
-template <int BN, bool RED>
+template <int BN>
 __global__ void __launch_bounds__(kWThreads) umma_wgrad_kernel(const __grid_constant__ CUtensorMap tm_x,
                                                               const __grid_constant__ CUtensorMap tm_dz,
                                                               const WgradGemm g, float *__restrict__ partials,
@@ -213,8 +188,7 @@ __global__ void __launch_bounds__(kWThreads) umma_wgrad_kernel(const __grid_cons
             }
             if (ok) umma_commit(&ctl->tmem_full);
         }
-        __syncwarp();
-    } else if constexpr (!RED) {
+    } else {
         const int quarter = warp & 3;
         const bool ok = __all_sync(0xffffffffu, mbar_wait_bounded(&ctl->tmem_full, 0, abort_flag));
         if (!ok && lane == 0) { atomicOr(err, ERRW_TIMEOUT); ctl->abort_flag = 1; }
@@ -245,90 +219,6 @@ __global__ void __launch_bounds__(kWThreads) umma_wgrad_kernel(const __grid_cons
             }
         }
     }
-    if constexpr (RED) {
-        // Column block d of the tile belongs to rank d of the cluster.  recv[source rank][column][128 rows] fp32 takes the
-        // place of the ring, which every CTA of the cluster has drained once all have met here.
-        const int quarter = warp & 3, row = quarter * 32 + lane;
-        const int C = g.cluster, sl = BN / C, rank = (int)(blockIdx.z % (unsigned)C), group = (int)(blockIdx.z / (unsigned)C);
-        const uint32_t recv = smem_u32(tiles);
-        if (warp >= 2 && num_kb > 0) {
-            const bool ok = __all_sync(0xffffffffu, mbar_wait_bounded(&ctl->tmem_full, 0, abort_flag));
-            if (!ok && lane == 0) { atomicOr(err, ERRW_TIMEOUT); ctl->abort_flag = 1; }
-            tc_fence_after_sync();
-        }
-        cluster_sync_all();
-        if (warp >= 2) {
-#pragma unroll 1
-            for (int c0 = 0; c0 < BN; c0 += 32) {
-                uint32_t v[32];
-                if (num_kb > 0) {
-                    tmem_ld_32x32(tmem_base + ((uint32_t)(quarter * 32) << 16) + (uint32_t)c0, v);
-                    tmem_ld_wait();
-                } else {
-#pragma unroll
-                    for (int j = 0; j < 32; ++j) v[j] = 0u;
-                }
-#pragma unroll
-                for (int j0 = 0; j0 < 32; j0 += 8) {              // 8 divides the column blocks
-                    const int col = c0 + j0, dst = col / sl;
-                    const uint32_t base = cluster_map(recv + (uint32_t)((rank * sl + col - dst * sl) * 128 + row) * 4u, (uint32_t)dst);
-#pragma unroll
-                    for (int j = 0; j < 8; ++j) cluster_store(base + (uint32_t)j * 512u, v[j0 + j]);
-                }
-            }
-        }
-        cluster_sync_all();
-        if (warp >= 2) {
-            const float *mine = (const float *)tiles + row;
-            const int k = k0 + row, co_base = n0 + rank * sl;
-            const bool row_ok = k < g.kdim, sum_row = k == g.kdim;
-            float *brow = bsum + (size_t)group * g.c_out;
-#pragma unroll 1
-            for (int c0 = 0; c0 < sl; c0 += 32) {
-                if (co_base + c0 >= g.c_out) break;                // (C_out and the column blocks are multiples of 8)
-                const int nc = sl - c0 < 32 ? sl - c0 : 32;
-                float v[32];
-#pragma unroll
-                for (int j = 0; j < 32; ++j) {
-                    v[j] = 0.f;
-                    if (j < nc)
-                        for (int r = 0; r < C; ++r) v[j] += mine[(size_t)(r * sl + c0 + j) * 128];
-                }
-                const int left = g.c_out - co_base - c0 < nc ? g.c_out - co_base - c0 : nc;
-                if (sum_row) {
-#pragma unroll
-                    for (int j = 0; j < 32; ++j)
-                        if (j < left) brow[co_base + c0 + j] = v[j];
-                }
-                if (!g.final) {
-                    if (row_ok) {
-                        float *orow = partials + ((size_t)group * g.kdim + k) * g.c_out + co_base + c0;
-#pragma unroll
-                        for (int j = 0; j < 32; j += 4)
-                            if (j < left) *(float4 *)(orow + j) = make_float4(v[j], v[j + 1], v[j + 2], v[j + 3]);
-                    }
-                    continue;
-                }
-                // lanes are consecutive k: each store is 128 contiguous bytes of a weight row
-#pragma unroll
-                for (int j = 0; j < 32; ++j) {
-                    float wv = 0.f;
-                    if (j < left && row_ok) {
-                        const size_t o = (size_t)(co_base + c0 + j) * g.kdim + k;
-                        g.dw[o] = (g.vec3 ? g.vec3[co_base + c0 + j] : 1.f) * v[j];
-                        if (g.dotpart) wv = load_h16(g.w + o, g.f16);
-                    }
-                    v[j] = row_ok ? v[j] * wv : 0.f;
-                }
-                if (g.dotpart) {
-                    halve_over_lanes<32>(v, lane); halve_over_lanes<16>(v, lane); halve_over_lanes<8>(v, lane);
-                    halve_over_lanes<4>(v, lane); halve_over_lanes<2>(v, lane);
-                    // lane l holds the sum of column l over the warp's 32 rows
-                    if (lane < left) g.dotpart[(size_t)(blockIdx.x * 4 + quarter) * g.c_out + co_base + c0 + lane] = v[0];
-                }
-            }
-        }
-    }
     tc_fence_before_sync();
     __syncthreads();
     if (warp == 1) tmem_dealloc(tmem_base, BN);
@@ -354,17 +244,17 @@ bool umma_wgrad_eligible(const Problem &pb) {
 
 static int wgrad_bn(const Problem &pb) { return pb.c_out >= 256 ? 256 : (pb.c_out >= 128 ? 128 : 64); }
 
-// Single CTAs, a partial tile each.  Resident CTAs: the 64- and 128-wide tiles run two CTAs per SM (their stage rings are
-// sized for it, launch_w), which measured 25-40 % faster than one CTA with a deeper ring; 256-wide tiles own an SM.  The
-// slice count minimises  rounds over the resident slots x (pixels per slice + a fixed cost per CTA, in pixels) + a small
-// cost per slice for the epilogue that adds the slices up; a grid a few CTAs larger than the slots would otherwise run a
-// second, nearly empty round.
-static UmmaWgradPlan single_cta_plan(const Problem &pb) {
+UmmaWgradPlan umma_wgrad_plan(const Problem &pb) {
     UmmaWgradPlan pl;
     const bool bd = pb.groups > 1;
     const int bn = bd ? 64 : wgrad_bn(pb);
     const long long kd = bd ? (long long)pb.kh * pb.kw * 64 : pb.kdim;
     const long long m_tiles = (kd / 64 + 1 + 1) / 2, n_tiles = (pb.c_out + bn - 1) / bn;   // + the ones slice
+    // Resident CTAs: the 64- and 128-wide tiles run two CTAs per SM (their stage rings are sized for it,
+    // launch_w), which measured 25-40 % faster than one CTA with a deeper ring; 256-wide tiles own an SM.
+    // The slice count minimises  rounds over the resident slots x (pixels per slice + a fixed cost per
+    // CTA, in pixels) + a small cost per slice for the epilogue that adds the slices up; a grid a few
+    // CTAs larger than the slots would otherwise run a second, nearly empty round.
     const long long slots = (long long)device_sm_count() * (bn == 256 ? 1 : 2), tiles = m_tiles * n_tiles;
     const long long max_splits = (pb.p + 4 * kWP - 1) / (4 * kWP);     // at least 256 pixels per slice
     long long splits = 1;
@@ -377,72 +267,10 @@ static UmmaWgradPlan single_cta_plan(const Problem &pb) {
     }
     long long per = (pb.p + splits - 1) / splits;
     per = (per + kWP - 1) / kWP * kWP;
-    pl.bn = bn;
     pl.per_split = per;
-    pl.splits = pl.scratch_splits = (int)((pb.p + per - 1) / per);
-    return pl;
-}
-
-// Estimated time (us) of `cluster` x `groups` slices and tiles of bn columns.  Measured inputs: an SM takes about 90 bytes
-// of operands per ns from L2; a CTA needs 3 us before its first and after its last MMA; the epilogue over partial tiles
-// takes 6 us and 3 TB/s.  (clusters of 8 and 4 do not fill the last SMs of a GPC: 128 and 144 of 148)
-static double wgrad_cost(const Problem &pb, int bn, int cluster, int groups, bool final) {
-    const int sms = device_sm_count();
-    const long long m_tiles = (pb.kdim / 64 + 2) / 2, n_tiles = (pb.c_out + bn - 1) / bn;
-    const long long ctas = m_tiles * n_tiles * cluster * groups, per_sm = bn == 256 ? 1 : 2;
-    const long long usable = cluster == 8 ? sms * 128 / 148 : (cluster == 4 ? sms * 144 / 148 : sms);
-    const long long rounds = (ctas + usable * per_sm - 1) / (usable * per_sm);
-    const double share = ctas > usable ? (double)per_sm : 1.0;
-    const double kb = (double)((pb.p + (long long)cluster * groups * kWP - 1) / ((long long)cluster * groups * kWP));
-    const double t_kb = share * (16384.0 + bn * 128.0) / 90000.0;
-    const double tile = bn / 64.0;
-    const double cta = kb * t_kb + 3.0 + 0.5 * tile + (final ? 0.6 * tile / cluster : 0.0);
-    return rounds * cta + (final ? 2.0 : 6.0 + (double)groups * pb.kdim * pb.c_out * 8.0 / 3.0e6);
-}
-
-static UmmaWgradPlan search_plan(const Problem &pb, bool partial_only) {
-    UmmaWgradPlan pl = single_cta_plan(pb);
-    if (pb.groups == 1) {
-        // (the scratch keeps the size of the single-CTA plan, which bounds every choice below)
-        double best = -1.0;
-        for (int bn = 64; bn <= 256; bn *= 2) {
-            if (bn > 64 && pb.c_out <= bn / 2) continue;
-            for (int c = 1; c <= 8; c *= 2)
-                for (int gr = 1; gr <= pl.scratch_splits; ++gr) {
-                    const bool final = gr == 1 && !partial_only;
-                    if ((long long)c * gr * kWP > pb.p + (long long)c * kWP && c * gr > 1) break;      // a block of pixels each
-                    const double t = wgrad_cost(pb, bn, c, gr, final);
-                    if (best >= 0 && t >= best) continue;
-                    best = t;
-                    pl.bn = bn; pl.cluster = c; pl.splits = gr; pl.final = final ? 1 : 0;
-                }
-        }
-        const long long z = (long long)pl.cluster * pl.splits, per = (pb.p + z - 1) / z;
-        pl.per_split = (per + kWP - 1) / kWP * kWP;
-    }
+    pl.splits = (int)((pb.p + per - 1) / per);
     wgrad_epilogue_shape(pb, &pl);
-    if (pl.final) pl.kt = (int)(4 * ((pb.kdim / 64 + 2) / 2));          // rows of dotpart
     return pl;
-}
-
-// The search takes some microseconds and is asked for several times per library call: its result is kept per thread, keyed
-// by all that it depends on.
-UmmaWgradPlan umma_wgrad_plan(const Problem &pb, bool partial_only) {
-    struct Key { long long p; int kdim, taps, c_out, groups, partial_only, sms; };
-    struct Entry { Key key; UmmaWgradPlan plan; bool used; };
-    thread_local Entry cache[64] = {};
-    thread_local unsigned next = 0;
-    Key key;
-    memset(&key, 0, sizeof(key));
-    key.p = pb.p; key.kdim = pb.kdim; key.taps = pb.kh * pb.kw; key.c_out = pb.c_out; key.groups = pb.groups;
-    key.partial_only = partial_only ? 1 : 0; key.sms = device_sm_count();
-    for (const Entry &e : cache)
-        if (e.used && memcmp(&e.key, &key, sizeof(key)) == 0) return e.plan;
-    Entry &slot = cache[next++ % 64];
-    slot.key = key;
-    slot.plan = search_plan(pb, partial_only);
-    slot.used = true;
-    return slot.plan;
 }
 
 // k rows per epilogue block (the block's other lanes split the slices): very many slices -> 2 rows x 16
@@ -455,41 +283,31 @@ void wgrad_epilogue_shape(const Problem &pb, UmmaWgradPlan *pl) {
     pl->kt = (pb.kdim + pl->kr - 1) / pl->kr;   // epilogue blocks along k = rows of dotpart
 }
 
-template <int BN, bool RED = false>
+template <int BN>
 static cudaError_t launch_w(const CUtensorMap &tx, const CUtensorMap &tdz, WgradGemm g, const UmmaWgradPlan &pl,
                             const Problem &pb, float *partials, float *bsum, unsigned int *counters, int *err,
                             cudaStream_t st, int ncounters = -1) {
     constexpr size_t stage = 2 * kChunkBytes + (BN / 64) * kChunkBytes;
     int stages = BN == 128 ? 3 : 4;                    // 128-wide: 3 x 32 KB, so that two CTAs share an SM
     const long long max_kb = (pl.per_split + kWP - 1) / kWP;
-    if (stages > max_kb && !RED) stages = (int)max_kb;
+    if (stages > max_kb) stages = (int)max_kb;
     g.stages = stages;
-    static_assert(!RED || (BN == 128 ? 3 : 4) * stage >= 128 * BN * sizeof(float), "the exchange buffer takes the ring's place");
     size_t smem = stages * stage + 1024 + sizeof(WgradSmemCtl);
     const size_t floor_smem = (size_t)(228 * 1024) / (512 / BN + 1) + 1024;
     if (smem < floor_smem) smem = floor_smem;
     static PerDevice attr_done;
-    if (cudaError_t e = max_dynamic_smem_once(umma_wgrad_kernel<BN, RED>, 210 * 1024, &attr_done); e != cudaSuccess) return e;
+    if (cudaError_t e = max_dynamic_smem_once(umma_wgrad_kernel<BN>, 210 * 1024, &attr_done); e != cudaSuccess) return e;
     static PerDevice carve;
-    prefer_max_shared_once(umma_wgrad_kernel<BN, RED>, &carve);
+    prefer_max_shared_once(umma_wgrad_kernel<BN>, &carve);
     dim3 grid((unsigned)((g.kdim / 64 + (g.no_ones ? 1 : 2)) / 2), (unsigned)((pb.c_out + BN - 1) / BN),
-              (unsigned)(pl.splits * pl.cluster));
-    if (RED)
-        return launch_pdl_cluster(umma_wgrad_kernel<BN, RED>, grid, dim3(kWThreads), dim3(1, 1, (unsigned)pl.cluster), smem, st,
-                                  tx, tdz, g, partials, bsum, counters, ncounters >= 0 ? ncounters : pb.c_out / 32, err);
-    return launch_pdl(umma_wgrad_kernel<BN, RED>, grid, dim3(kWThreads), smem, st, tx, tdz, g, partials, bsum, counters,
+              (unsigned)pl.splits);
+    return launch_pdl(umma_wgrad_kernel<BN>, grid, dim3(kWThreads), smem, st, tx, tdz, g, partials, bsum, counters,
                       ncounters >= 0 ? ncounters : pb.c_out / 32, err);
 }
 
 cudaError_t launch_umma_wgrad(const Problem &pb, const UmmaWgradPlan &pl, const void *dz, const void *x,
-                              float *partials, float *bsum, unsigned int *counters, cudaStream_t st, int ncounters,
-                              const WgradFinal *fin) {
+                              float *partials, float *bsum, unsigned int *counters, cudaStream_t st, int ncounters) {
     WgradGemm g;
-    g.cluster = pl.cluster; g.final = pl.final; g.w = nullptr; g.vec3 = nullptr; g.dw = g.dotpart = nullptr;
-    if (pl.final) {
-        if (!fin) return cudaErrorInvalidValue;
-        g.w = (const __nv_bfloat16 *)fin->w; g.vec3 = fin->vec3; g.dw = fin->dw; g.dotpart = fin->dotpart;
-    }
     g.ho = pb.h_out; g.wo = pb.w_out; g.c_in = pb.c_in; g.c_out = pb.c_out; g.taps_w = pb.kw;
     g.lower_h = -pb.pad_h; g.lower_w = -pb.pad_w; g.stride_h = pb.stride_h; g.stride_w = pb.stride_w;
     g.dil_h = pb.dil_h; g.dil_w = pb.dil_w; g.kdim = pb.kdim; g.p = pb.p; g.per_split = pl.per_split; g.stages = 1;
@@ -506,12 +324,10 @@ cudaError_t launch_umma_wgrad(const Problem &pb, const UmmaWgradPlan &pl, const 
     int *err = nullptr;
     cudaError_t e = error_word_address(&err);
     if (e != cudaSuccess) return e;
-    if (!g.blockdiag) {
-        if (pl.bn == 64) return launch_w<64, true>(tx, tdz, g, pl, pb, partials, bsum, counters, err, st, ncounters);
-        if (pl.bn == 128) return launch_w<128, true>(tx, tdz, g, pl, pb, partials, bsum, counters, err, st, ncounters);
-        return launch_w<256, true>(tx, tdz, g, pl, pb, partials, bsum, counters, err, st, ncounters);
-    }
-    return launch_w<64>(tx, tdz, g, pl, pb, partials, bsum, counters, err, st, ncounters);
+    const int bn = g.blockdiag ? 64 : wgrad_bn(pb);
+    if (bn == 64) return launch_w<64>(tx, tdz, g, pl, pb, partials, bsum, counters, err, st, ncounters);
+    if (bn == 128) return launch_w<128>(tx, tdz, g, pl, pb, partials, bsum, counters, err, st, ncounters);
+    return launch_w<256>(tx, tdz, g, pl, pb, partials, bsum, counters, err, st, ncounters);
 }
 
 // ---- epilogue over k-major partials ------------------------------------------------------------
@@ -702,50 +518,6 @@ cudaError_t launch_wgrad_epilogue_fused(const Problem &pb, const UmmaWgradPlan &
                       dgamma, dbeta, ns, call_f16());
 }
 
-// The per-channel gradients after a weight-gradient GEMM that stored domega itself: dotpart [rows][C_out], dsum [C_out].
-// One block per 32 channels, eight groups of rows added in order.
-__global__ void __launch_bounds__(256) wgrad_finish_kernel(int c_out, int rows, const float *__restrict__ dotpart,
-                                                           const float *__restrict__ dsum_v, const float *__restrict__ vec3,
-                                                           const float *__restrict__ b, const float *__restrict__ mean,
-                                                           float *__restrict__ db, float *__restrict__ dgamma,
-                                                           float *__restrict__ dbeta) {
-    __shared__ float red[8][33];
-    pdl_wait();
-    pdl_launch_dependents();
-    const int ch = threadIdx.x & 31, grp = threadIdx.x >> 5, co = blockIdx.x * 32 + ch;
-    float d = 0.f;
-    if (vec3)
-        for (int r = grp; r < rows; r += 64) {
-            float q[8];
-#pragma unroll
-            for (int u = 0; u < 8; ++u) q[u] = r + 8 * u < rows ? __ldcg(dotpart + (size_t)(r + 8 * u) * c_out + co) : 0.f;
-#pragma unroll
-            for (int u = 0; u < 8; ++u) d += q[u];
-        }
-    red[grp][ch] = d;
-    __syncthreads();
-    if (grp) return;
-    d = 0.f;
-    for (int i = 0; i < 8; ++i) d += red[i][ch];
-    const float dsum = __ldcg(dsum_v + co);
-    if (!vec3) {
-        if (db) db[co] = dsum;
-        return;
-    }
-    dbeta[co] = dsum;
-    if (db) db[co] = vec3[co] * dsum;
-    dgamma[co] = vec3[2 * c_out + co] * (d + dsum * ((b ? b[co] : 0.f) - mean[co]));
-}
-
-cudaError_t launch_wgrad_finish(const Problem &pb, const UmmaWgradPlan &pl, const float *dotpart, const float *dsum,
-                                const float *vec3, const float *b, const float *mean, float *db, float *dgamma, float *dbeta,
-                                cudaStream_t st) {
-    static PerDevice carve;
-    prefer_max_shared_once(wgrad_finish_kernel, &carve);
-    return launch_pdl(wgrad_finish_kernel, dim3(pb.c_out / 32), dim3(256), 0, st, pb.c_out, pl.kt, dotpart, dsum, vec3, b, mean,
-                      db, dgamma, dbeta);
-}
-
 // ---- small-C_in ("stem") layers -------------------------------------------------------------------
 UmmaWgradPlan stem_wgrad_plan(const Problem &pb) {
     UmmaWgradPlan pl;
@@ -767,7 +539,6 @@ cudaError_t launch_stem_wgrad(const Problem &pb, const UmmaWgradPlan &pl, const 
                               float *partials, float *bsum, cudaStream_t st) {
     const int krows = stem_krows(pb);
     WgradGemm g;
-    g.cluster = 1; g.final = 0; g.w = nullptr; g.vec3 = nullptr; g.dw = g.dotpart = nullptr;
     g.ho = pb.h_out; g.wo = pb.w_out; g.c_in = 64; g.c_out = pb.c_out; g.taps_w = 1;
     g.lower_h = g.lower_w = 0; g.stride_h = g.stride_w = g.dil_h = g.dil_w = 1;
     g.kdim = krows * 64;
