@@ -120,7 +120,6 @@ struct Plan {
     size_t dy = 0;         // Eval backward: s dZ, storage dtype
     size_t vec3 = 0;       // Eval forward: [s | beta - mean s | r]
     size_t dotpart = 0;    // [kt][C_out] fp32 (tensor-core weight-gradient path)
-    size_t counters = 0;   // C_out / 32 words (fused epilogue)
     int splits = 1, bsplits = 1, bn_splits = 1;
     size_t xpk = 0, wst = 0;   // small-C_in layers: packed input [n][hp][wp][8], expanded weights [C_out][kh][64]
     bool stem = false;
@@ -163,7 +162,6 @@ Plan make_plan(const convbn_desc *d, const Problem &pb, int phase) {
         pl.partials = put((size_t)pl.uw.splits * pb.c_out * pb.kdim * sizeof(float));
         pl.bsum = put((size_t)pl.uw.splits * pb.c_out * sizeof(float));
         pl.dotpart = put((size_t)pl.uw.kt * pb.c_out * sizeof(float));
-        pl.counters = put((size_t)(pb.c_out / 32 + 1) * sizeof(unsigned int));
         pl.total = o;
         return pl;
     }
@@ -243,14 +241,12 @@ Plan make_plan(const convbn_desc *d, const Problem &pb, int phase) {
             pl.partials = take(part_bytes);
             pl.bsum = take((size_t)pl.bsplits * pb.c_out * sizeof(float));
             pl.dotpart = take(dot_bytes);
-            pl.counters = take(dot_bytes ? (size_t)(pb.c_out / 32 + 1) * sizeof(unsigned int) : 0);
             break;
         case CONVBN_PHASE_TUNE_BWD_WEIGHT:
             pl.xpk = take(xpk_bytes);
             pl.partials = take(part_bytes);
             pl.bsum = take((size_t)pl.bsplits * pb.c_out * sizeof(float));
             pl.dotpart = take(dot_bytes);
-            pl.counters = take(dot_bytes ? (size_t)(pb.c_out / 32 + 1) * sizeof(unsigned int) : 0);
             break;
         case CONVBN_PHASE_EVAL_FWD:
             pl.vec3 = take(3 * (size_t)pb.c_out * sizeof(float));
@@ -274,7 +270,6 @@ Plan make_plan(const convbn_desc *d, const Problem &pb, int phase) {
             pl.bsum = take((size_t)(pl.bn_splits > pl.bsplits ? pl.bn_splits : pl.bsplits) * pb.c_out * sizeof(float));
             pl.partials = take(part_bytes);
             pl.dotpart = take(dot_bytes);
-            pl.counters = take(dot_bytes ? (size_t)(pb.c_out / 32 + 1) * sizeof(unsigned int) : 0);
             break;
         default:
             break;
@@ -636,10 +631,9 @@ int run_param_grads(const convbn_desc *d, const Problem &pb, const Plan &pl, con
         LAUNCH("channel_sum", launch_channel_sum_partial(pb, d->dtype, d->layout, dz, bsum, pl.bsplits, st));
     if (pl.stem_win_wgrad) {
         float *dotpart = (float *)at(ws, pl.dotpart);
-        unsigned int *counters = (unsigned int *)at(ws, pl.counters);
-        LAUNCH("stem_wgrad", launch_stem_window_wgrad(pb, dz, x, partials, bsum, counters, st));
+        LAUNCH("stem_wgrad", launch_stem_window_wgrad(pb, dz, x, partials, bsum, st));
         LAUNCH("wgrad_epilogue_fused", launch_wgrad_epilogue_fused(pb, pl.uw, partials, bsum, w, vec3, b, mean, dw,
-                                                                   dotpart, counters, db, dgamma, dbeta, need_bsum,
+                                                                   dotpart, db, dgamma, dbeta, need_bsum,
                                                                    st));
         *which = "umma-stem";
     } else if (pl.stem) {
@@ -654,17 +648,16 @@ int run_param_grads(const convbn_desc *d, const Problem &pb, const Plan &pl, con
                                                                     dgamma, dbeta, st));
         *which = "grouped-mma";
     } else if (pl.grouped_wgrad) {
-        LAUNCH("grouped_wgrad", launch_umma_wgrad(pb, pl.uw, dz, x, partials, bsum, nullptr, st));
+        LAUNCH("grouped_wgrad", launch_umma_wgrad(pb, pl.uw, dz, x, partials, bsum, st));
         LAUNCH("wgrad_epilogue_bd", launch_wgrad_epilogue_bd(pb, partials, pl.uw.splits, need_bsum ? bsum : nullptr,
                                                              need_bsum ? pl.bsplits : 0, w, vec3, b, mean, dw, db,
                                                              dgamma, dbeta, st));
         *which = "grouped-umma";
     } else if (pl.umma_wgrad) {
         float *dotpart = (float *)at(ws, pl.dotpart);
-        unsigned int *counters = (unsigned int *)at(ws, pl.counters);
-        LAUNCH("umma_wgrad", launch_umma_wgrad(pb, pl.uw, dz, x, partials, bsum, counters, st));
+        LAUNCH("umma_wgrad", launch_umma_wgrad(pb, pl.uw, dz, x, partials, bsum, st));
         LAUNCH("wgrad_epilogue_fused", launch_wgrad_epilogue_fused(pb, pl.uw, partials, bsum, w, vec3, b, mean, dw,
-                                                                   dotpart, counters, db, dgamma, dbeta, need_bsum,
+                                                                   dotpart, db, dgamma, dbeta, need_bsum,
                                                                    st));
         *which = "umma";
     } else if (pl.dw_tma_wgrad) {
@@ -977,9 +970,8 @@ static int tune_bwd_impl(const convbn_desc *desc, const void *dz, const void *x,
     cudaStream_t st = (cudaStream_t)stream;
     float *partials = (float *)at(workspace, pl.partials), *bsum = (float *)at(workspace, pl.bsum);
     float *dotpart = (float *)at(workspace, pl.dotpart);
-    unsigned int *counters = (unsigned int *)at(workspace, pl.counters);
     const float *vec3 = (const float *)saved;
-    LAUNCH("umma_bwd", launch_fused_bwd1x1(pb, dz, x, w, vec3, dx, partials, bsum, counters, st, &post));
+    LAUNCH("umma_bwd", launch_fused_bwd1x1(pb, dz, x, w, vec3, dx, partials, bsum, st, &post));
     t_last_kernel[CONVBN_PHASE_TUNE_BWD] = "umma-fused-bwd";
     if (defer_join && !g_prof.on) {
         // dX is complete on the caller's stream; the parameter gradients are finished on the side lane
@@ -989,13 +981,12 @@ static int tune_bwd_impl(const convbn_desc *desc, const void *dz, const void *x,
         CU(cudaStreamWaitEvent(lane->stream, lane->fork, 0));
         cudaStream_t st = lane->stream;
         LAUNCH("wgrad_epilogue_fused", launch_wgrad_epilogue_fused(pb, pl.uw, partials, bsum, w, vec3, b, run_mean, dw,
-                                                                   dotpart, counters, db, dgamma, dbeta, true, st));
+                                                                   dotpart, db, dgamma, dbeta, true, st));
         CU(cudaEventRecord(lane->join, lane->stream));
         lane->pending = true;
         return CONVBN_OK;
     }
-    LAUNCH("wgrad_epilogue_fused", launch_wgrad_epilogue_fused(pb, pl.uw, partials, bsum, w, vec3, b, run_mean, dw, dotpart,
-                                                               counters, db, dgamma, dbeta, true, st));
+    LAUNCH("wgrad_epilogue_fused", launch_wgrad_epilogue_fused(pb, pl.uw, partials, bsum, w, vec3, b, run_mean, dw, dotpart, db, dgamma, dbeta, true, st));
     return CONVBN_OK;
 }
 
@@ -1116,11 +1107,11 @@ int convbn_eval_bwd(const convbn_desc *desc, const void *dz, const void *x, cons
             [&]() -> int {
                 if (fused) {
                     LAUNCH("umma_bwd", launch_fused_bwd1x1(pb, dz, x, w, vec3, dx, (float *)at(inner, pt.partials),
-                                                           (float *)at(inner, pt.bsum), (unsigned int *)at(inner, pt.counters), st));
+                                                           (float *)at(inner, pt.bsum), st));
                     LAUNCH("wgrad_epilogue_fused",
                            launch_wgrad_epilogue_fused(pb, pt.uw, (const float *)at(inner, pt.partials),
                                                        (const float *)at(inner, pt.bsum), w, vec3, nullptr, run_mean, dw,
-                                                       (float *)at(inner, pt.dotpart), (unsigned int *)at(inner, pt.counters),
+                                                       (float *)at(inner, pt.dotpart),
                                                        nullptr, nullptr, nullptr, false, st));
                     t_last_kernel[CONVBN_PHASE_EVAL_BWD] = "umma-fused-bwd";
                     return CONVBN_OK;
@@ -1386,8 +1377,8 @@ int convbn_tconv_tune_bwd(const convbn_desc *desc, const void *dz, const void *x
             if (v.bwd.umma_wgrad) {
                 float *partials = (float *)at(inner_b, v.bwd.partials);
                 // (the GEMM's own sums, of X here, are not needed)
-                LAUNCH("umma_wgrad", launch_umma_wgrad(v.pb, v.bwd.uw, x, dz, partials, (float *)at(inner_b, v.bwd.bsum), counters,
-                                                       st, desc->c_out / 32));
+                LAUNCH("umma_wgrad", launch_umma_wgrad(v.pb, v.bwd.uw, x, dz, partials, (float *)at(inner_b, v.bwd.bsum), st,
+                                                       counters, desc->c_out / 32));
                 LAUNCH("tconv_epilogue", launch_tconv_wgrad_epilogue(desc->c_in, desc->c_out, taps, partials, v.bwd.uw.splits, w,
                                                                      vec3, b, run_mean, bsum, v.bsplits, dwp, counters, dw, db,
                                                                      dgamma, dbeta, st));

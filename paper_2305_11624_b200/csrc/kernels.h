@@ -133,22 +133,23 @@ struct UmmaWgradPlan {
     int splits = 1;           // pixel slices = partial tiles
     long long per_split = 0;  // pixels per slice
     int kt = 1;               // k ranges of the epilogue (rows of dotpart)
-    int kr = 8;               // k rows per epilogue block (8 or 2)
+    int kr = 8;               // k rows per block (32, 8 or 2)
 };
 bool umma_wgrad_eligible(const Problem &pb);
 UmmaWgradPlan umma_wgrad_plan(const Problem &pb);
 // partials: [splits][kdim][C_out] fp32 (k-major: the transpose of the weight layout)
 // bsum    : [splits][C_out] fp32 per-slice sums of dZ over pixels (from a ones row in the GEMM)
-// counters: C_out / 32 words (or `ncounters`) zeroed for the fused epilogue (may be NULL)
+// counters: `ncounters` words zeroed for an epilogue that counts its blocks (may be NULL)
 cudaError_t launch_umma_wgrad(const Problem &pb, const UmmaWgradPlan &pl, const void *dz, const void *x,
-                              float *partials, float *bsum, unsigned int *counters, cudaStream_t st, int ncounters = -1);
-// Everything after the GEMM in one kernel: dw[co][k] = scale[co] * sum_splits partials (scale = first
+                              float *partials, float *bsum, cudaStream_t st, unsigned int *counters = nullptr,
+                              int ncounters = 0);
+// Everything after the GEMM: dw[co][k] = scale[co] * sum_splits partials (scale = first
 // C_out floats of vec3, 1 if NULL); with need_sums also dbeta, db, dgamma (vec3 given) or db = sum dZ.
-// dotpart: [kt][C_out] scratch; counters: C_out / 32 zeroed words.
+// dotpart: [kt][C_out] scratch.
 cudaError_t launch_wgrad_epilogue_fused(const Problem &pb, const UmmaWgradPlan &pl, const float *partials,
                                         const float *bsum, const void *w, const float *vec3, const float *b,
-                                        const float *mean, float *dw, float *dotpart, unsigned int *counters,
-                                        float *db, float *dgamma, float *dbeta, bool need_sums, cudaStream_t st);
+                                        const float *mean, float *dw, float *dotpart, float *db, float *dgamma, float *dbeta,
+                                        bool need_sums, cudaStream_t st);
 
 // ---- first-layer convolutions with C_in <= 8 (see stem_kernels.cu) -------------------------------
 bool stem_eligible(const Problem &pb);
@@ -184,11 +185,11 @@ cudaError_t launch_stem_window_fwd(const Problem &pb, const void *x, const void 
                                    cudaStream_t st, const BnFold *fold = nullptr, int relu = 0);
 // Weight gradient of the same layers (C_in <= 3, C_out = 64) straight from X and dZ: one fp32 partial
 // [kdim][C_out] and one row of sums of dZ per CTA (stem_window_wgrad_ctas of them), in the layout the fused
-// epilogue of the dense weight-gradient path reads; `counters` are zeroed for it.
+// epilogue of the dense weight-gradient path reads.
 bool stem_window_wgrad_eligible(const Problem &pb);
 int stem_window_wgrad_ctas(const Problem &pb);
 cudaError_t launch_stem_window_wgrad(const Problem &pb, const void *dz, const void *x, float *partials, float *bsum,
-                                     unsigned int *counters, cudaStream_t st);
+                                     cudaStream_t st);
 // Backward data of the same layers (C_out = 64, W_out <= 128) as a scatter GEMM with the overlap-add of the
 // window positions done on chip (see stem_window_dgrad.cu); s_vec (NULL = 1) is folded into the weights.
 bool stem_window_dgrad_eligible(const Problem &pb);
@@ -284,11 +285,11 @@ cudaError_t launch_bn_eval_finish(const Problem &pb, const float *part_g, const 
 
 // ---- fused backward of 1x1 stride-1 layers (see umma_bwd1x1.cu) ----------------------------------------
 // dX plus one fp32 partial [C_in][C_out] and one row of sums of dZ per CTA (fused_bwd1x1_ctas of them), in the
-// layout the fused epilogue reads; `counters` are zeroed for it.  vec3 = saved [s | b' | r].
+// layout the fused epilogue reads.  vec3 = saved [s | b' | r].
 bool fused_bwd1x1_eligible(const Problem &pb);
 int fused_bwd1x1_ctas(const Problem &pb);
 cudaError_t launch_fused_bwd1x1(const Problem &pb, const void *dz, const void *x, const void *w, const float *vec3,
-                                void *dx, float *partials, float *bsum, unsigned int *counters, cudaStream_t st,
+                                void *dx, float *partials, float *bsum, cudaStream_t st,
                                 const PostOp *post = nullptr);
 
 // ---- elementwise glue between blocks (glue_kernels.cu): mode 0 relu(a), 1 relu(a + b), 2 a masked by b > 0, 3 a + b

@@ -416,7 +416,6 @@ __global__ void __launch_bounds__(kWgThreads) stem_window_wgrad_kernel(const __g
                                                                       const __nv_bfloat16 *__restrict__ x,
                                                                       float *__restrict__ partials,
                                                                       float *__restrict__ bsum,
-                                                                      unsigned int *__restrict__ counters, int ncounters,
                                                                       int *err) {
     extern __shared__ uint8_t smem_raw[];
     uint8_t *xs = (uint8_t *)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
@@ -454,8 +453,6 @@ __global__ void __launch_bounds__(kWgThreads) stem_window_wgrad_kernel(const __g
         tmem_relinquish();
     }
     pdl_wait();
-    if (counters && blockIdx.x == 0)
-        for (int i = threadIdx.x; i < ncounters; i += kWgThreads) counters[i] = 0u;
     tc_fence_before_sync();
     __syncthreads();
     tc_fence_after_sync();
@@ -737,12 +734,12 @@ bool stem_window_wgrad_eligible(const Problem &pb) { return plan_window_wgrad(pb
 // (one function per channel count: the once-per-device flags must not be shared between the kernels)
 template <int C>
 static cudaError_t launch_window_wgrad(const CUtensorMap &tdz, const WinWgrad &g, size_t smem, unsigned grid, const void *x,
-                                       float *partials, float *bsum, unsigned int *counters, int *err, cudaStream_t st) {
+                                       float *partials, float *bsum, int *err, cudaStream_t st) {
     static PerDevice attr, carve;
     if (cudaError_t e = max_dynamic_smem_once(stem_window_wgrad_kernel<C>, 227 * 1024, &attr); e != cudaSuccess) return e;
     prefer_max_shared_once(stem_window_wgrad_kernel<C>, &carve);
     return launch_pdl(stem_window_wgrad_kernel<C>, dim3(grid), dim3(kWgThreads), smem, st, tdz, g,
-                      (const __nv_bfloat16 *)x, partials, bsum, counters, g.c_out / 32, err);
+                      (const __nv_bfloat16 *)x, partials, bsum, err);
 }
 
 int stem_window_wgrad_ctas(const Problem &pb) {
@@ -751,7 +748,7 @@ int stem_window_wgrad_ctas(const Problem &pb) {
 }
 
 cudaError_t launch_stem_window_wgrad(const Problem &pb, const void *dz, const void *x, float *partials, float *bsum,
-                                     unsigned int *counters, cudaStream_t st) {
+                                     cudaStream_t st) {
     const WinWgPlan pl = plan_window_wgrad(pb);
     if (!pl.ok) return cudaErrorInvalidValue;
     WinWgrad g;
@@ -773,9 +770,9 @@ cudaError_t launch_stem_window_wgrad(const Problem &pb, const void *dz, const vo
     if (e != cudaSuccess) return e;
     const unsigned grid = (unsigned)stem_window_wgrad_ctas(pb);
     switch (pb.c_in) {
-        case 1: return launch_window_wgrad<1>(tdz, g, pl.smem, grid, x, partials, bsum, counters, err, st);
-        case 2: return launch_window_wgrad<2>(tdz, g, pl.smem, grid, x, partials, bsum, counters, err, st);
-        default: return launch_window_wgrad<3>(tdz, g, pl.smem, grid, x, partials, bsum, counters, err, st);
+        case 1: return launch_window_wgrad<1>(tdz, g, pl.smem, grid, x, partials, bsum, err, st);
+        case 2: return launch_window_wgrad<2>(tdz, g, pl.smem, grid, x, partials, bsum, err, st);
+        default: return launch_window_wgrad<3>(tdz, g, pl.smem, grid, x, partials, bsum, err, st);
     }
 }
 

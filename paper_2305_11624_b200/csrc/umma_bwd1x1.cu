@@ -62,7 +62,6 @@ __global__ void __launch_bounds__(kFbThreads) fused_bwd1x1_kernel(const __grid_c
                                                                  const __grid_constant__ CUtensorMap tm_dx,
                                                                  const FusedBwd g, const __nv_bfloat16 *__restrict__ w,
                                                                  float *__restrict__ partials, float *__restrict__ bsum,
-                                                                 unsigned int *__restrict__ counters, int ncounters,
                                                                  int *err) {
     using S = FbShape<CI, CO>;
     extern __shared__ uint8_t smem_raw[];
@@ -94,8 +93,6 @@ __global__ void __launch_bounds__(kFbThreads) fused_bwd1x1_kernel(const __grid_c
         for (int i = threadIdx.x; i < 1024 / 16; i += kFbThreads) ((uint4 *)ones)[i] = one4;
     }
     pdl_wait();
-    if (counters && blockIdx.x == 0)
-        for (int i = threadIdx.x; i < ncounters; i += kFbThreads) counters[i] = 0u;
     // omega' = s omega (Sec. 3.3), one rounding to bf16, laid out as the MN-major B operand of the data-gradient
     // GEMM: K = co rows of 128 bytes (64 ci), 128-byte swizzle, one block per 64 input channels
     for (int i = threadIdx.x; i < CO * (CI / 8); i += kFbThreads) {
@@ -347,21 +344,21 @@ __global__ void __launch_bounds__(kFbThreads) fused_bwd1x1_kernel(const __grid_c
 namespace {
 template <int CI, int CO, bool POST>
 cudaError_t launch_fb_as(const CUtensorMap &tdz, const CUtensorMap &tx, const CUtensorMap &tdx, const FusedBwd &g, unsigned grid,
-                      const void *w, float *partials, float *bsum, unsigned int *counters, int *err, cudaStream_t st) {
+                      const void *w, float *partials, float *bsum, int *err, cudaStream_t st) {
     using S = FbShape<CI, CO>;
     const size_t smem = 1024 + (size_t)kFbStages * S::kStageBytes + (size_t)CI * CO * 2 + 1024 + 8 * 4096 + sizeof(FbCtl) + 64;
     static PerDevice attr, carve;
     if (cudaError_t e = max_dynamic_smem_once(fused_bwd1x1_kernel<CI, CO, POST>, 227 * 1024, &attr); e != cudaSuccess) return e;
     prefer_max_shared_once(fused_bwd1x1_kernel<CI, CO, POST>, &carve);
     return launch_pdl(fused_bwd1x1_kernel<CI, CO, POST>, dim3(grid), dim3(kFbThreads), smem, st, tdz, tx, tdx, g,
-                      (const __nv_bfloat16 *)w, partials, bsum, counters, CO / 32, err);
+                      (const __nv_bfloat16 *)w, partials, bsum, err);
 }
 template <int CI, int CO>
 cudaError_t launch_fb(const CUtensorMap &tdz, const CUtensorMap &tx, const CUtensorMap &tdx, const FusedBwd &g, unsigned grid,
-                      const void *w, float *partials, float *bsum, unsigned int *counters, int *err, cudaStream_t st) {
+                      const void *w, float *partials, float *bsum, int *err, cudaStream_t st) {
     if (g.post_add || g.post_mask || g.post_relu)
-        return launch_fb_as<CI, CO, true>(tdz, tx, tdx, g, grid, w, partials, bsum, counters, err, st);
-    return launch_fb_as<CI, CO, false>(tdz, tx, tdx, g, grid, w, partials, bsum, counters, err, st);
+        return launch_fb_as<CI, CO, true>(tdz, tx, tdx, g, grid, w, partials, bsum, err, st);
+    return launch_fb_as<CI, CO, false>(tdz, tx, tdx, g, grid, w, partials, bsum, err, st);
 }
 }  // namespace
 
@@ -377,7 +374,7 @@ int fused_bwd1x1_ctas(const Problem &pb) {
 }
 
 cudaError_t launch_fused_bwd1x1(const Problem &pb, const void *dz, const void *x, const void *w, const float *vec3, void *dx,
-                                float *partials, float *bsum, unsigned int *counters, cudaStream_t st, const PostOp *post) {
+                                float *partials, float *bsum, cudaStream_t st, const PostOp *post) {
     if (!fused_bwd1x1_eligible(pb)) return cudaErrorInvalidValue;
     FusedBwd g;
     g.p = pb.p; g.m_tiles = (int)((pb.p + 127) / 128); g.vec3 = vec3; g.f16 = call_f16();
@@ -393,10 +390,10 @@ cudaError_t launch_fused_bwd1x1(const Problem &pb, const void *dz, const void *x
     cudaError_t e = error_word_address(&err);
     if (e != cudaSuccess) return e;
     const unsigned grid = (unsigned)fused_bwd1x1_ctas(pb);
-    if (pb.c_in == 256) return launch_fb<256, 64>(tdz, tx, tdx, g, grid, w, partials, bsum, counters, err, st);
-    if (pb.c_in == 128) return launch_fb<128, 64>(tdz, tx, tdx, g, grid, w, partials, bsum, counters, err, st);
-    if (pb.c_out == 256) return launch_fb<64, 256>(tdz, tx, tdx, g, grid, w, partials, bsum, counters, err, st);
-    return launch_fb<64, 128>(tdz, tx, tdx, g, grid, w, partials, bsum, counters, err, st);
+    if (pb.c_in == 256) return launch_fb<256, 64>(tdz, tx, tdx, g, grid, w, partials, bsum, err, st);
+    if (pb.c_in == 128) return launch_fb<128, 64>(tdz, tx, tdx, g, grid, w, partials, bsum, err, st);
+    if (pb.c_out == 256) return launch_fb<64, 256>(tdz, tx, tdx, g, grid, w, partials, bsum, err, st);
+    return launch_fb<64, 128>(tdz, tx, tdx, g, grid, w, partials, bsum, err, st);
 }
 
 }  // namespace convbn

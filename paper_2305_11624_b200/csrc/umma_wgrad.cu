@@ -273,20 +273,20 @@ UmmaWgradPlan umma_wgrad_plan(const Problem &pb) {
     return pl;
 }
 
-// k rows per epilogue block (the block's other lanes split the slices): very many slices -> 2 rows x 16
-// lanes; few slices or very many blocks -> 32 rows x 1 lane (every block pays a fence and an atomic)
+// k rows per block of wgrad_add_kernel (its other threads split the slices): as many as leave about 100 blocks and one
+// batch of eight loads per thread, 32 rows (1 or 2 slice groups), 8 (8 groups) or 2 (32 groups)
 void wgrad_epilogue_shape(const Problem &pb, UmmaWgradPlan *pl) {
-    const long long blocks8 = (long long)(pb.c_out / 32) * ((pb.kdim + 7) / 8);
-    pl->kr = pl->splits > 192 ? 2 : ((pl->splits <= 8 || blocks8 > 600) && blocks8 / 4 >= device_sm_count() ? 32 : 8);
-    // very large weight matrices in few slices: 8 groups of 8 rows per block halve the blocks (and their fences) again
-    if (pl->kr == 32 && pl->splits <= 4 && blocks8 / 8 >= 2 * device_sm_count()) pl->kr = 64;
-    pl->kt = (pb.kdim + pl->kr - 1) / pl->kr;   // epilogue blocks along k = rows of dotpart
+    const long long cols = pb.c_out / 64;
+    if (pl->splits <= 16 && cols * ((pb.kdim + 31) / 32) >= 96) pl->kr = 32;
+    else if (pl->splits <= 64 && cols * ((pb.kdim + 7) / 8) >= 48) pl->kr = 8;
+    else pl->kr = 2;
+    pl->kt = (pb.kdim + pl->kr - 1) / pl->kr;   // blocks along k = rows of dotpart
 }
 
 template <int BN>
 static cudaError_t launch_w(const CUtensorMap &tx, const CUtensorMap &tdz, WgradGemm g, const UmmaWgradPlan &pl,
-                            const Problem &pb, float *partials, float *bsum, unsigned int *counters, int *err,
-                            cudaStream_t st, int ncounters = -1) {
+                            const Problem &pb, float *partials, float *bsum, int *err, cudaStream_t st,
+                            unsigned int *counters = nullptr, int ncounters = 0) {
     constexpr size_t stage = 2 * kChunkBytes + (BN / 64) * kChunkBytes;
     int stages = BN == 128 ? 3 : 4;                    // 128-wide: 3 x 32 KB, so that two CTAs share an SM
     const long long max_kb = (pl.per_split + kWP - 1) / kWP;
@@ -302,11 +302,11 @@ static cudaError_t launch_w(const CUtensorMap &tx, const CUtensorMap &tdz, Wgrad
     dim3 grid((unsigned)((g.kdim / 64 + (g.no_ones ? 1 : 2)) / 2), (unsigned)((pb.c_out + BN - 1) / BN),
               (unsigned)pl.splits);
     return launch_pdl(umma_wgrad_kernel<BN>, grid, dim3(kWThreads), smem, st, tx, tdz, g, partials, bsum, counters,
-                      ncounters >= 0 ? ncounters : pb.c_out / 32, err);
+                      ncounters, err);
 }
 
 cudaError_t launch_umma_wgrad(const Problem &pb, const UmmaWgradPlan &pl, const void *dz, const void *x,
-                              float *partials, float *bsum, unsigned int *counters, cudaStream_t st, int ncounters) {
+                              float *partials, float *bsum, cudaStream_t st, unsigned int *counters, int ncounters) {
     WgradGemm g;
     g.ho = pb.h_out; g.wo = pb.w_out; g.c_in = pb.c_in; g.c_out = pb.c_out; g.taps_w = pb.kw;
     g.lower_h = -pb.pad_h; g.lower_w = -pb.pad_w; g.stride_h = pb.stride_h; g.stride_w = pb.stride_w;
@@ -325,197 +325,141 @@ cudaError_t launch_umma_wgrad(const Problem &pb, const UmmaWgradPlan &pl, const 
     cudaError_t e = error_word_address(&err);
     if (e != cudaSuccess) return e;
     const int bn = g.blockdiag ? 64 : wgrad_bn(pb);
-    if (bn == 64) return launch_w<64>(tx, tdz, g, pl, pb, partials, bsum, counters, err, st, ncounters);
-    if (bn == 128) return launch_w<128>(tx, tdz, g, pl, pb, partials, bsum, counters, err, st, ncounters);
-    return launch_w<256>(tx, tdz, g, pl, pb, partials, bsum, counters, err, st, ncounters);
+    if (bn == 64) return launch_w<64>(tx, tdz, g, pl, pb, partials, bsum, err, st, counters, ncounters);
+    if (bn == 128) return launch_w<128>(tx, tdz, g, pl, pb, partials, bsum, err, st, counters, ncounters);
+    return launch_w<256>(tx, tdz, g, pl, pb, partials, bsum, err, st, counters, ncounters);
 }
 
 // ---- epilogue over k-major partials ------------------------------------------------------------
-// One kernel finishes every parameter gradient (Table 2, Tune row) from the fp32 partial tiles:
-//   block (bx, by): 32 output channels x KR k rows x SL lanes over the pixel slices (KR SL = 32,
-//   up to 1024 threads), REP such row groups one after the other: (8, 4) when there are few slices, (2, 16)
-//   when there are many, (8, 1) x 4 with 256 threads when there are few slices and thousands of blocks
-//     acc[k][co] = sum_split part[split][k][co]        (each lane a strided subset, lanes added in order)
-//     dw[co][k]  = s[co] acc                           (transposed through shared memory)
-//     dotpart[by][co] = sum over the block's k rows of acc * w[co][k]
-//   the LAST block to finish for a group of 32 channels (a counter per group, zeroed by the GEMM
-//   kernel) adds dotpart over all k blocks and bsum over all slices, lanes strided + a fixed shuffle
-//   tree, so the result does not depend on which block came last:
-//     dbeta = sum dZ,  db = s dbeta,  dgamma = r (sum_k domega' omega + dbeta (b - mu_hat))
-//   plain mode (vec3 == NULL): dw = acc, db = sum dZ if requested.
-template <int KR, int SL, int REP>
-__global__ void __launch_bounds__(32 * KR * SL, SL == 16 ? 2 : (KR * SL == 8 ? 4 : 1)) wgrad_epilogue_fused_kernel(
-    int c_out, int kdim, const float *__restrict__ part, int splits, const float *__restrict__ bsum, int bsplits,
-    const __nv_bfloat16 *__restrict__ w, const float *__restrict__ vec3, const float *__restrict__ b,
-    const float *__restrict__ mean, float *__restrict__ dw, float *__restrict__ dotpart,
-    unsigned int *__restrict__ counters, float *__restrict__ db, float *__restrict__ dgamma,
-    float *__restrict__ dbeta, int need_sums, int f16) {
-    static_assert(KR * SL <= 32, "at most 32 warps per block");
-    // loads in flight per thread: the (2, 16) shape has the most blocks and is held to 32 registers, so
-    // that two of its 1024-thread blocks share an SM
-    constexpr int NB = SL == 16 ? 4 : 8;
-    __shared__ float tile[REP][SL][KR][33];
-    __shared__ int is_last;
+// Two kernels finish every parameter gradient (Table 2, Tune row) from the fp32 partial tiles part[split][k][co].
+//
+// wgrad_add_kernel: block = 64 output channels x KR weight rows k.  Thread (float4 of channels, k, slice group z < SL)
+// adds slices z, z + SL, ..., eight loads in flight, then the groups are added in order through shared memory and
+//     dw[co][k] = s[co] acc,    dotpart[k block][co] = sum over the block's k of acc w[co][k].
+// wgrad_finish_kernel: dbeta = sum dZ,  db = s dbeta,  dgamma = r (sum_k domega' omega + dbeta (b - mu_hat)).
+// Plain mode (vec3 == NULL): dw = acc, db = sum dZ if requested.
+//
+// Bound by the latency of the L2 reads (9 to 19 MB of partials): with (KR, SL) chosen so that a thread's loads are one
+// batch, a block is one round trip.  As one kernel whose last block per channel group did the finish (a fence, an atomic
+// and two more dependent reads behind every block) it took 10 us on the 3x3 64 -> 64 layer at 56 x 56, N = 32, and 16 us on
+// 3x3 512 -> 512 at 7 x 7, N = 64.
+template <int KR, int SL>
+__global__ void __launch_bounds__(KR * 16 * SL) wgrad_add_kernel(int c_out, int kdim, const float *__restrict__ part, int splits,
+                                                                const __nv_bfloat16 *__restrict__ w,
+                                                                const float *__restrict__ scale, float *__restrict__ dw,
+                                                                float *__restrict__ dotpart, int f16) {
+    constexpr int T = KR * 16 * SL, E = KR * 64;                    // threads, elements
+    constexpr int SUB = T > E ? T / E : 1, PER = T > E ? 1 : E / T; // threads per element, elements per thread
+    __shared__ float tile[SL][KR][65];
     pdl_wait();
     pdl_launch_dependents();
-    const int tx = threadIdx.x & 31, ty = (threadIdx.x >> 5) % KR, tz = (threadIdx.x >> 5) / KR;
-    const int co0 = blockIdx.x * 32, k0 = blockIdx.y * (KR * REP);   // REP groups of KR rows per block
-    const size_t slice = (size_t)kdim * c_out;
-    // the weights the second phase multiplies with are requested now, together with the partials
-    float wv[REP];
+    const int co0 = blockIdx.x * 64, k0 = blockIdx.y * KR;
+    // the element(s) this thread finishes: k runs fastest, over neighbouring groups of SUB lanes
+    const int sub = threadIdx.x % SUB;
+    float wv[PER], sv[PER];
 #pragma unroll
-    for (int rep = 0; rep < REP; ++rep) {
-        const int k = k0 + rep * KR + (int)(threadIdx.x % KR), co = co0 + (int)(threadIdx.x / KR);
-        wv[rep] = (vec3 && threadIdx.x < 32 * KR && k < kdim) ? load_h16(w + (size_t)co * kdim + k, f16) : 0.f;
+    for (int i = 0; i < PER; ++i) {
+        const int e = threadIdx.x / SUB + i * (T / SUB), k = k0 + e % KR, co = co0 + e / KR;
+        wv[i] = dotpart && sub == 0 && k < kdim ? load_h16(w + (size_t)co * kdim + k, f16) : 0.f;
+        sv[i] = scale ? scale[co] : 1.f;
     }
-    constexpr int NBF = REP > 1 ? 32 / REP : 1;      // slices the preloading path below can take
-    if (SL == 1 && REP > 1 && splits <= NBF) {
-        // few slices, several row groups: request every value of every group before the first use, so that
-        // REP x splits loads are in flight per thread instead of `splits`; same order of additions as below
-        float a[REP][NBF];
-#pragma unroll
-        for (int rep = 0; rep < REP; ++rep) {
-            const int k = k0 + rep * KR + ty;
-            const float *src = part + (size_t)k * c_out + co0 + tx;
-#pragma unroll
-            for (int u = 0; u < NBF; ++u) a[rep][u] = (k < kdim && u < splits) ? __ldcg(src + (size_t)u * slice) : 0.f;
-        }
-#pragma unroll
-        for (int rep = 0; rep < REP; ++rep) {
-            float tot = 0.f;
-#pragma unroll
-            for (int u = 0; u < NBF; ++u) tot += a[rep][u];
-            tile[rep][tz][ty][tx] = tot;
-        }
-    } else
-#pragma unroll
-    for (int rep = 0; rep < REP; ++rep) {
-        const int k = k0 + rep * KR + ty;
-        // NB independent sums per thread keep NB loads in flight; they are added in a fixed order
-        float a[NB];
-#pragma unroll
-        for (int u = 0; u < NB; ++u) a[u] = 0.f;
-        if (k < kdim) {
-            const float *src = part + (size_t)k * c_out + co0 + tx;
-            int sp = tz;
-            for (; sp + (NB - 1) * SL < splits; sp += NB * SL) {
-#pragma unroll
-                for (int u = 0; u < NB; ++u) a[u] += __ldcg(src + (size_t)(sp + u * SL) * slice);
-            }
-#pragma unroll
-            for (int u = 0; u < NB; ++u)
-                if (sp + u * SL < splits) a[u] += __ldcg(src + (size_t)(sp + u * SL) * slice);
-        }
-        float tot = 0.f;
-#pragma unroll
-        for (int u = 0; u < NB; ++u) tot += a[u];
-        tile[rep][tz][ty][tx] = tot;
-    }
-    __syncthreads();
-    if (threadIdx.x < 32 * KR) {
-        const int kk = threadIdx.x % KR, cl = threadIdx.x / KR, co = co0 + cl;
-        float d = 0.f;
-#pragma unroll
-        for (int rep = 0; rep < REP; ++rep) {
-            const int k = k0 + rep * KR + kk;
-            if (k < kdim) {
-                float v = 0.f;
-#pragma unroll
-                for (int z = 0; z < SL; ++z) v += tile[rep][z][kk][cl];
-                const size_t o = (size_t)co * kdim + k;
-                dw[o] = (vec3 ? vec3[co] : 1.f) * v;
-                d = fmaf(v, wv[rep], d);
-            }
-        }
-        if (vec3) {
-#pragma unroll
-            for (int o = 1; o < KR; o <<= 1) d += __shfl_xor_sync(0xffffffffu, d, o);
-            if (kk == 0) dotpart[(size_t)blockIdx.y * c_out + co] = d;
-        }
-    }
-    if (!need_sums) return;
-    // ---- last block of this channel group finishes the per-channel quantities ----
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        __threadfence();        // after the barrier: orders the whole block's dw / dotpart writes before the count
-        const unsigned int done = atomicAdd(&counters[blockIdx.x], 1u);
-        is_last = (done == gridDim.y - 1);
-    }
-    __syncthreads();
-    if (!is_last) return;
-    __threadfence();
-    // Thread (channel ch, row group grp) adds rows grp, grp + ngrp, ... of the dZ sums and of the dot
-    // partials: a row's 32 channels are one 128-byte read, a thread's (up to NB) rows are requested
-    // together, and the groups are then added in order: one memory round trip instead of one per row.
     {
-        __shared__ float fin[2][32][33];
-        const int ch = tx, grp = (int)(threadIdx.x >> 5), ngrp = KR * SL;
-        float ds = 0.f, dt = 0.f;
-        for (int base = grp; base < bsplits; base += ngrp * NB) {
-            float v[NB];
+        const int l = threadIdx.x & 15, ky = (threadIdx.x >> 4) % KR, z = threadIdx.x / (16 * KR), k = k0 + ky;
+        const size_t slice = (size_t)kdim * c_out;
+        const float *src = part + (size_t)k * c_out + co0 + l * 4;
+        float4 a = make_float4(0.f, 0.f, 0.f, 0.f);
+        if (k < kdim)
+            for (int sp = z; sp < splits; sp += 8 * SL) {
+                float4 v[8];
 #pragma unroll
-            for (int u = 0; u < NB; ++u) {
-                const int sp = base + u * ngrp;
-                v[u] = sp < bsplits ? __ldcg(bsum + (size_t)sp * c_out + co0 + ch) : 0.f;
+                for (int u = 0; u < 8; ++u)
+                    v[u] = sp + u * SL < splits ? __ldcg((const float4 *)(src + (size_t)(sp + u * SL) * slice))
+                                                : make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+                for (int u = 0; u < 8; ++u) { a.x += v[u].x; a.y += v[u].y; a.z += v[u].z; a.w += v[u].w; }
             }
+        float *t = &tile[z][ky][l * 4];
+        t[0] = a.x; t[1] = a.y; t[2] = a.z; t[3] = a.w;
+    }
+    __syncthreads();
 #pragma unroll
-            for (int u = 0; u < NB; ++u) ds += v[u];
-        }
-        if (vec3)
-            for (int base = grp; base < (int)gridDim.y; base += ngrp * NB) {
-                float v[NB];
+    for (int i = 0; i < PER; ++i) {
+        const int e = threadIdx.x / SUB + i * (T / SUB), k = k0 + e % KR, cl = e / KR;
+        float v = 0.f;
 #pragma unroll
-                for (int u = 0; u < NB; ++u) {
-                    const int t = base + u * ngrp;
-                    v[u] = t < (int)gridDim.y ? __ldcg(dotpart + (size_t)t * c_out + co0 + ch) : 0.f;
-                }
+        for (int z = sub; z < SL; z += SUB) v += tile[z][e % KR][cl];
 #pragma unroll
-                for (int u = 0; u < NB; ++u) dt += v[u];
-            }
-        fin[0][grp][ch] = ds;
-        fin[1][grp][ch] = dt;
-        __syncthreads();
-        if (threadIdx.x < 32) {
-            const int co = co0 + ch;
-            float dsum = 0.f, dot = 0.f;
-            for (int gq = 0; gq < ngrp; ++gq) { dsum += fin[0][gq][ch]; dot += fin[1][gq][ch]; }
-            if (!vec3) {
-                if (db) db[co] = dsum;
-            } else {
-                const float s = vec3[co], r = vec3[2 * c_out + co];
-                dbeta[co] = dsum;
-                if (db) db[co] = s * dsum;
-                dgamma[co] = r * (dot + dsum * ((b ? b[co] : 0.f) - mean[co]));
-            }
+        for (int o = 1; o < SUB; o <<= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+        if (sub == 0 && k < kdim) dw[(size_t)(co0 + cl) * kdim + k] = sv[i] * v;
+        if (dotpart) {
+            float d = v * wv[i];
+#pragma unroll
+            for (int o = SUB; o < SUB * KR; o <<= 1) d += __shfl_xor_sync(0xffffffffu, d, o);
+            if (sub == 0 && e % KR == 0) dotpart[(size_t)blockIdx.y * c_out + co0 + cl] = d;
         }
     }
-    if (threadIdx.x == 0) counters[blockIdx.x] = 0;   // leave the counter clean for the next call
+}
+
+// dotpart [rows][C_out], bsum [bsplits][C_out]: one block per 32 channels, 32 groups of rows added in order.
+__global__ void __launch_bounds__(1024) wgrad_finish_kernel(int c_out, int rows, const float *__restrict__ dotpart, int bsplits,
+                                                            const float *__restrict__ bsum, const float *__restrict__ vec3,
+                                                            const float *__restrict__ b, const float *__restrict__ mean,
+                                                            float *__restrict__ db, float *__restrict__ dgamma,
+                                                            float *__restrict__ dbeta) {
+    __shared__ float red[2][32][33];
+    pdl_wait();
+    pdl_launch_dependents();
+    const int ch = threadIdx.x & 31, grp = threadIdx.x >> 5, co = blockIdx.x * 32 + ch;
+    auto column = [&](const float *v, int n) {
+        float acc = 0.f;
+        for (int r = grp; r < n; r += 128) {
+            float q[4];
+#pragma unroll
+            for (int u = 0; u < 4; ++u) q[u] = r + 32 * u < n ? __ldcg(v + (size_t)(r + 32 * u) * c_out + co) : 0.f;
+            acc += (q[0] + q[1]) + (q[2] + q[3]);
+        }
+        return acc;
+    };
+    red[0][grp][ch] = column(bsum, bsplits);
+    red[1][grp][ch] = vec3 ? column(dotpart, rows) : 0.f;
+    __syncthreads();
+    if (grp) return;
+    float dsum = 0.f, d = 0.f;
+#pragma unroll
+    for (int i = 0; i < 32; ++i) { dsum += red[0][i][ch]; d += red[1][i][ch]; }
+    if (!vec3) {
+        if (db) db[co] = dsum;
+        return;
+    }
+    dbeta[co] = dsum;
+    if (db) db[co] = vec3[co] * dsum;
+    dgamma[co] = vec3[2 * c_out + co] * (d + dsum * ((b ? b[co] : 0.f) - mean[co]));
+}
+
+template <int KR, int SL>
+static cudaError_t launch_add(const Problem &pb, const UmmaWgradPlan &pl, const float *partials, const void *w, const float *vec3,
+                              float *dw, float *dotpart, cudaStream_t st) {
+    static PerDevice carve;
+    prefer_max_shared_once(wgrad_add_kernel<KR, SL>, &carve);
+    return launch_pdl(wgrad_add_kernel<KR, SL>, dim3(pb.c_out / 64, pl.kt), dim3(KR * 16 * SL), 0, st, pb.c_out, pb.kdim, partials,
+                      pl.splits, (const __nv_bfloat16 *)w, vec3, dw, dotpart, call_f16());
 }
 
 cudaError_t launch_wgrad_epilogue_fused(const Problem &pb, const UmmaWgradPlan &pl, const float *partials,
                                         const float *bsum, const void *w, const float *vec3, const float *b,
-                                        const float *mean, float *dw, float *dotpart, unsigned int *counters,
-                                        float *db, float *dgamma, float *dbeta, bool need_sums, cudaStream_t st) {
-    const dim3 grid(pb.c_out / 32, pl.kt);
-    const int ns = need_sums ? 1 : 0;
-    static PerDevice carve_a, carve_b;
-    prefer_max_shared_once(wgrad_epilogue_fused_kernel<8, 4, 1>, &carve_a);
-    prefer_max_shared_once(wgrad_epilogue_fused_kernel<2, 16, 1>, &carve_b);
-    if (pl.kr == 64)
-        return launch_pdl(wgrad_epilogue_fused_kernel<8, 1, 8>, grid, dim3(256), 0, st, pb.c_out, pb.kdim, partials,
-                          pl.splits, bsum, pl.splits, (const __nv_bfloat16 *)w, vec3, b, mean, dw, dotpart, counters, db,
-                          dgamma, dbeta, ns, call_f16());
-    if (pl.kr == 32)                                  // 4 groups of 8 rows, 256 threads: several blocks per SM
-        return launch_pdl(wgrad_epilogue_fused_kernel<8, 1, 4>, grid, dim3(256), 0, st, pb.c_out, pb.kdim, partials,
-                          pl.splits, bsum, pl.splits, (const __nv_bfloat16 *)w, vec3, b, mean, dw, dotpart, counters, db,
-                          dgamma, dbeta, ns, call_f16());
-    if (pl.kr == 8)
-        return launch_pdl(wgrad_epilogue_fused_kernel<8, 4, 1>, grid, dim3(1024), 0, st, pb.c_out, pb.kdim, partials,
-                          pl.splits, bsum, pl.splits, (const __nv_bfloat16 *)w, vec3, b, mean, dw, dotpart, counters, db,
-                          dgamma, dbeta, ns, call_f16());
-    return launch_pdl(wgrad_epilogue_fused_kernel<2, 16, 1>, grid, dim3(1024), 0, st, pb.c_out, pb.kdim, partials,
-                      pl.splits, bsum, pl.splits, (const __nv_bfloat16 *)w, vec3, b, mean, dw, dotpart, counters, db,
-                      dgamma, dbeta, ns, call_f16());
+                                        const float *mean, float *dw, float *dotpart, float *db, float *dgamma, float *dbeta,
+                                        bool need_sums, cudaStream_t st) {
+    float *dots = vec3 && need_sums ? dotpart : nullptr;
+    cudaError_t e;
+    if (pl.kr == 32 && pl.splits <= 8) e = launch_add<32, 1>(pb, pl, partials, w, vec3, dw, dots, st);
+    else if (pl.kr == 32) e = launch_add<32, 2>(pb, pl, partials, w, vec3, dw, dots, st);
+    else if (pl.kr == 8) e = launch_add<8, 8>(pb, pl, partials, w, vec3, dw, dots, st);
+    else e = launch_add<2, 32>(pb, pl, partials, w, vec3, dw, dots, st);
+    if (e != cudaSuccess || !need_sums) return e;
+    static PerDevice carve;
+    prefer_max_shared_once(wgrad_finish_kernel, &carve);
+    return launch_pdl(wgrad_finish_kernel, dim3(pb.c_out / 32), dim3(1024), 0, st, pb.c_out, pl.kt, dotpart, pl.splits, bsum, vec3,
+                      b, mean, db, dgamma, dbeta);
 }
 
 // ---- small-C_in ("stem") layers -------------------------------------------------------------------
@@ -571,9 +515,9 @@ cudaError_t launch_stem_wgrad(const Problem &pb, const UmmaWgradPlan &pl, const 
     Problem q = pb;
     q.kdim = g.kdim;                                   // grid: (kh + 2) / 2 row tiles
     const int bn = wgrad_bn(pb);
-    if (bn == 64) return launch_w<64>(tx, tdz, g, pl, q, partials, bsum, nullptr, err, st);
-    if (bn == 128) return launch_w<128>(tx, tdz, g, pl, q, partials, bsum, nullptr, err, st);
-    return launch_w<256>(tx, tdz, g, pl, q, partials, bsum, nullptr, err, st);
+    if (bn == 64) return launch_w<64>(tx, tdz, g, pl, q, partials, bsum, err, st);
+    if (bn == 128) return launch_w<128>(tx, tdz, g, pl, q, partials, bsum, err, st);
+    return launch_w<256>(tx, tdz, g, pl, q, partials, bsum, err, st);
 }
 
 // One block per output channel: gathers the kh x kw x C_in real entries out of the krows x 64 padded rows,
