@@ -157,11 +157,9 @@ Plan make_plan(const convbn_desc *d, const Problem &pb, int phase) {
         size_t o = 0;
         auto put = [&](size_t bytes) { size_t r = o; o = align_up(o + bytes, 256); return r; };
         pl.uw.splits = fused_bwd1x1_ctas(pb);
-        wgrad_epilogue_shape(pb, &pl.uw);
         pl.bsplits = pl.uw.splits;
         pl.partials = put((size_t)pl.uw.splits * pb.c_out * pb.kdim * sizeof(float));
         pl.bsum = put((size_t)pl.uw.splits * pb.c_out * sizeof(float));
-        pl.dotpart = put((size_t)pl.uw.kt * pb.c_out * sizeof(float));
         pl.total = o;
         return pl;
     }
@@ -211,17 +209,15 @@ Plan make_plan(const convbn_desc *d, const Problem &pb, int phase) {
             pl.stem_win_wgrad = true;
             pl.uw = UmmaWgradPlan();
             pl.uw.splits = stem_window_wgrad_ctas(pb);
-            wgrad_epilogue_shape(pb, &pl.uw);
-            pl.bsplits = pl.uw.splits;
+                pl.bsplits = pl.uw.splits;
             part_bytes = wrows * pl.uw.splits * sizeof(float);
-            dot_bytes = (size_t)pl.uw.kt * pb.c_out * sizeof(float);
+            dot_bytes = (size_t)wgrad_kmajor_rows(pb) * pb.c_out * sizeof(float);
         }
     }
     if (pl.umma_wgrad) {
         pl.uw = umma_wgrad_plan(pb);
         pl.bsplits = pl.uw.splits;
         part_bytes = wrows * pl.uw.splits * sizeof(float);
-        dot_bytes = (size_t)pl.uw.kt * pb.c_out * sizeof(float);
     }
     switch (phase) {
         case CONVBN_PHASE_TUNE_FWD:
@@ -632,9 +628,7 @@ int run_param_grads(const convbn_desc *d, const Problem &pb, const Plan &pl, con
     if (pl.stem_win_wgrad) {
         float *dotpart = (float *)at(ws, pl.dotpart);
         LAUNCH("stem_wgrad", launch_stem_window_wgrad(pb, dz, x, partials, bsum, st));
-        LAUNCH("wgrad_epilogue_fused", launch_wgrad_epilogue_fused(pb, pl.uw, partials, bsum, w, vec3, b, mean, dw,
-                                                                   dotpart, db, dgamma, dbeta, need_bsum,
-                                                                   st));
+        LAUNCH("wgrad_rows", launch_wgrad_epilogue_kmajor(pb, pl.uw.splits, partials, bsum, w, vec3, b, mean, dw, dotpart, db, dgamma, dbeta, need_bsum, st));
         *which = "umma-stem";
     } else if (pl.stem) {
         LAUNCH("stem_pack", launch_stem_pack(pb, x, at(ws, pl.xpk), st));
@@ -654,11 +648,8 @@ int run_param_grads(const convbn_desc *d, const Problem &pb, const Plan &pl, con
                                                              dgamma, dbeta, st));
         *which = "grouped-umma";
     } else if (pl.umma_wgrad) {
-        float *dotpart = (float *)at(ws, pl.dotpart);
         LAUNCH("umma_wgrad", launch_umma_wgrad(pb, pl.uw, dz, x, partials, bsum, st));
-        LAUNCH("wgrad_epilogue_fused", launch_wgrad_epilogue_fused(pb, pl.uw, partials, bsum, w, vec3, b, mean, dw,
-                                                                   dotpart, db, dgamma, dbeta, need_bsum,
-                                                                   st));
+        LAUNCH("wgrad_rows", launch_wgrad_rows(pb, pl.uw.splits, partials, bsum, w, vec3, b, mean, dw, db, dgamma, dbeta, need_bsum, st));
         *which = "umma";
     } else if (pl.dw_tma_wgrad) {
         int nparts = 0;
@@ -969,7 +960,6 @@ static int tune_bwd_impl(const convbn_desc *desc, const void *dz, const void *x,
     }
     cudaStream_t st = (cudaStream_t)stream;
     float *partials = (float *)at(workspace, pl.partials), *bsum = (float *)at(workspace, pl.bsum);
-    float *dotpart = (float *)at(workspace, pl.dotpart);
     const float *vec3 = (const float *)saved;
     LAUNCH("umma_bwd", launch_fused_bwd1x1(pb, dz, x, w, vec3, dx, partials, bsum, st, &post));
     t_last_kernel[CONVBN_PHASE_TUNE_BWD] = "umma-fused-bwd";
@@ -980,13 +970,12 @@ static int tune_bwd_impl(const convbn_desc *desc, const void *dz, const void *x,
         CU(cudaEventRecord(lane->fork, st));
         CU(cudaStreamWaitEvent(lane->stream, lane->fork, 0));
         cudaStream_t st = lane->stream;
-        LAUNCH("wgrad_epilogue_fused", launch_wgrad_epilogue_fused(pb, pl.uw, partials, bsum, w, vec3, b, run_mean, dw,
-                                                                   dotpart, db, dgamma, dbeta, true, st));
+        LAUNCH("wgrad_rows", launch_wgrad_rows(pb, pl.uw.splits, partials, bsum, w, vec3, b, run_mean, dw, db, dgamma, dbeta, true, st));
         CU(cudaEventRecord(lane->join, lane->stream));
         lane->pending = true;
         return CONVBN_OK;
     }
-    LAUNCH("wgrad_epilogue_fused", launch_wgrad_epilogue_fused(pb, pl.uw, partials, bsum, w, vec3, b, run_mean, dw, dotpart, db, dgamma, dbeta, true, st));
+    LAUNCH("wgrad_rows", launch_wgrad_rows(pb, pl.uw.splits, partials, bsum, w, vec3, b, run_mean, dw, db, dgamma, dbeta, true, st));
     return CONVBN_OK;
 }
 
@@ -1108,11 +1097,9 @@ int convbn_eval_bwd(const convbn_desc *desc, const void *dz, const void *x, cons
                 if (fused) {
                     LAUNCH("umma_bwd", launch_fused_bwd1x1(pb, dz, x, w, vec3, dx, (float *)at(inner, pt.partials),
                                                            (float *)at(inner, pt.bsum), st));
-                    LAUNCH("wgrad_epilogue_fused",
-                           launch_wgrad_epilogue_fused(pb, pt.uw, (const float *)at(inner, pt.partials),
-                                                       (const float *)at(inner, pt.bsum), w, vec3, nullptr, run_mean, dw,
-                                                       (float *)at(inner, pt.dotpart),
-                                                       nullptr, nullptr, nullptr, false, st));
+                    LAUNCH("wgrad_rows",
+                           launch_wgrad_rows(pb, pt.uw.splits, (const float *)at(inner, pt.partials), (const float *)at(inner, pt.bsum),
+                                             w, vec3, nullptr, run_mean, dw, nullptr, nullptr, nullptr, false, st));
                     t_last_kernel[CONVBN_PHASE_EVAL_BWD] = "umma-fused-bwd";
                     return CONVBN_OK;
                 }

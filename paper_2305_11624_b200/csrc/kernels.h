@@ -132,12 +132,10 @@ cudaError_t launch_reparam_dgrad_class(const Problem &pb, const void *w, const f
 struct UmmaWgradPlan {
     int splits = 1;           // pixel slices = partial tiles
     long long per_split = 0;  // pixels per slice
-    int kt = 1;               // k ranges of the epilogue (rows of dotpart)
-    int kr = 8;               // k rows per block (32, 8 or 2)
 };
 bool umma_wgrad_eligible(const Problem &pb);
 UmmaWgradPlan umma_wgrad_plan(const Problem &pb);
-// partials: [splits][kdim][C_out] fp32 (k-major: the transpose of the weight layout)
+// partials: [splits][C_out][kdim] fp32 (the layout of the weights; block-diagonal: [splits][block][k][64])
 // bsum    : [splits][C_out] fp32 per-slice sums of dZ over pixels (from a ones row in the GEMM)
 // counters: `ncounters` words zeroed for an epilogue that counts its blocks (may be NULL)
 cudaError_t launch_umma_wgrad(const Problem &pb, const UmmaWgradPlan &pl, const void *dz, const void *x,
@@ -145,11 +143,15 @@ cudaError_t launch_umma_wgrad(const Problem &pb, const UmmaWgradPlan &pl, const 
                               int ncounters = 0);
 // Everything after the GEMM: dw[co][k] = scale[co] * sum_splits partials (scale = first
 // C_out floats of vec3, 1 if NULL); with need_sums also dbeta, db, dgamma (vec3 given) or db = sum dZ.
-// dotpart: [kt][C_out] scratch.
-cudaError_t launch_wgrad_epilogue_fused(const Problem &pb, const UmmaWgradPlan &pl, const float *partials,
-                                        const float *bsum, const void *w, const float *vec3, const float *b,
-                                        const float *mean, float *dw, float *dotpart, float *db, float *dgamma, float *dbeta,
-                                        bool need_sums, cudaStream_t st);
+cudaError_t launch_wgrad_rows(const Problem &pb, int splits, const float *partials, const float *bsum, const void *w,
+                              const float *vec3, const float *b, const float *mean, float *dw, float *db, float *dgamma,
+                              float *dbeta, bool need_sums, cudaStream_t st);
+// The same over k-major partials [splits][kdim][C_out] (C_out a multiple of 64); dotpart: [wgrad_kmajor_rows][C_out] scratch.
+int wgrad_kmajor_rows(const Problem &pb);
+cudaError_t launch_wgrad_epilogue_kmajor(const Problem &pb, int splits, const float *partials, const float *bsum,
+                                         const void *w, const float *vec3, const float *b, const float *mean, float *dw,
+                                         float *dotpart, float *db, float *dgamma, float *dbeta, bool need_sums,
+                                         cudaStream_t st);
 
 // ---- first-layer convolutions with C_in <= 8 (see stem_kernels.cu) -------------------------------
 bool stem_eligible(const Problem &pb);
@@ -184,8 +186,8 @@ bool stem_window_eligible(const Problem &pb);
 cudaError_t launch_stem_window_fwd(const Problem &pb, const void *x, const void *w, const float *bias, void *z,
                                    cudaStream_t st, const BnFold *fold = nullptr, int relu = 0);
 // Weight gradient of the same layers (C_in <= 3, C_out = 64) straight from X and dZ: one fp32 partial
-// [kdim][C_out] and one row of sums of dZ per CTA (stem_window_wgrad_ctas of them), in the layout the fused
-// epilogue of the dense weight-gradient path reads.
+// [kdim][C_out] and one row of sums of dZ per CTA (stem_window_wgrad_ctas of them), for
+// launch_wgrad_epilogue_kmajor.
 bool stem_window_wgrad_eligible(const Problem &pb);
 int stem_window_wgrad_ctas(const Problem &pb);
 cudaError_t launch_stem_window_wgrad(const Problem &pb, const void *dz, const void *x, float *partials, float *bsum,
@@ -195,8 +197,6 @@ cudaError_t launch_stem_window_wgrad(const Problem &pb, const void *dz, const vo
 bool stem_window_dgrad_eligible(const Problem &pb);
 cudaError_t launch_stem_window_dgrad(const Problem &pb, const void *dz, const void *w, const float *s_vec, void *dx,
                                      cudaStream_t st);
-// k rows per block (kr) and row blocks (kt) of the fused epilogue for pl.splits partial tiles
-void wgrad_epilogue_shape(const Problem &pb, UmmaWgradPlan *pl);
 cudaError_t launch_stem_fwd(const Problem &pb, const void *x_packed, const void *wst, const float *bias, void *out,
                             cudaStream_t st, const BnFold *fold = nullptr);
 
@@ -284,8 +284,8 @@ cudaError_t launch_bn_eval_finish(const Problem &pb, const float *part_g, const 
                                   float *dgamma, float *dbeta, cudaStream_t st);
 
 // ---- fused backward of 1x1 stride-1 layers (see umma_bwd1x1.cu) ----------------------------------------
-// dX plus one fp32 partial [C_in][C_out] and one row of sums of dZ per CTA (fused_bwd1x1_ctas of them), in the
-// layout the fused epilogue reads.  vec3 = saved [s | b' | r].
+// dX plus one fp32 partial [C_out][C_in] and one row of sums of dZ per CTA (fused_bwd1x1_ctas of them), for
+// launch_wgrad_rows.  vec3 = saved [s | b' | r].
 bool fused_bwd1x1_eligible(const Problem &pb);
 int fused_bwd1x1_ctas(const Problem &pb);
 cudaError_t launch_fused_bwd1x1(const Problem &pb, const void *dz, const void *x, const void *w, const float *vec3,
@@ -307,7 +307,7 @@ cudaError_t launch_tconv_rescale(int dtype, bool nhwc, long long count, int taps
                                  const float *s, void *w_out, cudaStream_t st);
 cudaError_t launch_tconv_bias(int dtype, bool nhwc, long long count, int c, long long hw, const float *bias, void *z,
                               cudaStream_t st);
-// The same from the weight-gradient GEMM's partial tiles [splits][taps C_out][C_in] (groups = 1, NHWC, channels multiples
+// The same from the weight-gradient GEMM's partial tiles [splits][C_in][taps C_out] (groups = 1, NHWC, channels multiples
 // of 64): adds them, transposes, scales and finishes the per-channel gradients in one kernel.  dotpart: [C_in / 32][taps
 // C_out] scratch, counters: C_out / 32 zeroed words, bsum: [bsplits][C_out].
 cudaError_t launch_tconv_wgrad_epilogue(int c_in, int c_out, int taps, const float *part, int splits, const void *w,

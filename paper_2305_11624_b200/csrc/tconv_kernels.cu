@@ -94,11 +94,11 @@ __global__ void __launch_bounds__(256) tconv_param_epilogue_kernel(int c_out, in
     }
 }
 
-// Block (bx, by): input channels [32 bx, +32) x weight rows k = (tap, co) [32 by, +32), one output channel group since
-// 32 divides C_out.  Thread (tx = ci, ty = k) adds its element over the slices, eight loads in flight, in slice order;
-// the tile is transposed through shared memory, scaled by s[co] and stored along k.  The last block of a group of 32
+// Block (bx, by): input channels [32 bx, +32) x weight columns k = (tap, co) [32 by, +32), one output channel group since
+// 32 divides C_out.  Thread (tx = k, ty = ci) adds its element of part[split][C_in][k] over the slices, eight loads in
+// flight, in slice order, scales it by s[co] and stores it.  The last block of a group of 32
 // output channels (a counter) adds the dot products and the sums of dZ in fixed order.  Bound by the read of the
-// partials (L2): 256 -> 128 channels, 2 x 2, 29 slices: 15 MB; with the transposition, the scale and the per-channel
+// partials (L2): 256 -> 128 channels, 2 x 2, 29 slices: 15 MB; with the sum, the scale and the per-channel
 // sums in kernels of their own the same work took 87 us.
 __global__ void __launch_bounds__(1024) tconv_wgrad_epilogue_kernel(int c_in, int c_out, int kdim, const float *__restrict__ part,
                                                                     int splits, const __nv_bfloat16 *__restrict__ w,
@@ -115,21 +115,16 @@ __global__ void __launch_bounds__(1024) tconv_wgrad_epilogue_kernel(int c_in, in
     const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
     const int ci0 = blockIdx.x * 32, k0 = blockIdx.y * 32, co0 = k0 % c_out;
     const float wv = load_h16(w + (size_t)(ci0 + ty) * kdim + k0 + tx, f16);
-    {
-        const float *src = part + (size_t)(k0 + ty) * c_in + ci0 + tx;
-        const size_t slice = (size_t)kdim * c_in;
-        float acc = 0.f;
-        for (int sp = 0; sp < splits; sp += 8) {
-            float v[8];
+    const float *src = part + (size_t)(ci0 + ty) * kdim + k0 + tx;
+    const size_t slice = (size_t)kdim * c_in;
+    float v = 0.f;
+    for (int sp = 0; sp < splits; sp += 8) {
+        float q[8];
 #pragma unroll
-            for (int u = 0; u < 8; ++u) v[u] = sp + u < splits ? __ldcg(src + (size_t)(sp + u) * slice) : 0.f;
+        for (int u = 0; u < 8; ++u) q[u] = sp + u < splits ? __ldcg(src + (size_t)(sp + u) * slice) : 0.f;
 #pragma unroll
-            for (int u = 0; u < 8; ++u) acc += v[u];
-        }
-        tile[ty][tx] = acc;
+        for (int u = 0; u < 8; ++u) v += q[u];
     }
-    __syncthreads();
-    const float v = tile[tx][ty];                       // (ci = ty, k = tx) from here on
     dw[(size_t)(ci0 + ty) * kdim + k0 + tx] = vec3[co0 + tx] * v;
     prod[ty][tx] = v * wv;
     __syncthreads();

@@ -282,22 +282,22 @@ __global__ void __launch_bounds__(kFbThreads) fused_bwd1x1_kernel(const __grid_c
             }
         }
         if (lane == 0) tma_store_wait_all<0>();
-        // ---- the CTA's partial of domega' as part[cta][k = ci][co] and its row of sums of dZ ----
+        // ---- the CTA's partial of domega' as part[cta][co][ci] and its row of sums of dZ: 128 contiguous bytes per store ----
         if (ok) ok = __all_sync(0xffffffffu, mbar_wait_bounded(&ctl->acc_done, 0, abort_flag));
         if (ok) {
             tc_fence_after_sync();
             float *part = partials + (size_t)blockIdx.x * CI * CO;
             if (S::kWideIn) {
-                // accumulator row = ci (M block mb, lane), columns = co: each thread owns one k row of 64 floats
+                // accumulator row = ci (M block mb, lane), columns = co
                 for (int mb = egroup; mb < S::kMBlocks; mb += 2) {
-                    float *orow = part + (size_t)(mb * 128 + quarter * 32 + lane) * CO;
+                    float *ocol = part + mb * 128 + quarter * 32 + lane;
 #pragma unroll 1
                     for (int c0 = 0; c0 < CO; c0 += 32) {
                         uint32_t v[32];
                         tmem_ld_32x32(tmem_base + (uint32_t)(S::kDwCol0 + mb * CO + c0) + lane_sel, v);
                         tmem_ld_wait();
 #pragma unroll
-                        for (int j = 0; j < 32; j += 4) *(uint4 *)(orow + c0 + j) = make_uint4(v[j], v[j + 1], v[j + 2], v[j + 3]);
+                        for (int j = 0; j < 32; ++j) ocol[(size_t)(c0 + j) * CI] = __uint_as_float(v[j]);
                     }
                 }
                 if (warp == 2) {                               // every row of the sums tile is sum dZ: take this warp's first
@@ -314,22 +314,28 @@ __global__ void __launch_bounds__(kFbThreads) fused_bwd1x1_kernel(const __grid_c
                     }
                 }
             } else {
-                // accumulator row = co, columns = ci (64): part[ci][co] is the transpose; 32 consecutive co per ci
-                // row are written together (128 bytes), lane = co
+                // accumulator row = co, columns = ci (64): 32 x 32 blocks are transposed in the warp's staging buffer (word
+                // (row, column) at row 32 + (column ^ row): no bank conflicts either way), then lane = ci
+                uint32_t *tr = (uint32_t *)buf_s;
                 for (int mb = egroup; mb < S::kMBlocks; mb += 2) {
-                    const int co = mb * 128 + quarter * 32 + lane;
+                    const int co0 = mb * 128 + quarter * 32;
 #pragma unroll 1
                     for (int c0 = 0; c0 < CI; c0 += 32) {
                         uint32_t v[32];
                         tmem_ld_32x32(tmem_base + (uint32_t)(S::kDwCol0 + mb * CI + c0) + lane_sel, v);
                         tmem_ld_wait();
+                        __syncwarp();
 #pragma unroll
-                        for (int j = 0; j < 32; ++j) part[(size_t)(c0 + j) * CO + co] = __uint_as_float(v[j]);
+                        for (int j = 0; j < 32; ++j) tr[lane * 32 + (j ^ lane)] = v[j];
+                        __syncwarp();
+#pragma unroll
+                        for (int r = 0; r < 32; ++r)
+                            part[(size_t)(co0 + r) * CI + c0 + lane] = __uint_as_float(tr[r * 32 + (lane ^ r)]);
                     }
                     uint32_t sv[16];
                     tmem_ld_32x16(tmem_base + (uint32_t)(S::kSumCol0 + mb * 16) + lane_sel, sv);
                     tmem_ld_wait();
-                    bsum[(size_t)blockIdx.x * CO + co] = __uint_as_float(sv[0]);
+                    bsum[(size_t)blockIdx.x * CO + co0 + lane] = __uint_as_float(sv[0]);
                 }
             }
         }

@@ -6,7 +6,7 @@
 // tiles: the A tile is two [64 pixels][64 channels] im2col loads of X (two consecutive 64-wide slices
 // of k), the B tile is BN/64 plain [64 pixels][64 channels] boxes of dZ.  The pixel range is cut into
 // `splits` slices (grid.z); every CTA accumulates its slice in tensor memory in fp32 and writes one
-// fp32 partial tile part[split][k][co].  A second kernel adds the slices in fixed order and forms
+// fp32 partial tile, in the weights' layout part[split][co][k].  A second kernel adds the slices in fixed order and forms
 // domega, dgamma, ... from the fp32 sums (never from rounded values).
 #include "kernels.h"
 #include "sm100_ptx.cuh"
@@ -35,6 +35,7 @@ struct WgradGemm {
     int stem, stem_tiles_w, stem_tiles_h;
     int no_ones;            // 1: no slice of ones (the packed stem input carries a constant-1 slot instead)
     int f16;                // 16-bit storage type: 0 bf16, 1 IEEE half
+    int rows;               // 1: partials are [split][C_out][kdim], 0: [split][k][C_out]
 };
 
 struct WgradSmemCtl {
@@ -207,7 +208,12 @@ __global__ void __launch_bounds__(kWThreads) umma_wgrad_kernel(const __grid_cons
                 uint32_t v[32];
                 tmem_ld_32x32(tmem_base + ((uint32_t)(quarter * 32) << 16) + (uint32_t)c0, v);
                 tmem_ld_wait();
-                if (row_ok) {
+                if (row_ok && g.rows) {
+                    // lanes are consecutive k: each store is 128 contiguous bytes of a weight row
+                    float *wrow = partials + ((size_t)blockIdx.z * g.c_out + n0 + c0) * g.kdim + k;
+#pragma unroll
+                    for (int j = 0; j < 32; ++j) wrow[(size_t)j * g.kdim] = __uint_as_float(v[j]);
+                } else if (row_ok) {
 #pragma unroll
                     for (int j = 0; j < 32; j += 4)
                         *(uint4 *)(orow + c0 + j) = make_uint4(v[j], v[j + 1], v[j + 2], v[j + 3]);
@@ -269,19 +275,10 @@ UmmaWgradPlan umma_wgrad_plan(const Problem &pb) {
     per = (per + kWP - 1) / kWP * kWP;
     pl.per_split = per;
     pl.splits = (int)((pb.p + per - 1) / per);
-    wgrad_epilogue_shape(pb, &pl);
     return pl;
 }
 
-// k rows per block of wgrad_add_kernel (its other threads split the slices): as many as leave about 100 blocks and one
-// batch of eight loads per thread, 32 rows (1 or 2 slice groups), 8 (8 groups) or 2 (32 groups)
-void wgrad_epilogue_shape(const Problem &pb, UmmaWgradPlan *pl) {
-    const long long cols = pb.c_out / 64;
-    if (pl->splits <= 16 && cols * ((pb.kdim + 31) / 32) >= 96) pl->kr = 32;
-    else if (pl->splits <= 64 && cols * ((pb.kdim + 7) / 8) >= 48) pl->kr = 8;
-    else pl->kr = 2;
-    pl->kt = (pb.kdim + pl->kr - 1) / pl->kr;   // blocks along k = rows of dotpart
-}
+int wgrad_kmajor_rows(const Problem &pb) { return (pb.kdim + 1) / 2; }
 
 template <int BN>
 static cudaError_t launch_w(const CUtensorMap &tx, const CUtensorMap &tdz, WgradGemm g, const UmmaWgradPlan &pl,
@@ -312,6 +309,7 @@ cudaError_t launch_umma_wgrad(const Problem &pb, const UmmaWgradPlan &pl, const 
     g.lower_h = -pb.pad_h; g.lower_w = -pb.pad_w; g.stride_h = pb.stride_h; g.stride_w = pb.stride_w;
     g.dil_h = pb.dil_h; g.dil_w = pb.dil_w; g.kdim = pb.kdim; g.p = pb.p; g.per_split = pl.per_split; g.stages = 1;
     g.blockdiag = pb.groups > 1 ? 1 : 0;
+    g.rows = g.blockdiag ? 0 : 1;
     g.stem = 0; g.stem_tiles_w = g.stem_tiles_h = 1; g.no_ones = 0; g.f16 = call_f16();
     if (g.blockdiag) { g.c_in = 64; g.kdim = pb.kh * pb.kw * 64; }
     const int upper_h = g.lower_h + (pb.h_out - 1) * pb.stride_h - (pb.h_in - 1);
@@ -330,19 +328,111 @@ cudaError_t launch_umma_wgrad(const Problem &pb, const UmmaWgradPlan &pl, const 
     return launch_w<256>(tx, tdz, g, pl, pb, partials, bsum, err, st, counters, ncounters);
 }
 
-// ---- epilogue over k-major partials ------------------------------------------------------------
-// Two kernels finish every parameter gradient (Table 2, Tune row) from the fp32 partial tiles part[split][k][co].
+// ---- epilogue over partial weight tensors -----------------------------------------------------------
+// part[split][C_out][kdim] fp32, the layout of the weights.  One block per output channel finishes everything that
+// belongs to it (Table 2, Tune row):
+//     acc[k] = sum_split part[split][co][k]
+//     domega = s acc,   dbeta = sum_split bsum,   db = s dbeta,   dgamma = r (sum_k acc omega + dbeta (b - mu_hat)).
+// Plain mode (vec3 == NULL): domega = acc, db = sum dZ if requested; need_sums = 0: domega alone.
+// Threads: VL along k (a float4 each, so that reads and stores are whole lines) x SL groups of slices, added in order
+// through shared memory; a thread requests up to eight slices before it uses the first.  Bound by those reads (9 to 19 MB
+// from L2).  With k-major partial tiles the GEMM's stores were 16 bytes per lane in 32 lines, this kernel had to transpose,
+// and the per-channel sums needed a counter or a second kernel: weight phases of 17 to 36 us became RESULTS.
+__global__ void __launch_bounds__(1024) wgrad_rows_kernel(int c_out, int kdim, int VL, int SL, const float *__restrict__ part,
+                                                          int splits, const float *__restrict__ bsum,
+                                                          const __nv_bfloat16 *__restrict__ w, const float *__restrict__ vec3,
+                                                          const float *__restrict__ b, const float *__restrict__ mean,
+                                                          float *__restrict__ dw, float *__restrict__ db,
+                                                          float *__restrict__ dgamma, float *__restrict__ dbeta, int need_sums,
+                                                          int f16) {
+    __shared__ float4 red[1024];
+    __shared__ float fin[2][32];
+    pdl_wait();
+    pdl_launch_dependents();
+    const int co = blockIdx.x, l = threadIdx.x % VL, z = threadIdx.x / VL;
+    const float s = vec3 ? vec3[co] : 1.f;
+    const size_t slice = (size_t)c_out * kdim, row = (size_t)co * kdim;
+    float dot = 0.f, ds = 0.f;
+    if (need_sums)
+        for (int sp = threadIdx.x; sp < splits; sp += blockDim.x) ds += __ldcg(bsum + (size_t)sp * c_out + co);
+    for (int k0 = 0; k0 < kdim; k0 += 4 * VL) {
+        const int k = k0 + 4 * l;
+        uint2 wq = make_uint2(0u, 0u);
+        if (vec3 && need_sums && z == 0 && k < kdim) wq = *(const uint2 *)(w + row + k);
+        float4 a = make_float4(0.f, 0.f, 0.f, 0.f);
+        if (k < kdim) {
+            const float *src = part + row + k;
+            for (int sp = z; sp < splits; sp += 8 * SL) {
+                float4 v[8];
+#pragma unroll
+                for (int u = 0; u < 8; ++u)
+                    v[u] = sp + u * SL < splits ? __ldcg((const float4 *)(src + (size_t)(sp + u * SL) * slice))
+                                                : make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+                for (int u = 0; u < 8; ++u) { a.x += v[u].x; a.y += v[u].y; a.z += v[u].z; a.w += v[u].w; }
+            }
+        }
+        if (SL > 1) {
+            if (k0) __syncthreads();
+            red[threadIdx.x] = a;
+            // groups z and z + h in halves: log2(SL) short steps
+            for (int h = SL / 2; h > 0; h /= 2) {
+                __syncthreads();
+                if (z < h) {
+                    const float4 o = red[threadIdx.x + h * VL];
+                    a.x += o.x; a.y += o.y; a.z += o.z; a.w += o.w;
+                    red[threadIdx.x] = a;
+                }
+            }
+        }
+        if (z == 0 && k < kdim) {
+            *(float4 *)(dw + row + k) = make_float4(s * a.x, s * a.y, s * a.z, s * a.w);
+            dot = fmaf(a.x, unpack_h16((uint16_t)(wq.x & 0xFFFFu), f16), dot);
+            dot = fmaf(a.y, unpack_h16((uint16_t)(wq.x >> 16), f16), dot);
+            dot = fmaf(a.z, unpack_h16((uint16_t)(wq.y & 0xFFFFu), f16), dot);
+            dot = fmaf(a.w, unpack_h16((uint16_t)(wq.y >> 16), f16), dot);
+        }
+    }
+    if (!need_sums) return;
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) { dot += __shfl_xor_sync(0xffffffffu, dot, o); ds += __shfl_xor_sync(0xffffffffu, ds, o); }
+    if (threadIdx.x % 32 == 0) { fin[0][threadIdx.x / 32] = dot; fin[1][threadIdx.x / 32] = ds; }
+    __syncthreads();
+    if (threadIdx.x) return;
+    dot = ds = 0.f;
+    for (int i = 0; i < (int)blockDim.x / 32; ++i) { dot += fin[0][i]; ds += fin[1][i]; }
+    if (!vec3) {
+        if (db) db[co] = ds;
+        return;
+    }
+    dbeta[co] = ds;
+    if (db) db[co] = s * ds;
+    dgamma[co] = vec3[2 * c_out + co] * (dot + ds * ((b ? b[co] : 0.f) - mean[co]));
+}
+
+// kdim: a multiple of 4 (rows of the weight tensor start on 16-byte boundaries)
+cudaError_t launch_wgrad_rows(const Problem &pb, int splits, const float *partials, const float *bsum, const void *w,
+                              const float *vec3, const float *b, const float *mean, float *dw, float *db, float *dgamma,
+                              float *dbeta, bool need_sums, cudaStream_t st) {
+    // slice groups so that a thread adds at most eight slices, then as many threads along the row as are left
+    int SL = 1, VL = 16;
+    while (SL < 32 && SL * 8 < splits) SL *= 2;
+    while (VL * 4 < pb.kdim && VL * SL < 1024) VL *= 2;
+    while (VL * SL < 32) VL *= 2;
+    static PerDevice carve;
+    prefer_max_shared_once(wgrad_rows_kernel, &carve);
+    return launch_pdl(wgrad_rows_kernel, dim3(pb.c_out), dim3(VL * SL), 0, st, pb.c_out, pb.kdim, VL, SL, partials, splits, bsum,
+                      (const __nv_bfloat16 *)w, vec3, b, mean, dw, db, dgamma, dbeta, need_sums ? 1 : 0, call_f16());
+}
+
+// ---- epilogue over k-major partials (the stem's weight gradient) --------------------------------------
+// part[split][k][C_out]: the stem's accumulators hold an output channel per lane.  Two kernels:
 //
 // wgrad_add_kernel: block = 64 output channels x KR weight rows k.  Thread (float4 of channels, k, slice group z < SL)
 // adds slices z, z + SL, ..., eight loads in flight, then the groups are added in order through shared memory and
 //     dw[co][k] = s[co] acc,    dotpart[k block][co] = sum over the block's k of acc w[co][k].
 // wgrad_finish_kernel: dbeta = sum dZ,  db = s dbeta,  dgamma = r (sum_k domega' omega + dbeta (b - mu_hat)).
-// Plain mode (vec3 == NULL): dw = acc, db = sum dZ if requested.
-//
-// Bound by the latency of the L2 reads (9 to 19 MB of partials): with (KR, SL) chosen so that a thread's loads are one
-// batch, a block is one round trip.  As one kernel whose last block per channel group did the finish (a fence, an atomic
-// and two more dependent reads behind every block) it took 10 us on the 3x3 64 -> 64 layer at 56 x 56, N = 32, and 16 us on
-// 3x3 512 -> 512 at 7 x 7, N = 64.
+// Plain mode (vec3 == NULL): dw = acc, db = sum dZ if requested.  Bound by the latency of the L2 reads (5.5 MB).
 template <int KR, int SL>
 __global__ void __launch_bounds__(KR * 16 * SL) wgrad_add_kernel(int c_out, int kdim, const float *__restrict__ part, int splits,
                                                                 const __nv_bfloat16 *__restrict__ w,
@@ -436,30 +526,19 @@ __global__ void __launch_bounds__(1024) wgrad_finish_kernel(int c_out, int rows,
     dgamma[co] = vec3[2 * c_out + co] * (d + dsum * ((b ? b[co] : 0.f) - mean[co]));
 }
 
-template <int KR, int SL>
-static cudaError_t launch_add(const Problem &pb, const UmmaWgradPlan &pl, const float *partials, const void *w, const float *vec3,
-                              float *dw, float *dotpart, cudaStream_t st) {
-    static PerDevice carve;
-    prefer_max_shared_once(wgrad_add_kernel<KR, SL>, &carve);
-    return launch_pdl(wgrad_add_kernel<KR, SL>, dim3(pb.c_out / 64, pl.kt), dim3(KR * 16 * SL), 0, st, pb.c_out, pb.kdim, partials,
-                      pl.splits, (const __nv_bfloat16 *)w, vec3, dw, dotpart, call_f16());
-}
-
-cudaError_t launch_wgrad_epilogue_fused(const Problem &pb, const UmmaWgradPlan &pl, const float *partials,
-                                        const float *bsum, const void *w, const float *vec3, const float *b,
-                                        const float *mean, float *dw, float *dotpart, float *db, float *dgamma, float *dbeta,
-                                        bool need_sums, cudaStream_t st) {
-    float *dots = vec3 && need_sums ? dotpart : nullptr;
-    cudaError_t e;
-    if (pl.kr == 32 && pl.splits <= 8) e = launch_add<32, 1>(pb, pl, partials, w, vec3, dw, dots, st);
-    else if (pl.kr == 32) e = launch_add<32, 2>(pb, pl, partials, w, vec3, dw, dots, st);
-    else if (pl.kr == 8) e = launch_add<8, 8>(pb, pl, partials, w, vec3, dw, dots, st);
-    else e = launch_add<2, 32>(pb, pl, partials, w, vec3, dw, dots, st);
+cudaError_t launch_wgrad_epilogue_kmajor(const Problem &pb, int splits, const float *partials, const float *bsum,
+                                         const void *w, const float *vec3, const float *b, const float *mean, float *dw,
+                                         float *dotpart, float *db, float *dgamma, float *dbeta, bool need_sums,
+                                         cudaStream_t st) {
+    const int rows = wgrad_kmajor_rows(pb);
+    static PerDevice carve_a, carve_f;
+    prefer_max_shared_once(wgrad_add_kernel<2, 32>, &carve_a);
+    cudaError_t e = launch_pdl(wgrad_add_kernel<2, 32>, dim3(pb.c_out / 64, rows), dim3(1024), 0, st, pb.c_out, pb.kdim, partials,
+                               splits, (const __nv_bfloat16 *)w, vec3, dw, vec3 && need_sums ? dotpart : nullptr, call_f16());
     if (e != cudaSuccess || !need_sums) return e;
-    static PerDevice carve;
-    prefer_max_shared_once(wgrad_finish_kernel, &carve);
-    return launch_pdl(wgrad_finish_kernel, dim3(pb.c_out / 32), dim3(1024), 0, st, pb.c_out, pl.kt, dotpart, pl.splits, bsum, vec3,
-                      b, mean, db, dgamma, dbeta);
+    prefer_max_shared_once(wgrad_finish_kernel, &carve_f);
+    return launch_pdl(wgrad_finish_kernel, dim3(pb.c_out / 32), dim3(1024), 0, st, pb.c_out, rows, dotpart, splits, bsum, vec3, b,
+                      mean, db, dgamma, dbeta);
 }
 
 // ---- small-C_in ("stem") layers -------------------------------------------------------------------
@@ -474,7 +553,6 @@ UmmaWgradPlan stem_wgrad_plan(const Problem &pb) {
     const long long per = (patches + splits - 1) / splits;
     pl.per_split = per * kWP;                       // in pixels of 4 x 16 patches
     pl.splits = (int)((patches + per - 1) / per);
-    pl.kr = 8; pl.kt = 1;
     return pl;
 }
 
@@ -486,6 +564,7 @@ cudaError_t launch_stem_wgrad(const Problem &pb, const UmmaWgradPlan &pl, const 
     g.ho = pb.h_out; g.wo = pb.w_out; g.c_in = 64; g.c_out = pb.c_out; g.taps_w = 1;
     g.lower_h = g.lower_w = 0; g.stride_h = g.stride_w = g.dil_h = g.dil_w = 1;
     g.kdim = krows * 64;
+    g.rows = 0;
     g.stem = 1; g.stem_tiles_w = (pb.w_out + 15) / 16; g.stem_tiles_h = (pb.h_out + 3) / 4;
     g.no_ones = stem_ones_in_pack(pb) ? 1 : 0;
     g.f16 = call_f16();
