@@ -248,7 +248,9 @@ bool umma_wgrad_eligible(const Problem &pb) {
     return true;
 }
 
-static int wgrad_bn(const Problem &pb) { return pb.c_out >= 256 ? 256 : (pb.c_out >= 128 ? 128 : 64); }
+// (256-wide tiles, one CTA per SM, measured 0 to 5 % slower than two 128-wide ones; the packed stem still uses them)
+static int wgrad_bn(const Problem &pb) { return pb.c_out >= 128 ? 128 : 64; }
+static int stem_wgrad_bn(const Problem &pb) { return pb.c_out >= 256 ? 256 : wgrad_bn(pb); }
 
 UmmaWgradPlan umma_wgrad_plan(const Problem &pb) {
     UmmaWgradPlan pl;
@@ -256,12 +258,12 @@ UmmaWgradPlan umma_wgrad_plan(const Problem &pb) {
     const int bn = bd ? 64 : wgrad_bn(pb);
     const long long kd = bd ? (long long)pb.kh * pb.kw * 64 : pb.kdim;
     const long long m_tiles = (kd / 64 + 1 + 1) / 2, n_tiles = (pb.c_out + bn - 1) / bn;   // + the ones slice
-    // Resident CTAs: the 64- and 128-wide tiles run two CTAs per SM (their stage rings are sized for it,
-    // launch_w), which measured 25-40 % faster than one CTA with a deeper ring; 256-wide tiles own an SM.
+    // Resident CTAs: two per SM (the stage rings are sized for it, launch_w), which measured 25-40 % faster than one
+    // CTA with a deeper ring.
     // The slice count minimises  rounds over the resident slots x (pixels per slice + a fixed cost per
     // CTA, in pixels) + a small cost per slice for the epilogue that adds the slices up; a grid a few
     // CTAs larger than the slots would otherwise run a second, nearly empty round.
-    const long long slots = (long long)device_sm_count() * (bn == 256 ? 1 : 2), tiles = m_tiles * n_tiles;
+    const long long slots = (long long)device_sm_count() * 2, tiles = m_tiles * n_tiles;
     const long long max_splits = (pb.p + 4 * kWP - 1) / (4 * kWP);     // at least 256 pixels per slice
     long long splits = 1;
     double best_cost = -1.0;
@@ -324,8 +326,7 @@ cudaError_t launch_umma_wgrad(const Problem &pb, const UmmaWgradPlan &pl, const 
     if (e != cudaSuccess) return e;
     const int bn = g.blockdiag ? 64 : wgrad_bn(pb);
     if (bn == 64) return launch_w<64>(tx, tdz, g, pl, pb, partials, bsum, err, st, counters, ncounters);
-    if (bn == 128) return launch_w<128>(tx, tdz, g, pl, pb, partials, bsum, err, st, counters, ncounters);
-    return launch_w<256>(tx, tdz, g, pl, pb, partials, bsum, err, st, counters, ncounters);
+    return launch_w<128>(tx, tdz, g, pl, pb, partials, bsum, err, st, counters, ncounters);
 }
 
 // ---- epilogue over partial weight tensors -----------------------------------------------------------
@@ -337,7 +338,8 @@ cudaError_t launch_umma_wgrad(const Problem &pb, const UmmaWgradPlan &pl, const 
 // Threads: VL along k (a float4 each, so that reads and stores are whole lines) x SL groups of slices, added in order
 // through shared memory; a thread requests up to eight slices before it uses the first.  Bound by those reads (9 to 19 MB
 // from L2).  With k-major partial tiles the GEMM's stores were 16 bytes per lane in 32 lines, this kernel had to transpose,
-// and the per-channel sums needed a counter or a second kernel: weight phases of 17 to 36 us became RESULTS.
+// and the per-channel sums needed a counter or a second kernel.  Weight phase (GEMM + this), graph replay, N = 32: 1x1
+// 512 -> 128 at 28 x 28 20.3 -> 12.0 us, 3x3 256 at 14 x 14 22.8 -> 17.2, 3x3 512 at 7 x 7 30.0 -> 22.8.
 __global__ void __launch_bounds__(1024) wgrad_rows_kernel(int c_out, int kdim, int VL, int SL, const float *__restrict__ part,
                                                           int splits, const float *__restrict__ bsum,
                                                           const __nv_bfloat16 *__restrict__ w, const float *__restrict__ vec3,
@@ -544,7 +546,7 @@ cudaError_t launch_wgrad_epilogue_kmajor(const Problem &pb, int splits, const fl
 // ---- small-C_in ("stem") layers -------------------------------------------------------------------
 UmmaWgradPlan stem_wgrad_plan(const Problem &pb) {
     UmmaWgradPlan pl;
-    const int bn = wgrad_bn(pb);
+    const int bn = stem_wgrad_bn(pb);
     const long long patches = (long long)pb.n * ((pb.h_out + 3) / 4) * ((pb.w_out + 15) / 16);
     const long long m_tiles = (stem_krows(pb) + (stem_ones_in_pack(pb) ? 1 : 2)) / 2, n_tiles = (pb.c_out + bn - 1) / bn;
     long long splits = (device_sm_count() + m_tiles * n_tiles - 1) / (m_tiles * n_tiles);
@@ -593,7 +595,7 @@ cudaError_t launch_stem_wgrad(const Problem &pb, const UmmaWgradPlan &pl, const 
     if (e != cudaSuccess) return e;
     Problem q = pb;
     q.kdim = g.kdim;                                   // grid: (kh + 2) / 2 row tiles
-    const int bn = wgrad_bn(pb);
+    const int bn = stem_wgrad_bn(pb);
     if (bn == 64) return launch_w<64>(tx, tdz, g, pl, q, partials, bsum, err, st);
     if (bn == 128) return launch_w<128>(tx, tdz, g, pl, q, partials, bsum, err, st);
     return launch_w<256>(tx, tdz, g, pl, q, partials, bsum, err, st);
