@@ -887,6 +887,18 @@ int side_lane(SideLane **out) {
     return CONVBN_OK;
 }
 
+// Which of the two passes of a joined backward call stays on the caller's stream.  The lane's first kernel starts one event
+// later and the caller's stream resumes one event after the lane's last, a few us each, so the longer pass belongs on the
+// caller's stream: the parameter gradients (GEMM and epilogue), 59 -> 55 us per forward + backward of a 3x3 64 -> 64 layer at
+// 56 x 56, N = 32, 68 -> 65 at 3x3 stride 2 128 -> 128, 200 x 334.  With a million weights, or where it is a GEMM per
+// parity class, the data pass is the longer one: 3x3 512 -> 512 at 7 x 7, N = 64
+// takes 79 us this way and 87 the other, 3x3 stride 2 256 -> 256 at 28 x 28 57 and 60.
+bool data_pass_first(const convbn_desc *d, const Problem &pb) {
+    UmmaConvShape s;
+    const bool classes = strided_dgrad_ok(d, pb) && !(subpixel_wide_shape(pb, &s) && umma_strip_eligible(s));
+    return pb.groups == 1 && ((long long)pb.c_out * pb.kdim >= (1LL << 20) || classes);
+}
+
 // `side(lane stream)` and `main_pass()` side by side, the caller's stream joined to the lane before return.
 // Under the profiler (per-kernel event pairs on one stream) they run one after the other.
 template <class Side, class Main>
@@ -943,6 +955,13 @@ static int tune_bwd_impl(const convbn_desc *desc, const void *dz, const void *x,
             CK(tune_bwd_data_impl(desc, dz, w, saved, dx, post, workspace, bytes_d, stream));
             return convbn_tune_bwd_weight(desc, dz, x, w, b, run_mean, saved, dw, db, dgamma, dbeta, ws_w, bytes_w, stream);
         }
+        if (!defer_join && !data_pass_first(desc, pb))
+            return side_by_side(
+                (cudaStream_t)stream,
+                [&](cudaStream_t lane) { return tune_bwd_data_impl(desc, dz, w, saved, dx, post, workspace, bytes_d, lane); },
+                [&]() {
+                    return convbn_tune_bwd_weight(desc, dz, x, w, b, run_mean, saved, dw, db, dgamma, dbeta, ws_w, bytes_w, stream);
+                });
         SideLane *lane = nullptr;
         CK(side_lane(&lane));
         cudaStream_t st = (cudaStream_t)stream;
