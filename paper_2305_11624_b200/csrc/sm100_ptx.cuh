@@ -33,6 +33,10 @@ __device__ __forceinline__ uint32_t smem_u32(const void *p) {
     return (uint32_t)__cvta_generic_to_shared(p);
 }
 
+// Barriers and tiles may be named by their 32-bit shared-memory addresses: loops that step through a ring then do one
+// addition per slot instead of 64-bit address arithmetic and a conversion.
+__device__ __forceinline__ uint32_t smem_u32(uint32_t a) { return a; }
+
 __device__ __forceinline__ uint64_t globaltimer_ns() {
     uint64_t t;
     asm volatile("mov.u64 %0, %globaltimer;" : "=l"(t));
@@ -55,14 +59,17 @@ __device__ __forceinline__ void fence_barrier_init() {
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
 }
-__device__ __forceinline__ void mbar_arrive_expect_tx(uint64_t *bar, uint32_t bytes) {
+template <class Bar>
+__device__ __forceinline__ void mbar_arrive_expect_tx(Bar bar, uint32_t bytes) {
     asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(smem_u32(bar)), "r"(bytes)
                  : "memory");
 }
-__device__ __forceinline__ void mbar_arrive(uint64_t *bar) {
+template <class Bar>
+__device__ __forceinline__ void mbar_arrive(Bar bar) {
     asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(bar)) : "memory");
 }
-__device__ __forceinline__ bool mbar_try_wait(uint64_t *bar, uint32_t parity) {
+template <class Bar>
+__device__ __forceinline__ bool mbar_try_wait(Bar bar, uint32_t parity) {
     uint32_t ok;
     asm volatile(
         "{\n\t.reg .pred p;\n\tmbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\tselp.u32 %0, 1, 0, p;\n\t}"
@@ -75,7 +82,8 @@ __device__ __forceinline__ bool mbar_try_wait(uint64_t *bar, uint32_t parity) {
 // Waits for the phase with the given parity to complete, for at most `limit_ns` nanoseconds, and
 // gives up early when *abort_flag (shared memory, may be NULL) is set by another role.  Returns false on
 // give-up; the caller records the error and leaves its loop.
-__device__ __forceinline__ bool mbar_wait_bounded(uint64_t *bar, uint32_t parity, volatile int *abort_flag,
+template <class Bar>
+__device__ __forceinline__ bool mbar_wait_bounded(Bar bar, uint32_t parity, volatile int *abort_flag,
                                                   uint64_t limit_ns = 2000000000ull) {
     if (mbar_try_wait(bar, parity)) return true;
     const uint64_t t0 = globaltimer_ns();
@@ -135,7 +143,8 @@ __device__ __forceinline__ bool named_bar_all(uint32_t id, uint32_t count, bool 
 }
 
 // ---- TMA loads (global -> this CTA's shared memory, completion on an mbarrier) ----------------
-__device__ __forceinline__ void tma_load_2d(void *smem_dst, const CUtensorMap *map, uint64_t *bar, int x, int y) {
+template <class Dst, class Bar>
+__device__ __forceinline__ void tma_load_2d(Dst smem_dst, const CUtensorMap *map, Bar bar, int x, int y) {
     asm volatile(
         "cp.async.bulk.tensor.2d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%3, %4}], [%2];"
         ::"r"(smem_u32(smem_dst)), "l"((uint64_t)map), "r"(smem_u32(bar)), "r"(x), "r"(y)
@@ -155,7 +164,8 @@ __device__ __forceinline__ void tma_load_4d(void *smem_dst, const CUtensorMap *m
         ::"r"(smem_u32(smem_dst)), "l"((uint64_t)map), "r"(smem_u32(bar)), "r"(c), "r"(w), "r"(h), "r"(n)
         : "memory");
 }
-__device__ __forceinline__ void tma_load_5d(void *smem_dst, const CUtensorMap *map, uint64_t *bar, int c0, int c1,
+template <class Dst, class Bar>
+__device__ __forceinline__ void tma_load_5d(Dst smem_dst, const CUtensorMap *map, Bar bar, int c0, int c1,
                                             int c2, int c3, int c4) {
     asm volatile(
         "cp.async.bulk.tensor.5d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%3, %4, %5, %6, %7}], [%2];"
@@ -164,7 +174,8 @@ __device__ __forceinline__ void tma_load_5d(void *smem_dst, const CUtensorMap *m
 }
 // im2col mode over an NHWC tensor: (c, w, h, n) is the first pixel's base coordinate, (off_w, off_h)
 // the filter-tap offset added to every pixel of the column.
-__device__ __forceinline__ void tma_load_im2col_4d(void *smem_dst, const CUtensorMap *map, uint64_t *bar, int c,
+template <class Dst, class Bar>
+__device__ __forceinline__ void tma_load_im2col_4d(Dst smem_dst, const CUtensorMap *map, Bar bar, int c,
                                                    int w, int h, int n, uint16_t off_w, uint16_t off_h) {
     asm volatile(
         "cp.async.bulk.tensor.4d.shared::cluster.global.im2col.mbarrier::complete_tx::bytes"
@@ -238,7 +249,8 @@ __device__ __forceinline__ void umma_bf16_ss(uint32_t d_tmem, uint64_t a_desc, u
         : "memory");
 }
 // The mbarrier gets one arrival once every MMA issued so far by this thread has completed.
-__device__ __forceinline__ void umma_commit(uint64_t *bar) {
+template <class Bar>
+__device__ __forceinline__ void umma_commit(Bar bar) {
     asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(smem_u32(bar))
                  : "memory");
 }
@@ -331,6 +343,16 @@ __device__ __forceinline__ void umma_bf16_ss_halves(uint32_t d_tmem, uint32_t a_
             "tcgen05.mma.cta_group::1.kind::f16 [%0], da, db, %5, p;\n\t}"
             ::"r"(d_tmem), "r"(a_lo), "r"(a_hi), "r"(b_lo), "r"(b_hi), "r"(idesc)
             : "memory");
+}
+// The same with the choice made at run time.
+__device__ __forceinline__ void umma_bf16_ss_halves(uint32_t d_tmem, uint32_t a_lo, uint32_t a_hi, uint32_t b_lo,
+                                                    uint32_t b_hi, uint32_t idesc, uint32_t accumulate) {
+    asm volatile(
+        "{\n\t.reg .pred p;\n\t.reg .b64 da, db;\n\tmov.b64 da, {%1, %2};\n\tmov.b64 db, {%3, %4};\n\t"
+        "setp.ne.u32 p, %6, 0;\n\t"
+        "tcgen05.mma.cta_group::1.kind::f16 [%0], da, db, %5, p;\n\t}"
+        ::"r"(d_tmem), "r"(a_lo), "r"(a_hi), "r"(b_lo), "r"(b_hi), "r"(idesc), "r"(accumulate)
+        : "memory");
 }
 // Instruction descriptor of kind::f16 with bf16 operands and fp32 accumulation.
 // bits 4-5 D format (1 = f32), 7-9 A format (1 = bf16), 10-12 B format (1 = bf16),

@@ -182,74 +182,81 @@ __global__ void __launch_bounds__(MODE == kPlain || MODE == kTap ? 512 : kConvTh
 
     if (warp == 0) {
         // ---------------- TMA producer ----------------
-        // The whole warp runs the loop; lane 0 arms the barrier and loads the activation tile, lane 1
-        // loads the weight tile, so the two copies are issued in parallel.
-        uint32_t it = 0;                         // k-blocks issued so far
-        int s = 0;                               // ring slot and its phase, advanced incrementally
-        uint32_t ph = 0;
-        bool ok = true;
-        if (g.resident && lane == 1) {
-            const int n0 = (int)(blockIdx.x % n_tiles) * BN;
-            mbar_arrive_expect_tx(&ctl->bfull, (uint32_t)num_kb * kBBytes);
-            for (int kb = 0; kb < num_kb; ++kb) {
-                uint8_t *dst = slab + (size_t)kb * kBBytes;
-                if constexpr (TAP)
-                    for (int c = 0; c < BN; c += 64) tma_load_2d(dst + c * 128, &tm_w, &ctl->bfull, n0 + c, kb * kBK);
-                else
-                    tma_load_2d(dst, &tm_w, &ctl->bfull, kb * kBK, n0);
-            }
-        }
-        uint32_t mt, nt;
-        for (uint32_t i = 0; ok && tile_of(i, mt, nt); ++i) {
-            // 32-bit arithmetic: 64-bit divisions would cost about a microsecond per tile here
-            const uint32_t m0 = mt * kBM;
-            const int n0 = (int)nt * BN;
-            uint32_t tq, img;
-            int wo0, ho0;
-            if (g.stem) {       // m-tile -> (image, patch row, patch column)
-                tq = mt / (uint32_t)g.stem_tiles_w;
-                wo0 = (int)(mt - tq * (uint32_t)g.stem_tiles_w) * g.stem_tw;
-                img = tq / (uint32_t)g.stem_tiles_h;
-                ho0 = (int)(tq - img * (uint32_t)g.stem_tiles_h) * g.stem_th;
-            } else {
-                tq = m0 / (uint32_t)g.wo;
-                wo0 = (int)(m0 - tq * (uint32_t)g.wo);
-                img = tq / (uint32_t)g.ho;
-                ho0 = (int)(tq - img * (uint32_t)g.ho);
-            }
-            const int img0 = (int)img;
-            const int base_w = g.lower_w + wo0 * g.stride_w, base_h = g.lower_h + ho0 * g.stride_h;
-            int r = 0, q = 0, cc = 0;
-            for (int kb = 0; kb < num_kb; ++kb, ++it) {
-                { CONVBN_TRACE_T0();
-                ok = __all_sync(0xffffffffu, mbar_wait_bounded(&ctl->empty[s], ph ^ 1u, abort_flag));
-                if (lane == 0) CONVBN_TRACE_ACC(12); }
-                if (!ok) break;
-                uint8_t *a_dst = tiles + (size_t)s * kStageBytes, *b_dst = a_dst + kABytes;
-                if (lane == 0) {
-                    mbar_arrive_expect_tx(&ctl->full[s], kStageBytes);   // (activation + weight tile) or activation only
-                    if (g.stem)
-                        tma_load_5d(a_dst, &tm_act, &ctl->full[s], 0, wo0, ho0, kb, img0);
-                    else
-                    tma_load_im2col_4d(a_dst, &tm_act, &ctl->full[s], (g.blockdiag ? n0 : 0) + cc * kBK, base_w, base_h, img0,
-                                       (uint16_t)(q * g.dil_w), (uint16_t)(r * g.dil_h));
-                } else if (lane == 1 && !g.resident) {
+        // One thread, and as few instructions per k-block as will do: a k-block of 128 x 128 x 64 is 267 clocks of MMAs.
+        // (Two lanes arming and loading in turn, with every address and coordinate formed anew, took 515: 3x3 512 -> 512 at
+        // 7 x 7, N = 64, forward 27.3 us; neither smaller loads nor half of them, by CTA pairs, changed that.)
+        if (elect_one()) {
+            const uint32_t full0 = smem_u32(&ctl->full[0]), empty0 = smem_u32(&ctl->empty[0]), tiles0 = smem_u32(tiles);
+            uint32_t it = 0;                         // k-blocks issued so far
+            uint32_t sb = 0, slot = tiles0, ph = 1;  // ring slot: 8 x its number, its address; parity that says it is free
+            const uint32_t sb_end = 8u * (uint32_t)stages;
+            const bool resident = g.resident;
+            bool ok = true;
+            if (resident) {
+                const int n0 = (int)(blockIdx.x % n_tiles) * BN;
+                mbar_arrive_expect_tx(&ctl->bfull, (uint32_t)num_kb * kBBytes);
+                for (int kb = 0; kb < num_kb; ++kb) {
+                    uint8_t *dst = slab + (size_t)kb * kBBytes;
                     if constexpr (TAP)
-                        for (int c = 0; c < BN; c += 64) tma_load_2d(b_dst + c * 128, &tm_w, &ctl->full[s], n0 + c, kb * kBK);
+                        for (int c = 0; c < BN; c += 64) tma_load_2d(dst + c * 128, &tm_w, &ctl->bfull, n0 + c, kb * kBK);
                     else
-                        tma_load_2d(b_dst, &tm_w, &ctl->full[s], kb * kBK, n0);
+                        tma_load_2d(dst, &tm_w, &ctl->bfull, kb * kBK, n0);
                 }
-                if (++cc == cchunks) { cc = 0; if (++q == g.taps_w) { q = 0; ++r; } }
-                if (++s == stages) { s = 0; ph ^= 1u; }
             }
-        }
-        if (!ok && lane == 0) {
-            atomicOr(err, ERRW_TIMEOUT);
-            ctl->abort_flag = 1;
-            // Let the copies already issued land (bounded) before the CTA may exit.
-            const uint32_t first = it > (uint32_t)stages ? it - stages : 0;
-            for (uint32_t j = first; j < it; ++j)
-                mbar_wait_bounded(&ctl->full[j % stages], (j / stages) & 1u, nullptr, 200000000ull);
+            uint32_t mt, nt;
+            for (uint32_t i = 0; ok && tile_of(i, mt, nt); ++i) {
+                // 32-bit arithmetic: 64-bit divisions would cost about a microsecond per tile here
+                const uint32_t m0 = mt * kBM;
+                const int n0 = (int)nt * BN;
+                uint32_t tq, img;
+                int wo0, ho0;
+                if (g.stem) {       // m-tile -> (image, patch row, patch column)
+                    tq = mt / (uint32_t)g.stem_tiles_w;
+                    wo0 = (int)(mt - tq * (uint32_t)g.stem_tiles_w) * g.stem_tw;
+                    img = tq / (uint32_t)g.stem_tiles_h;
+                    ho0 = (int)(tq - img * (uint32_t)g.stem_tiles_h) * g.stem_th;
+                } else {
+                    tq = m0 / (uint32_t)g.wo;
+                    wo0 = (int)(m0 - tq * (uint32_t)g.wo);
+                    img = tq / (uint32_t)g.ho;
+                    ho0 = (int)(tq - img * (uint32_t)g.ho);
+                }
+                const int img0 = (int)img;
+                const int base_w = g.lower_w + wo0 * g.stride_w, base_h = g.lower_h + ho0 * g.stride_h;
+                const int c_first = g.blockdiag ? n0 : 0, c_end = c_first + cchunks * kBK, w_end = g.taps_w * g.dil_w;
+                int c = c_first, off_w = 0, off_h = 0;
+                for (int k = 0; k < num_kb * kBK; k += kBK) {
+                    ok = mbar_wait_bounded(empty0 + sb, ph, abort_flag);
+                    if (!ok) break;
+                    const uint32_t bar = full0 + sb;
+                    mbar_arrive_expect_tx(bar, kStageBytes);             // (activation + weight tile) or activation only
+                    if (g.stem)
+                        tma_load_5d(slot, &tm_act, bar, 0, wo0, ho0, k / kBK, img0);
+                    else
+                        tma_load_im2col_4d(slot, &tm_act, bar, c, base_w, base_h, img0, (uint16_t)off_w, (uint16_t)off_h);
+                    if (!resident) {
+                        if constexpr (TAP)
+                            for (int cb = 0; cb < BN; cb += 64) tma_load_2d(slot + kABytes + cb * 128, &tm_w, bar, n0 + cb, k);
+                        else
+                            tma_load_2d(slot + kABytes, &tm_w, bar, k, n0);
+                    }
+                    ++it;
+                    if ((c += kBK) == c_end) {
+                        c = c_first;
+                        if ((off_w += g.dil_w) == w_end) { off_w = 0; off_h += g.dil_h; }
+                    }
+                    sb += 8; slot += kStageBytes;
+                    if (sb == sb_end) { sb = 0; slot = tiles0; ph ^= 1u; }
+                }
+            }
+            if (!ok) {
+                atomicOr(err, ERRW_TIMEOUT);
+                ctl->abort_flag = 1;
+                // Let the copies already issued land (bounded) before the CTA may exit.
+                const uint32_t first = it > (uint32_t)stages ? it - stages : 0;
+                for (uint32_t j = first; j < it; ++j)
+                    mbar_wait_bounded(&ctl->full[j % stages], (j / stages) & 1u, nullptr, 200000000ull);
+            }
         }
     } else if (warp == 1) {
         // ---------------- MMA issuer ----------------
@@ -259,10 +266,13 @@ __global__ void __launch_bounds__(MODE == kPlain || MODE == kTap ? 512 : kConvTh
             const uint32_t hi = smem_desc_hi_sw128(1024), b_lead = TAP ? 8192u : 16u;
             const uint32_t tiles_lo = smem_desc_lo(smem_u32(tiles), 16), slab_lo = smem_desc_lo(smem_u32(slab), b_lead);
             const uint32_t ring_b_lo = smem_desc_lo(smem_u32(tiles) + kABytes, b_lead);
-            int s = 0;
-            uint32_t ph = 0;
+            const uint32_t full0 = smem_u32(&ctl->full[0]), empty0 = smem_u32(&ctl->empty[0]);
+            const bool resident = g.resident;
+            const uint32_t a_step = kStageBytes >> 4, b_step = resident ? kBBytes >> 4 : a_step, b_first = resident ? slab_lo : ring_b_lo;
+            const uint32_t sb_end = 8u * (uint32_t)stages;
+            uint32_t sb = 0, ph = 0, a_lo = tiles_lo, b_lo = b_first;
             bool ok = true;
-            if (g.resident) {
+            if (resident) {
                 ok = mbar_wait_bounded(&ctl->bfull, 0, abort_flag);
                 tc_fence_after_sync();
             }
@@ -274,23 +284,23 @@ __global__ void __launch_bounds__(MODE == kPlain || MODE == kTap ? 512 : kConvTh
                 CONVBN_TRACE_ACC(13); }
                 tc_fence_after_sync();
                 const uint32_t d_tmem = tmem_base + acc * BN;
+                if (resident) b_lo = b_first;
                 for (int kb = 0; kb < num_kb; ++kb) {
                     { CONVBN_TRACE_T0();
-                    if (!mbar_wait_bounded(&ctl->full[s], ph, abort_flag)) { ok = false; break; }
+                    if (!mbar_wait_bounded(full0 + sb, ph, abort_flag)) { ok = false; break; }
                     CONVBN_TRACE_ACC(14); }
                     if (i == 0 && kb == 0) CONVBN_TRACE_POINT(4);
-                    tc_fence_after_sync();
                     // descriptors as halves: only the start-address field (16-byte units) moves
-                    const uint32_t a_lo = tiles_lo + (uint32_t)s * (kStageBytes >> 4);
-                    const uint32_t b_lo = g.resident ? slab_lo + (uint32_t)kb * (kBBytes >> 4)
-                                                     : ring_b_lo + (uint32_t)s * (kStageBytes >> 4);
-                    if (kb == 0) umma_bf16_ss_halves<false>(d_tmem, a_lo, hi, b_lo, hi, idesc);
-                    else umma_bf16_ss_halves<true>(d_tmem, a_lo, hi, b_lo, hi, idesc);
+                    umma_bf16_ss_halves(d_tmem, a_lo, hi, b_lo, hi, idesc, (uint32_t)kb);
 #pragma unroll
                     for (int k = 1; k < kBK / kUmmaK; ++k)
                         umma_bf16_ss_halves<true>(d_tmem, a_lo + (uint32_t)k * 2u, hi, b_lo + (uint32_t)k * (TAP ? 128u : 2u), hi, idesc);
-                    umma_commit(&ctl->empty[s]);
-                    if (++s == stages) { s = 0; ph ^= 1u; }
+                    umma_commit(empty0 + sb);
+                    sb += 8; a_lo += a_step; b_lo += b_step;
+                    if (sb == sb_end) {
+                        sb = 0; ph ^= 1u; a_lo = tiles_lo;
+                        if (!resident) b_lo = b_first;
+                    }
                 }
                 if (ok) umma_commit(&ctl->tmem_full[acc]);
                 CONVBN_TRACE_POINT(6);
