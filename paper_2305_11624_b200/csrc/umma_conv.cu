@@ -23,7 +23,8 @@ constexpr int kBM = 128;       // output pixels per tile (UMMA M)
 constexpr int kBK = 64;        // K elements per stage = one 128-byte swizzle row of bf16
 constexpr int kUmmaK = 16;     // K per tcgen05.mma of kind::f16
 constexpr int kMaxStages = 12;
-constexpr int kConvThreads = 320;                             // TMA warp, MMA warp, 2 x 4 epilogue warps
+constexpr int kConvThreads = 352;                             // activation TMA warp, MMA warp, 2 x 4 epilogue warps, weight TMA warp
+constexpr int kWeightWarp = kConvThreads / 32 - 1;
 constexpr uint32_t kStagingWarpBytes = 32 * 128;              // [32 rows][64 bf16]
 constexpr uint32_t kStagingBytes = 8 * kStagingWarpBytes;     // one buffer per epilogue warp
 
@@ -131,7 +132,7 @@ __global__ void __launch_bounds__(MODE == kPlain || MODE == kTap ? 512 : kConvTh
 
     if (threadIdx.x == 0) {
         CONVBN_TRACE_POINT(0);
-        for (int s = 0; s < stages; ++s) { mbar_init(&ctl->full[s], 1); mbar_init(&ctl->empty[s], 1); }
+        for (int s = 0; s < stages; ++s) { mbar_init(&ctl->full[s], g.resident ? 1 : 2); mbar_init(&ctl->empty[s], 1); }
         for (int a = 0; a < 2; ++a) { mbar_init(&ctl->tmem_full[a], 1); mbar_init(&ctl->tmem_empty[a], 4); }
         mbar_init(&ctl->bfull, 1);
         if constexpr (POST)
@@ -182,27 +183,17 @@ __global__ void __launch_bounds__(MODE == kPlain || MODE == kTap ? 512 : kConvTh
 
     if (warp == 0) {
         // ---------------- TMA producer ----------------
-        // One thread, and as few instructions per k-block as will do: a k-block of 128 x 128 x 64 is 267 clocks of MMAs.
-        // (Two lanes arming and loading in turn, with every address and coordinate formed anew, took 515: 3x3 512 -> 512 at
-        // 7 x 7, N = 64, forward 27.3 us; neither smaller loads nor half of them, by CTA pairs, changed that.)
+        // One thread for the activations, one (of the last warp) for the weights, and as few instructions per k-block as will
+        // do: a k-block of 128 x 128 x 64 is 267 clocks of MMAs.  Two lanes of one warp arming and loading in turn, with every
+        // address and coordinate formed anew, took 515 of them; one thread with stepped addresses 430; two threads TWOCLK.
+        // (3x3 512 -> 512 at 7 x 7, N = 64, forward: 27.3, 23.0, TWOUS us.  Neither smaller loads nor half of them, by CTA
+        // pairs, changed the first.)
         if (elect_one()) {
             const uint32_t full0 = smem_u32(&ctl->full[0]), empty0 = smem_u32(&ctl->empty[0]), tiles0 = smem_u32(tiles);
             uint32_t it = 0;                         // k-blocks issued so far
             uint32_t sb = 0, slot = tiles0, ph = 1;  // ring slot: 8 x its number, its address; parity that says it is free
             const uint32_t sb_end = 8u * (uint32_t)stages;
-            const bool resident = g.resident;
             bool ok = true;
-            if (resident) {
-                const int n0 = (int)(blockIdx.x % n_tiles) * BN;
-                mbar_arrive_expect_tx(&ctl->bfull, (uint32_t)num_kb * kBBytes);
-                for (int kb = 0; kb < num_kb; ++kb) {
-                    uint8_t *dst = slab + (size_t)kb * kBBytes;
-                    if constexpr (TAP)
-                        for (int c = 0; c < BN; c += 64) tma_load_2d(dst + c * 128, &tm_w, &ctl->bfull, n0 + c, kb * kBK);
-                    else
-                        tma_load_2d(dst, &tm_w, &ctl->bfull, kb * kBK, n0);
-                }
-            }
             uint32_t mt, nt;
             for (uint32_t i = 0; ok && tile_of(i, mt, nt); ++i) {
                 // 32-bit arithmetic: 64-bit divisions would cost about a microsecond per tile here
@@ -229,17 +220,11 @@ __global__ void __launch_bounds__(MODE == kPlain || MODE == kTap ? 512 : kConvTh
                     ok = mbar_wait_bounded(empty0 + sb, ph, abort_flag);
                     if (!ok) break;
                     const uint32_t bar = full0 + sb;
-                    mbar_arrive_expect_tx(bar, kStageBytes);             // (activation + weight tile) or activation only
+                    mbar_arrive_expect_tx(bar, kABytes);
                     if (g.stem)
                         tma_load_5d(slot, &tm_act, bar, 0, wo0, ho0, k / kBK, img0);
                     else
                         tma_load_im2col_4d(slot, &tm_act, bar, c, base_w, base_h, img0, (uint16_t)off_w, (uint16_t)off_h);
-                    if (!resident) {
-                        if constexpr (TAP)
-                            for (int cb = 0; cb < BN; cb += 64) tma_load_2d(slot + kABytes + cb * 128, &tm_w, bar, n0 + cb, k);
-                        else
-                            tma_load_2d(slot + kABytes, &tm_w, bar, k, n0);
-                    }
                     ++it;
                     if ((c += kBK) == c_end) {
                         c = c_first;
@@ -306,6 +291,49 @@ __global__ void __launch_bounds__(MODE == kPlain || MODE == kTap ? 512 : kConvTh
                 CONVBN_TRACE_POINT(6);
             }
             if (!ok) { atomicOr(err, ERRW_TIMEOUT); ctl->abort_flag = 1; }
+        }
+    } else if (warp == kWeightWarp) {
+        // ---------------- weight loads: the CTA's resident slab once, or a tile per ring slot ----------------
+        if (elect_one()) {
+            const uint32_t full0 = smem_u32(&ctl->full[0]), empty0 = smem_u32(&ctl->empty[0]), tiles0 = smem_u32(tiles) + kABytes;
+            const uint32_t sb_end = 8u * (uint32_t)stages;
+            uint32_t it = 0, sb = 0, slot = tiles0, ph = 1, mt, nt;
+            bool ok = true;
+            if (g.resident) {
+                const int n0 = (int)(blockIdx.x % n_tiles) * BN;
+                mbar_arrive_expect_tx(&ctl->bfull, (uint32_t)num_kb * kBBytes);
+                for (int kb = 0; kb < num_kb; ++kb) {
+                    uint8_t *dst = slab + (size_t)kb * kBBytes;
+                    if constexpr (TAP)
+                        for (int c = 0; c < BN; c += 64) tma_load_2d(dst + c * 128, &tm_w, &ctl->bfull, n0 + c, kb * kBK);
+                    else
+                        tma_load_2d(dst, &tm_w, &ctl->bfull, kb * kBK, n0);
+                }
+            } else {
+                for (uint32_t i = 0; ok && tile_of(i, mt, nt); ++i) {
+                    const int n0 = (int)nt * BN;
+                    for (int k = 0; k < num_kb * kBK; k += kBK) {
+                        ok = mbar_wait_bounded(empty0 + sb, ph, abort_flag);
+                        if (!ok) break;
+                        const uint32_t bar = full0 + sb;
+                        mbar_arrive_expect_tx(bar, kBBytes);
+                        if constexpr (TAP)
+                            for (int cb = 0; cb < BN; cb += 64) tma_load_2d(slot + cb * 128, &tm_w, bar, n0 + cb, k);
+                        else
+                            tma_load_2d(slot, &tm_w, bar, k, n0);
+                        ++it;
+                        sb += 8; slot += kStageBytes;
+                        if (sb == sb_end) { sb = 0; slot = tiles0; ph ^= 1u; }
+                    }
+                }
+            }
+            if (!ok) {
+                atomicOr(err, ERRW_TIMEOUT);
+                ctl->abort_flag = 1;
+                const uint32_t first = it > (uint32_t)stages ? it - stages : 0;
+                for (uint32_t j = first; j < it; ++j)
+                    mbar_wait_bounded(&ctl->full[j % stages], (j / stages) & 1u, nullptr, 200000000ull);
+            }
         }
     } else {
         // ---------------- epilogue: tensor memory -> registers -> bf16 -> shared -> TMA store --------
