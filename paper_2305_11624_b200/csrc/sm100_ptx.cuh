@@ -100,7 +100,8 @@ __device__ __forceinline__ bool mbar_wait_bounded(Bar bar, uint32_t parity, vola
 // The same bounded wait with the non-blocking test_wait: try_wait may park the thread for a system-defined
 // time before it reports "not yet", which adds up to a microsecond to every hand-over of a fine-grained
 // pipeline; test_wait returns at once, at the price of issue slots for the spinning warp.
-__device__ __forceinline__ bool mbar_test_wait(uint64_t *bar, uint32_t parity) {
+template <class Bar>
+__device__ __forceinline__ bool mbar_test_wait(Bar bar, uint32_t parity) {
     uint32_t ok;
     asm volatile(
         "{\n\t.reg .pred p;\n\tmbarrier.test_wait.parity.shared::cta.b64 p, [%1], %2;\n\tselp.u32 %0, 1, 0, p;\n\t}"

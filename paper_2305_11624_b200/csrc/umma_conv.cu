@@ -183,17 +183,18 @@ __global__ void __launch_bounds__(MODE == kPlain || MODE == kTap ? 512 : kConvTh
 
     if (warp == 0) {
         // ---------------- TMA producer ----------------
-        // One thread for the activations, one (of the last warp) for the weights, and as few instructions per k-block as will
-        // do: a k-block of 128 x 128 x 64 is 267 clocks of MMAs.  Two lanes of one warp arming and loading in turn, with every
-        // address and coordinate formed anew, took 515 of them; one thread with stepped addresses 430; two threads TWOCLK.
-        // (3x3 512 -> 512 at 7 x 7, N = 64, forward: 27.3, 23.0, TWOUS us.  Neither smaller loads nor half of them, by CTA
-        // pairs, changed the first.)
+        // One thread for the activations, one (of the last warp) for the weights, stepped addresses, the next slot's barrier
+        // tested while this slot's load is issued, and loops unrolled by four: a taken branch back to a barrier wait costs
+        // about 100 clocks, and a k-block of 128 x 64 x 64 is only 199 clocks of MMAs (267 at 128 columns).  Clocks per k-block
+        // and forward time of 3x3 512 -> 512 at 7 x 7, N = 32: two lanes of one warp forming every address anew 515, 25.6 us;
+        // one thread, stepped 430, 21.0; two threads 350, 18.0; tested ahead 310, 17.2; unrolled 247, 14.6.  (Before, neither
+        // smaller loads nor half of them, by CTA pairs, changed the time: the chip was waiting for these loops.)
         if (elect_one()) {
             const uint32_t full0 = smem_u32(&ctl->full[0]), empty0 = smem_u32(&ctl->empty[0]), tiles0 = smem_u32(tiles);
             uint32_t it = 0;                         // k-blocks issued so far
             uint32_t sb = 0, slot = tiles0, ph = 1;  // ring slot: 8 x its number, its address; parity that says it is free
             const uint32_t sb_end = 8u * (uint32_t)stages;
-            bool ok = true;
+            bool ok = true, free = false;
             uint32_t mt, nt;
             for (uint32_t i = 0; ok && tile_of(i, mt, nt); ++i) {
                 // 32-bit arithmetic: 64-bit divisions would cost about a microsecond per tile here
@@ -216,22 +217,23 @@ __global__ void __launch_bounds__(MODE == kPlain || MODE == kTap ? 512 : kConvTh
                 const int base_w = g.lower_w + wo0 * g.stride_w, base_h = g.lower_h + ho0 * g.stride_h;
                 const int c_first = g.blockdiag ? n0 : 0, c_end = c_first + cchunks * kBK, w_end = g.taps_w * g.dil_w;
                 int c = c_first, off_w = 0, off_h = 0;
-                for (int k = 0; k < num_kb * kBK; k += kBK) {
-                    ok = mbar_wait_bounded(empty0 + sb, ph, abort_flag);
+#pragma unroll 4
+                for (int kb = 0; kb < num_kb; ++kb) {
+                    if (!free) ok = mbar_wait_bounded(empty0 + sb, ph, abort_flag);
                     if (!ok) break;
-                    const uint32_t bar = full0 + sb;
+                    const uint32_t bar = full0 + sb, dst = slot;
+                    ++it; sb += 8; slot += kStageBytes;
+                    if (sb == sb_end) { sb = 0; slot = tiles0; ph ^= 1u; }
+                    free = mbar_test_wait(empty0 + sb, ph);              // of the next slot, while this one's load is issued
                     mbar_arrive_expect_tx(bar, kABytes);
                     if (g.stem)
-                        tma_load_5d(slot, &tm_act, bar, 0, wo0, ho0, k / kBK, img0);
+                        tma_load_5d(dst, &tm_act, bar, 0, wo0, ho0, kb, img0);
                     else
-                        tma_load_im2col_4d(slot, &tm_act, bar, c, base_w, base_h, img0, (uint16_t)off_w, (uint16_t)off_h);
-                    ++it;
+                        tma_load_im2col_4d(dst, &tm_act, bar, c, base_w, base_h, img0, (uint16_t)off_w, (uint16_t)off_h);
                     if ((c += kBK) == c_end) {
                         c = c_first;
                         if ((off_w += g.dil_w) == w_end) { off_w = 0; off_h += g.dil_h; }
                     }
-                    sb += 8; slot += kStageBytes;
-                    if (sb == sb_end) { sb = 0; slot = tiles0; ph ^= 1u; }
                 }
             }
             if (!ok) {
@@ -256,7 +258,7 @@ __global__ void __launch_bounds__(MODE == kPlain || MODE == kTap ? 512 : kConvTh
             const uint32_t a_step = kStageBytes >> 4, b_step = resident ? kBBytes >> 4 : a_step, b_first = resident ? slab_lo : ring_b_lo;
             const uint32_t sb_end = 8u * (uint32_t)stages;
             uint32_t sb = 0, ph = 0, a_lo = tiles_lo, b_lo = b_first;
-            bool ok = true;
+            bool ok = true, ready = false;
             if (resident) {
                 ok = mbar_wait_bounded(&ctl->bfull, 0, abort_flag);
                 tc_fence_after_sync();
@@ -270,22 +272,25 @@ __global__ void __launch_bounds__(MODE == kPlain || MODE == kTap ? 512 : kConvTh
                 tc_fence_after_sync();
                 const uint32_t d_tmem = tmem_base + acc * BN;
                 if (resident) b_lo = b_first;
+#pragma unroll 4
                 for (int kb = 0; kb < num_kb; ++kb) {
                     { CONVBN_TRACE_T0();
-                    if (!mbar_wait_bounded(full0 + sb, ph, abort_flag)) { ok = false; break; }
+                    if (!ready && !mbar_wait_bounded(full0 + sb, ph, abort_flag)) { ok = false; break; }
                     CONVBN_TRACE_ACC(14); }
                     if (i == 0 && kb == 0) CONVBN_TRACE_POINT(4);
                     // descriptors as halves: only the start-address field (16-byte units) moves
-                    umma_bf16_ss_halves(d_tmem, a_lo, hi, b_lo, hi, idesc, (uint32_t)kb);
-#pragma unroll
-                    for (int k = 1; k < kBK / kUmmaK; ++k)
-                        umma_bf16_ss_halves<true>(d_tmem, a_lo + (uint32_t)k * 2u, hi, b_lo + (uint32_t)k * (TAP ? 128u : 2u), hi, idesc);
-                    umma_commit(empty0 + sb);
+                    const uint32_t a0 = a_lo, b0 = b_lo, done = empty0 + sb;
                     sb += 8; a_lo += a_step; b_lo += b_step;
                     if (sb == sb_end) {
                         sb = 0; ph ^= 1u; a_lo = tiles_lo;
                         if (!resident) b_lo = b_first;
                     }
+                    ready = mbar_test_wait(full0 + sb, ph);              // of the next slot, while these MMAs are issued
+                    umma_bf16_ss_halves(d_tmem, a0, hi, b0, hi, idesc, (uint32_t)kb);
+#pragma unroll
+                    for (int k = 1; k < kBK / kUmmaK; ++k)
+                        umma_bf16_ss_halves<true>(d_tmem, a0 + (uint32_t)k * 2u, hi, b0 + (uint32_t)k * (TAP ? 128u : 2u), hi, idesc);
+                    umma_commit(done);
                 }
                 if (ok) umma_commit(&ctl->tmem_full[acc]);
                 CONVBN_TRACE_POINT(6);
@@ -298,7 +303,7 @@ __global__ void __launch_bounds__(MODE == kPlain || MODE == kTap ? 512 : kConvTh
             const uint32_t full0 = smem_u32(&ctl->full[0]), empty0 = smem_u32(&ctl->empty[0]), tiles0 = smem_u32(tiles) + kABytes;
             const uint32_t sb_end = 8u * (uint32_t)stages;
             uint32_t it = 0, sb = 0, slot = tiles0, ph = 1, mt, nt;
-            bool ok = true;
+            bool ok = true, free = false;
             if (g.resident) {
                 const int n0 = (int)(blockIdx.x % n_tiles) * BN;
                 mbar_arrive_expect_tx(&ctl->bfull, (uint32_t)num_kb * kBBytes);
@@ -312,18 +317,19 @@ __global__ void __launch_bounds__(MODE == kPlain || MODE == kTap ? 512 : kConvTh
             } else {
                 for (uint32_t i = 0; ok && tile_of(i, mt, nt); ++i) {
                     const int n0 = (int)nt * BN;
+#pragma unroll 4
                     for (int k = 0; k < num_kb * kBK; k += kBK) {
-                        ok = mbar_wait_bounded(empty0 + sb, ph, abort_flag);
+                        if (!free) ok = mbar_wait_bounded(empty0 + sb, ph, abort_flag);
                         if (!ok) break;
-                        const uint32_t bar = full0 + sb;
+                        const uint32_t bar = full0 + sb, dst = slot;
+                        ++it; sb += 8; slot += kStageBytes;
+                        if (sb == sb_end) { sb = 0; slot = tiles0; ph ^= 1u; }
+                        free = mbar_test_wait(empty0 + sb, ph);
                         mbar_arrive_expect_tx(bar, kBBytes);
                         if constexpr (TAP)
-                            for (int cb = 0; cb < BN; cb += 64) tma_load_2d(slot + cb * 128, &tm_w, bar, n0 + cb, k);
+                            for (int cb = 0; cb < BN; cb += 64) tma_load_2d(dst + cb * 128, &tm_w, bar, n0 + cb, k);
                         else
-                            tma_load_2d(slot, &tm_w, bar, k, n0);
-                        ++it;
-                        sb += 8; slot += kStageBytes;
-                        if (sb == sb_end) { sb = 0; slot = tiles0; ph ^= 1u; }
+                            tma_load_2d(dst, &tm_w, bar, k, n0);
                     }
                 }
             }
