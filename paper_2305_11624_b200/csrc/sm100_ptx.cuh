@@ -151,14 +151,16 @@ __device__ __forceinline__ void tma_load_2d(Dst smem_dst, const CUtensorMap *map
         ::"r"(smem_u32(smem_dst)), "l"((uint64_t)map), "r"(smem_u32(bar)), "r"(x), "r"(y)
         : "memory");
 }
-__device__ __forceinline__ void tma_load_3d(void *smem_dst, const CUtensorMap *map, uint64_t *bar, int c0, int c1, int c2) {
+template <class Dst, class Bar>
+__device__ __forceinline__ void tma_load_3d(Dst smem_dst, const CUtensorMap *map, Bar bar, int c0, int c1, int c2) {
     asm volatile(
         "cp.async.bulk.tensor.3d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%3, %4, %5}], [%2];"
         ::"r"(smem_u32(smem_dst)), "l"((uint64_t)map), "r"(smem_u32(bar)), "r"(c0), "r"(c1), "r"(c2)
         : "memory");
 }
 // Tiled 4-D box (c, w, h, n); coordinates outside the tensor read zeros (c must stay 16-byte aligned).
-__device__ __forceinline__ void tma_load_4d(void *smem_dst, const CUtensorMap *map, uint64_t *bar, int c, int w,
+template <class Dst, class Bar>
+__device__ __forceinline__ void tma_load_4d(Dst smem_dst, const CUtensorMap *map, Bar bar, int c, int w,
                                             int h, int n) {
     asm volatile(
         "cp.async.bulk.tensor.4d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%3, %4, %5, %6}], [%2];"

@@ -19,7 +19,8 @@ constexpr int kWM = 128;          // k rows per tile (two 64-channel slices)
 constexpr int kWP = 64;           // pixels per stage (reduction depth per stage)
 constexpr int kWUmmaK = 16;
 constexpr int kWMaxStages = 8;
-constexpr int kWThreads = 192;
+constexpr int kWThreads = 224;    // X loads, MMA, 4 epilogue warps, dZ loads
+constexpr int kWDzWarp = kWThreads / 32 - 1;
 constexpr uint32_t kChunkBytes = kWP * 64 * 2;   // one [64 pixels][64 channels] bf16 box
 
 struct WgradGemm {
@@ -74,7 +75,7 @@ __global__ void __launch_bounds__(kWThreads) umma_wgrad_kernel(const __grid_cons
     volatile int *abort_flag = &ctl->abort_flag;
 
     if (threadIdx.x == 0) {
-        for (int s = 0; s < stages; ++s) { mbar_init(&ctl->full[s], 1); mbar_init(&ctl->empty[s], 1); }
+        for (int s = 0; s < stages; ++s) { mbar_init(&ctl->full[s], 2); mbar_init(&ctl->empty[s], 1); }
         mbar_init(&ctl->tmem_full, 1);
         ctl->abort_flag = 0;
         fence_barrier_init();
@@ -105,87 +106,124 @@ __global__ void __launch_bounds__(kWThreads) umma_wgrad_kernel(const __grid_cons
     pdl_launch_dependents();       // only now: this CTA owns its tensor-memory columns
     const uint32_t tmem_base = ctl->tmem_base;
 
+    // the two loading threads' walk through the ring
+    const uint32_t full0 = smem_u32(&ctl->full[0]), empty0 = smem_u32(&ctl->empty[0]), tiles0 = smem_u32(tiles), sb_end = 8u * (uint32_t)stages;
+    uint32_t sb = 0, slot = tiles0, ph = 1;
+    int issued = 0;
+    bool ok = true, free = false;
+    auto give_up = [&]() {
+        if (ok) return;
+        atomicOr(err, ERRW_TIMEOUT);
+        ctl->abort_flag = 1;
+        for (int kb = issued > stages ? issued - stages : 0; kb < issued; ++kb)     // let the copies in flight land
+            mbar_wait_bounded(&ctl->full[kb % stages], (uint32_t)(kb / stages) & 1u, nullptr, 200000000ull);
+    };
+    // stem: pixel block -> (image, patch row, patch column) of 4 x 16 output pixels
+    auto patch = [&](uint32_t blk, int &pw, int &phh, int &im) {
+        const uint32_t t1 = blk / (uint32_t)g.stem_tiles_w, i1 = t1 / (uint32_t)g.stem_tiles_h;
+        pw = (int)(blk - t1 * (uint32_t)g.stem_tiles_w) * 16;
+        phh = (int)(t1 - i1 * (uint32_t)g.stem_tiles_h) * 4;
+        im = (int)i1;
+    };
+
     if (warp == 0) {
-        // The whole warp runs the loop; lanes 0-1 load the two X slices, lanes 2.. the dZ boxes.
-        const uint32_t tx_bytes = (uint32_t)(a_chunks + b_chunks) * kChunkBytes;
-        // this lane's X slice: k = tap * c_in + ci is fixed for the whole CTA
-        const int kk = k0 + (lane & 1) * 64;
-        const int tap = kk / g.c_in, ci0 = kk - tap * g.c_in + (g.blockdiag ? n0 : 0);
-        const int tr = tap / g.taps_w, tq = tap - tr * g.taps_w;
-        const uint16_t off_w = (uint16_t)(tq * g.dil_w), off_h = (uint16_t)(tr * g.dil_h);
-        int issued = 0, s = 0;
-        uint32_t ph = 0;
-        bool ok = true;
-        // pixel coordinates of the slice start, advanced by 64 pixels per stage without divisions
-        uint32_t pp = (uint32_t)p0;
-        uint32_t t0 = pp / (uint32_t)g.wo;
-        int wo0 = (int)(pp - t0 * (uint32_t)g.wo);
-        uint32_t img = t0 / (uint32_t)g.ho;
-        int ho0 = (int)(t0 - img * (uint32_t)g.ho);
-        for (int kb = 0; kb < num_kb; ++kb) {
-            ok = __all_sync(0xffffffffu, mbar_wait_bounded(&ctl->empty[s], ph ^ 1u, abort_flag));
-            if (!ok) break;
-            const int base_w = g.lower_w + wo0 * g.stride_w, base_h = g.lower_h + ho0 * g.stride_h;
-            uint8_t *a_dst = tiles + (size_t)s * kStageBytes, *b_dst = a_dst + kABytes;
-            if (lane == 0) mbar_arrive_expect_tx(&ctl->full[s], tx_bytes);
-            if (g.stem) {
-                // pixel block -> (image, patch row, patch column) of 4 x 16 output pixels
-                const uint32_t blk = (uint32_t)(p0 / kWP) + (uint32_t)kb;
-                const uint32_t t1 = blk / (uint32_t)g.stem_tiles_w;
-                const int pw = (int)(blk - t1 * (uint32_t)g.stem_tiles_w) * 16;
-                const uint32_t im = t1 / (uint32_t)g.stem_tiles_h;
-                const int phh = (int)(t1 - im * (uint32_t)g.stem_tiles_h) * 4;
-                if (lane < a_chunks)
-                    tma_load_5d(a_dst + lane * kChunkBytes, &tm_x, &ctl->full[s], 0, pw, phh, c_first + lane, (int)im);
-                else if (lane >= 2 && lane - 2 < b_chunks)
-                    tma_load_4d(b_dst + (lane - 2) * kChunkBytes, &tm_dz, &ctl->full[s], n0 + (lane - 2) * 64, pw, phh,
-                                (int)im);
-            } else
-            if (lane < a_chunks)
-                tma_load_im2col_4d(a_dst + lane * kChunkBytes, &tm_x, &ctl->full[s], ci0, base_w, base_h, (int)img,
-                                   off_w, off_h);
-            else if (lane >= 2 && lane - 2 < b_chunks)
-                tma_load_2d(b_dst + (lane - 2) * kChunkBytes, &tm_dz, &ctl->full[s], n0 + (lane - 2) * 64, (int)pp);
-            ++issued;
-            if (++s == stages) { s = 0; ph ^= 1u; }
-            pp += kWP;
-            wo0 += kWP;
-            while (wo0 >= g.wo) { wo0 -= g.wo; if (++ho0 == g.ho) { ho0 = 0; ++img; } }
+        // One thread for the X slices, one (of the last warp) for dZ; stepped addresses, the next slot's barrier tested ahead,
+        // loops unrolled: what one thread has to do per stage bounded this kernel (see umma_conv.cu).
+        // Weight phase with its second kernel, graph replay: 3x3 512 at 7 x 7, N = 64 29.5 -> 25.5 us, N = 32 22.6 -> 20.6,
+        // 3x3 64 at 56 x 56, N = 32 21.9 -> 19.4.
+        if (elect_one()) {
+            const uint32_t tx_bytes = (uint32_t)a_chunks * kChunkBytes;
+            // the slices' k = tap * c_in + ci is fixed for the whole CTA
+            int ci[2];
+            uint16_t off_w[2], off_h[2];
+#pragma unroll
+            for (int j = 0; j < 2; ++j) {
+                const int kk = k0 + j * 64, tap = kk / g.c_in, tr = tap / g.taps_w;
+                ci[j] = kk - tap * g.c_in + (g.blockdiag ? n0 : 0);
+                off_w[j] = (uint16_t)((tap - tr * g.taps_w) * g.dil_w);
+                off_h[j] = (uint16_t)(tr * g.dil_h);
+            }
+            // pixel coordinates of the slice start, advanced by 64 pixels per stage without divisions
+            const uint32_t pp = (uint32_t)p0, t0 = pp / (uint32_t)g.wo;
+            int wo0 = (int)(pp - t0 * (uint32_t)g.wo);
+            uint32_t img = t0 / (uint32_t)g.ho;
+            int ho0 = (int)(t0 - img * (uint32_t)g.ho);
+            const uint32_t blk0 = (uint32_t)(p0 / kWP);
+#pragma unroll 4
+            for (int kb = 0; kb < num_kb; ++kb) {
+                if (!free) ok = mbar_wait_bounded(empty0 + sb, ph, abort_flag);
+                if (!ok) break;
+                const uint32_t bar = full0 + sb, dst = slot;
+                ++issued; sb += 8; slot += kStageBytes;
+                if (sb == sb_end) { sb = 0; slot = tiles0; ph ^= 1u; }
+                free = mbar_test_wait(empty0 + sb, ph);
+                mbar_arrive_expect_tx(bar, tx_bytes);
+                if (g.stem) {
+                    int pw, phh, im;
+                    patch(blk0 + (uint32_t)kb, pw, phh, im);
+                    if (a_chunks > 0) tma_load_5d(dst, &tm_x, bar, 0, pw, phh, c_first, im);
+                    if (a_chunks > 1) tma_load_5d(dst + kChunkBytes, &tm_x, bar, 0, pw, phh, c_first + 1, im);
+                } else {
+                    const int base_w = g.lower_w + wo0 * g.stride_w, base_h = g.lower_h + ho0 * g.stride_h;
+                    if (a_chunks > 0) tma_load_im2col_4d(dst, &tm_x, bar, ci[0], base_w, base_h, (int)img, off_w[0], off_h[0]);
+                    if (a_chunks > 1) tma_load_im2col_4d(dst + kChunkBytes, &tm_x, bar, ci[1], base_w, base_h, (int)img, off_w[1], off_h[1]);
+                    wo0 += kWP;
+                    while (wo0 >= g.wo) { wo0 -= g.wo; if (++ho0 == g.ho) { ho0 = 0; ++img; } }
+                }
+            }
+            give_up();
         }
-        if (!ok && lane == 0) {
-            atomicOr(err, ERRW_TIMEOUT);
-            ctl->abort_flag = 1;
-            const int first = issued > stages ? issued - stages : 0;
-            for (int kb = first; kb < issued; ++kb)
-                mbar_wait_bounded(&ctl->full[kb % stages], (uint32_t)(kb / stages) & 1u, nullptr, 200000000ull);
+    } else if (warp == kWDzWarp) {
+        if (elect_one()) {
+            const uint32_t blk0 = (uint32_t)(p0 / kWP);
+            slot += kABytes;
+#pragma unroll 4
+            for (int kb = 0; kb < num_kb; ++kb) {
+                if (!free) ok = mbar_wait_bounded(empty0 + sb, ph, abort_flag);
+                if (!ok) break;
+                const uint32_t bar = full0 + sb, dst = slot;
+                ++issued; sb += 8; slot += kStageBytes;
+                if (sb == sb_end) { sb = 0; slot = tiles0 + kABytes; ph ^= 1u; }
+                free = mbar_test_wait(empty0 + sb, ph);
+                if (g.stem) {
+                    int pw, phh, im;
+                    patch(blk0 + (uint32_t)kb, pw, phh, im);
+                    mbar_arrive_expect_tx(bar, (uint32_t)b_chunks * kChunkBytes);
+                    for (int j = 0; j < b_chunks; ++j) tma_load_4d(dst + j * kChunkBytes, &tm_dz, bar, n0 + j * 64, pw, phh, im);
+                } else {
+                    mbar_arrive_expect_tx(bar, kBBytes);             // (slices past C_out arrive as zeros)
+                    tma_load_3d(dst, &tm_dz, bar, 0, (int)p0 + kb * kWP, n0 / 64);
+                }
+            }
+            give_up();
         }
     } else if (warp == 1) {
         if (elect_one()) {
             const uint32_t idesc = idesc_h16_f32(kWM, BN, 1, 1, g.f16);   // both operands MN-major
             const uint32_t hi = smem_desc_hi_sw128(1024);
             const uint32_t tiles_lo = smem_desc_lo(smem_u32(tiles), kChunkBytes);
-            bool ok = true;
-            int s = 0;
-            uint32_t ph = 0;
+            uint32_t a_lo = tiles_lo;
+            ph = 0;
+#pragma unroll 4
             for (int kb = 0; kb < num_kb; ++kb) {
-                if (!mbar_wait_bounded(&ctl->full[s], ph, abort_flag)) {
+                if (!free && !mbar_wait_bounded(full0 + sb, ph, abort_flag)) {
                     atomicOr(err, ERRW_TIMEOUT);
                     ctl->abort_flag = 1;
                     ok = false;
                     break;
                 }
-                tc_fence_after_sync();
                 // 16 pixels = two groups of 8 rows (1024 B apart); 64-channel slices 8192 B apart; descriptors as
                 // halves, only the start-address field (16-byte units) moves
-                const uint32_t a_lo = tiles_lo + (uint32_t)s * (kStageBytes >> 4), b_lo = a_lo + (kABytes >> 4);
-                if (kb == 0) umma_bf16_ss_halves<false>(tmem_base, a_lo, hi, b_lo, hi, idesc);
-                else umma_bf16_ss_halves<true>(tmem_base, a_lo, hi, b_lo, hi, idesc);
+                const uint32_t a0 = a_lo, b0 = a_lo + (kABytes >> 4), done = empty0 + sb;
+                sb += 8; a_lo += kStageBytes >> 4;
+                if (sb == sb_end) { sb = 0; a_lo = tiles_lo; ph ^= 1u; }
+                free = mbar_test_wait(full0 + sb, ph);
+                umma_bf16_ss_halves(tmem_base, a0, hi, b0, hi, idesc, (uint32_t)kb);
 #pragma unroll
                 for (int k = 1; k < kWP / kWUmmaK; ++k)
-                    umma_bf16_ss_halves<true>(tmem_base, a_lo + (uint32_t)k * (kWUmmaK * 128 >> 4), hi,
-                                              b_lo + (uint32_t)k * (kWUmmaK * 128 >> 4), hi, idesc);
-                umma_commit(&ctl->empty[s]);
-                if (++s == stages) { s = 0; ph ^= 1u; }
+                    umma_bf16_ss_halves<true>(tmem_base, a0 + (uint32_t)k * (kWUmmaK * 128 >> 4), hi,
+                                              b0 + (uint32_t)k * (kWUmmaK * 128 >> 4), hi, idesc);
+                umma_commit(done);
             }
             if (ok) umma_commit(&ctl->tmem_full);
         }
@@ -320,11 +358,16 @@ cudaError_t launch_umma_wgrad(const Problem &pb, const UmmaWgradPlan &pl, const 
     if (!make_tmap_im2col_bf16(&tx, x, pb.n, pb.h_in, pb.w_in, pb.c_in, g.lower_h, g.lower_w, upper_h, upper_w,
                                pb.stride_h, pb.stride_w, kWP, 64))
         return cudaErrorInvalidValue;
-    if (!make_tmap_matrix_bf16(&tdz, dz, pb.p, pb.c_out, kWP, 64)) return cudaErrorInvalidValue;
+    const int bn = g.blockdiag ? 64 : wgrad_bn(pb);
+    {   // a stage's [64 pixels][64 channels] slices of dZ, side by side in shared memory, are one box
+        const unsigned long long dims[3] = {64, (unsigned long long)pb.p, (unsigned long long)pb.c_out / 64};
+        const unsigned long long str[3] = {0, (unsigned long long)pb.c_out * 2, 128};
+        const unsigned int box[3] = {64, (unsigned int)kWP, (unsigned int)(bn / 64)};
+        if (!make_tmap_tiled_bf16(&tdz, dz, 3, dims, str, box)) return cudaErrorInvalidValue;
+    }
     int *err = nullptr;
     cudaError_t e = error_word_address(&err);
     if (e != cudaSuccess) return e;
-    const int bn = g.blockdiag ? 64 : wgrad_bn(pb);
     if (bn == 64) return launch_w<64>(tx, tdz, g, pl, pb, partials, bsum, err, st, counters, ncounters);
     return launch_w<128>(tx, tdz, g, pl, pb, partials, bsum, err, st, counters, ncounters);
 }
