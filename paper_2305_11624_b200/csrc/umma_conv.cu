@@ -33,6 +33,7 @@ struct ConvGemm {
     int cn;                  // output channels (GEMM N)
     int ca;                  // activation channels (multiple of 64)
     int taps_h, taps_w;
+    int chunk_outer;         // order of K: 1: channel chunk by chunk, all taps of each; 0: tap by tap, all chunks of each
     int lower_h, lower_w;    // input coordinate read by output (0,0) at tap (0,0)
     int stride_h, stride_w, dil_h, dil_w;
     long long p;             // output pixels n * ho * wo
@@ -215,7 +216,7 @@ __global__ void __launch_bounds__(MODE == kPlain || MODE == kTap ? 512 : kConvTh
                 }
                 const int img0 = (int)img;
                 const int base_w = g.lower_w + wo0 * g.stride_w, base_h = g.lower_h + ho0 * g.stride_h;
-                const int c_first = g.blockdiag ? n0 : 0, c_end = c_first + cchunks * kBK, w_end = g.taps_w * g.dil_w;
+                const int c_first = g.blockdiag ? n0 : 0, c_end = c_first + cchunks * kBK, w_end = g.taps_w * g.dil_w, h_end = g.taps_h * g.dil_h;
                 int c = c_first, off_w = 0, off_h = 0;
 #pragma unroll 4
                 for (int kb = 0; kb < num_kb; ++kb) {
@@ -230,7 +231,12 @@ __global__ void __launch_bounds__(MODE == kPlain || MODE == kTap ? 512 : kConvTh
                         tma_load_5d(dst, &tm_act, bar, 0, wo0, ho0, kb, img0);
                     else
                         tma_load_im2col_4d(dst, &tm_act, bar, c, base_w, base_h, img0, (uint16_t)off_w, (uint16_t)off_h);
-                    if ((c += kBK) == c_end) {
+                    if (g.chunk_outer) {
+                        if ((off_w += g.dil_w) == w_end) {
+                            off_w = 0;
+                            if ((off_h += g.dil_h) == h_end) { off_h = 0; c += kBK; }
+                        }
+                    } else if ((c += kBK) == c_end) {
                         c = c_first;
                         if ((off_w += g.dil_w) == w_end) { off_w = 0; off_h += g.dil_h; }
                     }
@@ -303,22 +309,27 @@ __global__ void __launch_bounds__(MODE == kPlain || MODE == kTap ? 512 : kConvTh
             const uint32_t full0 = smem_u32(&ctl->full[0]), empty0 = smem_u32(&ctl->empty[0]), tiles0 = smem_u32(tiles) + kABytes;
             const uint32_t sb_end = 8u * (uint32_t)stages;
             uint32_t it = 0, sb = 0, slot = tiles0, ph = 1, mt, nt;
+            const int k_step = g.chunk_outer ? g.ca : kBK;
             bool ok = true, free = false;
             if (g.resident) {
                 const int n0 = (int)(blockIdx.x % n_tiles) * BN;
                 mbar_arrive_expect_tx(&ctl->bfull, (uint32_t)num_kb * kBBytes);
+                int k = 0;
                 for (int kb = 0; kb < num_kb; ++kb) {
                     uint8_t *dst = slab + (size_t)kb * kBBytes;
                     if constexpr (TAP)
-                        for (int c = 0; c < BN; c += 64) tma_load_2d(dst + c * 128, &tm_w, &ctl->bfull, n0 + c, kb * kBK);
+                        for (int c = 0; c < BN; c += 64) tma_load_2d(dst + c * 128, &tm_w, &ctl->bfull, n0 + c, k);
                     else
-                        tma_load_2d(dst, &tm_w, &ctl->bfull, kb * kBK, n0);
+                        tma_load_2d(dst, &tm_w, &ctl->bfull, k, n0);
+                    k += k_step;
+                    if (k >= num_kb * kBK) k += kBK - num_kb * kBK;
                 }
             } else {
                 for (uint32_t i = 0; ok && tile_of(i, mt, nt); ++i) {
                     const int n0 = (int)nt * BN;
+                    int k = 0;
 #pragma unroll 4
-                    for (int k = 0; k < num_kb * kBK; k += kBK) {
+                    for (int kb = 0; kb < num_kb; ++kb) {
                         if (!free) ok = mbar_wait_bounded(empty0 + sb, ph, abort_flag);
                         if (!ok) break;
                         const uint32_t bar = full0 + sb, dst = slot;
@@ -330,6 +341,8 @@ __global__ void __launch_bounds__(MODE == kPlain || MODE == kTap ? 512 : kConvTh
                             for (int cb = 0; cb < BN; cb += 64) tma_load_2d(dst + cb * 128, &tm_w, bar, n0 + cb, k);
                         else
                             tma_load_2d(dst, &tm_w, bar, k, n0);
+                        k += k_step;
+                        if (k >= num_kb * kBK) k += kBK - num_kb * kBK;      // (chunk_outer: the next chunk's first tap)
                     }
                 }
             }
@@ -759,6 +772,7 @@ cudaError_t launch_umma_conv(const UmmaConvShape &s, const void *act, const void
     g.lower_h = s.lower_h; g.lower_w = s.lower_w; g.stride_h = s.stride_h; g.stride_w = s.stride_w;
     g.dil_h = s.dil_h; g.dil_w = s.dil_w; g.p = (long long)s.n * s.ho * s.wo; g.stages = 1;
     g.blockdiag = s.blockdiag;
+    g.chunk_outer = umma_strip_possible(s);              // the strip kernel's order, so that results do not depend on the choice
     g.f16 = call_f16();
     g.stem = 0; g.stem_tw = g.stem_th = g.stem_tiles_w = g.stem_tiles_h = 1;
     g.fold = fold ? *fold : BnFold{nullptr, nullptr, nullptr, nullptr, nullptr, 0.f, nullptr};
@@ -808,6 +822,7 @@ cudaError_t launch_stem_fwd(const Problem &pb, const void *x_packed, const void 
                             cudaStream_t st, const BnFold *fold) {
     const int krows = stem_krows(pb);
     ConvGemm g;
+    g.chunk_outer = 0;
     g.tap_c = 0; g.post_add = g.post_mask = nullptr; g.post_relu = 0;
     g.ho = pb.h_out; g.wo = pb.w_out; g.cn = pb.c_out; g.ca = 64; g.taps_h = krows; g.taps_w = 1;
     g.lower_h = g.lower_w = 0; g.stride_h = g.stride_w = g.dil_h = g.dil_w = 1;

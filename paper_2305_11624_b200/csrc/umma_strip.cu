@@ -202,9 +202,11 @@ __global__ void __launch_bounds__(kSThreads) umma_strip_conv_kernel(const __grid
     } else if (warp == 1) {
         // ---------------- weight-tile loader ----------------
         if (elect_one()) {
-            int s = 0;
-            uint32_t ph = 0;
-            bool ok = true;
+            // (stepped addresses, the next slot's barrier tested ahead, unrolled: see umma_conv.cu)
+            const uint32_t full0 = smem_u32(&ctl->b_full[0]), empty0 = smem_u32(&ctl->b_empty[0]), ring0 = smem_u32(bring);
+            const uint32_t sb_end = 8u * (uint32_t)bstages;
+            uint32_t sb = 0, slot = ring0, ph = 1;
+            bool ok = true, free = false;
             if (g.resident) {
                 // one n-tile, every (channel chunk, tap) tile loaded once: tile index cc taps + tap
                 if (blockIdx.x < total_tiles) {
@@ -218,14 +220,21 @@ __global__ void __launch_bounds__(kSThreads) umma_strip_conv_kernel(const __grid
             for (uint32_t t = blockIdx.x; t < total_tiles && ok; t += gridDim.x) {
                 const int n0 = (int)(t % n_tiles) * BN;
                 const uint32_t mask = g.sub_wide ? g.sub_mask[n0 / g.sub_cin] : 0xffffffffu;
-                for (int cc = 0; cc < cchunks && ok; ++cc)
-                    for (int tap = 0; tap < taps; ++tap) {
+                for (int cc = 0; cc < cchunks && ok; ++cc) {
+                    int kx = cc * 64;
+#pragma unroll 3
+                    for (int tap = 0; tap < taps; ++tap, kx += w_ca) {
                         if (!((mask >> tap) & 1u)) continue;
-                        if (!mbar_wait_bounded(&ctl->b_empty[s], ph ^ 1u, abort_flag)) { ok = false; break; }
-                        mbar_arrive_expect_tx(&ctl->b_full[s], kBBytes);
-                        tma_load_2d(bring + (size_t)s * kBBytes, &tm_w, &ctl->b_full[s], tap * w_ca + cc * 64, n0);
-                        if (++s == bstages) { s = 0; ph ^= 1u; }
+                        if (!free) ok = mbar_wait_bounded(empty0 + sb, ph, abort_flag);
+                        if (!ok) break;
+                        const uint32_t bar = full0 + sb, dst = slot;
+                        sb += 8; slot += kBBytes;
+                        if (sb == sb_end) { sb = 0; slot = ring0; ph ^= 1u; }
+                        free = mbar_test_wait(empty0 + sb, ph);
+                        mbar_arrive_expect_tx(bar, kBBytes);
+                        tma_load_2d(dst, &tm_w, bar, kx, n0);
                     }
+                }
             }
             if (!ok) { atomicOr(err, ERRW_TIMEOUT); ctl->abort_flag = 1; }
             if (!ok) for (int q = 0; q < bstages; ++q) mbar_wait_bounded(&ctl->b_full[q], 0, nullptr, 2000000ull);
@@ -240,9 +249,11 @@ __global__ void __launch_bounds__(kSThreads) umma_strip_conv_kernel(const __grid
             const uint32_t idesc = idesc_h16_f32(128, BN, 0, 0, g.f16);
             const uint32_t hi = smem_desc_hi_sw128(1024);
             const uint32_t bres_lo = smem_desc_lo(smem_u32(bring), 16);
-            int sb = 0, s = 0;
+            const uint32_t bfull0 = smem_u32(&ctl->b_full[0]), bempty0 = smem_u32(&ctl->b_empty[0]), s8_end = 8u * (uint32_t)bstages;
+            int sb = 0;
+            uint32_t s8 = 0, b_lo = bres_lo;            // weight ring: 8 x the slot's number, the slot's descriptor
             uint32_t sph = 0, bph = 0, i = 0;
-            bool ok = true;
+            bool ok = true, ready = false;
             if (g.resident && blockIdx.x < total_tiles) {
                 ok = mbar_wait_bounded(&ctl->bres_full, 0, abort_flag);
                 tc_fence_after_sync();
@@ -253,11 +264,39 @@ __global__ void __launch_bounds__(kSThreads) umma_strip_conv_kernel(const __grid
                 tc_fence_after_sync();
                 const uint32_t d0 = tmem_base + a * (uint32_t)(g.nmb * BN);
                 const uint32_t mask = g.sub_wide ? g.sub_mask[(int)(t % n_tiles) * BN / g.sub_cin] : 0xffffffffu;
-                bool started = false;                   // false until the tile's first MMAs have been issued
+                uint32_t started = 0;                   // 0 until the tile's first MMAs have been issued
+                if (g.resident) b_lo = bres_lo;
                 for (int cc = 0; cc < cchunks && ok; ++cc) {
                     if (!mbar_wait_bounded(&ctl->strip_full[sb], sph, abort_flag)) { ok = false; break; }
                     tc_fence_after_sync();
                     if (i == 0 && cc == 0 && me == 0) CONVBN_TRACE_POINT(4);
+                    if constexpr (BN != 16) {
+                        // One M block per issuer (512 columns of two accumulator sets hold at most four of 64).
+                        uint32_t a_row = smem_desc_lo(smem_u32(strips + (size_t)sb * g.strip_bytes), 16) + (uint32_t)me * 1024u;
+                        uint32_t a_lo = a_row;
+                        int q = 0;
+#pragma unroll 3
+                        for (int tap = 0; tap < taps; ++tap) {
+                            const uint32_t a0 = a_lo;
+                            a_lo += 8u;
+                            if (++q == g.kw) { q = 0; a_row += (uint32_t)g.Wt * 8u; a_lo = a_row; }
+                            if (!((mask >> tap) & 1u)) continue;
+                            if (!g.resident && !ready && !mbar_wait_bounded(bfull0 + s8, bph, abort_flag)) { ok = false; break; }
+                            const uint32_t b0 = b_lo, done = bempty0 + s8;
+                            b_lo += kBBytes >> 4;
+                            if (!g.resident) {
+                                s8 += 8;
+                                if (s8 == s8_end) { s8 = 0; bph ^= 1u; b_lo = bres_lo; }
+                                ready = mbar_test_wait(bfull0 + s8, bph);
+                            }
+                            umma_bf16_ss_halves(d0 + (uint32_t)(me * BN), a0, hi, b0, hi, idesc, started);
+                            started = 1u;
+#pragma unroll
+                            for (int k = 1; k < 4; ++k)
+                                umma_bf16_ss_halves<true>(d0 + (uint32_t)(me * BN), a0 + (uint32_t)k * 2u, hi, b0 + (uint32_t)k * 2u, hi, idesc);
+                            if (!g.resident) umma_commit(done);
+                        }
+                    } else {
                     const uint32_t a_patch = smem_desc_lo(smem_u32(strips + (size_t)sb * g.strip_bytes), 16);
                     uint32_t row_shift = 0;             // (r Wt + q) pixels of 128 bytes, in 16-byte units
                     int q = 0;
@@ -265,33 +304,26 @@ __global__ void __launch_bounds__(kSThreads) umma_strip_conv_kernel(const __grid
                         const uint32_t a_tap = a_patch + row_shift + (uint32_t)q * 8u;
                         if (++q == g.kw) { q = 0; row_shift += (uint32_t)g.Wt * 8u; }
                         if (!((mask >> tap) & 1u)) continue;
-                        uint32_t b_lo;
-                        if (g.resident) {
-                            b_lo = bres_lo + (uint32_t)(cc * taps + tap) * (kBBytes >> 4);
-                        } else {
-                            if (!mbar_wait_bounded(&ctl->b_full[s], bph, abort_flag)) { ok = false; break; }
-                            tc_fence_after_sync();
-                            b_lo = smem_desc_lo(smem_u32(bring + (size_t)s * kBBytes), 16);
+                        if (!g.resident && !ready && !mbar_wait_bounded(bfull0 + s8, bph, abort_flag)) { ok = false; break; }
+                        const uint32_t b0 = b_lo, done = bempty0 + s8;
+                        b_lo += kBBytes >> 4;
+                        if (!g.resident) {
+                            s8 += 8;
+                            if (s8 == s8_end) { s8 = 0; bph ^= 1u; b_lo = bres_lo; }
+                            ready = mbar_test_wait(bfull0 + s8, bph);
                         }
                         // consecutive MMAs go to different accumulators (M blocks), so an MMA never has to
                         // wait for the previous one's accumulator update
-                        if (!started) {
-                            for (int mb = me; mb < g.nmb; mb += ni)
-                                umma_bf16_ss_halves<false>(d0 + (uint32_t)(mb * BN), a_tap + (uint32_t)mb * 1024u, hi, b_lo, hi, idesc);
-                            started = true;
-                        } else {
-                            for (int mb = me; mb < g.nmb; mb += ni)
-                                umma_bf16_ss_halves<true>(d0 + (uint32_t)(mb * BN), a_tap + (uint32_t)mb * 1024u, hi, b_lo, hi, idesc);
-                        }
+                        for (int mb = me; mb < g.nmb; mb += ni)
+                            umma_bf16_ss_halves(d0 + (uint32_t)(mb * BN), a_tap + (uint32_t)mb * 1024u, hi, b0, hi, idesc, started);
+                        started = 1u;
 #pragma unroll
                         for (int k = 1; k < 4; ++k)
                             for (int mb = me; mb < g.nmb; mb += ni)
                                 umma_bf16_ss_halves<true>(d0 + (uint32_t)(mb * BN), a_tap + (uint32_t)mb * 1024u + (uint32_t)k * 2u, hi,
-                                                          b_lo + (uint32_t)k * 2u, hi, idesc);
-                        if (!g.resident) {
-                            umma_commit(&ctl->b_empty[s]);
-                            if (++s == bstages) { s = 0; bph ^= 1u; }
-                        }
+                                                          b0 + (uint32_t)k * 2u, hi, idesc);
+                        if (!g.resident) umma_commit(done);
+                    }
                     }
                     if (ok) umma_commit(&ctl->strip_empty[sb]);
                     if (++sb == nstrips) { sb = 0; sph ^= 1u; }
@@ -588,6 +620,8 @@ cudaError_t launch_strip(const CUtensorMap &ta, const CUtensorMap &tw, const Str
 }
 
 }  // namespace
+
+bool umma_strip_possible(const UmmaConvShape &s) { return plan_strip(s).ok; }
 
 bool umma_strip_eligible(const UmmaConvShape &s) {
     return plan_strip(s).ok;
