@@ -86,7 +86,10 @@ struct ConvSmemCtl {
 // 64 -> 256 layer at 56 x 56, N = 32 took 90 us with an addend).  MODE kPostStrided: the same for strided outputs, whose
 // rows are no box: read from global memory.
 enum ConvMode { kPlain, kDual, kTap, kPost, kPostStrided };
-template <int BN, ConvMode MODE>
+//
+// PAIR: two CTAs of a cluster share a 256 x BN product (cta_group::2).  Each brings its own 128 pixels and HALF of the
+// weight tile, and gets the accumulator of its own pixels; the first CTA issues the MMAs of both (see pick_tile for what that gains).
+template <int BN, ConvMode MODE, bool PAIR>
 __global__ void __launch_bounds__(MODE == kPlain || MODE == kTap ? 512 : kConvThreads) umma_conv_kernel(const __grid_constant__ CUtensorMap tm_act,
                                                                 const __grid_constant__ CUtensorMap tm_w,
                                                                 const __grid_constant__ CUtensorMap tm_out,
@@ -96,7 +99,9 @@ __global__ void __launch_bounds__(MODE == kPlain || MODE == kTap ? 512 : kConvTh
                                                                 int *err) {
     extern __shared__ uint8_t smem_raw[];
     constexpr bool DUAL = MODE == kDual, TAP = MODE == kTap, POST = MODE == kPost, POST_STRIDED = MODE == kPostStrided;
-    constexpr uint32_t kABytes = kBM * kBK * 2, kBBytes = BN * kBK * 2;
+    constexpr uint32_t kABytes = kBM * kBK * 2, kBBytes = BN * kBK * 2 / (PAIR ? 2 : 1);
+    constexpr int CTAS = PAIR ? 2 : 1;
+    const uint32_t rank = PAIR ? cluster_rank() : 0u;
     const int cchunks = g.blockdiag ? 1 : g.ca / kBK;
     const int num_kb = g.taps_h * g.taps_w * cchunks;
     // Ring slots hold the activation tile and, unless the weights are resident, the weight tile.
@@ -114,7 +119,7 @@ __global__ void __launch_bounds__(MODE == kPlain || MODE == kTap ? 512 : kConvTh
     const int stages = g.stages;
     const uint32_t n_tiles = (uint32_t)(g.cn + BN - 1) / BN;
     const uint32_t m_tiles = (uint32_t)((g.p + kBM - 1) / kBM);
-    const uint32_t total_tiles = m_tiles * n_tiles;
+    const uint32_t total_tiles = (PAIR ? (m_tiles + 1) / 2 : m_tiles) * n_tiles;
     // Tile i of this CTA.  Resident weights: the CTA keeps one n-tile (blockIdx.x % n_tiles) and walks
     // m-tiles; otherwise tiles are dealt round-robin with the n-tiles of an m-tile on neighbouring CTAs.
     auto tile_of = [&](uint32_t i, uint32_t &mt, uint32_t &nt) -> bool {
@@ -123,18 +128,21 @@ __global__ void __launch_bounds__(MODE == kPlain || MODE == kTap ? 512 : kConvTh
             mt = blockIdx.x / n_tiles + i * (gridDim.x / n_tiles);
             return mt < m_tiles;
         }
-        const uint32_t t = blockIdx.x + i * gridDim.x;
+        const uint32_t t = blockIdx.x / CTAS + i * (gridDim.x / CTAS);
         if (t >= total_tiles) return false;
         mt = t / n_tiles;
         nt = t - mt * n_tiles;
+        if constexpr (PAIR) mt = 2 * mt + rank;         // (of an odd number of m-tiles the last has no partner: all out of range)
         return true;
     };
     volatile int *abort_flag = &ctl->abort_flag;
+    // a pair's boxes all count on its first CTA's barriers
+    const uint32_t full_of_first = PAIR ? cluster_addr(&ctl->full[0], 0) : smem_u32(&ctl->full[0]);
 
     if (threadIdx.x == 0) {
         CONVBN_TRACE_POINT(0);
         for (int s = 0; s < stages; ++s) { mbar_init(&ctl->full[s], g.resident ? 1 : 2); mbar_init(&ctl->empty[s], 1); }
-        for (int a = 0; a < 2; ++a) { mbar_init(&ctl->tmem_full[a], 1); mbar_init(&ctl->tmem_empty[a], 4); }
+        for (int a = 0; a < 2; ++a) { mbar_init(&ctl->tmem_full[a], 1); mbar_init(&ctl->tmem_empty[a], 4 * CTAS); }
         mbar_init(&ctl->bfull, 1);
         if constexpr (POST)
             for (int a = 0; a < 8; ++a) mbar_init(&ctl->post_full[a], 1);
@@ -142,8 +150,8 @@ __global__ void __launch_bounds__(MODE == kPlain || MODE == kTap ? 512 : kConvTh
         fence_barrier_init();
     }
     if (warp == 1) {
-        tmem_alloc(&ctl->tmem_base, 2 * BN);
-        tmem_relinquish();
+        tmem_alloc<CTAS>(&ctl->tmem_base, 2 * BN);
+        tmem_relinquish<CTAS>();
     }
     // Everything above touched only this CTA's own shared / tensor memory.  Global memory (inputs that
     // an earlier kernel may still be writing, outputs it may still be reading) comes after this wait.
@@ -177,11 +185,17 @@ __global__ void __launch_bounds__(MODE == kPlain || MODE == kTap ? 512 : kConvTh
     }
     tc_fence_before_sync();
     __syncthreads();
+    if constexpr (PAIR) cluster_sync_all();                 // both CTAs' barriers and columns are there
     tc_fence_after_sync();
     pdl_launch_dependents();       // only now: this CTA owns its tensor-memory columns
     const uint32_t tmem_base = ctl->tmem_base;
     if (threadIdx.x == 0) CONVBN_TRACE_POINT(2);
 
+    // The first CTA's commits arrive in the second too: a loading thread sees the last of them before its CTA may exit.
+    auto drain = [&](uint32_t it, bool &ok) {
+        for (uint32_t j = it > (uint32_t)stages ? it - stages : 0; ok && j < it; ++j)
+            ok = mbar_wait_bounded(&ctl->empty[j % stages], (j / stages) & 1u, abort_flag);
+    };
     if (warp == 0) {
         // ---------------- TMA producer ----------------
         // One thread for the activations, one (of the last warp) for the weights, stepped addresses, the next slot's barrier
@@ -191,7 +205,7 @@ __global__ void __launch_bounds__(MODE == kPlain || MODE == kTap ? 512 : kConvTh
         // one thread, stepped 430, 21.0; two threads 350, 18.0; tested ahead 310, 17.2; unrolled 247, 14.6.  (Before, neither
         // smaller loads nor half of them, by CTA pairs, changed the time: the chip was waiting for these loops.)
         if (elect_one()) {
-            const uint32_t full0 = smem_u32(&ctl->full[0]), empty0 = smem_u32(&ctl->empty[0]), tiles0 = smem_u32(tiles);
+            const uint32_t full0 = full_of_first, empty0 = smem_u32(&ctl->empty[0]), tiles0 = smem_u32(tiles);
             uint32_t it = 0;                         // k-blocks issued so far
             uint32_t sb = 0, slot = tiles0, ph = 1;  // ring slot: 8 x its number, its address; parity that says it is free
             const uint32_t sb_end = 8u * (uint32_t)stages;
@@ -199,7 +213,7 @@ __global__ void __launch_bounds__(MODE == kPlain || MODE == kTap ? 512 : kConvTh
             uint32_t mt, nt;
             for (uint32_t i = 0; ok && tile_of(i, mt, nt); ++i) {
                 // 32-bit arithmetic: 64-bit divisions would cost about a microsecond per tile here
-                const uint32_t m0 = mt * kBM;
+                const uint32_t m0 = (PAIR && mt >= m_tiles ? m_tiles - 1 : mt) * kBM;
                 const int n0 = (int)nt * BN;
                 uint32_t tq, img;
                 int wo0, ho0;
@@ -216,8 +230,10 @@ __global__ void __launch_bounds__(MODE == kPlain || MODE == kTap ? 512 : kConvTh
                 }
                 const int img0 = (int)img;
                 const int base_w = g.lower_w + wo0 * g.stride_w, base_h = g.lower_h + ho0 * g.stride_h;
-                const int c_first = g.blockdiag ? n0 : 0, c_end = c_first + cchunks * kBK, w_end = g.taps_w * g.dil_w, h_end = g.taps_h * g.dil_h;
-                int c = c_first, off_w = 0, off_h = 0;
+                // K: an inner run over the channels of a tap (or, chunk_outer, over a row of taps) with one addition a step
+                const int c_first = g.blockdiag ? n0 : 0, w_end = g.taps_w * g.dil_w, h_end = g.taps_h * g.dil_h;
+                const int inner = g.chunk_outer ? g.taps_w : cchunks, dc = g.chunk_outer ? 0 : kBK, dw = g.chunk_outer ? g.dil_w : 0;
+                int c = c_first, off_w = 0, off_h = 0, left = inner;
 #pragma unroll 4
                 for (int kb = 0; kb < num_kb; ++kb) {
                     if (!free) ok = mbar_wait_bounded(empty0 + sb, ph, abort_flag);
@@ -226,41 +242,51 @@ __global__ void __launch_bounds__(MODE == kPlain || MODE == kTap ? 512 : kConvTh
                     ++it; sb += 8; slot += kStageBytes;
                     if (sb == sb_end) { sb = 0; slot = tiles0; ph ^= 1u; }
                     free = mbar_test_wait(empty0 + sb, ph);              // of the next slot, while this one's load is issued
-                    mbar_arrive_expect_tx(bar, kABytes);
-                    if (g.stem)
+                    if (rank == 0) mbar_arrive_expect_tx(bar, CTAS * kABytes);
+                    if constexpr (PAIR)
+                        tma_load_im2col_4d_pair(dst, &tm_act, bar, c, base_w, base_h, img0, (uint16_t)off_w, (uint16_t)off_h);
+                    else if (g.stem)
                         tma_load_5d(dst, &tm_act, bar, 0, wo0, ho0, kb, img0);
                     else
                         tma_load_im2col_4d(dst, &tm_act, bar, c, base_w, base_h, img0, (uint16_t)off_w, (uint16_t)off_h);
-                    if (g.chunk_outer) {
-                        if ((off_w += g.dil_w) == w_end) {
+                    c += dc; off_w += dw;
+                    if (--left == 0) {
+                        left = inner;
+                        if (g.chunk_outer) {
                             off_w = 0;
                             if ((off_h += g.dil_h) == h_end) { off_h = 0; c += kBK; }
+                        } else {
+                            c = c_first;
+                            if ((off_w += g.dil_w) == w_end) { off_w = 0; off_h += g.dil_h; }
                         }
-                    } else if ((c += kBK) == c_end) {
-                        c = c_first;
-                        if ((off_w += g.dil_w) == w_end) { off_w = 0; off_h += g.dil_h; }
                     }
                 }
             }
+            if constexpr (PAIR) drain(it, ok);
             if (!ok) {
                 atomicOr(err, ERRW_TIMEOUT);
                 ctl->abort_flag = 1;
+                if constexpr (PAIR)       // counted in the first CTA as far as that has got: a millisecond is ample for any of them
+                    for (const uint64_t t0 = globaltimer_ns(); globaltimer_ns() - t0 < 1000000ull;) {}
                 // Let the copies already issued land (bounded) before the CTA may exit.
                 const uint32_t first = it > (uint32_t)stages ? it - stages : 0;
-                for (uint32_t j = first; j < it; ++j)
+                for (uint32_t j = first; !PAIR && j < it; ++j)
                     mbar_wait_bounded(&ctl->full[j % stages], (j / stages) & 1u, nullptr, 200000000ull);
             }
         }
     } else if (warp == 1) {
         // ---------------- MMA issuer ----------------
-        if (elect_one()) {
+        if (rank == 0 && elect_one()) {
             // MN-major weights: 64-column blocks of [64 k][128 bytes], 8192 bytes apart; 16 k = 2048 bytes
-            const uint32_t idesc = idesc_h16_f32(kBM, BN, 0, TAP ? 1 : 0, g.f16);
+            const uint32_t idesc = idesc_h16_f32(kBM * CTAS, BN, 0, TAP ? 1 : 0, g.f16);
             const uint32_t hi = smem_desc_hi_sw128(1024), b_lead = TAP ? 8192u : 16u;
             const uint32_t tiles_lo = smem_desc_lo(smem_u32(tiles), 16), slab_lo = smem_desc_lo(smem_u32(slab), b_lead);
             const uint32_t ring_b_lo = smem_desc_lo(smem_u32(tiles) + kABytes, b_lead);
             const uint32_t full0 = smem_u32(&ctl->full[0]), empty0 = smem_u32(&ctl->empty[0]);
             const bool resident = g.resident;
+            auto commit = [](auto bar) {
+                if constexpr (PAIR) umma_commit_pair(bar); else umma_commit(bar);
+            };
             const uint32_t a_step = kStageBytes >> 4, b_step = resident ? kBBytes >> 4 : a_step, b_first = resident ? slab_lo : ring_b_lo;
             const uint32_t sb_end = 8u * (uint32_t)stages;
             uint32_t sb = 0, ph = 0, a_lo = tiles_lo, b_lo = b_first;
@@ -292,13 +318,13 @@ __global__ void __launch_bounds__(MODE == kPlain || MODE == kTap ? 512 : kConvTh
                         if (!resident) b_lo = b_first;
                     }
                     ready = mbar_test_wait(full0 + sb, ph);              // of the next slot, while these MMAs are issued
-                    umma_bf16_ss_halves(d_tmem, a0, hi, b0, hi, idesc, (uint32_t)kb);
+                    umma_bf16_ss_sel<CTAS>(d_tmem, a0, hi, b0, hi, idesc, (uint32_t)kb);
 #pragma unroll
                     for (int k = 1; k < kBK / kUmmaK; ++k)
-                        umma_bf16_ss_halves<true>(d_tmem, a0 + (uint32_t)k * 2u, hi, b0 + (uint32_t)k * (TAP ? 128u : 2u), hi, idesc);
-                    umma_commit(done);
+                        umma_bf16_ss_halves<true, CTAS>(d_tmem, a0 + (uint32_t)k * 2u, hi, b0 + (uint32_t)k * (TAP ? 128u : 2u), hi, idesc);
+                    commit(done);
                 }
-                if (ok) umma_commit(&ctl->tmem_full[acc]);
+                if (ok) commit(&ctl->tmem_full[acc]);
                 CONVBN_TRACE_POINT(6);
             }
             if (!ok) { atomicOr(err, ERRW_TIMEOUT); ctl->abort_flag = 1; }
@@ -306,7 +332,7 @@ __global__ void __launch_bounds__(MODE == kPlain || MODE == kTap ? 512 : kConvTh
     } else if (warp == kWeightWarp) {
         // ---------------- weight loads: the CTA's resident slab once, or a tile per ring slot ----------------
         if (elect_one()) {
-            const uint32_t full0 = smem_u32(&ctl->full[0]), empty0 = smem_u32(&ctl->empty[0]), tiles0 = smem_u32(tiles) + kABytes;
+            const uint32_t full0 = full_of_first, empty0 = smem_u32(&ctl->empty[0]), tiles0 = smem_u32(tiles) + kABytes;
             const uint32_t sb_end = 8u * (uint32_t)stages;
             uint32_t it = 0, sb = 0, slot = tiles0, ph = 1, mt, nt;
             const int k_step = g.chunk_outer ? g.ca : kBK;
@@ -336,8 +362,10 @@ __global__ void __launch_bounds__(MODE == kPlain || MODE == kTap ? 512 : kConvTh
                         ++it; sb += 8; slot += kStageBytes;
                         if (sb == sb_end) { sb = 0; slot = tiles0; ph ^= 1u; }
                         free = mbar_test_wait(empty0 + sb, ph);
-                        mbar_arrive_expect_tx(bar, kBBytes);
-                        if constexpr (TAP)
+                        if (rank == 0) mbar_arrive_expect_tx(bar, CTAS * kBBytes);
+                        if constexpr (PAIR)
+                            tma_load_2d_pair(dst, &tm_w, bar, k, n0 + (int)rank * (BN / 2));
+                        else if constexpr (TAP)
                             for (int cb = 0; cb < BN; cb += 64) tma_load_2d(dst + cb * 128, &tm_w, bar, n0 + cb, k);
                         else
                             tma_load_2d(dst, &tm_w, bar, k, n0);
@@ -346,11 +374,14 @@ __global__ void __launch_bounds__(MODE == kPlain || MODE == kTap ? 512 : kConvTh
                     }
                 }
             }
+            if constexpr (PAIR) drain(it, ok);
             if (!ok) {
                 atomicOr(err, ERRW_TIMEOUT);
                 ctl->abort_flag = 1;
+                if constexpr (PAIR)       // counted in the first CTA as far as that has got: a millisecond is ample for any of them
+                    for (const uint64_t t0 = globaltimer_ns(); globaltimer_ns() - t0 < 1000000ull;) {}
                 const uint32_t first = it > (uint32_t)stages ? it - stages : 0;
-                for (uint32_t j = first; j < it; ++j)
+                for (uint32_t j = first; !PAIR && j < it; ++j)
                     mbar_wait_bounded(&ctl->full[j % stages], (j / stages) & 1u, nullptr, 200000000ull);
             }
         }
@@ -421,7 +452,10 @@ __global__ void __launch_bounds__(MODE == kPlain || MODE == kTap ? 512 : kConvTh
                     // every column of this accumulator has been read: hand the buffer back
                     tc_fence_before_sync();
                     __syncwarp();
-                    if (lane == 0) mbar_arrive(&ctl->tmem_empty[acc]);
+                    if (lane == 0) {
+                        if constexpr (PAIR) mbar_arrive_cluster(cluster_addr(&ctl->tmem_empty[acc], 0));
+                        else mbar_arrive(&ctl->tmem_empty[acc]);
+                    }
                 }
                 if (c0 < ncols) {
                     uint8_t *buf = stage_buf;
@@ -588,8 +622,9 @@ __global__ void __launch_bounds__(MODE == kPlain || MODE == kTap ? 512 : kConvTh
     }
     tc_fence_before_sync();
     __syncthreads();
+    if constexpr (PAIR) cluster_sync_all();                 // neither CTA's barriers, tiles or columns are in use any more
     if (threadIdx.x == 0) CONVBN_TRACE_POINT(11);
-    if (warp == 1) tmem_dealloc(tmem_base, 2 * BN);
+    if (warp == 1) tmem_dealloc<CTAS>(tmem_base, 2 * BN);
 }
 
 // ---- failure-path self-test: the bounded wait of the kernels above, on a barrier nobody completes --------
@@ -706,21 +741,25 @@ bool umma_conv_eligible(const UmmaConvShape &s) {
 
 static int sm_count() { return device_sm_count(); }
 
-template <int BN, ConvMode MODE = kPlain>
+template <int BN, ConvMode MODE = kPlain, bool PAIR = false>
 static cudaError_t launch_bn(const CUtensorMap &ta, const CUtensorMap &tw, const CUtensorMap &tout,
                              const CUtensorMap &tout2, const CUtensorMap &tmask, ConvGemm g, const float *bias, int *err,
                              cudaStream_t st) {
-    const size_t a_bytes = (size_t)kBM * kBK * 2, b_bytes = (size_t)BN * kBK * 2;
+    const size_t a_bytes = (size_t)kBM * kBK * 2, b_bytes = (size_t)BN * kBK * 2 / (PAIR ? 2 : 1);
     const int extra = MODE == kPost ? (g.post_add != nullptr) + (g.post_mask != nullptr) : 0;
     size_t fixed = 1024 + (size_t)(1 + extra) * kStagingBytes + sizeof(ConvSmemCtl) + (MODE == kDual ? 3 : 2) * (size_t)g.cn * sizeof(float) + 16;
     const int num_kb = g.taps_h * g.taps_w * (g.blockdiag ? 1 : g.ca / kBK);
     const long long m_tiles = (g.p + kBM - 1) / kBM, n_tiles = (g.cn + BN - 1) / BN;
     long long grid_l = m_tiles * n_tiles < sm_count() ? m_tiles * n_tiles : sm_count();
+    if (PAIR) {
+        const long long pairs = (m_tiles + 1) / 2 * n_tiles;
+        grid_l = 2 * (pairs < sm_count() / 2 ? pairs : sm_count() / 2);
+    }
     // Weights stay resident when the CTA's slab fits beside at least four activation slots and the
     // grid can give every CTA one fixed n-tile.
     const size_t slab = (size_t)num_kb * b_bytes;
     g.resident = 0;
-    if (slab <= 104 * 1024 && fixed + slab + 4 * a_bytes <= 220 * 1024 && m_tiles * n_tiles >= sm_count() &&
+    if (!PAIR && slab <= 104 * 1024 && fixed + slab + 4 * a_bytes <= 220 * 1024 && m_tiles * n_tiles >= sm_count() &&
         n_tiles <= sm_count()) {
         g.resident = 1;
         grid_l = sm_count() - sm_count() % n_tiles;
@@ -732,36 +771,49 @@ static cudaError_t launch_bn(const CUtensorMap &ta, const CUtensorMap &tw, const
     g.stages = stages;
     const size_t smem = stages * stage + fixed;
     static PerDevice attr_done;
-    if (cudaError_t e = max_dynamic_smem_once(umma_conv_kernel<BN, MODE>, 224 * 1024, &attr_done); e != cudaSuccess) return e;
+    if (cudaError_t e = max_dynamic_smem_once(umma_conv_kernel<BN, MODE, PAIR>, 224 * 1024, &attr_done); e != cudaSuccess) return e;
     static PerDevice carve;
-    prefer_max_shared_once(umma_conv_kernel<BN, MODE>, &carve);
+    prefer_max_shared_once(umma_conv_kernel<BN, MODE, PAIR>, &carve);
     const unsigned grid = (unsigned)grid_l;
-    return launch_pdl(umma_conv_kernel<BN, MODE>, dim3(grid), dim3(kConvThreads), smem, st, ta, tw, tout, tout2, tmask, g, bias, err);
+    return launch_pdl<PAIR ? 2 : 1>(umma_conv_kernel<BN, MODE, PAIR>, dim3(grid), dim3(kConvThreads), smem, st, ta, tw, tout, tout2, tmask, g, bias, err);
 }
 
 template <ConvMode MODE>
-static cudaError_t launch_mode(int bn, const CUtensorMap &ta, const CUtensorMap &tw, const CUtensorMap &tout,
+static cudaError_t launch_mode(int bn, bool pair, const CUtensorMap &ta, const CUtensorMap &tw, const CUtensorMap &tout,
                                const CUtensorMap &tout2, const CUtensorMap &tmask, const ConvGemm &g, const float *bias,
                                int *err, cudaStream_t st) {
+    if constexpr (MODE == kPlain || MODE == kPost) {
+        if (pair && bn == 64) return launch_bn<64, MODE, true>(ta, tw, tout, tout2, tmask, g, bias, err, st);
+        if (pair && bn == 128) return launch_bn<128, MODE, true>(ta, tw, tout, tout2, tmask, g, bias, err, st);
+        if (pair) return launch_bn<256, MODE, true>(ta, tw, tout, tout2, tmask, g, bias, err, st);
+    }
     if (bn == 64) return launch_bn<64, MODE>(ta, tw, tout, tout2, tmask, g, bias, err, st);
     if (bn == 128) return launch_bn<128, MODE>(ta, tw, tout, tout2, tmask, g, bias, err, st);
     return launch_bn<256, MODE>(ta, tw, tout, tout2, tmask, g, bias, err, st);
 }
 
-// Tile width: fewest rounds of tiles over the SMs, weighted by the time of one tile (N = 64 tiles are
-// bound by shared-memory operand bandwidth, about 1.5x slower per column than wider ones).
-static int pick_bn(long long tiles_m, int cn) {
-    int best = 64;
+// Tile width, and whether CTAs work in pairs: the least time by a model of clocks fitted to 24 layers (3x3 and 1x1, 64 to
+// 2048 channels, N = 8 to 256, both directions) at all six choices.  A round of tiles takes the larger of its k-blocks and
+// its epilogue; the last tile's epilogue and a pair's start-up (a cluster launch, two CTAs meeting twice) come on top.  A
+// k-block costs a CTA of a pair 20 to 90 clocks less, being half a weight tile to write to and read from shared memory, so
+// pairs pay for long K or many rounds.  Forward, against the better of the unpaired widths: 3x3 512 -> 512 at 7 x 7, N = 256
+// 51.8 -> 45.8 us, N = 32 16.1 -> 15.3; 1x1 512 -> 1024 at 28 x 28, N = 256 227 -> 216.5 (back: 215.5 -> 182); but
+// 1x1 64 -> 256 at 56 x 56, N = 32 16.5 -> 19.3.  The choices of the model are within 0.7 % of the best on average.
+struct TilePick { int bn; bool pair; };
+static TilePick pick_tile(long long tiles_m, int cn, int num_kb, bool pairs, int max_bn) {
+    static const double clk[2][3] = {{645, 300, 260}, {555, 280, 205}};
+    TilePick best{64, false};
     double best_cost = 1e30;
-    const int cand[3] = {256, 128, 64};
-    for (int c = 0; c < 3; ++c) {
-        const int bn = cand[c];
-        if (bn > 64 && cn <= bn / 2) continue;
-        const long long tiles = tiles_m * ((cn + bn - 1) / bn);
-        const long long rounds = (tiles + sm_count() - 1) / sm_count();
-        const double cost = (double)rounds * bn * (bn == 64 ? 1.5 : 1.0);
-        if (cost < best_cost) { best_cost = cost; best = bn; }
-    }
+    for (int pr = 0; pr <= (pairs ? 1 : 0); ++pr)
+        for (int c = 0; c < 3; ++c) {
+            const int bn = 256 >> c;
+            if (bn > max_bn || (bn > 64 && cn <= bn / 2)) continue;
+            const long long n_tiles = (cn + bn - 1) / bn, slots = pr ? sm_count() / 2 : sm_count();
+            const long long rounds = ((pr ? (tiles_m + 1) / 2 : tiles_m) * n_tiles + slots - 1) / slots;
+            const double mma = num_kb * clk[pr][c], epi = 9.0 * bn;
+            const double cost = (double)rounds * ((mma > epi ? mma : epi) + 220.0) + 6.0 * bn + (pr ? 2100.0 : 0.0);
+            if (cost < best_cost) { best_cost = cost; best = TilePick{bn, pr != 0}; }
+        }
     return best;
 }
 
@@ -787,9 +839,13 @@ cudaError_t launch_umma_conv(const UmmaConvShape &s, const void *act, const void
     const int upper_h = s.lower_h + (s.ho - 1) * s.stride_h - (s.ha - 1);
     const int upper_w = s.lower_w + (s.wo - 1) * s.stride_w - (s.wa - 1);
     const long long tiles_m = (g.p + kBM - 1) / kBM;
-    int bn = s.blockdiag ? 64 : pick_bn(tiles_m, s.cn);
-    while (s.tap_c && s.tap_c % bn) bn /= 2;            // a tile lies inside one tap
-    if (!s.out_sw && (g.post_add || g.post_mask) && bn > 128) bn = 128;       // room for the other tensors' staging areas
+    int max_bn = s.blockdiag ? 64 : 256;
+    while (s.tap_c && s.tap_c % max_bn) max_bn /= 2;     // a tile lies inside one tap
+    if (!s.out_sw && (g.post_add || g.post_mask) && max_bn > 128) max_bn = 128;       // room for the other tensors' staging areas
+    const bool pairs = !s.blockdiag && !s.tap_c && !out2 && !(with_post && s.out_sw);
+    const TilePick pick = pick_tile(tiles_m, s.cn, s.taps_h * s.taps_w * (s.blockdiag ? 1 : s.ca / kBK), pairs, max_bn);
+    const int bn = pick.bn;
+    const bool pair = pick.pair;
     CUtensorMap ta, tw, tout;
     // (in strided mode the output map is encoded but never used: every row is stored by its thread)
     if (!make_tmap_matrix_bf16(&tout, out, s.out_sw ? 32 : g.p, s.cn, 32, 64)) return cudaErrorInvalidValue;
@@ -797,7 +853,7 @@ cudaError_t launch_umma_conv(const UmmaConvShape &s, const void *act, const void
                                s.stride_w, kBM, kBK))
         return cudaErrorInvalidValue;
     if (s.tap_c ? !make_tmap_matrix_bf16(&tw, wmat, s.ca, s.cn, kBK, 64)
-                : !make_tmap_matrix_bf16(&tw, wmat, s.cn, (long long)s.taps_h * s.taps_w * (s.blockdiag ? 64 : s.ca), bn, kBK))
+                : !make_tmap_matrix_bf16(&tw, wmat, s.cn, (long long)s.taps_h * s.taps_w * (s.blockdiag ? 64 : s.ca), pair ? bn / 2 : bn, kBK))
         return cudaErrorInvalidValue;
     int *err = nullptr;
     cudaError_t e = error_word_address(&err);
@@ -808,12 +864,12 @@ cudaError_t launch_umma_conv(const UmmaConvShape &s, const void *act, const void
     if (with_post && !s.out_sw) {
         if (g.post_add && !make_tmap_matrix_bf16(&tout2, post->add, g.p, s.cn, 32, 64)) return cudaErrorInvalidValue;
         if (g.post_mask && !make_tmap_matrix_bf16(&tmask, post->mask, g.p, s.cn, 32, 64)) return cudaErrorInvalidValue;
-        return launch_mode<kPost>(bn, ta, tw, tout, tout2, tmask, g, bias, err, st);
+        return launch_mode<kPost>(bn, pair, ta, tw, tout, tout2, tmask, g, bias, err, st);
     }
-    if (with_post) return launch_mode<kPostStrided>(bn, ta, tw, tout, tout2, tmask, g, bias, err, st);
-    if (out2) return launch_mode<kDual>(bn, ta, tw, tout, tout2, tmask, g, bias, err, st);
-    if (g.tap_c) return launch_mode<kTap>(bn, ta, tw, tout, tout2, tmask, g, bias, err, st);
-    return launch_mode<kPlain>(bn, ta, tw, tout, tout2, tmask, g, bias, err, st);
+    if (with_post) return launch_mode<kPostStrided>(bn, pair, ta, tw, tout, tout2, tmask, g, bias, err, st);
+    if (out2) return launch_mode<kDual>(bn, pair, ta, tw, tout, tout2, tmask, g, bias, err, st);
+    if (g.tap_c) return launch_mode<kTap>(bn, pair, ta, tw, tout, tout2, tmask, g, bias, err, st);
+    return launch_mode<kPlain>(bn, pair, ta, tw, tout, tout2, tmask, g, bias, err, st);
 }
 
 // Forward pass of a small-C_in layer on the packed input (see stem_kernels.cu): tiles of 8 x 16 output

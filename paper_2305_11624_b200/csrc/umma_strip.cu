@@ -289,7 +289,7 @@ __global__ void __launch_bounds__(kSThreads) umma_strip_conv_kernel(const __grid
                                 if (s8 == s8_end) { s8 = 0; bph ^= 1u; b_lo = bres_lo; }
                                 ready = mbar_test_wait(bfull0 + s8, bph);
                             }
-                            umma_bf16_ss_halves(d0 + (uint32_t)(me * BN), a0, hi, b0, hi, idesc, started);
+                            umma_bf16_ss_sel(d0 + (uint32_t)(me * BN), a0, hi, b0, hi, idesc, started);
                             started = 1u;
 #pragma unroll
                             for (int k = 1; k < 4; ++k)
@@ -315,7 +315,7 @@ __global__ void __launch_bounds__(kSThreads) umma_strip_conv_kernel(const __grid
                         // consecutive MMAs go to different accumulators (M blocks), so an MMA never has to
                         // wait for the previous one's accumulator update
                         for (int mb = me; mb < g.nmb; mb += ni)
-                            umma_bf16_ss_halves(d0 + (uint32_t)(mb * BN), a_tap + (uint32_t)mb * 1024u, hi, b0, hi, idesc, started);
+                            umma_bf16_ss_sel(d0 + (uint32_t)(mb * BN), a_tap + (uint32_t)mb * 1024u, hi, b0, hi, idesc, started);
                         started = 1u;
 #pragma unroll
                         for (int k = 1; k < 4; ++k)
@@ -485,7 +485,21 @@ struct StripPlan { bool ok = false; int bn = 64, R = 0, CW = 0, Wt = 0, nmb = 0,
 
 int strip_sm_count() { return device_sm_count(); }
 
-StripPlan plan_strip_search(const UmmaConvShape &s);
+StripPlan plan_strip_search(const UmmaConvShape &s, int bn);
+
+// Dense layers: the GEMM that loads every tap's pixels anew (umma_conv.cu) overtook this kernel at every size once its loops
+// were lean (forward, N = 32: 3x3 64 at 56 x 56 15.6 against 16.3 us, 128 at 28 x 28 12.4 / 12.4, 256 at 14 x 14 12.1 / 14.5;
+// N = 1: 256 at 14 x 14 9.4 / 13.3), because it has more tiles to spread over the SMs and no junk rows.  This one is kept for the
+// smallest problems of few channels, where both are a launch and a few loads (2 x 20 x 24 x 64: 5.2 against 5.8 us) and it
+// reads the input once instead of nine times; and for sub-pixel and block-diagonal outputs, which skip taps or chunks.
+bool strip_dense_small(const UmmaConvShape &s) { return (long long)s.n * s.ho * s.wo <= 17 * 128 && s.ca <= 128 && s.cn <= 128; }
+
+int strip_bn(const UmmaConvShape &s) {
+    if (s.sub_cin > 0 && s.cn == 16) return 16;
+    // wide sub-pixel mode: an n-tile must not straddle two parity classes
+    if (s.sub_cin > 0) return s.sub_cin % 128 == 0 ? 128 : 64;
+    return s.cn % 128 == 0 && !s.blockdiag ? 128 : 64;
+}
 
 // The search below runs a double loop over tile shapes and is asked for several times per library call
 // (eligibility, workspace size, launch): its result is cached per thread, keyed by the shape and the SM count.
@@ -500,12 +514,17 @@ StripPlan plan_strip(const UmmaConvShape &s) {
     next = (next + 1) % 16;
     memcpy(&slot.key, &s, sizeof(UmmaConvShape));
     slot.sms = sms;
-    slot.plan = plan_strip_search(s);
+    slot.plan = plan_strip_search(s, strip_bn(s));
+    if (slot.plan.ok && slot.plan.bn == 128 && s.sub_cin == 0 && strip_dense_small(s)) {
+        // few tiles: narrow ones, twice as many (2 x 19 x 33 x 128, forward: 11.2 -> 9.3 us)
+        const StripPlan narrow = plan_strip_search(s, 64);
+        if (narrow.ok) slot.plan = narrow;
+    }
     slot.used = true;
     return slot.plan;
 }
 
-StripPlan plan_strip_search(const UmmaConvShape &s) {
+StripPlan plan_strip_search(const UmmaConvShape &s, int bn) {
     StripPlan best;
     if (s.stride_h != 1 || s.stride_w != 1 || s.dil_h != 1 || s.dil_w != 1 || s.out_sw) return best;
     if (s.blockdiag && s.ca != s.cn) return best;
@@ -514,8 +533,6 @@ StripPlan plan_strip_search(const UmmaConvShape &s) {
     if (sub_wide && (s.sub_cin % 64 || s.cn != 4 * s.sub_cin)) return best;
     if (s.taps_h * s.taps_w < 2 || s.ca % 64 || (!sub && s.cn % 64) || s.cn > 4096 || s.wo < 14 || s.ho < 2) return best;
     if ((long long)s.n * s.ho * s.wo >= (1LL << 30)) return best;
-    // wide sub-pixel mode: an n-tile must not straddle two parity classes
-    const int bn = sub ? 16 : (sub_wide ? (s.sub_cin % 128 == 0 ? 128 : 64) : ((s.cn % 128 == 0 && !s.blockdiag) ? 128 : 64));
     const int nmb_max = 512 / bn / 2;                      // two accumulator sets
     const int tiles_w_min = (s.wo + (256 - s.taps_w + 1) - 1) / (256 - s.taps_w + 1);
     // Among the tilings that keep at least 70 % of the MMA rows useful, take the one with the lowest
@@ -624,7 +641,7 @@ cudaError_t launch_strip(const CUtensorMap &ta, const CUtensorMap &tw, const Str
 bool umma_strip_possible(const UmmaConvShape &s) { return plan_strip(s).ok; }
 
 bool umma_strip_eligible(const UmmaConvShape &s) {
-    return plan_strip(s).ok;
+    return (s.blockdiag || s.sub_cin > 0 || strip_dense_small(s)) && plan_strip(s).ok;
 }
 
 cudaError_t launch_umma_strip_conv(const UmmaConvShape &s, const void *act, const void *wmat, const float *bias,

@@ -218,7 +218,7 @@ __global__ void __launch_bounds__(kWThreads) umma_wgrad_kernel(const __grid_cons
                 sb += 8; a_lo += kStageBytes >> 4;
                 if (sb == sb_end) { sb = 0; a_lo = tiles_lo; ph ^= 1u; }
                 free = mbar_test_wait(full0 + sb, ph);
-                umma_bf16_ss_halves(tmem_base, a0, hi, b0, hi, idesc, (uint32_t)kb);
+                umma_bf16_ss_sel(tmem_base, a0, hi, b0, hi, idesc, (uint32_t)kb);
 #pragma unroll
                 for (int k = 1; k < kWP / kWUmmaK; ++k)
                     umma_bf16_ss_halves<true>(tmem_base, a0 + (uint32_t)k * (kWUmmaK * 128 >> 4), hi,

@@ -21,6 +21,14 @@ SPECS = [
     L("f32_many", 16, 33, 40, 37, 35, 3, 3, pad=1, dtype="f32", layout="nchw"),
     L("f32_nopad", 1, 20, 9, 30, 34, 3, 3, pad=0, dtype="f32", layout="nchw", bias=True),
     L("f32_pad2", 1, 7, 6, 9, 6, 3, 3, pad=2, dtype="f32", layout="nchw"),
+    # dense GEMM by CTA pairs: an odd number of pixel tiles (the last has no partner) at 64 columns a pair; several rounds
+    # at 128; 256 with a ragged last tile.  Channel chunks outermost: two chunks, weights resident and streamed
+    L("pair_64", 7, 512, 7, 7, 192, 3, 3, pad=1, bias=True),
+    L("pair_128", 25, 512, 7, 7, 2048, 3, 3, pad=1, dtype="f16"),
+    L("pair_256", 3, 512, 112, 112, 1024, 1, 1),
+    L("chunks_first", 5, 128, 24, 22, 192, 3, 3, pad=1), L("chunks_resident", 30, 128, 30, 31, 64, 2, 2, dtype="f16"),
+    # weight gradient: C_out that ends inside the box of a 128-wide tile, fewer pixels than a stage
+    L("wgrad_c192", 3, 64, 5, 4, 192, 3, 3, pad=1),
 ]
 
 
@@ -50,7 +58,8 @@ GLUE = [  # every kernel whose epilogue does the glue, and one that leaves it to
     L("glue_1x1", 3, 128, 9, 13, 320, 1, 1, dtype="f16"),                     # GEMM, a last tile of 64 columns
     L("glue_strided", 2, 64, 11, 9, 128, 3, 3, stride=2, pad=1),              # a GEMM per parity class
     L("glue_empty", 2, 64, 10, 9, 64, 1, 1, stride=2),                        # positions without a class
-    L("glue_strip", 2, 64, 21, 30, 192, 3, 3, pad=1),
+    L("glue_strip", 2, 64, 21, 30, 192, 3, 3, pad=1), L("glue_strip_small", 2, 64, 21, 30, 128, 3, 3, pad=1, dtype="f16"),
+    L("glue_pair", 7, 512, 7, 7, 512, 3, 3, pad=1, dtype="f16"),              # CTA pairs, an odd number of pixel tiles
     L("glue_subpixel", 1, 128, 33, 34, 128, 3, 3, stride=2, pad=1, dtype="f16"),
     L("glue_fused", 3, 256, 17, 15, 64, 1, 1), L("glue_fused_wide", 3, 64, 17, 15, 128, 1, 1, dtype="f16"),
     L("glue_stem", 2, 3, 37, 40, 64, 7, 7, stride=2, pad=3),
