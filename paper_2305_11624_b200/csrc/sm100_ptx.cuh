@@ -377,6 +377,12 @@ __device__ __forceinline__ void tmem_st_32x32_x8(uint32_t taddr, const uint32_t 
                  ::"r"(taddr), "r"(v[0]), "r"(v[1]), "r"(v[2]), "r"(v[3]), "r"(v[4]), "r"(v[5]), "r"(v[6]), "r"(v[7])
                  : "memory");
 }
+// 16 lanes x 8 consecutive 32-bit columns: thread i holds columns i % 4 and 4 + i % 4 (v[0], v[1] and v[2], v[3]) of lanes
+// i / 4 and 8 + i / 4.
+__device__ __forceinline__ void tmem_st_16x128_x2(uint32_t taddr, const uint32_t (&v)[4]) {
+    asm volatile("tcgen05.st.sync.aligned.16x128b.x2.b32 [%0], {%1, %2, %3, %4};" ::"r"(taddr), "r"(v[0]), "r"(v[1]), "r"(v[2]), "r"(v[3])
+                 : "memory");
+}
 // D[tmem] (+)= A[smem] * B[smem] with the descriptors given as halves; ACC = false overwrites D.  CTAS = 2: the pair's
 // 256-row product, issued by its first CTA; the addresses hold in both.
 template <bool ACC, int CTAS = 1>

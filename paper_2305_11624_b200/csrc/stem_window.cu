@@ -15,6 +15,7 @@
 // (round-robin over output rows, disjoint accumulators), 12-23 drain accumulators: scale, shift, bf16,
 // swizzled staging, TMA store.  Every CTA owns a contiguous range of output rows.  Every wait is bounded.
 #include "kernels.h"
+#include "mma_sync.cuh"
 #include "sm100_ptx.cuh"
 
 namespace convbn {
@@ -322,33 +323,40 @@ __global__ void __launch_bounds__(kWinThreads) stem_window_fwd_kernel(const __gr
                             __syncwarp();
                         }
                         uint8_t *row = buf + lane * 128;
+                        // (type and ReLU fixed outside the loop over the columns)
+                        auto drain = [&](auto half_tag, auto relu_tag) {
+                            constexpr bool H = decltype(half_tag)::value, RELU = decltype(relu_tag)::value;
 #pragma unroll 1
-                        for (int half = 0; half < 2; ++half) {
-                            uint32_t v[32];
-                            if (live) {
+                            for (int half = 0; half < 2; ++half) {
+                                uint32_t v[32];
                                 tmem_ld_32x32(t_row + (uint32_t)(c0 + 32 * half), v);
                                 tmem_ld_wait();
-                            }
-                            if (half == 1 && c0 + 64 >= BN) {
-                                // every column of this accumulator has been read: hand it back
-                                tc_fence_before_sync();
-                                __syncwarp();
-                                if (lane == 0) mbar_arrive(&ctl->tmem_empty[slot]);
-                            }
-                            if (!live) continue;
 #pragma unroll
-                            for (int j = 0; j < 32; j += 8) {
-                                const int c = c0 + 32 * half + j;
-                                const float4 s0 = *(const float4 *)(scale_s + c), s1 = *(const float4 *)(scale_s + c + 4);
-                                const float4 b0 = *(const float4 *)(bias_s + c), b1 = *(const float4 *)(bias_s + c + 4);
-                                uint4 pk;
-                                pk.x = pack2_h16(fmaf(__uint_as_float(v[j]), s0.x, b0.x), fmaf(__uint_as_float(v[j + 1]), s0.y, b0.y), g.f16);
-                                pk.y = pack2_h16(fmaf(__uint_as_float(v[j + 2]), s0.z, b0.z), fmaf(__uint_as_float(v[j + 3]), s0.w, b0.w), g.f16);
-                                pk.z = pack2_h16(fmaf(__uint_as_float(v[j + 4]), s1.x, b1.x), fmaf(__uint_as_float(v[j + 5]), s1.y, b1.y), g.f16);
-                                pk.w = pack2_h16(fmaf(__uint_as_float(v[j + 6]), s1.z, b1.z), fmaf(__uint_as_float(v[j + 7]), s1.w, b1.w), g.f16);
-                                if (g.relu) { pk.x = relu2_h16(pk.x); pk.y = relu2_h16(pk.y); pk.z = relu2_h16(pk.z); pk.w = relu2_h16(pk.w); }
-                                *(uint4 *)(row + (((4 * half + (j >> 3)) ^ (lane & 7)) << 4)) = pk;
+                                for (int j = 0; j < 32; j += 8) {
+                                    const int c = c0 + 32 * half + j;
+                                    const float4 s0 = *(const float4 *)(scale_s + c), s1 = *(const float4 *)(scale_s + c + 4);
+                                    const float4 b0 = *(const float4 *)(bias_s + c), b1 = *(const float4 *)(bias_s + c + 4);
+                                    uint4 pk;
+                                    pk.x = pack2_t<H>(fmaf(__uint_as_float(v[j]), s0.x, b0.x), fmaf(__uint_as_float(v[j + 1]), s0.y, b0.y));
+                                    pk.y = pack2_t<H>(fmaf(__uint_as_float(v[j + 2]), s0.z, b0.z), fmaf(__uint_as_float(v[j + 3]), s0.w, b0.w));
+                                    pk.z = pack2_t<H>(fmaf(__uint_as_float(v[j + 4]), s1.x, b1.x), fmaf(__uint_as_float(v[j + 5]), s1.y, b1.y));
+                                    pk.w = pack2_t<H>(fmaf(__uint_as_float(v[j + 6]), s1.z, b1.z), fmaf(__uint_as_float(v[j + 7]), s1.w, b1.w));
+                                    if constexpr (RELU) { pk.x = relu2_h16(pk.x); pk.y = relu2_h16(pk.y); pk.z = relu2_h16(pk.z); pk.w = relu2_h16(pk.w); }
+                                    *(uint4 *)(row + (((4 * half + (j >> 3)) ^ (lane & 7)) << 4)) = pk;
+                                }
                             }
+                        };
+                        if (live) {
+                            constexpr std::true_type yes{};
+                            constexpr std::false_type no{};
+                            if (g.f16) { if (g.relu) drain(yes, yes); else drain(yes, no); }
+                            else { if (g.relu) drain(no, yes); else drain(no, no); }
+                        }
+                        if (c0 + 64 >= BN) {
+                            // every column of this accumulator has been read: hand it back
+                            tc_fence_before_sync();
+                            __syncwarp();
+                            if (lane == 0) mbar_arrive(&ctl->tmem_empty[slot]);
                         }
                         if (!live) continue;
                         fence_proxy_async_smem();
@@ -510,9 +518,14 @@ __global__ void __launch_bounds__(kWgThreads) stem_window_wgrad_kernel(const __g
         // the pair's row m >> 6; 16 pixels are 8 columns of two 16-bit elements.  (Read from tensor memory, the tile costs
         // the MMAs no shared-memory bandwidth: every pair meets up to 2 (T + 1) input rows.) ----------------
         const int q4 = (warp - (kWgLoaders + 4)) & 3, group = (warp - (kWgLoaders + 4)) >> 2;
-        const int m = 32 * q4 + lane, half = m >> 6, co = m & 63;
+        const int half = q4 >> 1;
         const uint32_t t_lane = tmem_base + ((uint32_t)(32 * q4) << 16) + (uint32_t)kWgAccCols;
-        const uint32_t in_row = (uint32_t)(co & 7) * 2u;       // byte of the channel inside its 16-byte chunk
+        // An 8 x 8 block (pixels x channels) read transposed leaves pixels 2 (l % 4), 2 (l % 4) + 1 of channel l / 4 in lane l:
+        // the layout in which 16 lanes x 4 columns are stored.  Lane l addresses row l % 8 of block l / 8: blocks 0, 1 are
+        // channels 0-7, 8-15 of the 16, blocks 2, 3 the same of the next 8 pixels.  (By 16-bit loads, a lane per channel,
+        // this was the kernel's longest chain; 51.9 -> 50.4 us at 64 x 112 x 112 x 64.)
+        const uint32_t bpx = (uint32_t)(lane & 7) + (uint32_t)(lane >> 4) * 8u, bch = (uint32_t)(q4 & 1) * 4u + (uint32_t)((lane >> 3) & 1);
+        const uint32_t off0 = bpx * 128u + (((bch ^ (bpx & 7u)) & 7u) << 4), off1 = bpx * 128u + ((((bch + 2u) ^ (bpx & 7u)) & 7u) << 4);
         long long cur = row_lo;
         WinChunk ck;
         int sb = 0, slot = 0;
@@ -532,17 +545,15 @@ __global__ void __launch_bounds__(kWgThreads) stem_window_wgrad_kernel(const __g
                 const bool have = i + half < ck.rows;           // an odd last pair has no second row: zeros
                 const uint8_t *rowb = dzs + (size_t)sb * dzstrip + (size_t)(have ? i + half : 0) * g.dzrow_bytes;
                 const uint32_t t0 = t_lane + (uint32_t)slot * slot_cols;
+                const uint32_t row_addr = smem_u32(rowb);
                 for (int k = group; k < g.ksteps; k += kWgMovers / 4) {
-                    uint32_t v[8];
-#pragma unroll
-                    for (int c = 0; c < 8; ++c) {
-                        // pixels 16 k + 2 c and the next one; rows are 128-byte swizzled: chunk (co / 8) ^ (pixel & 7)
-                        const uint32_t p0 = (uint32_t)(16 * k + 2 * c);
-                        const uint32_t lo = *(const uint16_t *)(rowb + p0 * 128u + ((((uint32_t)(co >> 3) ^ (p0 & 7u)) & 7u) << 4) + in_row);
-                        const uint32_t hi = *(const uint16_t *)(rowb + (p0 + 1u) * 128u + ((((uint32_t)(co >> 3) ^ ((p0 + 1u) & 7u)) & 7u) << 4) + in_row);
-                        v[c] = have ? (lo | (hi << 16)) : 0u;
+                    uint32_t v0[4] = {0u, 0u, 0u, 0u}, v1[4] = {0u, 0u, 0u, 0u};
+                    if (have) {
+                        ldmatrix_x4_trans(v0[0], v0[1], v0[2], v0[3], row_addr + (uint32_t)k * 2048u + off0);
+                        ldmatrix_x4_trans(v1[0], v1[1], v1[2], v1[3], row_addr + (uint32_t)k * 2048u + off1);
                     }
-                    tmem_st_32x32_x8(t0 + 8u * (uint32_t)k, v);
+                    tmem_st_16x128_x2(t0 + 8u * (uint32_t)k, v0);
+                    tmem_st_16x128_x2(t0 + 8u * (uint32_t)k + (16u << 16), v1);
                 }
                 tmem_st_wait();
                 tc_fence_before_sync();
