@@ -91,11 +91,19 @@ __global__ void __launch_bounds__(kFbThreads) fused_bwd1x1_kernel(const __grid_c
         const uint32_t one2 = one_h16(g.f16) * 0x10001u;
         const uint4 one4 = make_uint4(one2, one2, one2, one2);
         for (int i = threadIdx.x; i < 1024 / 16; i += kFbThreads) ((uint4 *)ones)[i] = one4;
+        fence_proxy_async_smem();
     }
+    tc_fence_before_sync();
+    __syncthreads();
+    tc_fence_after_sync();
     pdl_wait();
+    pdl_launch_dependents();       // not earlier than here: this CTA owns its tensor-memory columns
+    const uint32_t tmem_base = ctl->tmem_base;
+
+    if (warp != 0) {               // (the first boxes are under way meanwhile)
     // omega' = s omega (Sec. 3.3), one rounding to bf16, laid out as the MN-major B operand of the data-gradient
     // GEMM: K = co rows of 128 bytes (64 ci), 128-byte swizzle, one block per 64 input channels
-    for (int i = threadIdx.x; i < CO * (CI / 8); i += kFbThreads) {
+    for (int i = (int)threadIdx.x - 32; i < CO * (CI / 8); i += kFbThreads - 32) {
         const int co = i / (CI / 8), c8 = i - co * (CI / 8), ci = c8 * 8;
         const float sc = g.vec3[co];
         const uint4 raw = __ldg((const uint4 *)(w + (size_t)co * CI + ci));
@@ -110,30 +118,27 @@ __global__ void __launch_bounds__(kFbThreads) fused_bwd1x1_kernel(const __grid_c
             make_uint4(out[0], out[1], out[2], out[3]);
     }
     fence_proxy_async_smem();
-    tc_fence_before_sync();
-    __syncthreads();
-    tc_fence_after_sync();
-    pdl_launch_dependents();       // only now: this CTA owns its tensor-memory columns
-    const uint32_t tmem_base = ctl->tmem_base;
+    named_bar_sync(1, kFbThreads - 32);
+    }
 
     if (warp == 0) {
         // ---------------- producer: the dZ boxes, then the X boxes of a tile ----------------
         int s = 0, issued = 0;
         uint32_t ph = 0;
         bool ok = true;
-        for (int t = tile_lo; t < tile_hi; ++t) {
-            ok = __all_sync(0xffffffffu, mbar_wait_bounded(&ctl->empty[s], ph ^ 1u, abort_flag));
-            if (!ok) break;
-            uint8_t *dst = stages + (size_t)s * S::kStageBytes;
-            if (lane == 0) mbar_arrive_expect_tx(&ctl->full[s], S::kStageBytes);
-            __syncwarp();
-            if (lane < S::kDzBoxes) tma_load_2d(dst + (size_t)lane * kFbBox, &tm_dz, &ctl->full[s], lane * 64, t * 128);
-            else if (lane < S::kDzBoxes + S::kXBoxes)
-                tma_load_2d(dst + (size_t)lane * kFbBox, &tm_x, &ctl->full[s], (lane - S::kDzBoxes) * 64, t * 128);
-            ++issued;
-            if (++s == kFbStages) { s = 0; ph ^= 1u; }
+        if (elect_one()) {
+            for (int t = tile_lo; t < tile_hi; ++t) {
+                ok = mbar_wait_bounded(&ctl->empty[s], ph ^ 1u, abort_flag);
+                if (!ok) break;
+                uint8_t *dst = stages + (size_t)s * S::kStageBytes;
+                mbar_arrive_expect_tx(&ctl->full[s], S::kStageBytes);
+                tma_load_3d(dst, &tm_dz, &ctl->full[s], 0, t * 128, 0);
+                tma_load_3d(dst + (size_t)S::kDzBoxes * kFbBox, &tm_x, &ctl->full[s], 0, t * 128, 0);
+                ++issued;
+                if (++s == kFbStages) { s = 0; ph ^= 1u; }
+            }
         }
-        if (!ok && lane == 0) {
+        if (!ok) {
             atomicOr(err, ERRW_TIMEOUT);
             ctl->abort_flag = 1;
             for (int j = issued > kFbStages ? issued - kFbStages : 0; j < issued; ++j)
@@ -389,8 +394,14 @@ cudaError_t launch_fused_bwd1x1(const Problem &pb, const void *dz, const void *x
     g.post_mask = post ? (const __nv_bfloat16 *)post->mask : nullptr;
     g.post_relu = post ? post->relu : 0;
     CUtensorMap tdz, tx, tdx;
-    if (!make_tmap_matrix_bf16(&tdz, dz, pb.p, pb.c_out, 128, 64)) return cudaErrorInvalidValue;
-    if (!make_tmap_matrix_bf16(&tx, x, pb.p, pb.c_in, 128, 64)) return cudaErrorInvalidValue;
+    // a tile's [128 pixels][64 channels] blocks, side by side in shared memory, are one box of each tensor
+    auto blocks = [&](CUtensorMap *tm, const void *base, int c) {
+        const unsigned long long dims[3] = {64, (unsigned long long)pb.p, (unsigned long long)c / 64};
+        const unsigned long long str[3] = {0, (unsigned long long)c * 2, 128};
+        const unsigned int box[3] = {64, 128, (unsigned int)c / 64};
+        return make_tmap_tiled_bf16(tm, base, 3, dims, str, box);
+    };
+    if (!blocks(&tdz, dz, pb.c_out) || !blocks(&tx, x, pb.c_in)) return cudaErrorInvalidValue;
     if (!make_tmap_matrix_bf16(&tdx, dx, pb.p, pb.c_in, 32, 64)) return cudaErrorInvalidValue;
     int *err = nullptr;
     cudaError_t e = error_word_address(&err);

@@ -33,6 +33,7 @@ struct ConvGemm {
     int cn;                  // output channels (GEMM N)
     int ca;                  // activation channels (multiple of 64)
     int taps_h, taps_w;
+    int nbuf;                // staging buffers per epilogue warp: 1 or 2
     int chunk_outer;         // order of K: 1: channel chunk by chunk, all taps of each; 0: tap by tap, all chunks of each
     int lower_h, lower_w;    // input coordinate read by output (0,0) at tap (0,0)
     int stride_h, stride_w, dil_h, dil_w;
@@ -108,9 +109,9 @@ __global__ void __launch_bounds__(MODE == kPlain || MODE == kTap ? 512 : kConvTh
     const uint32_t kStageBytes = g.resident ? kABytes : kABytes + kBBytes;
     uint8_t *tiles = (uint8_t *)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
     uint8_t *slab = tiles + (size_t)g.stages * kStageBytes;            // resident weights: num_kb x [BN][64]
-    uint8_t *staging = slab + (g.resident ? (size_t)num_kb * kBBytes : 0);   // 8 warps x 2 x [32 rows][128 B]
+    uint8_t *staging = slab + (g.resident ? (size_t)num_kb * kBBytes : 0);   // 8 warps x nbuf x [32 rows][128 B]
     const int extra = POST ? (g.post_add != nullptr) + (g.post_mask != nullptr) : 0;     // staging areas of the other tensors
-    ConvSmemCtl *ctl = (ConvSmemCtl *)(staging + (size_t)(1 + extra) * kStagingBytes);
+    ConvSmemCtl *ctl = (ConvSmemCtl *)(staging + (size_t)(g.nbuf + extra) * kStagingBytes);
     float *bias_s = (float *)(((uintptr_t)(ctl + 1) + 15) & ~(uintptr_t)15);   // cn floats
     float *scale_s = bias_s + g.cn;                                            // cn floats (fold mode)
     float *shift_s = scale_s + g.cn;                                           // cn floats (DUAL)
@@ -153,41 +154,17 @@ __global__ void __launch_bounds__(MODE == kPlain || MODE == kTap ? 512 : kConvTh
         tmem_alloc<CTAS>(&ctl->tmem_base, 2 * BN);
         tmem_relinquish<CTAS>();
     }
-    // Everything above touched only this CTA's own shared / tensor memory.  Global memory (inputs that
-    // an earlier kernel may still be writing, outputs it may still be reading) comes after this wait.
     // the tensor maps are kernel parameters, not data of an earlier kernel: fetch them before the wait
     if (threadIdx.x == 0) { prefetch_tensormap(&tm_act); prefetch_tensormap(&tm_w); prefetch_tensormap(&tm_out); }
-    pdl_wait();
-    if (threadIdx.x == 0) CONVBN_TRACE_POINT(1);
-    const int pc = TAP ? g.tap_c : g.cn;               // channels the per-channel parameters belong to
-    if constexpr (DUAL) {
-        for (int c = threadIdx.x; c < g.cn; c += kConvThreads) {
-            const float sc = g.fold.gamma[c] * (1.0f / sqrtf(g.fold.var[c] + g.fold.eps));
-            bias_s[c] = g.fold.b ? g.fold.b[c] : 0.f;
-            scale_s[c] = sc;
-            shift_s[c] = g.fold.beta[c] - g.fold.mean[c] * sc;
-        }
-    } else if (fold) {
-        // On-the-fly reparameterisation (Sec. 3.3 / 3.4): s = gamma / sqrt(var + eps), b' = (b - mu) s + beta.
-        // s multiplies the fp32 accumulator (the associative law of Sec. 3.2.2), so omega is used unrounded.
-        for (int c = threadIdx.x; c < pc; c += kConvThreads) {
-            const float r = 1.0f / sqrtf(g.fold.var[c] + g.fold.eps);
-            const float sc = g.fold.gamma[c] * r;
-            const float bf = ((g.fold.b ? g.fold.b[c] : 0.f) - g.fold.mean[c]) * sc + g.fold.beta[c];
-            scale_s[c] = sc;
-            bias_s[c] = bf;
-            if (blockIdx.x == 0 && g.fold.vec3) {
-                g.fold.vec3[c] = sc; g.fold.vec3[pc + c] = bf; g.fold.vec3[2 * pc + c] = r;
-            }
-        }
-    } else if (bias) {
-        for (int c = threadIdx.x; c < g.cn; c += kConvThreads) bias_s[c] = bias[c];
-    }
     tc_fence_before_sync();
     __syncthreads();
     if constexpr (PAIR) cluster_sync_all();                 // both CTAs' barriers and columns are there
     tc_fence_after_sync();
-    pdl_launch_dependents();       // only now: this CTA owns its tensor-memory columns
+    // Everything above touched only this CTA's own shared / tensor memory.  Global memory (inputs that
+    // an earlier kernel may still be writing, outputs it may still be reading) comes after this wait.
+    pdl_wait();
+    if (threadIdx.x == 0) CONVBN_TRACE_POINT(1);
+    pdl_launch_dependents();       // not earlier than here: this CTA owns its tensor-memory columns
     const uint32_t tmem_base = ctl->tmem_base;
     if (threadIdx.x == 0) CONVBN_TRACE_POINT(2);
 
@@ -388,14 +365,49 @@ __global__ void __launch_bounds__(MODE == kPlain || MODE == kTap ? 512 : kConvTh
     } else {
         // ---------------- epilogue: tensor memory -> registers -> bf16 -> shared -> TMA store --------
         // Two groups of four warps; group e drains accumulator buffer e, i.e. every other tile of this
-        // CTA, so two tiles are in their epilogue at once.  Each warp owns 32 accumulator rows and two
+        // CTA, so two tiles are in their epilogue at once.  Each warp owns 32 accumulator rows and one or two
         // private [32 rows][64 columns] staging buffers (128-byte swizzle): warp-level sync only.
+        // First the per-channel parameters, by these warps alone: the loads and the first MMAs do not wait for them.
+        const int pc = TAP ? g.tap_c : g.cn;               // channels the per-channel parameters belong to
+        if constexpr (DUAL) {
+            for (int c = (int)threadIdx.x - 64; c < g.cn; c += 256) {
+                const float sc = g.fold.gamma[c] * (1.0f / sqrtf(g.fold.var[c] + g.fold.eps));
+                bias_s[c] = g.fold.b ? g.fold.b[c] : 0.f;
+                scale_s[c] = sc;
+                shift_s[c] = g.fold.beta[c] - g.fold.mean[c] * sc;
+            }
+        } else if (fold) {
+            // On-the-fly reparameterisation (Sec. 3.3 / 3.4): s = gamma / sqrt(var + eps), b' = (b - mu) s + beta.
+            // s multiplies the fp32 accumulator (the associative law of Sec. 3.2.2), so omega is used unrounded.
+            for (int c = (int)threadIdx.x - 64; c < pc; c += 256) {
+                const float r = 1.0f / sqrtf(g.fold.var[c] + g.fold.eps);
+                const float sc = g.fold.gamma[c] * r;
+                const float bf = ((g.fold.b ? g.fold.b[c] : 0.f) - g.fold.mean[c]) * sc + g.fold.beta[c];
+                scale_s[c] = sc;
+                bias_s[c] = bf;
+                if (blockIdx.x == 0 && g.fold.vec3) {
+                    g.fold.vec3[c] = sc; g.fold.vec3[pc + c] = bf; g.fold.vec3[2 * pc + c] = r;
+                }
+            }
+        } else if (bias) {
+            for (int c = (int)threadIdx.x - 64; c < g.cn; c += 256) bias_s[c] = bias[c];
+        }
+        named_bar_sync(1, 256);
         const int quarter = warp & 3;                      // tensor-memory lanes this warp may read
         const uint32_t egroup = (uint32_t)(warp - 2) >> 2; // 0: warps 2-5, 1: warps 6-9
         uint8_t *stage_buf = staging + (size_t)(warp - 2) * kStagingWarpBytes;
+        // the buffer for the next box: the last store from it has been read, an earlier one (nbuf = 2) may still be under way
+        uint32_t turn = 0;
+        auto next_buf = [&]() -> uint8_t * {
+            if (lane == 0) { if (MODE == kPlain && g.nbuf == 2) tma_store_wait_read<1>(); else tma_store_wait_read<0>(); }
+            __syncwarp();
+            uint8_t *b = stage_buf + turn;
+            if (MODE == kPlain && g.nbuf == 2) turn ^= kStagingBytes;
+            return b;
+        };
         uint32_t mt, nt;
         // kPost: tm_out2 is the addend's map.  One box of each tensor in flight per warp.
-        uint8_t *add_buf = stage_buf + kStagingBytes, *mask_buf = add_buf + (g.post_add ? kStagingBytes : 0);
+        uint8_t *add_buf = staging + (size_t)g.nbuf * kStagingBytes + (size_t)(warp - 2) * kStagingWarpBytes, *mask_buf = add_buf + (g.post_add ? kStagingBytes : 0);
         uint32_t post_ph = 0;
         bool post_pending = false;
         auto fetch_post = [&](uint32_t ti, int c0) {          // chunk c0 of tile ti of this CTA, if there is one
@@ -458,11 +470,7 @@ __global__ void __launch_bounds__(MODE == kPlain || MODE == kTap ? 512 : kConvTh
                     }
                 }
                 if (c0 < ncols) {
-                    uint8_t *buf = stage_buf;
-                    // the previous store read this buffer: wait until it no longer does (shared memory
-                    // is better spent on ring slots than on a second staging buffer)
-                    if (lane == 0) tma_store_wait_read<0>();
-                    __syncwarp();
+                    uint8_t *buf = next_buf();
                     uint8_t *row = buf + lane * 128;
                     if constexpr (POST) {
                         if (post_pending) {
@@ -600,8 +608,8 @@ __global__ void __launch_bounds__(MODE == kPlain || MODE == kTap ? 512 : kConvTh
                             }
                         };
                         if (g.f16) normalise(std::true_type{}); else normalise(std::false_type{});
-                        if (lane == 0) tma_store_wait_read<0>();
-                        __syncwarp();
+                        buf = next_buf();
+                        row = buf + lane * 128;
 #pragma unroll
                         for (int j = 0; j < 8; ++j) *(uint4 *)(row + (((j ^ (lane & 7)) & 7) << 4)) = zq[j];
                         fence_proxy_async_smem();
@@ -747,8 +755,11 @@ static cudaError_t launch_bn(const CUtensorMap &ta, const CUtensorMap &tw, const
                              cudaStream_t st) {
     const size_t a_bytes = (size_t)kBM * kBK * 2, b_bytes = (size_t)BN * kBK * 2 / (PAIR ? 2 : 1);
     const int extra = MODE == kPost ? (g.post_add != nullptr) + (g.post_mask != nullptr) : 0;
-    size_t fixed = 1024 + (size_t)(1 + extra) * kStagingBytes + sizeof(ConvSmemCtl) + (MODE == kDual ? 3 : 2) * (size_t)g.cn * sizeof(float) + 16;
     const int num_kb = g.taps_h * g.taps_w * (g.blockdiag ? 1 : g.ca / kBK);
+    // Short K: the epilogues bound the kernel, and the second buffer is worth more than the ring slots it takes (1x1 256 -> 64
+    // at 56 x 56, N = 256, forward 86.4 -> 82.6 us; the other modes, with staging areas of their own, gain nothing).
+    g.nbuf = MODE == kPlain && num_kb <= 8 ? 2 : 1;
+    size_t fixed = 1024 + (size_t)(g.nbuf + extra) * kStagingBytes + sizeof(ConvSmemCtl) + (MODE == kDual ? 3 : 2) * (size_t)g.cn * sizeof(float) + 16;
     const long long m_tiles = (g.p + kBM - 1) / kBM, n_tiles = (g.cn + BN - 1) / BN;
     long long grid_l = m_tiles * n_tiles < sm_count() ? m_tiles * n_tiles : sm_count();
     if (PAIR) {
