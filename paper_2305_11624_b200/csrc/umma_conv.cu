@@ -82,16 +82,18 @@ struct ConvSmemCtl {
 // of the kernels beside it fits next to a CTA: 3x3 512 -> 512 at 7 x 7, N = 64, forward + backward 85 -> 93 us.  The
 // bound of 512 threads holds the plain kernel to 128 registers for the same reason.)
 // MODE kTap: the transposed convolution of ConvGemm::tap_c.
+// MODE kRelu: the plain kernel with max(., 0) at the end (by kPost, with its 168 registers, 64 -> 256 at 56 x 56, N = 32 took 20.4 us, now
+// 16.7; 512 -> 128 at 28 x 28 9.3 and 8.2).
 // MODE kPost: post_add, post_relu, post_mask follow.  A warp's [32 rows][64 columns] of the other tensors are brought into
 // buffers of their own by TMA, the next one while this one is used (read from global memory beside the stores, the
 // 64 -> 256 layer at 56 x 56, N = 32 took 90 us with an addend).  MODE kPostStrided: the same for strided outputs, whose
 // rows are no box: read from global memory.
-enum ConvMode { kPlain, kDual, kTap, kPost, kPostStrided };
+enum ConvMode { kPlain, kDual, kTap, kPost, kPostStrided, kRelu };
 //
 // PAIR: two CTAs of a cluster share a 256 x BN product (cta_group::2).  Each brings its own 128 pixels and HALF of the
 // weight tile, and gets the accumulator of its own pixels; the first CTA issues the MMAs of both (see pick_tile for what that gains).
 template <int BN, ConvMode MODE, bool PAIR>
-__global__ void __launch_bounds__(MODE == kPlain || MODE == kTap ? 512 : kConvThreads) umma_conv_kernel(const __grid_constant__ CUtensorMap tm_act,
+__global__ void __launch_bounds__(MODE == kPlain || MODE == kRelu || MODE == kTap ? 512 : kConvThreads) umma_conv_kernel(const __grid_constant__ CUtensorMap tm_act,
                                                                 const __grid_constant__ CUtensorMap tm_w,
                                                                 const __grid_constant__ CUtensorMap tm_out,
                                                                 const __grid_constant__ CUtensorMap tm_out2,
@@ -399,10 +401,10 @@ __global__ void __launch_bounds__(MODE == kPlain || MODE == kTap ? 512 : kConvTh
         // the buffer for the next box: the last store from it has been read, an earlier one (nbuf = 2) may still be under way
         uint32_t turn = 0;
         auto next_buf = [&]() -> uint8_t * {
-            if (lane == 0) { if (MODE == kPlain && g.nbuf == 2) tma_store_wait_read<1>(); else tma_store_wait_read<0>(); }
+            if (lane == 0) { if ((MODE == kPlain || MODE == kRelu) && g.nbuf == 2) tma_store_wait_read<1>(); else tma_store_wait_read<0>(); }
             __syncwarp();
             uint8_t *b = stage_buf + turn;
-            if (MODE == kPlain && g.nbuf == 2) turn ^= kStagingBytes;
+            if ((MODE == kPlain || MODE == kRelu) && g.nbuf == 2) turn ^= kStagingBytes;
             return b;
         };
         uint32_t mt, nt;
@@ -507,6 +509,10 @@ __global__ void __launch_bounds__(MODE == kPlain || MODE == kTap ? 512 : kConvTh
                             pk.z = pack2_t<H>(f[4], f[5]);
                             pk.w = pack2_t<H>(f[6], f[7]);
                             const int at16 = (((j >> 3) ^ (lane & 7)) & 7) << 4;
+                            if constexpr (MODE == kRelu) {
+                                const uint4 none = make_uint4(0u, 0u, 0u, 0u);
+                                pk = post_chunk<H>(pk, false, none, true, false, none);
+                            }
                             if constexpr (POST) {
                                 uint4 a4 = make_uint4(0u, 0u, 0u, 0u), m4 = a4;
                                 if constexpr (ADD) a4 = *(const uint4 *)(add_buf + lane * 128 + at16);
@@ -524,8 +530,8 @@ __global__ void __launch_bounds__(MODE == kPlain || MODE == kTap ? 512 : kConvTh
                     constexpr std::false_type no{};
                     if constexpr (!POST) pack(no, no, no);
                     else if (g.post_mask) { if (g.post_add) pack(yes, no, yes); else pack(no, no, yes); }
-                    else if (g.post_add) { if (g.post_relu) pack(yes, yes, no); else pack(yes, no, no); }
-                    else pack(no, yes, no);
+                    else if (g.post_relu) pack(yes, yes, no);
+                    else pack(yes, no, no);
                     if constexpr (POST) {
                         __syncwarp();                          // every lane has read its rows of the boxes
                         if (c0 + 64 < ncols) fetch_post(i, c0 + 64); else fetch_post(i + 2, 0);
@@ -758,7 +764,7 @@ static cudaError_t launch_bn(const CUtensorMap &ta, const CUtensorMap &tw, const
     const int num_kb = g.taps_h * g.taps_w * (g.blockdiag ? 1 : g.ca / kBK);
     // Short K: the epilogues bound the kernel, and the second buffer is worth more than the ring slots it takes (1x1 256 -> 64
     // at 56 x 56, N = 256, forward 86.4 -> 82.6 us; the other modes, with staging areas of their own, gain nothing).
-    g.nbuf = MODE == kPlain && num_kb <= 8 ? 2 : 1;
+    g.nbuf = (MODE == kPlain || MODE == kRelu) && num_kb <= 8 ? 2 : 1;
     size_t fixed = 1024 + (size_t)(g.nbuf + extra) * kStagingBytes + sizeof(ConvSmemCtl) + (MODE == kDual ? 3 : 2) * (size_t)g.cn * sizeof(float) + 16;
     const long long m_tiles = (g.p + kBM - 1) / kBM, n_tiles = (g.cn + BN - 1) / BN;
     long long grid_l = m_tiles * n_tiles < sm_count() ? m_tiles * n_tiles : sm_count();
@@ -793,7 +799,7 @@ template <ConvMode MODE>
 static cudaError_t launch_mode(int bn, bool pair, const CUtensorMap &ta, const CUtensorMap &tw, const CUtensorMap &tout,
                                const CUtensorMap &tout2, const CUtensorMap &tmask, const ConvGemm &g, const float *bias,
                                int *err, cudaStream_t st) {
-    if constexpr (MODE == kPlain || MODE == kPost) {
+    if constexpr (MODE == kPlain || MODE == kRelu || MODE == kPost) {
         if (pair && bn == 64) return launch_bn<64, MODE, true>(ta, tw, tout, tout2, tmask, g, bias, err, st);
         if (pair && bn == 128) return launch_bn<128, MODE, true>(ta, tw, tout, tout2, tmask, g, bias, err, st);
         if (pair) return launch_bn<256, MODE, true>(ta, tw, tout, tout2, tmask, g, bias, err, st);
@@ -875,6 +881,7 @@ cudaError_t launch_umma_conv(const UmmaConvShape &s, const void *act, const void
     if (with_post && !s.out_sw) {
         if (g.post_add && !make_tmap_matrix_bf16(&tout2, post->add, g.p, s.cn, 32, 64)) return cudaErrorInvalidValue;
         if (g.post_mask && !make_tmap_matrix_bf16(&tmask, post->mask, g.p, s.cn, 32, 64)) return cudaErrorInvalidValue;
+        if (!g.post_add && !g.post_mask) return launch_mode<kRelu>(bn, pair, ta, tw, tout, tout2, tmask, g, bias, err, st);
         return launch_mode<kPost>(bn, pair, ta, tw, tout, tout2, tmask, g, bias, err, st);
     }
     if (with_post) return launch_mode<kPostStrided>(bn, pair, ta, tw, tout, tout2, tmask, g, bias, err, st);
