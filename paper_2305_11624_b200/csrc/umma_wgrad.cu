@@ -296,12 +296,17 @@ UmmaWgradPlan umma_wgrad_plan(const Problem &pb) {
     const int bn = bd ? 64 : wgrad_bn(pb);
     const long long kd = bd ? (long long)pb.kh * pb.kw * 64 : pb.kdim;
     const long long m_tiles = (kd / 64 + 1 + 1) / 2, n_tiles = (pb.c_out + bn - 1) / bn;   // + the ones slice
-    // Resident CTAs: two per SM (the stage rings are sized for it, launch_w), which measured 25-40 % faster than one
-    // CTA with a deeper ring.
+    // Resident CTAs: two per SM (the stage rings are sized for it, launch_w): one's partial tile leaves while the other
+    // multiplies.  A deeper ring for one CTA gains nothing.
     // The slice count minimises  rounds over the resident slots x (pixels per slice + a fixed cost per
     // CTA, in pixels) + a small cost per slice for the epilogue that adds the slices up; a grid a few
     // CTAs larger than the slots would otherwise run a second, nearly empty round.
-    const long long slots = (long long)device_sm_count() * 2, tiles = m_tiles * n_tiles;
+    // Few tiles mean many slices, and where those are short the partial tensors weigh more than what a second CTA hides: up to
+    // 24 tiles with slices of up to 2048 pixels get one CTA per SM (N = 32: 1x1 128 -> 512 at 28 x 28 15.3 -> 13.4 us, 1024 ->
+    // 256 at 14 x 14 13.3 -> 11.4, 3x3 128 at 28 x 28 17.6 -> 15.5; but 3x3 256 at 14 x 14, 38 tiles, 15.8 -> 18.1, and 1x1
+    // 128 -> 512 at 28 x 28, N = 256 58.3 -> 73.6).
+    const long long tiles = m_tiles * n_tiles, sms = device_sm_count();
+    const long long slots = sms * (tiles <= 24 && pb.p * tiles <= 2048 * sms ? 1 : 2);
     const long long max_splits = (pb.p + 4 * kWP - 1) / (4 * kWP);     // at least 256 pixels per slice
     long long splits = 1;
     double best_cost = -1.0;
