@@ -811,7 +811,7 @@ static cudaError_t launch_mode(int bn, bool pair, const CUtensorMap &ta, const C
 
 // Tile width, and whether CTAs work in pairs: the least time by a model of clocks fitted to 24 layers (3x3 and 1x1, 64 to
 // 2048 channels, N = 8 to 256, both directions) at all six choices.  A round of tiles takes the larger of its k-blocks and
-// its epilogue; the last tile's epilogue and a pair's start-up (a cluster launch, two CTAs meeting twice) come on top.  A
+// its epilogue (1x1 64 -> 256 at 56 x 56, N = 256: 86.5 us with 128 columns, 95 with 256); the last tile's epilogue and a pair's start-up (a cluster launch, two CTAs meeting twice) come on top.  A
 // k-block costs a CTA of a pair 20 to 90 clocks less, being half a weight tile to write to and read from shared memory, so
 // pairs pay for long K or many rounds.  Forward, against the better of the unpaired widths: 3x3 512 -> 512 at 7 x 7, N = 256
 // 51.8 -> 45.8 us, N = 32 16.1 -> 15.3; 1x1 512 -> 1024 at 28 x 28, N = 256 227 -> 216.5 (back: 215.5 -> 182); but
@@ -827,8 +827,8 @@ static TilePick pick_tile(long long tiles_m, int cn, int num_kb, bool pairs, int
             if (bn > max_bn || (bn > 64 && cn <= bn / 2)) continue;
             const long long n_tiles = (cn + bn - 1) / bn, slots = pr ? sm_count() / 2 : sm_count();
             const long long rounds = ((pr ? (tiles_m + 1) / 2 : tiles_m) * n_tiles + slots - 1) / slots;
-            const double mma = num_kb * clk[pr][c], epi = 9.0 * bn;
-            const double cost = (double)rounds * ((mma > epi ? mma : epi) + 220.0) + 6.0 * bn + (pr ? 2100.0 : 0.0);
+            const double mma = num_kb * clk[pr][c], epi = bn * (bn == 64 ? 17.0 : (bn == 128 ? 14.7 : 16.0));
+            const double cost = (double)rounds * ((mma > epi ? mma : epi) + 220.0) + 6.0 * bn + (pr ? 1900.0 : 0.0);
             if (cost < best_cost) { best_cost = cost; best = TilePick{bn, pr != 0}; }
         }
     return best;
