@@ -119,7 +119,7 @@ struct Plan {
     size_t part_g = 0;     // [bsplits][C_out] fp32 (Eval backward)
     size_t dy = 0;         // Eval backward: s dZ, storage dtype
     size_t vec3 = 0;       // Eval forward: [s | beta - mean s | r]
-    size_t dotpart = 0;    // [kt][C_out] fp32 (tensor-core weight-gradient path)
+    size_t dotpart = 0;    // [row block][C_out] fp32: parts of sum omega' domega' (k-major weight-gradient partials only)
     int splits = 1, bsplits = 1, bn_splits = 1;
     size_t xpk = 0, wst = 0;   // small-C_in layers: packed input [n][hp][wp][8], expanded weights [C_out][kh][64]
     bool stem = false;
@@ -628,7 +628,8 @@ int run_param_grads(const convbn_desc *d, const Problem &pb, const Plan &pl, con
     if (pl.stem_win_wgrad) {
         float *dotpart = (float *)at(ws, pl.dotpart);
         LAUNCH("stem_wgrad", launch_stem_window_wgrad(pb, dz, x, partials, bsum, st));
-        LAUNCH("wgrad_rows", launch_wgrad_epilogue_kmajor(pb, pl.uw.splits, partials, bsum, w, vec3, b, mean, dw, dotpart, db, dgamma, dbeta, need_bsum, st));
+        LAUNCH("wgrad_rows", launch_wgrad_epilogue_kmajor(pb, pl.uw.splits, partials, bsum, w, vec3, b, mean, dw, dotpart, db,
+                                                          dgamma, dbeta, need_bsum, st));
         *which = "umma-stem";
     } else if (pl.stem) {
         LAUNCH("stem_pack", launch_stem_pack(pb, x, at(ws, pl.xpk), st));

@@ -1,8 +1,8 @@
 // Stride-1 k x k convolution on the sm_100a tensor cores with the input staged ONCE per tile.
 //
-// The im2col kernel (umma_conv.cu) reloads every input pixel once per filter tap; for 3x3 layers that
-// is 9x the input through L2 and the TMA ring's latency bounds the kernel.  Here a tile is R output
-// rows x CW output columns of one image.  Its (R + kh - 1) x (CW + kw - 1) input patch is loaded by
+// The im2col kernel (umma_conv.cu) reloads every input pixel once per filter tap, 9x the input through L2 for 3x3 layers;
+// it is the faster one for dense layers all the same (strip_dense_small says why), this one serves outputs that skip taps
+// or chunks.  A tile is R output rows x CW output columns of one image.  Its (R + kh - 1) x (CW + kw - 1) input patch is loaded by
 // one tiled TMA copy per 64-channel chunk into shared memory as a flat list of pixels, 128 bytes
 // each, 128-byte swizzled.  Number the tile's outputs, halo columns included, as "virtual pixels"
 // v = i Wt + j (Wt = CW + kw - 1): tap (r, q) of virtual pixel v reads patch pixel v + r Wt + q, so the
