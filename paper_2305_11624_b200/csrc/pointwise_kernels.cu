@@ -558,7 +558,7 @@ cudaError_t launch_bn_eval_fwd(const Problem &pb, int dtype, int layout, const v
 }
 
 // ---- Eval-mode BatchNorm, backward (Table 2, Eval row) ---------------------------------------
-// dy = s dz, and per pixel slice: part_g = sum dz (y - mean) r, part_b = sum dz.
+// dy = s dz (if dy != NULL), and per pixel slice: part_g = sum dz (y - mean) r, part_b = sum dz.
 template <class T, class L>
 __global__ void __launch_bounds__(256) bn_eval_bwd_kernel(int c_out, int h_out, int w_out, long long p,
                                                           float eps, const T *__restrict__ dz,
@@ -579,7 +579,7 @@ __global__ void __launch_bounds__(256) bn_eval_bwd_kernel(int c_out, int h_out, 
     for (long long q = p0; q < p1; ++q) {
         const long long i = L::id == CONVBN_NHWC ? q * c_out + c : ((q / hw) * c_out + c) * hw + q % hw;
         const float d = to_f32(dz[i]);
-        dy[i] = from_f32<T>(s * d);
+        if (dy) dy[i] = from_f32<T>(s * d);
         ag = fmaf(d, (to_f32(y[i]) - m) * r, ag);
         ab += d;
     }

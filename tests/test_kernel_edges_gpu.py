@@ -41,6 +41,18 @@ def test_tune_block(spec):
         parity.compare(got, ref, parity.TOL[spec.dtype], parity.TUNE_OUTPUTS, spec.name, dtype=spec.dtype)
 
 
+EVAL = [  # Eval mode
+    # more than 2048 output channels: the backward's sums by the kernel that takes any channel count, which writes no s dZ here
+    L("eval_c2112", 3, 64, 5, 7, 2112, 1, 1, bias=True), L("eval_c2112_f16", 2, 128, 4, 9, 2112, 1, 1, dtype="f16"),
+]
+
+
+@pytest.mark.parametrize("spec", EVAL, ids=lambda s: s.name)
+def test_eval_block(spec):
+    import test_parity_gpu
+    test_parity_gpu.test_eval_and_deploy_comparators(spec)
+
+
 TCONV = [  # (dtype, n, c_in, h, w, c_out, k, stride, pad, dil, groups, bias): kernel = stride, the GEMM on omega as it is
     ("bf16", 3, 64, 5, 7, 192, 2, 2, 0, 1, 1, True),        # tiles of 64 columns, fewer pixels than a tile
     ("f16", 1, 192, 13, 11, 64, 3, 3, 0, 1, 1, False),      # nine taps, a last tile of 15 pixels
