@@ -584,7 +584,7 @@ int run_conv_dgrad(const convbn_desc *d, const Problem &pb, const void *dz, cons
         *which = "depthwise";
     } else if (f32_path(d, pb)) {
         LAUNCH("direct_dgrad", launch_f32_bwd(pb, (const float *)dz, nullptr, (const float *)w, scale, (float *)dx, nullptr,
-                                              nullptr, nullptr, nullptr, nullptr, nullptr, nullptr, st));
+                                              nullptr, nullptr, nullptr, nullptr, nullptr, nullptr, 1, nullptr, nullptr, st));
         *which = "direct";
     } else {
         const void *wd = w;
@@ -607,6 +607,19 @@ int run_post(const convbn_desc *d, const PostOp &post, void *t, long long count,
     return CONVBN_OK;
 }
 
+// fp32 layers of f32_kernels.cu: parameter gradients and, if dx is given, the input gradient of the weights times dx_scale.
+// partials, bsum: of the parameter-gradient plan, used by more than one group.
+int run_f32_bwd(const convbn_desc *d, const Problem &pb, int groups, float *partials, float *bsum, const void *dz, const void *x,
+                const void *w, const float *dx_scale, void *dx, const float *vec3, const float *b, const float *mean, float *dw,
+                float *db, float *dgamma, float *dbeta, cudaStream_t st) {
+    LAUNCH("direct_bwd", launch_f32_bwd(pb, (const float *)dz, (const float *)x, (const float *)w, dx_scale, (float *)dx, vec3, b,
+                                        mean, dw, db, dgamma, dbeta, groups, partials, bsum, st));
+    if (groups > 1)
+        LAUNCH("wgrad_epilogue", launch_wgrad_epilogue(pb, d->dtype, partials, groups, bsum, groups, w, vec3, b, mean, dw, db,
+                                                       dgamma, dbeta, st));
+    return CONVBN_OK;
+}
+
 // Parameter gradients from dZ and X, shared by all modes.
 //   vec3 != NULL (Tune): dw = s domega', dbeta, db = s dbeta, dgamma          (Table 2, Tune row)
 //   vec3 == NULL        : dw = domega', db = sum dZ if db != NULL               (Deploy / Eval rows)
@@ -614,13 +627,12 @@ int run_post(const convbn_desc *d, const PostOp &post, void *t, long long count,
 int run_param_grads(const convbn_desc *d, const Problem &pb, const Plan &pl, const void *dz, const void *x,
                     const void *w, const float *vec3, const float *b, const float *mean, float *dw, float *db,
                     float *dgamma, float *dbeta, void *ws, cudaStream_t st, const char **which, bool scale_only = false) {
-    if (f32_path(d, pb)) {
-        LAUNCH("direct_wgrad", launch_f32_bwd(pb, (const float *)dz, (const float *)x, (const float *)w, nullptr, nullptr, vec3, b,
-                                              mean, dw, db, dgamma, dbeta, st));
-        *which = "direct";
-        return CONVBN_OK;
-    }
     float *partials = (float *)at(ws, pl.partials), *bsum = (float *)at(ws, pl.bsum);
+    if (f32_path(d, pb))
+        if (const int groups = f32_wgrad_groups(pb); groups > 0) {
+            *which = "direct";
+            return run_f32_bwd(d, pb, groups, partials, bsum, dz, x, w, nullptr, nullptr, vec3, b, mean, dw, db, dgamma, dbeta, st);
+        }
     const bool need_bsum = (vec3 || db) && !scale_only;
     const bool tc = pl.grouped_wgrad || pl.umma_wgrad || pl.stem;   // tensor-core paths sum dZ inside the GEMM
     if (need_bsum && !tc && !pl.dw_tma_wgrad)
@@ -941,10 +953,16 @@ static int tune_bwd_impl(const convbn_desc *desc, const void *dz, const void *x,
         return CONVBN_EALIGN;
     const Plan pl = make_plan(desc, pb, CONVBN_PHASE_TUNE_BWD);
     CK(check_ws(pl, workspace, workspace_bytes));
-    if (f32_path(desc, pb)) {            // both passes in one launch
+    if (const int groups = f32_path(desc, pb) ? f32_wgrad_groups(pb) : 0; groups > 0) {            // both passes in one launch
         cudaStream_t st = (cudaStream_t)stream;
-        LAUNCH("direct_bwd", launch_f32_bwd(pb, (const float *)dz, (const float *)x, (const float *)w, (const float *)saved,
-                                            (float *)dx, (const float *)saved, b, run_mean, dw, db, dgamma, dbeta, st));
+        float *partials = nullptr, *bsum = nullptr;
+        if (groups > 1) {
+            const Plan pw = make_plan(desc, pb, CONVBN_PHASE_TUNE_BWD_WEIGHT);
+            partials = (float *)at(workspace, pl.w_scaled + pw.partials);
+            bsum = (float *)at(workspace, pl.w_scaled + pw.bsum);
+        }
+        CK(run_f32_bwd(desc, pb, groups, partials, bsum, dz, x, w, (const float *)saved, dx, (const float *)saved, b, run_mean, dw,
+                       db, dgamma, dbeta, st));
         t_last_kernel[CONVBN_PHASE_TUNE_BWD] = "two-calls";
         return run_post(desc, post, dx, pb.pin * pb.c_in, st);
     }

@@ -1,12 +1,13 @@
-// fp32 NCHW convolutions with unit stride and dilation, groups = 1 and a 1x1 or 3x3 kernel, up to 128 channels: the
-// small fp32 blocks of unit tests, gradient checks and small networks.  (Other fp32 shapes: direct_kernels.cu.)
+// fp32 NCHW convolutions with unit stride and dilation, groups = 1 and a 1x1 or 3x3 kernel, up to 128 channels.  (Other fp32
+// shapes: direct_kernels.cu.)
 //
-// At these sizes a pass is bound by its launches and by the length of each thread's chain of loads (a 3x3 block of
-// 16 -> 32 channels at 16 x 16, N = 2 is 14 MFLOP; one thread per output took 12 to 33 us a kernel in seven launches), so
-// each direction is ONE launch:
+// At the sizes of unit tests, gradient checks and small networks a pass is bound by its launches and by the length of each
+// thread's chain of loads (a 3x3 block of 16 -> 32 channels at 16 x 16, N = 2 is 14 MFLOP; one thread per output took 12 to
+// 33 us a kernel in seven launches), so each direction is ONE launch there:
 //   forward   Z = s (omega (*) X) + b', s and b' formed in the kernel;
 //   backward  blocks of two kinds: domega', sum dZ and all parameter gradients in clusters of eight blocks that add up
 //             through distributed shared memory, and dX = (s omega)_rot (*) dZ.
+// With more pixels several clusters share the output channels and a second launch adds their sums (f32_wgrad_groups).
 #include <cooperative_groups.h>
 
 #include "kernels.h"
@@ -17,7 +18,7 @@ namespace convbn {
 namespace {
 
 constexpr int kFThreads = 256;
-constexpr int kFPix = 64;           // output pixels of a convolution block (of one image plane)
+constexpr int kFPix = 64;           // output pixels of a convolution block (of any images)
 constexpr int kFChunk = 16;         // input channels whose weights are staged at a time
 constexpr int kFCluster = 8;        // blocks of a weight-gradient cluster
 constexpr int kFCo = 4;             // output channels of a cluster
@@ -30,20 +31,20 @@ struct F32Conv {
     int n, ic, h, wd, oc, ho, wo, pad;     // pad: of this pass
     const float *k_scale;                  // DGRAD: s of the layer's output channel, here the input channel (NULL = 1)
     const float *bias;                     // without fold (NULL = 0)
-    int tiles;                             // pixel tiles of a plane
+    int tiles;                             // tiles of the n ho wo output pixels
 };
 
-// Block (oc tile, pixel tile, image).  256 threads = 64 pixels x 4 groups.  S == 1: the groups are R output channels each,
+// Block (oc tile, pixel tile).  256 threads = 64 pixels x 4 groups.  S == 1: the groups are R output channels each,
 // the input channels go by in chunks of 16.  S == 4: the groups split the input channels and are added up at the end, R
 // output channels per block, which keeps the chain of a thread short when there are too few blocks to hide it.
 // Weights are staged as [ic][tap][oc]; a thread's value of the activation meets R of them in one or two broadcasts.
 template <int K, int R, int S, bool DGRAD>
-__device__ __forceinline__ void conv_tile(const F32Conv &c, int oc0, int tile, int img, const float *scale_s, const float *shift_s,
+__device__ __forceinline__ void conv_tile(const F32Conv &c, int oc0, int tile, const float *scale_s, const float *shift_s,
                                           float *smem) {
     constexpr int KK = K * K, OCT = S == 1 ? 4 * R : R;
     const int lane = threadIdx.x % kFPix, grp = threadIdx.x / kFPix;
-    const int p = tile * kFPix + lane, hw = c.ho * c.wo;
-    const bool valid = p < hw;
+    const int hw = c.ho * c.wo, pg = tile * kFPix + lane, img = pg / hw, p = pg - img * hw;
+    const bool valid = img < c.n;
     const int y = valid ? p / c.wo : 0, x = valid ? p - y * c.wo : 0;
     bool ok[KK];
 #pragma unroll
@@ -53,7 +54,8 @@ __device__ __forceinline__ void conv_tile(const F32Conv &c, int oc0, int tile, i
             const int yy = y - c.pad + r, xx = x - c.pad + q;
             ok[r * K + q] = valid && yy >= 0 && yy < c.h && xx >= 0 && xx < c.wd;
         }
-    const float *a0 = c.act + (size_t)img * c.ic * c.h * c.wd + (ptrdiff_t)(y - c.pad) * c.wd + (x - c.pad);
+    // (offsets fit an int: fewer than 2^30 elements)
+    const int a0 = img * c.ic * c.h * c.wd + (y - c.pad) * c.wd + (x - c.pad), out0 = valid ? (img * c.oc + oc0) * hw + p : -1;
     float acc[R];
 #pragma unroll
     for (int j = 0; j < R; ++j) acc[j] = 0.f;
@@ -82,7 +84,7 @@ __device__ __forceinline__ void conv_tile(const F32Conv &c, int oc0, int tile, i
         const int per = S == 1 ? nic : (nic + 3) / 4, lo = S == 1 ? 0 : grp * per, hi = S == 1 ? nic : min(nic, lo + per);
 #pragma unroll 2
         for (int ci = lo; ci < hi; ++ci) {
-            const float *a = a0 + (size_t)(ic0 + ci) * c.h * c.wd;
+            const float *a = c.act + (ptrdiff_t)(a0 + (ic0 + ci) * c.h * c.wd);
             float v[KK];
 #pragma unroll
             for (int t = 0; t < KK; ++t) v[t] = ok[t] ? __ldg(a + (t / K) * c.wd + t % K) : 0.f;
@@ -110,8 +112,8 @@ __device__ __forceinline__ void conv_tile(const F32Conv &c, int oc0, int tile, i
 #pragma unroll
     for (int j = 0; j < NO; ++j) {
         const int o = S == 1 ? grp * R + j : grp;
-        if (valid && oc0 + o < c.oc)
-            c.out[((size_t)img * c.oc + oc0 + o) * hw + p] = DGRAD ? acc[j] : fmaf(acc[j], scale_s[o], shift_s[o]);
+        if (out0 >= 0 && oc0 + o < c.oc)
+            c.out[(size_t)(out0 + o * hw)] = DGRAD ? acc[j] : fmaf(acc[j], scale_s[o], shift_s[o]);
     }
 }
 
@@ -121,7 +123,7 @@ constexpr int conv_smem_floats(int kk, int r, int s, int ic) {
 }
 
 template <int K, int R, int S>
-__global__ void __launch_bounds__(kFThreads) f32_fwd_kernel(const F32Conv c, const BnFold fold) {
+__global__ void __launch_bounds__(kFThreads, S == 1 ? 5 : 4) f32_fwd_kernel(const F32Conv c, const BnFold fold) {
     extern __shared__ __align__(16) float f32_smem[];
     constexpr int OCT = S == 1 ? 4 * R : R;
     __shared__ float scale_s[OCT], shift_s[OCT];
@@ -136,7 +138,7 @@ __global__ void __launch_bounds__(kFThreads) f32_fwd_kernel(const F32Conv c, con
                 const float r = 1.0f / sqrtf(fold.var[o] + fold.eps);
                 sc = fold.gamma[o] * r;
                 sh = ((fold.b ? fold.b[o] : 0.f) - fold.mean[o]) * sc + fold.beta[o];
-                if (blockIdx.x == 0 && blockIdx.z == 0 && fold.vec3) {
+                if (blockIdx.x == 0 && fold.vec3) {
                     fold.vec3[o] = sc; fold.vec3[c.oc + o] = sh; fold.vec3[2 * c.oc + o] = r;
                 }
             } else if (c.bias) {
@@ -146,13 +148,15 @@ __global__ void __launch_bounds__(kFThreads) f32_fwd_kernel(const F32Conv c, con
         scale_s[threadIdx.x] = sc;
         shift_s[threadIdx.x] = sh;
     }
-    conv_tile<K, R, S, false>(c, oc0, blockIdx.x, blockIdx.z, scale_s, shift_s, f32_smem);
+    conv_tile<K, R, S, false>(c, oc0, blockIdx.x, scale_s, shift_s, f32_smem);
 }
 
 struct F32Wgrad {
     const float *x, *dz, *w;
     const float *vec3, *b, *mean;          // vec3 NULL: dw = domega', db = sum dZ
     float *dw, *db, *dgamma, *dbeta;
+    int groups;                            // clusters that share kFCo output channels
+    float *partials, *bsum;                // groups > 1: sums of a cluster, [groups][c_out][c_in K K] and [groups][c_out]
     int n, c_in, h, wd, c_out, ho, wo, pad;
     int cip;                               // power of two >= c_in, 4 .. 128: threads along the input channels
     int rows, bands;                       // output rows of a band, bands of an image
@@ -160,24 +164,25 @@ struct F32Wgrad {
     int x_ci;                              // floats between the channels of the staged X (odd)
 };
 
-// Cluster = kFCo output channels, block rank r takes the row bands r, r + 8, ... of all images.  A band of X (all channels,
+// Cluster = kFCo output channels and one of `groups` shares of the row bands: the 8 groups blocks that have the same channels
+// take turns.  A band of X (all channels,
 // its halo rows, zeros outside) and of dZ is staged; thread (ci, channel pair, pixel group) slides a K x K window of X
 // along runs of eight pixels: K new values and two of dZ per 2 K K multiply-adds.  The pixel groups are added in the block,
 // the blocks through distributed shared memory, in rank order; rank j < 4 then finishes output channel j:
 //   domega = s domega', dbeta = sum dZ, db = s dbeta, dgamma = r (sum domega' omega + dbeta (b - mu_hat))   (Table 2)
 template <int K>
-__device__ __forceinline__ void wgrad_cluster(const F32Wgrad &g, int co0, float *smem) {
+__device__ __forceinline__ void wgrad_cluster(const F32Wgrad &g, int co0, int group, float *smem) {
     constexpr int KK = K * K;
     cg::cluster_group cluster = cg::this_cluster();
     const int rank = (int)cluster.block_rank();
     const int ci = threadIdx.x % g.cip, rest = threadIdx.x / g.cip;
     const int pair = rest & 1, pg = rest >> 1, npg = kFThreads / (2 * g.cip);
     float *xs = smem, *zs = smem + (size_t)g.c_in * g.x_ci + 1;
-    float acc[2][KK], sum[2] = {0.f, 0.f};
+    float acc[2][KK], sum[kFCo] = {0.f, 0.f, 0.f, 0.f};      // sum: of the dZ values this thread stages
 #pragma unroll
     for (int t = 0; t < KK; ++t) acc[0][t] = acc[1][t] = 0.f;
     const int xrows = g.rows + K - 1, runs = g.zp / kFRun, items = g.n * g.bands;
-    for (int it = rank; it < items; it += kFCluster) {
+    for (int it = group * kFCluster + rank; it < items; it += g.groups * kFCluster) {
         const int img = it / g.bands, y0 = (it - img * g.bands) * g.rows;
         __syncthreads();
         for (int i = threadIdx.x; i < g.c_in * xrows * g.xp; i += kFThreads) {
@@ -188,12 +193,16 @@ __device__ __forceinline__ void wgrad_cluster(const F32Wgrad &g, int co0, float 
         }
         for (int i = threadIdx.x; i < kFCo * g.rows * g.zp; i += kFThreads) {
             const int x = i % g.zp, t = i / g.zp, r = t % g.rows, o = t / g.rows;
-            zs[i] = (co0 + o < g.c_out && y0 + r < g.ho && x < g.wo)
-                        ? __ldg(g.dz + (((size_t)img * g.c_out + co0 + o) * g.ho + y0 + r) * g.wo + x) : 0.f;
+            const float v = (co0 + o < g.c_out && y0 + r < g.ho && x < g.wo)
+                                ? __ldg(g.dz + (((size_t)img * g.c_out + co0 + o) * g.ho + y0 + r) * g.wo + x) : 0.f;
+            zs[i] = v;
+#pragma unroll
+            for (int q = 0; q < kFCo; ++q) sum[q] += q == o ? v : 0.f;
         }
         __syncthreads();
+        const int nruns = min(g.rows, g.ho - y0) * runs;
         if (ci < g.c_in)
-            for (int j = pg; j < g.rows * runs; j += npg) {
+            for (int j = pg; j < nruns; j += npg) {
                 const int r = j / runs, x = (j - r * runs) * kFRun;
                 const float *xr = xs + (size_t)ci * g.x_ci + r * g.xp + x;
                 const float *z0 = zs + ((2 * pair) * g.rows + r) * g.zp + x, *z1 = z0 + g.rows * g.zp;
@@ -215,12 +224,13 @@ __device__ __forceinline__ void wgrad_cluster(const F32Wgrad &g, int co0, float 
                             acc[0][a * K + q] = fmaf(d0, v, acc[0][a * K + q]);
                             acc[1][a * K + q] = fmaf(d1, v, acc[1][a * K + q]);
                         }
-                    sum[0] += d0;
-                    sum[1] += d1;
                 }
             }
     }
-    // pixel groups -> block: [thread][K K + 1], then part[co][c_in K K + 1] (the last entry is sum dZ)
+    // pixel groups -> block: [thread][K K], then part[co][c_in K K + 1] (the last entry is sum dZ)
+    __shared__ float sums[kFCo][kFThreads];
+#pragma unroll
+    for (int q = 0; q < kFCo; ++q) sums[q][threadIdx.x] = sum[q];
     __syncthreads();
     const int kd = g.c_in * KK, row = kd + 1;
     float *part = smem, *red = smem + kFCo * row;
@@ -228,16 +238,22 @@ __device__ __forceinline__ void wgrad_cluster(const F32Wgrad &g, int co0, float 
         float *mine = red + ((size_t)((pg * g.cip + ci) * 2 + pair)) * (KK + 1);
 #pragma unroll
         for (int t = 0; t < KK; ++t) mine[t] = acc[h][t];
-        mine[KK] = sum[h];
         __syncthreads();
-        for (int i = threadIdx.x; i < 2 * row; i += kFThreads) {
-            const int pr = i / row, e = i - pr * row;
-            const int c = e < kd ? e / KK : 0, t = e < kd ? e % KK : KK;
+        for (int i = threadIdx.x; i < 2 * kd; i += kFThreads) {
+            const int pr = i / kd, e = i - pr * kd, c = e / KK, t = e % KK;
             float v = 0.f;
             for (int q = 0; q < npg; ++q) v += red[((size_t)((q * g.cip + c) * 2 + pr)) * (KK + 1) + t];
             part[(2 * pr + h) * row + e] = v;
         }
         __syncthreads();
+    }
+    if (threadIdx.x < 32 * kFCo) {        // one warp per output channel
+        const int o = threadIdx.x / 32;
+        float v = 0.f;
+        for (int i = threadIdx.x % 32; i < kFThreads; i += 32) v += sums[o][i];
+#pragma unroll
+        for (int m = 16; m > 0; m >>= 1) v += __shfl_xor_sync(0xffffffffu, v, m);
+        if (threadIdx.x % 32 == 0) part[o * row + kd] = v;
     }
     cluster.sync();
     const int co = co0 + rank;
@@ -251,7 +267,10 @@ __device__ __forceinline__ void wgrad_cluster(const F32Wgrad &g, int co0, float 
             float tot = 0.f;
 #pragma unroll
             for (int b = 0; b < kFCluster; ++b) tot += v[b];
-            if (e < kd) {
+            if (g.groups > 1) {
+                if (e < kd) g.partials[((size_t)group * g.c_out + co) * kd + e] = tot;
+                else g.bsum[(size_t)group * g.c_out + co] = tot;
+            } else if (e < kd) {
                 const size_t o = (size_t)co * kd + e;
                 g.dw[o] = s * tot;
                 if (g.vec3) dot = fmaf(tot, g.w[o], dot);
@@ -264,7 +283,7 @@ __device__ __forceinline__ void wgrad_cluster(const F32Wgrad &g, int co0, float 
         for (int o = 16; o > 0; o >>= 1) { dot += __shfl_xor_sync(0xffffffffu, dot, o); dsum += __shfl_xor_sync(0xffffffffu, dsum, o); }
         if (threadIdx.x % 32 == 0) { fin[0][threadIdx.x / 32] = dot; fin[1][threadIdx.x / 32] = dsum; }
         __syncthreads();
-        if (threadIdx.x == 0) {
+        if (threadIdx.x == 0 && g.groups == 1) {
             dot = dsum = 0.f;
             for (int i = 0; i < kFThreads / 32; ++i) { dot += fin[0][i]; dsum += fin[1][i]; }
             if (g.vec3) {
@@ -281,25 +300,30 @@ __device__ __forceinline__ void wgrad_cluster(const F32Wgrad &g, int co0, float 
 
 // blocks [0, nw): weight-gradient clusters; [nw, nw + nd): dX tiles (rounded up to whole clusters)
 template <int K, int R, int S>
-__global__ void __cluster_dims__(kFCluster, 1, 1) __launch_bounds__(kFThreads) f32_bwd_kernel(const F32Wgrad g, int nw, const F32Conv c,
+__global__ void __cluster_dims__(kFCluster, 1, 1) __launch_bounds__(kFThreads, 4) f32_bwd_kernel(const F32Wgrad g, int nw, const F32Conv c,
                                                                                           int oc_tiles) {
     extern __shared__ __align__(16) float f32_smem[];
     pdl_wait();
     pdl_launch_dependents();
     const int b = (int)blockIdx.x;
     if (b < nw) {
-        wgrad_cluster<K>(g, (b / kFCluster) * kFCo, f32_smem);
+        const int cl = b / kFCluster / g.groups;
+        wgrad_cluster<K>(g, cl * kFCo, b / kFCluster - cl * g.groups, f32_smem);
         return;
     }
     constexpr int OCT = S == 1 ? 4 * R : R;
-    const int i = b - nw, t = i / oc_tiles, img = t / c.tiles;
-    if (img < c.n) conv_tile<K, R, S, true>(c, (i - t * oc_tiles) * OCT, t - img * c.tiles, img, nullptr, nullptr, f32_smem);
+    const int i = b - nw, t = i / oc_tiles;
+    if (t < c.tiles) conv_tile<K, R, S, true>(c, (i - t * oc_tiles) * OCT, t, nullptr, nullptr, f32_smem);
 }
 
-// S = 4 while the 32-channel blocks of S = 1 would not give every SM two (16 -> 32 channels at 16 x 16, N = 2: 8 of them)
-bool split_channels(int n, int oc, int hw) {
-    return (long long)n * ((oc + 31) / 32) * ((hw + kFPix - 1) / kFPix) < 2LL * device_sm_count();
+// S = 4 while the 32-channel blocks of S = 1 would not give every SM two (16 -> 32 channels at 16 x 16, N = 2: 8 of them), and
+// where it has less to do: a block's fixed cost and, per input channel and tap of a thread, a load and R multiply-adds, padded
+// channels included (93 -> 1 at 96 x 96, N = 22: 119.9 us by 32 channels, 24 by 4; 3 -> 9 at 117 x 27, N = 37: 7.5 and 13.5).
+bool split_channels(int tiles, int ic, int oc, int kk) {
+    if ((long long)tiles * ((oc + 31) / 32) < 2LL * device_sm_count()) return true;
+    return (oc + 3) / 4 * (100 + (ic + 3) / 4 * kk * 6) < (oc + 31) / 32 * (100 + ic * kk * 10);
 }
+int pixel_tiles(long long pixels) { return (int)((pixels + kFPix - 1) / kFPix); }
 
 bool wgrad_geometry(const Problem &pb, F32Wgrad *g, size_t *bytes) {
     g->n = pb.n; g->c_in = pb.c_in; g->h = pb.h_in; g->wd = pb.w_in; g->c_out = pb.c_out; g->ho = pb.h_out; g->wo = pb.w_out;
@@ -345,33 +369,68 @@ bool f32_conv_eligible(const Problem &pb) {
     return wgrad_geometry(pb, &g, &bytes);
 }
 
+// How many clusters share four output channels (their sums then go through launch_wgrad_epilogue), or 0: the direct kernels
+// take the parameter gradients.  The least time by a model of microseconds, fitted to 400 layers (1 to 128 channels, planes of
+// 1 x 1 to 200 x 200, N = 1 to 20000) at up to 13 counts each: on average 2 % above the best of them, in one layer more than
+// 5 % above the direct kernels.  A block's row bands go by one after the other, each a staging pass and its multiply-adds; the
+// direct kernels' threads go through the pixels of a slice.  One cluster whatever the pixels left few output channels to few
+// blocks: 1x1 64 -> 8 at 56 x 56, N = 16 340 us, now 51, direct 145.  Planes narrower than a run of pixels
+// in many images stay with the direct kernels: 1x1 1 -> 89 on 6876 rows 991 us with one cluster, direct 46.
+int f32_wgrad_groups(const Problem &pb) {
+    F32Wgrad g;
+    size_t bytes;
+    if (!wgrad_geometry(pb, &g, &bytes)) return 0;
+    const int kk = pb.kh * pb.kw, items = g.n * g.bands, npg = kFThreads / (2 * g.cip), slots = 2 * device_sm_count();
+    const int blocks = (pb.c_out + kFCo - 1) / kFCo * kFCluster, inner = (g.rows * (g.zp / kFRun) + npg - 1) / npg * kFRun;
+    const double stage = (double)(g.c_in * (g.rows + pb.kh - 1) * g.xp + kFCo * g.rows * g.zp) / kFThreads;
+    const double item = 0.95 + 0.0049 * inner * kk + 0.176 * stage;
+    // the partial sums live in the direct kernels' workspace, and no thread adds up more pixels than one of those would
+    const int slices = direct_wgrad_splits(pb), sums = channel_sum_splits(pb), limit = slices < sums ? slices : sums;
+    const double chain = (double)pb.p / slices > 256.0 ? (double)pb.p / slices : 256.0;
+    const double rounds = (double)pb.c_out * pb.kdim * slices / (2048.0 * device_sm_count());
+    const int lines = (pb.kdim + 255) / 256;            // of the finishing kernel's threads
+    int best = 0;
+    // (times 1.2: with that least is lost where the two are close)
+    double best_cost = 1.2 * (6.0 + (0.25 + (rounds > 1.0 ? 1.57 * (rounds - 1.0) : 0.0)) * pb.p / slices + 0.166 * pb.p / sums +
+                              0.034 * slices * lines);
+    for (int groups = 1; groups <= limit; groups += 1 + groups / 4) {
+        const int per_block = (items + kFCluster * groups - 1) / (kFCluster * groups);
+        if ((double)per_block * inner > chain && groups + 1 + groups / 4 <= limit) continue;
+        const double waves = (double)blocks * groups > slots ? (double)blocks * groups / slots : 1.0;
+        const double cost = 3.8 + (groups > 1 ? 3.0 + 0.02 * groups * lines : 0.0) + per_block * item * waves;
+        if (cost < best_cost) { best_cost = cost; best = groups; }
+    }
+    return best;
+}
+
 cudaError_t launch_f32_fwd(const Problem &pb, const float *x, const float *w, const float *bias, float *z, cudaStream_t st,
                            const BnFold *fold) {
     F32Conv c{x, w, z, pb.n, pb.c_in, pb.h_in, pb.w_in, pb.c_out, pb.h_out, pb.w_out, pb.pad_h, nullptr, bias, 0};
-    c.tiles = (pb.h_out * pb.w_out + kFPix - 1) / kFPix;
+    c.tiles = pixel_tiles(pb.p);
     const BnFold fd = fold ? *fold : BnFold{nullptr, nullptr, nullptr, nullptr, nullptr, 0.f, nullptr};
-    return by_shape(pb.kh, split_channels(pb.n, pb.c_out, pb.h_out * pb.w_out), [&](auto k, auto r, auto s) {
+    return by_shape(pb.kh, split_channels(c.tiles, c.ic, c.oc, pb.kh * pb.kw), [&](auto k, auto r, auto s) {
         constexpr int K = decltype(k)::value, R = decltype(r)::value, S = decltype(s)::value, OCT = S == 1 ? 4 * R : R;
         const size_t smem = conv_smem_floats(K * K, R, S, pb.c_in) * sizeof(float);
-        return launch_pdl(f32_fwd_kernel<K, R, S>, dim3(c.tiles, (c.oc + OCT - 1) / OCT, c.n), dim3(kFThreads), smem, st, c, fd);
+        return launch_pdl(f32_fwd_kernel<K, R, S>, dim3(c.tiles, (c.oc + OCT - 1) / OCT), dim3(kFThreads), smem, st, c, fd);
     });
 }
 
 cudaError_t launch_f32_bwd(const Problem &pb, const float *dz, const float *x, const float *w, const float *scale, float *dx,
                            const float *vec3, const float *b, const float *mean, float *dw, float *db, float *dgamma,
-                           float *dbeta, cudaStream_t st) {
+                           float *dbeta, int groups, float *partials, float *bsum, cudaStream_t st) {
     F32Wgrad g{};
     size_t wbytes = 0;
     if (!wgrad_geometry(pb, &g, &wbytes)) return cudaErrorInvalidValue;
     g.x = x; g.dz = dz; g.w = w; g.vec3 = vec3; g.b = b; g.mean = mean; g.dw = dw; g.db = db; g.dgamma = dgamma; g.dbeta = dbeta;
+    g.groups = groups; g.partials = partials; g.bsum = bsum;
     // dX is a convolution of dZ with the rotated weights: padding k - 1 - pad
     F32Conv c{dz, w, dx, pb.n, pb.c_out, pb.h_out, pb.w_out, pb.c_in, pb.h_in, pb.w_in, pb.kh - 1 - pb.pad_h, scale, nullptr, 0};
-    c.tiles = (pb.h_in * pb.w_in + kFPix - 1) / kFPix;
-    const int nw = dw ? (pb.c_out + kFCo - 1) / kFCo * kFCluster : 0;
-    return by_shape(pb.kh, split_channels(pb.n, pb.c_in, pb.h_in * pb.w_in), [&](auto k, auto r, auto s) {
+    c.tiles = pixel_tiles(pb.pin);
+    const int nw = dw ? (pb.c_out + kFCo - 1) / kFCo * kFCluster * groups : 0;
+    return by_shape(pb.kh, split_channels(c.tiles, c.ic, c.oc, pb.kh * pb.kw), [&](auto k, auto r, auto s) {
         constexpr int K = decltype(k)::value, R = decltype(r)::value, S = decltype(s)::value, OCT = S == 1 ? 4 * R : R;
         const int oc_tiles = (c.oc + OCT - 1) / OCT;
-        const long long nd = dx ? ((long long)oc_tiles * c.tiles * c.n + kFCluster - 1) / kFCluster * kFCluster : 0;
+        const long long nd = dx ? ((long long)oc_tiles * c.tiles + kFCluster - 1) / kFCluster * kFCluster : 0;
         size_t smem = nw ? wbytes : 0;
         const size_t cbytes = conv_smem_floats(K * K, R, S, c.ic) * sizeof(float);
         if (nd && cbytes > smem) smem = cbytes;

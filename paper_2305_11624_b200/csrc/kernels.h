@@ -52,10 +52,12 @@ bool f32_conv_eligible(const Problem &pb);
 cudaError_t launch_f32_fwd(const Problem &pb, const float *x, const float *w, const float *bias, float *z, cudaStream_t st,
                            const BnFold *fold = nullptr);
 // dx != NULL: dX = (scale omega)_rot (*) dZ (scale NULL = 1).  dw != NULL: the parameter gradients (vec3 NULL: dw =
-// domega', db = sum dZ if wanted).
+// domega', db = sum dZ if wanted) by `groups` = f32_wgrad_groups clusters for every four output channels; more than one
+// leave their sums in partials [groups][C_out][kdim] and bsum [groups][C_out], for launch_wgrad_epilogue.
 cudaError_t launch_f32_bwd(const Problem &pb, const float *dz, const float *x, const float *w, const float *scale, float *dx,
                            const float *vec3, const float *b, const float *mean, float *dw, float *db, float *dgamma,
-                           float *dbeta, cudaStream_t st);
+                           float *dbeta, int groups, float *partials, float *bsum, cudaStream_t st);
+int f32_wgrad_groups(const Problem &pb);      // 0: the direct kernels are faster
 
 // ---- tensor-core implicit-GEMM convolution (bf16 NHWC, groups = 1) -----------------------------
 // out[n,ho,wo,:cn] = bias + sum over taps (r,q) and channels c of

@@ -21,6 +21,14 @@ SPECS = [
     L("f32_many", 16, 33, 40, 37, 35, 3, 3, pad=1, dtype="f32", layout="nchw"),
     L("f32_nopad", 1, 20, 9, 30, 34, 3, 3, pad=0, dtype="f32", layout="nchw", bias=True),
     L("f32_pad2", 1, 7, 6, 9, 6, 3, 3, pad=2, dtype="f32", layout="nchw"),
+    # ... several clusters for the same output channels: a share without a whole band for every block, bands that end early,
+    # one output channel; 32-channel blocks and 4-channel ones that split the inputs; pixel tiles across images
+    L("f32_shares", 9, 40, 19, 23, 7, 3, 3, pad=1, dtype="f32", layout="nchw", bias=True),
+    L("f32_one_out", 12, 93, 48, 47, 1, 1, 1, dtype="f32", layout="nchw"),
+    L("f32_shares_8", 16, 8, 56, 50, 8, 3, 3, pad=1, dtype="f32", layout="nchw"),
+    L("f32_planes", 130, 17, 3, 5, 41, 3, 3, pad=1, dtype="f32", layout="nchw", bias=True),
+    # rows of features: parameter gradients by the direct kernels, the rest by these
+    L("f32_rows", 3001, 24, 1, 1, 37, 1, 1, dtype="f32", layout="nchw", bias=True),
     # dense GEMM by CTA pairs: an odd number of pixel tiles (the last has no partner) at 64 columns a pair; several rounds
     # at 128; 256 with a ragged last tile.  Channel chunks outermost: two chunks, weights resident and streamed
     L("pair_64", 7, 512, 7, 7, 192, 3, 3, pad=1, bias=True),
