@@ -347,9 +347,8 @@ __global__ void __launch_bounds__(kGThreads) grouped8_wgrad_kernel(const __grid_
 // vec3 == NULL: domega = domega', db = sum dZ.  One block per output channel: thread (k, j) adds slots
 // j, j + ng, ... of entry k (a slot's kdim <= 80 entries are contiguous, so the loads coalesce), the ng
 // slot groups are then added in order, and the last group column does the same for sum dZ.
-// Bound by the latency of the slot reads (the partials are in L2): 1024 threads split 100 slots into 14 groups, and
-// a thread requests four slots before it adds the first (24.7 us with 256 threads and one slot at a time).
-constexpr int kGFinThreads = 1024;
+// Bound by the latency of the slot reads (the partials are in L2): a thread requests four slots before it adds the first.
+constexpr int kGFinThreads = 512;            // at most
 __global__ void __launch_bounds__(kGFinThreads) grouped8_wgrad_finish_kernel(int c, int kdim, int slots,
                                                                             const float *__restrict__ part,
                                                                             const float *__restrict__ bsum,
@@ -365,7 +364,7 @@ __global__ void __launch_bounds__(kGFinThreads) grouped8_wgrad_finish_kernel(int
     pdl_wait();
     pdl_launch_dependents();
     const int co = blockIdx.x;
-    const int ng = kGFinThreads / (kdim + 1);        // slot groups; column kdim of each group sums dZ
+    const int ng = (int)blockDim.x / (kdim + 1);     // slot groups; column kdim of each group sums dZ
     const int k = threadIdx.x % (kdim + 1), j = threadIdx.x / (kdim + 1);
     float sum = 0.f;
     if (j < ng) {
@@ -595,7 +594,11 @@ cudaError_t launch_grouped8_wgrad_finish(const Problem &pb, const float *part, c
                                          float *dgamma, float *dbeta, cudaStream_t st) {
     const int slots = grouped8_wgrad_slots(pb);
     if (slots <= 0) return cudaErrorInvalidValue;
-    return launch_pdl(grouped8_wgrad_finish_kernel, dim3(pb.c_out), dim3(kGFinThreads), 0, st, pb.c_out, pb.kh * pb.kw * 8,
+    // With 256 threads five blocks share an SM.  512 where a thread would go through more than six batches of slots (C = 256,
+    // 56 x 16, N = 31, 111 slots: 19.5 and 17.2 us with the GEMM); 1024, which many slots want alone, cost 1.3 to 3.8 times the
+    // whole phase from 640 channels on (C = 768, 34 x 12, N = 29: 19.9 and 28.7).
+    const int threads = slots > 24 * (256 / (pb.kh * pb.kw * 8 + 1)) ? kGFinThreads : 256;
+    return launch_pdl(grouped8_wgrad_finish_kernel, dim3(pb.c_out), dim3(threads), 0, st, pb.c_out, pb.kh * pb.kw * 8,
                       slots, part, bsum, (const __nv_bfloat16 *)w, vec3, b, mean, dw, db, dgamma, dbeta, call_f16());
 }
 

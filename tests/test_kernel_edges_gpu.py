@@ -12,6 +12,8 @@ SPECS = [
     # the widest row one box takes, a last band of one row
     L("g8_chunks", 13, 704, 9, 10, 704, 3, 3, pad=1, groups=88, bias=True),
     L("g8_wide", 1, 64, 5, 254, 64, 3, 3, pad=1, groups=8, dtype="f16"),
+    # more partial slots than one batch of every thread (512 threads finish), many channels with few slots (256)
+    L("g8_slots", 31, 64, 20, 16, 64, 3, 3, pad=1, groups=8), L("g8_few_slots", 2, 768, 9, 12, 768, 3, 3, pad=1, groups=96, dtype="f16"),
     L("g8_last_row", 9, 128, 17, 29, 128, 3, 3, pad=1, groups=16),
     # fp32 NCHW: one channel and one pixel row, 128 channels (nothing left for pixel groups), a plane of 64 pixels and one
     # more, more bands than blocks of a cluster, output channels that end inside a block and inside a cluster
