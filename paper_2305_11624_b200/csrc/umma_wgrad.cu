@@ -304,9 +304,11 @@ UmmaWgradPlan umma_wgrad_plan(const Problem &pb) {
     // Few tiles mean many slices, and where those are short the partial tensors weigh more than what a second CTA hides: up to
     // 24 tiles with slices of up to 2048 pixels get one CTA per SM (N = 32: 1x1 128 -> 512 at 28 x 28 15.3 -> 13.4 us, 1024 ->
     // 256 at 14 x 14 13.3 -> 11.4, 3x3 128 at 28 x 28 17.6 -> 15.5; but 3x3 256 at 14 x 14, 38 tiles, 15.8 -> 18.1, and 1x1
-    // 128 -> 512 at 28 x 28, N = 256 58.3 -> 73.6).
+    // 128 -> 512 at 28 x 28, N = 256 58.3 -> 73.6).  Not where output rows are shorter than four pixels: the boxes of X then
+    // arrive pixel by pixel and a second CTA hides that (29173 rows, 1024 -> 64: 44.5 and 27.4 us; 2 x 2 about even; from
+    // 4 x 4 on one CTA is the faster).
     const long long tiles = m_tiles * n_tiles, sms = device_sm_count();
-    const long long slots = sms * (tiles <= 24 && pb.p * tiles <= 2048 * sms ? 1 : 2);
+    const long long slots = sms * (tiles <= 24 && pb.p * tiles <= 2048 * sms && pb.w_out >= 4 ? 1 : 2);
     const long long max_splits = (pb.p + 4 * kWP - 1) / (4 * kWP);     // at least 256 pixels per slice
     long long splits = 1;
     double best_cost = -1.0;

@@ -39,6 +39,8 @@ SPECS = [
     L("chunks_first", 5, 128, 24, 22, 192, 3, 3, pad=1), L("chunks_resident", 30, 128, 30, 31, 64, 2, 2, dtype="f16"),
     # weight gradient: C_out that ends inside the box of a 128-wide tile, fewer pixels than a stage
     L("wgrad_c192", 3, 64, 5, 4, 192, 3, 3, pad=1),
+    # ... rows of features and one pixel-row images (two CTAs per SM), the same pixels in rows of four (one)
+    L("wgrad_rows", 9001, 192, 1, 1, 64, 1, 1), L("wgrad_w3", 701, 64, 4, 3, 128, 3, 3, pad=1, dtype="f16"), L("wgrad_w4", 701, 64, 3, 4, 128, 3, 3, pad=1),
 ]
 
 
