@@ -906,7 +906,12 @@ int side_lane(SideLane **out) {
 // 56 x 56, N = 32, 68 -> 65 at 3x3 stride 2 128 -> 128, 200 x 334.  With a million weights, or where it is a GEMM per
 // parity class, the data pass is the longer one: 3x3 512 -> 512 at 7 x 7, N = 64
 // takes 79 us this way and 87 the other, 3x3 stride 2 256 -> 256 at 28 x 28 57 and 60.
-bool data_pass_first(const convbn_desc *d, const Problem &pb) {
+// A captured call pays no events, and its lane's nodes come first: there the pass with two kernels, the parameter gradients,
+// belongs on the lane (graph replay of random layers, the other order = 1: grouped by 8 below 40 us 0.88, 1x1 below 15 us 0.93,
+// depthwise 0.97, 3x3 and longer calls 0.98 to 1).
+bool data_pass_first(const convbn_desc *d, const Problem &pb, cudaStream_t st) {
+    cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(st, &capture) == cudaSuccess && capture == cudaStreamCaptureStatusActive) return true;
     UmmaConvShape s;
     const bool classes = strided_dgrad_ok(d, pb) && !(subpixel_wide_shape(pb, &s) && umma_strip_eligible(s));
     return pb.groups == 1 && ((long long)pb.c_out * pb.kdim >= (1LL << 20) || classes);
@@ -974,7 +979,7 @@ static int tune_bwd_impl(const convbn_desc *desc, const void *dz, const void *x,
             CK(tune_bwd_data_impl(desc, dz, w, saved, dx, post, workspace, bytes_d, stream));
             return convbn_tune_bwd_weight(desc, dz, x, w, b, run_mean, saved, dw, db, dgamma, dbeta, ws_w, bytes_w, stream);
         }
-        if (!defer_join && !data_pass_first(desc, pb))
+        if (!defer_join && !data_pass_first(desc, pb, (cudaStream_t)stream))
             return side_by_side(
                 (cudaStream_t)stream,
                 [&](cudaStream_t lane) { return tune_bwd_data_impl(desc, dz, w, saved, dx, post, workspace, bytes_d, lane); },

@@ -127,3 +127,25 @@ def test_glue_in_the_epilogue_equals_the_passes(spec):
         assert torch.equal(blk.dx, want), (add is not None, mask)
         assert all(torch.equal(a, b) for a, b in zip((blk.dw, blk.dgamma, blk.dbeta), grads))
     C.convbn_check()
+
+
+@pytest.mark.parametrize("spec", [L("cap_3x3", 2, 64, 20, 24, 64, 3, 3, pad=1), L("cap_grouped", 2, 64, 12, 13, 64, 3, 3, pad=1, groups=8),
+                                  L("cap_f32", 9, 40, 19, 23, 7, 3, 3, pad=1, dtype="f32", layout="nchw")], ids=lambda s: s.name)
+def test_captured_backward_equals_the_plain_call(spec):
+    """A captured backward call puts its passes on the other streams: the same bits."""
+    import torch
+    from paper_2305_11624_b200 import convbn as C
+    from paper_2305_11624_b200.harness import Block
+    blk = Block(spec)
+    blk.randomize(5)
+    blk.tune_fwd(); blk.tune_bwd()
+    outs = (blk.dx, blk.dw, blk.dgamma, blk.dbeta)
+    want = [t.clone() for t in outs]
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph):
+        blk.tune_bwd()
+    for t in outs:
+        t.fill_(float("nan"))
+    graph.replay()
+    C.convbn_check()
+    assert all(torch.equal(a, b) for a, b in zip(outs, want))
