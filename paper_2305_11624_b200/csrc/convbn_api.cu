@@ -628,12 +628,12 @@ int run_param_grads(const convbn_desc *d, const Problem &pb, const Plan &pl, con
                     const void *w, const float *vec3, const float *b, const float *mean, float *dw, float *db,
                     float *dgamma, float *dbeta, void *ws, cudaStream_t st, const char **which, bool scale_only = false) {
     float *partials = (float *)at(ws, pl.partials), *bsum = (float *)at(ws, pl.bsum);
+    const bool need_bsum = (vec3 || db) && !scale_only;
     if (f32_path(d, pb))
-        if (const int groups = f32_wgrad_groups(pb); groups > 0) {
+        if (const int groups = f32_wgrad_groups(pb, need_bsum); groups > 0) {
             *which = "direct";
             return run_f32_bwd(d, pb, groups, partials, bsum, dz, x, w, nullptr, nullptr, vec3, b, mean, dw, db, dgamma, dbeta, st);
         }
-    const bool need_bsum = (vec3 || db) && !scale_only;
     const bool tc = pl.grouped_wgrad || pl.umma_wgrad || pl.stem;   // tensor-core paths sum dZ inside the GEMM
     if (need_bsum && !tc && !pl.dw_tma_wgrad)
         LAUNCH("channel_sum", launch_channel_sum_partial(pb, d->dtype, d->layout, dz, bsum, pl.bsplits, st));
@@ -958,7 +958,7 @@ static int tune_bwd_impl(const convbn_desc *desc, const void *dz, const void *x,
         return CONVBN_EALIGN;
     const Plan pl = make_plan(desc, pb, CONVBN_PHASE_TUNE_BWD);
     CK(check_ws(pl, workspace, workspace_bytes));
-    if (const int groups = f32_path(desc, pb) ? f32_wgrad_groups(pb) : 0; groups > 0) {            // both passes in one launch
+    if (const int groups = f32_path(desc, pb) ? f32_wgrad_groups(pb, true) : 0; groups > 0) {            // both passes in one launch
         cudaStream_t st = (cudaStream_t)stream;
         float *partials = nullptr, *bsum = nullptr;
         if (groups > 1) {

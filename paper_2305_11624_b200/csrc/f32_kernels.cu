@@ -123,7 +123,7 @@ constexpr int conv_smem_floats(int kk, int r, int s, int ic) {
 }
 
 template <int K, int R, int S>
-__global__ void __launch_bounds__(kFThreads, S == 1 ? 5 : 4) f32_fwd_kernel(const F32Conv c, const BnFold fold) {
+__global__ void __launch_bounds__(kFThreads, K == 1 ? 8 : (S == 1 ? 5 : 4)) f32_fwd_kernel(const F32Conv c, const BnFold fold) {
     extern __shared__ __align__(16) float f32_smem[];
     constexpr int OCT = S == 1 ? 4 * R : R;
     __shared__ float scale_s[OCT], shift_s[OCT];
@@ -371,33 +371,35 @@ bool f32_conv_eligible(const Problem &pb) {
 
 // How many clusters share four output channels (their sums then go through launch_wgrad_epilogue), or 0: the direct kernels
 // take the parameter gradients.  The least time by a model of microseconds, fitted to 400 layers (1 to 128 channels, planes of
-// 1 x 1 to 200 x 200, N = 1 to 20000) at up to 13 counts each: on average 2 % above the best of them, in one layer more than
-// 5 % above the direct kernels.  A block's row bands go by one after the other, each a staging pass and its multiply-adds; the
-// direct kernels' threads go through the pixels of a slice.  One cluster whatever the pixels left few output channels to few
-// blocks: 1x1 64 -> 8 at 56 x 56, N = 16 340 us, now 51, direct 145.  Planes narrower than a run of pixels
-// in many images stay with the direct kernels: 1x1 1 -> 89 on 6876 rows 991 us with one cluster, direct 46.
-int f32_wgrad_groups(const Problem &pb) {
+// 1 x 1 to 200 x 200, N = 1 to 20000) at up to 13 counts each: on average 2 % above the best of them.  A block's row bands go by one after the other, each a staging pass and its multiply-adds;
+// the direct kernels' threads go through the pixels of a slice.  One cluster whatever the pixels left few output channels to few
+// blocks: 1x1 64 -> 8 at 56 x 56, N = 16 340 us, now 51, direct 145.  Planes narrower than a run of pixels in many images stay
+// with the direct kernels: 1x1 1 -> 89 on 6876 rows 991 us with one cluster, direct 46.
+int f32_wgrad_groups(const Problem &pb, bool need_sums) {
     F32Wgrad g;
     size_t bytes;
     if (!wgrad_geometry(pb, &g, &bytes)) return 0;
-    const int kk = pb.kh * pb.kw, items = g.n * g.bands, npg = kFThreads / (2 * g.cip), slots = 2 * device_sm_count();
+    const int kk = pb.kh * pb.kw, items = g.n * g.bands, npg = kFThreads / (2 * g.cip), lines = (pb.kdim + 255) / 256;
     const int blocks = (pb.c_out + kFCo - 1) / kFCo * kFCluster, inner = (g.rows * (g.zp / kFRun) + npg - 1) / npg * kFRun;
-    const double stage = (double)(g.c_in * (g.rows + pb.kh - 1) * g.xp + kFCo * g.rows * g.zp) / kFThreads;
-    const double item = 0.95 + 0.0049 * inner * kk + 0.176 * stage;
-    // the partial sums live in the direct kernels' workspace, and no thread adds up more pixels than one of those would
-    const int slices = direct_wgrad_splits(pb), sums = channel_sum_splits(pb), limit = slices < sums ? slices : sums;
-    const double chain = (double)pb.p / slices > 256.0 ? (double)pb.p / slices : 256.0;
-    const double rounds = (double)pb.c_out * pb.kdim * slices / (2048.0 * device_sm_count());
-    const int lines = (pb.kdim + 255) / 256;            // of the finishing kernel's threads
+    const int steps = (g.c_in * (g.rows + pb.kh - 1) * g.xp + kFThreads - 1) / kFThreads + (kFCo * g.rows * g.zp + kFThreads - 1) / kFThreads;
+    // (what the fit leaves out: the bands of one- and two-pixel rows take about half as long again)
+    const double item = (0.72 + 0.0041 * inner * kk + 0.195 * steps) * (pb.w_out <= 2 ? 1.5 : 1.0);
+    const int per_sm = 227 * 1024 / ((int)bytes + 5 * 1024), slots = device_sm_count() * (per_sm < 1 ? 1 : (per_sm > 4 ? 4 : per_sm));
+    // The partial sums live in the direct kernels' workspace; no thread adds up more pixels than one of those would, or 512;
+    // and thousands of clusters take longer to launch than they save (16292 rows, 1 -> 1, by 512 groups: 73 us, direct 30).
+    const int slices = direct_wgrad_splits(pb), sums = channel_sum_splits(pb), most = slices < sums ? slices : sums, limit = most < 64 ? most : 64;
+    const double chain = (double)pb.p / slices > 512.0 ? (double)pb.p / slices : 512.0;
+    const double waves = (double)pb.c_out * pb.kdim * slices / (2048.0 * device_sm_count());
+    // (sum dZ is a kernel of its own there; without it, in Eval mode, the direct kernels beside f32_bwd_kernel's dX were measured
+    // to take 10 us more than the two alone; times 1.1: with that least is lost where the two are close)
+    double best_cost = 1.1 * ((need_sums ? 6.0 + 0.166 * pb.p / sums : 14.0) +
+                              (0.25 + (waves > 1.0 ? 1.57 * (waves - 1.0) : 0.0)) * pb.p / slices + 0.034 * slices * lines);
     int best = 0;
-    // (times 1.2: with that least is lost where the two are close)
-    double best_cost = 1.2 * (6.0 + (0.25 + (rounds > 1.0 ? 1.57 * (rounds - 1.0) : 0.0)) * pb.p / slices + 0.166 * pb.p / sums +
-                              0.034 * slices * lines);
     for (int groups = 1; groups <= limit; groups += 1 + groups / 4) {
         const int per_block = (items + kFCluster * groups - 1) / (kFCluster * groups);
-        if ((double)per_block * inner > chain && groups + 1 + groups / 4 <= limit) continue;
-        const double waves = (double)blocks * groups > slots ? (double)blocks * groups / slots : 1.0;
-        const double cost = 3.8 + (groups > 1 ? 3.0 + 0.02 * groups * lines : 0.0) + per_block * item * waves;
+        if (per_block > 1 && (double)per_block * inner > chain && groups + 1 + groups / 4 <= limit) continue;
+        const long long rounds = ((long long)blocks * groups + slots - 1) / slots;
+        const double cost = 3.8 + (groups > 1 ? 2.6 + 0.02 * groups * lines : 0.0) + 2.2 * (rounds - 1) + per_block * item * rounds;
         if (cost < best_cost) { best_cost = cost; best = groups; }
     }
     return best;

@@ -57,7 +57,7 @@ cudaError_t launch_f32_fwd(const Problem &pb, const float *x, const float *w, co
 cudaError_t launch_f32_bwd(const Problem &pb, const float *dz, const float *x, const float *w, const float *scale, float *dx,
                            const float *vec3, const float *b, const float *mean, float *dw, float *db, float *dgamma,
                            float *dbeta, int groups, float *partials, float *bsum, cudaStream_t st);
-int f32_wgrad_groups(const Problem &pb);      // 0: the direct kernels are faster
+int f32_wgrad_groups(const Problem &pb, bool need_sums);      // 0: the direct kernels are faster
 
 // ---- tensor-core implicit-GEMM convolution (bf16 NHWC, groups = 1) -----------------------------
 // out[n,ho,wo,:cn] = bias + sum over taps (r,q) and channels c of
