@@ -184,7 +184,9 @@ int convbn_tune_bwd(const convbn_desc *desc, const void *dz, const void *x, cons
  * itself performs no cudaMalloc / cudaFree and calls no allocating routine.
  *
  *   - Limit: if convbn_workspace_bytes(desc, CONVBN_PHASE_TUNE_BWD_WEIGHT) exceeds 16 MiB
- *     (16 * 2^20 bytes) the call returns CONVBN_ECAPACITY and launches nothing.
+ *     (16 * 2^20 bytes) the call cuts the pixels of a dense tensor-core layer into fewer slices (the
+ *     same sums, added in another order than convbn_tune_bwd_weight adds them); if that does not fit
+ *     either it returns CONVBN_ECAPACITY and launches nothing.
  *   - The first call on each device looks up the array's device address (a runtime query, made with
  *     that device current).  Make that first call before starting any stream capture.
  *   - All calls share the one array.  It still holds the previous call's partial sums when a call

@@ -144,7 +144,8 @@ bool fused_bwd_path(const convbn_desc *d, const Problem &pb) {
 bool strided_dgrad_ok(const convbn_desc *d, const Problem &pb);
 bool umma_dgrad_shape(const convbn_desc *d, const Problem &pb, UmmaConvShape *s);
 
-Plan make_plan(const convbn_desc *d, const Problem &pb, int phase) {
+// bounded: the tensor-core weight gradient in the slices of a call with a fixed scratch.
+Plan make_plan(const convbn_desc *d, const Problem &pb, int phase, bool bounded = false) {
     Plan pl;
     UmmaConvShape us;
     if (phase == CONVBN_PHASE_TUNE_BWD) {
@@ -190,7 +191,7 @@ Plan make_plan(const convbn_desc *d, const Problem &pb, int phase) {
     const size_t wbd_bytes = grouped ? (size_t)pb.c_out * pb.kh * pb.kw * 64 * elem_size(d->dtype) : 0;
     pl.grouped_wgrad = grouped;
     if (grouped) {
-        pl.uw = umma_wgrad_plan(pb);
+        pl.uw = bounded ? umma_wgrad_plan_bounded(pb) : umma_wgrad_plan(pb);
         pl.bsplits = pl.uw.splits;
         part_bytes = (size_t)pl.uw.splits * (pb.c_out / 64) * pb.kh * pb.kw * 64 * 64 * sizeof(float);
         const int slots = grouped8_eligible(pb) ? grouped8_wgrad_slots(pb) : 0;
@@ -215,7 +216,7 @@ Plan make_plan(const convbn_desc *d, const Problem &pb, int phase) {
         }
     }
     if (pl.umma_wgrad) {
-        pl.uw = umma_wgrad_plan(pb);
+        pl.uw = bounded ? umma_wgrad_plan_bounded(pb) : umma_wgrad_plan(pb);
         pl.bsplits = pl.uw.splits;
         part_bytes = wrows * pl.uw.splits * sizeof(float);
     }
@@ -847,10 +848,9 @@ int convbn_tune_bwd_data(const convbn_desc *desc, const void *dz, const void *w,
     return tune_bwd_data_impl(desc, dz, w, saved, dx, PostOp(), workspace, workspace_bytes, stream);
 }
 
-int convbn_tune_bwd_weight(const convbn_desc *desc, const void *dz, const void *x, const void *w,
-                           const float *b, const float *run_mean, const void *saved, float *dw,
-                           float *db, float *dgamma, float *dbeta, void *workspace,
-                           size_t workspace_bytes, void *stream) {
+static int tune_bwd_weight_impl(const convbn_desc *desc, const void *dz, const void *x, const void *w, const float *b,
+                                const float *run_mean, const void *saved, float *dw, float *db, float *dgamma, float *dbeta,
+                                void *workspace, size_t workspace_bytes, void *stream, bool bounded) {
     HalfCall half(desc);              // CONVBN_F16: checked here, then run as the 16-bit path with the half flag set
     if (half.status != CONVBN_OK) return half.status;
     desc = half.use;
@@ -864,12 +864,18 @@ int convbn_tune_bwd_weight(const convbn_desc *desc, const void *dz, const void *
         !aligned(dw, 16) || !aligned(b, 4) || !aligned(run_mean, 4) || !aligned(db, 4) ||
         !aligned(dgamma, 4) || !aligned(dbeta, 4))
         return CONVBN_EALIGN;
-    const Plan pl = make_plan(desc, pb, CONVBN_PHASE_TUNE_BWD_WEIGHT);
+    const Plan pl = make_plan(desc, pb, CONVBN_PHASE_TUNE_BWD_WEIGHT, bounded);
     CK(check_ws(pl, workspace, workspace_bytes));
     cudaStream_t st = (cudaStream_t)stream;
     CK(run_param_grads(desc, pb, pl, dz, x, w, (const float *)saved, b, run_mean, dw, db, dgamma, dbeta,
                        workspace, st, &t_last_kernel[CONVBN_PHASE_TUNE_BWD_WEIGHT]));
     return CONVBN_OK;
+}
+
+int convbn_tune_bwd_weight(const convbn_desc *desc, const void *dz, const void *x, const void *w, const float *b,
+                           const float *run_mean, const void *saved, float *dw, float *db, float *dgamma, float *dbeta,
+                           void *workspace, size_t workspace_bytes, void *stream) {
+    return tune_bwd_weight_impl(desc, dz, x, w, b, run_mean, saved, dw, db, dgamma, dbeta, workspace, workspace_bytes, stream, false);
 }
 
 }  // extern "C"
@@ -1673,15 +1679,15 @@ int convbn_tune_bwd_weight_noalloc(const convbn_desc *desc, const void *dz, cons
     t_prof_phase = "bwd_weight";
     CK(make_problem(desc, &pb));
     CK(check_pair(desc));
-    const size_t need = make_plan(desc, pb, CONVBN_PHASE_TUNE_BWD_WEIGHT).total;
-    if (need > (size_t)CONVBN_NOALLOC_SCRATCH_BYTES) return CONVBN_ECAPACITY;
+    const size_t room = (size_t)CONVBN_NOALLOC_SCRATCH_BYTES;
+    const bool bounded = make_plan(desc, pb, CONVBN_PHASE_TUNE_BWD_WEIGHT).total > room;
+    if (bounded && make_plan(desc, pb, CONVBN_PHASE_TUNE_BWD_WEIGHT, true).total > room) return CONVBN_ECAPACITY;
     void *scratch = nullptr;
     CK(noalloc_scratch_address(&scratch));
     // Same kernels as convbn_tune_bwd_weight, with the built-in array standing in for the caller's
-    // workspace.  Every scratch word those kernels read is written earlier in the same call, so
+    // workspace, and in the same slices wherever those fit.  Every scratch word those kernels read is written earlier in the same call, so
     // nothing left over from a previous call has to be cleared.
-    return convbn_tune_bwd_weight(desc, dz, x, w, b, run_mean, saved, dw, db, dgamma, dbeta, scratch,
-                                  (size_t)CONVBN_NOALLOC_SCRATCH_BYTES, stream);
+    return tune_bwd_weight_impl(desc, dz, x, w, b, run_mean, saved, dw, db, dgamma, dbeta, scratch, room, stream, bounded);
 }
 
 const char *convbn_status_string(int status) {

@@ -138,6 +138,7 @@ struct UmmaWgradPlan {
 };
 bool umma_wgrad_eligible(const Problem &pb);
 UmmaWgradPlan umma_wgrad_plan(const Problem &pb);
+UmmaWgradPlan umma_wgrad_plan_bounded(const Problem &pb);     // for calls with a fixed scratch
 // partials: [splits][C_out][kdim] fp32 (the layout of the weights; block-diagonal: [splits][block][k][64])
 // bsum    : [splits][C_out] fp32 per-slice sums of dZ over pixels (from a ones row in the GEMM)
 // counters: `ncounters` words zeroed for an epilogue that counts its blocks (may be NULL)

@@ -290,25 +290,17 @@ bool umma_wgrad_eligible(const Problem &pb) {
 static int wgrad_bn(const Problem &pb) { return pb.c_out >= 128 ? 128 : 64; }
 static int stem_wgrad_bn(const Problem &pb) { return pb.c_out >= 256 ? 256 : wgrad_bn(pb); }
 
-UmmaWgradPlan umma_wgrad_plan(const Problem &pb) {
+// Output tiles of bn columns (k rows of the ones slice included).
+static long long wgrad_tiles(const Problem &pb, int bn) {
+    const long long kd = pb.groups > 1 ? (long long)pb.kh * pb.kw * 64 : pb.kdim;
+    return (kd / 64 + 1 + 1) / 2 * ((pb.c_out + bn - 1) / bn);
+}
+
+// The slice count minimises  rounds over the resident slots x (pixels per slice + a fixed cost per
+// CTA, in pixels) + a small cost per slice for the epilogue that adds the slices up; a grid a few
+// CTAs larger than the slots would otherwise run a second, nearly empty round.
+static UmmaWgradPlan wgrad_slices(const Problem &pb, long long tiles, long long slots) {
     UmmaWgradPlan pl;
-    const bool bd = pb.groups > 1;
-    const int bn = bd ? 64 : wgrad_bn(pb);
-    const long long kd = bd ? (long long)pb.kh * pb.kw * 64 : pb.kdim;
-    const long long m_tiles = (kd / 64 + 1 + 1) / 2, n_tiles = (pb.c_out + bn - 1) / bn;   // + the ones slice
-    // Resident CTAs: two per SM (the stage rings are sized for it, launch_w): one's partial tile leaves while the other
-    // multiplies.  A deeper ring for one CTA gains nothing.
-    // The slice count minimises  rounds over the resident slots x (pixels per slice + a fixed cost per
-    // CTA, in pixels) + a small cost per slice for the epilogue that adds the slices up; a grid a few
-    // CTAs larger than the slots would otherwise run a second, nearly empty round.
-    // Few tiles mean many slices, and where those are short the partial tensors weigh more than what a second CTA hides: up to
-    // 24 tiles with slices of up to 2048 pixels get one CTA per SM (N = 32: 1x1 128 -> 512 at 28 x 28 15.3 -> 13.4 us, 1024 ->
-    // 256 at 14 x 14 13.3 -> 11.4, 3x3 128 at 28 x 28 17.6 -> 15.5; but 3x3 256 at 14 x 14, 38 tiles, 15.8 -> 18.1, and 1x1
-    // 128 -> 512 at 28 x 28, N = 256 58.3 -> 73.6).  Not where output rows are shorter than four pixels: the boxes of X then
-    // arrive pixel by pixel and a second CTA hides that (29173 rows, 1024 -> 64: 44.5 and 27.4 us; 2 x 2 about even; from
-    // 4 x 4 on one CTA is the faster).
-    const long long tiles = m_tiles * n_tiles, sms = device_sm_count();
-    const long long slots = sms * (tiles <= 24 && pb.p * tiles <= 2048 * sms && pb.w_out >= 4 ? 1 : 2);
     const long long max_splits = (pb.p + 4 * kWP - 1) / (4 * kWP);     // at least 256 pixels per slice
     long long splits = 1;
     double best_cost = -1.0;
@@ -323,6 +315,26 @@ UmmaWgradPlan umma_wgrad_plan(const Problem &pb) {
     pl.per_split = per;
     pl.splits = (int)((pb.p + per - 1) / per);
     return pl;
+}
+
+UmmaWgradPlan umma_wgrad_plan(const Problem &pb) {
+    // Resident CTAs: two per SM (the stage rings are sized for it, launch_w): one's partial tile leaves while the other
+    // multiplies.  A deeper ring for one CTA gains nothing.
+    // Few tiles mean many slices, and where those are short the partial tensors weigh more than what a second CTA hides: up to
+    // 24 tiles with slices of up to 2048 pixels get one CTA per SM (N = 32: 1x1 128 -> 512 at 28 x 28 15.3 -> 13.4 us, 1024 ->
+    // 256 at 14 x 14 13.3 -> 11.4, 3x3 128 at 28 x 28 17.6 -> 15.5; but 3x3 256 at 14 x 14, 38 tiles, 15.8 -> 18.1, and 1x1
+    // 128 -> 512 at 28 x 28, N = 256 58.3 -> 73.6).  Not where output rows are shorter than four pixels: the boxes of X then
+    // arrive pixel by pixel and a second CTA hides that (29173 rows, 1024 -> 64: 44.5 and 27.4 us; 2 x 2 about even; from
+    // 4 x 4 on one CTA is the faster).
+    const long long tiles = wgrad_tiles(pb, pb.groups > 1 ? 64 : wgrad_bn(pb)), sms = device_sm_count();
+    return wgrad_slices(pb, tiles, sms * (tiles <= 24 && pb.p * tiles <= 2048 * sms && pb.w_out >= 4 ? 1 : 2));
+}
+
+// The slices of a call whose scratch is bounded, where the plan above wants more than there is: 256 columns count as one tile
+// with an SM of its own, which makes fewer slices of wide layers (3x3 768 -> 384 at 13 x 13, N = 12: 10 MiB, above 30).
+UmmaWgradPlan umma_wgrad_plan_bounded(const Problem &pb) {
+    const int bn = pb.groups > 1 ? 64 : (pb.c_out >= 256 ? 256 : wgrad_bn(pb));
+    return wgrad_slices(pb, wgrad_tiles(pb, bn), (long long)device_sm_count() * (bn == 256 ? 1 : 2));
 }
 
 int wgrad_kmajor_rows(const Problem &pb) { return (pb.kdim + 1) / 2; }

@@ -68,6 +68,27 @@ def test_workspace_sizes_of_the_benchmark_layers():
                 assert wsw <= 16 << 20, (sp.name, wsw)
 
 
+def test_which_layers_the_no_allocation_call_takes():
+    """Decided by the layer alone, on the host, before any pointer is looked at: a scratch of up to 16 MiB, or one that fewer
+    slices bring down to that (the second and third layer)."""
+    one = dict(dtype=C.BF16, layout=C.NHWC)
+    taken = [good(n=2, c_in=64, h_in=20, w_in=24, c_out=128, kh=3, kw=3, pad_h=1, pad_w=1, **one),
+             good(n=12, c_in=768, h_in=13, w_in=13, c_out=384, kh=3, kw=3, pad_h=1, pad_w=1, **one),
+             good(n=2, c_in=1600, h_in=25, w_in=25, c_out=1856, kh=1, kw=1, pad_h=0, pad_w=0, **one)]
+    refused = [good(n=8, c_in=1024, h_in=7, w_in=7, c_out=1024, kh=3, kw=3, pad_h=1, pad_w=1, **one),
+               good(n=16, c_in=512, h_in=56, w_in=56, c_out=512, kh=3, kw=3, pad_h=1, pad_w=1, **one)]
+    assert C.convbn_workspace_bytes(taken[0], C.PHASE_TUNE_BWD_WEIGHT) <= 16 << 20
+    assert all(C.convbn_workspace_bytes(d, C.PHASE_TUNE_BWD_WEIGHT) > 16 << 20 for d in taken[1:])
+
+    def status(d):                     # dz = NULL: a layer that is taken gets as far as the pointer checks
+        with pytest.raises(C.ConvBNError) as e:
+            C.convbn_tune_bwd_weight_noalloc(d, None, 4096, 4096, None, 4096, 4096, 4096, None, 4096, 4096, stream=0)
+        return e.value.status
+
+    assert [status(d) for d in refused] == [C.ECAPACITY] * 2
+    assert all(status(d) != C.ECAPACITY for d in taken)
+
+
 @pytest.mark.parametrize("kw", [
     dict(n=0), dict(c_in=-1), dict(kh=0), dict(stride_h=0), dict(dil_w=0), dict(pad_h=-1),
     dict(groups=3), dict(groups=0), dict(h_in=1, w_in=1, pad_h=0, pad_w=0), dict(dtype=7),

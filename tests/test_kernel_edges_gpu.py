@@ -149,3 +149,23 @@ def test_captured_backward_equals_the_plain_call(spec):
     graph.replay()
     C.convbn_check()
     assert all(torch.equal(a, b) for a, b in zip(outs, want))
+
+
+def test_no_allocation_call_in_fewer_slices():
+    """A layer whose parameter-gradient scratch exceeds the built-in array: the call cuts it into fewer slices."""
+    from paper_2305_11624_b200 import convbn as C
+    from paper_2305_11624_b200.harness import Block
+    spec = L("few_slices", 2, 384, 33, 4, 640, 3, 3, pad=1, bias=True)
+    t = parity.make_inputs(spec, 12)
+    ref = parity.oracle_tune(spec, t)
+    blk = Block(spec)
+    assert C.convbn_workspace_bytes(blk.desc, C.PHASE_TUNE_BWD_WEIGHT) > 16 << 20
+    blk.load(t)
+    blk.tune_fwd()
+    for o in (blk.dw, blk.db, blk.dgamma, blk.dbeta):
+        o.fill_(float("nan"))
+    C.convbn_tune_bwd_weight_noalloc(blk.desc, blk.dz, blk.x, blk.w, blk.b, blk.mu_hat, blk.saved, blk.dw, blk.db, blk.dgamma,
+                                     blk.dbeta)
+    C.convbn_check()
+    parity.compare({k: blk.fetch(k) for k in ("dw", "db", "dgamma", "dbeta")}, ref, parity.TOL["bf16"],
+                   ("dw", "db", "dgamma", "dbeta"), spec.name, dtype=spec.dtype)
