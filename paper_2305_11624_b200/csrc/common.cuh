@@ -81,8 +81,6 @@ __device__ __forceinline__ void unpack2_t(uint32_t bits, float &lo, float &hi) {
     if constexpr (F16) { const float2 f = __half22float2(*reinterpret_cast<const __half2 *>(&bits)); lo = f.x; hi = f.y; }
     else { lo = __uint_as_float(bits << 16); hi = __uint_as_float(bits & 0xFFFF0000u); }
 }
-// max(v, 0) of two finite 16-bit values: a set sign bit clears its half
-__device__ __forceinline__ uint32_t relu2_h16(uint32_t v) { return v & ~(((v >> 15) & 0x00010001u) * 0xFFFFu); }
 // What a residual network does next with a block's result, on eight 16-bit values: v + a (rounded again, as an add of two
 // stored tensors is), max(v, 0), v where m > 0 and 0 elsewhere.  Two values per instruction: the 16-bit sum is the rounded
 // exact one, which an fp32 sum rounded to 16 bits is too (24 >= 2 * 11 + 2 significant bits).

@@ -341,7 +341,7 @@ __global__ void __launch_bounds__(kWinThreads) stem_window_fwd_kernel(const __gr
                                     pk.y = pack2_t<H>(fmaf(__uint_as_float(v[j + 2]), s0.z, b0.z), fmaf(__uint_as_float(v[j + 3]), s0.w, b0.w));
                                     pk.z = pack2_t<H>(fmaf(__uint_as_float(v[j + 4]), s1.x, b1.x), fmaf(__uint_as_float(v[j + 5]), s1.y, b1.y));
                                     pk.w = pack2_t<H>(fmaf(__uint_as_float(v[j + 6]), s1.z, b1.z), fmaf(__uint_as_float(v[j + 7]), s1.w, b1.w));
-                                    if constexpr (RELU) { pk.x = relu2_h16(pk.x); pk.y = relu2_h16(pk.y); pk.z = relu2_h16(pk.z); pk.w = relu2_h16(pk.w); }
+                                    if constexpr (RELU) pk = post_chunk<H>(pk, false, pk, true, false, pk);
                                     *(uint4 *)(row + (((4 * half + (j >> 3)) ^ (lane & 7)) << 4)) = pk;
                                 }
                             }

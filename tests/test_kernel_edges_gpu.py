@@ -129,6 +129,28 @@ def test_glue_in_the_epilogue_equals_the_passes(spec):
     C.convbn_check()
 
 
+@pytest.mark.parametrize("spec", [s for s in GLUE if s.name in ("glue_stem", "glue_1x1", "glue_strip_small", "glue_pair", "glue_dw", "glue_f32")],
+                         ids=lambda s: s.name)
+def test_fused_relu_of_non_finite_values(spec):
+    """NaN becomes 0 in every kernel's ReLU, as in convbn_relu; infinities and the other values are those of the passes."""
+    import torch
+    from paper_2305_11624_b200 import convbn as C
+    from paper_2305_11624_b200.harness import Block
+    blk = Block(spec)
+    blk.randomize(4)
+    for at, v in ((7, float("nan")), (blk.x.numel() // 2, float("inf")), (blk.x.numel() - 3, -float("inf"))):
+        blk.x[at] = v
+    blk.tune_fwd()
+    want = torch.empty_like(blk.z)
+    C.convbn_relu(blk.z, want)
+    assert bool(blk.z.isnan().any()) and not bool(want.isnan().any())
+    blk.z.fill_(float("nan"))
+    C.convbn_tune_fwd_glue(blk.desc, blk.x, blk.w, blk.b, blk.gamma, blk.beta, blk.mu_hat, blk.var_hat, blk.z, blk.saved, None,
+                           True, blk.workspace)
+    C.convbn_check()
+    assert torch.equal(blk.z, want)
+
+
 @pytest.mark.parametrize("spec", [L("cap_3x3", 2, 64, 20, 24, 64, 3, 3, pad=1), L("cap_grouped", 2, 64, 12, 13, 64, 3, 3, pad=1, groups=8),
                                   L("cap_f32", 9, 40, 19, 23, 7, 3, 3, pad=1, dtype="f32", layout="nchw")], ids=lambda s: s.name)
 def test_captured_backward_equals_the_plain_call(spec):
