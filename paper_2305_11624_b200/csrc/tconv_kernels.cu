@@ -94,7 +94,7 @@ __global__ void __launch_bounds__(256) tconv_param_epilogue_kernel(int c_out, in
     }
 }
 
-// Block (bx, by): input channels [32 bx, +32) x weight columns k = (tap, co) [32 by, +32), one output channel group since
+// Block (bx, by): weight columns k = (tap, co) [32 bx, +32) x input channels [32 by, +32), one output channel group since
 // 32 divides C_out.  Thread (tx = k, ty = ci) adds its element of part[split][C_in][k] over the slices, eight loads in
 // flight, in slice order, scales it by s[co] and stores it.  The last block of a group of 32
 // output channels (a counter) adds the dot products and the sums of dZ in fixed order.  Bound by the read of the
@@ -113,7 +113,7 @@ __global__ void __launch_bounds__(1024) tconv_wgrad_epilogue_kernel(int c_in, in
     pdl_wait();
     pdl_launch_dependents();
     const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
-    const int ci0 = blockIdx.x * 32, k0 = blockIdx.y * 32, co0 = k0 % c_out;
+    const int k0 = blockIdx.x * 32, ci0 = blockIdx.y * 32, co0 = k0 % c_out;       // (the longer dimension is the unbounded one)
     const float wv = load_h16(w + (size_t)(ci0 + ty) * kdim + k0 + tx, f16);
     const float *src = part + (size_t)(ci0 + ty) * kdim + k0 + tx;
     const size_t slice = (size_t)kdim * c_in;
@@ -132,12 +132,12 @@ __global__ void __launch_bounds__(1024) tconv_wgrad_epilogue_kernel(int c_in, in
         float d = prod[tx][ty];                         // warp ty adds the 32 input channels of row k0 + ty
 #pragma unroll
         for (int o = 16; o > 0; o >>= 1) d += __shfl_xor_sync(0xffffffffu, d, o);
-        if (tx == 0) dotpart[(size_t)blockIdx.x * kdim + k0 + ty] = d;
+        if (tx == 0) dotpart[(size_t)blockIdx.y * kdim + k0 + ty] = d;
     }
     __syncthreads();
     if (threadIdx.x == 0) {
         __threadfence();
-        const unsigned int per_group = gridDim.x * (unsigned)(kdim / c_out);
+        const unsigned int per_group = gridDim.y * (unsigned)(kdim / c_out);
         is_last = atomicAdd(&counters[co0 / 32], 1u) == per_group - 1;
     }
     __syncthreads();
@@ -145,7 +145,7 @@ __global__ void __launch_bounds__(1024) tconv_wgrad_epilogue_kernel(int c_in, in
     __threadfence();
     // thread (tx = channel, ty = row group): rows of dotpart are (input-channel block, tap), then the slices of sum dZ
     float d = 0.f, sum = 0.f;
-    const int taps = kdim / c_out, rows = (int)gridDim.x * taps;
+    const int taps = kdim / c_out, rows = (int)gridDim.y * taps;
     for (int r = ty; r < rows; r += 32) d += __ldcg(dotpart + (size_t)(r / taps) * kdim + (r % taps) * c_out + co0 + tx);
     for (int sp = ty; sp < bsplits; sp += 128) {
         float q[4];
@@ -186,7 +186,7 @@ cudaError_t launch_tconv_wgrad_epilogue(int c_in, int c_out, int taps, const flo
                                         float *dgamma, float *dbeta, cudaStream_t st) {
     static PerDevice carve;
     prefer_max_shared_once(tconv_wgrad_epilogue_kernel, &carve);
-    return launch_pdl(tconv_wgrad_epilogue_kernel, dim3(c_in / 32, taps * c_out / 32), dim3(1024), 0, st, c_in, c_out,
+    return launch_pdl(tconv_wgrad_epilogue_kernel, dim3(taps * c_out / 32, c_in / 32), dim3(1024), 0, st, c_in, c_out,
                       taps * c_out, part, splits, (const __nv_bfloat16 *)w, vec3, b, mean, bsum, bsplits, dotpart, counters,
                       dw, db, dgamma, dbeta, call_f16());
 }

@@ -78,6 +78,37 @@ def test_tconv_block(case):
     test_tconv.test_library_matches_the_oracle(case)
 
 
+def test_tconv_gradients_of_a_kernel_with_many_taps():
+    """More than 65535 blocks of 32 weight columns: one input pixel, whose weight gradient is an outer product."""
+    import torch
+    from paper_2305_11624_b200 import convbn as C
+    ci, co, k = 64, 128, 129
+    dev = "cuda:0"
+    desc = C.Desc.make(1, ci, 1, 1, co, k, k, dtype=C.BF16, layout=C.NHWC)
+    assert C.convbn_tconv_out_shape(desc) == (k, k) and k * k * co // 32 > 65535
+    gen = torch.Generator(device=dev)
+    gen.manual_seed(6)
+    rn = lambda *s: torch.randn(*s, generator=gen, device=dev)
+    x, w, dz = rn(ci).bfloat16(), rn(ci, k * k, co).bfloat16(), rn(k * k, co).bfloat16()
+    saved, mean = rn(3 * co), rn(co)
+    dx, dw, dgamma, dbeta = torch.empty_like(x), torch.empty(ci, k * k, co, device=dev), rn(co), rn(co)
+    ws = torch.empty(C.convbn_tconv_workspace_bytes(desc), dtype=torch.uint8, device=dev)
+    C.convbn_tconv_tune_bwd(desc, dz, x, w, None, mean, saved, dx, dw, None, dgamma, dbeta, ws)
+    C.convbn_check()
+    s, r, sums = saved[:co].double(), saved[2 * co:].double(), dz.double().sum(0)
+    close = lambda got, want, tol: assert_close(got.double(), want, tol)
+
+    def assert_close(got, want, tol):
+        assert bool(((got - want).norm() <= tol * want.norm()).item()), float((got - want).norm() / want.norm())
+
+    for i in range(0, ci, 16):
+        close(dw[i:i + 16], s * (x[i:i + 16, None, None].double() * dz.double()), 1e-6)      # one rounding of the product, one of s
+    dot = sum((x[i].double() * dz.double() * w[i].double()).sum(0) for i in range(ci))
+    close(dbeta, sums, 1e-5)
+    close(dgamma, r * (dot - sums * mean.double()), 1e-5)
+    close(dx, torch.stack([(w[i].double() * s * dz.double()).sum() for i in range(ci)]), parity.TOL["bf16"])
+
+
 GLUE = [  # every kernel whose epilogue does the glue, and one that leaves it to passes of its own
     L("glue_1x1", 3, 128, 9, 13, 320, 1, 1, dtype="f16"),                     # GEMM, a last tile of 64 columns
     L("glue_strided", 2, 64, 11, 9, 128, 3, 3, stride=2, pad=1),              # a GEMM per parity class
