@@ -94,7 +94,7 @@ def lib():
 
 def _ptr(t):
     """Address for a c_void_p parameter: a tensor's, an integer as it is, None for NULL."""
-    if t is None or type(t) is int:
+    if t is None or isinstance(t, int):
         return t
     return t.data_ptr()
 

@@ -159,6 +159,16 @@ def test_argument_checks_before_any_launch():
     assert e.value.status == C.EINVAL
 
 
+def test_addresses_may_be_integers_of_any_kind():
+    """Pointers, sizes and streams as plain integers or as subclasses of int (an address type of another package)."""
+    class Address(int):
+        pass
+    with pytest.raises(C.ConvBNError) as e:
+        C.convbn_tune_fwd(good(), Address(4096), 4096, None, 4096, 4096, 4096, 4096, 4096, Address(4096 + 8), Address(4096),
+                          Address(1 << 30), stream=Address(0))
+    assert e.value.status == C.EALIGN                       # `saved` is the one that is off
+
+
 def test_status_strings():
     assert C.status_string(C.OK) == "ok"
     assert "workspace" in C.status_string(C.EWORKSPACE)
