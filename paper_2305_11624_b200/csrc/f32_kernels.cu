@@ -24,6 +24,17 @@ constexpr int kFCluster = 8;        // blocks of a weight-gradient cluster
 constexpr int kFCo = 4;             // output channels of a cluster
 constexpr int kFRun = 8;            // consecutive pixels a thread slides its window over
 
+// Outside the image there is nothing to multiply: an infinite weight or dZ beside it must not become 0 x inf = NaN.  The
+// loops multiply by staged zeros there; a thread with a sum that is not finite at the end forms its sums again, from global
+// memory, without them.  (Looking at every value while it is staged cost the weight gradient 20 %.)
+template <int N>
+__device__ __forceinline__ bool all_finite(const float (&v)[N]) {
+    bool yes = true;
+#pragma unroll
+    for (int i = 0; i < N; ++i) yes = yes && fabsf(v[i]) < INFINITY;
+    return yes;
+}
+
 // out[n][oc][p] = scale[oc] sum_{ic, tap} act[n][ic][p + tap - pad] wt(oc, ic, tap) + shift[oc]
 struct F32Conv {
     const float *act, *w;
@@ -97,6 +108,24 @@ __device__ __forceinline__ void conv_tile(const F32Conv &c, int oc0, int tile, c
                     acc[j] = fmaf(v[t], q.x, acc[j]); acc[j + 1] = fmaf(v[t], q.y, acc[j + 1]);
                     acc[j + 2] = fmaf(v[t], q.z, acc[j + 2]); acc[j + 3] = fmaf(v[t], q.w, acc[j + 3]);
                 }
+        }
+    }
+    if (!all_finite(acc)) {
+        const int per = S == 1 ? c.ic : (c.ic + 3) / 4, lo = S == 1 ? 0 : grp * per, hi = min(c.ic, lo + per), o0 = oc0 + (S == 1 ? grp * R : 0);
+#pragma unroll
+        for (int j = 0; j < R; ++j) acc[j] = 0.f;
+#pragma unroll 1
+        for (int i = lo * KK; i < hi * KK; ++i) {
+            const int ci = i / KK, t = i - ci * KK, yy = y - c.pad + t / K, xx = x - c.pad + t % K;
+            if (!valid || yy < 0 || yy >= c.h || xx < 0 || xx >= c.wd) continue;
+            const float v = __ldg(c.act + (((size_t)img * c.ic + ci) * c.h + yy) * c.wd + xx);
+#pragma unroll
+            for (int j = 0; j < R; ++j) {
+                if (o0 + j >= c.oc) break;
+                const float w = DGRAD ? c.w[((size_t)ci * c.oc + o0 + j) * KK + KK - 1 - t] * (c.k_scale ? c.k_scale[ci] : 1.f)
+                                      : c.w[((size_t)(o0 + j) * c.ic + ci) * KK + t];
+                acc[j] = fmaf(v, w, acc[j]);
+            }
         }
     }
     if constexpr (S == 4) {
@@ -226,6 +255,33 @@ __device__ __forceinline__ void wgrad_cluster(const F32Wgrad &g, int co0, int gr
                         }
                 }
             }
+    }
+    if (ci < g.c_in && !(all_finite(acc[0]) && all_finite(acc[1]))) {
+#pragma unroll
+        for (int t = 0; t < KK; ++t) acc[0][t] = acc[1][t] = 0.f;
+#pragma unroll 1
+        for (int it = group * kFCluster + rank; it < items; it += g.groups * kFCluster) {
+            const int img = it / g.bands, y0 = (it - img * g.bands) * g.rows, nruns = min(g.rows, g.ho - y0) * runs;
+#pragma unroll 1
+            for (int i = pg * kFRun; i < nruns * kFRun; i += i % kFRun == kFRun - 1 ? (npg - 1) * kFRun + 1 : 1) {      // the same runs
+                const int r = i / g.zp, x = i - r * g.zp, y = y0 + r;
+                if (x >= g.wo) continue;
+                float d[2];
+#pragma unroll
+                for (int h = 0; h < 2; ++h) {
+                    const int o = co0 + 2 * pair + h;
+                    d[h] = o < g.c_out ? __ldg(g.dz + (((size_t)img * g.c_out + o) * g.ho + y) * g.wo + x) : 0.f;
+                }
+#pragma unroll
+                for (int t = 0; t < KK; ++t) {
+                    const int yy = y + t / K - g.pad, xx = x + t % K - g.pad;
+                    if (yy < 0 || yy >= g.h || xx < 0 || xx >= g.wd) continue;
+                    const float v = __ldg(g.x + (((size_t)img * g.c_in + ci) * g.h + yy) * g.wd + xx);
+                    acc[0][t] = fmaf(d[0], v, acc[0][t]);
+                    acc[1][t] = fmaf(d[1], v, acc[1][t]);
+                }
+            }
+        }
     }
     // pixel groups -> block: [thread][K K], then part[co][c_in K K + 1] (the last entry is sum dZ)
     __shared__ float sums[kFCo][kFThreads];

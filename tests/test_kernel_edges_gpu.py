@@ -65,6 +65,50 @@ def test_eval_block(spec):
     test_parity_gpu.test_eval_and_deploy_comparators(spec)
 
 
+@pytest.mark.parametrize("spec", [L("f32_inf", 2, 5, 9, 11, 6, 3, 3, pad=1, dtype="f32", layout="nchw"),
+                                  L("f32_inf_wide", 40, 18, 20, 21, 40, 3, 3, pad=1, dtype="f32", layout="nchw")], ids=lambda s: s.name)
+def test_fp32_block_does_not_multiply_by_its_padding(spec):
+    """Infinite values: the taps that lie outside the image are left out, as the definition of the convolution has it, and do
+    not add 0 x inf.  Against fp64 sums over the pixels inside the image: where those are finite, infinite, NaN."""
+    import numpy as np
+    from paper_2305_11624_b200 import convbn as C
+    from paper_2305_11624_b200.harness import Block
+    t = parity.make_inputs(spec, 21)
+    t["w"][1, 2, 0, 0] = np.inf                     # no tap (0, 0) at the first row and column
+    t["w"][3, 0, 2, 2] = -np.inf
+    t["x"][0, 1, 0, spec.w_in - 1] = np.inf
+    t["x"][1, 3, spec.h_in - 1, 4] = -np.inf
+    t["dz"][0, 2, spec.h_in - 1, 0] = np.inf
+    blk = Block(spec)
+    blk.load(t)
+    blk.tune_fwd()
+    blk.tune_bwd()
+    C.convbn_check()
+    n, h, w, k, p = spec.n, spec.h_in, spec.w_in, spec.kh, spec.pad
+    s = t["gamma"] / np.sqrt(t["var_hat"] + spec.eps)
+    sw = t["w"] * s[:, None, None, None]
+    z, dx, dw = np.zeros((n, spec.c_out, h, w)), np.zeros((n, spec.c_in, h, w)), np.zeros(t["w"].shape)
+    with np.errstate(invalid="ignore"):
+        for r in range(k):
+            for q in range(k):
+                o = tuple(slice(max(0, p - a), min(e, e + p - a)) for a, e in ((r, h), (q, w)))      # outputs with this tap inside
+                i = tuple(slice(v.start + a - p, v.stop + a - p) for v, a in zip(o, (r, q)))
+                xs, zs = t["x"][(slice(None), slice(None)) + i], t["dz"][(slice(None), slice(None)) + o]
+                each = lambda a, b, eq: sum(np.multiply(*np.broadcast_arrays(a(c), b(c))) for c in range(eq))
+                z[(slice(None), slice(None)) + o] += each(lambda c: xs[:, c, None], lambda c: t["w"][None, :, c, r, q, None, None], spec.c_in)
+                dx[(slice(None), slice(None)) + i] += each(lambda c: zs[:, c, None], lambda c: sw[c][None, :, r, q, None, None], spec.c_out)
+                for co in range(spec.c_out):
+                    dw[co, :, r, q] = (zs[:, co, None] * xs).sum(axis=(0, 2, 3))
+        z = z * s[None, :, None, None] + (-t["mu_hat"] * s + t["beta"])[None, :, None, None]
+        dw *= s[:, None, None, None]
+    for name, ref in (("z", z), ("dx", dx), ("dw", dw)):
+        got, ref = blk.fetch(name), ref.reshape(blk.fetch(name).shape)
+        assert np.array_equal(np.isnan(got), np.isnan(ref)), name
+        assert np.array_equal(np.isinf(got), np.isinf(ref)) and np.array_equal(np.sign(got[np.isinf(got)]), np.sign(ref[np.isinf(ref)])), name
+        fin = np.isfinite(ref)
+        assert fin.any() and not fin.all() and np.allclose(got[fin], ref[fin], rtol=1e-4, atol=1e-4 * np.abs(ref[fin]).max()), name
+
+
 TCONV = [  # (dtype, n, c_in, h, w, c_out, k, stride, pad, dil, groups, bias): kernel = stride, the GEMM on omega as it is
     ("bf16", 3, 64, 5, 7, 192, 2, 2, 0, 1, 1, True),        # tiles of 64 columns, fewer pixels than a tile
     ("f16", 1, 192, 13, 11, 64, 3, 3, 0, 1, 1, False),      # nine taps, a last tile of 15 pixels
