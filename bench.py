@@ -87,7 +87,8 @@ KIND_OF = {"strip_fwd": "fwd", "strip_dgrad": "dgrad", "direct_fwd": "fwd", "dir
            "umma_fwd": "fwd", "umma_dgrad": "dgrad", "umma_wgrad": "wgrad", "umma_bwd": "bwd",
            "dw_fwd": "fwd", "dw_dgrad": "dgrad", "dw_wgrad": "wgrad",
            "grouped_fwd": "fwd", "grouped_dgrad": "dgrad", "grouped_wgrad": "wgrad",
-           "stem_fwd": "fwd", "stem_dgrad": "dgrad", "stem_wgrad": "wgrad"}
+           "stem_fwd": "fwd", "stem_dgrad": "dgrad", "stem_wgrad": "wgrad",
+           "f32_fwd": "fwd", "f32_dgrad": "dgrad", "f32_wgrad": "wgrad", "f32_bwd": "bwd"}
 PHASE_KIND = {"fwd": "fwd", "bwd_data": "dgrad", "bwd_weight": "wgrad", "bwd": "bwd"}
 
 
@@ -694,6 +695,38 @@ def run_backbone(ctx, batch=32, size=224, iters=10):
     return out
 
 
+def short(v):
+    """Numbers with six digits, in containers too."""
+    if isinstance(v, float):
+        return float("%.6g" % v)
+    if isinstance(v, dict):
+        return {k: short(x) for k, x in v.items()}
+    return [short(x) for x in v] if isinstance(v, list) else v
+
+
+def result_line(args, world, workloads, value, ms_total, flops_total, launch, clocks, e2e, launches, roofline, cpu, backbone,
+                per_config):
+    """The result line, under 1500 characters, and the object with every figure behind it."""
+    pick = lambda d, *keys: None if d is None else {k: d.get(k) for k in keys}
+    line = {"metric": METRIC, "value": value, "unit": UNIT, "n_gpus": world, "steps": args.steps,
+            "warmup": args.warmup, "ms_per_step": ms_total / args.steps, "higher_is_better": True,
+            "scaling": "weak", "vs_baseline": None,
+            "dtype": "bf16" if any(w != 0 for w in workloads) else "f32", "data": "synthetic",
+            "config": {"workload": "; ".join(WORKLOAD_NAMES[w] for w in workloads if w in DENSE or len(workloads) == 1),
+                       "value_over": "total FLOPs / total time of one step of each",
+                       "l2": "rotating buffer sets, over twice the L2", "flops_per_step": flops_total,
+                       "parallelism": ("data parallel x%d, gradient all-reduce per step" if args.dp_allreduce and world > 1
+                                       else "replicas x%d") % world,
+                       "launch": launch},
+            "clocks": clocks, "e2e": pick(e2e, "value", "unit", "h2d_bytes_per_step", "d2h_bytes_per_step"),
+            "gpu_launches": launches,
+            "roofline": pick(roofline, "kernel", "layer", "bound", "achieved", "peak", "unit", "frac", "traffic"),
+            "cpu_baseline": pick(cpu, "value", "unit", "cores", "kind"),
+            "ms_per_config": {str(w): c.get("ms_per_step") for w, c in zip(workloads, per_config)}}
+    detail = {"roofline": roofline, "e2e": e2e, "cpu_baseline": cpu, "backbone": backbone, "per_config": per_config}
+    return short(line), detail
+
+
 def run_ours(args):
     import torch
     import torch.distributed as dist
@@ -753,23 +786,11 @@ def run_ours(args):
     if world > 1:
         dist.barrier()
     if rank == 0:
-        names = [WORKLOAD_NAMES[w] for w in workloads]
-        line = {"metric": METRIC, "value": value, "unit": UNIT, "n_gpus": world, "steps": args.steps,
-                "warmup": args.warmup, "ms_per_step": ms_total / args.steps, "higher_is_better": True,
-                "scaling": "weak", "vs_baseline": None,
-                "dtype": "bf16" if any(w != 0 for w in workloads) else "f32", "data": "synthetic",
-                "config": {"workload": "; ".join(names),
-                           "value_over": "configs %s (dense bf16): total FLOPs / total time of one step of each"
-                                         % ", ".join(str(w) for w in workloads if w in DENSE or len(workloads) == 1),
-                           "l2": "inputs larger than L2: per configuration, rotating buffer sets that together exceed "
-                                 "twice the L2 (see per_config[].l2); warm numbers beside them",
-                           "flops_per_step": flops_total,
-                           "parallelism": ("data parallel x%d, gradient all-reduce per step" if args.dp_allreduce and world > 1
-                                           else "replicas x%d") % world,
-                           "launch": headline[0]["launch"]},
-                "clocks": merge_clocks([c["clocks"] for c in per_config]), "e2e": e2e,
-                "gpu_launches": sum(r["gpu_launches"] for r in raw),
-                "roofline": roofline, "cpu_baseline": cpu, "backbone": backbone, "per_config": per_config}
+        line, detail = result_line(args, world, workloads, value, ms_total, flops_total, headline[0]["launch"],
+                                   merge_clocks([c["clocks"] for c in per_config]), e2e, sum(r["gpu_launches"] for r in raw),
+                                   roofline, cpu, backbone, per_config)
+        # everything measured goes to standard error; the one line on standard output stays short enough for any log's tail
+        print(json.dumps(detail), file=sys.stderr, flush=True)
         print(json.dumps(line), flush=True)
     if world > 1:
         dist.destroy_process_group()

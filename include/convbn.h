@@ -304,7 +304,9 @@ int convbn_tune_bwd_glue(const convbn_desc *desc, const void *dz, const void *x,
  *                                                convbn_tconv_tune_bwd  (b and db both NULL or both non-NULL)
  * The transposed convolution runs on the kernels of the convolution it transposes (forward = that layer's backward data,
  * input gradient = its forward, weight gradient = its weight gradient with the two tensors exchanged); the scale, the bias
- * and the per-channel sums are separate small kernels.  One workspace size serves both calls.  Pointers: device, 16-byte
+ * and the per-channel sums are separate small kernels, except where the kernel is the stride without padding (NHWC, channels
+ * multiples of 64): its forward pass is one GEMM that applies scale and bias itself.  The backward call runs its two passes
+ * side by side, as convbn_tune_bwd does.  One workspace size serves both calls.  Pointers: device, 16-byte
  * aligned (vectors 4), workspace 256.  Errors as for the convolution calls; nothing is launched after an error. */
 int convbn_tconv_out_shape(const convbn_desc *desc, int *h_out, int *w_out);
 size_t convbn_tconv_workspace_bytes(const convbn_desc *desc);
@@ -359,8 +361,10 @@ int convbn_selftest_wait_timeout(void *stream);
 const char *convbn_status_string(int status);
 
 /* Name of the kernel family the last call of `phase` selected on this thread, for logs and tests:
- * "direct", "umma", "umma-strip", "umma-strided", "umma-subpixel", "umma-stem", "stem-mma", "depthwise",
- * "grouped-mma", "grouped-umma", and for CONVBN_PHASE_TUNE_BWD "umma-fused-bwd" or "two-calls".
+ * "direct" (the plain-ALU kernels, those of small fp32 layers among them), "umma", "umma-strip", "umma-strided",
+ * "umma-subpixel", "umma-stem", "stem-mma", "depthwise", "grouped-mma", "grouped-umma", and for
+ * CONVBN_PHASE_TUNE_BWD "umma-fused-bwd" (the 1x1 kernel that reads dZ once) or "two-calls" (everything else, whatever
+ * the number of launches).
  * Static string, never NULL. */
 const char *convbn_last_kernel(int phase);
 

@@ -210,7 +210,7 @@ Plan make_plan(const convbn_desc *d, const Problem &pb, int phase, bool bounded 
             pl.stem_win_wgrad = true;
             pl.uw = UmmaWgradPlan();
             pl.uw.splits = stem_window_wgrad_ctas(pb);
-                pl.bsplits = pl.uw.splits;
+            pl.bsplits = pl.uw.splits;
             part_bytes = wrows * pl.uw.splits * sizeof(float);
             dot_bytes = (size_t)wgrad_kmajor_rows(pb) * pb.c_out * sizeof(float);
         }
@@ -429,7 +429,7 @@ int run_conv_fwd(const convbn_desc *d, const Problem &pb, const void *x, const v
         LAUNCH("dw_fwd", launch_dw_fwd(pb, x, w, bias, z, st));
         *which = "depthwise";
     } else if (f32_path(d, pb)) {
-        LAUNCH("direct_fwd", launch_f32_fwd(pb, (const float *)x, (const float *)w, bias, (float *)z, st));
+        LAUNCH("f32_fwd", launch_f32_fwd(pb, (const float *)x, (const float *)w, bias, (float *)z, st));
         *which = "direct";
     } else {
         LAUNCH("direct_fwd", launch_direct_fwd(pb, d->dtype, d->layout, x, w, bias, z, st));
@@ -584,7 +584,7 @@ int run_conv_dgrad(const convbn_desc *d, const Problem &pb, const void *dz, cons
         }
         *which = "depthwise";
     } else if (f32_path(d, pb)) {
-        LAUNCH("direct_dgrad", launch_f32_bwd(pb, (const float *)dz, nullptr, (const float *)w, scale, (float *)dx, nullptr,
+        LAUNCH("f32_dgrad", launch_f32_bwd(pb, (const float *)dz, nullptr, (const float *)w, scale, (float *)dx, nullptr,
                                               nullptr, nullptr, nullptr, nullptr, nullptr, nullptr, 1, nullptr, nullptr, st));
         *which = "direct";
     } else {
@@ -613,8 +613,9 @@ int run_post(const convbn_desc *d, const PostOp &post, void *t, long long count,
 int run_f32_bwd(const convbn_desc *d, const Problem &pb, int groups, float *partials, float *bsum, const void *dz, const void *x,
                 const void *w, const float *dx_scale, void *dx, const float *vec3, const float *b, const float *mean, float *dw,
                 float *db, float *dgamma, float *dbeta, cudaStream_t st) {
-    LAUNCH("direct_bwd", launch_f32_bwd(pb, (const float *)dz, (const float *)x, (const float *)w, dx_scale, (float *)dx, vec3, b,
-                                        mean, dw, db, dgamma, dbeta, groups, partials, bsum, st));
+    LAUNCH(dx ? "f32_bwd" : "f32_wgrad",
+           launch_f32_bwd(pb, (const float *)dz, (const float *)x, (const float *)w, dx_scale, (float *)dx, vec3, b, mean, dw, db,
+                          dgamma, dbeta, groups, partials, bsum, st));
     if (groups > 1)
         LAUNCH("wgrad_epilogue", launch_wgrad_epilogue(pb, d->dtype, partials, groups, bsum, groups, w, vec3, b, mean, dw, db,
                                                        dgamma, dbeta, st));
@@ -641,7 +642,7 @@ int run_param_grads(const convbn_desc *d, const Problem &pb, const Plan &pl, con
     if (pl.stem_win_wgrad) {
         float *dotpart = (float *)at(ws, pl.dotpart);
         LAUNCH("stem_wgrad", launch_stem_window_wgrad(pb, dz, x, partials, bsum, st));
-        LAUNCH("wgrad_rows", launch_wgrad_epilogue_kmajor(pb, pl.uw.splits, partials, bsum, w, vec3, b, mean, dw, dotpart, db,
+        LAUNCH("wgrad_kmajor", launch_wgrad_epilogue_kmajor(pb, pl.uw.splits, partials, bsum, w, vec3, b, mean, dw, dotpart, db,
                                                           dgamma, dbeta, need_bsum, st));
         *which = "umma-stem";
     } else if (pl.stem) {
@@ -790,7 +791,7 @@ static int tune_fwd_impl(const convbn_desc *desc, const void *x, const void *w, 
     }
     if (f32_path(desc, pb)) {
         const BnFold fold{gamma, beta, run_mean, run_var, b, pb.eps, vec3};
-        LAUNCH("direct_fwd", launch_f32_fwd(pb, (const float *)x, (const float *)w, nullptr, (float *)z, st, &fold));
+        LAUNCH("f32_fwd", launch_f32_fwd(pb, (const float *)x, (const float *)w, nullptr, (float *)z, st, &fold));
         t_last_kernel[CONVBN_PHASE_TUNE_FWD] = "direct";
         return run_post(desc, post, z, count, st);
     }

@@ -29,7 +29,6 @@ struct FusedBwd {
     int f16;                // 16-bit storage type: 0 bf16, 1 IEEE half
     __nv_bfloat16 *dx;      // POST: plain stores of dX with post_add and post_mask (tensors of its shape; may be NULL)
     const __nv_bfloat16 *post_add, *post_mask;
-    int post_relu;
 };
 
 struct FbCtl {
@@ -270,8 +269,8 @@ __global__ void __launch_bounds__(kFbThreads) fused_bwd1x1_kernel(const __grid_c
                     for (int it = 0; it < 8; ++it) {
                         const int rr = it * 4 + (lane >> 3);
                         const uint4 q = *(const uint4 *)(buf_s + rr * 128 + (((ch ^ (rr & 7)) & 7) << 4));
-                        const uint4 o = g.f16 ? post_chunk<true>(q, g.post_add, av[it], g.post_relu, g.post_mask, mv[it])
-                                              : post_chunk<false>(q, g.post_add, av[it], g.post_relu, g.post_mask, mv[it]);
+                        const uint4 o = g.f16 ? post_chunk<true>(q, g.post_add, av[it], false, g.post_mask, mv[it])
+                                              : post_chunk<false>(q, g.post_add, av[it], false, g.post_mask, mv[it]);
                         if (row0 + it * 4 < g.p) *(uint4 *)(g.dx + off0 + (size_t)it * 4 * CI) = o;
                     }
                     if (c0 + 64 < c_hi) fetch_post(c0 + 64);
@@ -367,7 +366,7 @@ cudaError_t launch_fb_as(const CUtensorMap &tdz, const CUtensorMap &tx, const CU
 template <int CI, int CO>
 cudaError_t launch_fb(const CUtensorMap &tdz, const CUtensorMap &tx, const CUtensorMap &tdx, const FusedBwd &g, unsigned grid,
                       const void *w, float *partials, float *bsum, int *err, cudaStream_t st) {
-    if (g.post_add || g.post_mask || g.post_relu)
+    if (g.post_add || g.post_mask)
         return launch_fb_as<CI, CO, true>(tdz, tx, tdx, g, grid, w, partials, bsum, err, st);
     return launch_fb_as<CI, CO, false>(tdz, tx, tdx, g, grid, w, partials, bsum, err, st);
 }
@@ -386,13 +385,12 @@ int fused_bwd1x1_ctas(const Problem &pb) {
 
 cudaError_t launch_fused_bwd1x1(const Problem &pb, const void *dz, const void *x, const void *w, const float *vec3, void *dx,
                                 float *partials, float *bsum, cudaStream_t st, const PostOp *post) {
-    if (!fused_bwd1x1_eligible(pb)) return cudaErrorInvalidValue;
+    if (!fused_bwd1x1_eligible(pb) || (post && post->relu)) return cudaErrorInvalidValue;      // (no caller wants a ReLU on dX)
     FusedBwd g;
     g.p = pb.p; g.m_tiles = (int)((pb.p + 127) / 128); g.vec3 = vec3; g.f16 = call_f16();
     g.dx = (__nv_bfloat16 *)dx;
     g.post_add = post ? (const __nv_bfloat16 *)post->add : nullptr;
     g.post_mask = post ? (const __nv_bfloat16 *)post->mask : nullptr;
-    g.post_relu = post ? post->relu : 0;
     CUtensorMap tdz, tx, tdx;
     // a tile's [128 pixels][64 channels] blocks, side by side in shared memory, are one box of each tensor
     auto blocks = [&](CUtensorMap *tm, const void *base, int c) {

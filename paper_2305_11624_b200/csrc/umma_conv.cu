@@ -6,9 +6,9 @@
 //                  taps flipped and channel roles swapped (stride-1 convolutions)
 // GEMM view (Sec. 3.2.2): M = output pixels, N = output channels, K = taps x input channels.
 //
-// CTA = 6 warps: warp 0 issues TMA loads, warp 1 owns tensor memory and issues the MMAs, warps 2-5
-// move the 128 x BN fp32 accumulator from tensor memory to registers, add the bias, round to bf16
-// and store.  A ring of `stages` shared-memory slots decouples loads from MMAs.  Every wait is
+// CTA = 11 warps: warp 0 loads the activation tiles by TMA, warp 10 the weight tiles, warp 1 owns tensor memory and issues the
+// MMAs, warps 2-5 and 6-9 take the two 128 x BN fp32 accumulators in turn from tensor memory to registers, apply scale and
+// bias, round to 16 bits and store.  A ring of `stages` shared-memory slots decouples loads from MMAs.  Every wait is
 // bounded; a wait that gives up sets the device error word and the CTA drains and exits.
 #include <mutex>
 
