@@ -56,6 +56,15 @@ def test_tune_block(spec):
 EVAL = [  # Eval mode
     # more than 2048 output channels: the backward's sums by the kernel that takes any channel count, which writes no s dZ here
     L("eval_c2112", 3, 64, 5, 7, 2112, 1, 1, bias=True), L("eval_c2112_f16", 2, 128, 4, 9, 2112, 1, 1, dtype="f16"),
+    # output channels that fill no 64-wide tile, strides, and the shapes of the one-launch 1x1 backward with a last tile of
+    # pixels that is not full
+    # (stride 2 with 1x1 in half: most of dX is zeros there, so that an exact sum of the dY that bf16 stores is already
+    # 1.09 of the bound for bf16 away from the oracle in one element; in half it is 0.46)
+    L("eval_o72", 3, 64, 9, 11, 72, 1, 1, bias=True), L("eval_o200_k3", 2, 64, 13, 7, 200, 3, 3, pad=1),
+    L("eval_s2_k1_f16", 3, 128, 9, 9, 72, 1, 1, stride=2, dtype="f16"),
+    L("eval_s2_k3", 2, 64, 11, 13, 128, 3, 3, stride=2, pad=1, bias=True),
+    L("eval_64_256", 3, 64, 9, 11, 256, 1, 1, bias=True), L("eval_256_64_f16", 3, 256, 9, 11, 64, 1, 1, dtype="f16"),
+    L("eval_128_64", 1, 128, 17, 19, 64, 1, 1), L("eval_64_128_f16", 5, 64, 7, 5, 128, 1, 1, bias=True, dtype="f16"),
 ]
 
 
