@@ -73,15 +73,17 @@ def kernel_bytes(kind, spec, out_hw):
     raise KeyError(kind)
 
 
-# DRAM bytes (read + write) per launch, from ncu captures of the kernels as they are now; a kernel that
-# changed after its capture has no entry (traffic: null).  key: (kernel family, layer) -> (bytes, summary file).
-_P1, _P2S, _P2D, _P4 = ("profiles/config1_kernels_ncu_full.md", "profiles/config2_stem_window_kernels_ncu_full.md",
-                        "profiles/config2_dense_gemm_ncu_full.md", "profiles/config4a_depthwise_kernels_ncu_full.md")
-NCU_TRAFFIC = {("stem_fwd", "c2s"): (66.3e6, _P2S), ("stem_dgrad", "c2s"): (116.6e6, _P2S), ("stem_wgrad", "c2s"): (126.9e6, _P2S),
-               ("umma_bwd", "c1a"): (76.4e6, _P1), ("strip_fwd", "c1b"): (13.0e6, _P1), ("strip_dgrad", "c1b"): (13.0e6, _P1),
-               ("umma_fwd", "c2a"): (14.99e6, _P2D), ("umma_dgrad", "c2a"): (5.35e6, _P2D), ("umma_wgrad", "c2a"): (16.10e6, _P2D),
-               ("umma_fwd", "c2b"): (7.98e6, _P2D),
-               ("dw_fwd", "c4a"): (259.0e6, _P4), ("dw_dgrad", "c4a"): (258.7e6, _P4), ("dw_wgrad", "c4a"): (312.0e6, _P4)}
+# DRAM bytes (read + write) per launch, from an ncu capture of the kernels as they are now; a kernel that
+# changes after its capture loses its entry (traffic: null).  (kernel family, layer) -> bytes.
+NCU_SUMMARY = "profiles/step_kernels_ncu_traffic.md"
+NCU_TRAFFIC = {("stem_fwd", "c2s"): 59.5e6, ("stem_dgrad", "c2s"): 112.5e6, ("stem_wgrad", "c2s"): 123.3e6,
+               ("umma_fwd", "c1a"): 51.5e6, ("umma_bwd", "c1a"): 70.6e6,
+               ("umma_fwd", "c1b"): 13.0e6, ("umma_dgrad", "c1b"): 13.0e6, ("umma_wgrad", "c1b"): 25.7e6,
+               ("umma_fwd", "c2a"): 15.0e6, ("umma_dgrad", "c2a"): 5.37e6, ("umma_wgrad", "c2a"): 16.1e6,
+               ("umma_fwd", "c2b"): 8.00e6, ("umma_dgrad", "c2b"): 7.99e6, ("umma_wgrad", "c2b"): 6.47e6,
+               ("umma_fwd", "c3a"): 17.2e6, ("umma_dgrad", "c3a"): 17.2e6, ("umma_wgrad", "c3a"): 34.2e6,
+               ("dw_fwd", "c4a"): 254.8e6, ("dw_dgrad", "c4a"): 254.6e6, ("dw_wgrad", "c4a"): 309.1e6,
+               ("grouped_fwd", "c4b"): 25.8e6, ("grouped_dgrad", "c4b"): 25.7e6, ("grouped_wgrad", "c4b"): 51.5e6}
 
 KIND_OF = {"strip_fwd": "fwd", "strip_dgrad": "dgrad", "direct_fwd": "fwd", "direct_dgrad": "dgrad", "direct_wgrad": "wgrad",
            "umma_fwd": "fwd", "umma_dgrad": "dgrad", "umma_wgrad": "wgrad", "umma_bwd": "bwd",
@@ -494,7 +496,8 @@ def bench_config(ctx, wl):
         fl = b.flops_per_phase() * (2 if kind == "bwd" else 1)
         by = kernel_bytes(kind, b.spec, (b.h_out, b.w_out))
         dense_bf16 = b.spec.dtype == "bf16" and b.spec.groups == 1
-        traffic, traffic_from = NCU_TRAFFIC.get((top["kernel"], top["layer"]), (None, None))
+        traffic = NCU_TRAFFIC.get((top["kernel"], top["layer"]))
+        traffic_from = NCU_SUMMARY if traffic else None
         if dense_bf16 and fl / by > ridge:
             ach = fl / dur / 1e12
             r = {"bound": "tensor", "achieved": ach, "peak": tc, "unit": "TFLOP/s", "frac": ach / tc,
@@ -706,18 +709,17 @@ def short(v):
 
 def result_line(args, world, workloads, value, ms_total, flops_total, launch, clocks, e2e, launches, roofline, cpu, backbone,
                 per_config):
-    """The result line, under 1500 characters, and the object with every figure behind it."""
+    """The result line, under 1400 characters, and the object with every figure behind it."""
     pick = lambda d, *keys: None if d is None else {k: d.get(k) for k in keys}
     line = {"metric": METRIC, "value": value, "unit": UNIT, "n_gpus": world, "steps": args.steps,
             "warmup": args.warmup, "ms_per_step": ms_total / args.steps, "higher_is_better": True,
             "scaling": "weak", "vs_baseline": None,
             "dtype": "bf16" if any(w != 0 for w in workloads) else "f32", "data": "synthetic",
             "config": {"workload": "; ".join(WORKLOAD_NAMES[w] for w in workloads if w in DENSE or len(workloads) == 1),
-                       "value_over": "total FLOPs / total time of one step of each",
                        "l2": "rotating buffer sets, over twice the L2", "flops_per_step": flops_total,
                        "parallelism": ("data parallel x%d, gradient all-reduce per step" if args.dp_allreduce and world > 1
                                        else "replicas x%d") % world,
-                       "launch": launch},
+                       "launch": launch.split(";")[0]},
             "clocks": clocks, "e2e": pick(e2e, "value", "unit", "h2d_bytes_per_step", "d2h_bytes_per_step"),
             "gpu_launches": launches,
             "roofline": pick(roofline, "kernel", "layer", "bound", "achieved", "peak", "unit", "frac", "traffic"),
