@@ -162,8 +162,8 @@ int convbn_tune_bwd_weight(const convbn_desc *desc, const void *dz, const void *
  * For the 1x1, stride-1 layers of a bottleneck (bf16 NHWC, one of C_in / C_out equal to 64 and the other
  * 128 or 256, at least 512 pixels) one kernel reads every dZ tile from memory ONCE and feeds both the
  * data-gradient and the weight-gradient GEMM from it (omega' = s omega is formed in shared memory and never
- * written); every other layer runs the two passes above SIDE BY SIDE: one of them (the one expected to be shorter) on a stream
- * the library owns (one per device and host thread, created on first use), forked from `stream` at the start of the call and
+ * written); every other layer runs the two passes above SIDE BY SIDE: one of them (the one expected to be shorter; in a
+ * stream capture always the parameter gradients) on a stream the library owns (one per device and host thread, created on first use), forked from `stream` at the start of the call and
  * joined into it before the call returns, so the caller sees plain stream order (and a stream capture stays well-formed); each
  * pass has its own region of the workspace.  dx may not alias dz or x.
  * Workspace: convbn_workspace_bytes(desc, CONVBN_PHASE_TUNE_BWD). */
