@@ -19,6 +19,18 @@ __device__ __forceinline__ f32x2 fma2(f32x2 a, f32x2 b, f32x2 c) {
     asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(a), "l"(b), "l"(c));
     return d;
 }
+// a s + b with the product rounded before the sum, as two multiplications and two additions give it.  `one`: (1, 1), read from
+// memory, where the compiler cannot see what it is: mul.rn.f32x2 followed by add.rn.f32x2 came out fused, and a sum times a
+// constant 1 too.
+__device__ __forceinline__ f32x2 mul_add2(f32x2 a, f32x2 s, f32x2 b, f32x2 one) {
+    return fma2(fma2(a, s, pair(-0.f, -0.f)), one, b);
+}
+// two consecutive floats of shared memory (8-byte aligned)
+__device__ __forceinline__ f32x2 lds_f32x2(uint32_t addr) {
+    f32x2 d;
+    asm volatile("ld.shared.b64 %0, [%1];" : "=l"(d) : "r"(addr) : "memory");
+    return d;
+}
 // two bf16 in one word -> two fp32
 __device__ __forceinline__ f32x2 widen(uint32_t u) { return pair(__uint_as_float(u << 16), __uint_as_float(u & 0xFFFF0000u)); }
 // two fp32 -> two bf16 in one word (round to nearest even)

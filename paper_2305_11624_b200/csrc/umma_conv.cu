@@ -13,6 +13,8 @@
 #include <mutex>
 
 #include "kernels.h"
+#include "mma_sync.cuh"
+#include "packed_f32.cuh"
 #include "sm100_ptx.cuh"
 
 namespace convbn {
@@ -69,6 +71,7 @@ struct ConvSmemCtl {
     uint64_t post_full[8];     // kPost: an epilogue warp's boxes of the other tensors have landed
     uint32_t tmem_base;
     int abort_flag;
+    float2 one;                // (1, 1) for mul_add2
 };
 
 // Persistent: CTA b works on tiles b, b + gridDim.x, ...; tile t covers output pixels
@@ -142,6 +145,8 @@ __global__ void __launch_bounds__(MODE == kPlain || MODE == kRelu || MODE == kTa
     // a pair's boxes all count on its first CTA's barriers
     const uint32_t full_of_first = PAIR ? cluster_addr(&ctl->full[0], 0) : smem_u32(&ctl->full[0]);
 
+    // the tensor maps are kernel parameters, not data of an earlier kernel: their way to the copy engine starts at once
+    if (threadIdx.x == 64) { prefetch_tensormap(&tm_act); prefetch_tensormap(&tm_w); prefetch_tensormap(&tm_out); }
     if (threadIdx.x == 0) {
         CONVBN_TRACE_POINT(0);
         for (int s = 0; s < stages; ++s) { mbar_init(&ctl->full[s], g.resident ? 1 : 2); mbar_init(&ctl->empty[s], 1); }
@@ -150,14 +155,13 @@ __global__ void __launch_bounds__(MODE == kPlain || MODE == kRelu || MODE == kTa
         if constexpr (POST)
             for (int a = 0; a < 8; ++a) mbar_init(&ctl->post_full[a], 1);
         ctl->abort_flag = 0;
+        ctl->one = make_float2(1.f, 1.f);
         fence_barrier_init();
     }
     if (warp == 1) {
         tmem_alloc<CTAS>(&ctl->tmem_base, 2 * BN);
         tmem_relinquish<CTAS>();
     }
-    // the tensor maps are kernel parameters, not data of an earlier kernel: fetch them before the wait
-    if (threadIdx.x == 0) { prefetch_tensormap(&tm_act); prefetch_tensormap(&tm_w); prefetch_tensormap(&tm_out); }
     tc_fence_before_sync();
     __syncthreads();
     if constexpr (PAIR) cluster_sync_all();                 // both CTAs' barriers and columns are there
@@ -391,13 +395,22 @@ __global__ void __launch_bounds__(MODE == kPlain || MODE == kRelu || MODE == kTa
                     g.fold.vec3[c] = sc; g.fold.vec3[pc + c] = bf; g.fold.vec3[2 * pc + c] = r;
                 }
             }
-        } else if (bias) {
-            for (int c = (int)threadIdx.x - 64; c < g.cn; c += 256) bias_s[c] = bias[c];
+        } else {
+            // (scale 1 and shift -0 leave every value as it is, so the epilogue has one form)
+            for (int c = (int)threadIdx.x - 64; c < g.cn; c += 256) { scale_s[c] = 1.f; bias_s[c] = bias ? bias[c] : -0.f; }
         }
         named_bar_sync(1, 256);
         const int quarter = warp & 3;                      // tensor-memory lanes this warp may read
         const uint32_t egroup = (uint32_t)(warp - 2) >> 2; // 0: warps 2-5, 1: warps 6-9
         uint8_t *stage_buf = staging + (size_t)(warp - 2) * kStagingWarpBytes;
+        // The accumulator is read as matrix fragments: this lane gets columns 8 i + 2 (lane % 4) and the next of rows lane / 4 and
+        // lane / 4 + 8 of every 16, so the parameters of a 64-column chunk are 16 values of each kind, read while the accumulator
+        // is on its way, and stmatrix writes the swizzled rows.  (A row per lane needs the parameters of all 64 columns in every
+        // lane, 32 16-byte loads: a chunk took 1550 clocks instead of 1040; forward + backward of the transposed 2x2 256 -> 128 layer
+        // at 56 x 56, N = 8 62.0 -> 57.7 us, Eval 64 -> 256 at 56 x 56, N = 32 94.4 -> 84.1, ResNet-50, N = 32 2586 -> 2512.)
+        const uint32_t shift_at = smem_u32(bias_s) + (uint32_t)(lane & 3) * 8u, scale_at = shift_at + (uint32_t)g.cn * 4u;
+        // stmatrix: lanes 8 m to 8 m + 7 name the rows of matrix m; matrices 0, 1: rows 0-7, 8-15, matrices 2, 3: the next 8 columns
+        const uint32_t frag_row = (uint32_t)((lane & 7) + (lane & 8)) * 128u, frag_chunk = (uint32_t)(((lane >> 4) ^ (lane & 7)) << 4);
         // the buffer for the next box: the last store from it has been read, an earlier one (nbuf = 2) may still be under way
         uint32_t turn = 0;
         auto next_buf = [&]() -> uint8_t * {
@@ -407,6 +420,7 @@ __global__ void __launch_bounds__(MODE == kPlain || MODE == kRelu || MODE == kTa
             if ((MODE == kPlain || MODE == kRelu) && g.nbuf == 2) turn ^= kStagingBytes;
             return b;
         };
+        const f32x2 one = lds_f32x2(smem_u32(&ctl->one));
         uint32_t mt, nt;
         // kPost: tm_out2 is the addend's map.  One box of each tensor in flight per warp.
         uint8_t *add_buf = staging + (size_t)g.nbuf * kStagingBytes + (size_t)(warp - 2) * kStagingWarpBytes, *mask_buf = add_buf + (g.post_add ? kStagingBytes : 0);
@@ -456,10 +470,19 @@ __global__ void __launch_bounds__(MODE == kPlain || MODE == kRelu || MODE == kTa
             const int p0 = TAP ? n0 % g.tap_c : n0;         // first per-channel parameter of this tile
 #pragma unroll 1
             for (int c0 = 0; c0 < BN; c0 += 64) {
-                uint32_t v[64];
+                uint32_t v[2][32];                          // rows 0-15 and 16-31 of this warp
+                f32x2 sc[4], sh[4];                         // parameters of 32 columns
+                auto params = [&](int i0, uint32_t sc_at, uint32_t sh_at) {
+#pragma unroll
+                    for (int i = 0; i < 4; ++i) {
+                        sh[i] = lds_f32x2(sh_at + (uint32_t)(p0 + c0 + 8 * (i0 + i)) * 4u);
+                        if (sc_at) sc[i] = lds_f32x2(sc_at + (uint32_t)(p0 + c0 + 8 * (i0 + i)) * 4u);
+                    }
+                };
                 if (c0 < ncols) {
-                    tmem_ld_32x32(t_row + (uint32_t)c0, *(uint32_t(*)[32]) & v[0]);
-                    tmem_ld_32x32(t_row + (uint32_t)c0 + 32, *(uint32_t(*)[32]) & v[32]);
+                    tmem_ld_16x64(t_row + (uint32_t)c0, v[0]);
+                    tmem_ld_16x64(t_row + (16u << 16) + (uint32_t)c0, v[1]);
+                    params(0, DUAL ? 0u : scale_at, shift_at);
                     tmem_ld_wait();
                 }
                 if (c0 + 64 >= BN) {
@@ -473,7 +496,7 @@ __global__ void __launch_bounds__(MODE == kPlain || MODE == kRelu || MODE == kTa
                 }
                 if (c0 < ncols) {
                     uint8_t *buf = next_buf();
-                    uint8_t *row = buf + lane * 128;
+                    const uint32_t frag = smem_u32(buf) + frag_row;
                     if constexpr (POST) {
                         if (post_pending) {
                             const bool here = mbar_wait_bounded(&ctl->post_full[warp - 2], post_ph, abort_flag);
@@ -486,40 +509,34 @@ __global__ void __launch_bounds__(MODE == kPlain || MODE == kRelu || MODE == kTa
                     auto pack_rows = [&](auto half_tag, auto add_tag, auto relu_tag, auto mask_tag) {
                         constexpr bool H = decltype(half_tag)::value, ADD = decltype(add_tag)::value;
                         constexpr bool RELU = decltype(relu_tag)::value, MASK = decltype(mask_tag)::value;
-    #pragma unroll
-                        for (int j = 0; j < 64; j += 8) {
-                            float f[8];
-    #pragma unroll
-                            for (int e = 0; e < 8; ++e) f[e] = __uint_as_float(v[j + e]);
-                            if (fold && !DUAL) {
-                                const float4 s0 = *(const float4 *)(scale_s + p0 + c0 + j);
-                                const float4 s1 = *(const float4 *)(scale_s + p0 + c0 + j + 4);
-                                f[0] *= s0.x; f[1] *= s0.y; f[2] *= s0.z; f[3] *= s0.w;
-                                f[4] *= s1.x; f[5] *= s1.y; f[6] *= s1.z; f[7] *= s1.w;
+#pragma unroll
+                        for (int i = 0; i < 8; i += 2) {
+                            if (i == 4) params(4, DUAL ? 0u : scale_at, shift_at);
+#pragma unroll
+                            for (int h = 0; h < 2; ++h) {
+                                uint32_t o[4];                 // columns 8 i and 8 i + 8: rows 0-7, 8-15 of each
+#pragma unroll
+                                for (int e = 0; e < 4; ++e) {
+                                    const uint32_t *q = &v[h][(i + (e >> 1)) * 4 + (e & 1) * 2];
+                                    const f32x2 f = pair(__uint_as_float(q[0]), __uint_as_float(q[1]));
+                                    const f32x2 shift = sh[(i & 3) + (e >> 1)];
+                                    o[e] = narrow_t<H>(DUAL ? fma2(f, one, shift) : mul_add2(f, sc[(i & 3) + (e >> 1)], shift, one));
+                                    if constexpr (MODE == kRelu) o[e] = post_pair<H>(o[e], false, 0u, true, false, 0u);
+                                }
+                                const uint32_t at16 = (uint32_t)h * 2048u + (((uint32_t)i << 4) ^ frag_chunk);
+                                if constexpr (POST) {
+                                    uint32_t a[4] = {0u, 0u, 0u, 0u}, m[4] = {0u, 0u, 0u, 0u};
+                                    if constexpr (ADD) ldmatrix_x4(a[0], a[1], a[2], a[3], smem_u32(add_buf) + frag_row + at16);
+                                    if constexpr (MASK) ldmatrix_x4(m[0], m[1], m[2], m[3], smem_u32(mask_buf) + frag_row + at16);
+#pragma unroll
+                                    for (int e = 0; e < 4; ++e) o[e] = post_pair<H>(o[e], ADD, a[e], RELU, MASK, m[e]);
+                                }
+                                stmatrix_x4(frag + at16, o[0], o[1], o[2], o[3]);
+                                if constexpr (DUAL) {          // kept for the second output, in the accumulator's registers
+#pragma unroll
+                                    for (int e = 0; e < 4; ++e) v[h][i * 2 + e] = o[e];
+                                }
                             }
-                            if (bias || fold) {
-                                const float4 b0 = *(const float4 *)(bias_s + p0 + c0 + j);
-                                const float4 b1 = *(const float4 *)(bias_s + p0 + c0 + j + 4);
-                                f[0] += b0.x; f[1] += b0.y; f[2] += b0.z; f[3] += b0.w;
-                                f[4] += b1.x; f[5] += b1.y; f[6] += b1.z; f[7] += b1.w;
-                            }
-                            uint4 pk;
-                            pk.x = pack2_t<H>(f[0], f[1]);
-                            pk.y = pack2_t<H>(f[2], f[3]);
-                            pk.z = pack2_t<H>(f[4], f[5]);
-                            pk.w = pack2_t<H>(f[6], f[7]);
-                            const int at16 = (((j >> 3) ^ (lane & 7)) & 7) << 4;
-                            if constexpr (MODE == kRelu) {
-                                const uint4 none = make_uint4(0u, 0u, 0u, 0u);
-                                pk = post_chunk<H>(pk, false, none, true, false, none);
-                            }
-                            if constexpr (POST) {
-                                uint4 a4 = make_uint4(0u, 0u, 0u, 0u), m4 = a4;
-                                if constexpr (ADD) a4 = *(const uint4 *)(add_buf + lane * 128 + at16);
-                                if constexpr (MASK) m4 = *(const uint4 *)(mask_buf + lane * 128 + at16);
-                                pk = post_chunk<H>(pk, ADD, a4, RELU, MASK, m4);
-                            }
-                            *(uint4 *)(row + at16) = pk;
                         }
                     };
                     auto pack = [&](auto add_tag, auto relu_tag, auto mask_tag) {
@@ -594,30 +611,24 @@ __global__ void __launch_bounds__(MODE == kPlain || MODE == kRelu || MODE == kTa
                         tma_store_commit();
                     }
                     if constexpr (DUAL) {
-                        uint4 zq[8];
+                        buf = next_buf();
+                        const uint32_t frag2 = smem_u32(buf) + frag_row;
                         auto normalise = [&](auto half_tag) {
                             constexpr bool H = decltype(half_tag)::value;
 #pragma unroll
-                            for (int j = 0; j < 8; ++j) {
-                                const uint4 q = *(const uint4 *)(row + (((j ^ (lane & 7)) & 7) << 4));
-                                const uint32_t u[4] = {q.x, q.y, q.z, q.w};
-                                uint32_t o[4];
+                            for (int i = 0; i < 8; i += 2) {
+                                if ((i & 3) == 0) params(i, scale_at, scale_at + (uint32_t)g.cn * 4u);
 #pragma unroll
-                                for (int e = 0; e < 4; ++e) {
-                                    const float2 sc = *(const float2 *)(scale_s + n0 + c0 + j * 8 + 2 * e);
-                                    const float2 sh = *(const float2 *)(shift_s + n0 + c0 + j * 8 + 2 * e);
-                                    float lo, hi2;
-                                    unpack2_t<H>(u[e], lo, hi2);
-                                    o[e] = pack2_t<H>(fmaf(sc.x, lo, sh.x), fmaf(sc.y, hi2, sh.y));
+                                for (int h = 0; h < 2; ++h) {
+                                    uint32_t o[4];
+#pragma unroll
+                                    for (int e = 0; e < 4; ++e)
+                                        o[e] = narrow_t<H>(fma2(widen_t<H>(v[h][i * 2 + e]), sc[(i & 3) + (e >> 1)], sh[(i & 3) + (e >> 1)]));
+                                    stmatrix_x4(frag2 + (uint32_t)h * 2048u + (((uint32_t)i << 4) ^ frag_chunk), o[0], o[1], o[2], o[3]);
                                 }
-                                zq[j] = make_uint4(o[0], o[1], o[2], o[3]);
                             }
                         };
                         if (g.f16) normalise(std::true_type{}); else normalise(std::false_type{});
-                        buf = next_buf();
-                        row = buf + lane * 128;
-#pragma unroll
-                        for (int j = 0; j < 8; ++j) *(uint4 *)(row + (((j ^ (lane & 7)) & 7) << 4)) = zq[j];
                         fence_proxy_async_smem();
                         __syncwarp();
                         if (lane == 0) {
@@ -765,7 +776,8 @@ static cudaError_t launch_bn(const CUtensorMap &ta, const CUtensorMap &tw, const
     // Short K: the epilogues bound the kernel, and the second buffer is worth more than the ring slots it takes (1x1 256 -> 64
     // at 56 x 56, N = 256, forward 86.4 -> 82.6 us; the other modes, with staging areas of their own, gain nothing).
     g.nbuf = (MODE == kPlain || MODE == kRelu) && num_kb <= 8 ? 2 : 1;
-    size_t fixed = 1024 + (size_t)(g.nbuf + extra) * kStagingBytes + sizeof(ConvSmemCtl) + (MODE == kDual ? 3 : 2) * (size_t)g.cn * sizeof(float) + 16;
+    // (256: the epilogue reads the per-channel parameters of whole 64-column chunks)
+    size_t fixed = 1024 + 256 + (size_t)(g.nbuf + extra) * kStagingBytes + sizeof(ConvSmemCtl) + (MODE == kDual ? 3 : 2) * (size_t)g.cn * sizeof(float) + 16;
     const long long m_tiles = (g.p + kBM - 1) / kBM, n_tiles = (g.cn + BN - 1) / BN;
     long long grid_l = m_tiles * n_tiles < sm_count() ? m_tiles * n_tiles : sm_count();
     if (PAIR) {
