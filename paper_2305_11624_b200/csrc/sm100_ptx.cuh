@@ -142,6 +142,9 @@ __device__ __forceinline__ uint32_t cluster_addr(P p, uint32_t rank) {
     asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(a) : "r"(smem_u32(p)), "r"(rank));
     return a;
 }
+__device__ __forceinline__ void st_cluster_f32(uint32_t addr_cluster, float v) {
+    asm volatile("st.shared::cluster.f32 [%0], %1;" ::"r"(addr_cluster), "f"(v) : "memory");
+}
 // (for a hand-over of tensor memory, which tcgen05.fence orders: the arrival publishes no writes to ordinary memory.  With
 // .release.cluster it waited about 1000 clocks for the thread's stores.)
 __device__ __forceinline__ void mbar_arrive_cluster(uint32_t bar_cluster) {

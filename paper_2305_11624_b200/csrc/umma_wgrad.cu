@@ -397,47 +397,67 @@ cudaError_t launch_umma_wgrad(const Problem &pb, const UmmaWgradPlan &pl, const 
 //     acc[k] = sum_split part[split][co][k]
 //     domega = s acc,   dbeta = sum_split bsum,   db = s dbeta,   dgamma = r (sum_k acc omega + dbeta (b - mu_hat)).
 // Plain mode (vec3 == NULL): domega = acc, db = sum dZ if requested; need_sums = 0: domega alone.
-// Threads: VL along k (a float4 each, so that reads and stores are whole lines) x SL groups of slices, added in order
-// through shared memory; a thread requests up to eight slices before it uses the first.  Bound by those reads (9 to 19 MB
-// from L2).  With k-major partial tiles the GEMM's stores were 16 bytes per lane in 32 lines, this kernel had to transpose,
+// CL blocks (a cluster) share a channel, a span of k each; their parts of the dot product meet in the first one.
+// Threads of a block: VL along k (a float4 each, so that reads and stores are whole lines) x SL groups of slices, added in
+// order through shared memory; a thread requests up to eight slices before it uses the first.  Bound by the latency of those
+// reads (9 to 19 MB, most of them from L2), so a layer is cut into blocks of a few hundred threads that go over their span
+// once: with a block of up to 1024 threads per channel, 64 channels left most SMs idle and 4608 weights took a second, nearly
+// empty turn (forward + backward of 3x3 64 -> 64 at 56 x 56, N = 32
+// 51.3 -> 49.5 us, of 1000 rows 256 -> 64 15.1 -> 14.6).
+// With k-major partial tiles the GEMM's stores were 16 bytes per lane in 32 lines, this kernel had to transpose,
 // and the per-channel sums needed a counter or a second kernel.  Weight phase (GEMM + this), graph replay, N = 32: 1x1
 // 512 -> 128 at 28 x 28 20.3 -> 12.0 us, 3x3 256 at 14 x 14 22.8 -> 17.2, 3x3 512 at 7 x 7 30.0 -> 22.8.
-__global__ void __launch_bounds__(1024) wgrad_rows_kernel(int c_out, int kdim, int VL, int SL, const float *__restrict__ part,
-                                                          int splits, const float *__restrict__ bsum,
-                                                          const __nv_bfloat16 *__restrict__ w, const float *__restrict__ vec3,
-                                                          const float *__restrict__ b, const float *__restrict__ mean,
-                                                          float *__restrict__ dw, float *__restrict__ db,
-                                                          float *__restrict__ dgamma, float *__restrict__ dbeta, int need_sums,
-                                                          int f16) {
-    __shared__ float4 red[1024];
-    __shared__ float fin[2][32];
+constexpr int kRowsMaxThreads = 512, kRowsMaxCluster = 8;
+template <int CL>
+__global__ void __launch_bounds__(kRowsMaxThreads) wgrad_rows_kernel(int c_out, int kdim, int span, int VL, int SL,
+                                                                     const float *__restrict__ part, int splits,
+                                                                     const float *__restrict__ bsum,
+                                                                     const __nv_bfloat16 *__restrict__ w,
+                                                                     const float *__restrict__ vec3, const float *__restrict__ b,
+                                                                     const float *__restrict__ mean, float *__restrict__ dw,
+                                                                     float *__restrict__ db, float *__restrict__ dgamma,
+                                                                     float *__restrict__ dbeta, int need_sums, int f16) {
+    __shared__ float4 red[kRowsMaxThreads];
+    __shared__ float fin[2][kRowsMaxThreads / 32], dots[kRowsMaxCluster];
+    const int rank = CL > 1 ? (int)cluster_rank() : 0, co = blockIdx.x / CL;
+    const int z = threadIdx.x / VL, l = threadIdx.x - z * VL;        // (z >= SL: threads that fill up the last warp)
+    const size_t slice = (size_t)c_out * kdim, row = (size_t)co * kdim;
     pdl_wait();
     pdl_launch_dependents();
-    const int co = blockIdx.x, l = threadIdx.x % VL, z = threadIdx.x / VL;
     const float s = vec3 ? vec3[co] : 1.f;
-    const size_t slice = (size_t)c_out * kdim, row = (size_t)co * kdim;
     float dot = 0.f, ds = 0.f;
-    if (need_sums)
+    if (need_sums && rank == 0)
         for (int sp = threadIdx.x; sp < splits; sp += blockDim.x) ds += __ldcg(bsum + (size_t)sp * c_out + co);
-    for (int k0 = 0; k0 < kdim; k0 += 4 * VL) {
+    const int k_end = min(kdim, (rank + 1) * span);
+    for (int k0 = rank * span; k0 < k_end; k0 += 4 * VL) {
         const int k = k0 + 4 * l;
+        const bool on = k < k_end;
         uint2 wq = make_uint2(0u, 0u);
-        if (vec3 && need_sums && z == 0 && k < kdim) wq = *(const uint2 *)(w + row + k);
+        if (vec3 && need_sums && z == 0 && on) wq = *(const uint2 *)(w + row + k);
         float4 a = make_float4(0.f, 0.f, 0.f, 0.f);
-        if (k < kdim) {
+        if (on && z < SL) {
             const float *src = part + row + k;
-            for (int sp = z; sp < splits; sp += 8 * SL) {
+            const size_t step = (size_t)SL * slice;
+            int sp = z;
+            src += (size_t)z * slice;
+            for (; sp + 7 * SL < splits; sp += 8 * SL, src += 8 * step) {
                 float4 v[8];
 #pragma unroll
-                for (int u = 0; u < 8; ++u)
-                    v[u] = sp + u * SL < splits ? __ldcg((const float4 *)(src + (size_t)(sp + u * SL) * slice))
-                                                : make_float4(0.f, 0.f, 0.f, 0.f);
+                for (int u = 0; u < 8; ++u) v[u] = __ldcg((const float4 *)(src + u * step));
 #pragma unroll
                 for (int u = 0; u < 8; ++u) { a.x += v[u].x; a.y += v[u].y; a.z += v[u].z; a.w += v[u].w; }
             }
+            if (sp < splits) {
+                float4 v[7];
+#pragma unroll
+                for (int u = 0; u < 7; ++u)
+                    v[u] = sp + u * SL < splits ? __ldcg((const float4 *)(src + u * step)) : make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+                for (int u = 0; u < 7; ++u) { a.x += v[u].x; a.y += v[u].y; a.z += v[u].z; a.w += v[u].w; }
+            }
         }
         if (SL > 1) {
-            if (k0) __syncthreads();
+            if (k0 != rank * span) __syncthreads();
             red[threadIdx.x] = a;
             // groups z and z + h in halves: log2(SL) short steps
             for (int h = SL / 2; h > 0; h /= 2) {
@@ -449,7 +469,7 @@ __global__ void __launch_bounds__(1024) wgrad_rows_kernel(int c_out, int kdim, i
                 }
             }
         }
-        if (z == 0 && k < kdim) {
+        if (z == 0 && on) {
             *(float4 *)(dw + row + k) = make_float4(s * a.x, s * a.y, s * a.z, s * a.w);
             dot = fmaf(a.x, unpack_h16((uint16_t)(wq.x & 0xFFFFu), f16), dot);
             dot = fmaf(a.y, unpack_h16((uint16_t)(wq.x >> 16), f16), dot);
@@ -458,13 +478,27 @@ __global__ void __launch_bounds__(1024) wgrad_rows_kernel(int c_out, int kdim, i
         }
     }
     if (!need_sums) return;
+    const int lane = threadIdx.x & 31, warps = blockDim.x / 32;
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) { dot += __shfl_xor_sync(0xffffffffu, dot, o); ds += __shfl_xor_sync(0xffffffffu, ds, o); }
-    if (threadIdx.x % 32 == 0) { fin[0][threadIdx.x / 32] = dot; fin[1][threadIdx.x / 32] = ds; }
+    if (lane == 0) { fin[0][threadIdx.x / 32] = dot; fin[1][threadIdx.x / 32] = ds; }
     __syncthreads();
-    if (threadIdx.x) return;
-    dot = ds = 0.f;
-    for (int i = 0; i < (int)blockDim.x / 32; ++i) { dot += fin[0][i]; ds += fin[1][i]; }
+    if (threadIdx.x < 32) {
+        dot = lane < warps ? fin[0][lane] : 0.f;
+        ds = lane < warps ? fin[1][lane] : 0.f;
+#pragma unroll
+        for (int o = kRowsMaxThreads / 64; o > 0; o >>= 1) { dot += __shfl_xor_sync(0xffffffffu, dot, o); ds += __shfl_xor_sync(0xffffffffu, ds, o); }
+    }
+    if constexpr (CL > 1) {
+        if (threadIdx.x == 0) st_cluster_f32(cluster_addr(&dots[rank], 0), dot);
+        cluster_sync_all();
+    }
+    if (threadIdx.x || rank) return;
+    if constexpr (CL > 1) {
+        dot = 0.f;
+#pragma unroll
+        for (int i = 0; i < CL; ++i) dot += dots[i];
+    }
     if (!vec3) {
         if (db) db[co] = ds;
         return;
@@ -478,15 +512,31 @@ __global__ void __launch_bounds__(1024) wgrad_rows_kernel(int c_out, int kdim, i
 cudaError_t launch_wgrad_rows(const Problem &pb, int splits, const float *partials, const float *bsum, const void *w,
                               const float *vec3, const float *b, const float *mean, float *dw, float *db, float *dgamma,
                               float *dbeta, bool need_sums, cudaStream_t st) {
-    // slice groups so that a thread adds at most eight slices, then as many threads along the row as are left
-    int SL = 1, VL = 16;
+    // slice groups so that a thread adds at most eight slices; a cluster as large as brings a block to 384 threads (spans of
+    // whole 128-byte lines) or the grid to four blocks per SM; then as many threads along the span as there is room for
+    int SL = 1, CL = 1;
     while (SL < 32 && SL * 8 < splits) SL *= 2;
-    while (VL * 4 < pb.kdim && VL * SL < 1024) VL *= 2;
-    while (VL * SL < 32) VL *= 2;
-    static PerDevice carve;
-    prefer_max_shared_once(wgrad_rows_kernel, &carve);
-    return launch_pdl(wgrad_rows_kernel, dim3(pb.c_out), dim3(VL * SL), 0, st, pb.c_out, pb.kdim, VL, SL, partials, splits, bsum,
-                      (const __nv_bfloat16 *)w, vec3, b, mean, dw, db, dgamma, dbeta, need_sums ? 1 : 0, call_f16());
+    auto vectors = [&](int cl) { return ((pb.kdim / 4 + cl - 1) / cl + 7) / 8 * 8; };
+    while (CL < kRowsMaxCluster && pb.kdim / 4 >= 16 * CL &&
+           (vectors(CL) * SL > 384 || (long long)pb.c_out * CL < 4LL * device_sm_count()))
+        CL *= 2;
+    const int span = 4 * vectors(CL);
+    int VL = vectors(CL);
+    if (VL * SL > kRowsMaxThreads) VL = kRowsMaxThreads / SL;
+    const int threads = (VL * SL + 31) / 32 * 32;
+    if ((long long)pb.c_out * CL > 0x7fffffffLL) return cudaErrorInvalidValue;
+    auto go = [&](auto cl) {
+        constexpr int N = decltype(cl)::value;
+        static PerDevice carve;
+        prefer_max_shared_once(wgrad_rows_kernel<N>, &carve);
+        return launch_pdl<N>(wgrad_rows_kernel<N>, dim3(pb.c_out * N), dim3(threads), 0, st, pb.c_out, pb.kdim, span, VL, SL,
+                             partials, splits, bsum, (const __nv_bfloat16 *)w, vec3, b, mean, dw, db, dgamma, dbeta,
+                             need_sums ? 1 : 0, call_f16());
+    };
+    if (CL == 1) return go(std::integral_constant<int, 1>());
+    if (CL == 2) return go(std::integral_constant<int, 2>());
+    if (CL == 4) return go(std::integral_constant<int, 4>());
+    return go(std::integral_constant<int, 8>());
 }
 
 // ---- epilogue over k-major partials (the stem's weight gradient) --------------------------------------
