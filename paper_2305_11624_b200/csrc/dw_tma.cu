@@ -70,6 +70,7 @@ __device__ __forceinline__ bool wait_slow(uint32_t bar, uint32_t parity, volatil
 }
 
 struct DwTmaGeom {
+    int cc;            // channels of a block (blockIdx.y: which); c of them in all
     int n, c, h_in, w_in, h_out, w_out, pad_h, pad_w;
     int cols_t;        // consumer thread columns per block (each TW output columns wide)
     int strips;        // column strips per row
@@ -100,14 +101,16 @@ __global__ void __launch_bounds__(TW >= 4 ? 384 : 288, TW >= 4 ? 1 : 2) dw_tma_k
         }
         ctl->abort_flag = 0;
         fence_barrier_init();
+        prefetch_tensormap(&tx);
     }
     __syncthreads();
+    pdl_wait();            // (the kernel behind it is let go at the end: its blocks would sit here and keep others out)
+    const int ch0 = (int)blockIdx.y * g.cc;                    // first channel of this block
     const uint32_t items = (uint32_t)g.n * g.bands * g.strips;
     const int bwo = g.cols_t * TW;                             // output columns per strip
     if (warp == g.consumer_warps) {
         // ---- producer: one elected lane streams the input rows of every item of this block ----
         if (lane == 0) {
-            prefetch_tensormap(&tx);
             uint32_t slot = 0, par = 0;                        // ring position of the next row
             bool ok = true;
             for (uint32_t it = blockIdx.x; it < items && ok; it += gridDim.x) {
@@ -119,7 +122,7 @@ __global__ void __launch_bounds__(TW >= 4 ? 384 : 288, TW >= 4 ? 1 : 2) dw_tma_k
                 for (int k = 0; k < steps; ++k) {
                     if (!mbar_wait_bounded(&ctl->empty[slot], par ^ 1u, abort_flag)) { ok = false; break; }
                     mbar_arrive_expect_tx(&ctl->full[slot], (uint32_t)g.row_bytes);
-                    tma_load_4d(ring + (size_t)slot * g.stage_stride, &tx, &ctl->full[slot], 0, wi0, hi0 + k, img);
+                    tma_load_4d(ring + (size_t)slot * g.stage_stride, &tx, &ctl->full[slot], ch0, wi0, hi0 + k, img);
                     if (++slot == (uint32_t)g.stages) { slot = 0; par ^= 1u; }
                 }
             }
@@ -128,9 +131,9 @@ __global__ void __launch_bounds__(TW >= 4 ? 384 : 288, TW >= 4 ? 1 : 2) dw_tma_k
         return;
     }
     // ---- consumers ----
-    const int v = g.c / 4;
-    const int cv = (int)threadIdx.x % v, tc = (int)threadIdx.x / v;
-    const bool active = tc < g.cols_t;
+    const int v = g.cc / 4, vz = g.c / 4;                      // channel quads of a block, of a pixel
+    const int tc = (int)threadIdx.x / v, cv = (int)threadIdx.x - tc * v;
+    const bool active = tc < g.cols_t && ch0 + cv * 4 < g.c;
     f32x2 wr[KH * KW][2];
     f32x2 bv[2] = {0ull, 0ull};
     if (active) {
@@ -139,7 +142,7 @@ __global__ void __launch_bounds__(TW >= 4 ? 384 : 288, TW >= 4 ? 1 : 2) dw_tma_k
         float sc[4] = {1.f, 1.f, 1.f, 1.f}, bf[4] = {0.f, 0.f, 0.f, 0.f};
 #pragma unroll
         for (int e = 0; e < 4; ++e) {
-            const int c = cv * 4 + e;
+            const int c = ch0 + cv * 4 + e;
             if (fold.gamma) {
                 const float r = 1.0f / sqrtf(fold.var[c] + fold.eps);
                 sc[e] = fold.gamma[c] * r;
@@ -157,7 +160,7 @@ __global__ void __launch_bounds__(TW >= 4 ? 384 : 288, TW >= 4 ? 1 : 2) dw_tma_k
             const int src = reverse_taps ? KH * KW - 1 - tp : tp;
             float f[4];
 #pragma unroll
-            for (int e = 0; e < 4; ++e) f[e] = sc[e] * load_h16(w + (size_t)(cv * 4 + e) * (KH * KW) + src, H ? 1 : 0);
+            for (int e = 0; e < 4; ++e) f[e] = sc[e] * load_h16(w + (size_t)(ch0 + cv * 4 + e) * (KH * KW) + src, H ? 1 : 0);
             wr[tp][0] = pair(f[0], f[1]);
             wr[tp][1] = pair(f[2], f[3]);
         }
@@ -167,7 +170,7 @@ __global__ void __launch_bounds__(TW >= 4 ? 384 : 288, TW >= 4 ? 1 : 2) dw_tma_k
 #pragma unroll
         for (int tp = 0; tp < KH * KW; ++tp) wr[tp][0] = wr[tp][1] = 0ull;
     }
-    const uint32_t col_bytes = (uint32_t)g.c * 2;
+    const uint32_t col_bytes = (uint32_t)g.cc * 2;
     uint32_t col_addr[NX];                                     // this thread's columns in ring slot 0
 #pragma unroll
     for (int j = 0; j < NX; ++j)
@@ -175,7 +178,7 @@ __global__ void __launch_bounds__(TW >= 4 ? 384 : 288, TW >= 4 ? 1 : 2) dw_tma_k
     const uint32_t full0 = smem_u32(&ctl->full[0]), empty0 = smem_u32(&ctl->empty[0]);
     const uint32_t ring_bytes = (uint32_t)g.stages * g.stage_stride;
     uint32_t slot = 0, slot_off = 0, par = 0;                  // ring position of the next row
-    const ptrdiff_t zpitch = (ptrdiff_t)g.w_out * v;
+    const ptrdiff_t zpitch = (ptrdiff_t)g.w_out * vz;
     bool ok = true;
     for (uint32_t it = blockIdx.x; it < items && ok; it += gridDim.x) {
         const int strip = (int)(it % (uint32_t)g.strips);
@@ -185,7 +188,7 @@ __global__ void __launch_bounds__(TW >= 4 ? 384 : 288, TW >= 4 ? 1 : 2) dw_tma_k
         int steps = rows + KH - 1;
         const int wo0 = strip * bwo + tc * TW;
         // output row pointer, KH - 1 rows behind the input row being read
-        uint2 *zr = z + ((ptrdiff_t)(img * g.h_out + band * g.th - (KH - 1)) * g.w_out + wo0) * v + cv;
+        uint2 *zr = z + ((ptrdiff_t)(img * g.h_out + band * g.th - (KH - 1)) * g.w_out + wo0) * vz + ch0 / 4 + cv;
         bool out_ok[TW];
 #pragma unroll
         for (int j = 0; j < TW; ++j) out_ok[j] = active && wo0 + j < g.w_out;
@@ -238,7 +241,7 @@ __global__ void __launch_bounds__(TW >= 4 ? 384 : 288, TW >= 4 ? 1 : 2) dw_tma_k
                             const bool row_done = k >= KH - 1;
 #pragma unroll
                             for (int j = 0; j < TW; ++j)
-                                stg_u2_if(zr + (ptrdiff_t)j * v, narrow_t<H>(acc[sl][j][0]), narrow_t<H>(acc[sl][j][1]), row_done && out_ok[j]);
+                                stg_u2_if(zr + (ptrdiff_t)j * vz, narrow_t<H>(acc[sl][j][0]), narrow_t<H>(acc[sl][j][1]), row_done && out_ok[j]);
                         }
                         zr += zpitch;
                     }
@@ -274,14 +277,18 @@ __global__ void __launch_bounds__(TW >= 4 ? 384 : 288, TW >= 4 ? 1 : 2) dw_tma_w
         }
         ctl->abort_flag = 0;
         fence_barrier_init();
+        prefetch_tensormap(&tx);
+        prefetch_tensormap(&tdz);
     }
     __syncthreads();
+    pdl_wait();
+    const int ch0 = (int)blockIdx.y * g.cc;                    // first channel of this block
     const uint32_t items = (uint32_t)g.n * g.bands * g.strips;
     const int bwo = g.cols_t * TW;                             // dZ columns per strip
-    const uint32_t x_bytes = (uint32_t)(bwo + KW - 1) * g.c * 2, dz_bytes = (uint32_t)bwo * g.c * 2;
+    const uint32_t x_bytes = (uint32_t)(bwo + KW - 1) * g.cc * 2, dz_bytes = (uint32_t)bwo * g.cc * 2;
     const uint32_t dz_off = (x_bytes + 127u) & ~127u;          // dZ row behind the X row in a slot
-    const int v = g.c / 4;
-    const int cv = (int)threadIdx.x % v, tc = (int)threadIdx.x / v;
+    const int v = g.cc / 4;
+    const int tc = (int)threadIdx.x / v, cv = (int)threadIdx.x - tc * v;
     const bool active = warp < g.consumer_warps && tc < g.cols_t;
     f32x2 acc[NACC][2];
 #pragma unroll
@@ -289,8 +296,6 @@ __global__ void __launch_bounds__(TW >= 4 ? 384 : 288, TW >= 4 ? 1 : 2) dw_tma_w
     if (warp == g.consumer_warps) {
         // ---- producer ----
         if (lane == 0) {
-            prefetch_tensormap(&tx);
-            prefetch_tensormap(&tdz);
             uint32_t slot = 0, par = 0;
             bool ok = true;
             for (uint32_t it = blockIdx.x; it < items && ok; it += gridDim.x) {
@@ -303,8 +308,8 @@ __global__ void __launch_bounds__(TW >= 4 ? 384 : 288, TW >= 4 ? 1 : 2) dw_tma_w
                     if (!mbar_wait_bounded(&ctl->empty[slot], par ^ 1u, abort_flag)) { ok = false; break; }
                     uint8_t *dst = ring + (size_t)slot * g.stage_stride;
                     mbar_arrive_expect_tx(&ctl->full[slot], x_bytes + (k < rows ? dz_bytes : 0u));
-                    tma_load_4d(dst, &tx, &ctl->full[slot], 0, wo0 - g.pad_w, ho0 - g.pad_h + k, img);
-                    if (k < rows) tma_load_4d(dst + dz_off, &tdz, &ctl->full[slot], 0, wo0, ho0 + k, img);
+                    tma_load_4d(dst, &tx, &ctl->full[slot], ch0, wo0 - g.pad_w, ho0 - g.pad_h + k, img);
+                    if (k < rows) tma_load_4d(dst + dz_off, &tdz, &ctl->full[slot], ch0, wo0, ho0 + k, img);
                     if (++slot == (uint32_t)g.stages) { slot = 0; par ^= 1u; }
                 }
             }
@@ -312,7 +317,7 @@ __global__ void __launch_bounds__(TW >= 4 ? 384 : 288, TW >= 4 ? 1 : 2) dw_tma_w
         }
     } else {
         // ---- consumers ----
-        const uint32_t col_bytes = (uint32_t)g.c * 2;
+        const uint32_t col_bytes = (uint32_t)g.cc * 2;
         uint32_t x_addr[NX], dz_addr[TW];
 #pragma unroll
         for (int j = 0; j < NX; ++j)
@@ -402,11 +407,12 @@ __global__ void __launch_bounds__(TW >= 4 ? 384 : 288, TW >= 4 ? 1 : 2) dw_tma_w
         }
     }
     __syncthreads();
-    for (int i = threadIdx.x; i < g.c * NACC; i += blockDim.x) {
+    const int mine_c = min(g.cc, g.c - ch0);
+    for (int i = threadIdx.x; i < mine_c * NACC; i += blockDim.x) {
         const int c = i / NACC, t = i - c * NACC;
         float sum = 0.f;
         for (int col = 0; col < g.cols_t; ++col) sum += red[((size_t)col * v + c / 4) * (NACC * 4) + t * 4 + (c & 3)];
-        part[(size_t)blockIdx.x * g.c * NACC + i] = sum;
+        part[((size_t)blockIdx.x * g.c + ch0) * NACC + i] = sum;
     }
 }
 
@@ -424,6 +430,8 @@ __global__ void __launch_bounds__(32 * (TAPS + 1)) dw_wgrad_finish_kernel(int c_
                                                                            float *__restrict__ dgamma,
                                                                            float *__restrict__ dbeta, int f16) {
     __shared__ float tot[TAPS + 1];
+    pdl_wait();
+    pdl_launch_dependents();
     const int c = blockIdx.x, t = threadIdx.x >> 5, lane = threadIdx.x & 31;
     float sum = 0.f;
     for (int p = lane; p < nparts; p += 32) sum += part[((size_t)p * c_total + c) * (TAPS + 1) + t];
@@ -450,7 +458,7 @@ __global__ void __launch_bounds__(32 * (TAPS + 1)) dw_wgrad_finish_kernel(int c_
 }  // namespace
 
 bool dw_tma_eligible(const Problem &pb) {
-    return pb.groups == pb.c_in && pb.c_in == pb.c_out && pb.c_in % 8 == 0 && pb.c_in <= 256 && pb.kh == 3 &&
+    return pb.groups == pb.c_in && pb.c_in == pb.c_out && pb.c_in % 8 == 0 && pb.c_in <= 65535 && pb.kh == 3 &&
            pb.kw == 3 && pb.stride_h == 1 && pb.stride_w == 1 && pb.dil_h == 1 && pb.dil_w == 1 && pb.pad_h >= 0 &&
            pb.pad_w >= 0 && pb.pad_h <= 2 && pb.pad_w <= 2 && pb.w_out >= 8 && pb.p * pb.c_out < (1LL << 31) &&
            pb.pin * pb.c_in < (1LL << 31);
@@ -467,7 +475,12 @@ static cudaError_t dw_tma_geometry(const Problem &pb, int tw, int kh, int kw, bo
     DwTmaGeom g{};
     g.n = pb.n; g.c = pb.c_in; g.h_in = pb.h_in; g.w_in = pb.w_in; g.h_out = pb.h_out; g.w_out = pb.w_out;
     g.pad_h = pb.pad_h; g.pad_w = pb.pad_w;
-    const int v = pb.c_in / 4;
+    // up to 256 channels a block; more are cut into equal parts (of whole 32-byte sectors), each with its share of the blocks
+    // (forward + backward on the row-streaming kernels of dw_kernels.cu and here: 320 channels at 136 x 202, N = 12 688 and
+    // 295 us, 352 at 32 x 49, N = 18 119 and 49, 352 at 19 x 20, N = 2 38 and 20)
+    const int parts = (pb.c_in + 255) / 256;
+    g.cc = parts == 1 ? pb.c_in : ((pb.c_in + parts - 1) / parts + 15) / 16 * 16;
+    const int v = g.cc / 4;
     const int tcols = (pb.w_out + tw - 1) / tw;                // thread columns in a row
     int cols_max = max_consumers / v;
     if (cols_max < 1) cols_max = 1;
@@ -476,9 +489,9 @@ static cudaError_t dw_tma_geometry(const Problem &pb, int tw, int kh, int kw, bo
     g.strips = (tcols + cols_max - 1) / cols_max;
     g.cols_t = (tcols + g.strips - 1) / g.strips;
     g.consumer_warps = (g.cols_t * v + 31) / 32;
-    g.row_bytes = (g.cols_t * tw + kw - 1) * pb.c_in * 2;
+    g.row_bytes = (g.cols_t * tw + kw - 1) * g.cc * 2;
     g.stage_stride = (g.row_bytes + 127) / 128 * 128;
-    if (with_dz) g.stage_stride += (g.cols_t * tw * pb.c_in * 2 + 127) / 128 * 128;
+    if (with_dz) g.stage_stride += (g.cols_t * tw * g.cc * 2 + 127) / 128 * 128;
     g.stages = (int)(ring_budget / g.stage_stride);
     if (g.stages > kDwMaxStages) g.stages = kDwMaxStages;
     if (g.stages < 4) return cudaErrorInvalidValue;
@@ -486,7 +499,7 @@ static cudaError_t dw_tma_geometry(const Problem &pb, int tw, int kh, int kw, bo
     cudaError_t e = cudaGetDevice(&dev);
     if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     if (e != cudaSuccess) return e;
-    const long long resident = (tw >= 4 ? 1LL : 2LL) * sms;
+    const long long slots = (tw >= 4 ? 1LL : 2LL) * sms, resident = slots / parts > 0 ? slots / parts : 1;
     // band height: the one that minimises (items per block, rounded up) x (input rows per item)
     long long best = -1;
     g.th = pb.h_out;
@@ -503,12 +516,12 @@ static cudaError_t dw_tma_geometry(const Problem &pb, int tw, int kh, int kw, bo
     return cudaSuccess;
 }
 
-static bool dw_tma_map(CUtensorMap *tm, const void *base, int n, int h, int w, int c, int box_w) {
+static bool dw_tma_map(CUtensorMap *tm, const void *base, int n, int h, int w, int c, int box_c, int box_w) {
     const unsigned long long dims[4] = {(unsigned long long)c, (unsigned long long)w, (unsigned long long)h,
                                         (unsigned long long)n};
     const unsigned long long str[4] = {0, (unsigned long long)c * 2, (unsigned long long)w * c * 2,
                                        (unsigned long long)h * w * c * 2};
-    const unsigned int box[4] = {(unsigned)c, (unsigned)box_w, 1, 1};
+    const unsigned int box[4] = {(unsigned)box_c, (unsigned)box_w, 1, 1};
     return make_tmap_tiled_bf16_linear(tm, base, 4, dims, str, box);
 }
 
@@ -527,21 +540,20 @@ cudaError_t launch_dw_tma(const Problem &pb, const void *x, const void *w, const
     cudaError_t e = dw_tma_geometry(pb, TW, KH, KW, false, &g, &grid);
     if (e != cudaSuccess) return e;
     CUtensorMap tx;
-    if (!dw_tma_map(&tx, x, pb.n, pb.h_in, pb.w_in, pb.c_in, g.cols_t * TW + KW - 1)) return cudaErrorInvalidValue;
+    if (!dw_tma_map(&tx, x, pb.n, pb.h_in, pb.w_in, pb.c_in, g.cc, g.cols_t * TW + KW - 1)) return cudaErrorInvalidValue;
+    const unsigned parts = (unsigned)((pb.c_in + g.cc - 1) / g.cc);
     int *err = nullptr;
     if ((e = error_word_address(&err)) != cudaSuccess) return e;
     static PerDevice attr, attr_h;        // (one flag per instantiation)
     const BnFold none{nullptr, nullptr, nullptr, nullptr, nullptr, 0.f, nullptr};
     if (call_f16()) {
         if ((e = max_dynamic_smem_once(dw_tma_kernel<TW, KH, KW, true>, 210 * 1024, &attr_h)) != cudaSuccess) return e;
-        dw_tma_kernel<TW, KH, KW, true><<<grid, (g.consumer_warps + 1) * 32, dw_tma_smem(g), st>>>(
+        return launch_pdl(dw_tma_kernel<TW, KH, KW, true>, dim3(grid, parts), dim3((g.consumer_warps + 1) * 32), dw_tma_smem(g), st, 
             tx, g, (const __nv_bfloat16 *)w, bias, fold ? *fold : none, scale, reverse_taps ? 1 : 0, (uint2 *)z, err);
-        return cudaGetLastError();
     }
     if ((e = max_dynamic_smem_once(dw_tma_kernel<TW, KH, KW, false>, 210 * 1024, &attr)) != cudaSuccess) return e;
-    dw_tma_kernel<TW, KH, KW, false><<<grid, (g.consumer_warps + 1) * 32, dw_tma_smem(g), st>>>(
+    return launch_pdl(dw_tma_kernel<TW, KH, KW, false>, dim3(grid, parts), dim3((g.consumer_warps + 1) * 32), dw_tma_smem(g), st, 
         tx, g, (const __nv_bfloat16 *)w, bias, fold ? *fold : none, scale, reverse_taps ? 1 : 0, (uint2 *)z, err);
-    return cudaGetLastError();
 }
 
 // Partial rows the backward-weight kernel writes: one per block, [C][KH KW + 1] floats each.
@@ -560,28 +572,26 @@ cudaError_t launch_dw_tma_wgrad(const Problem &pb, const void *dz, const void *x
     cudaError_t e = dw_tma_geometry(pb, TW, KH, KW, true, &g, &grid);
     if (e != cudaSuccess) return e;
     CUtensorMap tx, tdz;
-    if (!dw_tma_map(&tx, x, pb.n, pb.h_in, pb.w_in, pb.c_in, g.cols_t * TW + KW - 1)) return cudaErrorInvalidValue;
-    if (!dw_tma_map(&tdz, dz, pb.n, pb.h_out, pb.w_out, pb.c_in, g.cols_t * TW)) return cudaErrorInvalidValue;
+    if (!dw_tma_map(&tx, x, pb.n, pb.h_in, pb.w_in, pb.c_in, g.cc, g.cols_t * TW + KW - 1)) return cudaErrorInvalidValue;
+    if (!dw_tma_map(&tdz, dz, pb.n, pb.h_out, pb.w_out, pb.c_in, g.cc, g.cols_t * TW)) return cudaErrorInvalidValue;
+    const unsigned parts = (unsigned)((pb.c_in + g.cc - 1) / g.cc);
     int *err = nullptr;
     if ((e = error_word_address(&err)) != cudaSuccess) return e;
     static PerDevice attr, attr_h;
     *nparts = (int)grid;
     if (call_f16()) {
         if ((e = max_dynamic_smem_once(dw_tma_wgrad_kernel<TW, KH, KW, true>, 210 * 1024, &attr_h)) != cudaSuccess) return e;
-        dw_tma_wgrad_kernel<TW, KH, KW, true><<<grid, (g.consumer_warps + 1) * 32, dw_tma_smem(g), st>>>(tx, tdz, g, part, err);
-        return cudaGetLastError();
+        return launch_pdl(dw_tma_wgrad_kernel<TW, KH, KW, true>, dim3(grid, parts), dim3((g.consumer_warps + 1) * 32), dw_tma_smem(g), st, tx, tdz, g, part, err);
     }
     if ((e = max_dynamic_smem_once(dw_tma_wgrad_kernel<TW, KH, KW, false>, 210 * 1024, &attr)) != cudaSuccess) return e;
-    dw_tma_wgrad_kernel<TW, KH, KW, false><<<grid, (g.consumer_warps + 1) * 32, dw_tma_smem(g), st>>>(tx, tdz, g, part, err);
-    return cudaGetLastError();
+    return launch_pdl(dw_tma_wgrad_kernel<TW, KH, KW, false>, dim3(grid, parts), dim3((g.consumer_warps + 1) * 32), dw_tma_smem(g), st, tx, tdz, g, part, err);
 }
 
 cudaError_t launch_dw_wgrad_finish(const Problem &pb, const float *part, int nparts, const void *w, const float *vec3,
                                    const float *b, const float *mean, float *dw, float *db, float *dgamma,
                                    float *dbeta, cudaStream_t st) {
-    dw_wgrad_finish_kernel<9><<<pb.c_in, 32 * 10, 0, st>>>(pb.c_in, nparts, part, (const __nv_bfloat16 *)w, vec3, b, mean,
+    return launch_pdl(dw_wgrad_finish_kernel<9>, dim3(pb.c_in), dim3(32 * 10), 0, st, pb.c_in, nparts, part, (const __nv_bfloat16 *)w, vec3, b, mean,
                                                          dw, db, dgamma, dbeta, call_f16());
-    return cudaGetLastError();
 }
 
 }  // namespace convbn
