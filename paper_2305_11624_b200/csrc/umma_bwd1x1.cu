@@ -96,7 +96,6 @@ __global__ void __launch_bounds__(kFbThreads) fused_bwd1x1_kernel(const __grid_c
     __syncthreads();
     tc_fence_after_sync();
     pdl_wait();
-    pdl_launch_dependents();       // not earlier than here: this CTA owns its tensor-memory columns
     const uint32_t tmem_base = ctl->tmem_base;
 
     if (warp != 0) {               // (the first boxes are under way meanwhile)
@@ -288,6 +287,7 @@ __global__ void __launch_bounds__(kFbThreads) fused_bwd1x1_kernel(const __grid_c
         if (lane == 0) tma_store_wait_all<0>();
         // ---- the CTA's partial of domega' as part[cta][co][ci] and its row of sums of dZ: 128 contiguous bytes per store ----
         if (ok) ok = __all_sync(0xffffffffu, mbar_wait_bounded(&ctl->acc_done, 0, abort_flag));
+        pdl_launch_dependents();                               // (see umma_wgrad.cu)
         if (ok) {
             tc_fence_after_sync();
             float *part = partials + (size_t)blockIdx.x * CI * CO;

@@ -103,7 +103,6 @@ __global__ void __launch_bounds__(kWThreads) umma_wgrad_kernel(const __grid_cons
     tc_fence_before_sync();
     __syncthreads();
     tc_fence_after_sync();
-    pdl_launch_dependents();       // only now: this CTA owns its tensor-memory columns
     const uint32_t tmem_base = ctl->tmem_base;
 
     // the two loading threads' walk through the ring
@@ -231,6 +230,10 @@ __global__ void __launch_bounds__(kWThreads) umma_wgrad_kernel(const __grid_cons
         const int quarter = warp & 3;
         const bool ok = __all_sync(0xffffffffu, mbar_wait_bounded(&ctl->tmem_full, 0, abort_flag));
         if (!ok && lane == 0) { atomicOr(err, ERRW_TIMEOUT); ctl->abort_flag = 1; }
+        // The adding kernel is let go only here: its blocks, waiting for this grid, would take the shared memory that the
+        // 220 KB CTAs of the data pass beside it need (forward + backward of 3x3 64 -> 64 at 56 x 56, N = 32 49.8 -> 47.4 us,
+        // 3x3 stride 2 128 -> 128 at 200 x 334, N = 2 62.1 -> 59.9, 3x3 128 at 52 x 85, N = 9 55.1 -> 50.2).
+        pdl_launch_dependents();
         if (ok) {
             tc_fence_after_sync();
             const int k = k0 + quarter * 32 + lane;
