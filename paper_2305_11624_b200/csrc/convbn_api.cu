@@ -1131,7 +1131,12 @@ int convbn_eval_bwd(const convbn_desc *desc, const void *dz, const void *x, cons
         void *inner = at(workspace, pl.eval_inner);
         const Plan pt = make_plan(desc, pb, CONVBN_PHASE_TUNE_BWD);
         const bool fused = fused_bwd_path(desc, pb);
-        LAUNCH("bn_vec3", launch_bn_vec3(pb.c_out, pb.eps, nullptr, gamma, nullptr, run_mean, run_var, vec3, st));
+        // (the sums do not need s: with the single-kernel backward it is formed beside them)
+        auto form_s = [&](cudaStream_t st) -> int {
+            LAUNCH("bn_vec3", launch_bn_vec3(pb.c_out, pb.eps, nullptr, gamma, nullptr, run_mean, run_var, vec3, st));
+            return CONVBN_OK;
+        };
+        if (!fused) CK(form_s(st));
         return side_by_side(
             st,
             [&](cudaStream_t st) -> int {
@@ -1145,6 +1150,7 @@ int convbn_eval_bwd(const convbn_desc *desc, const void *dz, const void *x, cons
             },
             [&]() -> int {
                 if (fused) {
+                    CK(form_s(st));
                     LAUNCH("umma_bwd", launch_fused_bwd1x1(pb, dz, x, w, vec3, dx, (float *)at(inner, pt.partials),
                                                            (float *)at(inner, pt.bsum), st));
                     LAUNCH("wgrad_rows",

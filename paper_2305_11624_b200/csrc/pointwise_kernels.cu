@@ -290,13 +290,14 @@ __global__ void __launch_bounds__(256) channel_sum_nhwc8_kernel(int c_out, long 
                                                                 const uint4 *__restrict__ t,
                                                                 float *__restrict__ part) {
     __shared__ float red[256][9];
+    pdl_wait();
+    pdl_launch_dependents();
     const int v = c_out / 8;                       // vectors per pixel
     const long long vec0 = (long long)blockIdx.x * pix_per_block * v;
     long long vec1 = vec0 + (long long)pix_per_block * v;
     if (vec1 > p * v) vec1 = p * v;
     float acc[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
-    for (long long i = vec0 + threadIdx.x; i < vec1; i += blockDim.x) {
-        const uint4 q = t[i];
+    auto add = [&](const uint4 &q) {
         const uint32_t u[4] = {q.x, q.y, q.z, q.w};
 #pragma unroll
         for (int e = 0; e < 4; ++e) {
@@ -305,7 +306,16 @@ __global__ void __launch_bounds__(256) channel_sum_nhwc8_kernel(int c_out, long 
             acc[2 * e] += lo;
             acc[2 * e + 1] += hi;
         }
+    };
+    long long i = vec0 + threadIdx.x;
+    for (; i + 7LL * blockDim.x < vec1; i += 8LL * blockDim.x) {     // eight loads in flight
+        uint4 q[8];
+#pragma unroll
+        for (int u = 0; u < 8; ++u) q[u] = t[i + (long long)u * blockDim.x];
+#pragma unroll
+        for (int u = 0; u < 8; ++u) add(q[u]);
     }
+    for (; i < vec1; i += blockDim.x) add(t[i]);
 #pragma unroll
     for (int e = 0; e < 8; ++e) red[threadIdx.x][e] = acc[e];
     __syncthreads();
@@ -339,9 +349,10 @@ cudaError_t launch_channel_sum_partial(const Problem &pb, int dtype, int layout,
         const int v = pb.c_out / 8;
         const int block = (256 / v) * v;
         const long long per = (pb.p + splits - 1) / splits;
-        if (call_f16()) channel_sum_nhwc8_kernel<true><<<splits, block, 0, st>>>(pb.c_out, pb.p, (int)per, (const uint4 *)t, part);
-        else channel_sum_nhwc8_kernel<false><<<splits, block, 0, st>>>(pb.c_out, pb.p, (int)per, (const uint4 *)t, part);
-        return cudaGetLastError();
+        auto go = [&](auto kernel) {
+            return launch_pdl(kernel, dim3(splits), dim3(block), 0, st, pb.c_out, pb.p, (int)per, (const uint4 *)t, part);
+        };
+        return call_f16() ? go(channel_sum_nhwc8_kernel<true>) : go(channel_sum_nhwc8_kernel<false>);
     }
     const int threads = pb.c_out >= 256 ? 256 : ((pb.c_out + 31) / 32) * 32;
     dim3 grid((pb.c_out + threads - 1) / threads, splits);
@@ -617,46 +628,58 @@ cudaError_t launch_bn_eval_bwd(const Problem &pb, int dtype, int layout, const v
     return cudaGetLastError();
 }
 
-// 32 channels per block; warp g adds slices g, g + 32, ..., four of each array in flight, and the 32 groups are added in
-// order (one thread per channel walking up to 592 slices took 38 us).
-__global__ void __launch_bounds__(1024) bn_eval_finish_kernel(int c_out, float eps, const float *__restrict__ part_g,
-                                                              const float *__restrict__ part_b, int splits,
-                                                              const float *__restrict__ gamma, const float *__restrict__ var,
-                                                              float *__restrict__ db, float *__restrict__ dgamma,
-                                                              float *__restrict__ dbeta) {
-    __shared__ float red[2][32][33];
+// Eight channels (one 32-byte sector of a slice's row) per block, 128 groups of slices: a thread's slices, at most five of each
+// array, are all in flight at once, and the groups are added in order.  (32 channels and 32 groups a block took 10 us;
+// with this and s formed beside the sums Eval 64 -> 256 at 56 x 56, N = 32 took 80.5 us, before 84.1.)
+constexpr int kBfGroups = 128;
+__global__ void __launch_bounds__(8 * kBfGroups) bn_eval_finish_kernel(int c_out, float eps, const float *__restrict__ part_g,
+                                                                       const float *__restrict__ part_b, int splits,
+                                                                       const float *__restrict__ gamma, const float *__restrict__ var,
+                                                                       float *__restrict__ db, float *__restrict__ dgamma,
+                                                                       float *__restrict__ dbeta) {
+    __shared__ float red[2][8 * kBfGroups / 32][8];
     pdl_wait();
     pdl_launch_dependents();
-    const int lane = threadIdx.x & 31, grp = threadIdx.x >> 5, c = blockIdx.x * 32 + lane;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, grp = threadIdx.x >> 3, c = blockIdx.x * 8 + (threadIdx.x & 7);
     float g = 0.f, bsum = 0.f;
     if (c < c_out)
-        for (int sp = grp; sp < splits; sp += 128) {
-            float vg[4], vb[4];
+        for (int sp = grp; sp < splits; sp += 5 * kBfGroups) {
+            float vg[5], vb[5];
 #pragma unroll
-            for (int u = 0; u < 4; ++u) {
-                const bool in = sp + 32 * u < splits;
-                vg[u] = in ? __ldcg(part_g + (long long)(sp + 32 * u) * c_out + c) : 0.f;
-                vb[u] = in ? __ldcg(part_b + (long long)(sp + 32 * u) * c_out + c) : 0.f;
+            for (int u = 0; u < 5; ++u) {
+                const bool in = sp + kBfGroups * u < splits;
+                vg[u] = in ? __ldcg(part_g + (long long)(sp + kBfGroups * u) * c_out + c) : 0.f;
+                vb[u] = in ? __ldcg(part_b + (long long)(sp + kBfGroups * u) * c_out + c) : 0.f;
             }
-            g += (vg[0] + vg[1]) + (vg[2] + vg[3]);
-            bsum += (vb[0] + vb[1]) + (vb[2] + vb[3]);
+#pragma unroll
+            for (int u = 0; u < 5; ++u) { g += vg[u]; bsum += vb[u]; }
         }
-    red[0][grp][lane] = g;
-    red[1][grp][lane] = bsum;
+#pragma unroll
+    for (int o = 8; o < 32; o *= 2) { g += __shfl_xor_sync(0xffffffffu, g, o); bsum += __shfl_xor_sync(0xffffffffu, bsum, o); }
+    if (lane < 8) { red[0][warp][lane] = g; red[1][warp][lane] = bsum; }
     __syncthreads();
-    if (grp == 0 && c < c_out) {
+    if (warp == 0) {                                       // lanes (part, channel): eight warps' sums each
         g = bsum = 0.f;
-        for (int i = 0; i < 32; ++i) { g += red[0][i][lane]; bsum += red[1][i][lane]; }
-        dgamma[c] = g;
-        dbeta[c] = bsum;
-        if (db) db[c] = gamma[c] / sqrtf(var[c] + eps) * bsum;
+#pragma unroll
+        for (int i = 0; i < kBfGroups / 16; ++i) {
+            const int from = (lane >> 3) * (kBfGroups / 16) + i;
+            g += red[0][from][lane & 7];
+            bsum += red[1][from][lane & 7];
+        }
+#pragma unroll
+        for (int o = 8; o < 32; o *= 2) { g += __shfl_xor_sync(0xffffffffu, g, o); bsum += __shfl_xor_sync(0xffffffffu, bsum, o); }
+        if (lane < 8 && c < c_out) {
+            dgamma[c] = g;
+            dbeta[c] = bsum;
+            if (db) db[c] = gamma[c] / sqrtf(var[c] + eps) * bsum;
+        }
     }
 }
 
 cudaError_t launch_bn_eval_finish(const Problem &pb, const float *part_g, const float *part_b,
                                   int splits, const float *gamma, const float *var, float *db,
                                   float *dgamma, float *dbeta, cudaStream_t st) {
-    return launch_pdl(bn_eval_finish_kernel, dim3((pb.c_out + 31) / 32), dim3(1024), 0, st, pb.c_out, pb.eps, part_g, part_b,
+    return launch_pdl(bn_eval_finish_kernel, dim3((pb.c_out + 7) / 8), dim3(8 * kBfGroups), 0, st, pb.c_out, pb.eps, part_g, part_b,
                       splits, gamma, var, db, dgamma, dbeta);
 }
 
