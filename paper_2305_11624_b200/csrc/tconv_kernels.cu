@@ -43,6 +43,26 @@ __global__ void __launch_bounds__(256) tconv_rescale_kernel(long long count, int
         w_out[i] = from_f32<T>(to_f32(w[i]) * s[tconv_channel(i, taps, cig, cog, nhwc)]);
 }
 
+// NHWC with C_out/G a multiple of 8, 16-bit elements: eight consecutive channels a thread, 32-bit index arithmetic (the general
+// kernel divides 64-bit numbers twice per weight).
+template <bool H>
+__global__ void __launch_bounds__(256) tconv_rescale8_kernel(uint32_t vecs, uint32_t row, uint32_t cig, uint32_t cog,
+                                                             const uint4 *__restrict__ w, const float *__restrict__ s,
+                                                             uint4 *__restrict__ w_out) {
+    pdl_wait();
+    pdl_launch_dependents();
+    const uint32_t i = blockIdx.x * 256 + threadIdx.x;
+    if (i >= vecs) return;
+    const uint32_t j = i * 8 % cog, ci = i * 8 / row;                // row = taps C_out/G
+    const float *sp = s + ci / cig * cog + j;
+    const uint4 q = w[i];
+    const float4 s0 = *(const float4 *)sp, s1 = *(const float4 *)(sp + 4);
+    float f[8];
+    unpack2_t<H>(q.x, f[0], f[1]); unpack2_t<H>(q.y, f[2], f[3]); unpack2_t<H>(q.z, f[4], f[5]); unpack2_t<H>(q.w, f[6], f[7]);
+    w_out[i] = make_uint4(pack2_t<H>(f[0] * s0.x, f[1] * s0.y), pack2_t<H>(f[2] * s0.z, f[3] * s0.w),
+                          pack2_t<H>(f[4] * s1.x, f[5] * s1.y), pack2_t<H>(f[6] * s1.z, f[7] * s1.w));
+}
+
 // z += b' per channel, in place
 template <class T>
 __global__ void __launch_bounds__(256) tconv_bias_kernel(long long count, int c, long long hw, bool nhwc,
@@ -94,48 +114,67 @@ __global__ void __launch_bounds__(256) tconv_param_epilogue_kernel(int c_out, in
     }
 }
 
-// Block (bx, by): weight columns k = (tap, co) [32 bx, +32) x input channels [32 by, +32), one output channel group since
-// 32 divides C_out.  Thread (tx = k, ty = ci) adds its element of part[split][C_in][k] over the slices, eight loads in
-// flight, in slice order, scales it by s[co] and stores it.  The last block of a group of 32
-// output channels (a counter) adds the dot products and the sums of dZ in fixed order.  Bound by the read of the
-// partials (L2): 256 -> 128 channels, 2 x 2, 29 slices: 15 MB; with the sum, the scale and the per-channel
-// sums in kernels of their own the same work took 87 us.
-__global__ void __launch_bounds__(1024) tconv_wgrad_epilogue_kernel(int c_in, int c_out, int kdim, const float *__restrict__ part,
-                                                                    int splits, const __nv_bfloat16 *__restrict__ w,
-                                                                    const float *__restrict__ vec3, const float *__restrict__ b,
-                                                                    const float *__restrict__ mean, const float *__restrict__ bsum,
-                                                                    int bsplits, float *__restrict__ dotpart,
-                                                                    unsigned int *__restrict__ counters, float *__restrict__ dw,
-                                                                    float *__restrict__ db, float *__restrict__ dgamma,
-                                                                    float *__restrict__ dbeta, int f16) {
-    __shared__ float tile[32][33], prod[32][33];
+// Block (bx, by): weight columns k = (tap, co) [32 bx, +32) x input channels [8 by, +8), one output channel group since
+// 32 divides C_out.  Thread (l = four columns, ci, z = slice group) adds slices z, z + 8, ... of part[split][C_in][k], four
+// loads in flight; the groups are added in halves through shared memory.  The last block of a group of 32
+// output channels (a counter) adds the dot products and the sums of dZ in fixed order.  Bound by the latency of the reads of
+// the partials (L2): 256 -> 128 channels, 2 x 2, 29 slices: 15 MB.  A thread per weight and all its slices (128 blocks of
+// 1024 threads, four bytes a load) took 15 us; with the sum, the scale and the per-channel sums in kernels of their own the
+// same work took 87 us.
+constexpr int kTeCi = 8, kTeSlices = 8, kTeThreads = 8 * kTeCi * kTeSlices;
+__global__ void __launch_bounds__(kTeThreads) tconv_wgrad_epilogue_kernel(int c_in, int c_out, int kdim, const float *__restrict__ part,
+                                                                          int splits, const __nv_bfloat16 *__restrict__ w,
+                                                                          const float *__restrict__ vec3, const float *__restrict__ b,
+                                                                          const float *__restrict__ mean, const float *__restrict__ bsum,
+                                                                          int bsplits, float *__restrict__ dotpart,
+                                                                          unsigned int *__restrict__ counters, float *__restrict__ dw,
+                                                                          float *__restrict__ db, float *__restrict__ dgamma,
+                                                                          float *__restrict__ dbeta, int f16) {
+    __shared__ float4 red[kTeThreads];
+    __shared__ float tile[kTeThreads / 32][33], sums[kTeThreads / 32][33];
     __shared__ int is_last;
     pdl_wait();
     pdl_launch_dependents();
-    const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
-    const int k0 = blockIdx.x * 32, ci0 = blockIdx.y * 32, co0 = k0 % c_out;       // (the longer dimension is the unbounded one)
-    const float wv = load_h16(w + (size_t)(ci0 + ty) * kdim + k0 + tx, f16);
-    const float *src = part + (size_t)(ci0 + ty) * kdim + k0 + tx;
-    const size_t slice = (size_t)kdim * c_in;
-    float v = 0.f;
-    for (int sp = 0; sp < splits; sp += 8) {
-        float q[8];
+    const int tid = threadIdx.x, l = tid & 7, ci = (tid >> 3) & (kTeCi - 1), z = tid / (8 * kTeCi);
+    const int k0 = blockIdx.x * 32, ci0 = blockIdx.y * kTeCi, co0 = k0 % c_out;    // (the longer dimension is the unbounded one)
+    const size_t slice = (size_t)kdim * c_in, at = (size_t)(ci0 + ci) * kdim + k0 + 4 * l;
+    float4 a = make_float4(0.f, 0.f, 0.f, 0.f);
+    for (int sp = z; sp < splits; sp += 4 * kTeSlices) {
+        float4 q[4];
 #pragma unroll
-        for (int u = 0; u < 8; ++u) q[u] = sp + u < splits ? __ldcg(src + (size_t)(sp + u) * slice) : 0.f;
+        for (int u = 0; u < 4; ++u)
+            q[u] = sp + u * kTeSlices < splits ? __ldcg((const float4 *)(part + (size_t)(sp + u * kTeSlices) * slice + at))
+                                               : make_float4(0.f, 0.f, 0.f, 0.f);
 #pragma unroll
-        for (int u = 0; u < 8; ++u) v += q[u];
+        for (int u = 0; u < 4; ++u) { a.x += q[u].x; a.y += q[u].y; a.z += q[u].z; a.w += q[u].w; }
     }
-    dw[(size_t)(ci0 + ty) * kdim + k0 + tx] = vec3[co0 + tx] * v;
-    prod[ty][tx] = v * wv;
-    __syncthreads();
-    {
-        float d = prod[tx][ty];                         // warp ty adds the 32 input channels of row k0 + ty
+    red[tid] = a;
 #pragma unroll
-        for (int o = 16; o > 0; o >>= 1) d += __shfl_xor_sync(0xffffffffu, d, o);
-        if (tx == 0) dotpart[(size_t)blockIdx.y * kdim + k0 + ty] = d;
+    for (int h = kTeSlices / 2; h > 0; h /= 2) {
+        __syncthreads();
+        if (z < h) {
+            const float4 o = red[tid + h * 8 * kTeCi];
+            a.x += o.x; a.y += o.y; a.z += o.z; a.w += o.w;
+            red[tid] = a;
+        }
+    }
+    if (z == 0) {                                       // two warps: input channels 0-3 and 4-7
+        const uint2 wq = *(const uint2 *)(w + at);
+        const float4 s = *(const float4 *)(vec3 + co0 + 4 * l);
+        *(float4 *)(dw + at) = make_float4(s.x * a.x, s.y * a.y, s.z * a.z, s.w * a.w);
+        float d[4] = {a.x * unpack_h16((uint16_t)(wq.x & 0xFFFFu), f16), a.y * unpack_h16((uint16_t)(wq.x >> 16), f16),
+                      a.z * unpack_h16((uint16_t)(wq.y & 0xFFFFu), f16), a.w * unpack_h16((uint16_t)(wq.y >> 16), f16)};
+#pragma unroll
+        for (int e = 0; e < 4; ++e) {
+            d[e] += __shfl_xor_sync(0xffffffffu, d[e], 8);
+            d[e] += __shfl_xor_sync(0xffffffffu, d[e], 16);
+            if ((tid & 31) < 8) tile[tid / 32][4 * l + e] = d[e];
+        }
     }
     __syncthreads();
-    if (threadIdx.x == 0) {
+    if (tid < 32) dotpart[(size_t)blockIdx.y * kdim + k0 + tid] = tile[0][tid] + tile[1][tid];
+    __syncthreads();
+    if (tid == 0) {
         __threadfence();
         const unsigned int per_group = gridDim.y * (unsigned)(kdim / c_out);
         is_last = atomicAdd(&counters[co0 / 32], 1u) == per_group - 1;
@@ -144,22 +183,33 @@ __global__ void __launch_bounds__(1024) tconv_wgrad_epilogue_kernel(int c_in, in
     if (!is_last) return;
     __threadfence();
     // thread (tx = channel, ty = row group): rows of dotpart are (input-channel block, tap), then the slices of sum dZ
-    float d = 0.f, sum = 0.f;
+    constexpr int kTy = kTeThreads / 32;
+    const int tx = tid & 31, ty = tid >> 5;
     const int taps = kdim / c_out, rows = (int)gridDim.y * taps;
-    for (int r = ty; r < rows; r += 32) d += __ldcg(dotpart + (size_t)(r / taps) * kdim + (r % taps) * c_out + co0 + tx);
-    for (int sp = ty; sp < bsplits; sp += 128) {
+    float d = 0.f, sum = 0.f;
+    for (int r0 = ty; r0 < rows; r0 += 4 * kTy) {
         float q[4];
 #pragma unroll
-        for (int u = 0; u < 4; ++u) q[u] = sp + 32 * u < bsplits ? __ldcg(bsum + (size_t)(sp + 32 * u) * c_out + co0 + tx) : 0.f;
-        sum += (q[0] + q[1]) + (q[2] + q[3]);
+        for (int u = 0; u < 4; ++u) {
+            const int r = r0 + u * kTy;
+            q[u] = r < rows ? __ldcg(dotpart + (size_t)(r / taps) * kdim + (r % taps) * c_out + co0 + tx) : 0.f;
+        }
+        d += (q[0] + q[1]) + (q[2] + q[3]);
+    }
+    for (int sp = ty; sp < bsplits; sp += 8 * kTy) {
+        float q[8];
+#pragma unroll
+        for (int u = 0; u < 8; ++u) q[u] = sp + kTy * u < bsplits ? __ldcg(bsum + (size_t)(sp + kTy * u) * c_out + co0 + tx) : 0.f;
+        sum += ((q[0] + q[1]) + (q[2] + q[3])) + ((q[4] + q[5]) + (q[6] + q[7]));
     }
     tile[ty][tx] = d;
-    prod[ty][tx] = sum;
+    sums[ty][tx] = sum;
     __syncthreads();
     if (ty == 0) {
         const int co = co0 + tx;
         d = sum = 0.f;
-        for (int i = 0; i < 32; ++i) { d += tile[i][tx]; sum += prod[i][tx]; }
+#pragma unroll
+        for (int i = 0; i < kTy; ++i) { d += tile[i][tx]; sum += sums[i][tx]; }
         dbeta[co] = sum;
         if (db) db[co] = vec3[co] * sum;
         dgamma[co] = vec3[2 * c_out + co] * (d + sum * ((b ? b[co] : 0.0f) - mean[co]));
@@ -186,13 +236,21 @@ cudaError_t launch_tconv_wgrad_epilogue(int c_in, int c_out, int taps, const flo
                                         float *dgamma, float *dbeta, cudaStream_t st) {
     static PerDevice carve;
     prefer_max_shared_once(tconv_wgrad_epilogue_kernel, &carve);
-    return launch_pdl(tconv_wgrad_epilogue_kernel, dim3(taps * c_out / 32, c_in / 32), dim3(1024), 0, st, c_in, c_out,
+    return launch_pdl(tconv_wgrad_epilogue_kernel, dim3(taps * c_out / 32, c_in / kTeCi), dim3(kTeThreads), 0, st, c_in, c_out,
                       taps * c_out, part, splits, (const __nv_bfloat16 *)w, vec3, b, mean, bsum, bsplits, dotpart, counters,
                       dw, db, dgamma, dbeta, call_f16());
 }
 
 cudaError_t launch_tconv_rescale(int dtype, bool nhwc, long long count, int taps, int cig, int cog, const void *w,
                                  const float *s, void *w_out, cudaStream_t st) {
+    if (dtype == CONVBN_BF16 && nhwc && cog % 8 == 0 && count < (1LL << 31)) {
+        const uint32_t vecs = (uint32_t)(count / 8);
+        auto go = [&](auto kernel) {
+            return launch_pdl(kernel, dim3((vecs + 255) / 256), dim3(256), 0, st, vecs, (uint32_t)(taps * cog), (uint32_t)cig,
+                              (uint32_t)cog, (const uint4 *)w, s, (uint4 *)w_out);
+        };
+        return call_f16() ? go(tconv_rescale8_kernel<true>) : go(tconv_rescale8_kernel<false>);
+    }
     if (dtype == CONVBN_BF16 && call_f16())     // a half call runs as its bf16 twin
         return launch_pdl(tconv_rescale_kernel<__half>, dim3(grid_for(count)), dim3(256), 0, st, count, taps, cig, cog, nhwc,
                           (const __half *)w, s, (__half *)w_out);

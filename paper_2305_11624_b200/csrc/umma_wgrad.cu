@@ -34,10 +34,20 @@ struct WgradGemm {
     // Small-C_in ("stem") mode: tm_x is the 5-D window view of the packed input (one 64-wide slice per
     // filter row), tm_dz a 4-D map of dZ; a "pixel block" is a 4 x 16 patch of output pixels.
     int stem, stem_tiles_w, stem_tiles_h;
-    int no_ones;            // 1: no slice of ones (the packed stem input carries a constant-1 slot instead)
+    // Where the per-channel sums come from.  kSumNone: nowhere (the packed stem input carries a constant-1 slot instead).
+    // kSumSlice: a slice of ones behind the last slice of k; its accumulator rows are sum_p dZ[p][co].  kSumX: the X tile times
+    // ones, in an accumulator of its own, the tiles of channels taking turns at the stages (the sums of a transposed layer's dZ,
+    // which is the windowed operand there).  Ones times the dZ tile in the same way, instead of the slice, were measured where
+    // the number of slices is even and the slice costs another row of tiles: 2 to 6 % slower for most layers (3x3 256 at 23 x 21,
+    // N = 8 34.9 -> 36.7 us, ResNet-50, N = 32 2464 -> 2500), the products being a second full MMA per step.
+    int sums;
     int f16;                // 16-bit storage type: 0 bf16, 1 IEEE half
     int rows;               // 1: partials are [split][C_out][kdim], 0: [split][k][C_out]
 };
+
+enum { kSumNone, kSumSlice, kSumX };
+constexpr int kMaxTurns = 8;               // every turn leaves a row of sums for the adding kernel to read
+constexpr uint32_t kOnesBytes = 1024;      // one 8 x 128-byte group, read with all strides 0
 
 struct WgradSmemCtl {
     uint64_t full[kWMaxStages];
@@ -47,7 +57,8 @@ struct WgradSmemCtl {
     int abort_flag;
 };
 
-template <int BN>
+// X_SUMS: g.sums is kSumX (as a run-time branch in the issuing loop it cost the other layers 1 %).
+template <int BN, bool X_SUMS>
 __global__ void __launch_bounds__(kWThreads) umma_wgrad_kernel(const __grid_constant__ CUtensorMap tm_x,
                                                               const __grid_constant__ CUtensorMap tm_dz,
                                                               const WgradGemm g, float *__restrict__ partials,
@@ -57,7 +68,8 @@ __global__ void __launch_bounds__(kWThreads) umma_wgrad_kernel(const __grid_cons
     extern __shared__ uint8_t smem_raw[];
     constexpr uint32_t kABytes = 2 * kChunkBytes, kBBytes = (BN / 64) * kChunkBytes, kStageBytes = kABytes + kBBytes;
     uint8_t *tiles = (uint8_t *)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
-    WgradSmemCtl *ctl = (WgradSmemCtl *)(tiles + (size_t)g.stages * kStageBytes);
+    uint8_t *ones_tile = tiles + (size_t)g.stages * kStageBytes;
+    WgradSmemCtl *ctl = (WgradSmemCtl *)(ones_tile + kOnesBytes);
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int stages = g.stages;
     const int k0 = blockIdx.x * kWM;                    // first k row of this tile
@@ -65,11 +77,12 @@ __global__ void __launch_bounds__(kWThreads) umma_wgrad_kernel(const __grid_cons
     const long long p0 = (long long)blockIdx.z * g.per_split;
     const long long p1 = p0 + g.per_split < g.p ? p0 + g.per_split : g.p;
     const int num_kb = (int)((p1 - p0 + kWP - 1) / kWP);
-    // The list of 64-row slices is the K / 64 real ones followed by one slice of constant ones: its
-    // accumulator rows are sum_p dZ[p][co], the per-channel sums needed for dbeta (Table 2), for free.
     const int nch = g.kdim / 64, c_first = k0 / 64;
     const int a_chunks = nch - c_first >= 2 ? 2 : (nch - c_first >= 1 ? 1 : 0);   // slices loaded by TMA
-    const int ones_slot = g.no_ones ? -1 : ((c_first == nch) ? 0 : (c_first + 1 == nch ? 1 : -1));
+    const int ones_slot = g.sums != kSumSlice ? -1 : ((c_first == nch) ? 0 : (c_first + 1 == nch ? 1 : -1));
+    // kSumX: this CTA adds the stages turn, turn + turns, ... (the first kMaxTurns tiles do)
+    const int turn = (int)blockIdx.y, turns = min((int)gridDim.y, kMaxTurns);
+    const bool adds = X_SUMS && turn < turns;
     int b_chunks = (g.c_out - n0) / 64;
     if (b_chunks > BN / 64) b_chunks = BN / 64;
     volatile int *abort_flag = &ctl->abort_flag;
@@ -81,7 +94,7 @@ __global__ void __launch_bounds__(kWThreads) umma_wgrad_kernel(const __grid_cons
         fence_barrier_init();
     }
     if (warp == 1) {
-        tmem_alloc(&ctl->tmem_base, BN);
+        tmem_alloc(&ctl->tmem_base, X_SUMS ? 2 * BN : BN);
         tmem_relinquish();
     }
     // the tensor maps are kernel parameters, not data of an earlier kernel: fetch them before the wait
@@ -90,9 +103,13 @@ __global__ void __launch_bounds__(kWThreads) umma_wgrad_kernel(const __grid_cons
     // counters of the epilogue kernel that runs after this one start from zero
     if (counters && blockIdx.x == 0 && blockIdx.y == 0 && blockIdx.z == 0)
         for (int i = threadIdx.x; i < ncounters; i += kWThreads) counters[i] = 0u;
+    const uint32_t one2 = one_h16(g.f16) * 0x10001u;
+    if constexpr (X_SUMS) {
+        for (int i = threadIdx.x; i < (int)(kOnesBytes / 16); i += kWThreads) ((uint4 *)ones_tile)[i] = make_uint4(one2, one2, one2, one2);
+        fence_proxy_async_smem();
+    }
     if (ones_slot >= 0) {
         // 1.0 everywhere (invariant under the swizzle); TMA never writes this slice
-        const uint32_t one2 = one_h16(g.f16) * 0x10001u;
         const uint4 ones = make_uint4(one2, one2, one2, one2);
         for (int s = 0; s < stages; ++s) {
             uint4 *dst = (uint4 *)(tiles + (size_t)s * kStageBytes + (size_t)ones_slot * kChunkBytes);
@@ -202,6 +219,10 @@ __global__ void __launch_bounds__(kWThreads) umma_wgrad_kernel(const __grid_cons
             const uint32_t hi = smem_desc_hi_sw128(1024);
             const uint32_t tiles_lo = smem_desc_lo(smem_u32(tiles), kChunkBytes);
             uint32_t a_lo = tiles_lo;
+            const uint32_t ones_lo = smem_desc_lo(smem_u32(ones_tile), 0), ones_hi = smem_desc_hi_sw128(0);
+            const uint32_t idesc_x = idesc_h16_f32(kWM, 16, 1, 1, g.f16);
+            int wait_turn = adds ? turn : num_kb;
+            uint32_t adding = 0;
             ph = 0;
 #pragma unroll 4
             for (int kb = 0; kb < num_kb; ++kb) {
@@ -222,6 +243,15 @@ __global__ void __launch_bounds__(kWThreads) umma_wgrad_kernel(const __grid_cons
                 for (int k = 1; k < kWP / kWUmmaK; ++k)
                     umma_bf16_ss_halves<true>(tmem_base, a0 + (uint32_t)k * (kWUmmaK * 128 >> 4), hi,
                                               b0 + (uint32_t)k * (kWUmmaK * 128 >> 4), hi, idesc);
+                if (X_SUMS && wait_turn == 0) {
+                    wait_turn = turns;
+#pragma unroll 1
+                    for (uint32_t k = 0; k < kWP / kWUmmaK; ++k, adding = 1) {
+                        const uint32_t step = k * (kWUmmaK * 128 >> 4);
+                        umma_bf16_ss_sel(tmem_base + BN, a0 + step, hi, ones_lo, ones_hi, idesc_x, adding);
+                    }
+                }
+                if constexpr (X_SUMS) --wait_turn;
                 umma_commit(done);
             }
             if (ok) umma_commit(&ctl->tmem_full);
@@ -238,11 +268,18 @@ __global__ void __launch_bounds__(kWThreads) umma_wgrad_kernel(const __grid_cons
             tc_fence_after_sync();
             const int k = k0 + quarter * 32 + lane;
             const bool row_ok = k < g.kdim;
-            const bool sum_row = !g.no_ones && (k == g.kdim);   // first row of the ones slice
+            const bool sum_row = g.sums == kSumSlice && k == g.kdim;      // first row of the ones slice
             float *brow = bsum + (size_t)blockIdx.z * g.c_out + n0;
             float *orow = g.blockdiag
                               ? partials + (((size_t)blockIdx.z * gridDim.y + blockIdx.y) * g.kdim + (row_ok ? k : 0)) * 64
                               : partials + ((size_t)blockIdx.z * g.kdim + (row_ok ? k : 0)) * g.c_out + n0;
+            if (adds) {                                    // a row of the accumulator is a k, its columns are the same
+                uint32_t v[16];
+                tmem_ld_32x16(tmem_base + BN + ((uint32_t)(quarter * 32) << 16), v);
+                tmem_ld_wait();
+                // (0 where this CTA's turn never came)
+                if (row_ok) bsum[((size_t)blockIdx.z * turns + turn) * g.kdim + k] = turn < num_kb ? __uint_as_float(v[0]) : 0.f;
+            }
 #pragma unroll 1
             for (int c0 = 0; c0 < BN; c0 += 32) {
                 if (n0 + c0 >= g.c_out) break;
@@ -268,7 +305,7 @@ __global__ void __launch_bounds__(kWThreads) umma_wgrad_kernel(const __grid_cons
     }
     tc_fence_before_sync();
     __syncthreads();
-    if (warp == 1) tmem_dealloc(tmem_base, BN);
+    if (warp == 1) tmem_dealloc(tmem_base, X_SUMS ? 2 * BN : BN);
 }
 
 bool grouped_bd_eligible(const Problem &pb) {
@@ -293,10 +330,15 @@ bool umma_wgrad_eligible(const Problem &pb) {
 static int wgrad_bn(const Problem &pb) { return pb.c_out >= 128 ? 128 : 64; }
 static int stem_wgrad_bn(const Problem &pb) { return pb.c_out >= 256 ? 256 : wgrad_bn(pb); }
 
-// Output tiles of bn columns (k rows of the ones slice included).
-static long long wgrad_tiles(const Problem &pb, int bn) {
-    const long long kd = pb.groups > 1 ? (long long)pb.kh * pb.kw * 64 : pb.kdim;
-    return (kd / 64 + 1 + 1) / 2 * ((pb.c_out + bn - 1) / bn);
+// Output tiles of bn columns.
+static long long wgrad_k_slices(const Problem &pb) { return (pb.groups > 1 ? (long long)pb.kh * pb.kw * 64 : pb.kdim) / 64; }
+static long long wgrad_tiles(const Problem &pb, int bn, bool ones_slice) {
+    return (wgrad_k_slices(pb) + (ones_slice ? 2 : 1)) / 2 * ((pb.c_out + bn - 1) / bn);
+}
+
+int umma_wgrad_x_sum_rows(const Problem &pb) {
+    const int n = (pb.c_out + wgrad_bn(pb) - 1) / wgrad_bn(pb);
+    return n < kMaxTurns ? n : kMaxTurns;
 }
 
 // The slice count minimises  rounds over the resident slots x (pixels per slice + a fixed cost per
@@ -320,7 +362,7 @@ static UmmaWgradPlan wgrad_slices(const Problem &pb, long long tiles, long long 
     return pl;
 }
 
-UmmaWgradPlan umma_wgrad_plan(const Problem &pb) {
+UmmaWgradPlan umma_wgrad_plan(const Problem &pb, WgradSums sums) {
     // Resident CTAs: two per SM (the stage rings are sized for it, launch_w): one's partial tile leaves while the other
     // multiplies.  A deeper ring for one CTA gains nothing.
     // Few tiles mean many slices, and where those are short the partial tensors weigh more than what a second CTA hides: up to
@@ -329,7 +371,7 @@ UmmaWgradPlan umma_wgrad_plan(const Problem &pb) {
     // 128 -> 512 at 28 x 28, N = 256 58.3 -> 73.6).  Not where output rows are shorter than four pixels: the boxes of X then
     // arrive pixel by pixel and a second CTA hides that (29173 rows, 1024 -> 64: 44.5 and 27.4 us; 2 x 2 about even; from
     // 4 x 4 on one CTA is the faster).
-    const long long tiles = wgrad_tiles(pb, pb.groups > 1 ? 64 : wgrad_bn(pb)), sms = device_sm_count();
+    const long long tiles = wgrad_tiles(pb, pb.groups > 1 ? 64 : wgrad_bn(pb), sums == WgradSums::kDz), sms = device_sm_count();
     return wgrad_slices(pb, tiles, sms * (tiles <= 24 && pb.p * tiles <= 2048 * sms && pb.w_out >= 4 ? 1 : 2));
 }
 
@@ -337,12 +379,12 @@ UmmaWgradPlan umma_wgrad_plan(const Problem &pb) {
 // with an SM of its own, which makes fewer slices of wide layers (3x3 768 -> 384 at 13 x 13, N = 12: 10 MiB, above 30).
 UmmaWgradPlan umma_wgrad_plan_bounded(const Problem &pb) {
     const int bn = pb.groups > 1 ? 64 : (pb.c_out >= 256 ? 256 : wgrad_bn(pb));
-    return wgrad_slices(pb, wgrad_tiles(pb, bn), (long long)device_sm_count() * (bn == 256 ? 1 : 2));
+    return wgrad_slices(pb, wgrad_tiles(pb, bn, true), (long long)device_sm_count() * (bn == 256 ? 1 : 2));
 }
 
 int wgrad_kmajor_rows(const Problem &pb) { return (pb.kdim + 1) / 2; }
 
-template <int BN>
+template <int BN, bool X_SUMS = false>
 static cudaError_t launch_w(const CUtensorMap &tx, const CUtensorMap &tdz, WgradGemm g, const UmmaWgradPlan &pl,
                             const Problem &pb, float *partials, float *bsum, int *err, cudaStream_t st,
                             unsigned int *counters = nullptr, int ncounters = 0) {
@@ -351,28 +393,30 @@ static cudaError_t launch_w(const CUtensorMap &tx, const CUtensorMap &tdz, Wgrad
     const long long max_kb = (pl.per_split + kWP - 1) / kWP;
     if (stages > max_kb) stages = (int)max_kb;
     g.stages = stages;
-    size_t smem = stages * stage + 1024 + sizeof(WgradSmemCtl);
-    const size_t floor_smem = (size_t)(228 * 1024) / (512 / BN + 1) + 1024;
+    size_t smem = stages * stage + 1024 + kOnesBytes + sizeof(WgradSmemCtl);
+    const int columns = X_SUMS ? 2 * BN : BN;      // no more CTAs than there is tensor memory for
+    const size_t floor_smem = (size_t)(228 * 1024) / (512 / columns + 1) + 1024;
     if (smem < floor_smem) smem = floor_smem;
     static PerDevice attr_done;
-    if (cudaError_t e = max_dynamic_smem_once(umma_wgrad_kernel<BN>, 210 * 1024, &attr_done); e != cudaSuccess) return e;
+    if (cudaError_t e = max_dynamic_smem_once(umma_wgrad_kernel<BN, X_SUMS>, 210 * 1024, &attr_done); e != cudaSuccess) return e;
     static PerDevice carve;
-    prefer_max_shared_once(umma_wgrad_kernel<BN>, &carve);
-    dim3 grid((unsigned)((g.kdim / 64 + (g.no_ones ? 1 : 2)) / 2), (unsigned)((pb.c_out + BN - 1) / BN),
+    prefer_max_shared_once(umma_wgrad_kernel<BN, X_SUMS>, &carve);
+    dim3 grid((unsigned)((g.kdim / 64 + (g.sums == kSumSlice ? 2 : 1)) / 2), (unsigned)((pb.c_out + BN - 1) / BN),
               (unsigned)pl.splits);
-    return launch_pdl(umma_wgrad_kernel<BN>, grid, dim3(kWThreads), smem, st, tx, tdz, g, partials, bsum, counters,
+    return launch_pdl(umma_wgrad_kernel<BN, X_SUMS>, grid, dim3(kWThreads), smem, st, tx, tdz, g, partials, bsum, counters,
                       ncounters, err);
 }
 
 cudaError_t launch_umma_wgrad(const Problem &pb, const UmmaWgradPlan &pl, const void *dz, const void *x,
-                              float *partials, float *bsum, cudaStream_t st, unsigned int *counters, int ncounters) {
+                              float *partials, float *bsum, cudaStream_t st, unsigned int *counters, int ncounters, WgradSums sums) {
     WgradGemm g;
     g.ho = pb.h_out; g.wo = pb.w_out; g.c_in = pb.c_in; g.c_out = pb.c_out; g.taps_w = pb.kw;
     g.lower_h = -pb.pad_h; g.lower_w = -pb.pad_w; g.stride_h = pb.stride_h; g.stride_w = pb.stride_w;
     g.dil_h = pb.dil_h; g.dil_w = pb.dil_w; g.kdim = pb.kdim; g.p = pb.p; g.per_split = pl.per_split; g.stages = 1;
     g.blockdiag = pb.groups > 1 ? 1 : 0;
     g.rows = g.blockdiag ? 0 : 1;
-    g.stem = 0; g.stem_tiles_w = g.stem_tiles_h = 1; g.no_ones = 0; g.f16 = call_f16();
+    g.stem = 0; g.stem_tiles_w = g.stem_tiles_h = 1; g.f16 = call_f16();
+    g.sums = sums == WgradSums::kX ? kSumX : (sums == WgradSums::kNone ? kSumNone : kSumSlice);
     if (g.blockdiag) { g.c_in = 64; g.kdim = pb.kh * pb.kw * 64; }
     const int upper_h = g.lower_h + (pb.h_out - 1) * pb.stride_h - (pb.h_in - 1);
     const int upper_w = g.lower_w + (pb.w_out - 1) * pb.stride_w - (pb.w_in - 1);
@@ -390,6 +434,9 @@ cudaError_t launch_umma_wgrad(const Problem &pb, const UmmaWgradPlan &pl, const 
     int *err = nullptr;
     cudaError_t e = error_word_address(&err);
     if (e != cudaSuccess) return e;
+    if (g.sums == kSumX)
+        return bn == 64 ? launch_w<64, true>(tx, tdz, g, pl, pb, partials, bsum, err, st, counters, ncounters)
+                        : launch_w<128, true>(tx, tdz, g, pl, pb, partials, bsum, err, st, counters, ncounters);
     if (bn == 64) return launch_w<64>(tx, tdz, g, pl, pb, partials, bsum, err, st, counters, ncounters);
     return launch_w<128>(tx, tdz, g, pl, pb, partials, bsum, err, st, counters, ncounters);
 }
@@ -683,7 +730,7 @@ cudaError_t launch_stem_wgrad(const Problem &pb, const UmmaWgradPlan &pl, const 
     g.kdim = krows * 64;
     g.rows = 0;
     g.stem = 1; g.stem_tiles_w = (pb.w_out + 15) / 16; g.stem_tiles_h = (pb.h_out + 3) / 4;
-    g.no_ones = stem_ones_in_pack(pb) ? 1 : 0;
+    g.sums = stem_ones_in_pack(pb) ? kSumNone : kSumSlice;
     g.f16 = call_f16();
     g.p = (long long)pb.n * g.stem_tiles_h * g.stem_tiles_w * kWP;
     g.per_split = pl.per_split; g.stages = 1; g.blockdiag = 0;
