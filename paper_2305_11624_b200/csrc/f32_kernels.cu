@@ -157,7 +157,6 @@ __global__ void __launch_bounds__(kFThreads, K == 1 ? 8 : (S == 1 ? 5 : 4)) f32_
     constexpr int OCT = S == 1 ? 4 * R : R;
     __shared__ float scale_s[OCT], shift_s[OCT];
     pdl_wait();
-    pdl_launch_dependents();
     const int oc0 = blockIdx.y * OCT;
     if (threadIdx.x < OCT) {
         const int o = oc0 + threadIdx.x;
@@ -360,7 +359,6 @@ __global__ void __cluster_dims__(kFCluster, 1, 1) __launch_bounds__(kFThreads, 4
                                                                                           int oc_tiles) {
     extern __shared__ __align__(16) float f32_smem[];
     pdl_wait();
-    pdl_launch_dependents();
     const int b = (int)blockIdx.x;
     if (b < nw) {
         const int cl = b / kFCluster / g.groups;
