@@ -72,16 +72,15 @@ class _Layer:
         self.out_elems = n * c_out * self.blk.h_out * self.blk.w_out
         self.in_elems = n * c_in * hw[0] * hw[1]
 
-    def forward(self, x, add=None, relu=False):
+    def forward(self, x, add=None, relu=False, saved=None, scratch=None):
         """The block's output, or max(output + add, 0): in Tune mode the addend and the ReLU are part of the block's own
-        kernel, otherwise they are passes of their own."""
+        kernel, otherwise they are passes of their own.  saved, scratch (Tune mode): addresses of saved_bytes, which the
+        caller keeps for the backward pass, and of fwd_bytes for this call."""
         b = self.blk
         b.x = x
         z = torch.empty(self.out_elems, dtype=b.tdtype, device=b.device)
         if self.mode == "tune":
-            b.saved = torch.empty(self.saved_bytes, dtype=torch.uint8, device=b.device)
-            ws = torch.empty(self.fwd_bytes, dtype=torch.uint8, device=b.device)
-            C.convbn_tune_fwd_glue(b.desc, x, b.w, b.b, b.gamma, b.beta, b.mu_hat, b.var_hat, z, b.saved, add, relu, ws,
+            C.convbn_tune_fwd_glue(b.desc, x, b.w, b.b, b.gamma, b.beta, b.mu_hat, b.var_hat, z, saved, add, relu, scratch,
                                    self.fwd_bytes)
             return z
         b.z = z
@@ -97,21 +96,20 @@ class _Layer:
             C.convbn_relu(z, z)
         return z
 
-    def backward(self, dz, held=None, add=None, relu_mask=False):
+    def backward(self, dz, held=None, add=None, relu_mask=False, saved=None, scratch=None):
         """Gradient with respect to the block's input, plus `add`, and with `relu_mask` zero where the input (the output
         of a ReLU) is not positive; drops what the block kept for it.  With `held` (a list, Tune mode) the
-        parameter-gradient pass stays on the library's side stream: what it still reads (dZ, X, the saved vectors, the
-        scratch) is parked in `held` until the caller has joined."""
+        parameter-gradient pass stays on the library's side stream: what it still reads of the tensors allocated here (dZ, X)
+        is parked in `held` until the caller has joined.  saved, scratch (Tune mode): addresses of the forward pass's
+        vectors and of bwd_bytes, both in use until the pass is joined."""
         b = self.blk
         dx = torch.empty(self.in_elems, dtype=b.tdtype, device=b.device)
         x, b.x = b.x, None
         if self.mode == "tune":
-            ws = torch.empty(self.bwd_bytes, dtype=torch.uint8, device=b.device)
-            C.convbn_tune_bwd_glue(b.desc, dz, x, b.w, b.b, b.mu_hat, b.saved, dx, b.dw, b.db, b.dgamma, b.dbeta, add,
-                                   relu_mask, held is not None, ws, self.bwd_bytes)
+            C.convbn_tune_bwd_glue(b.desc, dz, x, b.w, b.b, b.mu_hat, saved, dx, b.dw, b.db, b.dgamma, b.dbeta, add,
+                                   relu_mask, held is not None, scratch, self.bwd_bytes)
             if held is not None:
-                held.append((ws, b.saved, x, dz))
-            b.saved = None
+                held.append((x, dz))
             return dx
         b.dz, b.dx, b.x = dz, dx, x
         if self.mode == "eval":
@@ -125,6 +123,10 @@ class _Layer:
         if relu_mask:
             C.convbn_relu_bwd(dx, x, dx)
         return dx
+
+
+def _aligned(n):
+    return (n + 255) // 256 * 256
 
 
 class BackboneReplay:
@@ -156,6 +158,25 @@ class BackboneReplay:
         self.first = plan[0]
         self.layers = ([self.stem] if self.stem else []) + [l for blk in self.blocks for l in blk if l is not None]
         self.flops = sum(3 * l.blk.flops_per_phase() for l in self.layers)
+        if mode == "tune":
+            # The vectors kept from forward to backward lie in one buffer per iteration, the forward calls share one scratch
+            # (one after the other on a stream), and a bottleneck's backward calls share one: with deferred gradients each
+            # has its part until the join, otherwise they take turns.  An allocation per call (265 of an iteration) took
+            # 1.8 us of host time each.
+            self.saved_at, at = {}, 0
+            for l in self.layers:
+                self.saved_at[l], at = at, at + _aligned(l.saved_bytes)
+            self.saved_total = at
+            self.fwd_scratch = max(l.fwd_bytes for l in self.layers)
+            self.bwd_at, self.bwd_total = [], []
+            for blk in self.blocks:
+                off, at = [], 0
+                for l in blk:
+                    off.append(at)
+                    if l is not None and async_param_grads:
+                        at += _aligned(l.bwd_bytes)
+                self.bwd_at.append(off)
+                self.bwd_total.append(at or max(l.bwd_bytes for l in blk if l is not None))
 
     # ---- one iteration ---------------------------------------------------------------------------------
     def make_inputs(self, seed: int = 1):
@@ -175,19 +196,29 @@ class BackboneReplay:
         """One training iteration.  `keep` (a dict) receives the network output, the input gradient and copies of
         every ReLU output (whose signs are the decisions a comparison has to share)."""
         relu_outs = []
+        tune = self.mode == "tune"
+        fwd = {}
+        if tune:
+            raw = lambda n: torch.empty(n, dtype=torch.uint8, device=self.device)
+            saved, scratch = raw(self.saved_total), raw(self.fwd_scratch)
+            base, at = saved.data_ptr(), scratch.data_ptr()
+            fwd = {l: (base + o, at) for l, o in self.saved_at.items()}
+        none = (None, None)
         if self.stem:
-            s = self.stem.forward(ins["image"], relu=True)
+            s = self.stem.forward(ins["image"], None, True, *fwd.get(self.stem, none))
         x = ins["x"]
         for c1, c2, c3, ds in self.blocks:
-            a = c1.forward(x, relu=True)
-            b = c2.forward(a, relu=True)
-            c = c3.forward(b, add=ds.forward(x) if ds is not None else x, relu=True)    # out = relu(c3(b) + identity)
+            a = c1.forward(x, None, True, *fwd.get(c1, none))
+            b = c2.forward(a, None, True, *fwd.get(c2, none))
+            # out = relu(c3(b) + identity)
+            c = c3.forward(b, ds.forward(x, None, False, *fwd.get(ds, none)) if ds is not None else x, True, *fwd.get(c3, none))
             relu_outs.append((x, a, b, c))
             if keep is not None:
                 keep.setdefault("relu_outputs", []).append((a.clone(), b.clone(), c.clone()))
             x = c
         if keep is not None:
             keep["out"] = x.clone()
+        scratch = None
         g = torch.empty_like(ins["g"])
         C.convbn_relu_bwd(ins["g"], x, g)                      # through the last block's ReLU
         del x, a, b, c
@@ -197,12 +228,18 @@ class BackboneReplay:
         for i in range(len(self.blocks) - 1, -1, -1):
             c1, c2, c3, ds = self.blocks[i]
             relu_outs.pop()
-            gb = c3.backward(g, held, relu_mask=True)
-            ga = c2.backward(gb, held, relu_mask=True)
+            at = none * 2
+            if tune:
+                scratch = raw(self.bwd_total[i])
+                base = scratch.data_ptr()
+                at = [base + o for o in self.bwd_at[i]]
+            kept = lambda l: fwd.get(l, none)[0]
+            gb = c3.backward(g, held, None, True, kept(c3), at[2])
+            ga = c2.backward(gb, held, None, True, kept(c2), at[1])
             del gb
-            gs = ds.backward(g, held) if ds is not None else g
+            gs = ds.backward(g, held, None, False, kept(ds), at[3]) if ds is not None else g
             # the two branches meet; the input of every block but the first is the ReLU output of the block below
-            g = c1.backward(ga, held, add=gs, relu_mask=i > 0)
+            g = c1.backward(ga, held, gs, i > 0, kept(c1), at[0])
             del ga, gs
             if held is not None:
                 C.convbn_tune_bwd_join()
@@ -212,7 +249,8 @@ class BackboneReplay:
         if self.stem:
             gs = torch.empty_like(ins["g_stem"])
             C.convbn_relu_bwd(ins["g_stem"], s, gs)
-            gi = self.stem.backward(gs)
+            scratch = raw(self.stem.bwd_bytes) if tune else None
+            gi = self.stem.backward(gs, None, None, False, fwd.get(self.stem, none)[0], scratch.data_ptr() if tune else None)
             if keep is not None:
                 keep["d_image"] = gi.clone()
         return g

@@ -1,5 +1,6 @@
 """Compile ``csrc/*.cu`` for sm_100a into ``paper_2305_11624_b200/libconvbn.so`` with nvcc.
 
+``csrc/binding.cpp``, the Python entry to the calls of a training step, becomes ``_binding.so`` beside it (g++).
 Sources are compiled in parallel to objects under ``_build/`` and linked with the static CUDA
 runtime; the driver API (tensor-map encoding) is resolved at run time through the runtime's
 entry-point query, so the library loads on a machine without a GPU driver.
@@ -7,12 +8,15 @@ entry-point query, so the library loads on a machine without a GPU driver.
 import os
 import subprocess
 import sys
+import sysconfig
 from concurrent.futures import ThreadPoolExecutor
 
 _HERE = os.path.dirname(os.path.abspath(__file__))
 CSRC = os.path.join(_HERE, "csrc")
 BUILD_DIR = os.path.join(_HERE, "_build")
 LIBRARY = os.path.join(_HERE, "libconvbn.so")
+BINDING = os.path.join(_HERE, "_binding.so")
+CXX = os.environ.get("CXX", "g++")
 NVCC = os.environ.get("NVCC", "/usr/local/cuda/bin/nvcc")
 ARCH = ["-gencode", "arch=compute_100a,code=sm_100a"]
 CFLAGS = ["-O3", "-std=c++17", "-lineinfo", "-Xcompiler", "-fPIC", "-Xptxas", "-v",
@@ -44,9 +48,18 @@ def _compile(src: str, verbose: bool) -> str:
     return obj
 
 
+def _build_binding():
+    tmp = BINDING + ".tmp.%d" % os.getpid()
+    cmd = [CXX, "-O2", "-std=c++17", "-shared", "-fPIC", "-fvisibility=hidden", "-Wall",
+           "-I" + sysconfig.get_paths()["include"], os.path.join(CSRC, "binding.cpp"), "-o", tmp,
+           "-L" + _HERE, "-l:libconvbn.so", "-Wl,-rpath,$ORIGIN"]
+    subprocess.run(cmd, check=True)
+    os.replace(tmp, BINDING)
+
+
 def build(force: bool = False, verbose: bool = False) -> str:
     """Build the library if missing or older than any source; return its path."""
-    if not force and os.path.exists(LIBRARY) and os.path.getmtime(LIBRARY) >= _deps_mtime():
+    if not force and all(os.path.exists(f) and os.path.getmtime(f) >= _deps_mtime() for f in (LIBRARY, BINDING)):
         return LIBRARY
     os.makedirs(BUILD_DIR, exist_ok=True)
     with ThreadPoolExecutor(max_workers=8) as ex:
@@ -55,6 +68,7 @@ def build(force: bool = False, verbose: bool = False) -> str:
     cmd = [NVCC] + ARCH + ["-shared", "-cudart", "static", "-o", tmp] + objs
     subprocess.run(cmd, check=True)
     os.replace(tmp, LIBRARY)
+    _build_binding()
     return LIBRARY
 
 

@@ -1,4 +1,5 @@
-"""Thin ctypes binding of ``libconvbn.so`` (declared in ``include/convbn.h``).
+"""Thin binding of ``libconvbn.so`` (declared in ``include/convbn.h``): ctypes, and ``_binding.so`` for the calls that a
+training step makes.
 
 Argument marshalling only: every function has the name and argument order of its C entry point,
 takes torch CUDA tensors (or raw integer device addresses, or None for NULL) and returns nothing;
@@ -6,6 +7,7 @@ a non-zero status raises ``ConvBNError``.  There is no fallback: if the compiled
 missing, importing succeeds but the first call raises.
 """
 import ctypes
+import importlib.util
 import os
 from typing import Optional
 
@@ -54,18 +56,13 @@ _lib = None
 
 
 def _signatures():
-    """argtypes of the entry points that take pointers: ctypes then converts plain integers itself, without an object per
+    """argtypes of entry points that take pointers: ctypes then converts plain integers itself, without an object per
     argument (d: descriptor, p: pointer or stream, z: size, i: int, q: long long, f: double)."""
     kinds = {"d": ctypes.POINTER(Desc), "p": ctypes.c_void_p, "z": ctypes.c_size_t, "i": ctypes.c_int,
              "q": ctypes.c_longlong, "f": ctypes.c_double}
     table = {
-        "convbn_tune_fwd": "dppppppppppzp", "convbn_tune_bwd_data": "dpppppzp", "convbn_tune_bwd_weight": "dppppppppppp" "zp",
-        "convbn_tune_bwd": "dppppppppppppzp", "convbn_tune_bwd_begin": "dppppppppppppzp", "convbn_tune_bwd_join": "p",
-        "convbn_tune_fwd_glue": "dppppppppppipzp", "convbn_tune_bwd_glue": "dppppppppppppiipzp",
-        "convbn_tconv_tune_fwd": "dppppppppppzp", "convbn_tconv_tune_bwd": "dppppppppppppzp",
-        "convbn_tune_bwd_weight_noalloc": "dppppppppppp", "convbn_eval_fwd": "dppppppppppzp",
-        "convbn_eval_bwd": "dpppppppppppppzp", "convbn_deploy_prepare": "dppppppppp", "convbn_deploy_fwd": "dpppppzp",
-        "convbn_deploy_bwd": "dpppppppzp", "convbn_relu": "ippqp", "convbn_add_relu": "ipppqp", "convbn_relu_bwd": "ipppqp",
+        "convbn_tune_bwd_weight_noalloc": "dppppppppppp", "convbn_deploy_prepare": "dppppppppp",
+        "convbn_relu": "ippqp", "convbn_add_relu": "ipppqp", "convbn_relu_bwd": "ipppqp",
         "convbn_add": "ipppqp", "convbn_workspace_bytes": "di", "convbn_saved_bytes": "di", "convbn_check": "p",
     }
     return {name: [kinds[k] for k in sig] for name, sig in table.items()}
@@ -90,6 +87,31 @@ def lib():
             getattr(L, name).argtypes = types
         _lib = L
     return _lib
+
+
+_native = None
+
+
+def _calls():
+    """The entry points of csrc/binding.cpp."""
+    global _native
+    if _native is None:
+        lib()
+        path = os.path.join(_HERE, "_binding.so")
+        if not os.path.exists(path):
+            raise OSError("%s not found: run `python -m paper_2305_11624_b200.build`" % path)
+        spec = importlib.util.spec_from_file_location(__package__ + "._binding", path)
+        module = importlib.util.module_from_spec(spec)
+        spec.loader.exec_module(module)
+        _native = module
+    return _native
+
+
+def _desc(desc):
+    """A descriptor given as ctypes.byref(d) or ctypes.pointer(d)."""
+    if hasattr(desc, "_obj"):
+        return desc._obj
+    return desc.contents if isinstance(desc, ctypes.POINTER(Desc)) else desc
 
 
 def _ptr(t):
@@ -160,70 +182,81 @@ def convbn_workspace_bytes(desc: Desc, phase: int) -> int:
 
 def convbn_tune_fwd(desc, x, w, b, gamma, beta, run_mean, run_var, z, saved, workspace=None,
                     workspace_bytes: Optional[int] = None, stream=None):
-    wb = _nbytes(workspace) if workspace_bytes is None else workspace_bytes
-    _raise(lib().convbn_tune_fwd(desc, _ptr(x), _ptr(w), _ptr(b), _ptr(gamma),
-                                 _ptr(beta), _ptr(run_mean), _ptr(run_var), _ptr(z), _ptr(saved),
-                                 _ptr(workspace), wb, _stream(stream)),
-           "convbn_tune_fwd")
+    if type(desc) is not Desc:
+        desc = _desc(desc)
+    status = (_native or _calls()).convbn_tune_fwd(desc, x, w, b, gamma, beta, run_mean, run_var, z, saved,
+                                                   workspace, workspace_bytes, stream)
+    if status:
+        _raise(status, "convbn_tune_fwd")
 
 
 def convbn_tune_bwd_data(desc, dz, w, saved, dx, workspace=None,
                          workspace_bytes: Optional[int] = None, stream=None):
-    wb = _nbytes(workspace) if workspace_bytes is None else workspace_bytes
-    _raise(lib().convbn_tune_bwd_data(desc, _ptr(dz), _ptr(w), _ptr(saved), _ptr(dx),
-                                      _ptr(workspace), wb, _stream(stream)),
-           "convbn_tune_bwd_data")
+    if type(desc) is not Desc:
+        desc = _desc(desc)
+    status = (_native or _calls()).convbn_tune_bwd_data(desc, dz, w, saved, dx, workspace, workspace_bytes, stream)
+    if status:
+        _raise(status, "convbn_tune_bwd_data")
 
 
 def convbn_tune_bwd_weight(desc, dz, x, w, b, run_mean, saved, dw, db, dgamma, dbeta,
                            workspace=None, workspace_bytes: Optional[int] = None, stream=None):
-    wb = _nbytes(workspace) if workspace_bytes is None else workspace_bytes
-    _raise(lib().convbn_tune_bwd_weight(desc, _ptr(dz), _ptr(x), _ptr(w), _ptr(b),
-                                        _ptr(run_mean), _ptr(saved), _ptr(dw), _ptr(db),
-                                        _ptr(dgamma), _ptr(dbeta), _ptr(workspace),
-                                        wb, _stream(stream)),
-           "convbn_tune_bwd_weight")
+    if type(desc) is not Desc:
+        desc = _desc(desc)
+    status = (_native or _calls()).convbn_tune_bwd_weight(desc, dz, x, w, b, run_mean, saved, dw, db, dgamma, dbeta,
+                                                          workspace, workspace_bytes, stream)
+    if status:
+        _raise(status, "convbn_tune_bwd_weight")
 
 
 def convbn_tune_bwd(desc, dz, x, w, b, run_mean, saved, dx, dw, db, dgamma, dbeta, workspace=None,
                     workspace_bytes: Optional[int] = None, stream=None):
-    wb = _nbytes(workspace) if workspace_bytes is None else workspace_bytes
-    _raise(lib().convbn_tune_bwd(desc, _ptr(dz), _ptr(x), _ptr(w), _ptr(b), _ptr(run_mean),
-                                 _ptr(saved), _ptr(dx), _ptr(dw), _ptr(db), _ptr(dgamma), _ptr(dbeta),
-                                 _ptr(workspace), wb, _stream(stream)),
-           "convbn_tune_bwd")
+    if type(desc) is not Desc:
+        desc = _desc(desc)
+    status = (_native or _calls()).convbn_tune_bwd(desc, dz, x, w, b, run_mean, saved, dx, dw, db, dgamma, dbeta,
+                                                   workspace, workspace_bytes, stream)
+    if status:
+        _raise(status, "convbn_tune_bwd")
 
 
 def convbn_tune_bwd_begin(desc, dz, x, w, b, run_mean, saved, dx, dw, db, dgamma, dbeta, workspace=None,
                           workspace_bytes: Optional[int] = None, stream=None):
     """convbn_tune_bwd that returns with the parameter-gradient pass still running on the library's side lane."""
-    wb = _nbytes(workspace) if workspace_bytes is None else workspace_bytes
-    _raise(lib().convbn_tune_bwd_begin(desc, _ptr(dz), _ptr(x), _ptr(w), _ptr(b), _ptr(run_mean),
-                                       _ptr(saved), _ptr(dx), _ptr(dw), _ptr(db), _ptr(dgamma), _ptr(dbeta),
-                                       _ptr(workspace), wb, _stream(stream)), "convbn_tune_bwd_begin")
+    if type(desc) is not Desc:
+        desc = _desc(desc)
+    status = (_native or _calls()).convbn_tune_bwd_begin(desc, dz, x, w, b, run_mean, saved, dx, dw, db, dgamma,
+                                                         dbeta, workspace, workspace_bytes, stream)
+    if status:
+        _raise(status, "convbn_tune_bwd_begin")
 
 
 def convbn_tune_bwd_join(stream=None) -> None:
     """Make `stream` wait for every parameter-gradient pass begun by this thread on the current device."""
-    _raise(lib().convbn_tune_bwd_join(_stream(stream)), "convbn_tune_bwd_join")
+    status = (_native or _calls()).convbn_tune_bwd_join(stream)
+    if status:
+        _raise(status, "convbn_tune_bwd_join")
 
 
 def convbn_tune_fwd_glue(desc, x, w, b, gamma, beta, run_mean, run_var, z, saved, add, relu, workspace=None,
                          workspace_bytes: Optional[int] = None, stream=None):
     """convbn_tune_fwd with the addend and the ReLU of a residual network in its epilogue."""
-    wb = _nbytes(workspace) if workspace_bytes is None else workspace_bytes
-    _raise(lib().convbn_tune_fwd_glue(desc, _ptr(x), _ptr(w), _ptr(b), _ptr(gamma), _ptr(beta), _ptr(run_mean),
-                                      _ptr(run_var), _ptr(z), _ptr(saved), _ptr(add), 1 if relu else 0, _ptr(workspace), wb,
-                                      _stream(stream)), "convbn_tune_fwd_glue")
+    if type(desc) is not Desc:
+        desc = _desc(desc)
+    status = (_native or _calls()).convbn_tune_fwd_glue(desc, x, w, b, gamma, beta, run_mean, run_var, z, saved, add,
+                                                        1 if relu else 0, workspace, workspace_bytes, stream)
+    if status:
+        _raise(status, "convbn_tune_fwd_glue")
 
 
 def convbn_tune_bwd_glue(desc, dz, x, w, b, run_mean, saved, dx, dw, db, dgamma, dbeta, add, relu_mask, begin,
                          workspace=None, workspace_bytes: Optional[int] = None, stream=None):
     """convbn_tune_bwd (or, with `begin`, convbn_tune_bwd_begin) with dx += add and the mask x > 0 in its epilogue."""
-    wb = _nbytes(workspace) if workspace_bytes is None else workspace_bytes
-    _raise(lib().convbn_tune_bwd_glue(desc, _ptr(dz), _ptr(x), _ptr(w), _ptr(b), _ptr(run_mean), _ptr(saved), _ptr(dx),
-                                      _ptr(dw), _ptr(db), _ptr(dgamma), _ptr(dbeta), _ptr(add), 1 if relu_mask else 0,
-                                      1 if begin else 0, _ptr(workspace), wb, _stream(stream)), "convbn_tune_bwd_glue")
+    if type(desc) is not Desc:
+        desc = _desc(desc)
+    status = (_native or _calls()).convbn_tune_bwd_glue(desc, dz, x, w, b, run_mean, saved, dx, dw, db, dgamma,
+                                                        dbeta, add, 1 if relu_mask else 0, 1 if begin else 0, workspace, workspace_bytes, stream)
+    if status:
+        _raise(status, "convbn_tune_bwd_glue")
 
 
 def convbn_tconv_out_shape(desc):
@@ -240,18 +273,22 @@ def convbn_tconv_workspace_bytes(desc) -> int:
 
 def convbn_tconv_tune_fwd(desc, x, w, b, gamma, beta, run_mean, run_var, z, saved, workspace=None,
                           workspace_bytes: Optional[int] = None, stream=None):
-    wb = _nbytes(workspace) if workspace_bytes is None else workspace_bytes
-    _raise(lib().convbn_tconv_tune_fwd(desc, _ptr(x), _ptr(w), _ptr(b), _ptr(gamma), _ptr(beta),
-                                       _ptr(run_mean), _ptr(run_var), _ptr(z), _ptr(saved), _ptr(workspace),
-                                       wb, _stream(stream)), "convbn_tconv_tune_fwd")
+    if type(desc) is not Desc:
+        desc = _desc(desc)
+    status = (_native or _calls()).convbn_tconv_tune_fwd(desc, x, w, b, gamma, beta, run_mean, run_var, z, saved,
+                                                         workspace, workspace_bytes, stream)
+    if status:
+        _raise(status, "convbn_tconv_tune_fwd")
 
 
 def convbn_tconv_tune_bwd(desc, dz, x, w, b, run_mean, saved, dx, dw, db, dgamma, dbeta, workspace=None,
                           workspace_bytes: Optional[int] = None, stream=None):
-    wb = _nbytes(workspace) if workspace_bytes is None else workspace_bytes
-    _raise(lib().convbn_tconv_tune_bwd(desc, _ptr(dz), _ptr(x), _ptr(w), _ptr(b), _ptr(run_mean),
-                                       _ptr(saved), _ptr(dx), _ptr(dw), _ptr(db), _ptr(dgamma), _ptr(dbeta),
-                                       _ptr(workspace), wb, _stream(stream)), "convbn_tconv_tune_bwd")
+    if type(desc) is not Desc:
+        desc = _desc(desc)
+    status = (_native or _calls()).convbn_tconv_tune_bwd(desc, dz, x, w, b, run_mean, saved, dx, dw, db, dgamma,
+                                                         dbeta, workspace, workspace_bytes, stream)
+    if status:
+        _raise(status, "convbn_tconv_tune_bwd")
 
 
 def convbn_tune_bwd_weight_noalloc(desc, dz, x, w, b, run_mean, saved, dw, db, dgamma, dbeta,
@@ -268,21 +305,22 @@ def convbn_tune_bwd_weight_noalloc(desc, dz, x, w, b, run_mean, saved, dw, db, d
 
 def convbn_eval_fwd(desc, x, w, b, gamma, beta, run_mean, run_var, z, y_saved, workspace=None,
                     workspace_bytes: Optional[int] = None, stream=None):
-    wb = _nbytes(workspace) if workspace_bytes is None else workspace_bytes
-    _raise(lib().convbn_eval_fwd(desc, _ptr(x), _ptr(w), _ptr(b), _ptr(gamma),
-                                 _ptr(beta), _ptr(run_mean), _ptr(run_var), _ptr(z), _ptr(y_saved),
-                                 _ptr(workspace), wb, _stream(stream)),
-           "convbn_eval_fwd")
+    if type(desc) is not Desc:
+        desc = _desc(desc)
+    status = (_native or _calls()).convbn_eval_fwd(desc, x, w, b, gamma, beta, run_mean, run_var, z, y_saved,
+                                                   workspace, workspace_bytes, stream)
+    if status:
+        _raise(status, "convbn_eval_fwd")
 
 
 def convbn_eval_bwd(desc, dz, x, y_saved, w, gamma, run_mean, run_var, dx, dw, db, dgamma, dbeta,
                     workspace=None, workspace_bytes: Optional[int] = None, stream=None):
-    wb = _nbytes(workspace) if workspace_bytes is None else workspace_bytes
-    _raise(lib().convbn_eval_bwd(desc, _ptr(dz), _ptr(x), _ptr(y_saved), _ptr(w),
-                                 _ptr(gamma), _ptr(run_mean), _ptr(run_var), _ptr(dx), _ptr(dw),
-                                 _ptr(db), _ptr(dgamma), _ptr(dbeta), _ptr(workspace),
-                                 wb, _stream(stream)),
-           "convbn_eval_bwd")
+    if type(desc) is not Desc:
+        desc = _desc(desc)
+    status = (_native or _calls()).convbn_eval_bwd(desc, dz, x, y_saved, w, gamma, run_mean, run_var, dx, dw, db,
+                                                   dgamma, dbeta, workspace, workspace_bytes, stream)
+    if status:
+        _raise(status, "convbn_eval_bwd")
 
 
 def convbn_deploy_prepare(desc, w, b, gamma, beta, run_mean, run_var, w_fused, b_fused, stream=None):
@@ -294,19 +332,21 @@ def convbn_deploy_prepare(desc, w, b, gamma, beta, run_mean, run_var, w_fused, b
 
 def convbn_deploy_fwd(desc, x, w_fused, b_fused, z, workspace=None,
                       workspace_bytes: Optional[int] = None, stream=None):
-    wb = _nbytes(workspace) if workspace_bytes is None else workspace_bytes
-    _raise(lib().convbn_deploy_fwd(desc, _ptr(x), _ptr(w_fused), _ptr(b_fused), _ptr(z),
-                                   _ptr(workspace), wb, _stream(stream)),
-           "convbn_deploy_fwd")
+    if type(desc) is not Desc:
+        desc = _desc(desc)
+    status = (_native or _calls()).convbn_deploy_fwd(desc, x, w_fused, b_fused, z, workspace, workspace_bytes, stream)
+    if status:
+        _raise(status, "convbn_deploy_fwd")
 
 
 def convbn_deploy_bwd(desc, dz, x, w_fused, dx, dw_fused, db_fused, workspace=None,
                       workspace_bytes: Optional[int] = None, stream=None):
-    wb = _nbytes(workspace) if workspace_bytes is None else workspace_bytes
-    _raise(lib().convbn_deploy_bwd(desc, _ptr(dz), _ptr(x), _ptr(w_fused), _ptr(dx),
-                                   _ptr(dw_fused), _ptr(db_fused), _ptr(workspace),
-                                   wb, _stream(stream)),
-           "convbn_deploy_bwd")
+    if type(desc) is not Desc:
+        desc = _desc(desc)
+    status = (_native or _calls()).convbn_deploy_bwd(desc, dz, x, w_fused, dx, dw_fused, db_fused, workspace,
+                                                     workspace_bytes, stream)
+    if status:
+        _raise(status, "convbn_deploy_bwd")
 
 
 def _dtype_of(t) -> int:

@@ -7,6 +7,7 @@
 
 #include <map>
 #include <mutex>
+#include <new>
 #include <string>
 #include <vector>
 
@@ -145,7 +146,47 @@ bool strided_dgrad_ok(const convbn_desc *d, const Problem &pb);
 bool umma_dgrad_shape(const convbn_desc *d, const Problem &pb, UmmaConvShape *s);
 
 // bounded: the tensor-core weight gradient in the slices of a call with a fixed scratch; sums: what it sums beside.
+Plan form_plan(const convbn_desc *d, const Problem &pb, int phase, bool bounded, WgradSums sums);
+
+// The plans of the last layers of this thread: a function of the descriptor, the phase and the device (its SM count).  A
+// backward call asks for five of them, 2 us together.
+struct PlanKey {
+    convbn_desc d;
+    int phase, bounded, sums, device, f16;
+};
+struct PlanSlot { PlanKey key; Plan plan; bool used = false; };
+constexpr int kPlanSlots = 256;
+thread_local PlanSlot *t_plans = nullptr;        // made on first use and kept for the life of the thread
+struct PlanOwner { ~PlanOwner() { delete[] t_plans; t_plans = nullptr; } };
+thread_local PlanOwner t_plan_owner;
+
 Plan make_plan(const convbn_desc *d, const Problem &pb, int phase, bool bounded = false, WgradSums sums = WgradSums::kDz) {
+    PlanKey k;
+    memset(&k, 0, sizeof(k));
+    k.d.n = d->n; k.d.c_in = d->c_in; k.d.h_in = d->h_in; k.d.w_in = d->w_in; k.d.c_out = d->c_out; k.d.kh = d->kh; k.d.kw = d->kw;
+    k.d.stride_h = d->stride_h; k.d.stride_w = d->stride_w; k.d.pad_h = d->pad_h; k.d.pad_w = d->pad_w; k.d.dil_h = d->dil_h;
+    k.d.dil_w = d->dil_w; k.d.groups = d->groups; k.d.dtype = d->dtype; k.d.layout = d->layout;      // (no plan depends on eps)
+    k.phase = phase; k.bounded = bounded; k.sums = (int)sums; k.device = current_device_slot(); k.f16 = call_f16();
+    unsigned long long h = 1469598103934665603ull;
+    const int *word = (const int *)&k;
+    for (size_t i = 0; i < sizeof(k) / sizeof(int); ++i) h = (h ^ (unsigned)word[i]) * 1099511628211ull;
+    if (!t_plans) {
+        (void)&t_plan_owner;
+        t_plans = new (std::nothrow) PlanSlot[kPlanSlots];
+        if (!t_plans) return form_plan(d, pb, phase, bounded, sums);
+    }
+    const unsigned at = (unsigned)(h >> 40) % kPlanSlots;
+    if (!t_plans[at].used || memcmp(&t_plans[at].key, &k, sizeof(k)) != 0) {
+        const Plan pl = form_plan(d, pb, phase, bounded, sums);       // (it asks for other plans, which may take this slot)
+        t_plans[at].key = k;
+        t_plans[at].plan = pl;
+        t_plans[at].used = true;
+        return pl;
+    }
+    return t_plans[at].plan;
+}
+
+Plan form_plan(const convbn_desc *d, const Problem &pb, int phase, bool bounded, WgradSums sums) {
     Plan pl;
     UmmaConvShape us;
     if (phase == CONVBN_PHASE_TUNE_BWD) {
@@ -1001,7 +1042,7 @@ static int tune_bwd_impl(const convbn_desc *desc, const void *dz, const void *x,
         const int sw = convbn_tune_bwd_weight(desc, dz, x, w, b, run_mean, saved, dw, db, dgamma, dbeta, ws_w, bytes_w,
                                               lane->stream);
         // whatever happened on the lane, the caller's stream joins it again (a capture must not be left forked)
-        const bool joined = cudaEventRecord(lane->join, lane->stream) == cudaSuccess;
+        const bool joined = defer_join || cudaEventRecord(lane->join, lane->stream) == cudaSuccess;
         const int sd = tune_bwd_data_impl(desc, dz, w, saved, dx, post, workspace, bytes_d, stream);
         if (!joined) return CONVBN_ECUDA;
         if (defer_join) lane->pending = true;
@@ -1021,7 +1062,6 @@ static int tune_bwd_impl(const convbn_desc *desc, const void *dz, const void *x,
         CU(cudaStreamWaitEvent(lane->stream, lane->fork, 0));
         cudaStream_t st = lane->stream;
         LAUNCH("wgrad_rows", launch_wgrad_rows(pb, pl.uw.splits, partials, bsum, w, vec3, b, run_mean, dw, db, dgamma, dbeta, true, st));
-        CU(cudaEventRecord(lane->join, lane->stream));
         lane->pending = true;
         return CONVBN_OK;
     }
