@@ -249,7 +249,6 @@ __global__ void __launch_bounds__(kGThreads) grouped8_wgrad_kernel(const __grid_
     if (threadIdx.x == 256) { prefetch_tensormap(&tm_x); prefetch_tensormap(&tm_dz); }
     __syncthreads();
     pdl_wait();
-    pdl_launch_dependents();
     const int cc = (int)(blockIdx.x % (uint32_t)chunks), slot = (int)(blockIdx.x / (uint32_t)chunks);
     const uint32_t items = (uint32_t)g.n * g.tiles_h;          // bands of this chunk
     const uint32_t x_bytes = g.patch_bytes, dz_bytes = (uint32_t)g.R * g.Wt * 128u;
@@ -319,6 +318,8 @@ __global__ void __launch_bounds__(kGThreads) grouped8_wgrad_kernel(const __grid_
         if (++s == (uint32_t)g.stages) { s = 0; ph ^= 1u; }
     }
     if (!ok && lane == 0) { atomicOr(err, ERRW_TIMEOUT); ctl->abort_flag = 1; }
+    pdl_launch_dependents();       // (earlier, the adding kernel's blocks would wait here and take the data pass's room:
+                                   // forward + backward of 256 channels at 28 x 28, N = 64 57.9 -> 53.9 us)
     // accumulator registers: (row gr = input channel of the first tap, columns 2t, 2t + 1 = output channels),
     // (row gr + 8 = the same input channel of the second tap)
     const int ch0 = cc * 64 + warp * 8, kdim = taps * 8;
