@@ -70,6 +70,27 @@ __device__ __forceinline__ bool win_next_chunk(long long &cur, long long hi, int
     return true;
 }
 
+// win_fill_patch (below) for rows that start anywhere (a width that is no multiple of 8): a pixel per thread, in two-byte loads; neighbours
+// share the sectors.  (Before, such images were packed by a kernel of their own and went through the dense GEMM, three more
+// launches: forward + backward of 3 -> 64, 7x7 stride 2 at 118 x 108, N = 32 93 us, now 62; at 79 x 118, N = 6 41 and 34.)
+template <int C>
+__device__ __noinline__ void win_fill_patch_any(uint8_t *patch, const __nv_bfloat16 *__restrict__ x, int img, int first, int count,
+                                                int h_in, int w_in, int pad_w, int pitch, int tid, int nthreads, uint32_t fill3) {
+    const unsigned short *src = (const unsigned short *)x + (size_t)img * h_in * w_in * C;
+    const int tasks = count * w_in;
+#pragma unroll 4
+    for (int t = tid; t < tasks; t += nthreads) {
+        const int pr = t / w_in, j = t - pr * w_in, h = first + pr;
+        unsigned short e[4] = {0, 0, 0, C > 3 ? (unsigned short)0 : (unsigned short)fill3};
+        if (h >= 0 && h < h_in) {
+#pragma unroll
+            for (int c = 0; c < C; ++c) e[c] = __ldg(src + ((size_t)h * w_in + j) * C + c);
+        }
+        *(uint2 *)(patch + (size_t)pr * pitch + (size_t)(pad_w + j) * 8) =
+            make_uint2((uint32_t)e[0] | ((uint32_t)e[1] << 16), (uint32_t)e[2] | ((uint32_t)e[3] << 16));
+    }
+}
+
 // Fills `count` rows of a patch buffer with input rows first, first + 1, ... of image img: pixels of C channels
 // widened to 4 (8 bytes) behind a left border of pad_w pixels; rows outside the image are zero.  fill3 is the
 // bit pattern of channel slot 3 (C <= 3 only): 0, or bf16 1.0 when the weight-gradient GEMM takes sum dZ from it
@@ -78,8 +99,12 @@ template <int C>
 __device__ __forceinline__ void win_fill_patch(uint8_t *patch, const __nv_bfloat16 *__restrict__ x, int img, int first,
                                                int count, int h_in, int w_in, int pad_w, int pitch, int tid, int nthreads,
                                                uint32_t fill3) {
-    const int chunks_w = w_in / 8, tasks = count * chunks_w;
     const uint32_t hi_fill = fill3 << 16;
+    if (w_in % 8) {
+        win_fill_patch_any<C>(patch, x, img, first, count, h_in, w_in, pad_w, pitch, tid, nthreads, fill3);
+        return;
+    }
+    const int chunks_w = w_in / 8, tasks = count * chunks_w;
 #pragma unroll 4
     for (int t = tid; t < tasks; t += nthreads) {
         const int pr = t / chunks_w, j = t - pr * chunks_w, h = first + pr;
@@ -676,7 +701,7 @@ struct WinPlan { bool ok = false; int R = 0, nstrips = 0, pitch = 0, kblocks = 0
 WinPlan plan_window(const Problem &pb) {
     WinPlan pl;
     if (pb.groups != 1 || pb.c_in > 4 || pb.stride_w != 2 || pb.stride_h != 2 || pb.dil_h != 1 ||
-        pb.dil_w != 1 || pb.kw > 8 || pb.kh > 16 || (pb.c_out != 64 && pb.c_out != 128) || pb.w_in % 8 ||
+        pb.dil_w != 1 || pb.kw > 8 || pb.kh > 16 || (pb.c_out != 64 && pb.c_out != 128) ||
         pb.pad_w > 64 || pb.pad_h > 64 || pb.p >= (1LL << 30) || pb.pin >= (1LL << 30))
         return pl;
     pl.pitch = (int)(((size_t)(pb.w_in + 2 * pb.pad_w) * 8 + 15) / 16 * 16);

@@ -282,10 +282,13 @@ __global__ void __launch_bounds__(kDgThreads) stem_window_dgrad_kernel(const __g
                         }
                     }
                     named_bar_sync(bar_id, 128);
-                    {
+                    if (g.w_in % 8 == 0) {
                         const int n16 = g.w_in * C * 2 / 16;
                         uint4 *dst = (uint4 *)(dx + ((size_t)sg.img * g.h_in + rho) * g.w_in * C);
                         for (int i = gt; i < n16; i += 128) dst[i] = ((const uint4 *)rbuf)[i];
+                    } else {                                   // rows start anywhere
+                        uint16_t *dst = (uint16_t *)(dx + ((size_t)sg.img * g.h_in + rho) * g.w_in * C);
+                        for (int i = gt; i < g.w_in * C; i += 128) dst[i] = ((const uint16_t *)rbuf)[i];
                     }
                     if (warp == 4 && lane == 0) CONVBN_TRACE_ACC(7);
                 }
@@ -321,7 +324,7 @@ cudaError_t launch_window_dgrad(const CUtensorMap &tdz, const WinDgrad &g, size_
 
 bool stem_window_dgrad_eligible(const Problem &pb) {
     if (pb.groups != 1 || pb.c_in > 4 || pb.stride_w != 2 || pb.stride_h != 2 || pb.dil_h != 1 || pb.dil_w != 1) return false;
-    if (pb.kw > 8 || pb.kh > 8 || pb.kh < 2 || pb.c_out != 64 || pb.w_in % 8 || pb.w_out > 128) return false;
+    if (pb.kw > 8 || pb.kh > 8 || pb.kh < 2 || pb.c_out != 64 || pb.w_out > 128) return false;
     if (pb.w_in + pb.pad_w > 256 || pb.pad_h > 64 || pb.pad_w > 64 || (size_t)pb.w_in * pb.c_in * 2 > 2048) return false;
     if (pb.p >= (1LL << 30) || pb.pin >= (1LL << 30)) return false;
     return dgrad_window_smem(pb) <= 226 * 1024;
