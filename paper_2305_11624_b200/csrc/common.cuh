@@ -192,6 +192,27 @@ inline cudaError_t max_dynamic_smem_once(K kernel, int bytes, PerDevice *flag) {
 #define CONVBN_TRACE_ACC(id) ((void)0)         // ... whose duration is added to slot id
 #endif
 
+// n / d for n < 2^31 by a multiplication: m = floor(2^(31 + l) / d) + 1 with 2^(l - 1) < d <= 2^l (Granlund and Montgomery,
+// "Division by invariant integers using multiplication", 1994).  A division by a variable is a chain of some 25 instructions.
+struct FastDiv {
+    uint32_t d = 1, mul = 0, shift = 0;
+    FastDiv() = default;
+    explicit FastDiv(uint32_t div) : d(div) {
+        if (d == 1) return;
+        uint32_t l = 0;
+        while ((1ull << l) < d) ++l;
+        mul = (uint32_t)((1ull << (31 + l)) / d + 1);
+        shift = l - 1;
+    }
+    __host__ __device__ __forceinline__ uint32_t div(uint32_t n) const {
+#ifdef __CUDA_ARCH__
+        return d == 1 ? n : __umulhi(n, mul) >> shift;
+#else
+        return d == 1 ? n : (uint32_t)(((unsigned long long)n * mul) >> 32) >> shift;
+#endif
+    }
+};
+
 static inline int ceil_div_i(long long a, long long b) { return (int)((a + b - 1) / b); }
 static inline size_t align_up(size_t v, size_t a) { return (v + a - 1) / a * a; }
 

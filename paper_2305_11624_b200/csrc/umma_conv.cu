@@ -58,6 +58,7 @@ struct ConvGemm {
     // c of output pixel (i kh + r, j kw + q), tap = r kw + q, in out_strided; out_sh / out_sw are the steps of i and j,
     // tap_sh / tap_sw those of r and q.  The weight tensor is then read as it is, [ca][cn], as an MN-major operand.
     int tap_c, tap_kw, tap_sh, tap_sw;
+    FastDiv by_n, by_wo, by_ho;                     // by the tiles of a row of tiles, wo, ho
     const __nv_bfloat16 *post_add, *post_mask;      // at the output's offsets
     int post_relu;
 };
@@ -123,20 +124,21 @@ __global__ void __launch_bounds__(MODE == kPlain || MODE == kRelu || MODE == kTa
     const bool fold = g.fold.gamma != nullptr;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int stages = g.stages;
-    const uint32_t n_tiles = (uint32_t)(g.cn + BN - 1) / BN;
+    const uint32_t n_tiles = g.by_n.d;
     const uint32_t m_tiles = (uint32_t)((g.p + kBM - 1) / kBM);
     const uint32_t total_tiles = (PAIR ? (m_tiles + 1) / 2 : m_tiles) * n_tiles;
     // Tile i of this CTA.  Resident weights: the CTA keeps one n-tile (blockIdx.x % n_tiles) and walks
     // m-tiles; otherwise tiles are dealt round-robin with the n-tiles of an m-tile on neighbouring CTAs.
     auto tile_of = [&](uint32_t i, uint32_t &mt, uint32_t &nt) -> bool {
         if (g.resident) {
-            nt = blockIdx.x % n_tiles;
-            mt = blockIdx.x / n_tiles + i * (gridDim.x / n_tiles);
+            const uint32_t row = g.by_n.div(blockIdx.x);
+            nt = blockIdx.x - row * n_tiles;
+            mt = row + i * g.by_n.div(gridDim.x);
             return mt < m_tiles;
         }
         const uint32_t t = blockIdx.x / CTAS + i * (gridDim.x / CTAS);
         if (t >= total_tiles) return false;
-        mt = t / n_tiles;
+        mt = g.by_n.div(t);
         nt = t - mt * n_tiles;
         if constexpr (PAIR) mt = 2 * mt + rank;         // (of an odd number of m-tiles the last has no partner: all out of range)
         return true;
@@ -147,7 +149,28 @@ __global__ void __launch_bounds__(MODE == kPlain || MODE == kRelu || MODE == kTa
 
     // the tensor maps are kernel parameters, not data of an earlier kernel: their way to the copy engine starts at once
     if (threadIdx.x == 64) { prefetch_tensormap(&tm_act); prefetch_tensormap(&tm_w); prefetch_tensormap(&tm_out); }
-    if (threadIdx.x == 0) {
+    // What the first load of the activations needs is worked out beside the set-up (after it, with divisions, that load went out
+    // 1100 clocks late: with the same in umma_wgrad.cu ResNet-50, N = 32 2463 -> 2426 us).
+    auto pixel_of = [&](uint32_t mt, int &img, int &ho, int &wo) {
+        if (g.stem) {           // m-tile -> (image, patch row, patch column)
+            const uint32_t tq = mt / (uint32_t)g.stem_tiles_w;
+            wo = (int)(mt - tq * (uint32_t)g.stem_tiles_w) * g.stem_tw;
+            img = (int)(tq / (uint32_t)g.stem_tiles_h);
+            ho = (int)(tq - (uint32_t)img * (uint32_t)g.stem_tiles_h) * g.stem_th;
+        } else {
+            const uint32_t m0 = (PAIR && mt >= m_tiles ? m_tiles - 1 : mt) * kBM, tq = g.by_wo.div(m0);
+            wo = (int)(m0 - tq * (uint32_t)g.wo);
+            img = (int)g.by_ho.div(tq);
+            ho = (int)(tq - (uint32_t)img * (uint32_t)g.ho);
+        }
+    };
+    uint32_t first_mt = 0, first_nt = 0;
+    int first_img = 0, first_ho = 0, first_wo = 0;
+    if (warp == 0) {
+        tile_of(0, first_mt, first_nt);
+        pixel_of(first_mt, first_img, first_ho, first_wo);
+    }
+    if (threadIdx.x == 96) {
         CONVBN_TRACE_POINT(0);
         for (int s = 0; s < stages; ++s) { mbar_init(&ctl->full[s], g.resident ? 1 : 2); mbar_init(&ctl->empty[s], 1); }
         for (int a = 0; a < 2; ++a) { mbar_init(&ctl->tmem_full[a], 1); mbar_init(&ctl->tmem_empty[a], 4 * CTAS); }
@@ -195,23 +218,9 @@ __global__ void __launch_bounds__(MODE == kPlain || MODE == kRelu || MODE == kTa
             bool ok = true, free = false;
             uint32_t mt, nt;
             for (uint32_t i = 0; ok && tile_of(i, mt, nt); ++i) {
-                // 32-bit arithmetic: 64-bit divisions would cost about a microsecond per tile here
-                const uint32_t m0 = (PAIR && mt >= m_tiles ? m_tiles - 1 : mt) * kBM;
                 const int n0 = (int)nt * BN;
-                uint32_t tq, img;
-                int wo0, ho0;
-                if (g.stem) {       // m-tile -> (image, patch row, patch column)
-                    tq = mt / (uint32_t)g.stem_tiles_w;
-                    wo0 = (int)(mt - tq * (uint32_t)g.stem_tiles_w) * g.stem_tw;
-                    img = tq / (uint32_t)g.stem_tiles_h;
-                    ho0 = (int)(tq - img * (uint32_t)g.stem_tiles_h) * g.stem_th;
-                } else {
-                    tq = m0 / (uint32_t)g.wo;
-                    wo0 = (int)(m0 - tq * (uint32_t)g.wo);
-                    img = tq / (uint32_t)g.ho;
-                    ho0 = (int)(tq - img * (uint32_t)g.ho);
-                }
-                const int img0 = (int)img;
+                int img0 = first_img, ho0 = first_ho, wo0 = first_wo;
+                if (i) pixel_of(mt, img0, ho0, wo0);
                 const int base_w = g.lower_w + wo0 * g.stride_w, base_h = g.lower_h + ho0 * g.stride_h;
                 // K: an inner run over the channels of a tap (or, chunk_outer, over a row of taps) with one addition a step
                 const int c_first = g.blockdiag ? n0 : 0, w_end = g.taps_w * g.dil_w, h_end = g.taps_h * g.dil_h;
@@ -321,7 +330,7 @@ __global__ void __launch_bounds__(MODE == kPlain || MODE == kRelu || MODE == kTa
             const int k_step = g.chunk_outer ? g.ca : kBK;
             bool ok = true, free = false;
             if (g.resident) {
-                const int n0 = (int)(blockIdx.x % n_tiles) * BN;
+                const int n0 = (int)(blockIdx.x - g.by_n.div(blockIdx.x) * n_tiles) * BN;
                 mbar_arrive_expect_tx(&ctl->bfull, (uint32_t)num_kb * kBBytes);
                 int k = 0;
                 for (int kb = 0; kb < num_kb; ++kb) {
@@ -426,9 +435,21 @@ __global__ void __launch_bounds__(MODE == kPlain || MODE == kRelu || MODE == kTa
         uint8_t *add_buf = staging + (size_t)g.nbuf * kStagingBytes + (size_t)(warp - 2) * kStagingWarpBytes, *mask_buf = add_buf + (g.post_add ? kStagingBytes : 0);
         uint32_t post_ph = 0;
         bool post_pending = false;
-        auto fetch_post = [&](uint32_t ti, int c0) {          // chunk c0 of tile ti of this CTA, if there is one
-            uint32_t m, n;
-            post_pending = extra > 0 && tile_of(ti, m, n);
+        // Columns [lo, hi) of tile i are this group's: the groups take tiles in turn, and halve the last one, which nothing is
+        // left to overlap with (forward + backward of 3x3 stride 2 128 -> 128 at 200 x 334, N = 2 58.9 -> 57.4 us,
+        // ResNet-50, N = 32 2480 -> 2463).
+        auto columns_of = [&](uint32_t i, uint32_t &m, uint32_t &n, int &lo, int &hi) -> bool {
+            if (!tile_of(i, m, n)) return false;
+            const bool own = (i & 1u) == egroup;
+            uint32_t m2, n2;
+            if (BN >= 128 && !tile_of(i + 1, m2, n2)) { lo = own ? 0 : BN / 2; hi = lo + BN / 2; }
+            else { lo = 0; hi = own ? BN : 0; }
+            const int valid = g.cn - (int)n * BN;
+            if (hi > valid) hi = valid;
+            return true;
+        };
+        auto fetch_post = [&](uint32_t m, uint32_t n, int c0) {
+            post_pending = extra > 0;
             if (!post_pending || lane != 0) return;
             uint64_t *bar = &ctl->post_full[warp - 2];
             mbar_arrive_expect_tx(bar, (uint32_t)extra * kStagingWarpBytes);
@@ -436,9 +457,18 @@ __global__ void __launch_bounds__(MODE == kPlain || MODE == kRelu || MODE == kTa
             if (g.post_add) tma_load_2d(add_buf, &tm_out2, bar, x, y);
             if (g.post_mask) tma_load_2d(mask_buf, &tm_mask, bar, x, y);
         };
-        if constexpr (POST) fetch_post(egroup, 0);
-        for (uint32_t i = egroup; tile_of(i, mt, nt); i += 2) {
-            const uint32_t acc = egroup;
+        auto fetch_from = [&](uint32_t i) {                   // the first chunk of this group's next tile, from tile i on
+            uint32_t m, n;
+            int lo, hi;
+            post_pending = false;
+            for (; columns_of(i, m, n, lo, hi); ++i)
+                if (lo < hi) { fetch_post(m, n, lo); return; }
+        };
+        if constexpr (POST) fetch_from(0);
+        int c_lo, c_hi;
+        for (uint32_t i = 0; columns_of(i, mt, nt, c_lo, c_hi); ++i) {
+            if (c_lo >= c_hi) continue;
+            const uint32_t acc = i & 1u;
             CONVBN_TRACE_T0();
             const bool ok = __all_sync(0xffffffffu, mbar_wait_bounded(&ctl->tmem_full[acc], (i >> 1) & 1u, abort_flag));
             if (warp == 2 && lane == 0) CONVBN_TRACE_ACC(15);
@@ -450,13 +480,11 @@ __global__ void __launch_bounds__(MODE == kPlain || MODE == kRelu || MODE == kTa
             const uint32_t m0 = mt * kBM;
             const int n0 = (int)nt * BN;
             const uint32_t t_row = tmem_base + acc * BN + ((uint32_t)(quarter * 32) << 16);
-            int ncols = g.cn - n0;                          // valid columns of this tile
-            if (ncols > BN) ncols = BN;
             __nv_bfloat16 *srow = nullptr;                  // strided mode: this thread's output pixel
             if (g.out_strided) {
                 const uint32_t m = m0 + quarter * 32 + lane;
                 if ((long long)m < g.p) {
-                    const uint32_t tq = m / (uint32_t)g.wo, img = tq / (uint32_t)g.ho;
+                    const uint32_t tq = g.by_wo.div(m), img = g.by_ho.div(tq);
                     srow = g.out_strided + (size_t)img * g.out_sn + (size_t)(tq - img * (uint32_t)g.ho) * g.out_sh +
                            (size_t)(m - tq * (uint32_t)g.wo) * g.out_sw;
                     if constexpr (TAP) {                    // (a tile lies inside one tap: BN divides tap_c)
@@ -469,7 +497,7 @@ __global__ void __launch_bounds__(MODE == kPlain || MODE == kRelu || MODE == kTa
             }
             const int p0 = TAP ? n0 % g.tap_c : n0;         // first per-channel parameter of this tile
 #pragma unroll 1
-            for (int c0 = 0; c0 < BN; c0 += 64) {
+            for (int c0 = c_lo; c0 < c_hi; c0 += 64) {
                 uint32_t v[2][32];                          // rows 0-15 and 16-31 of this warp
                 f32x2 sc[4], sh[4];                         // parameters of 32 columns
                 auto params = [&](int i0, uint32_t sc_at, uint32_t sh_at) {
@@ -479,14 +507,12 @@ __global__ void __launch_bounds__(MODE == kPlain || MODE == kRelu || MODE == kTa
                         if (sc_at) sc[i] = lds_f32x2(sc_at + (uint32_t)(p0 + c0 + 8 * (i0 + i)) * 4u);
                     }
                 };
-                if (c0 < ncols) {
-                    tmem_ld_16x64(t_row + (uint32_t)c0, v[0]);
-                    tmem_ld_16x64(t_row + (16u << 16) + (uint32_t)c0, v[1]);
-                    params(0, DUAL ? 0u : scale_at, shift_at);
-                    tmem_ld_wait();
-                }
-                if (c0 + 64 >= BN) {
-                    // every column of this accumulator has been read: hand the buffer back
+                tmem_ld_16x64(t_row + (uint32_t)c0, v[0]);
+                tmem_ld_16x64(t_row + (16u << 16) + (uint32_t)c0, v[1]);
+                params(0, DUAL ? 0u : scale_at, shift_at);
+                tmem_ld_wait();
+                if (c0 + 64 >= c_hi && acc == egroup) {
+                    // every column of this accumulator has been read: hand the buffer back (nobody waits for the last one)
                     tc_fence_before_sync();
                     __syncwarp();
                     if (lane == 0) {
@@ -494,7 +520,7 @@ __global__ void __launch_bounds__(MODE == kPlain || MODE == kRelu || MODE == kTa
                         else mbar_arrive(&ctl->tmem_empty[acc]);
                     }
                 }
-                if (c0 < ncols) {
+                {
                     uint8_t *buf = next_buf();
                     const uint32_t frag = smem_u32(buf) + frag_row;
                     if constexpr (POST) {
@@ -551,7 +577,7 @@ __global__ void __launch_bounds__(MODE == kPlain || MODE == kRelu || MODE == kTa
                     else pack(yes, no, no);
                     if constexpr (POST) {
                         __syncwarp();                          // every lane has read its rows of the boxes
-                        if (c0 + 64 < ncols) fetch_post(i, c0 + 64); else fetch_post(i + 2, 0);
+                        if (c0 + 64 < c_hi) fetch_post(mt, nt, c0 + 64); else fetch_from(i + 1);
                     }
                     if constexpr (POST_STRIDED) {
                         // as below, with the other tensors' values of four pixels requested before the first is used
@@ -565,7 +591,7 @@ __global__ void __launch_bounds__(MODE == kPlain || MODE == kRelu || MODE == kTa
                             for (int k = 0; k < 4; ++k) {
                                 const __nv_bfloat16 *dst = (const __nv_bfloat16 *)__shfl_sync(
                                     0xffffffffu, (unsigned long long)srow, (i0 + k) * 4 + (lane >> 3));
-                                const bool on = dst && c0 + ch * 8 < ncols;
+                                const bool on = dst && c0 + ch * 8 < c_hi;
                                 at8[k] = on ? dst - g.out_strided + c0 + ch * 8 : -1;
                                 av[k] = mv[k] = make_uint4(0u, 0u, 0u, 0u);
                                 if (on && g.post_add) av[k] = *(const uint4 *)(g.post_add + at8[k]);
@@ -591,7 +617,7 @@ __global__ void __launch_bounds__(MODE == kPlain || MODE == kRelu || MODE == kTa
                             const int rr = it * 4 + (lane >> 3), ch = lane & 7;
                             __nv_bfloat16 *dst = (__nv_bfloat16 *)__shfl_sync(0xffffffffu, (unsigned long long)srow, rr);
                             const uint4 q = *(const uint4 *)(buf + rr * 128 + (((ch ^ (rr & 7)) & 7) << 4));
-                            if (dst && c0 + ch * 8 < ncols) *(uint4 *)(dst + c0 + ch * 8) = q;
+                            if (dst && c0 + ch * 8 < c_hi) *(uint4 *)(dst + c0 + ch * 8) = q;
                         }
                         __syncwarp();
                         continue;
@@ -779,6 +805,7 @@ static cudaError_t launch_bn(const CUtensorMap &ta, const CUtensorMap &tw, const
     // (256: the epilogue reads the per-channel parameters of whole 64-column chunks)
     size_t fixed = 1024 + 256 + (size_t)(g.nbuf + extra) * kStagingBytes + sizeof(ConvSmemCtl) + (MODE == kDual ? 3 : 2) * (size_t)g.cn * sizeof(float) + 16;
     const long long m_tiles = (g.p + kBM - 1) / kBM, n_tiles = (g.cn + BN - 1) / BN;
+    g.by_n = FastDiv((uint32_t)n_tiles); g.by_wo = FastDiv((uint32_t)g.wo); g.by_ho = FastDiv((uint32_t)g.ho);
     long long grid_l = m_tiles * n_tiles < sm_count() ? m_tiles * n_tiles : sm_count();
     if (PAIR) {
         const long long pairs = (m_tiles + 1) / 2 * n_tiles;
