@@ -1328,13 +1328,13 @@ int tconv_view(const convbn_desc *d, TconvView *v) {
     v->bsplits = channel_sum_splits(v->sum_pb);
     v->fwd = make_plan(&v->conv, v->pb, CONVBN_PHASE_DEPLOY_FWD);
     // Where the windows of the convolution tile dZ (kernel = stride), the tensor-core weight gradient sums it, its windowed
-    // operand, itself: a row per slice, turn and tap.
+    // operand, itself: two rows per slice and tap.
     v->sums = d->kh == d->stride_h && d->kw == d->stride_w && !d->pad_h && !d->pad_w && d->dil_h == 1 &&
                       d->dil_w == 1
                   ? WgradSums::kX : WgradSums::kNone;
     v->bwd = make_plan(&v->conv, v->pb, CONVBN_PHASE_DEPLOY_BWD, false, v->sums);
     v->gemm_sums = v->bwd.umma_wgrad && v->sums == WgradSums::kX;
-    if (v->gemm_sums) v->bsplits = v->bwd.uw.splits * umma_wgrad_x_sum_rows(v->pb) * d->kh * d->kw;
+    if (v->gemm_sums) v->bsplits = v->bwd.uw.splits * 2 * d->kh * d->kw;
     v->wcount = (size_t)d->c_in * (d->c_out / d->groups) * d->kh * d->kw;
     size_t off = 0;
     auto take = [&](size_t bytes) { const size_t at0 = off; off += (bytes + 255) / 256 * 256; return at0; };

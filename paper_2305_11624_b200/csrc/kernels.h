@@ -142,12 +142,11 @@ UmmaWgradPlan umma_wgrad_plan(const Problem &pb, WgradSums sums = WgradSums::kDz
 UmmaWgradPlan umma_wgrad_plan_bounded(const Problem &pb);     // for calls with a fixed scratch
 // partials: [splits][C_out][kdim] fp32 (the layout of the weights; block-diagonal: [splits][block][k][64])
 // bsum    : [splits][C_out] fp32 per-slice sums of dZ over pixels (from a ones row in the GEMM); with kX
-//           [splits umma_wgrad_x_sum_rows][kdim] sums over pixels of the im2col operand instead
+//           [2 splits][kdim] sums over pixels of the im2col operand instead
 // counters: `ncounters` words zeroed for an epilogue that counts its blocks (may be NULL)
 cudaError_t launch_umma_wgrad(const Problem &pb, const UmmaWgradPlan &pl, const void *dz, const void *x,
                               float *partials, float *bsum, cudaStream_t st, unsigned int *counters = nullptr,
                               int ncounters = 0, WgradSums sums = WgradSums::kDz);
-int umma_wgrad_x_sum_rows(const Problem &pb);
 // Everything after the GEMM: dw[co][k] = scale[co] * sum_splits partials (scale = first
 // C_out floats of vec3, 1 if NULL); with need_sums also dbeta, db, dgamma (vec3 given) or db = sum dZ.
 cudaError_t launch_wgrad_rows(const Problem &pb, int splits, const float *partials, const float *bsum, const void *w,

@@ -29,26 +29,25 @@ struct WgradGemm {
     int kdim;               // taps * c_in
     long long p;            // output pixels
     long long per_split;    // pixels per slice (multiple of 64)
+    FastDiv by_wo, by_ho, by_ci, by_tw;      // by wo, ho, c_in, taps_w
     int stages;
     int blockdiag;          // grouped conv: c_in = 64 here, k rows are (tap, channel of block blockIdx.y)
     // Small-C_in ("stem") mode: tm_x is the 5-D window view of the packed input (one 64-wide slice per
     // filter row), tm_dz a 4-D map of dZ; a "pixel block" is a 4 x 16 patch of output pixels.
     int stem, stem_tiles_w, stem_tiles_h;
     // Where the per-channel sums come from.  kSumNone: nowhere (the packed stem input carries a constant-1 slot instead).
-    // kSumSlice: a slice of ones behind the last slice of k; its accumulator rows are sum_p dZ[p][co].  kSumX: the X tile times
-    // ones, in an accumulator of its own, the tiles of channels taking turns at the stages (the sums of a transposed layer's dZ,
-    // which is the windowed operand there).  Ones times the dZ tile in the same way, instead of the slice, were measured where
-    // the number of slices is even and the slice costs another row of tiles: 2 to 6 % slower for most layers (3x3 256 at 23 x 21,
-    // N = 8 34.9 -> 36.7 us, ResNet-50, N = 32 2464 -> 2500), the products being a second full MMA per step.
+    // kSumSlice: a slice of ones behind the last slice of k; its accumulator rows are sum_p dZ[p][co].  kSumX: the rows of the X
+    // tiles, added in fp32 by the epilogue warps while the tiles are multiplied (the sums of a transposed layer's dZ, which is
+    // the windowed operand there; by products of ones in a second accumulator they were 1.2e-6 off instead of 1e-7).  Ones times
+    // the dZ tile in an accumulator of its own, instead of the slice, were measured where the number of slices is even and the
+    // slice costs another row of tiles: 2 to 6 % slower for most layers (3x3 256 at 23 x 21, N = 8 34.9 -> 36.7 us, ResNet-50,
+    // N = 32 2464 -> 2500), the products being a second full MMA per step.
     int sums;
     int f16;                // 16-bit storage type: 0 bf16, 1 IEEE half
     int rows;               // 1: partials are [split][C_out][kdim], 0: [split][k][C_out]
 };
 
 enum { kSumNone, kSumSlice, kSumX };
-constexpr int kMaxTurns = 8;               // every turn leaves a row of sums for the adding kernel to read
-constexpr uint32_t kOnesBytes = 1024;      // one 8 x 128-byte group, read with all strides 0
-
 struct WgradSmemCtl {
     uint64_t full[kWMaxStages];
     uint64_t empty[kWMaxStages];
@@ -57,7 +56,7 @@ struct WgradSmemCtl {
     int abort_flag;
 };
 
-// X_SUMS: g.sums is kSumX (as a run-time branch in the issuing loop it cost the other layers 1 %).
+// X_SUMS: g.sums is kSumX.
 template <int BN, bool X_SUMS>
 __global__ void __launch_bounds__(kWThreads) umma_wgrad_kernel(const __grid_constant__ CUtensorMap tm_x,
                                                               const __grid_constant__ CUtensorMap tm_dz,
@@ -68,8 +67,7 @@ __global__ void __launch_bounds__(kWThreads) umma_wgrad_kernel(const __grid_cons
     extern __shared__ uint8_t smem_raw[];
     constexpr uint32_t kABytes = 2 * kChunkBytes, kBBytes = (BN / 64) * kChunkBytes, kStageBytes = kABytes + kBBytes;
     uint8_t *tiles = (uint8_t *)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
-    uint8_t *ones_tile = tiles + (size_t)g.stages * kStageBytes;
-    WgradSmemCtl *ctl = (WgradSmemCtl *)(ones_tile + kOnesBytes);
+    WgradSmemCtl *ctl = (WgradSmemCtl *)(tiles + (size_t)g.stages * kStageBytes);
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int stages = g.stages;
     const int k0 = blockIdx.x * kWM;                    // first k row of this tile
@@ -80,36 +78,48 @@ __global__ void __launch_bounds__(kWThreads) umma_wgrad_kernel(const __grid_cons
     const int nch = g.kdim / 64, c_first = k0 / 64;
     const int a_chunks = nch - c_first >= 2 ? 2 : (nch - c_first >= 1 ? 1 : 0);   // slices loaded by TMA
     const int ones_slot = g.sums != kSumSlice ? -1 : ((c_first == nch) ? 0 : (c_first + 1 == nch ? 1 : -1));
-    // kSumX: this CTA adds the stages turn, turn + turns, ... (the first kMaxTurns tiles do)
-    const int turn = (int)blockIdx.y, turns = min((int)gridDim.y, kMaxTurns);
-    const bool adds = X_SUMS && turn < turns;
+    const bool adds = X_SUMS && blockIdx.y == 0;         // (kSumX: the first tile of channels)
     int b_chunks = (g.c_out - n0) / 64;
     if (b_chunks > BN / 64) b_chunks = BN / 64;
     volatile int *abort_flag = &ctl->abort_flag;
 
-    if (threadIdx.x == 0) {
-        for (int s = 0; s < stages; ++s) { mbar_init(&ctl->full[s], 2); mbar_init(&ctl->empty[s], 1); }
+    // the tensor maps are kernel parameters, not data of an earlier kernel: fetch them before the wait
+    if (threadIdx.x == 96) { prefetch_tensormap(&tm_x); prefetch_tensormap(&tm_dz); }
+    // The X loads' coordinates, worked out beside the set-up: the slices' k = tap * c_in + ci is fixed for the whole CTA, the pixel
+    // is that of the slice's start.
+    int ci[2] = {0, 0}, wo0 = 0, ho0 = 0;
+    uint16_t off_w[2] = {0, 0}, off_h[2] = {0, 0};
+    uint32_t img = 0;
+    if (warp == 0) {
+#pragma unroll
+        for (int j = 0; j < 2; ++j) {
+            const int kk = k0 + j * 64, tap = (int)g.by_ci.div((uint32_t)kk), tr = (int)g.by_tw.div((uint32_t)tap);
+            ci[j] = kk - tap * g.c_in + (g.blockdiag ? n0 : 0);
+            off_w[j] = (uint16_t)((tap - tr * g.taps_w) * g.dil_w);
+            off_h[j] = (uint16_t)(tr * g.dil_h);
+        }
+        const uint32_t pp = (uint32_t)p0, t0 = g.by_wo.div(pp);
+        wo0 = (int)(pp - t0 * (uint32_t)g.wo);
+        img = g.by_ho.div(t0);
+        ho0 = (int)(t0 - img * (uint32_t)g.ho);
+    }
+    if (threadIdx.x == 64) {
+        for (int s = 0; s < stages; ++s) { mbar_init(&ctl->full[s], 2); mbar_init(&ctl->empty[s], adds ? 5 : 1); }
         mbar_init(&ctl->tmem_full, 1);
         ctl->abort_flag = 0;
         fence_barrier_init();
     }
     if (warp == 1) {
-        tmem_alloc(&ctl->tmem_base, X_SUMS ? 2 * BN : BN);
+        tmem_alloc(&ctl->tmem_base, BN);
         tmem_relinquish();
     }
-    // the tensor maps are kernel parameters, not data of an earlier kernel: fetch them before the wait
-    if (threadIdx.x == 0) { prefetch_tensormap(&tm_x); prefetch_tensormap(&tm_dz); }
     pdl_wait();                 // global memory only after every earlier kernel has finished
     // counters of the epilogue kernel that runs after this one start from zero
     if (counters && blockIdx.x == 0 && blockIdx.y == 0 && blockIdx.z == 0)
         for (int i = threadIdx.x; i < ncounters; i += kWThreads) counters[i] = 0u;
-    const uint32_t one2 = one_h16(g.f16) * 0x10001u;
-    if constexpr (X_SUMS) {
-        for (int i = threadIdx.x; i < (int)(kOnesBytes / 16); i += kWThreads) ((uint4 *)ones_tile)[i] = make_uint4(one2, one2, one2, one2);
-        fence_proxy_async_smem();
-    }
     if (ones_slot >= 0) {
         // 1.0 everywhere (invariant under the swizzle); TMA never writes this slice
+        const uint32_t one2 = one_h16(g.f16) * 0x10001u;
         const uint4 ones = make_uint4(one2, one2, one2, one2);
         for (int s = 0; s < stages; ++s) {
             uint4 *dst = (uint4 *)(tiles + (size_t)s * kStageBytes + (size_t)ones_slot * kChunkBytes);
@@ -149,21 +159,6 @@ __global__ void __launch_bounds__(kWThreads) umma_wgrad_kernel(const __grid_cons
         // 3x3 64 at 56 x 56, N = 32 21.9 -> 19.4.
         if (elect_one()) {
             const uint32_t tx_bytes = (uint32_t)a_chunks * kChunkBytes;
-            // the slices' k = tap * c_in + ci is fixed for the whole CTA
-            int ci[2];
-            uint16_t off_w[2], off_h[2];
-#pragma unroll
-            for (int j = 0; j < 2; ++j) {
-                const int kk = k0 + j * 64, tap = kk / g.c_in, tr = tap / g.taps_w;
-                ci[j] = kk - tap * g.c_in + (g.blockdiag ? n0 : 0);
-                off_w[j] = (uint16_t)((tap - tr * g.taps_w) * g.dil_w);
-                off_h[j] = (uint16_t)(tr * g.dil_h);
-            }
-            // pixel coordinates of the slice start, advanced by 64 pixels per stage without divisions
-            const uint32_t pp = (uint32_t)p0, t0 = pp / (uint32_t)g.wo;
-            int wo0 = (int)(pp - t0 * (uint32_t)g.wo);
-            uint32_t img = t0 / (uint32_t)g.ho;
-            int ho0 = (int)(t0 - img * (uint32_t)g.ho);
             const uint32_t blk0 = (uint32_t)(p0 / kWP);
 #pragma unroll 4
             for (int kb = 0; kb < num_kb; ++kb) {
@@ -219,10 +214,6 @@ __global__ void __launch_bounds__(kWThreads) umma_wgrad_kernel(const __grid_cons
             const uint32_t hi = smem_desc_hi_sw128(1024);
             const uint32_t tiles_lo = smem_desc_lo(smem_u32(tiles), kChunkBytes);
             uint32_t a_lo = tiles_lo;
-            const uint32_t ones_lo = smem_desc_lo(smem_u32(ones_tile), 0), ones_hi = smem_desc_hi_sw128(0);
-            const uint32_t idesc_x = idesc_h16_f32(kWM, 16, 1, 1, g.f16);
-            int wait_turn = adds ? turn : num_kb;
-            uint32_t adding = 0;
             ph = 0;
 #pragma unroll 4
             for (int kb = 0; kb < num_kb; ++kb) {
@@ -243,21 +234,43 @@ __global__ void __launch_bounds__(kWThreads) umma_wgrad_kernel(const __grid_cons
                 for (int k = 1; k < kWP / kWUmmaK; ++k)
                     umma_bf16_ss_halves<true>(tmem_base, a0 + (uint32_t)k * (kWUmmaK * 128 >> 4), hi,
                                               b0 + (uint32_t)k * (kWUmmaK * 128 >> 4), hi, idesc);
-                if (X_SUMS && wait_turn == 0) {
-                    wait_turn = turns;
-#pragma unroll 1
-                    for (uint32_t k = 0; k < kWP / kWUmmaK; ++k, adding = 1) {
-                        const uint32_t step = k * (kWUmmaK * 128 >> 4);
-                        umma_bf16_ss_sel(tmem_base + BN, a0 + step, hi, ones_lo, ones_hi, idesc_x, adding);
-                    }
-                }
-                if constexpr (X_SUMS) --wait_turn;
                 umma_commit(done);
             }
             if (ok) umma_commit(&ctl->tmem_full);
         }
     } else {
         const int quarter = warp & 3;
+        if (adds) {
+            // two warps per 64-channel slice, half of the pixels each; a lane has two channels, a row is 128 bytes
+            const int slice = quarter >> 1, half = quarter & 1;
+            float lo = 0.f, hi = 0.f;
+            auto add_rows = [&](auto half_tag, uint32_t tile) {
+                constexpr bool H = decltype(half_tag)::value;
+#pragma unroll 8
+                for (int r = 0; r < 32; ++r) {
+                    uint32_t u;
+                    asm volatile("ld.shared.u32 %0, [%1];" : "=r"(u) : "r"(tile + (uint32_t)r * 128u + (((uint32_t)(lane >> 2) ^ (r & 7)) << 4)));
+                    float a, b;
+                    unpack2_t<H>(u, a, b);
+                    lo += a;
+                    hi += b;
+                }
+            };
+            const uint32_t first = tiles0 + (uint32_t)slice * kChunkBytes + (uint32_t)half * 32u * 128u + (uint32_t)(lane & 3) * 4u;
+            uint32_t at = first, sb2 = 0, ph2 = 0;
+            bool fine = true;
+            for (int kb = 0; kb < num_kb && fine; ++kb) {
+                fine = __all_sync(0xffffffffu, mbar_wait_bounded(full0 + sb2, ph2, abort_flag));
+                if (!fine) break;
+                if (slice < a_chunks) { if (g.f16) add_rows(std::true_type{}, at); else add_rows(std::false_type{}, at); }
+                __syncwarp();
+                if (lane == 0) mbar_arrive(empty0 + sb2);
+                sb2 += 8; at += kStageBytes;
+                if (sb2 == sb_end) { sb2 = 0; at = first; ph2 ^= 1u; }
+            }
+            const int k = k0 + slice * 64 + 2 * lane;
+            if (slice < a_chunks) *(float2 *)(bsum + ((size_t)blockIdx.z * 2 + half) * g.kdim + k) = make_float2(lo, hi);
+        }
         const bool ok = __all_sync(0xffffffffu, mbar_wait_bounded(&ctl->tmem_full, 0, abort_flag));
         if (!ok && lane == 0) { atomicOr(err, ERRW_TIMEOUT); ctl->abort_flag = 1; }
         // The adding kernel is let go only here: its blocks, waiting for this grid, would take the shared memory that the
@@ -273,13 +286,6 @@ __global__ void __launch_bounds__(kWThreads) umma_wgrad_kernel(const __grid_cons
             float *orow = g.blockdiag
                               ? partials + (((size_t)blockIdx.z * gridDim.y + blockIdx.y) * g.kdim + (row_ok ? k : 0)) * 64
                               : partials + ((size_t)blockIdx.z * g.kdim + (row_ok ? k : 0)) * g.c_out + n0;
-            if (adds) {                                    // a row of the accumulator is a k, its columns are the same
-                uint32_t v[16];
-                tmem_ld_32x16(tmem_base + BN + ((uint32_t)(quarter * 32) << 16), v);
-                tmem_ld_wait();
-                // (0 where this CTA's turn never came)
-                if (row_ok) bsum[((size_t)blockIdx.z * turns + turn) * g.kdim + k] = turn < num_kb ? __uint_as_float(v[0]) : 0.f;
-            }
 #pragma unroll 1
             for (int c0 = 0; c0 < BN; c0 += 32) {
                 if (n0 + c0 >= g.c_out) break;
@@ -305,7 +311,7 @@ __global__ void __launch_bounds__(kWThreads) umma_wgrad_kernel(const __grid_cons
     }
     tc_fence_before_sync();
     __syncthreads();
-    if (warp == 1) tmem_dealloc(tmem_base, X_SUMS ? 2 * BN : BN);
+    if (warp == 1) tmem_dealloc(tmem_base, BN);
 }
 
 bool grouped_bd_eligible(const Problem &pb) {
@@ -334,11 +340,6 @@ static int stem_wgrad_bn(const Problem &pb) { return pb.c_out >= 256 ? 256 : wgr
 static long long wgrad_k_slices(const Problem &pb) { return (pb.groups > 1 ? (long long)pb.kh * pb.kw * 64 : pb.kdim) / 64; }
 static long long wgrad_tiles(const Problem &pb, int bn, bool ones_slice) {
     return (wgrad_k_slices(pb) + (ones_slice ? 2 : 1)) / 2 * ((pb.c_out + bn - 1) / bn);
-}
-
-int umma_wgrad_x_sum_rows(const Problem &pb) {
-    const int n = (pb.c_out + wgrad_bn(pb) - 1) / wgrad_bn(pb);
-    return n < kMaxTurns ? n : kMaxTurns;
 }
 
 // The slice count minimises  rounds over the resident slots x (pixels per slice + a fixed cost per
@@ -388,14 +389,14 @@ template <int BN, bool X_SUMS = false>
 static cudaError_t launch_w(const CUtensorMap &tx, const CUtensorMap &tdz, WgradGemm g, const UmmaWgradPlan &pl,
                             const Problem &pb, float *partials, float *bsum, int *err, cudaStream_t st,
                             unsigned int *counters = nullptr, int ncounters = 0) {
+    g.by_wo = FastDiv((uint32_t)g.wo); g.by_ho = FastDiv((uint32_t)g.ho); g.by_ci = FastDiv((uint32_t)g.c_in); g.by_tw = FastDiv((uint32_t)g.taps_w);
     constexpr size_t stage = 2 * kChunkBytes + (BN / 64) * kChunkBytes;
     int stages = BN == 128 ? 3 : 4;                    // 128-wide: 3 x 32 KB, so that two CTAs share an SM
     const long long max_kb = (pl.per_split + kWP - 1) / kWP;
     if (stages > max_kb) stages = (int)max_kb;
     g.stages = stages;
-    size_t smem = stages * stage + 1024 + kOnesBytes + sizeof(WgradSmemCtl);
-    const int columns = X_SUMS ? 2 * BN : BN;      // no more CTAs than there is tensor memory for
-    const size_t floor_smem = (size_t)(228 * 1024) / (512 / columns + 1) + 1024;
+    size_t smem = stages * stage + 1024 + sizeof(WgradSmemCtl);
+    const size_t floor_smem = (size_t)(228 * 1024) / (512 / BN + 1) + 1024;
     if (smem < floor_smem) smem = floor_smem;
     static PerDevice attr_done;
     if (cudaError_t e = max_dynamic_smem_once(umma_wgrad_kernel<BN, X_SUMS>, 210 * 1024, &attr_done); e != cudaSuccess) return e;
