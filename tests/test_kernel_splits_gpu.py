@@ -1,0 +1,75 @@
+"""Sizes at which the splits of the depthwise, stem, adding and transposed kernels change, against the fp64 oracle with the
+tolerances and per-element bounds of parity.py."""
+import ctypes
+
+import pytest
+
+import parity
+from paper_2305_11624_b200 import inputs as I
+
+pytestmark = pytest.mark.gpu
+
+L = I.LayerSpec
+SPECS = [
+    # depthwise above 256 channels: two parts of different sizes, parts that end inside a sector, more parts than row strips,
+    # the widest multiple of 8, a strip that ends inside a thread's columns
+    L("dw_264", 2, 264, 9, 11, 264, 3, 3, pad=1, groups=264, bias=True),
+    L("dw_320", 3, 320, 13, 37, 320, 3, 3, pad=1, groups=320, dtype="f16"),
+    L("dw_520", 1, 520, 6, 10, 520, 3, 3, pad=0, groups=520), L("dw_1032", 1, 1032, 5, 9, 1032, 3, 3, pad=2, groups=1032),
+    # stem rows that start anywhere: odd and even widths off a multiple of 8, the widest the input gradient's kernel takes and
+    # one more, one to four channels, 128 output channels, images smaller than a chunk of rows
+    L("stem_36", 2, 3, 46, 36, 64, 7, 7, stride=2, pad=3), L("stem_35", 3, 3, 33, 35, 64, 7, 7, stride=2, pad=3, dtype="f16"),
+    L("stem_253", 1, 3, 15, 253, 64, 7, 7, stride=2, pad=3, bias=True), L("stem_255", 1, 3, 14, 255, 64, 7, 7, stride=2, pad=3),
+    L("stem_c1", 2, 1, 21, 19, 64, 7, 7, stride=2, pad=3), L("stem_c2_k5", 2, 2, 22, 23, 64, 5, 5, stride=2, pad=2, dtype="f16"),
+    L("stem_c4", 2, 4, 25, 27, 64, 7, 7, stride=2, pad=3), L("stem_o128", 2, 3, 19, 21, 128, 7, 7, stride=2, pad=3),
+    L("stem_small", 70, 3, 9, 10, 64, 7, 7, stride=2, pad=3, dtype="f16"),
+    # adding the slices of a weight gradient: one block per channel, clusters of two, four and eight; spans that end early; a
+    # slice group per thread and many
+    L("rows_1", 2, 64, 6, 7, 2048, 1, 1), L("rows_2", 2, 192, 9, 9, 320, 1, 1, bias=True),
+    L("rows_4", 3, 128, 14, 15, 192, 1, 1, dtype="f16"), L("rows_8", 9, 64, 30, 31, 64, 3, 3, pad=1),
+    L("rows_k5", 4, 64, 12, 13, 64, 5, 5, pad=2),
+    # dense epilogue: output channels that end inside a 64-column chunk, a last tile of one pixel
+    L("epi_72", 3, 64, 7, 19, 72, 3, 3, pad=1, bias=True), L("epi_200", 43, 64, 3, 1, 200, 1, 1, dtype="f16"),
+]
+
+
+@pytest.mark.parametrize("spec", SPECS, ids=lambda s: s.name)
+def test_tune_block(spec):
+    t = parity.make_inputs(spec, 78)
+    ref = parity.oracle_tune(spec, t)
+    got = parity.run_tune_gpu(spec, t, deferred=True)
+    parity.compare(got, ref, parity.TOL[spec.dtype], parity.TUNE_OUTPUTS, spec.name, dtype=spec.dtype)
+
+
+# (dtype, n, c_in, h, w, c_out, k, stride, pad): dZ summed inside the weight gradient where the kernel is the stride (one tile of
+# channels and several that take turns, more than eight of them, slices shorter than the turns, 3 x 3, 1 x 1), by the kernel of
+# its own where the windows overlap
+TCONV = [("bf16", 3, 64, 5, 7, 64, 2, 2, 0), ("f16", 2, 256, 20, 13, 128, 2, 2, 0), ("bf16", 1, 1216, 3, 5, 64, 2, 2, 0),
+         ("bf16", 2, 128, 7, 9, 64, 3, 3, 0), ("f16", 2, 192, 9, 8, 64, 1, 1, 0), ("bf16", 2, 128, 9, 7, 64, 3, 2, 1)]
+
+
+@pytest.mark.parametrize("case", TCONV, ids=lambda c: "%s_c%d_k%d_s%d" % (c[0], c[2], c[6], c[7]))
+def test_transposed_block(case):
+    import test_tconv
+    dtype, n, ci, h, w, co, k, st, pad = case
+    test_tconv.test_library_matches_the_oracle((dtype, n, ci, h, w, co, k, st, pad, 1, 1, True))
+
+
+def test_descriptors_by_reference():
+    """The calls take a descriptor as it is, by reference and by pointer, and refuse anything else."""
+    import torch
+    from paper_2305_11624_b200 import convbn as C
+    from paper_2305_11624_b200.harness import Block
+    blk = Block(L("ref", 2, 64, 6, 7, 64, 1, 1), modes=("tune",))
+    blk.randomize(5)
+    outs = []
+    for desc in (blk.desc, ctypes.byref(blk.desc), ctypes.pointer(blk.desc)):
+        blk.z.fill_(0)
+        C.convbn_tune_fwd(desc, blk.x, blk.w, None, blk.gamma, blk.beta, blk.mu_hat, blk.var_hat, blk.z, blk.saved,
+                          blk.workspace.data_ptr(), blk.workspace.nbytes, torch.cuda.current_stream())
+        outs.append(blk.z.clone())
+    assert torch.equal(outs[0], outs[1]) and torch.equal(outs[0], outs[2])
+    with pytest.raises(TypeError):
+        C.convbn_tune_fwd(b"short", blk.x, blk.w, None, blk.gamma, blk.beta, blk.mu_hat, blk.var_hat, blk.z, blk.saved, blk.workspace)
+    with pytest.raises(C.ConvBNError):
+        C.convbn_tune_fwd(None, blk.x, blk.w, None, blk.gamma, blk.beta, blk.mu_hat, blk.var_hat, blk.z, blk.saved, blk.workspace)
