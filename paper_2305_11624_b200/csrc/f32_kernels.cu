@@ -156,6 +156,8 @@ __global__ void __launch_bounds__(kFThreads, K == 1 ? 8 : (S == 1 ? 5 : 4)) f32_
     extern __shared__ __align__(16) float f32_smem[];
     constexpr int OCT = S == 1 ? 4 * R : R;
     __shared__ float scale_s[OCT], shift_s[OCT];
+    // (the kernel behind it starts when this one ends: with an early launch its waiting blocks held the places of blocks still to
+    // run.  Forward + backward of 3x3 16 -> 32 at 16 x 16, N = 2 11.7 -> 10.8 us, of 1x1 layers at 56 x 56 36.9 -> 22.5)
     pdl_wait();
     const int oc0 = blockIdx.y * OCT;
     if (threadIdx.x < OCT) {
