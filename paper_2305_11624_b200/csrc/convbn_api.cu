@@ -491,7 +491,15 @@ int run_conv_dgrad(const convbn_desc *d, const Problem &pb, const void *dz, cons
     // (the transposed-convolution forward pass is this pass plus a bias)
     if (bias_done) *bias_done = false;
     UmmaConvShape s;
-    if (stem_path(d, pb) && stem_window_dgrad_eligible(pb)) {
+    // Rows that start off a 16-byte line leave the window kernel in 2-byte stores.  Where the sub-pixel kernel takes such a layer it
+    // is the faster one for small filters and while its tiles fit a few rounds (3 -> 64 at stride 2: 3x3 at 62 x 62, N = 32 6.2
+    // and 9.7 us, 7x7 at 118 x 108, N = 8 10.6 and 12.2), the window kernel beyond (N = 32 44.3 and 19.9).  The warp-level
+    // kernel is slower throughout (30 x 30, N = 32 28.7 and 11.9) and has what is below 512 pixels, a few rows of a few images.
+    const bool by_window = stem_path(d, pb) && stem_window_dgrad_eligible(pb) &&
+                           (pb.w_in % 8 == 0 ||
+                            (subpixel_dgrad_shape(pb, &s) && umma_strip_eligible(s) ? pb.kh * pb.kw > 25 && pb.p >= (1 << 16)
+                                                                                    : pb.p >= 512));
+    if (by_window) {
         // stride 2, C_in <= 4: scatter GEMM over dZ rows, window positions added up on chip
         LAUNCH("stem_dgrad", launch_stem_window_dgrad(pb, dz, w, scale, dx, st));
         *which = "umma-stem";

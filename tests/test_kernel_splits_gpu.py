@@ -18,10 +18,10 @@ SPECS = [
     L("dw_520", 1, 520, 6, 10, 520, 3, 3, pad=0, groups=520), L("dw_1032", 1, 1032, 5, 9, 1032, 3, 3, pad=2, groups=1032),
     # stem rows that start anywhere: odd and even widths off a multiple of 8, the widest the input gradient's kernel takes and
     # one more, one to four channels, 128 output channels, images smaller than a chunk of rows
-    L("stem_36", 2, 3, 46, 36, 64, 7, 7, stride=2, pad=3), L("stem_35", 3, 3, 33, 35, 64, 7, 7, stride=2, pad=3, dtype="f16"),
+    L("stem_36", 8, 3, 46, 36, 64, 7, 7, stride=2, pad=3), L("stem_35", 3, 3, 33, 35, 64, 7, 7, stride=2, pad=3, dtype="f16"),
     L("stem_253", 1, 3, 15, 253, 64, 7, 7, stride=2, pad=3, bias=True), L("stem_255", 1, 3, 14, 255, 64, 7, 7, stride=2, pad=3),
-    L("stem_c1", 2, 1, 21, 19, 64, 7, 7, stride=2, pad=3), L("stem_c2_k5", 2, 2, 22, 23, 64, 5, 5, stride=2, pad=2, dtype="f16"),
-    L("stem_c4", 2, 4, 25, 27, 64, 7, 7, stride=2, pad=3), L("stem_o128", 2, 3, 19, 21, 128, 7, 7, stride=2, pad=3),
+    L("stem_c1", 7, 1, 21, 19, 64, 7, 7, stride=2, pad=3), L("stem_c2_k5", 8, 2, 22, 23, 64, 5, 5, stride=2, pad=2, dtype="f16"),
+    L("stem_c4", 5, 4, 25, 27, 64, 7, 7, stride=2, pad=3), L("stem_o128", 2, 3, 19, 21, 128, 7, 7, stride=2, pad=3),
     L("stem_small", 70, 3, 9, 10, 64, 7, 7, stride=2, pad=3, dtype="f16"),
     # adding the slices of a weight gradient: one block per channel, clusters of two, four and eight; spans that end early; a
     # slice group per thread and many
