@@ -135,6 +135,10 @@ __device__ __forceinline__ void cluster_sync_all() {
     asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
     asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
 }
+// The two halves, where work fits between them: the CTAs of a cluster start together but not at one instant, and none may touch
+// another's shared memory before that one is known to run.  (No data is handed over: the arrival orders no writes.)
+__device__ __forceinline__ void cluster_arrive_started() { asm volatile("barrier.cluster.arrive.relaxed.aligned;" ::: "memory"); }
+__device__ __forceinline__ void cluster_wait_started() { asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory"); }
 // Cluster address of CTA `rank`'s copy of a shared-memory object of this CTA.
 template <class P>
 __device__ __forceinline__ uint32_t cluster_addr(P p, uint32_t rank) {

@@ -473,6 +473,7 @@ __global__ void __launch_bounds__(kRowsMaxThreads) wgrad_rows_kernel(int c_out, 
     const int rank = CL > 1 ? (int)cluster_rank() : 0, co = blockIdx.x / CL;
     const int z = threadIdx.x / VL, l = threadIdx.x - z * VL;        // (z >= SL: threads that fill up the last warp)
     const size_t slice = (size_t)c_out * kdim, row = (size_t)co * kdim;
+    if (CL > 1 && need_sums) cluster_arrive_started();
     pdl_wait();
     pdl_launch_dependents();
     const float s = vec3 ? vec3[co] : 1.f;
@@ -541,7 +542,11 @@ __global__ void __launch_bounds__(kRowsMaxThreads) wgrad_rows_kernel(int c_out, 
         for (int o = kRowsMaxThreads / 64; o > 0; o >>= 1) { dot += __shfl_xor_sync(0xffffffffu, dot, o); ds += __shfl_xor_sync(0xffffffffu, ds, o); }
     }
     if constexpr (CL > 1) {
+        // the first block has started (a block whose span lies past the row's end comes here at once); then its `dots` may be
+        // written, and the second meeting says that all are there
+        cluster_wait_started();
         if (threadIdx.x == 0) st_cluster_f32(cluster_addr(&dots[rank], 0), dot);
+        __syncwarp();
         cluster_sync_all();
     }
     if (threadIdx.x || rank) return;

@@ -41,6 +41,30 @@ def test_tune_block(spec):
     parity.compare(got, ref, parity.TOL[spec.dtype], parity.TUNE_OUTPUTS, spec.name, dtype=spec.dtype)
 
 
+# rows of 48, 80 and 144 vectors in clusters of four, eight and eight blocks: the last one, three and two have no columns and go
+# straight to the exchange of the dot products
+@pytest.mark.parametrize("c_in,k", [(192, 1), (320, 1), (64, 3)], ids=["row192", "row320", "row576"])
+def test_clusters_with_blocks_beyond_the_row(c_in, k):
+    """Every block's part of the dot product arrives: dgamma matches the oracle, and is the same in every one of many runs."""
+    import torch
+    from paper_2305_11624_b200 import convbn as C
+    from paper_2305_11624_b200.harness import Block
+    spec = L("clusters", 3, c_in, 11, 12, 64, k, k, pad=k // 2)
+    t = parity.make_inputs(spec, 79)
+    parity.compare(parity.run_tune_gpu(spec, t, deferred=True), parity.oracle_tune(spec, t), parity.TOL["bf16"],
+                   parity.TUNE_OUTPUTS, spec.name, dtype="bf16")
+    blk = Block(spec, modes=("tune",))
+    blk.load(t)
+    blk.tune_fwd()
+    seen = torch.empty(200, 64, device=blk.device)
+    for i in range(200):
+        blk.dgamma.fill_(float("nan"))
+        blk.tune_bwd_weight()
+        seen[i].copy_(blk.dgamma)
+    C.convbn_check()
+    assert bool((seen == seen[0]).all())
+
+
 # (dtype, n, c_in, h, w, c_out, k, stride, pad): dZ summed inside the weight gradient where the kernel is the stride (one tile of
 # channels and several that take turns, more than eight of them, slices shorter than the turns, 3 x 3, 1 x 1), by the kernel of
 # its own where the windows overlap
