@@ -114,14 +114,15 @@ __global__ void __launch_bounds__(256) tconv_param_epilogue_kernel(int c_out, in
     }
 }
 
-// Block (bx, by): weight columns k = (tap, co) [32 bx, +32) x input channels [8 by, +8), one output channel group since
-// 32 divides C_out.  Thread (l = four columns, ci, z = slice group) adds slices z, z + 8, ... of part[split][C_in][k], four
-// loads in flight; the groups are added in halves through shared memory.  The last block of a group of 32
+// Block (bx, by): weight columns k = (tap, co) [32 bx, +32) x input channels [64 / Z by, + 64 / Z), one output channel group
+// since 32 divides C_out.  Thread (l = four columns, ci, z = slice group) adds slices z, z + Z, ... of part[split][C_in][k], four
+// loads in flight; the Z groups are added in halves through shared memory.  The last block of a group of 32
 // output channels (a counter) adds the dot products and the sums of dZ in fixed order.  Bound by the latency of the reads of
 // the partials (L2): 256 -> 128 channels, 2 x 2, 29 slices: 15 MB.  A thread per weight and all its slices (128 blocks of
 // 1024 threads, four bytes a load) took 15 us; with the sum, the scale and the per-channel sums in kernels of their own the
-// same work took 87 us.
-constexpr int kTeCi = 8, kTeSlices = 8, kTeThreads = 8 * kTeCi * kTeSlices;
+// same work took 87 us.  Z follows the slices (see the launch).
+constexpr int kTeThreads = 512;
+template <int Z>
 __global__ void __launch_bounds__(kTeThreads) tconv_wgrad_epilogue_kernel(int c_in, int c_out, int kdim, const float *__restrict__ part,
                                                                           int splits, const __nv_bfloat16 *__restrict__ w,
                                                                           const float *__restrict__ vec3, const float *__restrict__ b,
@@ -130,35 +131,38 @@ __global__ void __launch_bounds__(kTeThreads) tconv_wgrad_epilogue_kernel(int c_
                                                                           unsigned int *__restrict__ counters, float *__restrict__ dw,
                                                                           float *__restrict__ db, float *__restrict__ dgamma,
                                                                           float *__restrict__ dbeta, int f16) {
-    __shared__ float4 red[kTeThreads];
+    constexpr int CI = 64 / Z;
+    __shared__ float4 red[Z > 1 ? kTeThreads : 1];
     __shared__ float tile[kTeThreads / 32][33], sums[kTeThreads / 32][33];
     __shared__ int is_last;
     pdl_wait();
     pdl_launch_dependents();
-    const int tid = threadIdx.x, l = tid & 7, ci = (tid >> 3) & (kTeCi - 1), z = tid / (8 * kTeCi);
-    const int k0 = blockIdx.x * 32, ci0 = blockIdx.y * kTeCi, co0 = k0 % c_out;    // (the longer dimension is the unbounded one)
+    const int tid = threadIdx.x, l = tid & 7, ci = (tid >> 3) & (CI - 1), z = tid / (8 * CI);
+    const int k0 = blockIdx.x * 32, ci0 = blockIdx.y * CI, co0 = k0 % c_out;    // (the longer dimension is the unbounded one)
     const size_t slice = (size_t)kdim * c_in, at = (size_t)(ci0 + ci) * kdim + k0 + 4 * l;
     float4 a = make_float4(0.f, 0.f, 0.f, 0.f);
-    for (int sp = z; sp < splits; sp += 4 * kTeSlices) {
+    for (int sp = z; sp < splits; sp += 4 * Z) {
         float4 q[4];
 #pragma unroll
         for (int u = 0; u < 4; ++u)
-            q[u] = sp + u * kTeSlices < splits ? __ldcg((const float4 *)(part + (size_t)(sp + u * kTeSlices) * slice + at))
-                                               : make_float4(0.f, 0.f, 0.f, 0.f);
+            q[u] = sp + u * Z < splits ? __ldcg((const float4 *)(part + (size_t)(sp + u * Z) * slice + at))
+                                       : make_float4(0.f, 0.f, 0.f, 0.f);
 #pragma unroll
         for (int u = 0; u < 4; ++u) { a.x += q[u].x; a.y += q[u].y; a.z += q[u].z; a.w += q[u].w; }
     }
-    red[tid] = a;
+    if constexpr (Z > 1) {
+        red[tid] = a;
 #pragma unroll
-    for (int h = kTeSlices / 2; h > 0; h /= 2) {
-        __syncthreads();
-        if (z < h) {
-            const float4 o = red[tid + h * 8 * kTeCi];
-            a.x += o.x; a.y += o.y; a.z += o.z; a.w += o.w;
-            red[tid] = a;
+        for (int h = Z / 2; h > 0; h /= 2) {
+            __syncthreads();
+            if (z < h) {
+                const float4 o = red[tid + h * 8 * CI];
+                a.x += o.x; a.y += o.y; a.z += o.z; a.w += o.w;
+                red[tid] = a;
+            }
         }
     }
-    if (z == 0) {                                       // two warps: input channels 0-3 and 4-7
+    if (z == 0) {                                       // CI / 4 warps: four input channels each
         const uint2 wq = *(const uint2 *)(w + at);
         const float4 s = *(const float4 *)(vec3 + co0 + 4 * l);
         *(float4 *)(dw + at) = make_float4(s.x * a.x, s.y * a.y, s.z * a.z, s.w * a.w);
@@ -172,7 +176,12 @@ __global__ void __launch_bounds__(kTeThreads) tconv_wgrad_epilogue_kernel(int c_
         }
     }
     __syncthreads();
-    if (tid < 32) dotpart[(size_t)blockIdx.y * kdim + k0 + tid] = tile[0][tid] + tile[1][tid];
+    if (tid < 32) {
+        float d = tile[0][tid];
+#pragma unroll
+        for (int i = 1; i < CI / 4; ++i) d += tile[i][tid];
+        dotpart[(size_t)blockIdx.y * kdim + k0 + tid] = d;
+    }
     __syncthreads();
     if (tid == 0) {
         __threadfence();
@@ -234,11 +243,26 @@ cudaError_t launch_tconv_wgrad_epilogue(int c_in, int c_out, int taps, const flo
                                         const float *vec3, const float *b, const float *mean, const float *bsum,
                                         int bsplits, float *dotpart, unsigned int *counters, float *dw, float *db,
                                         float *dgamma, float *dbeta, cudaStream_t st) {
-    static PerDevice carve;
-    prefer_max_shared_once(tconv_wgrad_epilogue_kernel, &carve);
-    return launch_pdl(tconv_wgrad_epilogue_kernel, dim3(taps * c_out / 32, c_in / kTeCi), dim3(kTeThreads), 0, st, c_in, c_out,
-                      taps * c_out, part, splits, (const __nv_bfloat16 *)w, vec3, b, mean, bsum, bsplits, dotpart, counters,
-                      dw, db, dgamma, dbeta, call_f16());
+    // One batch of loads per thread: four slices a group, up to eight groups.  More groups than that leave threads idle, and what a
+    // block does beside its loads (sums, counter, the last block's walk over a row of dot products per block) is then paid for
+    // fewer weights: with eight groups always, forward + backward of 1024 -> 512, 14 x 14, N = 2 (three slices) took 86.9 us at
+    // 2 x 2 and 431 at 4 x 4, with this rule 33.5 and 195.  Few weights spread over more blocks while there are slices to share.
+    int z = 1;
+    while (z < 8 && z * 4 < splits) z *= 2;
+    while (z < 8 && z < splits && (long long)(taps * (long long)c_out / 32) * (c_in / 64) * z < 2LL * device_sm_count()) z *= 2;
+    while (z > 1 && c_in / 64 * (long long)z > 65535) z /= 2;
+    auto go = [&](auto groups) {
+        constexpr int Z = decltype(groups)::value;
+        static PerDevice carve;
+        prefer_max_shared_once(tconv_wgrad_epilogue_kernel<Z>, &carve);
+        return launch_pdl(tconv_wgrad_epilogue_kernel<Z>, dim3(taps * c_out / 32, c_in / 64 * Z), dim3(kTeThreads), 0, st, c_in,
+                          c_out, taps * c_out, part, splits, (const __nv_bfloat16 *)w, vec3, b, mean, bsum, bsplits, dotpart,
+                          counters, dw, db, dgamma, dbeta, call_f16());
+    };
+    if (z == 1) return go(std::integral_constant<int, 1>());
+    if (z == 2) return go(std::integral_constant<int, 2>());
+    if (z == 4) return go(std::integral_constant<int, 4>());
+    return go(std::integral_constant<int, 8>());
 }
 
 cudaError_t launch_tconv_rescale(int dtype, bool nhwc, long long count, int taps, int cig, int cog, const void *w,

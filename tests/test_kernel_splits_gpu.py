@@ -69,7 +69,9 @@ def test_clusters_with_blocks_beyond_the_row(c_in, k):
 # channels and several that take turns, more than eight of them, slices shorter than the turns, 3 x 3, 1 x 1), by the kernel of
 # its own where the windows overlap
 TCONV = [("bf16", 3, 64, 5, 7, 64, 2, 2, 0), ("f16", 2, 256, 20, 13, 128, 2, 2, 0), ("bf16", 1, 1216, 3, 5, 64, 2, 2, 0),
-         ("bf16", 2, 128, 7, 9, 64, 3, 3, 0), ("f16", 2, 192, 9, 8, 64, 1, 1, 0), ("bf16", 2, 128, 9, 7, 64, 3, 2, 1)]
+         ("bf16", 2, 128, 7, 9, 64, 3, 3, 0), ("f16", 2, 192, 9, 8, 64, 1, 1, 0), ("bf16", 2, 128, 9, 7, 64, 3, 2, 1),
+         # the finish with one group of slices (three slices, many weights), two (six slices) and eight (more than 16)
+         ("bf16", 1, 512, 20, 31, 512, 2, 2, 0), ("f16", 1, 192, 38, 39, 512, 2, 2, 0), ("bf16", 5, 64, 33, 30, 64, 2, 2, 0)]
 
 
 @pytest.mark.parametrize("case", TCONV, ids=lambda c: "%s_c%d_k%d_s%d" % (c[0], c[2], c[6], c[7]))
