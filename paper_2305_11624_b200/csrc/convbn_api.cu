@@ -1468,34 +1468,37 @@ int convbn_tconv_tune_bwd(const convbn_desc *desc, const void *dz, const void *x
     unsigned int *counters = (unsigned int *)at(workspace, v.off_count);
     // dX gathers dZ through omega' (re-formed from omega and the saved scale, Sec. 3.4): the forward pass of that
     // convolution, without a bias.  domega' contracts X with windows of dZ: that convolution's weight gradient with the
-    // two tensors exchanged.  The two passes share nothing they write and run side by side, the longer one, the parameters', on the
-    // caller's stream (256 -> 128 at 56 x 56, N = 8, 2 x 2: forward + backward 49.7 us, 58.0 the other way).
-    return side_by_side(
-        st,
-        [&](cudaStream_t st) -> int {
-            const char *which = nullptr;
-            LAUNCH("tconv_rescale", launch_tconv_rescale(desc->dtype, nhwc, (long long)v.wcount, taps, cig, cog, w, vec3, wf, st));
-            return run_conv_fwd(&v.conv, v.pb, dz, wf, nullptr, dx, v.fwd, inner, st, &which);
-        },
-        [&]() -> int {
-            const char *which = nullptr;
-            if (!v.gemm_sums)
-                LAUNCH("channel_sum", launch_channel_sum_partial(v.sum_pb, desc->dtype, desc->layout, dz, bsum, v.bsplits, st));
-            if (v.bwd.umma_wgrad) {
-                float *partials = (float *)at(inner_b, v.bwd.partials);
-                LAUNCH("umma_wgrad", launch_umma_wgrad(v.pb, v.bwd.uw, x, dz, partials, bsum, st, counters, desc->c_out / 32,
-                                                       v.sums));
-                LAUNCH("tconv_epilogue", launch_tconv_wgrad_epilogue(desc->c_in, desc->c_out, taps, partials, v.bwd.uw.splits, w,
-                                                                     vec3, b, run_mean, bsum, v.bsplits, dwp, counters, dw, db,
-                                                                     dgamma, dbeta, st));
-                return CONVBN_OK;
-            }
-            CK(run_param_grads(&v.conv, v.pb, v.bwd, x, dz, w, nullptr, nullptr, nullptr, dwp, nullptr, nullptr, nullptr, inner_b,
-                               st, &which));
-            LAUNCH("tconv_epilogue", launch_tconv_param_epilogue(desc->dtype, nhwc, desc->c_out, taps, cig, cog, dwp, w, vec3, b,
-                                                                 run_mean, bsum, v.bsplits, dw, db, dgamma, dbeta, st));
+    // two tensors exchanged.  The two passes share nothing they write and run side by side.
+    auto data = [&](cudaStream_t st) -> int {
+        const char *which = nullptr;
+        LAUNCH("tconv_rescale", launch_tconv_rescale(desc->dtype, nhwc, (long long)v.wcount, taps, cig, cog, w, vec3, wf, st));
+        return run_conv_fwd(&v.conv, v.pb, dz, wf, nullptr, dx, v.fwd, inner, st, &which);
+    };
+    auto params = [&](cudaStream_t st) -> int {
+        const char *which = nullptr;
+        if (!v.gemm_sums)
+            LAUNCH("channel_sum", launch_channel_sum_partial(v.sum_pb, desc->dtype, desc->layout, dz, bsum, v.bsplits, st));
+        if (v.bwd.umma_wgrad) {
+            float *partials = (float *)at(inner_b, v.bwd.partials);
+            LAUNCH("umma_wgrad", launch_umma_wgrad(v.pb, v.bwd.uw, x, dz, partials, bsum, st, counters, desc->c_out / 32,
+                                                   v.sums));
+            LAUNCH("tconv_epilogue", launch_tconv_wgrad_epilogue(desc->c_in, desc->c_out, taps, partials, v.bwd.uw.splits, w,
+                                                                 vec3, b, run_mean, bsum, v.bsplits, dwp, counters, dw, db,
+                                                                 dgamma, dbeta, st));
             return CONVBN_OK;
-        });
+        }
+        CK(run_param_grads(&v.conv, v.pb, v.bwd, x, dz, w, nullptr, nullptr, nullptr, dwp, nullptr, nullptr, nullptr, inner_b,
+                           st, &which));
+        LAUNCH("tconv_epilogue", launch_tconv_param_epilogue(desc->dtype, nhwc, desc->c_out, taps, cig, cog, dwp, w, vec3, b,
+                                                             run_mean, bsum, v.bsplits, dw, db, dgamma, dbeta, st));
+        return CONVBN_OK;
+    };
+    // The longer pass belongs on the caller's stream.  That is the parameters' (256 -> 128 at 56 x 56, N = 8, 2 x 2: forward +
+    // backward 49.6 us, 58.5 the other way), but not where a sum of dZ goes before its GEMM (overlapping windows) and there are
+    // many pixels: the other pass then has the GPU to itself until the sum is done (128 -> 64, 4 x 4 stride 2: 9 x 198 x 271
+    // pixels 721 and 683 us, 16 x 40 x 70 100.7 and 98.6; but 100 x 100 93.4 and 98.1, 32 x 16 x 16 even).
+    if (!v.gemm_sums && v.pb.p >= (1 << 14)) return side_by_side(st, params, [&] { return data(st); });
+    return side_by_side(st, data, [&] { return params(st); });
 }
 
 int convbn_check(void *stream) {
