@@ -23,6 +23,9 @@ SPECS = [
     L("stem_c1", 7, 1, 21, 19, 64, 7, 7, stride=2, pad=3), L("stem_c2_k5", 8, 2, 22, 23, 64, 5, 5, stride=2, pad=2, dtype="f16"),
     L("stem_c4", 5, 4, 25, 27, 64, 7, 7, stride=2, pad=3), L("stem_o128", 2, 3, 19, 21, 128, 7, 7, stride=2, pad=3),
     L("stem_small", 70, 3, 9, 10, 64, 7, 7, stride=2, pad=3, dtype="f16"),
+    # more than 32 taps on the strip kernel: dense and block-diagonal layers
+    L("taps_49", 2, 64, 20, 24, 64, 7, 7, pad=3), L("taps_81", 1, 64, 21, 20, 128, 9, 9, pad=4, dtype="f16"),
+    L("taps_49_groups", 2, 128, 19, 23, 128, 7, 7, pad=3, groups=8),
     # adding the slices of a weight gradient: one block per channel, clusters of two, four and eight; spans that end early; a
     # slice group per thread and many
     L("rows_1", 2, 64, 6, 7, 2048, 1, 1), L("rows_2", 2, 192, 9, 9, 320, 1, 1, bias=True),
