@@ -43,12 +43,13 @@ struct WinGemm {
     int relu;              // 1: max(Z, 0) is stored
 };
 
+constexpr int kWinMaxRow = 256;          // weights of an output channel (16 x 8 taps of 4 channels would be 512)
 struct WinCtl {
     uint64_t strip_full[kWinMaxStrips], strip_empty[kWinMaxStrips];
     uint64_t tmem_full[8], tmem_empty[8];
     uint32_t tmem_base;
     int abort_flag;
-    unsigned short slot_of[256];   // weight element (r, q, c) -> (K block << 8) | position in the 64-wide K row
+    unsigned short slot_of[kWinMaxRow];    // weight element (r, q, c) -> (K block << 8) | position in the 64-wide K row
 };
 
 // descriptor halves of the un-swizzled K-major window operand: LBO 16 bytes, SBO 128 bytes
@@ -701,7 +702,7 @@ struct WinPlan { bool ok = false; int R = 0, nstrips = 0, pitch = 0, kblocks = 0
 WinPlan plan_window(const Problem &pb) {
     WinPlan pl;
     if (pb.groups != 1 || pb.c_in > 4 || pb.stride_w != 2 || pb.stride_h != 2 || pb.dil_h != 1 ||
-        pb.dil_w != 1 || pb.kw > 8 || pb.kh > 16 || (pb.c_out != 64 && pb.c_out != 128) ||
+        pb.dil_w != 1 || pb.kw > 8 || pb.kh > 16 || pb.kdim > kWinMaxRow || (pb.c_out != 64 && pb.c_out != 128) ||
         pb.pad_w > 64 || pb.pad_h > 64 || pb.p >= (1LL << 30) || pb.pin >= (1LL << 30))
         return pl;
     pl.pitch = (int)(((size_t)(pb.w_in + 2 * pb.pad_w) * 8 + 15) / 16 * 16);

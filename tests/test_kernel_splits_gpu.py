@@ -26,6 +26,10 @@ SPECS = [
     # more than 32 taps on the strip kernel: dense and block-diagonal layers
     L("taps_49", 2, 64, 20, 24, 64, 7, 7, pad=3), L("taps_81", 1, 64, 21, 20, 128, 9, 9, pad=4, dtype="f16"),
     L("taps_49_groups", 2, 128, 19, 23, 128, 7, 7, pad=3, groups=8),
+    # stem filters of 257 to 512 weights per output channel, more than the window kernel's table holds, at both kinds of width; and the
+    # largest that it takes
+    L("stem_16x8", 2, 4, 31, 37, 64, 16, 8, stride=2, pad=3), L("stem_16x8_w40", 2, 4, 31, 40, 64, 16, 8, stride=2, pad=3),
+    L("stem_13x7", 2, 3, 30, 33, 64, 13, 7, stride=2, pad=3, dtype="f16"), L("stem_16x8_c2", 2, 2, 31, 37, 64, 16, 8, stride=2, pad=3),
     # adding the slices of a weight gradient: one block per channel, clusters of two, four and eight; spans that end early; a
     # slice group per thread and many
     L("rows_1", 2, 64, 6, 7, 2048, 1, 1), L("rows_2", 2, 192, 9, 9, 320, 1, 1, bias=True),
