@@ -56,11 +56,18 @@ _lib = None
 
 
 def _signatures():
-    """argtypes of entry points that take pointers: ctypes then converts plain integers itself, without an object per
-    argument (d: descriptor, p: pointer or stream, z: size, i: int, q: long long, f: double)."""
+    """argtypes of the entry points that take pointers: ctypes then converts plain integers itself, without an object per
+    argument, and to their full width (d: descriptor, p: pointer or stream, z: size, i: int, q: long long, f: double).  The
+    calls of a training step go through _binding.so here; whoever takes them from lib() gets them typed all the same."""
     kinds = {"d": ctypes.POINTER(Desc), "p": ctypes.c_void_p, "z": ctypes.c_size_t, "i": ctypes.c_int,
              "q": ctypes.c_longlong, "f": ctypes.c_double}
     table = {
+        "convbn_tune_fwd": "dppppppppppzp", "convbn_tune_bwd_data": "dpppppzp", "convbn_tune_bwd_weight": "dppppppppppp" "zp",
+        "convbn_tune_bwd": "dppppppppppppzp", "convbn_tune_bwd_begin": "dppppppppppppzp", "convbn_tune_bwd_join": "p",
+        "convbn_tune_fwd_glue": "dppppppppppipzp", "convbn_tune_bwd_glue": "dppppppppppppiipzp",
+        "convbn_tconv_tune_fwd": "dppppppppppzp", "convbn_tconv_tune_bwd": "dppppppppppppzp",
+        "convbn_eval_fwd": "dppppppppppzp", "convbn_eval_bwd": "dpppppppppppppzp",
+        "convbn_deploy_fwd": "dpppppzp", "convbn_deploy_bwd": "dpppppppzp",
         "convbn_tune_bwd_weight_noalloc": "dppppppppppp", "convbn_deploy_prepare": "dppppppppp",
         "convbn_relu": "ippqp", "convbn_add_relu": "ipppqp", "convbn_relu_bwd": "ipppqp",
         "convbn_add": "ipppqp", "convbn_workspace_bytes": "di", "convbn_saved_bytes": "di", "convbn_check": "p",

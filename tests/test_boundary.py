@@ -169,6 +169,26 @@ def test_addresses_may_be_integers_of_any_kind():
     assert e.value.status == C.EALIGN                       # `saved` is the one that is off
 
 
+def test_the_library_takes_plain_addresses_in_full_width():
+    """lib() itself, with descriptors and integer addresses as they are: an address whose lower half is zero is no NULL."""
+    d, ok, high = good(), 4096, 1 << 32
+    two = C.Desc.make(1, 8, 4, 4, 8, 3, 3, 2, 2, 1, 1)
+    lib = C.lib()
+    assert lib.convbn_tune_fwd(d, high, ok + 8, None, ok, ok, ok, ok, ok, ok, ok, 1 << 33, 0) == C.EALIGN
+    assert lib.convbn_tune_bwd_data(d, high, ok + 8, ok, ok, ok, 1 << 33, 0) == C.EALIGN
+    assert lib.convbn_tune_bwd_weight(d, high, ok, ok + 8, None, ok, ok, ok, None, ok, ok, ok, 1 << 33, 0) == C.EALIGN
+    assert lib.convbn_tune_bwd(d, high, ok, ok + 8, None, ok, ok, ok, ok, None, ok, ok, ok, 1 << 33, 0) == C.EALIGN
+    assert lib.convbn_tune_bwd_begin(d, high, ok, ok + 8, None, ok, ok, ok, ok, None, ok, ok, ok, 1 << 33, 0) == C.EALIGN
+    assert lib.convbn_tune_fwd_glue(d, high, ok + 8, None, ok, ok, ok, ok, ok, ok, None, 0, ok, 1 << 33, 0) == C.EALIGN
+    assert lib.convbn_tune_bwd_glue(d, high, ok, ok + 8, None, ok, ok, ok, ok, None, ok, ok, None, 0, 0, ok, 1 << 33, 0) == C.EALIGN
+    assert lib.convbn_eval_fwd(d, high, ok + 8, None, ok, ok, ok, ok, ok, ok, ok, 1 << 33, 0) == C.EALIGN
+    assert lib.convbn_eval_bwd(d, high, ok, ok, ok + 8, ok, ok, ok, ok, ok, None, ok, ok, ok, 1 << 33, 0) == C.EALIGN
+    assert lib.convbn_deploy_fwd(d, high, ok + 8, ok, ok, ok, 1 << 33, 0) == C.EALIGN
+    assert lib.convbn_deploy_bwd(d, high, ok, ok + 8, ok, ok, ok, ok, 1 << 33, 0) == C.EALIGN
+    assert lib.convbn_tconv_tune_fwd(two, high, ok + 8, None, ok, ok, ok, ok, ok, ok, ok, 1 << 33, 0) == C.EALIGN
+    assert lib.convbn_tconv_tune_bwd(two, high, ok, ok + 8, None, ok, ok, ok, ok, None, ok, ok, ok, 1 << 33, 0) == C.EALIGN
+
+
 def test_status_strings():
     assert C.status_string(C.OK) == "ok"
     assert "workspace" in C.status_string(C.EWORKSPACE)
