@@ -115,10 +115,16 @@ def _calls():
 
 
 def _desc(desc):
-    """A descriptor given as ctypes.byref(d) or ctypes.pointer(d)."""
-    if hasattr(desc, "_obj"):
-        return desc._obj
-    return desc.contents if isinstance(desc, ctypes.POINTER(Desc)) else desc
+    """A descriptor given in another form that a `const convbn_desc *` takes (by reference, by pointer, an array's first, a
+    structure derived from it, None), as a Desc at that address; anything else is a TypeError."""
+    if desc is None:
+        return None
+    address = ctypes.cast(ctypes.POINTER(Desc).from_param(desc), ctypes.c_void_p).value
+    if address is None:
+        return None
+    view = Desc.from_address(address)
+    view.given = desc                    # (keeps what it points into)
+    return view
 
 
 def _ptr(t):

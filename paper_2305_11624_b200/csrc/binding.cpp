@@ -76,8 +76,13 @@ bool convert(PyObject *o, T *out) {
         *out = (T)p;
         return true;
     } else {
-        const long long v = PyLong_AsLongLong(o);
-        if (v == -1 && PyErr_Occurred()) return false;
+        // (as ctypes does: integers only, and cut to the parameter's width)
+        if (!PyLong_Check(o)) {
+            PyErr_Format(PyExc_TypeError, "an integer is expected, not %.100s", Py_TYPE(o)->tp_name);
+            return false;
+        }
+        const unsigned long long v = PyLong_AsUnsignedLongLongMask(o);
+        if (v == (unsigned long long)-1 && PyErr_Occurred()) return false;
         *out = (T)v;
         return true;
     }

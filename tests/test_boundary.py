@@ -189,6 +189,35 @@ def test_the_library_takes_plain_addresses_in_full_width():
     assert lib.convbn_tconv_tune_bwd(two, high, ok, ok + 8, None, ok, ok, ok, ok, None, ok, ok, ok, 1 << 33, 0) == C.EALIGN
 
 
+def test_descriptors_in_every_form():
+    """The forms a C parameter `const convbn_desc *` takes are taken, with the bytes that they point at; others are refused."""
+    class Longer(C.Desc):
+        _fields_ = [("more", ctypes.c_int)]
+
+    bad, d = good(n=0), good()
+    longer = Longer(*[getattr(d, f) for f, _ in C.Desc._fields_], 7)
+    args = (4096, 4096, None, 4096, 4096, 4096, 4096, 4096, 4096 + 8, 4096)
+
+    def status(desc, size=1 << 30):
+        with pytest.raises(C.ConvBNError) as e:
+            C.convbn_tune_fwd(desc, *args, size, stream=0)
+        return e.value.status
+
+    good_forms = [d, ctypes.byref(d), ctypes.pointer(d), (C.Desc * 1)(d), (C.Desc * 2)(d, bad), longer, ctypes.byref(longer)]
+    assert [status(f) for f in good_forms] == [C.EALIGN] * len(good_forms)          # `saved` is off
+    second = (C.Desc * 2)(bad, d)
+    assert status(second) == C.EINVAL and status(ctypes.byref(second[0])) == C.EINVAL
+    assert status(ctypes.byref(second[0], ctypes.sizeof(C.Desc))) == C.EALIGN
+    assert status(None) == C.EINVAL and status(ctypes.POINTER(C.Desc)()) == C.EINVAL
+    for other in (bytes(d), bytearray(d), 4096, 1.0, "desc", ctypes.byref(ctypes.c_int(1))):
+        with pytest.raises(TypeError):
+            C.convbn_tune_fwd(other, *args, 1 << 30, stream=0)
+    assert status(d, (1 << 64) - 1) == C.EALIGN                                     # the largest size_t
+    for size in (1.5, "1"):
+        with pytest.raises(TypeError):
+            C.convbn_tune_fwd(d, *args, size, stream=0)
+
+
 def test_status_strings():
     assert C.status_string(C.OK) == "ok"
     assert "workspace" in C.status_string(C.EWORKSPACE)
