@@ -336,10 +336,6 @@ __global__ void __launch_bounds__(TW >= 4 ? 384 : 288, TW >= 4 ? 1 : 2) dw_tma_w
             const int rows = min(g.th, g.h_out - band * g.th);
             int steps = rows + KH - 1;
             f32x2 dzw[KH][TW][2];                              // dZ row o of the band lives in slot o % KH
-#pragma unroll
-            for (int sl = 0; sl < KH; ++sl)
-#pragma unroll
-                for (int j = 0; j < TW; ++j) dzw[sl][j][0] = dzw[sl][j][1] = 0ull;
             for (int k0 = 0; k0 < steps; k0 += KH) {
 #pragma unroll
                 for (int ph = 0; ph < KH; ++ph) {
@@ -365,19 +361,18 @@ __global__ void __launch_bounds__(TW >= 4 ? 384 : 288, TW >= 4 ? 1 : 2) dw_tma_w
                                     acc[KH * KW][0] = fma2(dzw[ph][j][0], ones, acc[KH * KW][0]);
                                     acc[KH * KW][1] = fma2(dzw[ph][j][1], ones, acc[KH * KW][1]);
                                 }
-                            } else {
-#pragma unroll
-                                for (int j = 0; j < TW; ++j) dzw[ph][j][0] = dzw[ph][j][1] = 0ull;
                             }
                             __syncwarp();
                             arrive_lane0(empty0 + slot * 8, lane);
                             ++slot;
                             slot_off += (uint32_t)g.stage_stride;
                             if (slot_off == ring_bytes) { slot = 0; slot_off = 0; par ^= 1u; }
-                            // X row k is tap row r of dZ row k - r (slot (ph - r) mod KH; zero outside the band)
+                            // X row k is tap row r of dZ row k - r (slot (ph - r) mod KH), if the band has that row (the same for
+                            // the whole block; multiplying by zeros instead made NaN of an infinite X)
 #pragma unroll
                             for (int r = 0; r < KH; ++r) {
                                 const int sl = (ph - r + KH) % KH;
+                                if ((r > 0 && k < r) || (r < KH - 1 && k - r >= rows)) continue;
 #pragma unroll
                                 for (int q = 0; q < KW; ++q)
 #pragma unroll

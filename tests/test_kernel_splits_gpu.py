@@ -2,6 +2,7 @@
 tolerances and per-element bounds of parity.py."""
 import ctypes
 
+import numpy as np
 import pytest
 
 import parity
@@ -70,6 +71,43 @@ def test_clusters_with_blocks_beyond_the_row(c_in, k):
         seen[i].copy_(blk.dgamma)
     C.convbn_check()
     assert bool((seen == seen[0]).all())
+
+
+def weight_gradient(spec, x, dz):
+    """fp64 sums of dZ X over the pixels inside the image, tap by tap: nothing is multiplied that is not in the sum."""
+    dw = np.zeros((spec.c_out, spec.c_in // spec.groups, spec.kh, spec.kw))
+    (ho, wo), st, p = dz.shape[2:], spec.stride, spec.pad
+    for r in range(spec.kh):
+        for q in range(spec.kw):
+            h = [i for i in range(ho) if 0 <= i * st + r - p < spec.h_in]
+            w = [i for i in range(wo) if 0 <= i * st + q - p < spec.w_in]
+            if h and w:
+                xs = x[:, :, h[0] * st + r - p:h[-1] * st + r - p + 1:st, w[0] * st + q - p:w[-1] * st + q - p + 1:st]
+                ds = dz[:, :, h[0]:h[-1] + 1, w[0]:w[-1] + 1]
+                dw[:, :, r, q] = (np.einsum("nohw,nchw->oc", ds, xs) if spec.groups == 1 else (ds * xs).sum((0, 2, 3))[:, None])
+    return dw
+
+
+def same_kind(got, ref, name):
+    assert np.array_equal(np.isnan(got), np.isnan(ref)) and np.array_equal(np.isinf(got), np.isinf(ref)), name
+    assert np.array_equal(np.sign(got[np.isinf(got)]), np.sign(ref[np.isinf(ref)])), name
+
+
+def test_depthwise_rows_beyond_a_band_are_not_multiplied():
+    """An infinite X, in every row of the image and so at every edge of a band: domega is infinite where the pixel is in its
+    sum, and finite elsewhere."""
+    from paper_2305_11624_b200 import convbn as C
+    spec = L("inf_dw", 2, 264, 11, 12, 264, 3, 3, pad=1, groups=264)
+    t = parity.make_inputs(spec, 80)
+    for c in range(0, 264, 2):
+        t["x"][c % 4 // 2, c, c % 11, c % 12] = -np.inf if c % 3 else np.inf
+    with np.errstate(invalid="ignore"):
+        ref = weight_gradient(spec, t["x"], t["dz"])
+        got = parity.run_tune_gpu(spec, t)["dw"]
+    C.convbn_check()
+    assert np.isinf(ref).any() and not np.isnan(ref).any()
+    s = t["gamma"] / np.sqrt(t["var_hat"] + spec.eps)
+    same_kind(got, s[:, None, None, None] * ref, spec.name)
 
 
 # (dtype, n, c_in, h, w, c_out, k, stride, pad): dZ summed inside the weight gradient where the kernel is the stride (one tile of
