@@ -268,16 +268,17 @@ __global__ void __launch_bounds__(kDgThreads) stem_window_dgrad_kernel(const __g
 #pragma unroll
                         for (int c = 0; c < C; ++c) tile[((q - 2) * 4 + c) * 128 + j] = __uint_as_float(v[4 * q + c]);
                     named_bar_sync(bar_id, 128);
-                    // padded pixel u = 2 j + b gets window position q = b + 2 t of accumulator row j - t, t = 0 .. 3
+                    // padded pixel u = 2 j + b gets window position q = b + 2 t of accumulator row j - t, t = 0 .. 3; positions from kw on
+                    // are left out (their weights are zeros, which an infinite dZ would make NaN)
 #pragma unroll
                     for (int b = 0; b < 2; ++b) {
                         const int p = 2 * j + b - g.pad_w;
 #pragma unroll
                         for (int c = 0; c < C; ++c) {
-                            float acc = __uint_as_float(v[4 * b + c]);
+                            float acc = b < g.kw ? __uint_as_float(v[4 * b + c]) : 0.f;
 #pragma unroll
                             for (int t = 1; t < 4; ++t)
-                                if (j - t >= 0) acc += tile[((b + 2 * t - 2) * 4 + c) * 128 + j - t];
+                                if (j - t >= 0 && b + 2 * t < g.kw) acc += tile[((b + 2 * t - 2) * 4 + c) * 128 + j - t];
                             if (p >= 0 && p < g.w_in) *(uint16_t *)(rbuf + ((size_t)p * C + c) * 2) = pack1_h16(acc, g.f16);
                         }
                     }

@@ -110,6 +110,23 @@ def test_depthwise_rows_beyond_a_band_are_not_multiplied():
     same_kind(got, s[:, None, None, None] * ref, spec.name)
 
 
+@pytest.mark.parametrize("kh,kw", [(7, 7), (4, 5), (2, 1), (8, 8)])
+def test_stem_input_gradient_of_infinite_values(kh, kw):
+    """dX is infinite or NaN exactly where an infinite dZ meets a weight (window kernel, an odd width)."""
+    from paper_2305_11624_b200 import convbn as C
+    spec = L("inf_stem_dx", 40, 3, 18, 21, 64, kh, kw, stride=2, pad=1)
+    t = parity.make_inputs(spec, 81)
+    t["dz"][0, 3, 2, 1] = t["dz"][5, 60, 0, 0] = t["dz"][39, 0, -1, -1] = np.inf
+    got = parity.run_tune_gpu(spec, t)
+    C.convbn_check()
+    assert got["_kernels"][1] == "umma-stem"
+    met = np.zeros(t["x"].shape, dtype=bool)
+    for n, _, i, j in np.argwhere(np.isinf(t["dz"])):
+        rows, cols = np.arange(2 * i - 1, 2 * i - 1 + kh), np.arange(2 * j - 1, 2 * j - 1 + kw)
+        met[n][np.ix_(range(3), rows[(rows >= 0) & (rows < 18)], cols[(cols >= 0) & (cols < 21)])] = True
+    assert np.array_equal(~np.isfinite(got["dx"]), met)
+
+
 # (dtype, n, c_in, h, w, c_out, k, stride, pad): dZ summed inside the weight gradient where the kernel is the stride (one tile of
 # channels and several that take turns, more than eight of them, slices shorter than the turns, 3 x 3, 1 x 1), by the kernel of
 # its own where the windows overlap
