@@ -46,7 +46,10 @@ struct WinGemm {
 constexpr int kWinMaxRow = 256;          // weights of an output channel (16 x 8 taps of 4 channels would be 512)
 struct WinCtl {
     uint64_t strip_full[kWinMaxStrips], strip_empty[kWinMaxStrips];
-    uint64_t tmem_full[8], tmem_empty[8];
+    // An accumulator's units go to the three warp groups in turn, and a warp need not be near the others (one whose pixels lie beyond
+    // the row end only passes by).  So each group has a barrier of its own per accumulator and meets every phase of it: on
+    // one barrier for all it could take the phase before last for its own, two phases having the same parity.
+    uint64_t tmem_full[kWinEpiGroups][8], tmem_empty[8];
     uint32_t tmem_base;
     int abort_flag;
     unsigned short slot_of[kWinMaxRow];    // weight element (r, q, c) -> (K block << 8) | position in the 64-wide K row
@@ -143,6 +146,7 @@ __global__ void __launch_bounds__(kWinThreads) stem_window_fwd_kernel(const __gr
                                                                      const float *__restrict__ bias, int *err) {
     extern __shared__ uint8_t smem_raw[];
     constexpr int NA = 512 / BN;                           // accumulators in tensor memory
+    static_assert(NA % kWinEpiGroups != 0 && NA % kWinIssuers == 0, "units of an accumulator: all groups in turn, one issuer");
     uint8_t *strips = (uint8_t *)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
     uint8_t *wres = strips + (size_t)g.nstrips * g.strip_bytes;          // [kblocks][BN][128 B], 128-byte swizzle
     uint8_t *staging = wres + (size_t)g.kblocks * BN * 128;              // per epilogue warp [32 rows][128 B]
@@ -159,7 +163,10 @@ __global__ void __launch_bounds__(kWinThreads) stem_window_fwd_kernel(const __gr
         if (threadIdx.x == 0) {
             CONVBN_TRACE_POINT(0);
             for (int s = 0; s < kWinMaxStrips; ++s) { mbar_init(&ctl->strip_full[s], 32 * kWinLoaders); mbar_init(&ctl->strip_empty[s], kWinIssuers); }
-            for (int s = 0; s < 8; ++s) { mbar_init(&ctl->tmem_full[s], 1); mbar_init(&ctl->tmem_empty[s], 4); }
+            for (int s = 0; s < 8; ++s) {
+                for (int e = 0; e < kWinEpiGroups; ++e) mbar_init(&ctl->tmem_full[e][s], 1);
+                mbar_init(&ctl->tmem_empty[s], 4);
+            }
             ctl->abort_flag = 0;
             fence_barrier_init();
             prefetch_tensormap(&tm_out);
@@ -310,7 +317,7 @@ __global__ void __launch_bounds__(kWinThreads) stem_window_fwd_kernel(const __gr
                             else umma_bf16_ss_halves<true>(d, a_lo, a_hi, b_lo, b_hi, idesc);
                             umma_bf16_ss_halves<true>(d, a_lo + 2u, a_hi, b_lo + 2u, b_hi, idesc);
                         }
-                        umma_commit(&ctl->tmem_full[slot]);
+                        umma_commit(&ctl->tmem_full[u % kWinEpiGroups][slot]);
                     }
                 // this issuer's share of the patch is read once its MMAs complete (arrives at once if it had none)
                 if (ok) umma_commit(&ctl->strip_empty[sb]);
@@ -320,7 +327,7 @@ __global__ void __launch_bounds__(kWinThreads) stem_window_fwd_kernel(const __gr
             if (!ok) { atomicOr(err, ERRW_TIMEOUT); ctl->abort_flag = 1; }
         }
     } else {
-        // ---------------- epilogue: unit u goes to warp group u % 4; tensor memory -> scale, shift -> bf16 ->
+        // ---------------- epilogue: unit u goes to warp group u % 3; tensor memory -> scale, shift -> bf16 ->
         // swizzled staging -> TMA store of [32 pixels][64 channels] (pixels beyond the row end are clipped)
         const int quarter = warp & 3, egroup = (warp - kWinEpiWarp0) >> 2;
         uint8_t *buf = staging + (size_t)(warp - kWinEpiWarp0) * 4096;
@@ -332,9 +339,9 @@ __global__ void __launch_bounds__(kWinThreads) stem_window_fwd_kernel(const __gr
             for (int i = 0; i < ck.rows && ok; ++i)
                 for (int cb = 0; cb < g.colblocks; ++cb, ++u) {
                     if ((int)(u % kWinEpiGroups) != egroup) continue;
-                    const uint32_t slot = u % NA, use = u / NA;
+                    const uint32_t slot = u % NA, use = u / NA / kWinEpiGroups;      // (this group's: every third, since 3 does not divide NA)
                     { CONVBN_TRACE_T0();
-                    ok = __all_sync(0xffffffffu, mbar_wait_bounded(&ctl->tmem_full[slot], use & 1u, abort_flag));
+                    ok = __all_sync(0xffffffffu, mbar_wait_bounded(&ctl->tmem_full[egroup][slot], use & 1u, abort_flag));
                     if (warp == kWinEpiWarp0 && lane == 0) CONVBN_TRACE_ACC(15); }
                     if (!ok) break;
                     tc_fence_after_sync();

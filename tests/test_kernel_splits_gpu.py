@@ -49,6 +49,30 @@ def test_tune_block(spec):
     parity.compare(got, ref, parity.TOL[spec.dtype], parity.TUNE_OUTPUTS, spec.name, dtype=spec.dtype)
 
 
+@pytest.mark.parametrize("c_out,n,h,w", [(128, 700, 18, 21), (128, 260, 30, 32), (64, 900, 9, 10)], ids=["o128", "o128_w32", "o64"])
+def test_stem_forward_of_many_short_rows(c_out, n, h, w):
+    """Rows shorter than a quarter of an accumulator, thousands of them: three of a group's four warps have nothing to store and
+    pass by.  No wait expires, and every image of a batch of equal images comes out the same."""
+    import torch
+    from paper_2305_11624_b200 import convbn as C
+    from paper_2305_11624_b200.harness import Block
+    blk = Block(L("rows", n, 3, h, w, c_out, 7, 7, stride=2, pad=3), modes=("tune",))
+    blk.randomize(83)
+    x = blk.x.view(n, -1)
+    x.copy_(x[:1].expand(n, -1).clone())
+    for _ in range(5):
+        blk.z.fill_(float("nan"))
+        blk.tune_fwd()
+        C.convbn_check()
+        z = blk.z.view(n, -1)
+        assert bool((z == z[:1]).all())
+    one = Block(L("rows", 1, 3, h, w, c_out, 7, 7, stride=2, pad=3), modes=("tune",))
+    one.randomize(83)
+    one.x.copy_(x[0])
+    one.tune_fwd()
+    assert torch.equal(one.z, z[0])
+
+
 # rows of 48, 80 and 144 vectors in clusters of four, eight and eight blocks: the last one, three and two have no columns and go
 # straight to the exchange of the dot products
 @pytest.mark.parametrize("c_in,k", [(192, 1), (320, 1), (64, 3)], ids=["row192", "row320", "row576"])
