@@ -760,6 +760,11 @@ namespace {
 struct WinWgPlan { bool ok = false; int pitch = 0, ksteps = 0; uint32_t xstrip = 0, dzrow = 0, work = 0; size_t smem = 0; };
 WinWgPlan plan_window_wgrad(const Problem &pb) {
     WinWgPlan pl;
+    // Rows of a multiple of 8 pixels only.  At other widths the GEMM on the packed input is the faster one by far where rows are
+    // short, this kernel's work going by rows (3 -> 64, 7x7 at 62 x 62, N = 64 21.9 and 34.7 us, at 9 x 10, N = 640 21.3 and
+    // 40.6), and behind where they are long (225 x 225, N = 16 33.4 and 26.7); and it reads what is beyond a row as zeros, where this
+    // one multiplies zeros of dZ by the next pixels, which an infinite X makes NaN.
+    if (pb.w_in % 8) return pl;
     if (!plan_window(pb).ok || pb.c_in > 3 || pb.c_out != 64 || pb.kh < 2 || pb.kh > 8 || pb.w_out > 256) return pl;
     pl.pitch = (int)(((size_t)(pb.w_in + 2 * pb.pad_w) * 8 + 15) / 16 * 16);
     pl.ksteps = (pb.w_out + 15) / 16;

@@ -151,6 +151,23 @@ def test_stem_input_gradient_of_infinite_values(kh, kw):
     assert np.array_equal(~np.isfinite(got["dx"]), met)
 
 
+@pytest.mark.parametrize("n,h,w,k", [(3, 17, 33, 7), (1, 35, 33, 3), (41, 15, 38, 5), (2, 40, 94, 7)])
+def test_stem_weight_gradient_of_infinite_values(n, h, w, k):
+    """domega is infinite exactly in the taps whose sums an infinite X is part of (widths off a multiple of 8); sum dZ does not see
+    X at all."""
+    from paper_2305_11624_b200 import convbn as C
+    spec = L("inf_stem_dw", n, 3, h, w, 64, k, k, stride=2, pad=k // 2)
+    t = parity.make_inputs(spec, 82)
+    t["x"][0, 0, 0, 0], t["x"][n - 1, 0, h // 2, 3], t["x"][0, 1, h - 1, w - 1] = np.inf, np.inf, -np.inf
+    with np.errstate(invalid="ignore"):
+        got, ref = parity.run_tune_gpu(spec, t), weight_gradient(spec, t["x"], t["dz"])
+    C.convbn_check()
+    assert got["_kernels"][2] == "umma-stem"
+    s = t["gamma"] / np.sqrt(t["var_hat"] + spec.eps)
+    same_kind(got["dw"], s[:, None, None, None] * ref, spec.name)
+    np.testing.assert_allclose(got["dbeta"], t["dz"].sum((0, 2, 3)), rtol=1e-4, atol=1e-3)
+
+
 # (dtype, n, c_in, h, w, c_out, k, stride, pad): dZ summed inside the weight gradient where the kernel is the stride (one tile of
 # channels and several that take turns, more than eight of them, slices shorter than the turns, 3 x 3, 1 x 1), by the kernel of
 # its own where the windows overlap
