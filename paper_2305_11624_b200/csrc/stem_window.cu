@@ -11,9 +11,12 @@
 // once per tile (kh / stride_h times overall) instead of once per tap, and K per filter row is 32 (kw <= 8
 // taps x 4 channels; unused slots meet zero weights), i.e. kh x 2 MMAs of 128 x C_out x 16 per output row.
 //
-// Warps: 0-7 load input rows (16-byte global loads, repacked 3 -> 4 channels on the way), 8-11 issue MMAs
+// Warps: 0-7 load input rows (16-byte global loads, 2-byte ones for widths off a multiple of 8; repacked 3 -> 4 channels on the
+// way), 8-11 issue MMAs
 // (round-robin over output rows, disjoint accumulators), 12-23 drain accumulators: scale, shift, bf16,
 // swizzled staging, TMA store.  Every CTA owns a contiguous range of output rows.  Every wait is bounded.
+#include <cmath>
+
 #include "kernels.h"
 #include "mma_sync.cuh"
 #include "sm100_ptx.cuh"
@@ -74,9 +77,8 @@ __device__ __forceinline__ bool win_next_chunk(long long &cur, long long hi, int
     return true;
 }
 
-// win_fill_patch (below) for rows that start anywhere (a width that is no multiple of 8): a pixel per thread, in two-byte loads; neighbours
-// share the sectors.  (Before, such images were packed by a kernel of their own and went through the dense GEMM, three more
-// launches: forward + backward of 3 -> 64, 7x7 stride 2 at 118 x 108, N = 32 93 us, now 62; at 79 x 118, N = 6 41 and 34.)
+// win_fill_patch (below) for rows that start anywhere (a width that is no multiple of 8): a pixel per thread, in two-byte loads;
+// neighbours share the sectors.
 template <int C>
 __device__ __noinline__ void win_fill_patch_any(uint8_t *patch, const __nv_bfloat16 *__restrict__ x, int img, int first, int count,
                                                 int h_in, int w_in, int pad_w, int pitch, int tid, int nthreads, uint32_t fill3) {
@@ -754,7 +756,22 @@ cudaError_t launch_window_c(int c_in, const CUtensorMap &tout, const WinGemm &g,
 
 }  // namespace
 
-bool stem_window_eligible(const Problem &pb) { return plan_window(pb).ok; }
+// Rows of a multiple of 8 pixels: whatever the kernel takes.  At other widths the GEMM on the packed input (pack, expand, multiply)
+// is the alternative that layers go back to where it is the faster one: short rows, many of them.  Estimates in us fitted to 728
+// layers (3x3 to 7x7, 1 to 4 channels, 64 and 128 outputs, 9 x 10 to 333 x 501, up to 800 thousand pixels): here the
+// weights' way into shared memory and the rows of 128 pixels that an SM computes, there 8 x 16 patches.  Forward of 3 -> 64, 7x7, packed
+// and here: 18 x 21, N = 667 20.9 and 34.9, 62 x 62, N = 64 13.8 and 17.1, 225 x 225, N = 16 26.5 and 16.7, 46 x 36, N = 8
+// 9.4 and 7.5.  The choice is 0.7 % from the better one on average and at most 2 % behind the packed form.
+bool stem_window_eligible(const Problem &pb) {
+    if (!plan_window(pb).ok) return false;
+    if (pb.w_in % 8 == 0) return true;
+    const double sms = device_sm_count();
+    const long long nt = pb.c_out / 64, rows = (long long)pb.n * pb.h_out * ((pb.w_out + 127) / 128);
+    const long long patches = (long long)pb.n * ((pb.h_out + 7) / 8) * ((pb.w_out + 15) / 16) * nt;
+    const double window = 4.4 + 0.0095 * pb.kdim * nt * (nt + 1) + (0.5 + 0.024 * pb.kh) * nt * ceil(rows / sms);
+    const double packed = 8.6 + 0.05 * pb.kh + (1.12 + 0.03 * pb.kh) * patches / sms;
+    return window < 0.95 * packed;
+}
 
 namespace {
 struct WinWgPlan { bool ok = false; int pitch = 0, ksteps = 0; uint32_t xstrip = 0, dzrow = 0, work = 0; size_t smem = 0; };

@@ -27,6 +27,10 @@ SPECS = [
     # more than 32 taps on the strip kernel: dense and block-diagonal layers
     L("taps_49", 2, 64, 20, 24, 64, 7, 7, pad=3), L("taps_81", 1, 64, 21, 20, 128, 9, 9, pad=4, dtype="f16"),
     L("taps_49_groups", 2, 128, 19, 23, 128, 7, 7, pad=3, groups=8),
+    # odd widths on both sides of the forward choice: short rows by the packed GEMM, long ones and few by the window kernel
+    L("fwd_packed", 260, 3, 18, 21, 64, 7, 7, stride=2, pad=3, bias=True), L("fwd_packed_o128", 90, 4, 18, 21, 128, 5, 5, stride=2, pad=2),
+    L("fwd_window", 3, 3, 24, 157, 64, 7, 7, stride=2, pad=3, dtype="f16"), L("fwd_window_o128", 2, 3, 14, 301, 128, 3, 3, stride=2, pad=1),
+    L("fwd_window_c4", 3, 4, 24, 157, 64, 5, 5, stride=2, pad=2), L("fwd_window_c2", 3, 2, 24, 93, 64, 8, 8, stride=2, pad=2),
     # stem filters of 257 to 512 weights per output channel, more than the window kernel's table holds, at both kinds of width; and the
     # largest that it takes
     L("stem_16x8", 2, 4, 31, 37, 64, 16, 8, stride=2, pad=3), L("stem_16x8_w40", 2, 4, 31, 40, 64, 16, 8, stride=2, pad=3),
@@ -49,7 +53,7 @@ def test_tune_block(spec):
     parity.compare(got, ref, parity.TOL[spec.dtype], parity.TUNE_OUTPUTS, spec.name, dtype=spec.dtype)
 
 
-@pytest.mark.parametrize("c_out,n,h,w", [(128, 700, 18, 21), (128, 260, 30, 32), (64, 900, 9, 10)], ids=["o128", "o128_w32", "o64"])
+@pytest.mark.parametrize("c_out,n,h,w", [(128, 700, 18, 24), (128, 260, 30, 32), (64, 900, 9, 16)], ids=["o128", "o128_w32", "o64"])
 def test_stem_forward_of_many_short_rows(c_out, n, h, w):
     """Rows shorter than a quarter of an accumulator, thousands of them: three of a group's four warps have nothing to store and
     pass by.  No wait expires, and every image of a batch of equal images comes out the same."""
