@@ -479,6 +479,32 @@ int run_conv_fwd(const convbn_desc *d, const Problem &pb, const void *x, const v
     return CONVBN_OK;
 }
 
+// Whether a stem layer's input gradient goes to the window kernel.  Rows of a multiple of 8 pixels: where that kernel takes the layer.
+// At other widths (its rows then leave in 2-byte stores) the shorter estimate decides, in us: here the weights' way into shared memory and
+// the rows of dZ that an SM multiplies; against
+// - the sub-pixel kernel's rounds of tiles, where that kernel takes the layer.  Fitted to 359 layers (3x3 to 7x7, 2 to 4 channels,
+//   18 x 20 to 239 x 251, up to 800 thousand pixels): 1 % from the better one on average, at most 7 % behind the sub-pixel
+//   kernel.  3 -> 64, 7x7, sub-pixel and window: 118 x 108, N = 32 44.5 and 20.0, 225 x 225, N = 8 44.7 and 15.1, 62 x 62,
+//   N = 69 15.7 and 22.0, 46 x 45, N = 1512 109 and 213.  Below 4096 pixels the sub-pixel kernel keeps the layer: the parity tests'
+//   small ones are there to run it (30 x 30, 5x5, N = 1 7.9 and 6.6);
+// - otherwise the warp-level kernel's windows of 29 or more positions.  160 layers: 0.4 % from the better one, never behind the
+//   warp-level kernel.  7x7 at 30 x 30, N = 32 28.8 and 12.0, 3x3 at 18 x 21, N = 667 31.7 and 36.7.  Below 512 pixels that kernel
+//   keeps the layer (7x7 at 30 x 30, N = 1 28.4 and 9.0), once more for the parity tests: it serves what the others do not take.
+bool stem_dgrad_by_window(const convbn_desc *d, const Problem &pb) {
+    if (!stem_path(d, pb) || !stem_window_dgrad_eligible(pb)) return false;
+    if (pb.w_in % 8 == 0) return true;
+    UmmaConvShape s;
+    const bool by_subpixel = subpixel_dgrad_shape(pb, &s) && umma_strip_eligible(s);
+    if (pb.p < (by_subpixel ? 4096 : 512)) return false;
+    const long long rows = (long long)pb.n * pb.h_out, sms = device_sm_count();
+    const long long windows = (long long)pb.n * ((pb.h_in + 1) / 2) * (((pb.w_in + 1) / 2 + 28) / 29);
+    const double taps = pb.kh * pb.kw;
+    const double window = 3.8 + taps * (0.044 + 0.006 * pb.c_in * pb.c_in) + (0.73 + 0.0185 * pb.kh) * (double)((rows + sms - 1) / sms);
+    const double other = by_subpixel ? 5.0 + 0.02 * taps + 0.0007 * umma_strip_clocks(s)
+                                     : 6.3 + 0.37 * taps + (0.42 + 0.015 * taps) * (double)windows / (double)sms;
+    return window < 0.95 * other;
+}
+
 // Backward data.  `scale` (C_out floats or NULL) is folded into the weights on the way:
 // w_scratch receives omega' in the layout the chosen kernel wants.
 int run_conv_dgrad(const convbn_desc *d, const Problem &pb, const void *dz, const void *w, const float *scale,
@@ -491,15 +517,7 @@ int run_conv_dgrad(const convbn_desc *d, const Problem &pb, const void *dz, cons
     // (the transposed-convolution forward pass is this pass plus a bias)
     if (bias_done) *bias_done = false;
     UmmaConvShape s;
-    // Rows that start off a 16-byte line leave the window kernel in 2-byte stores.  Where the sub-pixel kernel takes such a layer it
-    // is the faster one for small filters and while its tiles fit a few rounds (3 -> 64 at stride 2: 3x3 at 62 x 62, N = 32 6.2
-    // and 9.7 us, 7x7 at 118 x 108, N = 8 10.6 and 12.2), the window kernel beyond (N = 32 44.3 and 19.9).  The warp-level
-    // kernel is slower throughout (30 x 30, N = 32 28.7 and 11.9) and has what is below 512 pixels, a few rows of a few images.
-    const bool by_window = stem_path(d, pb) && stem_window_dgrad_eligible(pb) &&
-                           (pb.w_in % 8 == 0 ||
-                            (subpixel_dgrad_shape(pb, &s) && umma_strip_eligible(s) ? pb.kh * pb.kw > 25 && pb.p >= (1 << 16)
-                                                                                    : pb.p >= 512));
-    if (by_window) {
+    if (stem_dgrad_by_window(d, pb)) {
         // stride 2, C_in <= 4: scatter GEMM over dZ rows, window positions added up on chip
         LAUNCH("stem_dgrad", launch_stem_window_dgrad(pb, dz, w, scale, dx, st));
         *which = "umma-stem";

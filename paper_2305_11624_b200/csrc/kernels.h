@@ -98,6 +98,7 @@ cudaError_t launch_umma_conv(const UmmaConvShape &s, const void *act, const void
 // contract as launch_umma_conv (dense output mode, groups = 1).  Eligibility depends on the image size.
 bool umma_strip_possible(const UmmaConvShape &s);        // it can run this shape ...
 bool umma_strip_eligible(const UmmaConvShape &s);        // ... and is the better choice for it
+double umma_strip_clocks(const UmmaConvShape &s);         // of an eligible shape, estimated
 cudaError_t launch_umma_strip_conv(const UmmaConvShape &s, const void *act, const void *wmat, const float *bias,
                                    void *out, cudaStream_t st, const BnFold *fold = nullptr,
                                    const PostOp *post = nullptr);

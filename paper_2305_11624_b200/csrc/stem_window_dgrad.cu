@@ -10,7 +10,8 @@
 // Tensor memory holds a ring of 16 blocks of 32 columns, one per input row in flight; the kh blocks a dZ row
 // touches are consecutive in the ring, the blocks of rows that no later dZ row reaches are drained: the
 // epilogue adds the up to four window positions that meet one input pixel (a shift over accumulator rows,
-// done through shared memory), rounds to bf16 and writes the input row with coalesced 16-byte stores.
+// done through shared memory), rounds to bf16 and writes the input row with coalesced stores, of 16 bytes where rows are a multiple
+// of 8 pixels, of 2 elsewhere.
 // A CTA owns a contiguous range of dZ rows and the input rows 2 ho, 2 ho + 1 (padded coordinates) that go with
 // them; it also runs the (kh - 1) / 2 dZ rows before its range, whose contributions its first rows need.
 //

@@ -481,7 +481,7 @@ __global__ void __launch_bounds__(kSThreads) umma_strip_conv_kernel(const __grid
 // ---- host side --------------------------------------------------------------------------------------
 namespace {
 
-struct StripPlan { bool ok = false; int bn = 64, R = 0, CW = 0, Wt = 0, nmb = 0, nacc = 2, tiles_w = 1 << 20, nstrips = 2, resident = 0, bstages = 4; uint32_t strip_bytes = 0; size_t smem = 0; };
+struct StripPlan { bool ok = false; int bn = 64, R = 0, CW = 0, Wt = 0, nmb = 0, nacc = 2, tiles_w = 1 << 20, nstrips = 2, resident = 0, bstages = 4; uint32_t strip_bytes = 0; size_t smem = 0; double clk = 0.0; };
 
 int strip_sm_count() { return device_sm_count(); }
 
@@ -588,6 +588,7 @@ StripPlan plan_strip_search(const UmmaConvShape &s, int bn) {
         if (best_cost < 0 || cost < best_cost) {
             best_cost = cost;
             best_eff = eff;
+            best.clk = cost;
             best.ok = true; best.bn = bn; best.R = r; best.CW = cw; best.Wt = wt; best.nmb = nmb;
             best.strip_bytes = sbytes; best.smem = smem; best.tiles_w = tiles_w;
             best.nstrips = nstrips; best.resident = resident ? 1 : 0; best.bstages = bstages;
@@ -786,6 +787,13 @@ bool subpixel_dgrad_shape(const Problem &pb, UmmaConvShape *s) {
                        dmax_h - dmin_h + 1, dmax_w - dmin_w + 1, dmin_h, dmin_w, 1, 1, 1, 1};
     s->sub_cin = pb.c_in; s->sub_hin = pb.h_in; s->sub_win = pb.w_in;
     return true;
+}
+
+// Clocks of the plan's rounds of tiles.  With one or two M blocks the MMAs of an accumulator wait for each other: 1.7 and 1.2 times
+// what the search counts.
+double umma_strip_clocks(const UmmaConvShape &s) {
+    const StripPlan pl = plan_strip(s);
+    return pl.clk * (pl.nmb == 1 ? 1.7 : (pl.nmb == 2 ? 1.2 : 1.0));
 }
 
 size_t subpixel_weight_bytes(const Problem &pb) {

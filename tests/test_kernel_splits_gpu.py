@@ -17,13 +17,18 @@ SPECS = [
     L("dw_264", 2, 264, 9, 11, 264, 3, 3, pad=1, groups=264, bias=True),
     L("dw_320", 3, 320, 13, 37, 320, 3, 3, pad=1, groups=320, dtype="f16"),
     L("dw_520", 1, 520, 6, 10, 520, 3, 3, pad=0, groups=520), L("dw_1032", 1, 1032, 5, 9, 1032, 3, 3, pad=2, groups=1032),
-    # stem rows that start anywhere: odd and even widths off a multiple of 8, the widest the input gradient's kernel takes and
-    # one more, one to four channels, 128 output channels, images smaller than a chunk of rows
+    # stem rows that start anywhere: odd and even widths off a multiple of 8, one to four channels, 128 output channels, images
+    # smaller than a chunk of rows (STEM_DATA: which kernel forms their input gradient)
     L("stem_36", 8, 3, 46, 36, 64, 7, 7, stride=2, pad=3), L("stem_35", 3, 3, 33, 35, 64, 7, 7, stride=2, pad=3, dtype="f16"),
     L("stem_253", 1, 3, 15, 253, 64, 7, 7, stride=2, pad=3, bias=True), L("stem_255", 1, 3, 14, 255, 64, 7, 7, stride=2, pad=3),
     L("stem_c1", 7, 1, 21, 19, 64, 7, 7, stride=2, pad=3), L("stem_c2_k5", 8, 2, 22, 23, 64, 5, 5, stride=2, pad=2, dtype="f16"),
     L("stem_c4", 5, 4, 25, 27, 64, 7, 7, stride=2, pad=3), L("stem_o128", 2, 3, 19, 21, 128, 7, 7, stride=2, pad=3),
     L("stem_small", 70, 3, 9, 10, 64, 7, 7, stride=2, pad=3, dtype="f16"),
+    # ... the window kernel where the sub-pixel kernel would take them too: three and four channels, the widest rows it takes; and one
+    # pixel wider, and more rows than pay
+    L("dx_c3", 8, 3, 46, 45, 64, 7, 7, stride=2, pad=3, bias=True), L("dx_c4", 8, 4, 46, 45, 64, 7, 7, stride=2, pad=3),
+    L("dx_253", 9, 3, 31, 253, 64, 7, 7, stride=2, pad=3), L("dx_253_f16", 9, 3, 32, 253, 64, 6, 6, stride=2, pad=2, dtype="f16"),
+    L("dx_254", 9, 3, 31, 254, 64, 7, 7, stride=2, pad=3), L("dx_rows", 17, 3, 62, 62, 64, 7, 7, stride=2, pad=3),
     # more than 32 taps on the strip kernel: dense and block-diagonal layers
     L("taps_49", 2, 64, 20, 24, 64, 7, 7, pad=3), L("taps_81", 1, 64, 21, 20, 128, 9, 9, pad=4, dtype="f16"),
     L("taps_49_groups", 2, 128, 19, 23, 128, 7, 7, pad=3, groups=8),
@@ -45,12 +50,18 @@ SPECS = [
 ]
 
 
+STEM_DATA = dict.fromkeys(("stem_c1", "stem_c2_k5", "stem_small", "dx_c3", "dx_c4", "dx_253", "dx_253_f16"), "umma-stem")
+STEM_DATA.update(dict.fromkeys(("stem_36", "stem_35", "stem_253", "stem_255", "stem_c4", "stem_16x8", "dx_254", "dx_rows"), "umma-subpixel"))
+STEM_DATA["stem_o128"] = "stem-mma"
+
+
 @pytest.mark.parametrize("spec", SPECS, ids=lambda s: s.name)
 def test_tune_block(spec):
     t = parity.make_inputs(spec, 78)
     ref = parity.oracle_tune(spec, t)
     got = parity.run_tune_gpu(spec, t, deferred=True)
     parity.compare(got, ref, parity.TOL[spec.dtype], parity.TUNE_OUTPUTS, spec.name, dtype=spec.dtype)
+    assert got["_kernels"][1] == STEM_DATA.get(spec.name, got["_kernels"][1])
 
 
 @pytest.mark.parametrize("c_out,n,h,w", [(128, 700, 18, 24), (128, 260, 30, 32), (64, 900, 9, 16)], ids=["o128", "o128_w32", "o64"])
