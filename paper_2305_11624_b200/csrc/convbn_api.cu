@@ -227,7 +227,10 @@ Plan form_plan(const convbn_desc *d, const Problem &pb, int phase, bool bounded,
         if (pl.dw_tma_wgrad && dw_tma_wgrad_partial_bytes(pb) > part_bytes) part_bytes = dw_tma_wgrad_partial_bytes(pb);
     }
     pl.stem = stem_path(d, pb);
-    const size_t xpk_bytes = pl.stem ? stem_packed_bytes(pb) : 0, wst_bytes = pl.stem ? stem_weight_bytes(pb) : 0;
+    // (the window kernels read X as it is)
+    const bool weight_phase = phase == CONVBN_PHASE_TUNE_BWD_WEIGHT || phase == CONVBN_PHASE_DEPLOY_BWD || phase == CONVBN_PHASE_EVAL_BWD;
+    const bool packed = pl.stem && !(weight_phase ? stem_window_wgrad_eligible(pb) : stem_window_eligible(pb));
+    const size_t xpk_bytes = packed ? stem_packed_bytes(pb) : 0, wst_bytes = packed ? stem_weight_bytes(pb) : 0;
     const bool grouped = grouped_path(d, pb);
     const size_t wbd_bytes = grouped ? (size_t)pb.c_out * pb.kh * pb.kw * 64 * elem_size(d->dtype) : 0;
     pl.grouped_wgrad = grouped;

@@ -68,6 +68,18 @@ def test_workspace_sizes_of_the_benchmark_layers():
                 assert wsw <= 16 << 20, (sp.name, wsw)
 
 
+def test_stems_read_as_they_are_ask_for_no_packed_copy():
+    """3 -> 64, 7 x 7, 224 x 224, N = 32: the packed copy of X is 13.5 MB, which the forward pass asked for without a use, and
+    partial sums are all that the weight gradient writes."""
+    d = good(n=32, c_in=3, h_in=224, w_in=224, c_out=64, kh=7, kw=7, stride_h=2, stride_w=2, pad_h=3, pad_w=3, dtype=C.BF16,
+             layout=C.NHWC)
+    assert all(C.convbn_workspace_bytes(d, ph) < 1 << 18 for ph in (C.PHASE_TUNE_FWD, C.PHASE_EVAL_FWD, C.PHASE_DEPLOY_FWD))
+    assert C.convbn_workspace_bytes(d, C.PHASE_TUNE_BWD_WEIGHT) < 8 << 20
+    d.w_in = 31                                                       # short rows, many of them: packed
+    d.n = 512
+    assert C.convbn_workspace_bytes(d, C.PHASE_TUNE_FWD) > 1 << 20 and C.convbn_workspace_bytes(d, C.PHASE_TUNE_BWD_WEIGHT) > 1 << 20
+
+
 def test_which_layers_the_no_allocation_call_takes():
     """Decided by the layer alone, on the host, before any pointer is looked at: a scratch of up to 16 MiB, or one that fewer
     slices bring down to that (the second and third layer)."""
