@@ -1,10 +1,12 @@
 """Compile ``csrc/*.cu`` for sm_100a into ``paper_2305_11624_b200/libconvbn.so`` with nvcc.
 
-``csrc/binding.cpp``, the Python entry to the calls of a training step, becomes ``_binding.so`` beside it (g++).
+``csrc/binding.cpp``, the Python entry to the calls of a training step, becomes ``_binding`` with this interpreter's extension
+suffix beside it (g++); without Python's C headers the library is built alone, for use from C.
 Sources are compiled in parallel to objects under ``_build/`` and linked with the static CUDA
 runtime; the driver API (tensor-map encoding) is resolved at run time through the runtime's
 entry-point query, so the library loads on a machine without a GPU driver.
 """
+import importlib.machinery
 import os
 import subprocess
 import sys
@@ -15,7 +17,7 @@ _HERE = os.path.dirname(os.path.abspath(__file__))
 CSRC = os.path.join(_HERE, "csrc")
 BUILD_DIR = os.path.join(_HERE, "_build")
 LIBRARY = os.path.join(_HERE, "libconvbn.so")
-BINDING = os.path.join(_HERE, "_binding.so")
+BINDING = os.path.join(_HERE, "_binding" + importlib.machinery.EXTENSION_SUFFIXES[0])    # (an interpreter loads its own only)
 CXX = os.environ.get("CXX", "g++")
 NVCC = os.environ.get("NVCC", "/usr/local/cuda/bin/nvcc")
 ARCH = ["-gencode", "arch=compute_100a,code=sm_100a"]
@@ -57,10 +59,23 @@ def _build_binding():
     os.replace(tmp, BINDING)
 
 
+def _headers() -> bool:
+    return os.path.exists(os.path.join(sysconfig.get_paths()["include"], "Python.h"))
+
+
 def build(force: bool = False, verbose: bool = False) -> str:
-    """Build the library if missing or older than any source; return its path."""
-    if not force and all(os.path.exists(f) and os.path.getmtime(f) >= _deps_mtime() for f in (LIBRARY, BINDING)):
-        return LIBRARY
+    """Build the library and the binding if missing or older than any source; return the library's path."""
+    fresh = lambda f: not force and os.path.exists(f) and os.path.getmtime(f) >= _deps_mtime()
+    if not fresh(LIBRARY):
+        _build_library(verbose)
+    if not fresh(BINDING) and _headers():
+        _build_binding()
+    elif not os.path.exists(BINDING):
+        print("no Python.h in %s: %s is not built" % (sysconfig.get_paths()["include"], os.path.basename(BINDING)), file=sys.stderr)
+    return LIBRARY
+
+
+def _build_library(verbose: bool):
     os.makedirs(BUILD_DIR, exist_ok=True)
     with ThreadPoolExecutor(max_workers=8) as ex:
         objs = list(ex.map(lambda s: _compile(s, verbose), sources()))
@@ -68,8 +83,6 @@ def build(force: bool = False, verbose: bool = False) -> str:
     cmd = [NVCC] + ARCH + ["-shared", "-cudart", "static", "-o", tmp] + objs
     subprocess.run(cmd, check=True)
     os.replace(tmp, LIBRARY)
-    _build_binding()
-    return LIBRARY
 
 
 if __name__ == "__main__":

@@ -1,4 +1,4 @@
-"""Thin binding of ``libconvbn.so`` (declared in ``include/convbn.h``): ctypes, and ``_binding.so`` for the calls that a
+"""Thin binding of ``libconvbn.so`` (declared in ``include/convbn.h``): ctypes, and the extension module ``_binding`` for the calls that a
 training step makes.
 
 Argument marshalling only: every function has the name and argument order of its C entry point,
@@ -7,6 +7,7 @@ a non-zero status raises ``ConvBNError``.  There is no fallback: if the compiled
 missing, importing succeeds but the first call raises.
 """
 import ctypes
+import importlib.machinery
 import importlib.util
 import os
 from typing import Optional
@@ -58,7 +59,7 @@ _lib = None
 def _signatures():
     """argtypes of the entry points that take pointers: ctypes then converts plain integers itself, without an object per
     argument, and to their full width (d: descriptor, p: pointer or stream, z: size, i: int, q: long long, f: double).  The
-    calls of a training step go through _binding.so here; whoever takes them from lib() gets them typed all the same."""
+    calls of a training step go through _binding here; whoever takes them from lib() gets them typed all the same."""
     kinds = {"d": ctypes.POINTER(Desc), "p": ctypes.c_void_p, "z": ctypes.c_size_t, "i": ctypes.c_int,
              "q": ctypes.c_longlong, "f": ctypes.c_double}
     table = {
@@ -104,7 +105,7 @@ def _calls():
     global _native
     if _native is None:
         lib()
-        path = os.path.join(_HERE, "_binding.so")
+        path = os.path.join(_HERE, "_binding" + importlib.machinery.EXTENSION_SUFFIXES[0])
         if not os.path.exists(path):
             raise OSError("%s not found: run `python -m paper_2305_11624_b200.build`" % path)
         spec = importlib.util.spec_from_file_location(__package__ + "._binding", path)

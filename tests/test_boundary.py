@@ -230,6 +230,26 @@ def test_descriptors_in_every_form():
             C.convbn_tune_fwd(d, *args, size, stream=0)
 
 
+def test_the_binding_is_built_per_interpreter_and_only_with_its_headers(monkeypatch, tmp_path, capsys):
+    """A library that is up to date stays, a binding of another interpreter is not this one's, and without Python's headers the
+    library is there alone."""
+    import importlib.machinery
+    from paper_2305_11624_b200 import build as B
+    assert os.path.basename(B.BINDING) == "_binding" + importlib.machinery.EXTENSION_SUFFIXES[0]
+    made = []
+    monkeypatch.setattr(B, "LIBRARY", str(tmp_path / "lib.so"))
+    monkeypatch.setattr(B, "BINDING", str(tmp_path / "_binding.here.so"))
+    monkeypatch.setattr(B, "_build_library", lambda verbose: (made.append("library"), open(B.LIBRARY, "w").close()))
+    monkeypatch.setattr(B, "_build_binding", lambda: (made.append("binding"), open(B.BINDING, "w").close()))
+    (tmp_path / "_binding.other.so").write_text("")
+    monkeypatch.setattr(B, "_headers", lambda: False)
+    assert B.build() == B.LIBRARY and made == ["library"] and "Python.h" in capsys.readouterr().err
+    monkeypatch.setattr(B, "_headers", lambda: True)
+    B.build()
+    B.build()
+    assert made == ["library", "binding"]
+
+
 def test_status_strings():
     assert C.status_string(C.OK) == "ok"
     assert "workspace" in C.status_string(C.EWORKSPACE)
