@@ -250,6 +250,51 @@ def test_the_binding_is_built_per_interpreter_and_only_with_its_headers(monkeypa
     assert made == ["library", "binding"]
 
 
+def test_plans_kept_per_thread():
+    """More layers than a thread keeps plans of, asked for in changing order, in both 16-bit types in turn, by two threads at
+    once: every size is the one that a thread asked for nothing else gives."""
+    import random
+    import threading
+    rng, asked = random.Random(3), []
+    for i in range(300):
+        kind = i % 4
+        kw = dict(n=rng.randint(1, 40), h_in=rng.randint(8, 60), w_in=rng.randint(8, 60), dtype=C.BF16 if i % 2 else C.F16, layout=C.NHWC)
+        c = 64 * rng.randint(1, 6)
+        if kind == 0:
+            d = good(c_in=c, c_out=64 * rng.randint(1, 6), **kw)
+        elif kind == 1:
+            d = good(c_in=3, c_out=64, kh=7, kw=7, stride_h=2, stride_w=2, pad_h=3, pad_w=3, **kw)
+        elif kind == 2:
+            d = good(c_in=c, c_out=c, groups=rng.choice((c, c // 8)), **kw)
+        else:
+            d = good(c_in=c, c_out=64, kh=2, kw=2, stride_h=2, stride_w=2, pad_h=0, pad_w=0, **kw)
+        asked += [(d, ph) for ph in range(7)] + ([(d, "transposed")] if kind == 3 else [])
+    size = lambda d, ph: C.convbn_tconv_workspace_bytes(d) if ph == "transposed" else C.convbn_workspace_bytes(d, ph)
+    alone = {}
+
+    def one(i):
+        alone[i] = size(*asked[i])
+
+    def many(order, out):
+        out.extend((i, size(*asked[i])) for i in order)
+
+    def run(*targets):
+        threads = [threading.Thread(target=f, args=a) for f, a in targets]
+        for t in threads:
+            t.start()
+        for t in threads:
+            t.join()
+
+    for i in range(len(asked)):
+        run((one, (i,)))
+    orders = [rng.sample(range(len(asked)), len(asked)) for _ in range(3)]
+    got = [[], [], []]
+    many(orders[0] + orders[0][:700], got[0])
+    run((many, (orders[1], got[1])), (many, (orders[2], got[2])))
+    assert len(alone) == len(asked) and len(set(alone.values())) > 500
+    assert all(alone[i] == v for g in got for i, v in g)
+
+
 def test_status_strings():
     assert C.status_string(C.OK) == "ok"
     assert "workspace" in C.status_string(C.EWORKSPACE)
