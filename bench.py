@@ -76,14 +76,14 @@ def kernel_bytes(kind, spec, out_hw):
 # DRAM bytes (read + write) per launch, from an ncu capture of the kernels as they are now; a kernel that
 # changes after its capture loses its entry (traffic: null).  (kernel family, layer) -> bytes.
 NCU_SUMMARY = "profiles/step_kernels_ncu_traffic.md"
-NCU_TRAFFIC = {("stem_fwd", "c2s"): 59.5e6, ("stem_dgrad", "c2s"): 112.5e6, ("stem_wgrad", "c2s"): 123.3e6,
-               ("umma_fwd", "c1a"): 51.5e6, ("umma_bwd", "c1a"): 70.6e6,
+NCU_TRAFFIC = {("stem_fwd", "c2s"): 59.2e6, ("stem_dgrad", "c2s"): 113.1e6, ("stem_wgrad", "c2s"): 123.1e6,
+               ("umma_fwd", "c1a"): 51.5e6, ("umma_bwd", "c1a"): 70.8e6,
                ("umma_fwd", "c1b"): 13.0e6, ("umma_dgrad", "c1b"): 13.0e6, ("umma_wgrad", "c1b"): 25.7e6,
-               ("umma_fwd", "c2a"): 15.0e6, ("umma_dgrad", "c2a"): 5.37e6, ("umma_wgrad", "c2a"): 16.1e6,
-               ("umma_fwd", "c2b"): 8.00e6, ("umma_dgrad", "c2b"): 7.99e6, ("umma_wgrad", "c2b"): 6.47e6,
+               ("umma_fwd", "c2a"): 15.0e6, ("umma_dgrad", "c2a"): 5.4e6, ("umma_wgrad", "c2a"): 16.1e6,
+               ("umma_fwd", "c2b"): 8.0e6, ("umma_dgrad", "c2b"): 8.0e6, ("umma_wgrad", "c2b"): 6.5e6,
                ("umma_fwd", "c3a"): 17.2e6, ("umma_dgrad", "c3a"): 17.2e6, ("umma_wgrad", "c3a"): 34.2e6,
-               ("dw_fwd", "c4a"): 254.8e6, ("dw_dgrad", "c4a"): 254.6e6, ("dw_wgrad", "c4a"): 309.1e6,
-               ("grouped_fwd", "c4b"): 25.8e6, ("grouped_dgrad", "c4b"): 25.7e6, ("grouped_wgrad", "c4b"): 51.5e6}
+               ("dw_fwd", "c4a"): 255.4e6, ("dw_dgrad", "c4a"): 255.4e6, ("dw_wgrad", "c4a"): 308.4e6,
+               ("grouped_fwd", "c4b"): 25.8e6, ("grouped_dgrad", "c4b"): 25.7e6, ("grouped_wgrad", "c4b"): 51.4e6}
 
 KIND_OF = {"strip_fwd": "fwd", "strip_dgrad": "dgrad", "direct_fwd": "fwd", "direct_dgrad": "dgrad", "direct_wgrad": "wgrad",
            "umma_fwd": "fwd", "umma_dgrad": "dgrad", "umma_wgrad": "wgrad", "umma_bwd": "bwd",

@@ -979,10 +979,11 @@ int side_lane(SideLane **out) {
 
 // Which of the two passes of a joined backward call stays on the caller's stream.  The lane's first kernel starts one event
 // later and the caller's stream resumes one event after the lane's last, a few us each, so the longer pass belongs on the
-// caller's stream: the parameter gradients (GEMM and epilogue), 59 -> 55 us per forward + backward of a 3x3 64 -> 64 layer at
-// 56 x 56, N = 32, 68 -> 65 at 3x3 stride 2 128 -> 128, 200 x 334.  With a million weights, or where it is a GEMM per
-// parity class, the data pass is the longer one: 3x3 512 -> 512 at 7 x 7, N = 64
-// takes 79 us this way and 87 the other, 3x3 stride 2 256 -> 256 at 28 x 28 57 and 60.
+// caller's stream: the parameter gradients (GEMM and epilogue).  Forward + backward that way and the other: 3x3 64 -> 64 at
+// 56 x 56, N = 32 45.4 and 48.0 us, 3x3 stride 2 128 -> 128 at 200 x 334, N = 2 55.6 and 59.6, 256 -> 256 at 28 x 28, N = 32 47.2
+// and 49.3.  With a million weights, or where it is a GEMM per parity class, the data pass was the longer one while the kernel that
+// adds the slices was launched early (3x3 512 -> 512 at 7 x 7, N = 64 87 and 79).  It no longer is (57.6 and 62.1, 1x1 512 -> 2048
+// 35.0 and 42.4, 3x3 1024 at 14 x 14, N = 4 113.9 and 113.5): these layers keep the order they had.
 // A captured call pays no events, and its lane's nodes come first: there the pass with two kernels, the parameter gradients,
 // belongs on the lane (graph replay of random layers, the other order = 1: grouped by 8 below 40 us 0.88, 1x1 below 15 us 0.93,
 // depthwise 0.97, 3x3 and longer calls 0.98 to 1).

@@ -343,8 +343,8 @@ static long long wgrad_tiles(const Problem &pb, int bn, bool ones_slice) {
 }
 
 // The slice count minimises  rounds over the resident slots x (pixels per slice + a fixed cost per
-// CTA, in pixels) + a small cost per slice for the epilogue that adds the slices up; a grid a few
-// CTAs larger than the slots would otherwise run a second, nearly empty round.
+// CTA, in pixels) + a small cost per slice for the epilogue that adds the slices up (four pixels, set when a block added a whole
+// channel); a grid a few CTAs larger than the slots would otherwise run a second, nearly empty round.
 static UmmaWgradPlan wgrad_slices(const Problem &pb, long long tiles, long long slots) {
     UmmaWgradPlan pl;
     const long long max_splits = (pb.p + 4 * kWP - 1) / (4 * kWP);     // at least 256 pixels per slice
