@@ -369,18 +369,22 @@ __global__ void __launch_bounds__(TW >= 4 ? 384 : 288, TW >= 4 ? 1 : 2) dw_tma_w
                             if (slot_off == ring_bytes) { slot = 0; slot_off = 0; par ^= 1u; }
                             // X row k is tap row r of dZ row k - r (slot (ph - r) mod KH), if the band has that row (the same for
                             // the whole block; multiplying by zeros instead made NaN of an infinite X)
+                            auto products = [&](auto inner) {
 #pragma unroll
-                            for (int r = 0; r < KH; ++r) {
-                                const int sl = (ph - r + KH) % KH;
-                                if ((r > 0 && k < r) || (r < KH - 1 && k - r >= rows)) continue;
+                                for (int r = 0; r < KH; ++r) {
+                                    const int sl = (ph - r + KH) % KH;
+                                    if (!decltype(inner)::value && ((r > 0 && k < r) || (r < KH - 1 && k - r >= rows))) continue;
 #pragma unroll
-                                for (int q = 0; q < KW; ++q)
+                                    for (int q = 0; q < KW; ++q)
 #pragma unroll
-                                    for (int j = 0; j < TW; ++j) {
-                                        acc[r * KW + q][0] = fma2(dzw[sl][j][0], xs[j + q][0], acc[r * KW + q][0]);
-                                        acc[r * KW + q][1] = fma2(dzw[sl][j][1], xs[j + q][1], acc[r * KW + q][1]);
-                                    }
-                            }
+                                        for (int j = 0; j < TW; ++j) {
+                                            acc[r * KW + q][0] = fma2(dzw[sl][j][0], xs[j + q][0], acc[r * KW + q][0]);
+                                            acc[r * KW + q][1] = fma2(dzw[sl][j][1], xs[j + q][1], acc[r * KW + q][1]);
+                                        }
+                                }
+                            };
+                            if (k >= KH - 1 && k < rows) products(std::true_type{});
+                            else products(std::false_type{});
                         }
                     }
                 }
