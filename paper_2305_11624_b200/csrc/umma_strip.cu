@@ -53,7 +53,8 @@ struct StripGemm {
     int f16;                          // 16-bit storage type: 0 bf16, 1 IEEE half
     int sub_cin, sub_hin, sub_win;    // sub-pixel output mode, see UmmaConvShape
     int sub_wide;                     // 1: wide sub-pixel mode (BN = 64 / 128), n-tile -> parity class
-    uint32_t sub_mask[4];             // sub_wide, at most 32 taps: those with weights, per class (all others have every tap)
+    uint32_t sub_mask[4];             // sub_wide, at most 32 taps: those with weights, per class (all others, of any number, have every tap:
+                                      // a mask of ones, read round and round)
     __nv_bfloat16 *out;
     BnFold fold;
     const __nv_bfloat16 *post_add, *post_mask;      // POST: at the output's offsets
@@ -219,12 +220,12 @@ __global__ void __launch_bounds__(kSThreads) umma_strip_conv_kernel(const __grid
             } else
             for (uint32_t t = blockIdx.x; t < total_tiles && ok; t += gridDim.x) {
                 const int n0 = (int)(t % n_tiles) * BN;
-                const uint32_t mask = g.sub_wide ? g.sub_mask[n0 / g.sub_cin] : 0u;
+                const uint32_t mask = g.sub_wide ? g.sub_mask[n0 / g.sub_cin] : 0xffffffffu;
                 for (int cc = 0; cc < cchunks && ok; ++cc) {
                     int kx = cc * 64;
 #pragma unroll 3
                     for (int tap = 0; tap < taps; ++tap, kx += w_ca) {
-                        if (g.sub_wide && !((mask >> tap) & 1u)) continue;
+                        if (!((mask >> (tap & 31)) & 1u)) continue;
                         if (!free) ok = mbar_wait_bounded(empty0 + sb, ph, abort_flag);
                         if (!ok) break;
                         const uint32_t bar = full0 + sb, dst = slot;
@@ -263,7 +264,7 @@ __global__ void __launch_bounds__(kSThreads) umma_strip_conv_kernel(const __grid
                 if (!mbar_wait_bounded(&ctl->tmem_empty[a], (use & 1u) ^ 1u, abort_flag)) { ok = false; break; }
                 tc_fence_after_sync();
                 const uint32_t d0 = tmem_base + a * (uint32_t)(g.nmb * BN);
-                const uint32_t mask = g.sub_wide ? g.sub_mask[(int)(t % n_tiles) * BN / g.sub_cin] : 0u;
+                const uint32_t mask = g.sub_wide ? g.sub_mask[(int)(t % n_tiles) * BN / g.sub_cin] : 0xffffffffu;
                 uint32_t started = 0;                   // 0 until the tile's first MMAs have been issued
                 if (g.resident) b_lo = bres_lo;
                 for (int cc = 0; cc < cchunks && ok; ++cc) {
@@ -280,7 +281,7 @@ __global__ void __launch_bounds__(kSThreads) umma_strip_conv_kernel(const __grid
                             const uint32_t a0 = a_lo;
                             a_lo += 8u;
                             if (++q == g.kw) { q = 0; a_row += (uint32_t)g.Wt * 8u; a_lo = a_row; }
-                            if (g.sub_wide && !((mask >> tap) & 1u)) continue;
+                            if (!((mask >> (tap & 31)) & 1u)) continue;
                             if (!g.resident && !ready && !mbar_wait_bounded(bfull0 + s8, bph, abort_flag)) { ok = false; break; }
                             const uint32_t b0 = b_lo, done = bempty0 + s8;
                             b_lo += kBBytes >> 4;
@@ -303,7 +304,7 @@ __global__ void __launch_bounds__(kSThreads) umma_strip_conv_kernel(const __grid
                     for (int tap = 0; tap < taps; ++tap) {
                         const uint32_t a_tap = a_patch + row_shift + (uint32_t)q * 8u;
                         if (++q == g.kw) { q = 0; row_shift += (uint32_t)g.Wt * 8u; }
-                        if (g.sub_wide && !((mask >> tap) & 1u)) continue;
+                        if (!((mask >> (tap & 31)) & 1u)) continue;
                         if (!g.resident && !ready && !mbar_wait_bounded(bfull0 + s8, bph, abort_flag)) { ok = false; break; }
                         const uint32_t b0 = b_lo, done = bempty0 + s8;
                         b_lo += kBBytes >> 4;
