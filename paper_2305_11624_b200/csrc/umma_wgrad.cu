@@ -451,14 +451,12 @@ cudaError_t launch_umma_wgrad(const Problem &pb, const UmmaWgradPlan &pl, const 
 // CL blocks (a cluster) share a channel, a span of k each; their parts of the dot product meet in the first one.
 // Threads of a block: VL along k (a float4 each, so that reads and stores are whole lines) x SL groups of slices, added in
 // order through shared memory; a thread requests up to eight slices before it uses the first.  Bound by the latency of those
-// reads (9 to 19 MB, most of them from L2), so a layer is cut into blocks of a few hundred threads that go over their span
-// once: with a block of up to 1024 threads per channel, 64 channels left most SMs idle and 4608 weights took a second, nearly
-// empty turn (forward + backward of 3x3 64 -> 64 at 56 x 56, N = 32
-// 51.3 -> 49.5 us, of 1000 rows 256 -> 64 15.1 -> 14.6).
+// reads (9 to 19 MB, most of them from L2): few channels of long rows would leave most SMs idle with a block each (how many: see
+// the launch).
 // With k-major partial tiles the GEMM's stores were 16 bytes per lane in 32 lines, this kernel had to transpose,
 // and the per-channel sums needed a counter or a second kernel.  Weight phase (GEMM + this), graph replay, N = 32: 1x1
 // 512 -> 128 at 28 x 28 20.3 -> 12.0 us, 3x3 256 at 14 x 14 22.8 -> 17.2, 3x3 512 at 7 x 7 30.0 -> 22.8.
-constexpr int kRowsMaxThreads = 512, kRowsMaxCluster = 8;
+constexpr int kRowsMaxThreads = 512, kRowsMaxCluster = 4;
 template <int CL>
 __global__ void __launch_bounds__(kRowsMaxThreads) wgrad_rows_kernel(int c_out, int kdim, int span, int VL, int SL,
                                                                      const float *__restrict__ part, int splits,
@@ -568,17 +566,25 @@ __global__ void __launch_bounds__(kRowsMaxThreads) wgrad_rows_kernel(int c_out, 
 cudaError_t launch_wgrad_rows(const Problem &pb, int splits, const float *partials, const float *bsum, const void *w,
                               const float *vec3, const float *b, const float *mean, float *dw, float *db, float *dgamma,
                               float *dbeta, bool need_sums, cudaStream_t st) {
-    // slice groups so that a thread adds at most eight slices; a cluster as large as brings a block to 384 threads (spans of
-    // whole 128-byte lines) or the grid to four blocks per SM; then as many threads along the span as there is room for
+    // Slice groups so that a thread adds at most eight slices, threads along the span in equal turns.  Blocks per channel: up to two per
+    // SM for rows with 1600 vectors (of all slices) or more to read, one otherwise: below that and with more channels the blocks' meeting
+    // and their number cost more than they share.  Weight phase with 1, 2, 4, 8 blocks per channel: 1x1 256 -> 64, 1000 rows, 256 vectors
+    // 9.4 9.7 10.0 9.8 us; 3x3 256 -> 128, 26 x 26, 1728 vectors 7.8 7.2 7.4 7.4; 3x3 64 -> 64, 56 x 56, N = 32, 8496 vectors
+    // 21.1 18.2 16.2 16.3; 3x3 512 -> 512, 7 x 7, N = 64 21.0 22.5 25.3 26.0; 5x5 640 -> 384, 13 x 13, N = 9 40.4 44.7 49.8 60.2;
+    // whole backward calls at 192 and 256 channels, 4000 to 4400 vectors: 3x3 256 -> 256, 14 x 14, N = 32 27.0 27.4 27.1 29.0, 1x1
+    // 832 -> 256 57.0 58.8 57.9 59.2, 3x3 192 -> 192, 28 x 28, N = 16 32.8 34.1 33.4 34.6.
     int SL = 1, CL = 1;
     while (SL < 32 && SL * 8 < splits) SL *= 2;
     auto vectors = [&](int cl) { return ((pb.kdim / 4 + cl - 1) / cl + 7) / 8 * 8; };
-    while (CL < kRowsMaxCluster && pb.kdim / 4 >= 16 * CL &&
-           (vectors(CL) * SL > 384 || (long long)pb.c_out * CL < 4LL * device_sm_count()))
-        CL *= 2;
+    const long long work = (long long)(pb.kdim / 4) * splits;
+    while (work >= 1600 && CL < kRowsMaxCluster && pb.kdim / 4 >= 16 * CL && (long long)pb.c_out * CL <= device_sm_count()) CL *= 2;
     const int span = 4 * vectors(CL);
     int VL = vectors(CL);
-    if (VL * SL > kRowsMaxThreads) VL = kRowsMaxThreads / SL;
+    if (VL * SL > kRowsMaxThreads) {
+        const int turns = (VL * SL + kRowsMaxThreads - 1) / kRowsMaxThreads;
+        VL = ((VL + turns - 1) / turns + 7) / 8 * 8;
+        if (VL * SL > kRowsMaxThreads) VL = kRowsMaxThreads / SL;
+    }
     const int threads = (VL * SL + 31) / 32 * 32;
     if ((long long)pb.c_out * CL > 0x7fffffffLL) return cudaErrorInvalidValue;
     auto go = [&](auto cl) {
@@ -591,8 +597,7 @@ cudaError_t launch_wgrad_rows(const Problem &pb, int splits, const float *partia
     };
     if (CL == 1) return go(std::integral_constant<int, 1>());
     if (CL == 2) return go(std::integral_constant<int, 2>());
-    if (CL == 4) return go(std::integral_constant<int, 4>());
-    return go(std::integral_constant<int, 8>());
+    return go(std::integral_constant<int, 4>());
 }
 
 // ---- epilogue over k-major partials (the stem's weight gradient) --------------------------------------

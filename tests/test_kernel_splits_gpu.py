@@ -40,11 +40,12 @@ SPECS = [
     # largest that it takes
     L("stem_16x8", 2, 4, 31, 37, 64, 16, 8, stride=2, pad=3), L("stem_16x8_w40", 2, 4, 31, 40, 64, 16, 8, stride=2, pad=3),
     L("stem_13x7", 2, 3, 30, 33, 64, 13, 7, stride=2, pad=3, dtype="f16"), L("stem_16x8_c2", 2, 2, 31, 37, 64, 16, 8, stride=2, pad=3),
-    # adding the slices of a weight gradient: one block per channel, clusters of two, four and eight; spans that end early; a
-    # slice group per thread and many
-    L("rows_1", 2, 64, 6, 7, 2048, 1, 1), L("rows_2", 2, 192, 9, 9, 320, 1, 1, bias=True),
-    L("rows_4", 3, 128, 14, 15, 192, 1, 1, dtype="f16"), L("rows_8", 9, 64, 30, 31, 64, 3, 3, pad=1),
-    L("rows_k5", 4, 64, 12, 13, 64, 5, 5, pad=2),
+    # adding the slices of a weight gradient: one block per channel, in one turn and several, clusters of two and four; spans that
+    # end early; a slice group per thread and many
+    L("rows_64", 2, 64, 6, 7, 2048, 1, 1), L("rows_192", 2, 192, 9, 9, 320, 1, 1, bias=True),
+    L("rows_128", 3, 128, 14, 15, 192, 1, 1, dtype="f16"), L("rows_slices", 9, 64, 30, 31, 64, 3, 3, pad=1),
+    L("rows_k5", 4, 64, 12, 13, 64, 5, 5, pad=2), L("rows_turns", 2, 640, 9, 8, 320, 3, 3, pad=1),
+    L("rows_pairs", 4, 64, 30, 31, 128, 3, 3, pad=1, bias=True), L("rows_fours", 5, 64, 28, 29, 64, 3, 3, pad=1, dtype="f16"),
     # dense epilogue: output channels that end inside a 64-column chunk, a last tile of one pixel
     L("epi_72", 3, 64, 7, 19, 72, 3, 3, pad=1, bias=True), L("epi_200", 43, 64, 3, 1, 200, 1, 1, dtype="f16"),
 ]
@@ -88,15 +89,15 @@ def test_stem_forward_of_many_short_rows(c_out, n, h, w):
     assert torch.equal(one.z, z[0])
 
 
-# rows of 48, 80 and 144 vectors in clusters of four, eight and eight blocks: the last one, three and two have no columns and go
-# straight to the exchange of the dot products
-@pytest.mark.parametrize("c_in,k", [(192, 1), (320, 1), (64, 3)], ids=["row192", "row320", "row576"])
-def test_clusters_with_blocks_beyond_the_row(c_in, k):
+# rows of 48, 80 and 144 vectors in clusters of four: with 48 the last block has no columns and goes straight to the exchange of the
+# dot products
+@pytest.mark.parametrize("n,c_in,k", [(10, 192, 1), (14, 320, 1), (9, 64, 3)], ids=["row192", "row320", "row576"])
+def test_clusters_with_blocks_beyond_the_row(n, c_in, k):
     """Every block's part of the dot product arrives: dgamma matches the oracle, and is the same in every one of many runs."""
     import torch
     from paper_2305_11624_b200 import convbn as C
     from paper_2305_11624_b200.harness import Block
-    spec = L("clusters", 3, c_in, 11, 12, 64, k, k, pad=k // 2)
+    spec = L("clusters", n, c_in, 30, 31, 64, k, k, pad=k // 2)
     t = parity.make_inputs(spec, 79)
     parity.compare(parity.run_tune_gpu(spec, t, deferred=True), parity.oracle_tune(spec, t), parity.TOL["bf16"],
                    parity.TUNE_OUTPUTS, spec.name, dtype="bf16")
