@@ -145,7 +145,7 @@ bool fused_bwd_path(const convbn_desc *d, const Problem &pb) {
 bool strided_dgrad_ok(const convbn_desc *d, const Problem &pb);
 bool umma_dgrad_shape(const convbn_desc *d, const Problem &pb, UmmaConvShape *s);
 
-// bounded: the tensor-core weight gradient in the slices of a call with a fixed scratch; sums: what it sums beside.
+// bounded: the tensor-core weight gradient in the slices of a call with a fixed scratch, a stem's without a packed copy of X; sums: what it sums beside.
 Plan form_plan(const convbn_desc *d, const Problem &pb, int phase, bool bounded, WgradSums sums);
 
 // The plans of the last layers of this thread: a function of the descriptor, the phase and the device (its SM count).  A
@@ -229,7 +229,7 @@ Plan form_plan(const convbn_desc *d, const Problem &pb, int phase, bool bounded,
     pl.stem = stem_path(d, pb);
     // (the window kernels read X as it is)
     const bool weight_phase = phase == CONVBN_PHASE_TUNE_BWD_WEIGHT || phase == CONVBN_PHASE_DEPLOY_BWD || phase == CONVBN_PHASE_EVAL_BWD;
-    const bool packed = pl.stem && !(weight_phase ? stem_window_wgrad_eligible(pb) : stem_window_eligible(pb));
+    const bool packed = pl.stem && !(weight_phase ? stem_window_wgrad_eligible(pb, bounded) : stem_window_eligible(pb));
     const size_t xpk_bytes = packed ? stem_packed_bytes(pb) : 0, wst_bytes = packed ? stem_weight_bytes(pb) : 0;
     const bool grouped = grouped_path(d, pb);
     const size_t wbd_bytes = grouped ? (size_t)pb.c_out * pb.kh * pb.kw * 64 * elem_size(d->dtype) : 0;
@@ -250,7 +250,7 @@ Plan form_plan(const convbn_desc *d, const Problem &pb, int phase, bool bounded,
         pl.uw = stem_wgrad_plan(pb);
         pl.bsplits = pl.uw.splits;
         part_bytes = (size_t)pl.uw.splits * stem_krows(pb) * 64 * pb.c_out * sizeof(float);
-        if (stem_window_wgrad_eligible(pb)) {
+        if (stem_window_wgrad_eligible(pb, bounded)) {
             pl.stem_win_wgrad = true;
             pl.uw = UmmaWgradPlan();
             pl.uw.splits = stem_window_wgrad_ctas(pb);

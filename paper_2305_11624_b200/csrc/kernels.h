@@ -195,7 +195,7 @@ cudaError_t launch_stem_window_fwd(const Problem &pb, const void *x, const void 
 // Weight gradient of the same layers (C_in <= 3, C_out = 64) straight from X and dZ: one fp32 partial
 // [kdim][C_out] and one row of sums of dZ per CTA (stem_window_wgrad_ctas of them), for
 // launch_wgrad_epilogue_kmajor.
-bool stem_window_wgrad_eligible(const Problem &pb);
+bool stem_window_wgrad_eligible(const Problem &pb, bool any_width = false);
 int stem_window_wgrad_ctas(const Problem &pb);
 cudaError_t launch_stem_window_wgrad(const Problem &pb, const void *dz, const void *x, float *partials, float *bsum,
                                      cudaStream_t st);

@@ -775,13 +775,14 @@ bool stem_window_eligible(const Problem &pb) {
 
 namespace {
 struct WinWgPlan { bool ok = false; int pitch = 0, ksteps = 0; uint32_t xstrip = 0, dzrow = 0, work = 0; size_t smem = 0; };
-WinWgPlan plan_window_wgrad(const Problem &pb) {
+WinWgPlan plan_window_wgrad(const Problem &pb, bool any_width) {
     WinWgPlan pl;
     // Rows of a multiple of 8 pixels only.  At other widths the GEMM on the packed input is the faster one by far where rows are
     // short, this kernel's work going by rows (3 -> 64, 7x7 at 62 x 62, N = 64 21.9 and 34.7 us, at 9 x 10, N = 640 21.3 and
     // 40.6), and behind where they are long (225 x 225, N = 16 33.4 and 26.7); and it reads what is beyond a row as zeros, where this
-    // one multiplies zeros of dZ by the next pixels, which an infinite X makes NaN.
-    if (pb.w_in % 8) return pl;
+    // one multiplies zeros of dZ by the next pixels, which an infinite X makes NaN.  (any_width: the call whose fixed scratch has no room for
+    // the packed input.)
+    if (pb.w_in % 8 && !any_width) return pl;
     if (!plan_window(pb).ok || pb.c_in > 3 || pb.c_out != 64 || pb.kh < 2 || pb.kh > 8 || pb.w_out > 256) return pl;
     pl.pitch = (int)(((size_t)(pb.w_in + 2 * pb.pad_w) * 8 + 15) / 16 * 16);
     pl.ksteps = (pb.w_out + 15) / 16;
@@ -795,7 +796,7 @@ WinWgPlan plan_window_wgrad(const Problem &pb) {
 }
 }  // namespace
 
-bool stem_window_wgrad_eligible(const Problem &pb) { return plan_window_wgrad(pb).ok; }
+bool stem_window_wgrad_eligible(const Problem &pb, bool any_width) { return plan_window_wgrad(pb, any_width).ok; }
 
 // (one function per channel count: the once-per-device flags must not be shared between the kernels)
 template <int C>
@@ -815,7 +816,7 @@ int stem_window_wgrad_ctas(const Problem &pb) {
 
 cudaError_t launch_stem_window_wgrad(const Problem &pb, const void *dz, const void *x, float *partials, float *bsum,
                                      cudaStream_t st) {
-    const WinWgPlan pl = plan_window_wgrad(pb);
+    const WinWgPlan pl = plan_window_wgrad(pb, true);
     if (!pl.ok) return cudaErrorInvalidValue;
     WinWgrad g;
     g.n = pb.n; g.h_in = pb.h_in; g.w_in = pb.w_in; g.h_out = pb.h_out; g.w_out = pb.w_out; g.c_out = pb.c_out;

@@ -184,6 +184,23 @@ def test_stem_weight_gradient_of_infinite_values(n, h, w, k):
     np.testing.assert_allclose(got["dbeta"], t["dz"].sum((0, 2, 3)), rtol=1e-4, atol=1e-3)
 
 
+def test_stem_weight_gradient_without_room_for_a_packed_copy():
+    """At an odd width and 17.9 MB of scratch for the packed form, the no-allocation call goes to the window kernel."""
+    from paper_2305_11624_b200 import convbn as C
+    from paper_2305_11624_b200.harness import Block
+    spec = L("stem_noalloc", 64, 1, 239, 99, 64, 4, 3, stride=2, pad=2)
+    t = parity.make_inputs(spec, 84)
+    ref = parity.oracle_tune(spec, t)
+    blk = Block(spec, modes=("tune",))
+    assert C.convbn_workspace_bytes(blk.desc, C.PHASE_TUNE_BWD_WEIGHT) > 16 << 20
+    blk.load(t)
+    blk.tune_fwd()
+    C.convbn_tune_bwd_weight_noalloc(blk.desc, blk.dz, blk.x, blk.w, blk.b, blk.mu_hat, blk.saved, blk.dw, blk.db, blk.dgamma, blk.dbeta)
+    C.convbn_check()
+    got = {k: blk.fetch(k) for k in ("dw", "dgamma", "dbeta")}
+    parity.compare(got, ref, parity.TOL["f32"], ("dw", "dgamma", "dbeta"), spec.name, dtype="bf16")
+
+
 # (dtype, n, c_in, h, w, c_out, k, stride, pad): dZ summed inside the weight gradient where the kernel is the stride (one tile of
 # channels and several that take turns, more than eight of them, slices shorter than the turns, 3 x 3, 1 x 1), by the kernel of
 # its own where the windows overlap
