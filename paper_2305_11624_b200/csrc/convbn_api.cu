@@ -145,7 +145,8 @@ bool fused_bwd_path(const convbn_desc *d, const Problem &pb) {
 bool strided_dgrad_ok(const convbn_desc *d, const Problem &pb);
 bool umma_dgrad_shape(const convbn_desc *d, const Problem &pb, UmmaConvShape *s);
 
-// bounded: the tensor-core weight gradient in the slices of a call with a fixed scratch, a stem's without a packed copy of X; sums: what it sums beside.
+// bounded: the tensor-core weight gradient in the slices of a call with a fixed scratch, a stem's without a packed copy of X;
+// sums: what it sums beside.
 Plan form_plan(const convbn_desc *d, const Problem &pb, int phase, bool bounded, WgradSums sums);
 
 // The plans of the last layers of this thread: a function of the descriptor, the phase and the device (its SM count).  A
@@ -482,17 +483,18 @@ int run_conv_fwd(const convbn_desc *d, const Problem &pb, const void *x, const v
     return CONVBN_OK;
 }
 
-// Whether a stem layer's input gradient goes to the window kernel.  Rows of a multiple of 8 pixels: where that kernel takes the layer.
-// At other widths (its rows then leave in 2-byte stores) the shorter estimate decides, in us: here the weights' way into shared memory and
-// the rows of dZ that an SM multiplies; against
-// - the sub-pixel kernel's rounds of tiles, where that kernel takes the layer.  Fitted to 359 layers (3x3 to 7x7, 2 to 4 channels,
-//   18 x 20 to 239 x 251, up to 800 thousand pixels): 1 % from the better one on average, at most 7 % behind the sub-pixel
-//   kernel.  3 -> 64, 7x7, sub-pixel and window: 118 x 108, N = 32 44.5 and 20.0, 225 x 225, N = 8 44.7 and 15.1, 62 x 62,
-//   N = 69 15.7 and 22.0, 46 x 45, N = 1512 109 and 213.  Below 4096 pixels the sub-pixel kernel keeps the layer: the parity tests'
-//   small ones are there to run it (30 x 30, 5x5, N = 1 7.9 and 6.6);
+// Whether a stem layer's input gradient goes to the window kernel.  Rows of a multiple of 8 pixels: where that kernel takes the
+// layer. At other widths (its rows then leave in 2-byte stores) the shorter estimate decides, in us: here the weights' way into
+// shared memory and the rows of dZ that an SM multiplies; against
+// - the sub-pixel kernel's rounds of tiles, where that kernel takes the layer.  Fitted to 359 layers (3x3 to 7x7, 2 to 4
+//   channels, 18 x 20 to 239 x 251, up to 800 thousand pixels): 1 % from the better one on average, at most 7 % behind the
+//   sub-pixel kernel.  3 -> 64, 7x7, sub-pixel and window: 118 x 108, N = 32 44.5 and 20.0, 225 x 225, N = 8 44.7 and 15.1, 62
+//   x 62, N = 69 15.7 and 22.0, 46 x 45, N = 1512 109 and 213.  Below 4096 pixels the sub-pixel kernel keeps the layer: the
+//   parity tests' small ones are there to run it (30 x 30, 5x5, N = 1 7.9 and 6.6);
 // - otherwise the warp-level kernel's windows of 29 or more positions.  160 layers: 0.4 % from the better one, never behind the
-//   warp-level kernel.  7x7 at 30 x 30, N = 32 28.8 and 12.0, 3x3 at 18 x 21, N = 667 31.7 and 36.7.  Below 512 pixels that kernel
-//   keeps the layer (7x7 at 30 x 30, N = 1 28.4 and 9.0), once more for the parity tests: it serves what the others do not take.
+//   warp-level kernel.  7x7 at 30 x 30, N = 32 28.8 and 12.0, 3x3 at 18 x 21, N = 667 31.7 and 36.7.  Below 512 pixels that
+//   kernel keeps the layer (7x7 at 30 x 30, N = 1 28.4 and 9.0), once more for the parity tests: it serves what the others do
+//   not take.
 bool stem_dgrad_by_window(const convbn_desc *d, const Problem &pb) {
     if (!stem_path(d, pb) || !stem_window_dgrad_eligible(pb)) return false;
     if (pb.w_in % 8 == 0) return true;

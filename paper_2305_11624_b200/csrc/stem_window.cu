@@ -49,9 +49,9 @@ struct WinGemm {
 constexpr int kWinMaxRow = 256;          // weights of an output channel (16 x 8 taps of 4 channels would be 512)
 struct WinCtl {
     uint64_t strip_full[kWinMaxStrips], strip_empty[kWinMaxStrips];
-    // An accumulator's units go to the three warp groups in turn, and a warp need not be near the others (one whose pixels lie beyond
-    // the row end only passes by).  So each group has a barrier of its own per accumulator and meets every phase of it: on
-    // one barrier for all it could take the phase before last for its own, two phases having the same parity.
+    // An accumulator's units go to the three warp groups in turn, and a warp need not be near the others (one whose pixels lie
+    // beyond the row end only passes by).  So each group has a barrier of its own per accumulator and meets every phase of it:
+    // on one barrier for all it could take the phase before last for its own, two phases having the same parity.
     uint64_t tmem_full[kWinEpiGroups][8], tmem_empty[8];
     uint32_t tmem_base;
     int abort_flag;
@@ -756,12 +756,12 @@ cudaError_t launch_window_c(int c_in, const CUtensorMap &tout, const WinGemm &g,
 
 }  // namespace
 
-// Rows of a multiple of 8 pixels: whatever the kernel takes.  At other widths the GEMM on the packed input (pack, expand, multiply)
-// is the alternative that layers go back to where it is the faster one: short rows, many of them.  Estimates in us fitted to 728
-// layers (3x3 to 7x7, 1 to 4 channels, 64 and 128 outputs, 9 x 10 to 333 x 501, up to 800 thousand pixels): here the
-// weights' way into shared memory and the rows of 128 pixels that an SM computes, there 8 x 16 patches.  Forward of 3 -> 64, 7x7, packed
-// and here: 18 x 21, N = 667 20.9 and 34.9, 62 x 62, N = 64 13.8 and 17.1, 225 x 225, N = 16 26.5 and 16.7, 46 x 36, N = 8
-// 9.4 and 7.5.  The choice is 0.7 % from the better one on average and at most 2 % behind the packed form.
+// Rows of a multiple of 8 pixels: whatever the kernel takes.  At other widths the GEMM on the packed input (pack, expand,
+// multiply) is the alternative that layers go back to where it is the faster one: short rows, many of them.  Estimates in us
+// fitted to 728 layers (3x3 to 7x7, 1 to 4 channels, 64 and 128 outputs, 9 x 10 to 333 x 501, up to 800 thousand pixels): here
+// the weights' way into shared memory and the rows of 128 pixels that an SM computes, there 8 x 16 patches.  Forward of 3 ->
+// 64, 7x7, packed and here: 18 x 21, N = 667 20.9 and 34.9, 62 x 62, N = 64 13.8 and 17.1, 225 x 225, N = 16 26.5 and 16.7, 46
+// x 36, N = 8 9.4 and 7.5.  The choice is 0.7 % from the better one on average and at most 2 % behind the packed form.
 bool stem_window_eligible(const Problem &pb) {
     if (!plan_window(pb).ok) return false;
     if (pb.w_in % 8 == 0) return true;
@@ -777,11 +777,11 @@ namespace {
 struct WinWgPlan { bool ok = false; int pitch = 0, ksteps = 0; uint32_t xstrip = 0, dzrow = 0, work = 0; size_t smem = 0; };
 WinWgPlan plan_window_wgrad(const Problem &pb, bool any_width) {
     WinWgPlan pl;
-    // Rows of a multiple of 8 pixels only.  At other widths the GEMM on the packed input is the faster one by far where rows are
-    // short, this kernel's work going by rows (3 -> 64, 7x7 at 62 x 62, N = 64 21.9 and 34.7 us, at 9 x 10, N = 640 21.3 and
-    // 40.6), and behind where they are long (225 x 225, N = 16 33.4 and 26.7); and it reads what is beyond a row as zeros, where this
-    // one multiplies zeros of dZ by the next pixels, which an infinite X makes NaN.  (any_width: the call whose fixed scratch has no room for
-    // the packed input.)
+    // Rows of a multiple of 8 pixels only.  At other widths the GEMM on the packed input is the faster one by far where rows
+    // are short, this kernel's work going by rows (3 -> 64, 7x7 at 62 x 62, N = 64 21.9 and 34.7 us, at 9 x 10, N = 640 21.3
+    // and 40.6), and behind where they are long (225 x 225, N = 16 33.4 and 26.7); and it reads what is beyond a row as zeros,
+    // where this one multiplies zeros of dZ by the next pixels, which an infinite X makes NaN.  (any_width: the call whose
+    // fixed scratch has no room for the packed input.)
     if (pb.w_in % 8 && !any_width) return pl;
     if (!plan_window(pb).ok || pb.c_in > 3 || pb.c_out != 64 || pb.kh < 2 || pb.kh > 8 || pb.w_out > 256) return pl;
     pl.pitch = (int)(((size_t)(pb.w_in + 2 * pb.pad_w) * 8 + 15) / 16 * 16);

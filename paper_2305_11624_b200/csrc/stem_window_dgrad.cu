@@ -269,8 +269,8 @@ __global__ void __launch_bounds__(kDgThreads) stem_window_dgrad_kernel(const __g
 #pragma unroll
                         for (int c = 0; c < C; ++c) tile[((q - 2) * 4 + c) * 128 + j] = __uint_as_float(v[4 * q + c]);
                     named_bar_sync(bar_id, 128);
-                    // padded pixel u = 2 j + b gets window position q = b + 2 t of accumulator row j - t, t = 0 .. 3; positions from kw on
-                    // are left out (their weights are zeros, which an infinite dZ would make NaN)
+                    // padded pixel u = 2 j + b gets window position q = b + 2 t of accumulator row j - t, t = 0 .. 3; positions
+                    // from kw on are left out (their weights are zeros, which an infinite dZ would make NaN)
 #pragma unroll
                     for (int b = 0; b < 2; ++b) {
                         const int p = 2 * j + b - g.pad_w;

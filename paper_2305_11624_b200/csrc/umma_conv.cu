@@ -470,8 +470,8 @@ __global__ void __launch_bounds__(MODE == kPlain || MODE == kRelu || MODE == kTa
         for (uint32_t i = 0; columns_of(i, mt, nt, c_lo, c_hi); ++i) {
             if (c_lo >= c_hi) continue;
             const uint32_t acc = i & 1u;
-            // (the other group's buffer, for the last tile: this group has drained tile i - 1, whose products were complete after those
-            // of tile i - 2, so the barrier is past that earlier phase of the same parity)
+            // (the other group's buffer, for the last tile: this group has drained tile i - 1, whose products were complete
+            // after those of tile i - 2, so the barrier is past that earlier phase of the same parity)
             CONVBN_TRACE_T0();
             const bool ok = __all_sync(0xffffffffu, mbar_wait_bounded(&ctl->tmem_full[acc], (i >> 1) & 1u, abort_flag));
             if (warp == 2 && lane == 0) CONVBN_TRACE_ACC(15);
@@ -851,15 +851,15 @@ static cudaError_t launch_mode(int bn, bool pair, const CUtensorMap &ta, const C
     return launch_bn<256, MODE>(ta, tw, tout, tout2, tmask, g, bias, err, st);
 }
 
-// Tile width, and whether CTAs work in pairs: the least time by a model of clocks fitted to 24 layers (3x3 and 1x1, 64 to
-// 2048 channels, N = 8 to 256, both directions) at all six choices.  A round of tiles takes the larger of its k-blocks and
-// its epilogue (1x1 64 -> 256 at 56 x 56, N = 256: 83.7 us with 128 columns, 96.5 with 256); the last tile's epilogue and a pair's
-// start-up (a cluster launch, two CTAs meeting twice) come on top.  A k-block costs a CTA of a pair 20 to 90 clocks less, being half
-// a weight tile to write to and read from shared memory, so pairs pay for long K or many rounds (1x1 512 -> 1024 at 28 x 28, N = 32
-// 28.6 us alone with 128 columns, 22.7 in pairs with 256; 64 -> 64 at 56 x 56, N = 8 3.7 alone, 4.6 in pairs).  The terms of the epilogue date
-// from one that took 1.5 times as long: over 112 passes (the layers above, also at N = 64) the choice is now 3 % from the best on
-// average, and furthest where wide pairs win (1x1 512 -> 256 at 14 x 14, N = 256
-// 18.1 us and 13.4).
+// Tile width, and whether CTAs work in pairs: the least time by a model of clocks fitted to 24 layers (3x3 and 1x1, 64 to 2048
+// channels, N = 8 to 256, both directions) at all six choices.  A round of tiles takes the larger of its k-blocks and its
+// epilogue (1x1 64 -> 256 at 56 x 56, N = 256: 83.7 us with 128 columns, 96.5 with 256); the last tile's epilogue and a pair's
+// start-up (a cluster launch, two CTAs meeting twice) come on top.  A k-block costs a CTA of a pair 20 to 90 clocks less, being
+// half a weight tile to write to and read from shared memory, so pairs pay for long K or many rounds (1x1 512 -> 1024 at 28 x
+// 28, N = 32 28.6 us alone with 128 columns, 22.7 in pairs with 256; 64 -> 64 at 56 x 56, N = 8 3.7 alone, 4.6 in pairs).  The
+// terms of the epilogue date from one that took 1.5 times as long: over 112 passes (the layers above, also at N = 64) the
+// choice is now 3 % from the best on average, and furthest where wide pairs win (1x1 512 -> 256 at 14 x 14, N = 256 18.1 us and
+// 13.4).
 struct TilePick { int bn; bool pair; };
 static TilePick pick_tile(long long tiles_m, int cn, int num_kb, bool pairs, int max_bn) {
     static const double clk[2][3] = {{645, 300, 260}, {555, 280, 205}};

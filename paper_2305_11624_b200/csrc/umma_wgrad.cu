@@ -566,13 +566,14 @@ __global__ void __launch_bounds__(kRowsMaxThreads) wgrad_rows_kernel(int c_out, 
 cudaError_t launch_wgrad_rows(const Problem &pb, int splits, const float *partials, const float *bsum, const void *w,
                               const float *vec3, const float *b, const float *mean, float *dw, float *db, float *dgamma,
                               float *dbeta, bool need_sums, cudaStream_t st) {
-    // Slice groups so that a thread adds at most eight slices, threads along the span in equal turns.  Blocks per channel: up to two per
-    // SM for rows with 1600 vectors (of all slices) or more to read, one otherwise: below that and with more channels the blocks' meeting
-    // and their number cost more than they share.  Weight phase with 1, 2, 4, 8 blocks per channel: 1x1 256 -> 64, 1000 rows, 256 vectors
-    // 9.4 9.7 10.0 9.8 us; 3x3 256 -> 128, 26 x 26, 1728 vectors 7.8 7.2 7.4 7.4; 3x3 64 -> 64, 56 x 56, N = 32, 8496 vectors
-    // 21.1 18.2 16.2 16.3; 3x3 512 -> 512, 7 x 7, N = 64 21.0 22.5 25.3 26.0; 5x5 640 -> 384, 13 x 13, N = 9 40.4 44.7 49.8 60.2;
-    // whole backward calls at 192 and 256 channels, 4000 to 4400 vectors: 3x3 256 -> 256, 14 x 14, N = 32 27.0 27.4 27.1 29.0, 1x1
-    // 832 -> 256 57.0 58.8 57.9 59.2, 3x3 192 -> 192, 28 x 28, N = 16 32.8 34.1 33.4 34.6.
+    // Slice groups so that a thread adds at most eight slices, threads along the span in equal turns.  Blocks per channel: up
+    // to two per SM for rows with 1600 vectors (of all slices) or more to read, one otherwise: below that and with more
+    // channels the blocks' meeting and their number cost more than they share.  Weight phase with 1, 2, 4, 8 blocks per
+    // channel: 1x1 256 -> 64, 1000 rows, 256 vectors 9.4 9.7 10.0 9.8 us; 3x3 256 -> 128, 26 x 26, 1728 vectors 7.8 7.2 7.4
+    // 7.4; 3x3 64 -> 64, 56 x 56, N = 32, 8496 vectors 21.1 18.2 16.2 16.3; 3x3 512 -> 512, 7 x 7, N = 64 21.0 22.5 25.3 26.0;
+    // 5x5 640 -> 384, 13 x 13, N = 9 40.4 44.7 49.8 60.2; whole backward calls at 192 and 256 channels, 4000 to 4400 vectors:
+    // 3x3 256 -> 256, 14 x 14, N = 32 27.0 27.4 27.1 29.0, 1x1 832 -> 256 57.0 58.8 57.9 59.2, 3x3 192 -> 192, 28 x 28, N = 16
+    // 32.8 34.1 33.4 34.6.
     int SL = 1, CL = 1;
     while (SL < 32 && SL * 8 < splits) SL *= 2;
     auto vectors = [&](int cl) { return ((pb.kdim / 4 + cl - 1) / cl + 7) / 8 * 8; };
